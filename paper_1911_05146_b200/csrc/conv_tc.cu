@@ -32,17 +32,17 @@
 // device status word, stops issuing work, waits (bounded) for its TMA copies in flight, frees its
 // tensor memory and returns.
 #include "conv_tc.h"
+#include "tc_ptx.cuh"
 
-#include <cuda.h>
 #include <stdint.h>
 #include <string.h>
 
 namespace hpf {
 
+EncodeTiledFn g_encode = nullptr;
+
 namespace {
 
-constexpr int kTileM = 128;                 // MMA M (TMEM lanes)
-constexpr long long kWaitLimit = 4000000000LL;   // clock64 ticks (~2 s) before a wait gives up
 constexpr uint32_t kSmemBudget = 200 * 1024;
 constexpr uint32_t kWgradSmemBudget = 220 * 1024;   // the weight-gradient kernel has next to no static shared memory
 constexpr int kFwdMaxStages = 4;
@@ -54,154 +54,6 @@ constexpr int kMultiTileFrom = 2 * 296;     // CTAs (two per SM) beyond which a 
 constexpr unsigned int kCellTmemCols = 256;  // tensor-memory columns a persistent cell CTA may hold (two such CTAs share an SM's 512)
 constexpr unsigned int kCellSmemBudget = 100 * 1024;   // dynamic shared memory of a cell CTA (two per SM)
 constexpr unsigned int kWgradSlack = 16384;   // an MMA reads 128 operand rows (16 KB) from a base that may be the last one in use
-
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-EncodeTiledFn g_encode = nullptr;
-
-// ------------------------------------------------------------------------------------------------
-// PTX wrappers
-// ------------------------------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_inval(uint32_t bar)
-{
-    asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ uint32_t mbar_try_wait(uint32_t bar, uint32_t parity)
-{
-    uint32_t ok;
-    asm volatile(
-        "{\n"
-        ".reg .pred p;\n"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-        "selp.u32 %0, 1, 0, p;\n"
-        "}\n"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    return ok;
-}
-// Bounded wait.  Returns false if it gave up (or another role already did).
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag)
-{
-    if (mbar_try_wait(bar, parity)) return true;
-    const long long t0 = clock64();
-    for (;;) {
-        if (mbar_try_wait(bar, parity)) return true;
-        if (*abort_flag) return false;
-        if (clock64() - t0 > kWaitLimit) { *abort_flag = 1; return false; }
-    }
-}
-__device__ __forceinline__ void tma_load_4d(uint32_t dst, const void* tmap, uint32_t bar, int c0, int c1, int c2, int c3)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
-        ::"r"(dst), "l"(tmap), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
-        : "memory");
-}
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const void* tmap, uint32_t bar, int c0, int c1)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-        ::"r"(dst), "l"(tmap), "r"(bar), "r"(c0), "r"(c1)
-        : "memory");
-}
-__device__ __forceinline__ void tmem_alloc(uint32_t smem_dst, uint32_t ncols)
-{
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_dst), "r"(ncols) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols)
-{
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
-}
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void umma_tf32(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate)
-{
-    asm volatile(
-        "{\n"
-        ".reg .pred p;\n"
-        "setp.ne.b32 p, %4, 0;\n"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n"
-        "}\n"
-        ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-__device__ __forceinline__ void umma_commit(uint32_t bar)
-{
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-// 32 lanes x 16 consecutive 32-bit columns: thread i of the warp receives lane (base lane + i)
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v)
-{
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr)
-        : "memory");
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
-
-// The same without the wait, so that several loads can be in flight before one tmem_ld_wait().
-__device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, float* v)
-{
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr)
-        : "memory");
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
-__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-__device__ __forceinline__ void prefetch_tmap(const void* tmap)
-{
-    asm volatile("prefetch.tensormap [%0];" ::"l"(tmap) : "memory");
-}
-
-// Shared-memory matrix descriptor (sm_100 format): start address, leading / stride byte offsets in
-// 16-byte units, descriptor version 1, swizzle mode in the top bits (2 = 128 B, 4 = 64 B).
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo_bytes, uint32_t sbo_bytes, uint32_t swizzle_bytes)
-{
-    const uint64_t layout = swizzle_bytes == 128 ? 2ull : 4ull;
-    return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)((lbo_bytes >> 4) & 0x3FFFu) << 16) |
-           ((uint64_t)((sbo_bytes >> 4) & 0x3FFFu) << 32) | (1ull << 46) | (layout << 61);
-}
-
-// MN-major TF32 operand (the reduction index runs over the rows of the tile, channels are contiguous): the one layout
-// the tensor core accepts for 32-bit MN-major operands is rows of 128 bytes whose 32-byte chunks are XOR-swizzled by
-// (row % 4) (layout type 1, what a TMA box with CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B delivers).  One MMA of K = 8 reads
-// 8 consecutive rows (two groups of 4, `stride` = 512 bytes apart) of every 32-channel block; `block_bytes` is the
-// distance between consecutive 32-channel blocks (the leading-dimension offset).
-__device__ __forceinline__ uint64_t smem_desc_mn(uint32_t addr, uint32_t block_bytes)
-{
-    return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)((block_bytes >> 4) & 0x3FFFu) << 16) |
-           ((uint64_t)((512u >> 4) & 0x3FFFu) << 32) | (1ull << 46) | (1ull << 61);
-}
-
-// Instruction descriptor: fp32 accumulator, TF32 A and B, M = 128, N = n; major bits select MN-major operands.
-inline uint32_t instr_desc(int n, bool a_mn_major, bool b_mn_major)
-{
-    return (1u << 4) | (2u << 7) | (2u << 10) | ((a_mn_major ? 1u : 0u) << 15) | ((b_mn_major ? 1u : 0u) << 16) |
-           ((uint32_t)(n >> 3) << 17) | ((uint32_t)(kTileM >> 4) << 24);
-}
 
 // Optional timelines for latency studies (debug builds only).  HPF_TC_TIMELINE=2: every CTA of the forward kernel
 // stamps its milestones in shared memory and adds the elapsed times to per-class totals (class = window size and
@@ -226,11 +78,6 @@ __device__ unsigned long long g_tl_acc[8][16];
 #else
 #define HPF_TL(slot) do {} while (0)
 #endif
-
-__device__ __forceinline__ void report(DeviceStatus* status, unsigned int code)
-{
-    if (atomicCAS(&status->code, 0u, code) == 0u) status->detail = blockIdx.x;
-}
 
 // ------------------------------------------------------------------------------------------------
 // kernel parameters
@@ -341,23 +188,6 @@ struct alignas(64) WgradDirectParams {
     WgradDirectScalars s;
 };
 
-template <class T>
-__device__ __forceinline__ void load_scalars(T* dst, const T* src)
-{
-    static_assert(sizeof(T) % 4 == 0, "scalar block must be a whole number of words");
-    const uint32_t* w = reinterpret_cast<const uint32_t*>(src);
-    for (int i = threadIdx.x; i < (int)(sizeof(T) / 4); i += blockDim.x) reinterpret_cast<uint32_t*>(dst)[i] = w[i];
-}
-
-__device__ __forceinline__ void mbar_arrive(uint32_t bar)
-{
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-
-// x = hi + lo, hi = x with the low 13 significand bits cleared (what a TF32 operand keeps)
-__device__ __forceinline__ float tf32_hi(float x) { return __uint_as_float(__float_as_uint(x) & 0xFFFFE000u); }
-
 // BN statistics from per-tile moments [n_tiles][2][C]: per tile and channel the mean of the tile's values and the sum
 // of their squared deviations from that mean (M2).  Every tile holds the same number of values (the host fuses only
 // launches whose tiles are all full), so the total is
@@ -466,7 +296,7 @@ __device__ __forceinline__ int conv_fwd_cta(const FwdParams* gpp, FwdScalars& p,
     const uint32_t base_off = ((smem_u32(smem_raw) + 1023u) & ~1023u) - smem_u32(smem_raw);
     uint8_t* smem = smem_raw + base_off;
     const uint32_t smem_base = smem_u32(smem);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const uint32_t full0 = smem_u32(&bars[0]), empty0 = smem_u32(&bars[8]), split0 = smem_u32(&bars[16]),
                    accum_bar = smem_u32(&bars[24]);
     // stage layout: A | A_lo | B_hi | B_lo   (the lo parts only in three-pass mode)
@@ -494,11 +324,11 @@ __device__ __forceinline__ int conv_fwd_cta(const FwdParams* gpp, FwdScalars& p,
     // this CTA's share of the K loop (all of it unless the launch splits K over gridDim.z)
     const int kb = KSPLIT ? (int)(((long long)total * vb.z) / p.ksplit) : 0;
     const int ke = KSPLIT ? (int)(((long long)total * (vb.z + 1)) / p.ksplit) : total;
-    // Thread 0 is the TMA producer.  The origin of its first tile and its first K step are a chain of dependent
+    // One lane of warp 0 is the TMA producer.  The origin of its first tile and its first K step are a chain of dependent
     // shared-memory reads and integer divisions in ONE thread (most of a microsecond): worked out here, while the CTA
     // still waits for tensor memory and for the preceding kernel, not between that wait and the first copy.
     int f_q0 = 0, f_p0 = 0, f_n0 = 0, f_tap = 0, f_kc = 0, f_r = 0, f_sx = 0;
-    if (threadIdx.x == 0) {
+    if (warp == 0) {
         HPF_TILE_ORIGIN(tile0);
         f_q0 = q0; f_p0 = p0; f_n0 = n0;
         if (KSPLIT) { f_tap = kb / p.n_kchunks; f_kc = kb % p.n_kchunks; f_r = f_tap / p.R; f_sx = f_tap % p.R; }
@@ -516,14 +346,14 @@ __device__ __forceinline__ int conv_fwd_cta(const FwdParams* gpp, FwdScalars& p,
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    // Everything above touched only parameters, shared and tensor memory.  The TMA producer (thread 0) first works out
+    // Everything above touched only parameters, shared and tensor memory.  The TMA producer (warp 0) first works out
     // its first tile's coordinates - a chain of dependent shared-memory reads and integer divisions of most of a
     // microsecond - and waits for the preceding kernel only then, right before its first copy.
-    if (!CELL && threadIdx.x != 0) pdl_wait();
+    if (!CELL && warp != 0) pdl_wait();
     const uint32_t tmem_base = CELL ? cell_tmem_base : tmem_slot;
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             // ---- TMA producer ----
             // no division in the loop: stage, parity, tap and K chunk are counters
             int it = 0, st = 0;
@@ -567,7 +397,7 @@ __device__ __forceinline__ int conv_fwd_cta(const FwdParams* gpp, FwdScalars& p,
             issued = it;
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             // ---- MMA issuer ----
             // One thread issues every MMA, so the loop is kept to a few instructions per MMA: the descriptor's
             // constant part is built once and only its 14-bit address field is advanced (32 bytes = 2 units per K step).
@@ -1196,7 +1026,7 @@ __global__ void __launch_bounds__(192) conv_tc_wgrad_kernel(const __grid_constan
     const uint32_t base_off = ((smem_u32(smem_raw) + 1023u) & ~1023u) - smem_u32(smem_raw);
     uint8_t* smem = smem_raw + base_off;
     const uint32_t smem_base = smem_u32(smem);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const uint32_t full_raw0 = smem_u32(&bars[0]), empty_raw0 = smem_u32(&bars[4]), full_t0 = smem_u32(&bars[8]),
                    empty_t0 = smem_u32(&bars[12]), accum_bar = smem_u32(&bars[16]);
     // shared memory: raw stages first, then the transposed stages
@@ -1257,7 +1087,7 @@ __global__ void __launch_bounds__(192) conv_tc_wgrad_kernel(const __grid_constan
     const uint32_t tmem_base = tmem_slot;
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             // ---- TMA producer ----
             // no division in the loop: the stage, its parity, the tile's position and the taps' offsets are counters
             const int raw_stages = p.raw_stages, tiles_w = p.tiles_w, tiles_h = p.tiles_h, R = p.R, pad = p.pad;
@@ -1286,7 +1116,7 @@ __global__ void __launch_bounds__(192) conv_tc_wgrad_kernel(const __grid_constan
             issued = it;
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             // ---- MMA issuer ----
             const int t_stages = p.t_stages;
             int it = 0, t = 0;
@@ -1419,7 +1249,7 @@ __global__ void __launch_bounds__(192) conv_tc_wgrad_direct_kernel(const __grid_
     const uint32_t base_off = ((smem_u32(smem_raw) + 1023u) & ~1023u) - smem_u32(smem_raw);
     uint8_t* smem = smem_raw + base_off;
     const uint32_t smem_base = smem_u32(smem);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const uint32_t full0 = smem_u32(&bars[0]), empty0 = smem_u32(&bars[8]), split0 = smem_u32(&bars[16]), accum_bar = smem_u32(&bars[24]);
 
     const int split = blockIdx.x;
@@ -1465,7 +1295,7 @@ __global__ void __launch_bounds__(192) conv_tc_wgrad_direct_kernel(const __grid_
     const uint32_t tmem_base = tmem_slot;
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             // ---- TMA producer ----
             const int stages = p.stages, tiles_w = p.tiles_w, tiles_h = p.tiles_h, R = p.R, pad = p.pad;
             const int box_w = p.box_w, box_h = p.box_h, box_n = p.box_n, m_blocks = p.m_blocks, n_blocks = p.n_blocks;
@@ -1495,7 +1325,7 @@ __global__ void __launch_bounds__(192) conv_tc_wgrad_direct_kernel(const __grid_
             issued = it;
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             // ---- MMA issuer ----
             const int stages = p.stages, k8n = p.rows >> 3;
             const bool three = p.passes == 3;
