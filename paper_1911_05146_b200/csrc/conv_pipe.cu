@@ -1,0 +1,1472 @@
+// Forward convolution and data gradient (a forward convolution of dy with rearranged weights), sm_100a: one persistent CTA
+// per SM walks units of work, every role of the pipeline on warps of its own.
+//
+//   D[position, c_out] = sum over channel chunks of 16 and taps  A[position + tap, c] * W[c_out, tap, c]
+//
+// What bounds these launches.  At 16..256 channels the convolutions of a residual network move far more bytes than the
+// tensor core needs time for, so the kernel is built as a stream: loads of the next operand block, the split of this one,
+// its MMAs and the write-out of the one before run side by side, and no step of a tile waits for the whole tile before it.
+//
+// Positions.  A 3x3 window (pad 1) is computed on a padded grid of positions: every map row is followed by ONE zero column
+// (it is the right border of its row and the left border of the next), every map by one zero row.  In shared memory the
+// positions are consecutive 128-byte rows, so the operand of tap (r, s) is the same block of rows read from
+// (r-1)*Wp + (s-1) rows further on: a block is loaded, normalised and split ONCE for its nine taps.  (A K-major operand may
+// start at any 128-byte row: the swizzle is a function of the address.)  The padding costs MMA rows (1/17 of them at 16
+// pixels, 1/9 at 8) and saves eight of nine copies.  Maps wider than 254 pixels are cut into column strips with a zero or
+// neighbour column on either side.  A 1x1 window has no halo: positions are the output pixels.
+//
+// Operand rows.  A chunk is 16 channels: bytes 0-63 of the 128-byte row hold the value (the tensor core ignores the low 13
+// mantissa bits: that is the hi part), bytes 64-127 the lo part of the three-pass form, in the 128-byte swizzle.
+//
+// Roles (16 warps): warp 0 copies the operand, warp 1 the weights (TMA; kept in shared memory for the whole launch when they
+// fit), warp 2 issues the MMAs, warps 4-7 rewrite the operand in place (BN+ReLU, lo part), warps 8-15 read finished
+// accumulators from tensor memory, add the residual, store and form the BN moments.
+#include "conv_pipe.h"
+#include "tc_ptx.cuh"
+
+#include <algorithm>
+#include <string.h>
+#include <type_traits>
+
+namespace hpf {
+
+namespace {
+
+constexpr int kSplitWarps = 4, kEpiWarps = 8;
+constexpr int kFirstSplit = 4;                        // warps 0..2: operand copies, weight copies, MMAs; 3 idle
+constexpr int kSplitThreads = 32 * kSplitWarps, kRowStep = 8 * kSplitWarps;
+constexpr int kPipeThreads = 32 * (kFirstSplit + kSplitWarps + kEpiWarps);
+constexpr int kMaxBlockRows = 768, kRowBatch = 4;     // operand rows of a block at most; rows a splitter thread has in flight
+constexpr uint32_t kPipeSmem = 222 * 1024;            // dynamic shared memory of a CTA
+constexpr int kMaxA = 4, kMaxB = 8;
+
+struct PipeScalars {
+    const float* in;
+    float* out;
+    const float* extra;
+    DeviceStatus* status;
+    long long in_ms, out_ms;                          // floats between micro-batches (extra is laid out like out)
+    int accumulate;
+    int units_per_m, unit_block, blocks_per_m, tiles_per_m, T, slices, n_chunk, ksplit;
+    int R, taps, n_chunks, c_in, c_out;
+    int pos_per_m, Wp, img_pos, Hv, W, halo, strips, strip_w, col0;
+    uint32_t magic_w, magic_img, magic_strip;
+    int in_sw, in_sh, in_sn, os_w, os_h, os_n;
+    int zero_fill, out_h, out_w, dense_h, dense_w;
+    int a_stages, b_stages, b_resident, acc_bufs, split_groups, epi_alternate;
+    // how the operand is copied: flat (128 consecutive pixels per box) or blocks of box_h padded rows of one map
+    int flat, box_h, box_pos, blocks_per_img;
+    uint32_t magic_box, magic_bpi;
+    long long pix_ms;                                 // flat: pixels per micro-batch; else maps per micro-batch
+    uint32_t a_stage_bytes, b_stage_bytes, acc_cols, tmem_cols, idesc, idesc2;
+    uint32_t off_b, off_bn, off_red, off_stat, off_stage;
+    int three, stacked, pdl_late, w_ready;
+    // BN+ReLU on the way in
+    const float* bn_partials;
+    const float* bn_gamma;
+    const float* bn_beta;
+    float* bn_stats;
+    float* bn_y;
+    int bn_units;
+    float bn_eps;
+    double bn_inv_rows;
+    // BN moments of the output
+    float* st_partials;
+    // split K
+    char* sk_base;                                    // per micro-batch: tickets, then partial tiles
+    long long sk_ms;                                  // bytes between micro-batches
+};
+struct alignas(64) PipeParams {
+    CUtensorMap tm_a, tm_b, tm_b_lo;
+    PipeScalars s;
+};
+
+// x / d with magic = floor(2^32 / d) + 1: the estimate is at most one too large
+__device__ __forceinline__ int div_magic(int x, int d, uint32_t magic)
+{
+    if (d == 1) return x;
+    int q = (int)__umulhi((uint32_t)x, magic);
+    return q * d > x ? q - 1 : q;
+}
+inline uint32_t magic_of(int d) { return d <= 1 ? 0u : (uint32_t)((1ull << 32) / (uint64_t)d) + 1u; }
+
+struct Pixel { int n, y, x; bool in, own; };
+// position -> pixel; in: a pixel of the map (padding otherwise), own: an output of this position (not a strip's halo column)
+__device__ __forceinline__ Pixel locate(const PipeScalars& p, int pos)
+{
+    Pixel r;
+    const bool some = (unsigned)pos < (unsigned)p.pos_per_m;
+    const int q = some ? pos : 0;
+    int img = div_magic(q, p.img_pos, p.magic_img);
+    const int rem = q - img * p.img_pos;
+    r.y = div_magic(rem, p.Wp, p.magic_w);
+    const int col = rem - r.y * p.Wp - p.col0;
+    int x0 = 0;
+    if (p.strips > 1) {
+        const int n = div_magic(img, p.strips, p.magic_strip);
+        x0 = (img - n * p.strips) * p.strip_w;
+        img = n;
+    }
+    r.n = img; r.x = x0 + col;
+    r.in = some && r.y < p.Hv && (unsigned)r.x < (unsigned)p.W;
+    r.own = r.in && (unsigned)col < (unsigned)p.strip_w;
+    return r;
+}
+
+// 16 consecutive floats of one thread: two full sectors
+__device__ __forceinline__ void store16(float* d, const float* v)
+{
+    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(d), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]),
+                 "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]) : "memory");
+    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(d + 8), "f"(v[8]), "f"(v[9]), "f"(v[10]), "f"(v[11]),
+                 "f"(v[12]), "f"(v[13]), "f"(v[14]), "f"(v[15]) : "memory");
+}
+__device__ __forceinline__ void load16(const float* s, float* v)
+{
+#pragma unroll
+    for (int j = 0; j < 16; j += 4) {
+        const float4 t = __ldcg(reinterpret_cast<const float4*>(s + j));
+        v[j] = t.x; v[j + 1] = t.y; v[j + 2] = t.z; v[j + 3] = t.w;
+    }
+}
+__device__ __forceinline__ void split_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kSplitThreads) : "memory"); }
+__device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 2, 256;" ::: "memory"); }
+
+__host__ __device__ inline size_t partial_floats(int units, int C) { return (size_t)units * 2 * C + (size_t)((units + 3) & ~3); }
+
+// Statistics of a BN's input from the partial moments of one micro-batch: rows of (mean[C], M2[C]) with n values each.
+//   mean = ref + sum n (mean_u - ref) / N,   M2 = sum M2_u + sum n (mean_u - ref)^2 - N (mean - ref)^2,   ref = row 0's mean:
+// no difference of large numbers appears however far a channel's mean is from zero compared with its spread.  Fixed order
+// (every CTA of a launch gets the same bits), fp32 terms, the last combination in fp64.  THREADS threads, which share named barrier 1;
+// tab: mean[C], rstd[C]; red: 3 x THREADS float4.
+template <int THREADS>
+__device__ __forceinline__ void merge_moments(const float* partials, int units, int C, double inv_rows, float eps, float* tab, float4* red,
+                                              int tid)
+{
+    const float* counts = partials + (size_t)units * 2 * C;
+    const int c4n = C >> 2;
+    const int L = c4n <= THREADS ? THREADS / c4n : 1;
+    for (int c0 = 0; c0 < c4n; c0 += THREADS) {
+        const int col = c0 + (L > 1 ? tid % c4n : tid), ln = L > 1 ? tid / c4n : 0;
+        const bool mine = col < c4n && ln < L;
+        float4 sd = make_float4(0.f, 0.f, 0.f, 0.f), sq = sd, m2 = sd, ref = sd;
+        if (mine) {
+            ref = __ldcg(reinterpret_cast<const float4*>(partials) + col);
+            for (int k0 = ln; k0 < units; k0 += 4 * L) {
+                float4 a[4], b[4];
+                float n[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int k = k0 + j * L;
+                    const bool have = k < units;
+                    const float4* row = reinterpret_cast<const float4*>(partials + (size_t)(have ? k : 0) * 2 * C);
+                    n[j] = have ? __ldcg(counts + k) : 0.f;
+                    a[j] = __ldcg(row + col);
+                    b[j] = have ? __ldcg(row + c4n + col) : make_float4(0.f, 0.f, 0.f, 0.f);
+                }
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float dx = a[j].x - ref.x, dy = a[j].y - ref.y, dz = a[j].z - ref.z, dw = a[j].w - ref.w;
+                    sd.x = fmaf(n[j], dx, sd.x); sd.y = fmaf(n[j], dy, sd.y); sd.z = fmaf(n[j], dz, sd.z); sd.w = fmaf(n[j], dw, sd.w);
+                    sq.x = fmaf(n[j] * dx, dx, sq.x); sq.y = fmaf(n[j] * dy, dy, sq.y); sq.z = fmaf(n[j] * dz, dz, sq.z); sq.w = fmaf(n[j] * dw, dw, sq.w);
+                    m2.x += b[j].x; m2.y += b[j].y; m2.z += b[j].z; m2.w += b[j].w;
+                }
+            }
+        }
+        int lanes = L;                               // row lanes left to add, red[l * c4n + col]
+        if (c4n <= 16 && (c4n & (c4n - 1)) == 0) {
+            // the row lanes of a column inside a warp first: a fixed butterfly
+            for (int o = 16; o >= c4n; o >>= 1) {
+                sd.x += __shfl_xor_sync(0xffffffffu, sd.x, o); sd.y += __shfl_xor_sync(0xffffffffu, sd.y, o);
+                sd.z += __shfl_xor_sync(0xffffffffu, sd.z, o); sd.w += __shfl_xor_sync(0xffffffffu, sd.w, o);
+                sq.x += __shfl_xor_sync(0xffffffffu, sq.x, o); sq.y += __shfl_xor_sync(0xffffffffu, sq.y, o);
+                sq.z += __shfl_xor_sync(0xffffffffu, sq.z, o); sq.w += __shfl_xor_sync(0xffffffffu, sq.w, o);
+                m2.x += __shfl_xor_sync(0xffffffffu, m2.x, o); m2.y += __shfl_xor_sync(0xffffffffu, m2.y, o);
+                m2.z += __shfl_xor_sync(0xffffffffu, m2.z, o); m2.w += __shfl_xor_sync(0xffffffffu, m2.w, o);
+            }
+            lanes = THREADS / 32;
+            const int at = (tid >> 5) * c4n + (tid & 31);
+            if ((tid & 31) < c4n) { red[at] = sd; red[THREADS + at] = sq; red[2 * THREADS + at] = m2; }
+        } else if (L > 1) {
+            red[tid] = sd; red[THREADS + tid] = sq; red[2 * THREADS + tid] = m2;
+        }
+        if (lanes > 1) {
+            asm volatile("bar.sync 1, %0;" ::"n"(THREADS) : "memory");
+            if (mine && ln == 0)
+                for (int l = 1; l < lanes; ++l) {
+                    const float4 x = red[l * c4n + col], y = red[THREADS + l * c4n + col], z = red[2 * THREADS + l * c4n + col];
+                    sd.x += x.x; sd.y += x.y; sd.z += x.z; sd.w += x.w;
+                    sq.x += y.x; sq.y += y.y; sq.z += y.z; sq.w += y.w;
+                    m2.x += z.x; m2.y += z.y; m2.z += z.z; m2.w += z.w;
+                }
+        }
+        if (mine && ln == 0) {
+            const float d[4] = {sd.x, sd.y, sd.z, sd.w}, q[4] = {sq.x, sq.y, sq.z, sq.w}, v[4] = {m2.x, m2.y, m2.z, m2.w},
+                        r[4] = {ref.x, ref.y, ref.z, ref.w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const double dm = (double)d[j] * inv_rows;
+                double var = ((double)v[j] + (double)q[j]) * inv_rows - dm * dm;
+                if (var < 0.0) var = 0.0;
+                tab[4 * col + j] = (float)((double)r[j] + dm);
+                tab[C + 4 * col + j] = 1.0f / sqrtf((float)(var + (double)eps));
+            }
+        }
+    }
+}
+
+// Walks the units of this CTA: micro-batch, unit of the micro-batch, part of the K loop.  What a CTA takes are whole blocks of
+// `unit_block` consecutive units of a micro-batch, so that the BN moments of a block are formed by one CTA.
+struct UnitWalk {
+    int m, ul, z, left;          // left: blocks, the current one included
+    int end;                     // first unit beyond the current block
+    __device__ __forceinline__ UnitWalk(const PipeScalars& p, int m_first, int first, int count) : left(count)
+    {
+        z = 0;
+        if (p.ksplit > 1) { z = first % p.ksplit; first /= p.ksplit; }
+        m = first / p.blocks_per_m;
+        ul = (first - m * p.blocks_per_m) * p.unit_block;
+        m += m_first;
+        set_end(p);
+    }
+    __device__ __forceinline__ void set_end(const PipeScalars& p) { end = ul + p.unit_block < p.units_per_m ? ul + p.unit_block : p.units_per_m; }
+    __device__ __forceinline__ void next(const PipeScalars& p)
+    {
+        if (p.ksplit > 1) {      // (blocks of one unit)
+            --left;
+            if (++z < p.ksplit) return;
+            z = 0;
+            if (++ul == p.units_per_m) { ul = 0; ++m; }
+            return;
+        }
+        if (++ul < end) return;
+        --left;
+        if (ul == p.units_per_m) { ul = 0; ++m; }
+        set_end(p);
+    }
+    __device__ __forceinline__ bool last_of_block() const { return ul + 1 == end; }
+    __device__ __forceinline__ bool last(const PipeScalars& p) const { return left == 1 && (p.ksplit > 1 || last_of_block()); }
+    __device__ __forceinline__ int tiles(const PipeScalars& p) const { const int n = p.tiles_per_m - ul * p.T; return n < p.T ? n : p.T; }
+    __device__ __forceinline__ int kb(const PipeScalars& p) const { return p.ksplit > 1 ? z * p.n_chunks / p.ksplit : 0; }
+    __device__ __forceinline__ int ke(const PipeScalars& p) const { return p.ksplit > 1 ? (z + 1) * p.n_chunks / p.ksplit : p.n_chunks; }
+};
+
+// The operand block of a unit: whole copy blocks around the positions it needs.
+struct Span {
+    int block0, blocks;          // copy blocks (block0 may be -1: the zero row above the first map)
+    int pos0, rows, lead;        // position of the first row, rows, rows in front of the unit's first halo row
+};
+__device__ __forceinline__ Span span_of(const PipeScalars& p, const UnitWalk& u)
+{
+    Span r;
+    const int start = u.ul * p.T * kTileM - p.halo, need = u.tiles(p) * kTileM + 2 * p.halo;
+    if (p.flat) { r.block0 = start / kTileM; r.blocks = need / kTileM; r.pos0 = start; r.rows = need; r.lead = 0; return r; }
+    const int bp = p.box_pos;
+    r.block0 = div_magic(start + bp * 2, bp, p.magic_box) - 2;      // halo <= 2 blocks: the dividend is never negative
+    r.pos0 = r.block0 * bp;
+    r.lead = start - r.pos0;
+    r.blocks = div_magic(r.lead + need + bp - 1, bp, p.magic_box);
+    r.rows = r.blocks * bp;
+    return r;
+}
+
+struct EmitArgs {
+    float* out;                  // this warp's column group
+    const float* extra;
+    float4* patch;
+    float4* moments;             // this lane's k, sum (x - k), sum (x - k)^2 of its four columns: three planes of kMomentPlane, or null
+    bool accumulate, ok;
+    int fill;
+    bool zero_fill;
+    int dense_h, dense_w;
+    int step;                    // dense rows: floats between rows
+};
+constexpr int kMomentPlane = kEpiWarps * 32 * 2;      // two column groups per warp
+
+// One warp's 32 rows x (4 * LPR) columns of a tile: LPR lanes hold a row's 16-byte pieces.  Loads, shared-memory reads and
+// stores are batched by kind, so that a batch's latencies overlap.  DENSE: all 32 rows are stored, one after the other in
+// memory (row 0 at ro of lane 0); otherwise ro is this lane's row offset or -1.
+// Moments are taken about the first value the warp stored for a column: sums of x and x*x themselves would cancel for a
+// channel whose mean is large against its spread.
+template <int LPR, bool DENSE, class Stage>
+__device__ __forceinline__ void emit_rows(const EmitArgs& a, int ro, int lane, bool have_shift, Stage stage)
+{
+    constexpr int RSTEP = 32 / LPR;
+    const int cq = lane & (LPR - 1), rq = lane / LPR;
+    float4 e[4];
+    int so[4];
+    const int base = DENSE ? __shfl_sync(0xffffffffu, ro, 0) + rq * a.step + 4 * cq : 0;
+    auto offsets = [&](int b) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (DENSE) so[i] = base + (b + i) * RSTEP * a.step;
+            else {
+                const int r = __shfl_sync(0xffffffffu, ro, rq + RSTEP * (b + i));
+                so[i] = r >= 0 ? r + 4 * cq : -1;
+            }
+        }
+        if (a.extra) {
+            // (not the read-only path: the preceding kernel may have written it)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) e[i] = __ldcg(reinterpret_cast<const float4*>(a.extra + (DENSE || so[i] >= 0 ? so[i] : 0)));
+        }
+    };
+    offsets(0);                                       // the first residuals travel while the accumulator is read
+    stage();
+    __syncwarp();
+    const unsigned int who = DENSE ? 0xffffffffu : __ballot_sync(0xffffffffu, ro >= 0);      // lane = row here
+    float4 k = make_float4(0.f, 0.f, 0.f, 0.f), sd = k, sq = k;
+    if (a.moments && have_shift) k = a.moments[0];
+#pragma unroll
+    for (int b = 0; b < LPR; b += 4) {
+        if (b > 0) offsets(b);
+        float4 v[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) { const int r = rq + RSTEP * (b + i); v[i] = a.patch[r * 8 + (cq ^ (r & 7))]; }
+        if (a.extra) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) { v[i].x += e[i].x; v[i].y += e[i].y; v[i].z += e[i].z; v[i].w += e[i].w; }
+        }
+        if (a.accumulate) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (DENSE || so[i] >= 0) { const float4 o = __ldcg(reinterpret_cast<const float4*>(a.out + so[i])); v[i].x += o.x; v[i].y += o.y; v[i].z += o.z; v[i].w += o.w; }
+        }
+        if (a.ok) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) if (DENSE || so[i] >= 0) *reinterpret_cast<float4*>(a.out + so[i]) = v[i];
+        }
+        if (!DENSE && a.zero_fill) {
+            // strided data gradient: the positions between the samples receive no contribution
+            const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int f = __shfl_sync(0xffffffffu, a.fill, rq + RSTEP * (b + i));
+                if (so[i] >= 0 && a.ok) {
+                    if (f & 1) *reinterpret_cast<float4*>(a.out + so[i] + a.dense_w) = zero;
+                    if (f & 2) *reinterpret_cast<float4*>(a.out + so[i] + a.dense_h) = zero;
+                    if (f & 4) *reinterpret_cast<float4*>(a.out + so[i] + a.dense_h + a.dense_w) = zero;
+                }
+            }
+        }
+        if (a.moments && who) {
+            if (!have_shift) {
+                const int r0 = DENSE ? 0 : __ffs(who) - 1, src = (r0 % RSTEP) * LPR + cq, step = r0 / RSTEP - b;
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (step == i) {
+                        k.x = __shfl_sync(0xffffffffu, v[i].x, src); k.y = __shfl_sync(0xffffffffu, v[i].y, src);
+                        k.z = __shfl_sync(0xffffffffu, v[i].z, src); k.w = __shfl_sync(0xffffffffu, v[i].w, src);
+                        have_shift = true;
+                        a.moments[0] = k;
+                    }
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const bool real = DENSE || so[i] >= 0;
+                const float d0 = real ? v[i].x - k.x : 0.f, d1 = real ? v[i].y - k.y : 0.f, d2 = real ? v[i].z - k.z : 0.f, d3 = real ? v[i].w - k.w : 0.f;
+                sd.x += d0; sd.y += d1; sd.z += d2; sd.w += d3;
+                sq.x = fmaf(d0, d0, sq.x); sq.y = fmaf(d1, d1, sq.y); sq.z = fmaf(d2, d2, sq.z); sq.w = fmaf(d3, d3, sq.w);
+            }
+        }
+    }
+    if (a.moments && who) {
+        float4 t = a.moments[kMomentPlane];
+        t.x += sd.x; t.y += sd.y; t.z += sd.z; t.w += sd.w;
+        a.moments[kMomentPlane] = t;
+        t = a.moments[2 * kMomentPlane];
+        t.x += sq.x; t.y += sq.y; t.z += sq.z; t.w += sq.w;
+        a.moments[2 * kMomentPlane] = t;
+    }
+    __syncwarp();
+}
+
+// The MMA issuer (one thread).  RESIDENT: the weights of all chunks and taps stand in shared memory; otherwise a ring.
+// KIND 0: one pass; 1: hi*hi and hi*lo from one MMA over [B_hi; B_lo]; 2: three MMAs.  Everything that does not change is
+// taken out of the loops and nothing in the tap loop waits or branches on loaded values: with the modes told apart inside it
+// an MMA took 115 clocks to issue, against 40 (N = 32) the tensor core needs.
+struct MmaEnv {
+    volatile int* abort_flag;
+    uint32_t smem_base, tmem_base, a_full, a_empty, b_full, b_empty, acc_full, acc_empty;
+    int m_first, u_first, u_count;
+    int *a_used, *b_used;
+    bool drain;                  // wait until every barrier has seen its last arrival (they are used again)
+};
+template <int KIND>
+__device__ __forceinline__ void issue_tile(uint32_t acc, uint64_t a, uint64_t b, uint64_t b_half, uint32_t idesc, uint32_t idesc2, uint32_t keep)
+{
+    // (a: value or hi part, +4: lo part; +2: the chunk's second K step)
+    if (KIND == 0) {
+        umma_tf32(acc, a, b, idesc, keep);
+        umma_tf32(acc, a + 2, b + 2, idesc, 1u);
+    } else if (KIND == 1) {
+        umma_tf32(acc, a, b, idesc2, keep);
+        umma_tf32(acc, a + 4, b, idesc, 1u);
+        umma_tf32(acc, a + 2, b + 2, idesc2, 1u);
+        umma_tf32(acc, a + 6, b + 2, idesc, 1u);
+    } else {
+        const uint64_t bl = b + b_half;
+        umma_tf32(acc, a, b, idesc, keep);
+        umma_tf32(acc, a + 4, b, idesc, 1u);
+        umma_tf32(acc, a, bl, idesc, 1u);
+        umma_tf32(acc, a + 2, b + 2, idesc, 1u);
+        umma_tf32(acc, a + 6, b + 2, idesc, 1u);
+        umma_tf32(acc, a + 2, bl + 2, idesc, 1u);
+    }
+}
+template <bool RESIDENT, int KIND>
+__device__ __forceinline__ void mma_role(const PipeScalars& p, const MmaEnv& e)
+{
+    const uint64_t a_desc = smem_desc(0, 16, 1024, 128), b_desc = smem_desc(0, 16, 512, 64);
+    const uint32_t idesc = p.idesc, idesc2 = p.idesc2, acc_cols = p.acc_cols, a_step = p.a_stage_bytes >> 4, b_step = p.b_stage_bytes >> 4;
+    const uint64_t b_half = ((uint32_t)p.n_chunk * 64u) >> 4;
+    const int taps = p.taps, R = p.R, a_stages = p.a_stages, b_stages = p.b_stages, acc_bufs = p.acc_bufs, T = p.T;
+    const uint64_t row_step = (uint64_t)((p.Wp - (R - 1)) * 8);      // from a window row's last tap to the next row's first
+    const uint64_t a_first = a_desc | (uint64_t)(e.smem_base >> 4), b_first = b_desc | (uint64_t)((e.smem_base + p.off_b) >> 4);
+    int s = 0, bs = 0, buf = 0, b_it = 0, a_it = 0;
+    uint32_t apar = 0, bpar = 0, cpar = 1u;
+    if (RESIDENT) {
+        b_it = 1;
+        if (!mbar_wait(e.b_full, 0, e.abort_flag)) { report(p.status, 22); return; }
+    }
+    for (UnitWalk u(p, e.m_first, e.u_first, e.u_count); u.left > 0; u.next(p)) {
+        const int nt = u.tiles(p), kb = u.kb(p), ke = u.ke(p);
+        const uint64_t lead = (uint64_t)(span_of(p, u).lead * 8);
+        if (!mbar_wait(e.acc_empty + 8 * buf, cpar, e.abort_flag)) { report(p.status, 23); return; }
+        tc_fence_after();
+        const uint32_t acc0 = e.tmem_base + (uint32_t)(buf * T) * acc_cols;
+        uint32_t keep = 0u;
+        for (int c = kb; c < ke; ++c) {
+            if (!mbar_wait(e.a_full + 8 * s, apar, e.abort_flag)) { report(p.status, 24); return; }
+            uint64_t a = a_first + (uint64_t)((uint32_t)s * a_step) + lead;
+            uint64_t b = RESIDENT ? b_first + (uint64_t)((uint32_t)(c * taps) * b_step) : 0;
+            int sx = 0;
+            for (int tap = 0; tap < taps; ++tap) {
+                if (!RESIDENT) {
+                    if (!mbar_wait(e.b_full + 8 * bs, bpar, e.abort_flag)) { report(p.status, 25); *e.b_used = b_it; *e.a_used = a_it; return; }
+                    b = b_first + (uint64_t)((uint32_t)bs * b_step);
+                }
+                for (int t = 0; t < nt; ++t) issue_tile<KIND>(acc0 + (uint32_t)t * acc_cols, a + (uint64_t)(t * 1024), b, b_half, idesc, idesc2, keep);
+                keep = 1u;
+                if (RESIDENT) b += b_step;
+                else {
+                    umma_commit(e.b_empty + 8 * bs);
+                    ++b_it;
+                    if (++bs == b_stages) { bs = 0; bpar ^= 1u; }
+                }
+                a += 8;
+                if (++sx == R) { sx = 0; a += row_step - 8; }
+            }
+            umma_commit(e.a_empty + 8 * s);
+            ++a_it;
+            if (++s == a_stages) { s = 0; apar ^= 1u; }
+        }
+        umma_commit(e.acc_full + 8 * buf);
+        if (++buf == acc_bufs) { buf = 0; cpar ^= 1u; }
+        *e.b_used = b_it; *e.a_used = a_it;
+    }
+    if (e.drain) {
+        for (int i = 0; i < a_stages && i < a_it; ++i) mbar_wait(e.a_empty + 8 * i, (uint32_t)((a_it - 1 - i) / a_stages) & 1u, e.abort_flag);
+        if (!RESIDENT)
+            for (int i = 0; i < b_stages && i < b_it; ++i) mbar_wait(e.b_empty + 8 * i, (uint32_t)((b_it - 1 - i) / b_stages) & 1u, e.abort_flag);
+    }
+}
+
+struct PipeShared {
+    uint64_t bars[3 * kMaxA + 2 * kMaxB + 4];         // a_raw, a_full, a_empty, acc_full[2], acc_empty[2], b_full, b_empty
+    uint32_t tmem_slot;
+    int abort_flag, b_issued, b_used, a_issued, a_used;
+    int last_of_unit;
+};
+__device__ __forceinline__ void pipe_init_barriers(const PipeScalars& p, PipeShared& sh)
+{
+    const uint32_t bar = smem_u32(&sh.bars[0]);
+    for (int s = 0; s < 3 * kMaxA + 2 * kMaxB + 4; ++s) {
+        const bool full = s >= kMaxA && s < 2 * kMaxA, acc_empty = s >= 3 * kMaxA + 2 && s < 3 * kMaxA + 4;
+        mbar_init(bar + 8 * s, full ? kSplitWarps / p.split_groups : (acc_empty ? (p.epi_alternate ? kEpiWarps / 2 : kEpiWarps) : 1));
+    }
+    sh.abort_flag = 0; sh.b_issued = 0; sh.b_used = 0; sh.a_issued = 0; sh.a_used = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+}
+
+// The work of one CTA (number bid of nblk) of a launch: the barriers are initialised, tensor memory is allocated.
+// FLAT: the operand's positions and the output's pixels are the same consecutive rows (1x1 windows without a stride).
+// CELL: inside the persistent cell kernel, which keeps its tensor memory and has no successor to trigger.
+template <bool BN_IN, bool FLAT, bool CELL>
+__device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars& p, PipeShared& sh, uint8_t* smem, const uint32_t tmem_base,
+                                         const int m_first, const int m_count, const int bid, const int nblk)
+{
+    const uint32_t smem_base = smem_u32(smem);
+    const int warp = warp_index(), lane = threadIdx.x & 31;
+    uint64_t* bars = sh.bars;
+    int &abort_flag = sh.abort_flag, &b_issued = sh.b_issued, &b_used = sh.b_used, &a_issued = sh.a_issued, &a_used = sh.a_used, &last_of_unit = sh.last_of_unit;
+    const uint32_t a_raw = smem_u32(&bars[0]), a_full = smem_u32(&bars[kMaxA]), a_empty = smem_u32(&bars[2 * kMaxA]),
+                   acc_full = smem_u32(&bars[3 * kMaxA]), acc_empty = smem_u32(&bars[3 * kMaxA + 2]), b_full = smem_u32(&bars[3 * kMaxA + 4]),
+                   b_empty = smem_u32(&bars[3 * kMaxA + 4 + kMaxB]);
+    // a CTA keeps one channel slice and takes consecutive blocks of units: as many as the others or one more
+    int slice = 0, cta = bid, ctas = nblk;
+    if (p.slices > 1) { slice = cta % p.slices; cta /= p.slices; ctas /= p.slices; }
+    const int total = m_count * p.blocks_per_m * p.ksplit;
+    const int each = total / ctas, more = total - each * ctas;
+    const int u_first = cta * each + (cta < more ? cta : more), u_count = each + (cta < more ? 1 : 0);
+    const int co0 = slice * p.n_chunk;
+
+    if (warp == 0) {
+        if (elect_one()) {
+            // ---- operand copies ----
+            if (!CELL) pdl_wait();
+            const int S = p.a_stages;
+            int s = 0, it = 0;
+            uint32_t par = 1u;
+            bool live = true;
+            for (UnitWalk u(p, m_first, u_first, u_count); u.left > 0 && live; u.next(p)) {
+                const Span sp = span_of(p, u);
+                const uint32_t tx = (uint32_t)sp.rows * 64u;
+                // first block: map, row within it
+                int img0 = 0, h0 = 0, strip0 = 0;
+                if (!p.flat) {
+                    if (sp.block0 < 0) { img0 = -1; h0 = p.blocks_per_img + sp.block0; if (h0 < 0) h0 = 0; }
+                    else { img0 = div_magic(sp.block0, p.blocks_per_img, p.magic_bpi); h0 = sp.block0 - img0 * p.blocks_per_img; }
+                    if (p.strips > 1 && img0 >= 0) { const int n = div_magic(img0, p.strips, p.magic_strip); strip0 = img0 - n * p.strips; img0 = n; }
+                }
+                const int first = (int)((long long)u.m * p.pix_ms);
+                for (int c = u.kb(p), ce = u.ke(p); c < ce; ++c, ++it) {
+                    if (!mbar_wait(a_empty + 8 * s, par, &abort_flag)) { report(p.status, 20); live = false; break; }
+                    const uint32_t bar = a_raw + 8 * s;
+                    uint32_t dst = smem_base + (uint32_t)s * p.a_stage_bytes;
+                    mbar_expect_tx(bar, tx);
+                    if (p.flat) {
+                        for (int k = 0; k < sp.blocks; ++k, dst += kTileM * 128u) tma_load_2d(dst, &gp.tm_a, bar, 16 * c, first + (sp.block0 + k) * kTileM);
+                    } else {
+                        int img = img0, h = h0, strip = strip0;
+                        const uint32_t step = (uint32_t)p.box_pos * 128u;
+                        for (int k = 0; k < sp.blocks; ++k, dst += step) {
+                            // (a block beyond the last row of its map is the zero row: outside the tensor, filled with zeros)
+                            tma_load_4d(dst, &gp.tm_a, bar, 16 * c, strip * p.strip_w - p.col0, h * p.box_h, first + (img < 0 ? 0 : img));
+                            if (++h == p.blocks_per_img) { h = 0; if (img < 0 || ++strip == p.strips) { strip = 0; ++img; } }
+                        }
+                    }
+                    if (++s == S) { s = 0; par ^= 1u; }
+                }
+            }
+            a_issued = it;
+        }
+    } else if (warp == 1) {
+        if (elect_one()) {
+            // ---- weights ----
+            if (!CELL && !p.w_ready) pdl_wait();
+            const uint32_t half = (uint32_t)p.n_chunk * 64u, stage_bytes = p.b_stage_bytes, dst0 = smem_base + p.off_b;
+            const bool three = p.three != 0;
+            const uint32_t tx = three ? 2u * half : half;
+            const int taps = p.taps, c_in = p.c_in;
+            if (p.b_resident) {
+                const int n = p.n_chunks * taps;
+                mbar_expect_tx(b_full, tx * (uint32_t)n);
+                uint32_t dst = dst0;
+                for (int c = 0; c < p.n_chunks; ++c)
+                    for (int tap = 0; tap < taps; ++tap, dst += stage_bytes) {
+                        tma_load_2d(dst, &gp.tm_b, b_full, tap * c_in + 16 * c, co0);
+                        if (three) tma_load_2d(dst + half, &gp.tm_b_lo, b_full, tap * c_in + 16 * c, co0);
+                    }
+                b_issued = 1;
+            } else {
+                int s = 0, it = 0;
+                uint32_t par = 1u;
+                bool live = true;
+                for (UnitWalk u(p, m_first, u_first, u_count); u.left > 0 && live; u.next(p))
+                    for (int c = u.kb(p), ce = u.ke(p); c < ce && live; ++c)
+                        for (int tap = 0; tap < taps; ++tap, ++it) {
+                            if (!mbar_wait(b_empty + 8 * s, par, &abort_flag)) { report(p.status, 21); live = false; break; }
+                            const uint32_t bar = b_full + 8 * s, dst = dst0 + (uint32_t)s * stage_bytes;
+                            mbar_expect_tx(bar, tx);
+                            tma_load_2d(dst, &gp.tm_b, bar, tap * c_in + 16 * c, co0);
+                            if (three) tma_load_2d(dst + half, &gp.tm_b_lo, bar, tap * c_in + 16 * c, co0);
+                            if (++s == p.b_stages) { s = 0; par ^= 1u; }
+                        }
+                b_issued = it;
+            }
+        }
+    } else if (warp == 2) {
+        if (elect_one()) {
+            // ---- MMAs ----
+            const MmaEnv env{&abort_flag, smem_base, tmem_base, a_full, a_empty, b_full, b_empty, acc_full, acc_empty, m_first, u_first, u_count, &a_used, &b_used, CELL};
+            if (p.b_resident) {
+                if (!p.three) mma_role<true, 0>(p, env);
+                else if (p.stacked) mma_role<true, 1>(p, env);
+                else mma_role<true, 2>(p, env);
+            } else {
+                if (!p.three) mma_role<false, 0>(p, env);
+                else if (p.stacked) mma_role<false, 1>(p, env);
+                else mma_role<false, 2>(p, env);
+            }
+        }
+    } else if (warp >= kFirstSplit && warp < kFirstSplit + kSplitWarps) {
+        // ---- the operand: normalise, split ----
+        // The warps work on `split_groups` blocks at a time (as many as the ring holds, up to four): what a block costs is a
+        // chain of latencies - copy, shared-memory reads, arithmetic, stores, fence, hand-over - and not instructions.
+        const int tid = threadIdx.x - 32 * kFirstSplit;
+        const int groups = p.split_groups, wpg = kSplitWarps / groups, my_group = (tid >> 5) / wpg, gw = (tid >> 5) - my_group * wpg;
+        // a thread owns one 16-byte quarter of the rows row0 + row_step * j; the eight rows of a warp are taken so that a
+        // quarter-warp holds a row and the one four further on: their swizzled quarters cover all banks
+        const int row_step = 8 * wpg;
+        const int cph = lane & 3, r8 = ((lane >> 2) & 1) * 4 + (lane >> 3), row0 = gw * 8 + r8;
+        const uint32_t at_hi = (uint32_t)row0 * 128u + (uint32_t)((cph ^ r8) << 4), at_lo = (uint32_t)row0 * 128u + (uint32_t)(((cph + 4) ^ r8) << 4);
+        const uint32_t byte_step = (uint32_t)row_step * 128u;
+        const int S = p.a_stages, C = p.c_in, halo = p.halo;
+        const bool three = p.three != 0;
+        float* tab = reinterpret_cast<float*>(smem + p.off_bn);
+        if (BN_IN) {
+            for (int i = tid; i < C; i += kSplitThreads) { tab[2 * C + i] = __ldg(p.bn_gamma + i); tab[3 * C + i] = __ldg(p.bn_beta + i); }
+            if (!CELL) pdl_wait();
+        }
+        // a step of row_step positions in maps, rows and columns of the padded grid
+        const int dn = BN_IN && !FLAT ? row_step / p.img_pos : 0, drem = row_step - dn * p.img_pos;
+        const int dy = BN_IN && !FLAT ? drem / p.Wp : 0, dx = drem - dy * p.Wp, Hp = BN_IN && !FLAT ? p.img_pos / p.Wp : 1;
+        int s = 0, turn = 0, cur_m = -1;
+        uint32_t par = 0;
+        const bool store_y = BN_IN && slice == 0;
+        bool ok = true;
+        for (UnitWalk cu(p, m_first, u_first, u_count); cu.left > 0; cu.next(p)) {
+            const int kb = cu.kb(p), ke = cu.ke(p);
+            const Span sp = span_of(p, cu);
+            const int own_lo = sp.lead + halo, own_hi = own_lo + cu.tiles(p) * kTileM, valid = p.pos_per_m - sp.pos0;
+            if (BN_IN) {
+                if (cu.m != cur_m) {
+                    cur_m = cu.m;
+                    split_sync();                     // everybody is done with the table of the micro-batch before
+                    merge_moments<kSplitThreads>(p.bn_partials + (size_t)cur_m * partial_floats(p.bn_units, C), p.bn_units, C, p.bn_inv_rows, p.bn_eps, tab,
+                                  reinterpret_cast<float4*>(smem + p.off_red), tid);
+                    split_sync();
+                }
+                if (slice == 0 && cu.ul == 0 && cu.z == 0)
+                    for (int i = tid; i < 2 * C; i += kSplitThreads) p.bn_stats[(size_t)cur_m * 2 * C + i] = tab[i];
+            }
+            for (int c = kb; c < ke; ++c) {
+                if (turn == my_group) {
+                    ok = mbar_wait(a_raw + 8 * s, par, &abort_flag) && ok;
+                    // (after a wait that gave up the warps run through the rest without waiting: they still have to meet at
+                    // the named barriers)
+                    if (!ok && lane == 0) report(p.status, 26);
+                    uint8_t* hi = smem + (uint32_t)s * p.a_stage_bytes + at_hi;
+                    uint8_t* lo = smem + (uint32_t)s * p.a_stage_bytes + at_lo;
+                    if (BN_IN) {
+                        const int ch = 16 * c + 4 * cph;
+                        const float4 mu = *reinterpret_cast<const float4*>(tab + ch), rs = *reinterpret_cast<const float4*>(tab + C + ch);
+                        const float4 g = *reinterpret_cast<const float4*>(tab + 2 * C + ch), b = *reinterpret_cast<const float4*>(tab + 3 * C + ch);
+                        float* ydst = p.bn_y + (long long)cur_m * p.in_ms + 16 * c + 4 * cph;
+                        int yo = (sp.pos0 + row0) * C;                   // FLAT: offset of this thread's first row
+                        int pn = 0, py = 0, px = 0;                      // otherwise its map, row and column
+                        if (!FLAT) {
+                            int pos = sp.pos0 + row0;
+                            if (pos < 0) { pos += p.img_pos; pn = -1; }
+                            const int q = div_magic(pos, p.img_pos, p.magic_img);
+                            pn += q; pos -= q * p.img_pos;
+                            py = div_magic(pos, p.Wp, p.magic_w); px = pos - py * p.Wp;
+                        }
+                        // four rows in flight; the block is allocated in whole batches, so the last one needs no bounds
+                        for (int row = row0; row < sp.rows; row += kRowBatch * row_step, hi += kRowBatch * byte_step, lo += kRowBatch * byte_step) {
+                            float4 v[kRowBatch];
+#pragma unroll
+                            for (int j = 0; j < kRowBatch; ++j) v[j] = *reinterpret_cast<const float4*>(hi + byte_step * j);
+                            int off[kRowBatch];
+                            bool inside[kRowBatch], own[kRowBatch];
+#pragma unroll
+                            for (int j = 0; j < kRowBatch; ++j) {
+                                const int r = row + row_step * j;
+                                if (FLAT) {
+                                    inside[j] = own[j] = r < valid;
+                                    off[j] = yo; yo += row_step * C;
+                                } else if (p.strips > 1) {
+                                    const Pixel w = locate(p, sp.pos0 + r);
+                                    inside[j] = w.in; own[j] = w.own && r >= own_lo && r < own_hi;
+                                    off[j] = w.n * p.in_sn + w.y * p.in_sh + w.x * p.in_sw;
+                                } else {
+                                    inside[j] = px < p.W && py < p.Hv && pn >= 0 && r < valid;
+                                    own[j] = inside[j] && r >= own_lo && r < own_hi;
+                                    off[j] = pn * p.in_sn + py * p.in_sh + px * p.in_sw;
+                                    px += dx; py += dy; pn += dn;
+                                    if (px >= p.Wp) { px -= p.Wp; ++py; }
+                                    if (py >= Hp) { py -= Hp; ++pn; }
+                                }
+                            }
+#pragma unroll
+                            for (int j = 0; j < kRowBatch; ++j) {
+                                v[j].x = fmaxf(fmaf(g.x, (v[j].x - mu.x) * rs.x, b.x), 0.f);
+                                v[j].y = fmaxf(fmaf(g.y, (v[j].y - mu.y) * rs.y, b.y), 0.f);
+                                v[j].z = fmaxf(fmaf(g.z, (v[j].z - mu.z) * rs.z, b.z), 0.f);
+                                v[j].w = fmaxf(fmaf(g.w, (v[j].w - mu.w) * rs.w, b.w), 0.f);
+                                if (!inside[j]) v[j] = make_float4(0.f, 0.f, 0.f, 0.f);      // the padding is zero AFTER the activation
+                                *reinterpret_cast<float4*>(hi + byte_step * j) = v[j];
+                            }
+                            if (three)
+#pragma unroll
+                                for (int j = 0; j < kRowBatch; ++j)
+                                    *reinterpret_cast<float4*>(lo + byte_step * j) =
+                                        make_float4(v[j].x - tf32_hi(v[j].x), v[j].y - tf32_hi(v[j].y), v[j].z - tf32_hi(v[j].z), v[j].w - tf32_hi(v[j].w));
+                            if (store_y)
+#pragma unroll
+                                for (int j = 0; j < kRowBatch; ++j) if (own[j]) *reinterpret_cast<float4*>(ydst + off[j]) = v[j];
+                        }
+                    } else if (three) {
+                        for (int row = row0; row < sp.rows; row += kRowBatch * row_step, hi += kRowBatch * byte_step, lo += kRowBatch * byte_step) {
+                            float4 v[kRowBatch];
+#pragma unroll
+                            for (int j = 0; j < kRowBatch; ++j) v[j] = *reinterpret_cast<const float4*>(hi + byte_step * j);
+#pragma unroll
+                            for (int j = 0; j < kRowBatch; ++j)
+                                *reinterpret_cast<float4*>(lo + byte_step * j) =
+                                    make_float4(v[j].x - tf32_hi(v[j].x), v[j].y - tf32_hi(v[j].y), v[j].z - tf32_hi(v[j].z), v[j].w - tf32_hi(v[j].w));
+                        }
+                    }
+                    fence_async_smem();               // generic-proxy writes -> tensor-core reads
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(a_full + 8 * s);
+                }
+                if (++turn == groups) turn = 0;
+                if (++s == S) { s = 0; par ^= 1u; }
+            }
+        }
+    } else if (warp >= kFirstSplit + kSplitWarps) {
+        // ---- write-out: tensor memory -> registers -> a 32 x 32 patch of shared memory -> global memory ----
+        // A TMEM lane is a position, so stores straight from the registers touch 32 lines per instruction (measured: half a
+        // sector per clock and SM); through a warp's own patch eight lanes write a row's 128 bytes, and a thread that keeps
+        // four columns forms their moments without crossing lanes.
+        const int tid = threadIdx.x - 32 * (kFirstSplit + kSplitWarps), ew = warp - kFirstSplit - kSplitWarps;
+        const int quad = warp & 3, half = ew >> 2;    // a warp reads the 32 lanes of its quadrant; two warps share one
+        const int n_chunk = p.n_chunk, groups = (n_chunk + 31) >> 5, T = p.T, C_out = p.c_out, ksplit = p.ksplit;
+        const bool stacked = p.stacked != 0, stats = p.st_partials != nullptr;
+        // Two sets of four warps.  With two accumulator sets and at most 64 channels each takes every other unit, so that the
+        // latencies of one unit's write-out run beside the other's; otherwise they share a unit: alternate groups of 32
+        // channels, or alternate tiles where there is one group.
+        const bool alternate = p.epi_alternate != 0, by_tile = !alternate && groups == 1, whole = alternate || by_tile;
+        const int g_first = whole ? 0 : half, g_step = whole ? 1 : 2, t_first = by_tile ? half : 0, t_step = by_tile ? 2 : 1;
+        const int parts = whole ? 8 : 4, part = whole ? ew : quad;
+        int turn = 0;
+        float4* patch = reinterpret_cast<float4*>(smem + p.off_stage) + ew * 256;
+        if (!CELL) pdl_wait();
+        int buf = alternate ? half : 0, flip = 0;
+        uint32_t par = 0;
+        // moments of the block so far: this lane's columns in shared memory, rows counted per warp
+        float4* mom = reinterpret_cast<float4*>(smem + p.off_stat) + ew * 64 + lane;
+        unsigned int have_mask = 0;
+        int count = 0;
+        if (stats)
+            for (int gi = 0; gi < 2; ++gi) { mom[gi * 32 + kMomentPlane] = make_float4(0.f, 0.f, 0.f, 0.f); mom[gi * 32 + 2 * kMomentPlane] = make_float4(0.f, 0.f, 0.f, 0.f); }
+        for (UnitWalk u(p, m_first, u_first, u_count); u.left > 0; u.next(p)) {
+            bool finish = true, ok = true;
+            if (!alternate || turn == half) {
+            const int nt = u.tiles(p);
+            // this lane's row of every tile, and which neighbours of a strided data gradient's sample get zeros
+            int roff[4], fill = 0;
+#pragma unroll
+            for (int t = 0; t < 4; ++t)
+                if (t < nt) {
+                    const int pos = (u.ul * T + t) * kTileM + quad * 32 + lane;
+                    if (FLAT) { roff[t] = pos < p.pos_per_m ? pos * C_out + co0 : -1; continue; }
+                    const Pixel px = locate(p, pos);
+                    roff[t] = px.own ? px.n * p.os_n + px.y * p.os_h + px.x * p.os_w + co0 : -1;
+                    if (p.zero_fill == 2 && px.own) {
+                        const bool right = 2 * px.x + 1 < p.out_w, below = 2 * px.y + 1 < p.out_h;
+                        fill |= ((right ? 1 : 0) | (below ? 2 : 0) | (right && below ? 4 : 0)) << (4 * t);
+                    }
+                }
+            float* out = p.out + (long long)u.m * p.out_ms;
+            const float* extra = p.extra ? p.extra + (long long)u.m * p.out_ms : nullptr;
+            ok = mbar_wait(acc_full + 8 * buf, par, &abort_flag);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok && lane == 0) report(p.status, 27);
+            if (!CELL && p.pdl_late && u.last(p)) pdl_launch_dependents();
+            tc_fence_after();
+            const uint32_t acc0 = tmem_base + (uint32_t)(buf * T) * p.acc_cols + ((uint32_t)(quad * 32) << 16);
+            // 16 columns of this lane's row, hi and lo products added
+            auto accumulator = [&](int t, int col, float* v) {
+                const uint32_t at = acc0 + (uint32_t)t * p.acc_cols + (uint32_t)col;
+                tmem_ld16_nowait(at, v);
+                if (stacked) {
+                    float w[16];
+                    tmem_ld16_nowait(at + (uint32_t)n_chunk, w);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) v[j] += w[j];
+                } else {
+                    tmem_ld_wait();
+                }
+            };
+            finish = true;
+            const float* sk_all = nullptr;
+            const size_t sk_tile = (size_t)kTileM * n_chunk;
+            if (ksplit > 1) {
+                // this CTA's partial sums; the CTA that takes the last ticket of the unit adds them in split order
+                const size_t key = (size_t)u.ul * p.slices + slice;
+                char* base = p.sk_base + u.m * p.sk_ms;
+                unsigned int* ticket = reinterpret_cast<unsigned int*>(base) + key;
+                float* partials = reinterpret_cast<float*>(base + kSplitKTicketBytes);
+                sk_all = partials + key * ksplit * T * sk_tile;
+                float* mine = partials + (key * ksplit + u.z) * T * sk_tile;
+                for (int g = g_first; g < groups; g += g_step)
+                    for (int t = t_first; t < nt; t += t_step)
+                        for (int h = 2 * g; h < 2 * g + 2 && 16 * h < n_chunk; ++h) {
+                            float v[16];
+                            accumulator(t, 16 * h, v);
+                            if (ok) store16(mine + t * sk_tile + ((size_t)h * kTileM + quad * 32 + lane) * 16, v);
+                        }
+                __threadfence();
+                epi_sync();
+                if (tid == 0) {
+                    last_of_unit = atomicAdd(ticket, 1u) == (unsigned int)ksplit - 1u;
+                    if (last_of_unit) *ticket = 0u;
+                }
+                epi_sync();
+                finish = last_of_unit != 0;
+                if (finish) __threadfence();
+            }
+            if (finish)
+                for (int g = g_first, gi = 0; g < groups; g += g_step, ++gi) {
+                    const bool full = n_chunk - 32 * g >= 32;
+                    for (int t = t_first; t < nt; t += t_step) {
+                        const int ro = t == 0 ? roff[0] : (t == 1 ? roff[1] : (t == 2 ? roff[2] : roff[3]));
+                        // 16 columns of the row into the patch; the next 16 are on their way while these are stored
+                        const uint32_t at = acc0 + (uint32_t)t * p.acc_cols + (uint32_t)(32 * g);
+                        auto to_patch = [&](int h, const float* v) {
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) patch[lane * 8 + ((4 * h + j) ^ (lane & 7))] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+                        };
+                        auto stage = [&](auto width) {
+                            constexpr int H = decltype(width)::value / 16;
+                            float v[16], w[16];
+                            if (ksplit > 1) {
+                                for (int h = 0; h < H; ++h) {
+#pragma unroll
+                                    for (int j = 0; j < 16; ++j) v[j] = 0.f;
+                                    for (int z = 0; z < ksplit; ++z) {
+                                        load16(sk_all + ((size_t)z * T + t) * sk_tile + ((size_t)(2 * g + h) * kTileM + quad * 32 + lane) * 16, w);
+#pragma unroll
+                                        for (int j = 0; j < 16; ++j) v[j] += w[j];
+                                    }
+                                    to_patch(h, v);
+                                }
+                            } else if (stacked) {
+                                tmem_ld16_nowait(at, v);
+                                tmem_ld16_nowait(at + (uint32_t)n_chunk, w);
+                                tmem_ld_wait();
+#pragma unroll
+                                for (int j = 0; j < 16; ++j) v[j] += w[j];
+                                if (H == 2) {
+                                    float x[16];
+                                    tmem_ld16_nowait(at + 16u, x);
+                                    tmem_ld16_nowait(at + (uint32_t)n_chunk + 16u, w);
+                                    to_patch(0, v);
+                                    tmem_ld_wait();
+#pragma unroll
+                                    for (int j = 0; j < 16; ++j) v[j] = x[j] + w[j];
+                                    to_patch(1, v);
+                                } else {
+                                    to_patch(0, v);
+                                }
+                            } else {
+                                tmem_ld16_nowait(at, v);
+                                if (H == 2) tmem_ld16_nowait(at + 16u, w);
+                                tmem_ld_wait();
+                                to_patch(0, v);
+                                if (H == 2) to_patch(1, w);
+                            }
+                        };
+                        const EmitArgs ea{out + 32 * g, extra ? extra + 32 * g : nullptr, patch, stats ? mom + gi * 32 : nullptr, p.accumulate != 0, ok,
+                                          p.zero_fill == 2 ? fill >> (4 * t) : 0, p.zero_fill == 2, p.dense_h, p.dense_w, C_out};
+                        const bool have = (have_mask >> gi) & 1u;
+                        const auto go32 = [&] { stage(std::integral_constant<int, 32>()); };
+                        const auto go16 = [&] { stage(std::integral_constant<int, 16>()); };
+                        if (FLAT && (u.ul * T + t) * kTileM + quad * 32 + 32 <= p.pos_per_m) {
+                            if (full) emit_rows<8, true>(ea, ro, lane, have, go32);
+                            else emit_rows<4, true>(ea, ro, lane, have, go16);
+                            if (stats) { have_mask |= 1u << gi; if (gi == 0) count += 32; }
+                        } else {
+                            if (full) emit_rows<8, false>(ea, ro, lane, have, go32);
+                            else emit_rows<4, false>(ea, ro, lane, have, go16);
+                            if (stats) {
+                                const int n = __popc(__ballot_sync(0xffffffffu, ro >= 0));
+                                if (n) have_mask |= 1u << gi;
+                                if (gi == 0) count += n;
+                            }
+                        }
+                    }
+                }
+            // the accumulator is read: the next unit's MMAs may have it
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(acc_empty + 8 * buf);
+            if (alternate) par ^= 1u;                 // (a set of warps always meets its own accumulator set)
+            else if (++buf == p.acc_bufs) { buf = 0; par ^= 1u; }
+            }
+            turn ^= 1;
+            if (stats && finish && (ksplit > 1 || u.last_of_block())) {
+                // the block's moments: lanes, then the warps' parts, each about its own shift
+                float* contrib = reinterpret_cast<float*>(smem + p.off_stat + 3u * 16u * kMomentPlane) + (size_t)flip * parts * (3 * n_chunk + 1);
+                for (int g = g_first, gi = 0; g < groups; g += g_step, ++gi) {
+                    const int lpr = n_chunk - 32 * g >= 32 ? 8 : 4;
+                    float4 sd = mom[gi * 32 + kMomentPlane], sq = mom[gi * 32 + 2 * kMomentPlane];
+                    const float4 k = mom[gi * 32], zero = make_float4(0.f, 0.f, 0.f, 0.f);
+                    mom[gi * 32 + kMomentPlane] = zero; mom[gi * 32 + 2 * kMomentPlane] = zero;
+                    for (int o = 16; o >= lpr; o >>= 1) {
+                        sd.x += __shfl_xor_sync(0xffffffffu, sd.x, o); sd.y += __shfl_xor_sync(0xffffffffu, sd.y, o);
+                        sd.z += __shfl_xor_sync(0xffffffffu, sd.z, o); sd.w += __shfl_xor_sync(0xffffffffu, sd.w, o);
+                        sq.x += __shfl_xor_sync(0xffffffffu, sq.x, o); sq.y += __shfl_xor_sync(0xffffffffu, sq.y, o);
+                        sq.z += __shfl_xor_sync(0xffffffffu, sq.z, o); sq.w += __shfl_xor_sync(0xffffffffu, sq.w, o);
+                    }
+                    if (lane < lpr) {
+                        float* c3 = contrib + (size_t)part * 3 * n_chunk + 32 * g + 4 * lane;
+                        *reinterpret_cast<float4*>(c3) = k;
+                        *reinterpret_cast<float4*>(c3 + n_chunk) = sd;
+                        *reinterpret_cast<float4*>(c3 + 2 * n_chunk) = sq;
+                    }
+                }
+                float* counts = contrib + (size_t)parts * 3 * n_chunk;
+                if (lane == 0 && (whole || half == 0)) counts[part] = (float)count;
+                count = 0; have_mask = 0;
+                epi_sync();
+                if (tid < n_chunk) {
+                    float N = 0.f, k0 = 0.f, sum = 0.f, m2 = 0.f;
+                    for (int w = 0; w < parts; ++w)
+                        if (counts[w] > 0.f) {
+                            const float k = contrib[(size_t)w * 3 * n_chunk + tid];
+                            if (N == 0.f) k0 = k;
+                            N += counts[w];
+                            sum += fmaf(counts[w], k - k0, contrib[(size_t)w * 3 * n_chunk + n_chunk + tid]);
+                        }
+                    const float dm = N > 0.f ? sum / N : 0.f;
+                    for (int w = 0; w < parts; ++w)
+                        if (counts[w] > 0.f) {
+                            const float n = counts[w], d = contrib[(size_t)w * 3 * n_chunk + n_chunk + tid], e = d / n;
+                            const float away = contrib[(size_t)w * 3 * n_chunk + tid] - k0 + e - dm;
+                            m2 += contrib[(size_t)w * 3 * n_chunk + 2 * n_chunk + tid] - d * e + n * away * away;
+                        }
+                    float* dst = p.st_partials + (size_t)u.m * partial_floats(p.blocks_per_m, C_out);
+                    const int r = u.ul / p.unit_block;
+                    float* row = dst + (size_t)r * 2 * C_out + co0 + tid;
+                    if (ok) { row[0] = k0 + dm; row[C_out] = m2; }
+                    if (tid == 0 && slice == 0 && ok) dst[(size_t)p.blocks_per_m * 2 * C_out + r] = N;
+                }
+                flip ^= 1;
+            }
+        }
+    }
+
+    // ---- teardown ----
+    tc_fence_before();
+    __syncthreads();
+    if (abort_flag && threadIdx.x == 0) {
+        // copies still in flight must land before the shared memory is given back
+        for (int it = a_used; it < a_issued; ++it) {
+            const long long t0 = clock64();
+            while (!mbar_try_wait(a_raw + 8 * (it % p.a_stages), (uint32_t)(it / p.a_stages) & 1u) && clock64() - t0 < kWaitLimit) {}
+        }
+        for (int it = b_used; it < b_issued; ++it) {
+            const int s = p.b_resident ? 0 : it % p.b_stages;
+            const uint32_t parity = p.b_resident ? 0u : (uint32_t)(it / p.b_stages) & 1u;
+            const long long t0 = clock64();
+            while (!mbar_try_wait(b_full + 8 * s, parity) && clock64() - t0 < kWaitLimit) {}
+        }
+    }
+    __syncthreads();
+}
+
+template <bool BN_IN, bool FLAT>
+__global__ void __launch_bounds__(kPipeThreads, 1) conv_pipe_kernel(const __grid_constant__ PipeParams gp, const int m_first, const int m_count)
+{
+    const PipeScalars& p = gp.s;
+    {
+        // The scalar parameters span several lines of the constant cache: one warp touches them all at once, so that the
+        // roles do not meet the misses one after the other.
+        const uint32_t* w = reinterpret_cast<const uint32_t*>(&gp.s);
+        uint32_t x = 0;
+        if (threadIdx.x < 32)
+            for (int i = threadIdx.x; i < (int)(sizeof(PipeScalars) / 4); i += 32) x |= w[i];
+        asm volatile("" ::"r"(x));
+    }
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ PipeShared sh;
+    uint8_t* smem = smem_raw + (((smem_u32(smem_raw) + 1023u) & ~1023u) - smem_u32(smem_raw));
+    if (threadIdx.x == 0) pipe_init_barriers(p, sh);
+    if (threadIdx.x == 32) { prefetch_tmap(&gp.tm_a); prefetch_tmap(&gp.tm_b); prefetch_tmap(&gp.tm_b_lo); }
+    if (warp_index() == 0) tmem_alloc(smem_u32(&sh.tmem_slot), p.tmem_cols);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    // The successor may be scheduled from here on: not before this CTA holds its tensor memory, or the successor's CTA could
+    // take the columns this one needs and wait for this one to finish.
+    if (!p.pdl_late) pdl_launch_dependents();
+    const uint32_t tmem_base = sh.tmem_slot;
+    pipe_cta<BN_IN, FLAT, false>(gp, p, sh, smem, tmem_base, m_first, m_count, (int)blockIdx.x, (int)gridDim.x);
+    if (warp_index() == 0) tmem_dealloc(tmem_base, p.tmem_cols);
+}
+
+// ------------------------------------------------------------------------------------------------
+// persistent cells: the forward convolutions of a cell in ONE resident grid
+// ------------------------------------------------------------------------------------------------
+// A fixed grid stays resident for the whole cell and walks the list of launches: its CTAs take the place of each launch's
+// CTAs, run the same code, and meet at a grid-wide barrier before the next launch, whose input the whole grid has just
+// produced.  Every CTA must be resident at the same time; the host sizes the grids so that all cells that can run
+// concurrently fit the GPU together.  The barrier wait is bounded like every other wait here.
+struct CellOp {
+    PipeParams p;                // exactly what the stand-alone launch would receive
+    int bn_in, flat;             // which kernel it would be
+};
+struct CellParams {
+    const CellOp* ops;           // device memory, written before the launch and read-only for the kernel
+    int n_ops;
+    unsigned int* barrier;       // {arrivals, generation}: zero before the first use, left with arrivals at zero
+    DeviceStatus* status;
+    unsigned int tmem_cols;      // the largest accumulators of the list
+};
+
+__device__ __forceinline__ unsigned int ld_acquire_gpu(const unsigned int* ptr)
+{
+    unsigned int v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(ptr) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_release_gpu(unsigned int* ptr, unsigned int v)
+{
+    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(ptr), "r"(v) : "memory");
+}
+
+// All CTAs of the grid arrive; the last one opens the next generation.  What the CTAs wrote before the barrier is visible to
+// all of them after it, also to copies issued through the async proxy (TMA).  Returns false when the wait ran out or another
+// kernel already reported a failure.
+__device__ __forceinline__ bool cell_grid_barrier(unsigned int* bar, DeviceStatus* status, int* stop_flag)
+{
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const unsigned int gen = ld_acquire_gpu(bar + 1);      // cannot advance before this CTA has arrived
+        __threadfence();
+        int stop = 0;
+        if (atomicAdd(bar, 1u) == gridDim.x - 1) {
+            bar[0] = 0u;
+            __threadfence();
+            st_release_gpu(bar + 1, gen + 1u);
+        } else {
+            const long long t0 = clock64();
+            int polls = 0;
+            while (ld_acquire_gpu(bar + 1) == gen) {
+                if ((++polls & 63) == 0 && (clock64() - t0 > kWaitLimit || ld_acquire_gpu(&status->code) != 0u)) { report(status, 9); stop = 1; break; }
+            }
+        }
+        *stop_flag = stop;
+    }
+    __syncthreads();
+    asm volatile("fence.proxy.async;" ::: "memory");
+    return *stop_flag == 0;
+}
+
+__global__ void __launch_bounds__(kPipeThreads, 1) conv_pipe_cell_kernel(const __grid_constant__ CellParams cp, const int m_first, const int m_count)
+{
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ PipeShared sh;
+    __shared__ PipeScalars p;
+    __shared__ int cell_stop;
+    constexpr int kWords = (int)(sizeof(PipeScalars) / 4);
+    static_assert(sizeof(PipeScalars) % 4 == 0 && kWords <= kPipeThreads, "one parameter word per thread");
+    uint8_t* smem = smem_raw + (((smem_u32(smem_raw) + 1023u) & ~1023u) - smem_u32(smem_raw));
+    const int tid = threadIdx.x;
+    if (warp_index() == 0) tmem_alloc(smem_u32(&sh.tmem_slot), cp.tmem_cols);
+    if (tid == 0) { cell_stop = 0; sh.abort_flag = 0; }
+    // one word of the parameters per thread: the first launch's now, the next one's while the current one runs
+    uint32_t nxt = tid < kWords ? __ldg(reinterpret_cast<const uint32_t*>(&cp.ops[0].p.s) + tid) : 0u;
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = sh.tmem_slot;
+    bool first = true;
+    for (int op = 0; op < cp.n_ops; ++op) {
+        if (tid < kWords) reinterpret_cast<uint32_t*>(&p)[tid] = nxt;
+        if (op + 1 < cp.n_ops && tid < kWords) nxt = __ldg(reinterpret_cast<const uint32_t*>(&cp.ops[op + 1].p.s) + tid);
+        __syncthreads();
+        const PipeParams& gp = cp.ops[op].p;
+        const int bn_in = __ldg(&cp.ops[op].bn_in), flat = __ldg(&cp.ops[op].flat);
+        const int tasks = m_count * p.blocks_per_m * p.ksplit;
+        int per_slice = (int)gridDim.x / p.slices;
+        if (per_slice < 1) per_slice = 1;
+        if (per_slice > tasks) per_slice = tasks;
+        const int V = per_slice * p.slices;
+        for (int v = blockIdx.x; v < V; v += gridDim.x) {
+            // the barriers of the call before have seen their last arrival: they start over
+            if (tid == 0) {
+                if (!first)
+                    for (int i = 0; i < 3 * kMaxA + 2 * kMaxB + 4; ++i) mbar_inval(smem_u32(&sh.bars[i]));
+                pipe_init_barriers(p, sh);
+            }
+            first = false;
+            __syncthreads();
+            tc_fence_after();
+            if (bn_in) {
+                if (flat) pipe_cta<true, true, true>(gp, p, sh, smem, tmem_base, m_first, m_count, v, V);
+                else pipe_cta<true, false, true>(gp, p, sh, smem, tmem_base, m_first, m_count, v, V);
+            } else {
+                if (flat) pipe_cta<false, true, true>(gp, p, sh, smem, tmem_base, m_first, m_count, v, V);
+                else pipe_cta<false, false, true>(gp, p, sh, smem, tmem_base, m_first, m_count, v, V);
+            }
+            if (sh.abort_flag) { if (tid == 0) cell_stop = 1; break; }
+        }
+        if (sh.abort_flag || (op + 1 < cp.n_ops && !cell_grid_barrier(cp.barrier, cp.status, &cell_stop))) break;
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp_index() == 0) tmem_dealloc(tmem_base, cp.tmem_cols);
+}
+
+// Statistics for a BN that runs a kernel of its own although its input came from a convolution that left moments.
+__global__ void __launch_bounds__(256) bn_finalize_kernel(const float* __restrict__ partials, int units, int C, double inv_rows, float eps, float* stats)
+{
+    extern __shared__ float4 dyn[];                   // 3 x 256 float4, then the table
+    float* tab = reinterpret_cast<float*>(dyn + 768);
+    const int m = blockIdx.x;
+    pdl_launch_dependents();
+    pdl_wait();
+    merge_moments<256>(partials + (size_t)m * partial_floats(units, C), units, C, inv_rows, eps, tab, dyn, threadIdx.x);
+    __syncthreads();
+    for (int i = threadIdx.x; i < 2 * C; i += 256) stats[(size_t)m * 2 * C + i] = tab[i];
+}
+
+// Forward pass, or the data gradient seen as a forward problem.
+struct PipeView {
+    int P, Q;                    // output grid of the GEMM
+    int c_in, c_out;
+    int in_W, in_H;              // input pixels the positions may touch
+    int in_sw, in_sh, in_sn, os_w, os_h, os_n, zero_fill, out_h, out_w, dense_h, dense_w;
+    long long in_ms, out_ms;
+};
+
+bool pipe_view(const ConvShape& s, int pass, PipeView* v)
+{
+    if (s.C % 16 || s.K % 16) return false;
+    if (s.R == 3 ? (s.stride != 1 || s.pad != 1) : (s.R != 1 || s.pad != 0)) return false;
+    if (s.stride < 1 || s.stride > 2) return false;
+    const long long x = (long long)s.N * s.H * s.W * s.C, y = (long long)s.N * s.P * s.Q * s.K;
+    if (x >= (1LL << 31) || y >= (1LL << 31)) return false;        // 32-bit offsets inside a micro-batch
+    if (pass == PASS_FWD) {
+        v->P = s.P; v->Q = s.Q; v->c_in = s.C; v->c_out = s.K;
+        v->in_W = s.Q; v->in_H = s.P;                              // in steps of the stride
+        v->in_sw = s.stride * s.C; v->in_sh = s.stride * s.W * s.C; v->in_sn = s.H * s.W * s.C;
+        v->os_w = s.K; v->os_h = s.Q * s.K; v->os_n = s.P * s.Q * s.K;
+        v->zero_fill = 1; v->out_h = s.P; v->out_w = s.Q; v->dense_h = v->os_h; v->dense_w = v->os_w;
+        v->in_ms = x; v->out_ms = y;
+    } else {
+        v->P = s.P; v->Q = s.Q; v->c_in = s.K; v->c_out = s.C;
+        v->in_W = s.Q; v->in_H = s.P;
+        v->in_sw = s.K; v->in_sh = s.Q * s.K; v->in_sn = s.P * s.Q * s.K;
+        v->dense_w = s.C; v->dense_h = s.W * s.C;
+        v->os_w = s.stride * s.C; v->os_h = s.stride * s.W * s.C; v->os_n = s.H * s.W * s.C;
+        v->zero_fill = s.stride; v->out_h = s.H; v->out_w = s.W;
+        v->in_ms = y; v->out_ms = x;
+    }
+    return true;
+}
+
+int sm_count()
+{
+    static const int n = [] {
+        int dev = 0, v = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) { (void)cudaGetLastError(); return 148; }
+        return v;
+    }();
+    return n;
+}
+
+constexpr int kPlanSms = 148;                         // the split of the work is planned for a whole B200, with or without a device at hand
+inline unsigned int stat_bytes(int n_chunk) { return 3u * 16u * kMomentPlane + (unsigned int)(2 * (n_chunk <= 64 ? 8 : 4) * (3 * n_chunk + 1) * 4 + 127) & ~127u; }
+inline unsigned int bn_bytes(int c_in) { return (unsigned int)(4 * c_in * 4 + 3 * kSplitThreads * 16); }
+
+}  // namespace
+
+size_t conv_pipe_partial_floats(int units_per_m, int channels) { return partial_floats(units_per_m, channels); }
+
+bool conv_pipe_geom(const ConvShape& s, int pass, int passes, int M, ConvPipeGeom* g)
+{
+    PipeView v;
+    if (pass == PASS_WGRAD || !pipe_view(s, pass, &v)) return false;
+    const bool three = passes == 3;
+    // Channel slices of 128 beyond 128 channels: a unit of 256 positions x 128 channels reads half as many weight bytes from
+    // L2 per MMA as 128 positions x 256 channels do.
+    g->n_chunk = v.c_out <= 128 ? v.c_out : (v.c_out % 128 == 0 ? 128 : (v.c_out <= 256 ? v.c_out : 0));
+    if (!g->n_chunk) return false;
+    g->slices = v.c_out / g->n_chunk;
+    g->strips = 1; g->col0 = 0; g->strip_w = v.Q; g->halo = 0; g->Wp = v.Q; g->Hp = v.P;
+    if (s.R == 3) {
+        g->Wp = v.Q + 1; g->Hp = v.P + 1;
+        if (v.Q > 254) {
+            g->strips = (v.Q + 251) / 252;
+            g->strip_w = (v.Q + g->strips - 1) / g->strips;
+            g->Wp = g->strip_w + 2; g->col0 = 1;
+        }
+        g->halo = g->Wp + 1;
+    }
+    g->flat = s.R == 1 && (s.stride == 1 || pass == PASS_DGRAD) ? 1 : 0;
+    if (!g->flat && g->Wp > 256) return false;
+    // one copy per padded map row, or per whole map where that is no more than 40 positions
+    g->box_h = g->Wp * g->Hp <= 40 ? g->Hp : 1;
+    const int bp = g->flat ? kTileM : g->box_h * g->Wp;
+    const long long pos = (long long)s.N * g->strips * g->Wp * g->Hp;
+    if (pos >= (1LL << 30)) return false;
+    g->pos_per_m = (int)pos;
+    g->tiles_per_m = (g->pos_per_m + kTileM - 1) / kTileM;
+    const int taps = s.R * s.R, chunks = v.c_in / 16, n = g->n_chunk;
+    g->b_stage_bytes = (unsigned int)(three ? 2 : 1) * (unsigned int)n * 64u;
+    const unsigned int all_b = g->b_stage_bytes * (unsigned int)(taps * chunks);
+    const unsigned int fixed = kEpiWarps * 4096u + stat_bytes(n) + (pass == PASS_FWD ? bn_bytes(v.c_in <= 512 ? v.c_in : 0) : 0u);
+    // Tiles per unit, stacked weights (hi*hi and hi*lo from one MMA over [B_hi; B_lo]) and accumulator sets: the combination
+    // with the least modelled time for the busiest CTA.  Clocks per MMA (K = 8) as measured alone; at 128 columns an unstacked
+    // MMA reads 128 bytes of shared memory per clock, all there is, and pays for every other access; operand and weight
+    // bytes at 20 and 28 per clock and SM; about 350 clocks per 128 x 32 outputs written.
+    auto clk = [](int c) { return c <= 32 ? 40.0 : (c <= 64 ? 48.0 : (c <= 96 ? 58.0 : (c <= 128 ? 68.0 : 0.5 * c))); };
+    double best = 0.0;
+    g->T = 0;
+    for (int T = 4; T >= 1; T >>= 1)
+        for (int stacked = three && 2 * n <= 256 ? 1 : 0; stacked >= 0; --stacked)
+            for (int bufs = 2; bufs >= 1; --bufs) {
+                const int cols = stacked ? 2 * n : n;
+                if (bufs * T * cols > 512) continue;
+                const int need = T * kTileM + 2 * g->halo, rows = g->flat ? need : need + 2 * bp - 2;
+                const int nj = (rows + kRowStep * kRowBatch - 1) / (kRowStep * kRowBatch) * kRowBatch;
+                if (nj * kRowStep > kMaxBlockRows) continue;
+                const unsigned int a_stage = (unsigned int)(nj * kRowStep) * 128u;
+                // room for two operand blocks beside the weights: all of them, or a ring of at least three stages
+                const bool resident = all_b <= 100u * 1024u && all_b + fixed + 2 * a_stage <= kPipeSmem;
+                if (!resident && 3 * g->b_stage_bytes + fixed + 2 * a_stage > kPipeSmem) continue;
+                const int units = (g->tiles_per_m + T - 1) / T;
+                const int per_slice = kPlanSms / g->slices > 0 ? kPlanSms / g->slices : 1;
+                const double rounds = (double)(((long long)M * units + per_slice - 1) / per_slice);
+                const double step = !three ? clk(n) : (stacked ? clk(2 * n) + clk(n) : 3.0 * (n == 128 ? 80.0 : clk(n)));
+                double mma = (double)T * 2.0 * taps * chunks * step;
+                if (!resident) mma = std::max(mma, (double)all_b / 28.0);
+                const double load = (double)rows * v.c_in * 4.0 / 20.0, epi = 350.0 * T * ((n + 31) / 32);
+                const double body = bufs == 2 ? std::max(std::max(mma, load), epi) : std::max(mma, load) + epi;
+                const double cost = rounds * body + std::max(mma, load) * 0.3 + epi;
+                if (g->T == 0 || cost < best * 0.999) {
+                    best = cost;
+                    g->T = T; g->units_per_m = units; g->a_rows = nj * kRowStep; g->a_stage_bytes = a_stage; g->b_resident = resident ? 1 : 0;
+                    g->stacked = stacked; g->acc_cols = (unsigned int)cols; g->acc_bufs = bufs;
+                }
+            }
+    if (!g->T) return false;
+    // Few units with a long K loop: several CTAs share it (partial tiles in L2, added in order by the last to finish).
+    g->ksplit = 1;
+    const int tasks = M * g->units_per_m * g->slices, ksteps = 2 * taps * chunks;
+    if (2 * tasks <= kPlanSms && ksteps >= 128) {
+        int S = kPlanSms / tasks;
+        if (S > 8) S = 8;
+        if (S > ksteps / 32) S = ksteps / 32;
+        if (S > chunks) S = chunks;
+        if (S > 1) g->ksplit = S;
+    }
+    if (g->ksplit > 1) g->b_resident = 0;
+    // Blocks of units: the reader of the BN moments merges one row per block, so as few as leave the busiest CTA with at most
+    // a tenth more work.
+    g->unit_block = 1;
+    if (g->ksplit == 1) {
+        const int per_slice = kPlanSms / g->slices > 0 ? kPlanSms / g->slices : 1;
+        const int most = (M * g->units_per_m + per_slice - 1) / per_slice;
+        for (int u = 2; u <= 16 && u <= most; ++u) {
+            const int blocks = M * ((g->units_per_m + u - 1) / u);
+            if (10 * u * ((blocks + per_slice - 1) / per_slice) <= 11 * most) g->unit_block = u;
+        }
+    }
+    g->blocks_per_m = (g->units_per_m + g->unit_block - 1) / g->unit_block;
+    if (!g->b_resident && 3 * g->b_stage_bytes + fixed + 2 * g->a_stage_bytes > kPipeSmem) return false;
+    unsigned int left = kPipeSmem - fixed;
+    if (g->b_resident) { g->b_stages = taps * chunks; left -= all_b; }
+    else {
+        // the operand ring first gets two stages; the weights up to eight of what is left, the operand the rest
+        int bs = (int)((left - 2 * g->a_stage_bytes) / g->b_stage_bytes);
+        if (bs > kMaxB) bs = kMaxB;
+        if (bs > taps * chunks) bs = taps * chunks;
+        g->b_stages = bs;
+        left -= (unsigned int)bs * g->b_stage_bytes;
+    }
+    g->a_stages = (int)(left / g->a_stage_bytes);
+    if (g->a_stages > kMaxA) g->a_stages = kMaxA;
+    return g->a_stages >= 2;
+}
+
+bool conv_pipe_can_fuse_bn_output(const ConvPipeGeom& g) { return g.n_chunk <= 128; }      // a warp keeps the moments of two groups of 32 channels
+bool conv_pipe_can_fuse_bn_input(const ConvShape& s) { return s.stride == 1 && s.C % 16 == 0 && s.C <= 512; }
+
+size_t conv_pipe_splitk_bytes(const ConvShape& s, int pass, int passes, int M)
+{
+    ConvPipeGeom g;
+    if (!conv_pipe_geom(s, pass, passes, M, &g) || g.ksplit < 2) return 0;
+    return (kSplitKTicketBytes + (size_t)g.units_per_m * g.slices * g.ksplit * g.T * kTileM * g.n_chunk * sizeof(float) + 255) & ~(size_t)255;
+}
+
+struct ConvPipeLaunch { PipeParams p; unsigned int smem; int bn_in; };
+static_assert(sizeof(ConvPipeLaunch) <= sizeof(((ConvPipePlan*)0)->storage), "plan storage too small");
+
+cudaError_t conv_pipe_init()
+{
+    static bool done = false;
+    if (done) return cudaSuccess;
+    cudaError_t e = cudaSuccess;
+    for (auto kernel : {conv_pipe_kernel<false, false>, conv_pipe_kernel<false, true>, conv_pipe_kernel<true, false>, conv_pipe_kernel<true, true>})
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPipeSmem + 1024);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(conv_pipe_cell_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPipeSmem + 1024);
+    done = e == cudaSuccess;
+    return e;
+}
+
+namespace {
+cudaError_t encode_map(CUtensorMap* tm, const float* base, int rank, const cuuint64_t* dims, const cuuint64_t* strides, const cuuint32_t* box,
+                       CUtensorMapSwizzle swizzle)
+{
+    if (!g_encode) return cudaErrorNotReady;
+    const cuuint32_t ones[4] = {1, 1, 1, 1};
+    const CUresult r = g_encode(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, (cuuint32_t)rank, const_cast<float*>(base), dims, strides, box, ones,
+                                CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+cudaError_t encode_weights(CUtensorMap* tm, const float* base, long long kdim, int c_out, int n_chunk)
+{
+    const cuuint64_t dims[2] = {(cuuint64_t)kdim, (cuuint64_t)c_out}, strides[1] = {(cuuint64_t)kdim * 4};
+    const cuuint32_t box[2] = {16, (cuuint32_t)n_chunk};
+    return encode_map(tm, base, 2, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_64B);
+}
+unsigned int columns_pow2(unsigned int need)
+{
+    unsigned int c = 32;
+    while (c < need) c <<= 1;
+    return c;
+}
+}  // namespace
+
+cudaError_t conv_pipe_prepare(ConvPipePlan* plan, const ConvShape& s, int pass, int passes, int M, const float* in, const float* w_hi,
+                              const float* w_lo, float* out, const float* extra, bool accumulate, const ConvPipeBn* bn, void* splitk,
+                              size_t splitk_bytes, bool w_ready)
+{
+    plan->valid = 0;
+    ConvPipeGeom g;
+    PipeView v;
+    if ((passes != 1 && passes != 3) || !conv_pipe_geom(s, pass, passes, M, &g) || !pipe_view(s, pass, &v)) return cudaErrorNotSupported;
+    ConvPipeLaunch* L = reinterpret_cast<ConvPipeLaunch*>(plan->storage);
+    memset(L, 0, sizeof *L);
+    const long long kdim = (long long)s.R * s.R * v.c_in;
+    cudaError_t e = encode_weights(&L->p.tm_b, w_hi, kdim, v.c_out, g.n_chunk);
+    if (e == cudaSuccess) e = encode_weights(&L->p.tm_b_lo, passes == 3 ? w_lo : w_hi, kdim, v.c_out, g.n_chunk);
+    if (e != cudaSuccess) return e;
+    PipeScalars& p = L->p.s;
+    p.in = in; p.out = out; p.extra = extra; p.in_ms = v.in_ms; p.out_ms = v.out_ms;
+    p.accumulate = accumulate ? 1 : 0;
+    p.units_per_m = g.units_per_m; p.unit_block = g.unit_block; p.blocks_per_m = g.blocks_per_m; p.tiles_per_m = g.tiles_per_m; p.T = g.T; p.slices = g.slices; p.n_chunk = g.n_chunk; p.ksplit = g.ksplit;
+    p.R = s.R; p.taps = s.R * s.R; p.n_chunks = v.c_in / 16; p.c_in = v.c_in; p.c_out = v.c_out;
+    p.pos_per_m = g.pos_per_m; p.Wp = g.Wp; p.img_pos = g.Wp * g.Hp; p.Hv = v.P; p.W = v.Q; p.halo = g.halo;
+    p.strips = g.strips; p.strip_w = g.strip_w; p.col0 = g.col0;
+    p.magic_w = magic_of(g.Wp); p.magic_img = magic_of(p.img_pos); p.magic_strip = magic_of(g.strips);
+    p.in_sw = v.in_sw; p.in_sh = v.in_sh; p.in_sn = v.in_sn; p.os_w = v.os_w; p.os_h = v.os_h; p.os_n = v.os_n;
+    p.zero_fill = v.zero_fill; p.out_h = v.out_h; p.out_w = v.out_w; p.dense_h = v.dense_h; p.dense_w = v.dense_w;
+    p.flat = g.flat; p.box_h = g.box_h; p.box_pos = g.box_h * g.Wp; p.blocks_per_img = g.Hp / g.box_h;
+    p.magic_box = magic_of(p.box_pos); p.magic_bpi = magic_of(p.blocks_per_img);
+    p.pix_ms = g.flat ? (long long)s.N * v.P * v.Q : s.N;
+    if ((long long)M * p.pix_ms >= (1LL << 31)) return cudaErrorNotSupported;
+    {
+        CUtensorMap* tm = &L->p.tm_a;
+        const cuuint64_t fd[2] = {(cuuint64_t)v.c_in, (cuuint64_t)(M * p.pix_ms)}, fs[1] = {(cuuint64_t)v.c_in * 4};
+        const cuuint32_t fb[2] = {16, kTileM};
+        const cuuint64_t rd[4] = {(cuuint64_t)v.c_in, (cuuint64_t)v.in_W, (cuuint64_t)v.in_H, (cuuint64_t)M * s.N};
+        const cuuint64_t rs[3] = {(cuuint64_t)v.in_sw * 4, (cuuint64_t)v.in_sh * 4, (cuuint64_t)v.in_sn * 4};
+        const cuuint32_t rb[4] = {16, (cuuint32_t)g.Wp, (cuuint32_t)g.box_h, 1};
+        e = g.flat ? encode_map(tm, in, 2, fd, fs, fb, CU_TENSOR_MAP_SWIZZLE_128B) : encode_map(tm, in, 4, rd, rs, rb, CU_TENSOR_MAP_SWIZZLE_128B);
+        if (e != cudaSuccess) return e;
+    }
+    p.a_stages = g.a_stages; p.b_stages = g.b_stages; p.b_resident = g.b_resident; p.acc_bufs = g.acc_bufs;
+    p.a_stage_bytes = g.a_stage_bytes; p.b_stage_bytes = g.b_stage_bytes; p.acc_cols = g.acc_cols;
+    p.tmem_cols = columns_pow2((unsigned int)(g.acc_bufs * g.T) * g.acc_cols);
+    p.idesc = instr_desc(g.n_chunk, false, false);
+    p.idesc2 = instr_desc(g.stacked ? 2 * g.n_chunk : g.n_chunk, false, false);
+    p.split_groups = g.a_stages >= 4 ? 4 : 2;
+    p.epi_alternate = g.acc_bufs == 2 && g.n_chunk <= 64 && g.ksplit == 1 ? 1 : 0;
+    p.three = passes == 3 ? 1 : 0; p.stacked = g.stacked; p.w_ready = w_ready ? 1 : 0;
+    const unsigned int a_bytes = (unsigned int)g.a_stages * g.a_stage_bytes;
+    p.off_b = a_bytes;
+    p.off_stage = (p.off_b + (unsigned int)g.b_stages * g.b_stage_bytes + 127u) & ~127u;
+    p.off_stat = p.off_stage + kEpiWarps * 4096u;
+    p.off_red = p.off_stat + stat_bytes(g.n_chunk);
+    p.off_bn = p.off_red + 3 * kSplitThreads * 16;
+    L->smem = p.off_red + 1024;
+    if (bn && bn->out_partials) {
+        if (!conv_pipe_can_fuse_bn_output(g)) return cudaErrorNotSupported;
+        p.st_partials = bn->out_partials;
+    }
+    if (bn && bn->in_partials) {
+        if (pass != PASS_FWD || s.stride != 1 || v.c_in > 512 || bn->in_blocks < 1) return cudaErrorNotSupported;
+        p.bn_partials = bn->in_partials; p.bn_units = bn->in_blocks; p.bn_gamma = bn->in_gamma; p.bn_beta = bn->in_beta;
+        p.bn_stats = bn->in_stats; p.bn_y = bn->in_y; p.bn_eps = bn->in_eps;
+        p.bn_inv_rows = 1.0 / ((double)s.N * s.H * s.W);
+        L->smem = p.off_bn + 4u * (unsigned int)v.c_in * 4u + 1024;
+        L->bn_in = 1;
+    }
+    if (g.ksplit > 1) {
+        if (!splitk || conv_pipe_splitk_bytes(s, pass, passes, M) > splitk_bytes) return cudaErrorInvalidValue;
+        p.sk_base = reinterpret_cast<char*>(splitk); p.sk_ms = (long long)splitk_bytes;
+    }
+    if (L->smem > kPipeSmem + 1024) return cudaErrorNotSupported;
+    plan->valid = 1;
+    return cudaSuccess;
+}
+
+cudaError_t conv_pipe_launch(const ConvPipePlan* plan, int m_first, int m_count, bool pdl_late, DeviceStatus* status, cudaStream_t st, int64_t* n_launch)
+{
+    if (!plan->valid || m_count < 1) return cudaErrorInvalidValue;
+    ConvPipeLaunch L = *reinterpret_cast<const ConvPipeLaunch*>(plan->storage);
+    L.p.s.status = status;
+    // (a launch that waits for its weights lets its successor start only after that wait: the successor may not wait for them)
+    L.p.s.pdl_late = pdl_late || !L.p.s.w_ready ? 1 : 0;
+    const PipeScalars& p = L.p.s;
+    const int tasks = m_count * p.blocks_per_m * p.ksplit;
+    int per_slice = sm_count() / p.slices;
+    if (per_slice < 1) per_slice = 1;
+    if (per_slice > tasks) per_slice = tasks;
+    const bool flat = p.flat && p.zero_fill == 1;
+    auto kernel = L.bn_in ? (flat ? conv_pipe_kernel<true, true> : conv_pipe_kernel<true, false>)
+                          : (flat ? conv_pipe_kernel<false, true> : conv_pipe_kernel<false, false>);
+    launch_pdl(kernel, dim3(per_slice * p.slices), dim3(kPipeThreads), L.smem, st, L.p, m_first, m_count);
+    if (n_launch) ++*n_launch;
+    return cudaGetLastError();
+}
+
+size_t conv_pipe_cell_op_bytes() { return sizeof(CellOp); }
+
+void conv_pipe_cell_op(const ConvPipePlan* plan, DeviceStatus* status, void* dst_host, unsigned int* smem, unsigned int* tmem_cols)
+{
+    const ConvPipeLaunch* L = reinterpret_cast<const ConvPipeLaunch*>(plan->storage);
+    CellOp op;
+    memset(&op, 0, sizeof op);
+    op.p = L->p;
+    op.p.s.status = status;
+    op.bn_in = L->bn_in; op.flat = L->p.s.flat && L->p.s.zero_fill == 1;
+    memcpy(dst_host, &op, sizeof op);
+    *smem = L->smem; *tmem_cols = L->p.s.tmem_cols;
+}
+
+int conv_pipe_cell_max_ctas() { return sm_count(); }
+
+cudaError_t conv_pipe_cell_launch(const void* d_ops, int n_ops, int m_first, int m_count, int ctas, unsigned int smem, unsigned int tmem_cols,
+                                  unsigned int* d_barrier, DeviceStatus* status, cudaStream_t st, int64_t* n_launch)
+{
+    if (n_ops < 1 || ctas < 1 || m_count < 1 || tmem_cols < 32 || tmem_cols > 512) return cudaErrorInvalidValue;
+    CellParams cp;
+    cp.ops = reinterpret_cast<const CellOp*>(d_ops); cp.n_ops = n_ops; cp.barrier = d_barrier; cp.status = status; cp.tmem_cols = tmem_cols;
+    // Over half of an SM's shared memory in any case: two cells' CTAs never share an SM, where one could wait for tensor
+    // memory that the other holds while it waits for that one's grid.
+    if (smem < 120u * 1024u) smem = 120u * 1024u;
+    // a plain stream-ordered launch: a resident grid that started early would only hold SM slots while it waits
+    conv_pipe_cell_kernel<<<dim3(ctas), dim3(kPipeThreads), smem, st>>>(cp, m_first, m_count);
+    if (n_launch) ++*n_launch;
+    return cudaGetLastError();
+}
+
+cudaError_t bn_finalize_partials(const float* partials, int units, int C, float eps, double rows, float* stats, int m_count, cudaStream_t st,
+                                 int64_t* n_launch)
+{
+    launch_pdl(bn_finalize_kernel, dim3(m_count), dim3(256), (size_t)768 * 16 + 2 * (size_t)C * 4, st, partials, units, C, 1.0 / rows, eps, stats);
+    if (n_launch) ++*n_launch;
+    return cudaGetLastError();
+}
+
+}  // namespace hpf

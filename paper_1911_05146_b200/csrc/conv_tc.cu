@@ -159,6 +159,8 @@ struct WgradScalars {
     int raw_stages, t_stages;
     int passes;                  // 1 or 3
     unsigned int raw_bytes, t_bytes, tx_per_tap, tx_a, tmem_cols, idesc, idesc_tail;
+    int splits;                  // pixel splits of one micro-batch (block index = micro-batch * splits + split)
+    long long out_ms;            // floats between the micro-batches' outputs (partials, or gradient slots)
     long long split_stride;      // floats between partials
 };
 struct alignas(64) WgradParams {
@@ -180,6 +182,8 @@ struct WgradDirectScalars {
     int taps_per_cta, taps_per_mma;
     int stages, passes;
     unsigned int stage_bytes, lo_off, tx_bytes_a, tx_per_tap, tmem_cols, idesc, idesc_tail;
+    int splits;                  // pixel splits of one micro-batch (block index = micro-batch * splits + split)
+    long long out_ms;            // floats between the micro-batches' outputs (partials, or gradient slots)
     long long split_stride;      // floats between partials
 };
 struct alignas(64) WgradDirectParams {
@@ -1011,7 +1015,7 @@ __device__ __forceinline__ void transpose_tile(const uint8_t* raw, uint8_t* dst,
     }
 }
 
-__global__ void __launch_bounds__(192) conv_tc_wgrad_kernel(const __grid_constant__ WgradParams gp)
+__global__ void __launch_bounds__(192) conv_tc_wgrad_kernel(const __grid_constant__ WgradParams gp, const int m_first)
 {
     __shared__ WgradScalars p;                 // scalar parameters, see load_scalars
     pdl_launch_dependents();
@@ -1032,7 +1036,7 @@ __global__ void __launch_bounds__(192) conv_tc_wgrad_kernel(const __grid_constan
     // shared memory: raw stages first, then the transposed stages
     const uint32_t t_region0 = (uint32_t)p.raw_stages * p.raw_bytes;
 
-    const int split = blockIdx.x;
+    const int micro = m_first + (int)blockIdx.x / p.splits, split = (int)blockIdx.x % p.splits;
     const int tap0 = blockIdx.y * p.taps_per_cta;
     const int m_chunks = p.c_out / p.m_chunk;
     const int m0 = (blockIdx.z % m_chunks) * p.m_chunk;
@@ -1104,10 +1108,10 @@ __global__ void __launch_bounds__(192) conv_tc_wgrad_kernel(const __grid_constan
                 const uint32_t dst = smem_base + s * raw_bytes;
                 const uint32_t bar = full_raw0 + 8 * s;
                 mbar_expect_tx(bar, tx);
-                tma_load_4d(dst, &gp.tm_a, bar, m0, q0, p0, n0);
+                tma_load_5d(dst, &gp.tm_a, bar, m0, q0, p0, n0, micro);
                 int r = r_first, sx = sx_first;
                 for (int tp = 0; tp < ntaps; ++tp) {
-                    tma_load_4d(dst + raw_a + tp * raw_b, &gp.tm_b, bar, cn0, q0 + sx - pad, p0 + r - pad, n0);
+                    tma_load_5d(dst + raw_a + tp * raw_b, &gp.tm_b, bar, cn0, q0 + sx - pad, p0 + r - pad, n0, micro);
                     if (++sx == R) { sx = 0; ++r; }
                 }
                 if (++tw == tiles_w) { tw = 0; if (++th == tiles_h) { th = 0; ++tn; } }
@@ -1189,7 +1193,7 @@ __global__ void __launch_bounds__(192) conv_tc_wgrad_kernel(const __grid_constan
             const int row = (warp & 3) * 32 + lane;          // TMEM lane = output channel within the chunk
             const bool valid = row < p.m_chunk;
             const uint32_t lane_addr = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
-            float* obase = p.out + (long long)split * p.split_stride + ((long long)(m0 + row) * p.R * p.R) * p.c_in + cn0;
+            float* obase = p.out + (long long)micro * p.out_ms + (long long)split * p.split_stride + ((long long)(m0 + row) * p.R * p.R) * p.c_in + cn0;
             for (int tp = 0; tp < ntaps; ++tp)
                 for (int c0 = 0; c0 < p.n_cols; c0 += 16) {
                     float v[16];
@@ -1234,7 +1238,7 @@ __global__ void __launch_bounds__(192) conv_tc_wgrad_kernel(const __grid_constan
 // accumulator hold products of whatever the shared memory held and are never read.  An MMA always reads 128 operand
 // rows = 4 blocks from the dy tile's base: blocks beyond the tile's own are the x tile or what follows it, and land in
 // accumulator lanes nobody reads.
-__global__ void __launch_bounds__(192) conv_tc_wgrad_direct_kernel(const __grid_constant__ WgradDirectParams gp)
+__global__ void __launch_bounds__(192) conv_tc_wgrad_direct_kernel(const __grid_constant__ WgradDirectParams gp, const int m_first)
 {
     __shared__ WgradDirectScalars p;
     pdl_launch_dependents();
@@ -1252,7 +1256,7 @@ __global__ void __launch_bounds__(192) conv_tc_wgrad_direct_kernel(const __grid_
     const int warp = warp_index(), lane = threadIdx.x & 31;
     const uint32_t full0 = smem_u32(&bars[0]), empty0 = smem_u32(&bars[8]), split0 = smem_u32(&bars[16]), accum_bar = smem_u32(&bars[24]);
 
-    const int split = blockIdx.x;
+    const int micro = m_first + (int)blockIdx.x / p.splits, split = (int)blockIdx.x % p.splits;
     const int tap0 = blockIdx.y * p.taps_per_cta;
     const int m_chunks = p.c_out / p.m_chunk;
     const int m0 = (blockIdx.z % m_chunks) * p.m_chunk;
@@ -1312,11 +1316,11 @@ __global__ void __launch_bounds__(192) conv_tc_wgrad_direct_kernel(const __grid_
                 uint32_t dst = smem_base + s * stage_bytes;
                 const uint32_t bar = full0 + 8 * s;
                 mbar_expect_tx(bar, tx);
-                for (int b = 0; b < m_blocks; ++b, dst += block_bytes) tma_load_4d(dst, &gp.tm_a, bar, m0 + b * m_box, q0, p0, n0);
+                for (int b = 0; b < m_blocks; ++b, dst += block_bytes) tma_load_5d(dst, &gp.tm_a, bar, m0 + b * m_box, q0, p0, n0, micro);
                 int r = r_first, sx = sx_first;
                 for (int tp = 0; tp < ntaps; ++tp) {
                     for (int b = 0; b < n_blocks; ++b, dst += block_bytes)
-                        tma_load_4d(dst, &gp.tm_b, bar, cn0 + b * n_box, q0 + sx - pad, p0 + r - pad, n0);
+                        tma_load_5d(dst, &gp.tm_b, bar, cn0 + b * n_box, q0 + sx - pad, p0 + r - pad, n0, micro);
                     if (++sx == R) { sx = 0; ++r; }
                 }
                 if (++tw == tiles_w) { tw = 0; if (++th == tiles_h) { th = 0; ++tn; } }
@@ -1406,7 +1410,7 @@ __global__ void __launch_bounds__(192) conv_tc_wgrad_direct_kernel(const __grid_
             const int row = (warp & 3) * 32 + lane;          // TMEM lane = output channel within the chunk
             const bool valid = row < p.m_chunk;
             const uint32_t lane_addr = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
-            float* obase = p.out + (long long)split * p.split_stride + ((long long)(m0 + row) * p.R * p.R) * p.c_in + cn0;
+            float* obase = p.out + (long long)micro * p.out_ms + (long long)split * p.split_stride + ((long long)(m0 + row) * p.R * p.R) * p.c_in + cn0;
             if ((warp & 3) * 32 < p.m_chunk)                 // a whole warp of lanes beyond the chunk has nothing to read
                 for (int tp = 0; tp < ntaps; ++tp)
                     for (int c0 = 0; c0 < p.n_cols; c0 += 16) {
@@ -1444,8 +1448,10 @@ __global__ void __launch_bounds__(192) conv_tc_wgrad_direct_kernel(const __grid_
 // dw[i] = sum over splits of partials[z][i], in an order fixed by the launch shape: thread (lane, zl) adds the
 // splits zl, zl+8, ... ascending, then the 8 partial sums are added ascending.  32 float4 per block.
 __global__ void __launch_bounds__(256)
-wgrad_partials_reduce_kernel(const float* __restrict__ partials, float* __restrict__ dw, long long n, int splits)
+wgrad_partials_reduce_kernel(const float* __restrict__ partials, float* __restrict__ dw, long long n, int splits, long long part_ms, long long dw_ms,
+                             int m_first)
 {
+    partials += (m_first + (int)blockIdx.y) * part_ms; dw += (m_first + (int)blockIdx.y) * dw_ms;
     __shared__ float4 sh[8][32];
     pdl_launch_dependents();
     pdl_wait();
@@ -1640,7 +1646,7 @@ cudaError_t encode(CUtensorMap* tm, const float* base, int rank, const cuuint64_
 }
 
 // How many pixel splits (CTAs along x) a weight-gradient launch of n_tiles pixel tiles gets.
-void wgrad_splits(const ConvShape& s, int n_tiles, int ctas_per_split, int max_ctas, int* splits_out, int* tiles_per_split_out)
+void wgrad_splits(const ConvShape& s, int n_tiles, int ctas_per_split, int M, int* splits_out, int* tiles_per_split_out)
 {
     const int taps = s.R * s.R;
     // enough CTAs to spread the pixel walk, few enough that the partials stay a fraction of the operand bytes
@@ -1653,9 +1659,9 @@ void wgrad_splits(const ConvShape& s, int n_tiles, int ctas_per_split, int max_c
     if (cap < want) cap = want;
     if (splits > cap) splits = cap;
     if (splits > 296) splits = 296;          // two CTAs per SM
-    if (max_ctas > 0) {
-        // the caller wants the launch to take little SM time (CTAs x (fixed cost + tiles)) rather than to be short
-        int ms = max_ctas / ctas_per_split;
+    if (M > 1) {
+        // the launch covers the model's M micro-batches, each with its own sums: two waves of two CTAs per SM between them
+        int ms = 592 / (ctas_per_split * M);
         if (ms < 1) ms = 1;
         if (splits > ms) splits = ms;
     }
@@ -1671,7 +1677,7 @@ struct WgradGeom {
     unsigned int raw_bytes, t_bytes, tmem_cols;
 };
 
-bool wgrad_geom(const ConvShape& s, int passes, WgradGeom* g, int max_ctas = 0)
+bool wgrad_geom(const ConvShape& s, int passes, WgradGeom* g, int M = 1)
 {
     if (s.C % 16 || s.K % 16) return false;
     if (s.R != 1 && s.R != 3) return false;
@@ -1718,7 +1724,7 @@ bool wgrad_geom(const ConvShape& s, int passes, WgradGeom* g, int max_ctas = 0)
     g->tmem_cols = pow2_cols(g->taps_per_cta * g->n_cols);
     const int tiles_w = (s.Q + g->box.w - 1) / g->box.w, tiles_h = (s.P + g->box.h - 1) / g->box.h, tiles_n = (s.N + g->box.n - 1) / g->box.n;
     g->n_tiles = tiles_w * tiles_h * tiles_n;
-    wgrad_splits(s, g->n_tiles, g->tap_groups * (s.K / g->m_chunk) * (s.C / g->n_cols), max_ctas, &g->splits, &g->tiles_per_split);
+    wgrad_splits(s, g->n_tiles, g->tap_groups * (s.K / g->m_chunk) * (s.C / g->n_cols), M, &g->splits, &g->tiles_per_split);
     return true;
 }
 
@@ -1733,7 +1739,7 @@ struct WgradDirectGeom {
 // the first combination whose accumulators take at most half of an SM's tensor memory (other kernels' CTAs share the
 // SM) and that gets at least three pipeline stages into 100 KB of shared memory - failing that two stages, failing
 // that two stages into 200 KB with all of the tensor memory.
-bool wgrad_direct_geom(const ConvShape& s, int passes, WgradDirectGeom* g, int max_ctas = 0)
+bool wgrad_direct_geom(const ConvShape& s, int passes, WgradDirectGeom* g, int M = 1)
 {
     if (s.C % 16 || s.K % 16) return false;
     if ((s.C > 16 && s.C % 32) || (s.K > 16 && s.K % 32)) return false;
@@ -1795,7 +1801,7 @@ bool wgrad_direct_geom(const ConvShape& s, int passes, WgradDirectGeom* g, int m
     g->tmem_cols = pow2_cols(g->taps_per_cta * g->n_blocks * 32);
     const int tiles_w = (s.Q + g->box.w - 1) / g->box.w, tiles_h = (s.P + g->box.h - 1) / g->box.h, tiles_n = (s.N + g->box.n - 1) / g->box.n;
     g->n_tiles = tiles_w * tiles_h * tiles_n;
-    wgrad_splits(s, g->n_tiles, g->tap_groups * (s.K / g->m_chunk) * (s.C / g->n_cols), max_ctas, &g->splits, &g->tiles_per_split);
+    wgrad_splits(s, g->n_tiles, g->tap_groups * (s.K / g->m_chunk) * (s.C / g->n_cols), M, &g->splits, &g->tiles_per_split);
     return true;
 }
 
@@ -1912,16 +1918,16 @@ size_t conv_tc_splitk_bytes(const ConvShape& s, int pass, int passes)
     return kSplitKTicketBytes + (size_t)tiles * (v.c_out / n_chunk) * S * kTileM * n_chunk * sizeof(float);
 }
 
-size_t conv_tc_scratch_bytes(const ConvShape& s)
+size_t conv_tc_scratch_bytes(const ConvShape& s, int M)
 {
     size_t need = 0;
     for (int passes = 1; passes <= 3; passes += 2) {
         WgradGeom g;
-        if (!wgrad_geom(s, passes, &g)) continue;
+        if (!wgrad_geom(s, passes, &g, M)) continue;
         const size_t b = g.splits > 1 ? (size_t)g.splits * s.K * s.R * s.R * s.C * sizeof(float) : 0;
         if (b > need) need = b;
         WgradDirectGeom d;
-        if (!wgrad_direct_geom(s, passes, &d)) continue;
+        if (!wgrad_direct_geom(s, passes, &d, M)) continue;
         const size_t bd = d.splits > 1 ? (size_t)d.splits * s.K * s.R * s.R * s.C * sizeof(float) : 0;
         if (bd > need) need = bd;
     }
@@ -1929,8 +1935,8 @@ size_t conv_tc_scratch_bytes(const ConvShape& s)
 }
 
 struct ConvTcFwdLaunch { FwdParams p; dim3 grid; unsigned int smem; };
-struct ConvTcWgradLaunch { WgradParams p; dim3 grid; unsigned int smem; int splits; float* dw; long long n_out; };
-struct ConvTcWgradDirectLaunch { WgradDirectParams p; dim3 grid; unsigned int smem; int splits; float* dw; long long n_out; };
+struct ConvTcWgradLaunch { WgradParams p; dim3 grid; unsigned int smem; int splits; float* dw; long long n_out, dw_ms; };
+struct ConvTcWgradDirectLaunch { WgradDirectParams p; dim3 grid; unsigned int smem; int splits; float* dw; long long n_out, dw_ms; };
 static_assert(sizeof(ConvTcWgradDirectLaunch) <= sizeof(((ConvTcPlan*)0)->storage), "plan storage too small");
 static_assert(sizeof(ConvTcFwdLaunch) <= sizeof(((ConvTcPlan*)0)->storage) && sizeof(ConvTcWgradLaunch) <= sizeof(((ConvTcPlan*)0)->storage),
               "plan storage too small");
@@ -1940,26 +1946,29 @@ cudaError_t conv_tc_prepare(ConvTcPlan* plan, const ConvShape& s, int pass, int 
                             const ConvBnFuse* fuse)
 {
     plan->valid = 0; plan->s = s; plan->pass = pass; plan->direct = 0;
+    const int M = fuse && fuse->micro_batches > 1 ? fuse->micro_batches : 1;
+    const long long dw_ms = fuse ? fuse->slot_stride : 0;
     if (passes != 1 && passes != 3) return cudaErrorInvalidValue;
     WgradDirectGeom dg;
-    if (pass == PASS_WGRAD && !(fuse && fuse->wgrad_transposing) && wgrad_direct_geom(s, passes, &dg, fuse ? fuse->wgrad_max_ctas : 0)) {
+    if (pass == PASS_WGRAD && !(fuse && fuse->wgrad_transposing) && wgrad_direct_geom(s, passes, &dg, M)) {
         ConvTcWgradDirectLaunch* L = reinterpret_cast<ConvTcWgradDirectLaunch*>(plan->storage);
         WgradDirectParams& P = L->p;
         memset(&P, 0, sizeof P);
         WgradDirectScalars& p = P.s;
         {   // dy {K, Q, P, N}
-            cuuint64_t dims[4] = {(cuuint64_t)s.K, (cuuint64_t)s.Q, (cuuint64_t)s.P, (cuuint64_t)s.N};
-            cuuint64_t str[3] = {(cuuint64_t)s.K * 4, (cuuint64_t)s.Q * s.K * 4, (cuuint64_t)s.P * s.Q * s.K * 4};
-            cuuint32_t box[4] = {(cuuint32_t)dg.m_box, (cuuint32_t)dg.box.w, (cuuint32_t)dg.box.h, (cuuint32_t)dg.box.n};
-            cudaError_t e = encode(&P.tm_a, in, 4, dims, str, box, kSwizzle128Atom32);
+            cuuint64_t dims[5] = {(cuuint64_t)s.K, (cuuint64_t)s.Q, (cuuint64_t)s.P, (cuuint64_t)s.N, (cuuint64_t)M};
+            cuuint64_t str[4] = {(cuuint64_t)s.K * 4, (cuuint64_t)s.Q * s.K * 4, (cuuint64_t)s.P * s.Q * s.K * 4, (cuuint64_t)s.N * s.P * s.Q * s.K * 4};
+            cuuint32_t box[5] = {(cuuint32_t)dg.m_box, (cuuint32_t)dg.box.w, (cuuint32_t)dg.box.h, (cuuint32_t)dg.box.n, 1};
+            cudaError_t e = encode(&P.tm_a, in, 5, dims, str, box, kSwizzle128Atom32);
             if (e != cudaSuccess) return e;
         }
         {   // x {C, Wv, Hv, N}: a strided 1x1 convolution samples every stride-th pixel
             const int wv = s.stride == 1 ? s.W : s.Q, hv = s.stride == 1 ? s.H : s.P;
-            cuuint64_t dims[4] = {(cuuint64_t)s.C, (cuuint64_t)wv, (cuuint64_t)hv, (cuuint64_t)s.N};
-            cuuint64_t str[3] = {(cuuint64_t)s.stride * s.C * 4, (cuuint64_t)s.stride * s.W * s.C * 4, (cuuint64_t)s.H * s.W * s.C * 4};
-            cuuint32_t box[4] = {(cuuint32_t)dg.n_box, (cuuint32_t)dg.box.w, (cuuint32_t)dg.box.h, (cuuint32_t)dg.box.n};
-            cudaError_t e = encode(&P.tm_b, in2, 4, dims, str, box, kSwizzle128Atom32);
+            cuuint64_t dims[5] = {(cuuint64_t)s.C, (cuuint64_t)wv, (cuuint64_t)hv, (cuuint64_t)s.N, (cuuint64_t)M};
+            cuuint64_t str[4] = {(cuuint64_t)s.stride * s.C * 4, (cuuint64_t)s.stride * s.W * s.C * 4, (cuuint64_t)s.H * s.W * s.C * 4,
+                                 (cuuint64_t)s.N * s.H * s.W * s.C * 4};
+            cuuint32_t box[5] = {(cuuint32_t)dg.n_box, (cuuint32_t)dg.box.w, (cuuint32_t)dg.box.h, (cuuint32_t)dg.box.n, 1};
+            cudaError_t e = encode(&P.tm_b, in2, 5, dims, str, box, kSwizzle128Atom32);
             if (e != cudaSuccess) return e;
         }
         const long long n_out = (long long)s.K * s.R * s.R * s.C;
@@ -1977,7 +1986,7 @@ cudaError_t conv_tc_prepare(ConvTcPlan* plan, const ConvShape& s, int pass, int 
         p.taps_per_mma = 256 / slot < dg.taps_per_cta ? 256 / slot : dg.taps_per_cta;
         p.idesc = instr_desc(slot * p.taps_per_mma, true, true);
         p.idesc_tail = instr_desc(slot * (dg.taps_per_cta % p.taps_per_mma ? dg.taps_per_cta % p.taps_per_mma : p.taps_per_mma), true, true);
-        p.split_stride = n_out;
+        p.split_stride = n_out; p.splits = dg.splits; p.out_ms = dg.splits > 1 ? (fuse && fuse->partial_stride ? fuse->partial_stride : n_out * dg.splits) : dw_ms; L->dw_ms = dw_ms;
         L->grid = dim3(dg.splits, dg.tap_groups, (s.K / dg.m_chunk) * (s.C / dg.n_cols));
         L->smem = (unsigned int)dg.stages * dg.stage_bytes + dg.slack + 1024;
         L->splits = dg.splits; L->dw = out; L->n_out = n_out;
@@ -1987,26 +1996,27 @@ cudaError_t conv_tc_prepare(ConvTcPlan* plan, const ConvShape& s, int pass, int 
     }
     if (pass == PASS_WGRAD) {
         WgradGeom g;
-        if (!wgrad_geom(s, passes, &g, fuse ? fuse->wgrad_max_ctas : 0)) return cudaErrorNotSupported;
+        if (!wgrad_geom(s, passes, &g, M)) return cudaErrorNotSupported;
         ConvTcWgradLaunch* L = reinterpret_cast<ConvTcWgradLaunch*>(plan->storage);
         WgradParams& P = L->p;
         memset(&P, 0, sizeof P);
         WgradScalars& p = P.s;
         // dy {K, Q, P, N}
         {
-            cuuint64_t dims[4] = {(cuuint64_t)s.K, (cuuint64_t)s.Q, (cuuint64_t)s.P, (cuuint64_t)s.N};
-            cuuint64_t str[3] = {(cuuint64_t)s.K * 4, (cuuint64_t)s.Q * s.K * 4, (cuuint64_t)s.P * s.Q * s.K * 4};
-            cuuint32_t box[4] = {(cuuint32_t)g.m_chunk, (cuuint32_t)g.box.w, (cuuint32_t)g.box.h, (cuuint32_t)g.box.n};
-            cudaError_t e = encode(&P.tm_a, in, 4, dims, str, box, 0);
+            cuuint64_t dims[5] = {(cuuint64_t)s.K, (cuuint64_t)s.Q, (cuuint64_t)s.P, (cuuint64_t)s.N, (cuuint64_t)M};
+            cuuint64_t str[4] = {(cuuint64_t)s.K * 4, (cuuint64_t)s.Q * s.K * 4, (cuuint64_t)s.P * s.Q * s.K * 4, (cuuint64_t)s.N * s.P * s.Q * s.K * 4};
+            cuuint32_t box[5] = {(cuuint32_t)g.m_chunk, (cuuint32_t)g.box.w, (cuuint32_t)g.box.h, (cuuint32_t)g.box.n, 1};
+            cudaError_t e = encode(&P.tm_a, in, 5, dims, str, box, 0);
             if (e != cudaSuccess) return e;
         }
         // x {C, Wv, Hv, N}: a strided 1x1 convolution samples every stride-th pixel
         {
             const int wv = s.stride == 1 ? s.W : s.Q, hv = s.stride == 1 ? s.H : s.P;
-            cuuint64_t dims[4] = {(cuuint64_t)s.C, (cuuint64_t)wv, (cuuint64_t)hv, (cuuint64_t)s.N};
-            cuuint64_t str[3] = {(cuuint64_t)s.stride * s.C * 4, (cuuint64_t)s.stride * s.W * s.C * 4, (cuuint64_t)s.H * s.W * s.C * 4};
-            cuuint32_t box[4] = {(cuuint32_t)g.n_cols, (cuuint32_t)g.box.w, (cuuint32_t)g.box.h, (cuuint32_t)g.box.n};
-            cudaError_t e = encode(&P.tm_b, in2, 4, dims, str, box, 0);
+            cuuint64_t dims[5] = {(cuuint64_t)s.C, (cuuint64_t)wv, (cuuint64_t)hv, (cuuint64_t)s.N, (cuuint64_t)M};
+            cuuint64_t str[4] = {(cuuint64_t)s.stride * s.C * 4, (cuuint64_t)s.stride * s.W * s.C * 4, (cuuint64_t)s.H * s.W * s.C * 4,
+                                 (cuuint64_t)s.N * s.H * s.W * s.C * 4};
+            cuuint32_t box[5] = {(cuuint32_t)g.n_cols, (cuuint32_t)g.box.w, (cuuint32_t)g.box.h, (cuuint32_t)g.box.n, 1};
+            cudaError_t e = encode(&P.tm_b, in2, 5, dims, str, box, 0);
             if (e != cudaSuccess) return e;
         }
         const long long n_out = (long long)s.K * s.R * s.R * s.C;
@@ -2023,7 +2033,7 @@ cudaError_t conv_tc_prepare(ConvTcPlan* plan, const ConvShape& s, int pass, int 
         p.taps_per_mma = 256 / g.n_cols < g.taps_per_cta ? 256 / g.n_cols : g.taps_per_cta;
         p.idesc = instr_desc(g.n_cols * p.taps_per_mma, false, false);
         p.idesc_tail = instr_desc(g.n_cols * (g.taps_per_cta % p.taps_per_mma ? g.taps_per_cta % p.taps_per_mma : p.taps_per_mma), false, false);
-        p.split_stride = n_out;
+        p.split_stride = n_out; p.splits = g.splits; p.out_ms = g.splits > 1 ? (fuse && fuse->partial_stride ? fuse->partial_stride : n_out * g.splits) : dw_ms; L->dw_ms = dw_ms;
         L->grid = dim3(g.splits, g.tap_groups, (s.K / g.m_chunk) * (s.C / g.n_cols));
         L->smem = (unsigned int)g.raw_stages * g.raw_bytes + (unsigned int)g.t_stages * g.t_bytes + (g.m_chunk < 128 ? kWgradSlack : 0u) + 1024;
         L->splits = g.splits; L->dw = out; L->n_out = n_out;
@@ -2160,17 +2170,17 @@ cudaError_t conv_tc_prepare(ConvTcPlan* plan, const ConvShape& s, int pass, int 
     return cudaSuccess;
 }
 
-cudaError_t conv_tc_launch(const ConvTcPlan* plan, DeviceStatus* status, cudaStream_t st, int64_t* n_launch)
+cudaError_t conv_tc_launch(const ConvTcPlan* plan, DeviceStatus* status, cudaStream_t st, int64_t* n_launch, int m_first, int m_count)
 {
     if (!plan->valid) return cudaErrorInvalidValue;
     if (plan->pass == PASS_WGRAD && plan->direct) {
         ConvTcWgradDirectLaunch L = *reinterpret_cast<const ConvTcWgradDirectLaunch*>(plan->storage);
         L.p.s.status = status;
-        launch_pdl(conv_tc_wgrad_direct_kernel, L.grid, dim3(192), L.smem, st, L.p);
+        launch_pdl(conv_tc_wgrad_direct_kernel, dim3(L.grid.x * m_count, L.grid.y, L.grid.z), dim3(192), L.smem, st, L.p, m_first);
         count(n_launch, 1);
         if (L.splits > 1) {
             const int nb = (int)((L.n_out / 4 + 31) / 32);
-            launch_pdl(wgrad_partials_reduce_kernel, dim3(nb), dim3(256), 0, st, (const float*)L.p.s.out, L.dw, L.n_out, L.splits);
+            launch_pdl(wgrad_partials_reduce_kernel, dim3(nb, m_count), dim3(256), 0, st, (const float*)L.p.s.out, L.dw, L.n_out, L.splits, L.p.s.out_ms, L.dw_ms, m_first);
             count(n_launch, 1);
         }
         return cudaGetLastError();
@@ -2178,11 +2188,11 @@ cudaError_t conv_tc_launch(const ConvTcPlan* plan, DeviceStatus* status, cudaStr
     if (plan->pass == PASS_WGRAD) {
         ConvTcWgradLaunch L = *reinterpret_cast<const ConvTcWgradLaunch*>(plan->storage);
         L.p.s.status = status;
-        launch_pdl(conv_tc_wgrad_kernel, L.grid, dim3(192), L.smem, st, L.p);
+        launch_pdl(conv_tc_wgrad_kernel, dim3(L.grid.x * m_count, L.grid.y, L.grid.z), dim3(192), L.smem, st, L.p, m_first);
         count(n_launch, 1);
         if (L.splits > 1) {
             const int nb = (int)((L.n_out / 4 + 31) / 32);
-            launch_pdl(wgrad_partials_reduce_kernel, dim3(nb), dim3(256), 0, st, (const float*)L.p.s.out, L.dw, L.n_out, L.splits);
+            launch_pdl(wgrad_partials_reduce_kernel, dim3(nb, m_count), dim3(256), 0, st, (const float*)L.p.s.out, L.dw, L.n_out, L.splits, L.p.s.out_ms, L.dw_ms, m_first);
             count(n_launch, 1);
         }
         return cudaGetLastError();

@@ -12,7 +12,8 @@ bool conv_tc_supported(const ConvShape& s, int pass);
 // Resolves the driver entry point used to encode tensor maps.  Needs a CUDA driver.
 cudaError_t conv_tc_init();
 
-size_t conv_tc_scratch_bytes(const ConvShape& s);
+// weight-gradient partials of one micro-batch, of a model with M of them
+size_t conv_tc_scratch_bytes(const ConvShape& s, int M = 1);
 
 // A prepared launch: tensor maps are encoded once (they bake in the device pointers) and the kernel
 // parameters are kept ready in `storage`.
@@ -48,9 +49,10 @@ struct ConvBnFuse {
     const float* in_beta = nullptr;
     float* in_stats = nullptr;
     float* in_y = nullptr;
-    // weight gradient only: > 0 caps the CTAs of the launch (fewer pixel splits, each walking more tiles): less SM time
-    // at a longer duration, for launches that run beside a chain of latency-bound kernels
-    int wgrad_max_ctas = 0;
+    // weight gradient only: the model's micro-batches, contiguous in `in` and `in2`, and the floats between their outputs
+    int micro_batches = 1;
+    long long slot_stride = 0;
+    long long partial_stride = 0;        // floats between the micro-batches' partial sums (0: packed)
     // weight gradient only: 1 keeps the kernel that transposes its tiles in shared memory (a cross-check)
     int wgrad_transposing = 0;
     const float* in_partials = nullptr;
@@ -85,7 +87,8 @@ bool conv_tc_can_fuse_bn(const ConvShape& s, int pass);
 cudaError_t conv_tc_prepare(ConvTcPlan* plan, const ConvShape& s, int pass, int passes, const float* in, const float* in2,
                             const float* w_hi, const float* w_lo, float* out, const float* extra, bool accumulate, void* scratch,
                             const ConvBnFuse* fuse = nullptr);
-cudaError_t conv_tc_launch(const ConvTcPlan* plan, DeviceStatus* status, cudaStream_t st, int64_t* n_launch);
+// m_first, m_count: the micro-batches a weight-gradient launch covers
+cudaError_t conv_tc_launch(const ConvTcPlan* plan, DeviceStatus* status, cudaStream_t st, int64_t* n_launch, int m_first = 0, int m_count = 1);
 
 // Persistent cell kernel: a list of prepared forward / data-gradient launches run one after the other by ONE resident grid
 // with a grid-wide barrier between them (see conv_tc.cu).  conv_tc_cell_op writes the device-side record of a prepared

@@ -60,16 +60,26 @@ int api_cuda_fail(cudaError_t e, const char* where);
 struct DeviceStatus { unsigned int code; unsigned int detail; };
 
 // ---------------- memory-bound kernels (kernels_mem.cu) ----------------
+// Several micro-batches in one launch: what belongs to micro-batch k lies k strides further on (floats; scratch in bytes).
+// The split of the work inside a micro-batch does not depend on `count`, so neither do the results.
+struct BnGroup {
+    int count = 1;
+    int64_t x = 0;           // x, dy, dx, y, addend
+    int64_t stats = 0;
+    int64_t param = 0;       // dgamma, dbeta
+    int64_t scratch = 0;
+};
 size_t bn_scratch_bytes(int64_t rows, int C);
 // scratch: first 256 bytes hold the block ticket (must be zero before the first use; the kernels
 // leave it zero), the rest holds per-block partial sums.
 // relu = false: batch normalisation without the activation (the post-activation block's second BN)
 cudaError_t bnrelu_fwd(const float* x, const float* gamma, const float* beta, float eps, float* y, float* stats,
-                       int64_t rows, int C, void* scratch, cudaStream_t st, int64_t* n_launch, bool relu = true);
+                       int64_t rows, int C, void* scratch, cudaStream_t st, int64_t* n_launch, bool relu = true,
+                       const BnGroup& grp = BnGroup());
 cudaError_t bnrelu_bwd(const float* x, const float* dy, const float* gamma, const float* beta, const float* stats,
                        float* dx, const float* addend, bool accumulate, float* dgamma, float* dbeta,
                        int64_t rows, int C, void* scratch, cudaStream_t st, int64_t* n_launch, bool relu = true,
-                       bool x_is_old = false);
+                       bool x_is_old = false, const BnGroup& grp = BnGroup());
 // x_is_old: x, stats, gamma and beta were complete before the kernels just ahead of this call in the stream were
 // enqueued (forward results read by a backward pass), so the kernel may fetch them while its predecessor still runs.
 // The forward from an on-chip copy of the tensor (bn_resident.cu): one cooperative launch that holds every SM, for
@@ -94,7 +104,7 @@ cudaError_t relu_bwd(const float* x, const float* dy, float* dx, const float* ad
                      int64_t* n_launch);
 // The forward's second half alone: the statistics (mean[C], rstd[C]) were left by the convolution kernel that produced x.
 cudaError_t bnrelu_fwd_apply(const float* x, const float* gamma, const float* beta, const float* stats, float* y,
-                             int64_t rows, int C, cudaStream_t st, int64_t* n_launch);
+                             int64_t rows, int C, cudaStream_t st, int64_t* n_launch, const BnGroup& grp = BnGroup());
 cudaError_t add_fwd(const float* a, const float* b, float* out, int64_t n, cudaStream_t st, int64_t* n_launch);
 // dst (+)= src
 cudaError_t grad_accumulate(float* dst, const float* src, int64_t n, bool accumulate, cudaStream_t st, int64_t* n_launch);

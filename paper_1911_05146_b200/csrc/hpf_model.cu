@@ -1,6 +1,7 @@
 // Host side of the library: layer-list validation, partition / micro-batch bookkeeping, the memory
 // plan, the gradient-flow plan, the stream/event (or captured-graph) pipeline scheduler, and the C ABI.
 #include "../../include/hpf.h"
+#include "conv_pipe.h"
 #include "conv_tc.h"
 #include "hpf_kernels.h"
 
@@ -91,10 +92,8 @@ struct hpf_model {
     std::vector<int> bn_fwd_from;              // BN -> conv whose forward kernel also produces the statistics of the BN (its input), or -1
     std::vector<int> conv_fwd_bn;              // the inverse map
     std::vector<int> bn_into, conv_in_bn;      // BN -> the convolution that applies it to its own input operand (no BN kernel), and the inverse
-    std::vector<int> bn_late;                  // BN -> 1: the applying convolution derives the statistics from the per-tile sums itself
-    std::vector<int> bn_buf;                   // BN -> which of the stream's two per-tile-sum buffers carries its sums
-    std::vector<size_t> bn_part_bytes;         // per partition: size of one per-tile-sum buffer
-    int opt_bn_late_floats = 8192;             // largest [tiles][2][C] block of per-tile sums a reading convolution adds itself
+    std::vector<size_t> bn_moments_off;        // BN -> per-unit moments of its input left by the producing convolution, all micro-batches
+    std::vector<ConvPipeGeom> pipe_geom[2];    // conv -> split of its forward / data-gradient launches
     bool opt_pdl = true;       // programmatic dependent launch for this model's kernels
     bool opt_bn_cluster = true; // BN backward of micro-batch sized tensors as one thread-block-cluster launch
     int opt_cell_times = 0;    // record a device timestamp at the start and end of every (partition, micro-batch) cell
@@ -104,12 +103,14 @@ struct hpf_model {
     struct CellRun {
         int part = 0;
         std::vector<int> convs;               // ops of the run, ascending; the kernel is enqueued at convs[0]'s place
-        std::vector<size_t> ops_off;          // per micro-batch: device records (conv_tc_cell_op) in the workspace
-        unsigned int smem = 0, tmem = 0, smem_budget = 0;
-        int ctas = 0;
+        size_t ops_off = 0;                   // device records (conv_pipe_cell_op) in the workspace
+        unsigned int smem = 0, tmem = 0;
         bool ready = false;
     };
     int opt_cell = 0;          // CTAs of a persistent forward cell kernel; 0: every convolution is its own launch
+    std::vector<CellRun> cell_runs;
+    std::vector<int> cell_of_op;              // conv -> run, or -1
+    std::vector<size_t> cell_bar_off;         // per stream of cells: the grid barrier's two words (zeroed at bind)
     // Stage lanes: a stage keeps up to `lanes` of its micro-batches under way at once, micro-batch m on lane m % lanes; every
     // lane has its own streams and its own scratch, so cells of different lanes share nothing but the parameters.  One
     // lane is the paper's schedule (a stage works through its micro-batches one after the other).
@@ -119,17 +120,22 @@ struct hpf_model {
     int n_slots() const { return P * lanes(); }
     int slot_of(int p, int m) const { return p * lanes() + m % lanes(); }
     int opt_pdl_late_from = 8;   // forward cells that run while at least this many cells are under way trigger their successors late
-    std::vector<CellRun> cell_runs;
-    std::vector<int> cell_of_op;              // conv -> run, or -1
-    std::vector<size_t> cell_bar_off;         // per partition: the grid barrier's two words (zeroed at bind)
+    // Groups: on one GPU the stages share the same SMs, and a micro-batch's launches are too small to fill them, so one launch
+    // covers `group_size()` micro-batches of a stage wherever nothing asks for cells of their own.  Every micro-batch keeps
+    // its own statistics, losses and gradient slot, formed in the same order whatever the size of the group.
+    int group_size() const;
+    int n_groups() const { const int g = group_size(); return (M + g - 1) / g; }
     int opt_fuse_bn = 3;       // bit 0: BN statistics in the producing convolution's write-out, bit 1: BN+ReLU applied by the reading convolution
     std::vector<GradEdge> edge0;              // per op: contribution to src0
     std::vector<AccumAction> accums;
     std::vector<std::vector<MessagePlan>> msg_plan;   // per cut
     // memory plan (byte offsets into the workspace)
-    std::vector<size_t> act_off, grad_off, stats_off;   // [m * n_ops + op]
-    std::vector<size_t> bn_scratch_off, conv_scratch_off;   // per stream slot (partition, lane)
-    std::vector<size_t> splitk_off, splitk_bytes;            // per stream: tickets + partial tiles of K-split convolutions (zeroed at bind)
+    // tensors: micro-batch m of op i starts at act_off[i] + m * tensor_stride[i] floats (contiguous for whole multiples of 16)
+    std::vector<size_t> act_off, grad_off, stats_off;   // per op
+    std::vector<int64_t> tensor_stride;
+    // scratch, per partition; what a micro-batch needs of its own is indexed by the micro-batch
+    std::vector<size_t> bn_scratch_off, bn_scratch_bytes_, conv_scratch_off, conv_scratch_ms;
+    std::vector<size_t> splitk_off, splitk_bytes;            // tickets + partial tiles of K-split convolutions (zeroed at bind)
     // the backward kernels of a partition have scratch of their own: in the one-graph schedule (hpf_forward_backward) a
     // partition's backward cells run while its forward cells of later micro-batches are still under way
     std::vector<size_t> bn_scratch_bwd_off, splitk_bwd_off;
@@ -153,8 +159,9 @@ struct hpf_model {
     std::vector<cudaEvent_t> ev_fdone, ev_bjoin;   // forward (P-1, m) done; backward stream p done
     std::vector<cudaEvent_t> ev_side, ev_side_join;   // per partition: gradient ready -> side stream; side stream done
     cudaEvent_t ev_fork = nullptr, ev_sync = nullptr;
-    // tensor-core plans [m * n_ops + op] per pass
-    std::vector<ConvTcPlan> tc_plan[3];
+    // tensor-core plans per op: forward / data gradient, weight gradient
+    std::vector<ConvPipePlan> pipe_plan[2];
+    std::vector<ConvTcPlan> wgrad_plan;
     std::vector<char> use_tc[3];              // per op
     // graphs
     struct FwdGraph { const float* x = nullptr; const int32_t* labels = nullptr; cudaGraphExec_t exec = nullptr; int64_t nodes = 0; };
@@ -171,14 +178,11 @@ struct hpf_model {
     int state = ST_CREATED;
     int64_t launches = 0;
 
-    float* act(int op, int m) const { return reinterpret_cast<float*>(ws + act_off[(size_t)m * n_ops + op]); }
-    float* grad(int op, int m) const { return reinterpret_cast<float*>(ws + grad_off[(size_t)m * n_ops + op]); }
-    float* stats(int op, int m) const { return reinterpret_cast<float*>(ws + stats_off[(size_t)m * n_ops + op]); }
-    float* bn_partials(int bn, int m) const
-    {
-        const int p = ops[bn].part;
-        return reinterpret_cast<float*>(ws + bn_scratch_off[slot_of(p, m)] + 256 + (size_t)bn_buf[bn] * bn_part_bytes[p]);
-    }
+    float* act(int op, int m) const { return reinterpret_cast<float*>(ws + act_off[op]) + m * tensor_stride[op]; }
+    float* grad(int op, int m) const { return reinterpret_cast<float*>(ws + grad_off[op]) + m * tensor_stride[op]; }
+    float* stats(int op, int m) const { return reinterpret_cast<float*>(ws + stats_off[op]) + (int64_t)m * 2 * ops[op].C; }
+    float* moments(int bn) const { return reinterpret_cast<float*>(ws + bn_moments_off[bn]); }
+    bool contiguous(int op) const { return op < 0 || tensor_stride[op] == numel(op); }
     unsigned long long* cell_time_slot(int phase, int p, int m) const
     {
         return reinterpret_cast<unsigned long long*>(ws + cell_times_off) + 2 * (((size_t)(phase == PH_BWD) * P + p) * M + m);
@@ -187,6 +191,14 @@ struct hpf_model {
     cudaStream_t stream_of(int p, int m = 0) const { return opt_single ? streams[0] : streams[slot_of(p, m)]; }
     DeviceStatus* status() const { return reinterpret_cast<DeviceStatus*>(ws + status_off); }
 };
+
+int hpf_model::group_size() const
+{
+    if (opt_messages || opt_cell_times || lanes() > 1) return 1;
+    const char* v = getenv("HPF_GROUP");
+    int g = v ? atoi(v) : M;
+    return g < 1 ? 1 : (g > M ? M : g);
+}
 
 namespace {
 
@@ -386,7 +398,8 @@ void build_fusion_plan(hpf_model* mdl)
 }
 
 ConvShape conv_shape_of(const hpf_model* mdl, int i);
-bool op_uses_tc(const hpf_model* mdl, int i, int pass);
+int passes_of(const hpf_model* mdl);
+bool op_uses_tc(hpf_model* mdl, int i, int pass);
 
 ConvShape conv_shape_of(const hpf_model* mdl, int i)
 {
@@ -394,51 +407,44 @@ ConvShape conv_shape_of(const hpf_model* mdl, int i)
     return make_conv_shape(mdl->b, o.iH, o.iW, o.iC, o.op.c_out, o.op.ksize, o.op.stride, o.op.pad);
 }
 
+int passes_of(const hpf_model* mdl) { return mdl->opt_conv_path == 2 ? 1 : 3; }
+
 // Which convolutions run on the tensor cores, and which BN work rides inside them: the statistics of a BN in the
 // forward kernel that produces its input (only when producer and BN run back to back on the same stream: same
-// partition, nothing but a fused residual add between them, so that the per-stream scratch can carry the per-tile
-// sums), and the BN+ReLU itself on the operand path of the convolution that reads it.
+// partition, nothing but a fused residual add between them), and the BN+ReLU itself on the operand path of the convolution
+// that reads it.
 void build_kernel_plan(hpf_model* mdl)
 {
     const int n = mdl->n_ops;
+    for (int pass = 0; pass < 2; ++pass) mdl->pipe_geom[pass].assign(n, ConvPipeGeom());
     for (int pass = 0; pass < 3; ++pass) {
         mdl->use_tc[pass].assign(n, 0);
         for (int i = 0; i < n; ++i) mdl->use_tc[pass][i] = op_uses_tc(mdl, i, pass) ? 1 : 0;
     }
     mdl->bn_fwd_from.assign(n, -1);
     mdl->conv_fwd_bn.assign(n, -1);
-    mdl->bn_into.assign(n, -1); mdl->conv_in_bn.assign(n, -1); mdl->bn_late.assign(n, 0); mdl->bn_buf.assign(n, 0);
-    std::vector<int> n_fused(mdl->P, 0);
-    if (!mdl->opt_fuse_bn) return;
+    mdl->bn_into.assign(n, -1); mdl->conv_in_bn.assign(n, -1);
+    if (!(mdl->opt_fuse_bn & 1)) return;
     for (int j = 0; j < n; ++j) {
         const OpInfo& bn = mdl->ops[j];
-        if (bn.op.kind != HPF_OP_BNRELU || bn.C > 2048) continue;
+        if (bn.op.kind != HPF_OP_BNRELU) continue;
         // forward: the kernel that writes the BN's input
         int t = bn.op.src0, prod = -1;
         if (mdl->ops[t].op.kind == HPF_OP_CONV && mdl->fused_into[t] < 0) prod = t;
         else if (mdl->ops[t].op.kind == HPF_OP_ADD && mdl->add_done_by[t] >= 0) prod = mdl->add_done_by[t];
-        if ((mdl->opt_fuse_bn & 1) && prod >= 0 && mdl->use_tc[PASS_FWD][prod] && mdl->ops[prod].part == bn.part && mdl->conv_fwd_bn[prod] < 0 &&
-            conv_tc_can_fuse_bn(conv_shape_of(mdl, prod), PASS_FWD)) {
-            bool adjacent = true;
-            for (int k = prod + 1; k < j; ++k)
-                if (!(mdl->ops[k].op.kind == HPF_OP_ADD && mdl->add_done_by[k] >= 0)) adjacent = false;
-            if (adjacent) {
-                mdl->bn_fwd_from[j] = prod; mdl->conv_fwd_bn[prod] = j;
-                // A convolution that reads BN j's sums may still be reading them while its own write-out already
-                // produces the next BN's: successive fused BNs of a stream alternate between two buffers.
-                mdl->bn_buf[j] = n_fused[bn.part]++ & 1;
-            }
-        }
+        if (prod < 0 || !mdl->use_tc[PASS_FWD][prod] || mdl->ops[prod].part != bn.part || mdl->conv_fwd_bn[prod] >= 0 ||
+            !conv_pipe_can_fuse_bn_output(mdl->pipe_geom[PASS_FWD][prod])) continue;
+        bool adjacent = true;
+        for (int k = prod + 1; k < j; ++k)
+            if (!(mdl->ops[k].op.kind == HPF_OP_ADD && mdl->add_done_by[k] >= 0)) adjacent = false;
+        if (!adjacent) continue;
+        mdl->bn_fwd_from[j] = prod; mdl->conv_fwd_bn[prod] = j;
         // the BN+ReLU itself: applied by its only reader, the next op, a stride-1 tensor-core convolution
-        if ((mdl->opt_fuse_bn & 2) && mdl->bn_fwd_from[j] >= 0 && bn.consumers.size() == 1 && bn.consumers[0] == j + 1) {
+        if ((mdl->opt_fuse_bn & 2) && bn.consumers.size() == 1 && bn.consumers[0] == j + 1) {
             const int i = j + 1;
-            if (mdl->ops[i].op.kind == HPF_OP_CONV && mdl->ops[i].op.src0 == j && mdl->use_tc[PASS_FWD][i] &&
-                mdl->ops[i].part == bn.part && conv_tc_can_fuse_bn_input(conv_shape_of(mdl, i))) {
+            if (mdl->ops[i].op.kind == HPF_OP_CONV && mdl->ops[i].op.src0 == j && mdl->use_tc[PASS_FWD][i] && mdl->ops[i].part == bn.part &&
+                conv_pipe_can_fuse_bn_input(conv_shape_of(mdl, i))) {
                 mdl->bn_into[j] = i; mdl->conv_in_bn[i] = j;
-                // Few per-tile sums: the reading convolution adds them under the latency of its first copy and the
-                // producer ends without a ticket.  Many: the producer's last CTA adds them once.
-                const long long floats = (long long)conv_tc_tiles(conv_shape_of(mdl, mdl->bn_fwd_from[j]), PASS_FWD) * 2 * bn.C;
-                mdl->bn_late[j] = floats <= mdl->opt_bn_late_floats ? 1 : 0;
             }
         }
     }
@@ -473,6 +479,7 @@ void build_cell_runs(hpf_model* mdl)
     }
 }
 
+
 // ------------------------------------------------------------------------------------------------
 // memory plan
 // ------------------------------------------------------------------------------------------------
@@ -486,69 +493,43 @@ void build_memory_plan(hpf_model* mdl)
     // region that must start as zeros: status word and BN tickets (with their partials)
     mdl->zero_lo = at;
     mdl->status_off = take(sizeof(DeviceStatus));
-    const int L = mdl->lanes(), S = P * L;
-    mdl->bn_scratch_off.assign(S, 0);
-    mdl->conv_scratch_off.assign(S, 0);
-    mdl->bn_part_bytes.assign(P, 0);
+    mdl->bn_scratch_off.assign(P, 0); mdl->bn_scratch_bwd_off.assign(P, 0); mdl->bn_scratch_bytes_.assign(P, 256);
+    mdl->splitk_off.assign(P, 0); mdl->splitk_bwd_off.assign(P, 0); mdl->splitk_bytes.assign(P, 0);
     for (int p = 0; p < P; ++p) {
-        size_t bn = 256, part = 0;
-        for (int i = mdl->part_lo[p]; i < mdl->part_hi[p]; ++i)
-            if (mdl->ops[i].op.kind == HPF_OP_BNRELU || mdl->ops[i].op.kind == HPF_OP_BN) {
-                const OpInfo& o = mdl->ops[i];
-                size_t need = bn_scratch_bytes((int64_t)mdl->b * o.H * o.W, o.C);
-                if (need > bn) bn = need;
-                const int from = mdl->bn_fwd_from[i];
-                if (from >= 0) {
-                    need = align_up((size_t)conv_tc_tiles(conv_shape_of(mdl, from), PASS_FWD) * 2 * o.C * sizeof(float), 256);
-                    if (need > part) part = need;
-                }
-            }
-        mdl->bn_part_bytes[p] = part;
-        if (256 + 2 * part > bn) bn = 256 + 2 * part;
-        for (int l = 0; l < L; ++l) mdl->bn_scratch_off[p * L + l] = take(bn);
-    }
-    mdl->splitk_off.assign(S, 0); mdl->splitk_bytes.assign(P, 0);
-    for (int p = 0; p < P; ++p) {
-        size_t need = 0;
-        if (mdl->opt_conv_path != 1)
-            for (int i = mdl->part_lo[p]; i < mdl->part_hi[p]; ++i)
-                if (mdl->ops[i].op.kind == HPF_OP_CONV) {
-                    const ConvShape s = conv_shape_of(mdl, i);
-                    need = std::max(need, std::max(conv_tc_splitk_bytes(s, PASS_FWD, 3), conv_tc_splitk_bytes(s, PASS_DGRAD, 3)));
-                }
-        mdl->splitk_bytes[p] = need;
-        for (int l = 0; l < L; ++l) mdl->splitk_off[p * L + l] = take(need ? need : 16);
-    }
-    mdl->bn_scratch_bwd_off.assign(S, 0); mdl->splitk_bwd_off.assign(S, 0);
-    for (int p = 0; p < P; ++p) {
-        size_t bn = 256;
-        for (int i = mdl->part_lo[p]; i < mdl->part_hi[p]; ++i)
-            if (mdl->ops[i].op.kind == HPF_OP_BNRELU || mdl->ops[i].op.kind == HPF_OP_BN)
-                bn = std::max(bn, bn_scratch_bytes((int64_t)mdl->b * mdl->ops[i].H * mdl->ops[i].W, mdl->ops[i].C));
-        for (int l = 0; l < L; ++l) {
-            mdl->bn_scratch_bwd_off[p * L + l] = take(bn);
-            mdl->splitk_bwd_off[p * L + l] = take(mdl->splitk_bytes[p] ? mdl->splitk_bytes[p] : 16);
+        size_t bn = 256, sk = 0;
+        for (int i = mdl->part_lo[p]; i < mdl->part_hi[p]; ++i) {
+            const OpInfo& o = mdl->ops[i];
+            if (o.op.kind == HPF_OP_BNRELU || o.op.kind == HPF_OP_BN) bn = std::max(bn, bn_scratch_bytes((int64_t)mdl->b * o.H * o.W, o.C));
+            if (o.op.kind == HPF_OP_CONV && mdl->opt_conv_path != 1)
+                for (int pass : {PASS_FWD, PASS_DGRAD})
+                    if (mdl->use_tc[pass][i]) sk = std::max(sk, conv_pipe_splitk_bytes(conv_shape_of(mdl, i), pass, passes_of(mdl), M));
         }
+        mdl->bn_scratch_bytes_[p] = align_up(bn, 256);
+        mdl->splitk_bytes[p] = sk;
+        mdl->bn_scratch_off[p] = take(mdl->bn_scratch_bytes_[p] * M);
+        mdl->bn_scratch_bwd_off[p] = take(mdl->bn_scratch_bytes_[p] * M);
+        mdl->splitk_off[p] = take(sk ? sk * M : 16);
+        mdl->splitk_bwd_off[p] = take(sk ? sk * M : 16);
     }
-    mdl->cell_bar_off.assign(S, 0);
-    for (int k = 0; k < S; ++k) mdl->cell_bar_off[k] = take(16);
+    mdl->cell_bar_off.assign(mdl->n_slots(), 0);
+    for (size_t& off : mdl->cell_bar_off) off = take(16);
     mdl->zero_hi = at;
     build_cell_runs(mdl);
-    for (auto& run : mdl->cell_runs) {
-        run.ops_off.assign(M, 0);
-        for (int m = 0; m < M; ++m) run.ops_off[m] = take(conv_tc_cell_op_bytes() * run.convs.size());
-    }
+    for (auto& run : mdl->cell_runs) run.ops_off = take(conv_pipe_cell_op_bytes() * run.convs.size());
+    mdl->bn_moments_off.assign(n, 0);
+    for (int j = 0; j < n; ++j)
+        if (mdl->bn_fwd_from[j] >= 0)
+            mdl->bn_moments_off[j] = take(sizeof(float) * M * conv_pipe_partial_floats(mdl->pipe_geom[PASS_FWD][mdl->bn_fwd_from[j]].blocks_per_m, mdl->ops[j].C));
+    mdl->conv_scratch_off.assign(P, 0); mdl->conv_scratch_ms.assign(P, 0);
     for (int p = 0; p < P; ++p) {
         size_t cv = 256;
         for (int i = mdl->part_lo[p]; i < mdl->part_hi[p]; ++i)
             if (mdl->ops[i].op.kind == HPF_OP_CONV) {
                 const ConvShape s = conv_shape_of(mdl, i);
-                size_t need = conv_simt_scratch_bytes(s);
-                size_t need2 = conv_tc_scratch_bytes(s);
-                if (need2 > need) need = need2;
-                if (need > cv) cv = need;
+                cv = std::max(cv, std::max(conv_simt_scratch_bytes(s), conv_tc_scratch_bytes(s, M)));
             }
-        for (int l = 0; l < L; ++l) mdl->conv_scratch_off[p * L + l] = take(cv);
+        mdl->conv_scratch_ms[p] = align_up(cv, 256);
+        mdl->conv_scratch_off[p] = take(mdl->conv_scratch_ms[p] * M);
     }
     mdl->cell_times_off = take(sizeof(unsigned long long) * 2 * 2 * (size_t)P * M);
     mdl->loss_slots_off = take(sizeof(float) * M);
@@ -564,21 +545,17 @@ void build_memory_plan(hpf_model* mdl)
         mdl->pooled_off[m] = take(sizeof(float) * (size_t)mdl->b * headC);
         mdl->persample_off[m] = take(sizeof(float) * (size_t)mdl->b);
     }
-    mdl->act_off.assign((size_t)n * M, 0); mdl->grad_off.assign((size_t)n * M, 0); mdl->stats_off.assign((size_t)n * M, 0);
-    for (int m = 0; m < M; ++m) {
-        for (int i = n - 1; i >= 0; --i) {
-            const int f = mdl->fused_into[i];
-            if (f >= 0) mdl->act_off[(size_t)m * n + i] = mdl->act_off[(size_t)m * n + f];   // f > i: already placed
-            else mdl->act_off[(size_t)m * n + i] = take(sizeof(float) * (size_t)mdl->numel(i));
-        }
-        for (int i = n - 1; i >= 0; --i) {
-            const int a = mdl->grad_alias[i];
-            if (a >= 0) mdl->grad_off[(size_t)m * n + i] = mdl->grad_off[(size_t)m * n + a];   // a > i: already placed
-            else mdl->grad_off[(size_t)m * n + i] = take(sizeof(float) * (size_t)mdl->numel(i));
-        }
-        for (int i = 0; i < n; ++i)
-            if (mdl->ops[i].op.kind == HPF_OP_BNRELU || mdl->ops[i].op.kind == HPF_OP_BN)
-                mdl->stats_off[(size_t)m * n + i] = take(sizeof(float) * 2 * (size_t)mdl->ops[i].C);
+    mdl->act_off.assign(n, 0); mdl->grad_off.assign(n, 0); mdl->stats_off.assign(n, 0); mdl->tensor_stride.assign(n, 0);
+    for (int i = 0; i < n; ++i) {
+        const int64_t e = mdl->numel(i);
+        mdl->tensor_stride[i] = e % 16 == 0 ? e : (e + 63) / 64 * 64;       // whole micro-batches side by side: one launch, one tensor map
+    }
+    for (int i = n - 1; i >= 0; --i) {
+        const int f = mdl->fused_into[i], a = mdl->grad_alias[i];              // f, a > i: already placed
+        mdl->act_off[i] = f >= 0 ? mdl->act_off[f] : take(sizeof(float) * (size_t)mdl->tensor_stride[i] * M);
+        mdl->grad_off[i] = a >= 0 ? mdl->grad_off[a] : take(sizeof(float) * (size_t)mdl->tensor_stride[i] * M);
+        if (mdl->ops[i].op.kind == HPF_OP_BNRELU || mdl->ops[i].op.kind == HPF_OP_BN)
+            mdl->stats_off[i] = take(sizeof(float) * 2 * (size_t)mdl->ops[i].C * M);
     }
     mdl->fmsg_off.assign(mdl->cuts.size(), {}); mdl->bmsg_off.assign(mdl->cuts.size(), {});
     if (mdl->opt_messages)
@@ -594,7 +571,7 @@ void build_memory_plan(hpf_model* mdl)
     mdl->planned = true;
 }
 
-bool op_uses_tc(const hpf_model* mdl, int i, int pass)
+bool op_uses_tc(hpf_model* mdl, int i, int pass)
 {
     if (mdl->opt_conv_path == 1) return false;
     if (mdl->ops[i].op.kind != HPF_OP_CONV) return false;
@@ -602,7 +579,8 @@ bool op_uses_tc(const hpf_model* mdl, int i, int pass)
     if (mdl->ops[i].w_off % 4) return false;            // the weight tensor map needs a 16-byte aligned base
     // a strided data gradient zero-fills between its samples, so it cannot also add to what is there
     if (pass == PASS_DGRAD && mdl->ops[i].op.stride > 1 && (mdl->edge0[i].accumulate || mdl->edge0[i].addend >= 0)) return false;
-    return conv_tc_supported(conv_shape_of(mdl, i), pass);
+    if (pass == PASS_WGRAD) return conv_tc_supported(conv_shape_of(mdl, i), pass);
+    return conv_pipe_geom(conv_shape_of(mdl, i), pass, passes_of(mdl), mdl->M, &mdl->pipe_geom[pass][i]);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -614,137 +592,6 @@ const float* src_act(const hpf_model* mdl, int src, int m)
     return mdl->act(src, m);
 }
 
-// sl: the stream slot (partition, lane) whose scratch and side stream the op uses
-int forward_op(hpf_model* mdl, int i, int m, cudaStream_t st, int sl)
-{
-    const OpInfo& o = mdl->ops[i];
-    const hpf_op& q = o.op;
-    const float* in0 = src_act(mdl, q.src0, m);
-    float* out = mdl->act(i, m);
-    switch (q.kind) {
-    case HPF_OP_CONV: {
-        // with a fused residual ADD, `out` is the ADD's output tensor and the other addend rides in the epilogue
-        const float* residual = nullptr;
-        if (mdl->fused_into[i] >= 0) {
-            const hpf_op& a = mdl->ops[mdl->fused_into[i]].op;
-            residual = mdl->act(a.src0 == i ? a.src1 : a.src0, m);
-        }
-        if (mdl->cell_of_op[i] >= 0 && mdl->cell_runs[mdl->cell_of_op[i]].ready) {
-            // the whole run of convolutions is one resident grid, enqueued where its first convolution stands
-            const hpf_model::CellRun& run = mdl->cell_runs[mdl->cell_of_op[i]];
-            if (run.convs[0] == i)
-                CU(conv_tc_cell_launch(mdl->ws + run.ops_off[m], (int)run.convs.size(), run.ctas, run.smem, run.tmem,
-                                       reinterpret_cast<unsigned int*>(mdl->ws + mdl->cell_bar_off[sl]), mdl->status(), st, &mdl->launches));
-        } else if (mdl->use_tc[PASS_FWD][i]) {
-            CU(conv_tc_launch(&mdl->tc_plan[PASS_FWD][(size_t)m * mdl->n_ops + i], mdl->status(), st, &mdl->launches));
-        } else {
-            CU(conv_fwd_simt(in0, mdl->params + o.w_off, out, residual, conv_shape_of(mdl, i), st, &mdl->launches));
-        }
-        break;
-    }
-    case HPF_OP_BNRELU:
-        if (mdl->bn_into[i] >= 0) break;   // the convolution that reads this BN applies it (and stores `out` and the statistics)
-        if (mdl->bn_fwd_from[i] >= 0)      // the producing convolution left mean and 1/sigma
-            CU(bnrelu_fwd_apply(in0, mdl->params + o.w_off, mdl->params + o.b_off, mdl->stats(i, m), out,
-                                (int64_t)mdl->b * o.H * o.W, o.C, st, &mdl->launches));
-        else
-            CU(bnrelu_fwd(in0, mdl->params + o.w_off, mdl->params + o.b_off, q.eps, out, mdl->stats(i, m),
-                          (int64_t)mdl->b * o.H * o.W, o.C, mdl->ws + mdl->bn_scratch_off[sl], st, &mdl->launches));
-        break;
-    case HPF_OP_BN:                        // batch normalisation without the activation
-        CU(bnrelu_fwd(in0, mdl->params + o.w_off, mdl->params + o.b_off, q.eps, out, mdl->stats(i, m),
-                      (int64_t)mdl->b * o.H * o.W, o.C, mdl->ws + mdl->bn_scratch_off[sl], st, &mdl->launches, false));
-        break;
-    case HPF_OP_RELU:
-        CU(relu_fwd(in0, out, mdl->numel(i), st, &mdl->launches));
-        break;
-    case HPF_OP_ADD:
-        if (mdl->add_done_by[i] < 0) CU(add_fwd(in0, mdl->act(q.src1, m), out, mdl->numel(i), st, &mdl->launches));
-        break;
-    case HPF_OP_MAXPOOL:
-        CU(maxpool_fwd(in0, out, conv_shape_of(mdl, i), st, &mdl->launches));
-        break;
-    case HPF_OP_HEAD:
-        CU(head_fwd(in0, mdl->params + o.w_off, mdl->params + o.b_off, mdl->cur_labels + (int64_t)m * mdl->b, out,
-                    reinterpret_cast<float*>(mdl->ws + mdl->pooled_off[m]),
-                    reinterpret_cast<float*>(mdl->ws + mdl->persample_off[m]),
-                    reinterpret_cast<float*>(mdl->ws + mdl->loss_slots_off) + m, mdl->b, o.iH * o.iW, o.iC, q.c_out, st,
-                    &mdl->launches));
-        break;
-    }
-    return HPF_OK;
-}
-
-int backward_op(hpf_model* mdl, int i, int m, cudaStream_t st, int sl)
-{
-    const OpInfo& o = mdl->ops[i];
-    const hpf_op& q = o.op;
-    const GradEdge& e = mdl->edge0[i];
-    // explicit accumulations scheduled at this op
-    for (const AccumAction& a : mdl->accums)
-        if (a.at == i) CU(grad_accumulate(mdl->grad(a.dst, m), mdl->grad(a.src, m), mdl->numel(a.dst), a.accumulate != 0, st, &mdl->launches));
-    const float* in0 = src_act(mdl, q.src0, m);
-    float* dout = mdl->grad(i, m);
-    float* slot = mdl->gslots + (int64_t)m * mdl->G;
-    const float* addend = e.addend >= 0 ? mdl->grad(e.addend, m) : nullptr;
-    switch (q.kind) {
-    case HPF_OP_CONV: {
-        const ConvShape s = conv_shape_of(mdl, i);
-        // The weight gradient feeds nothing but the final average, so it leaves the chain of dependent kernels:
-        // it runs on the partition's side stream once dL/d(output) is ready (everything before this point on st).
-        cudaStream_t wst = st;
-        if (!mdl->side.empty() && !mdl->opt_single) {
-            wst = mdl->side[sl];
-            CU(cudaEventRecord(mdl->ev_side[sl], st));
-            CU(cudaStreamWaitEvent(wst, mdl->ev_side[sl], 0));
-        }
-        if (mdl->use_tc[PASS_WGRAD][i]) {
-            CU(conv_tc_launch(&mdl->tc_plan[PASS_WGRAD][(size_t)m * mdl->n_ops + i], mdl->status(), wst, &mdl->launches));
-        } else {
-            CU(conv_wgrad_simt(in0, dout, slot + o.w_off, s, mdl->ws + mdl->conv_scratch_off[sl], wst, &mdl->launches));
-        }
-        if (q.src0 >= 0) {
-            if (mdl->use_tc[PASS_DGRAD][i]) {
-                CU(conv_tc_launch(&mdl->tc_plan[PASS_DGRAD][(size_t)m * mdl->n_ops + i], mdl->status(), st, &mdl->launches));
-            } else {
-                CU(conv_dgrad_simt(dout, mdl->params + o.w_off, mdl->grad(q.src0, m), addend, e.accumulate != 0, s, st, &mdl->launches));
-            }
-        }
-        break;
-    }
-    case HPF_OP_BNRELU:
-        CU(bnrelu_bwd(in0, dout, mdl->params + o.w_off, mdl->params + o.b_off, mdl->stats(i, m), mdl->grad(q.src0, m), addend,
-                      e.accumulate != 0, slot + o.w_off, slot + o.b_off, (int64_t)mdl->b * o.H * o.W, o.C,
-                      mdl->ws + mdl->bn_scratch_bwd_off[sl], st, &mdl->launches, true, true));
-        break;
-    case HPF_OP_BN:
-        CU(bnrelu_bwd(in0, dout, mdl->params + o.w_off, mdl->params + o.b_off, mdl->stats(i, m), mdl->grad(q.src0, m), addend,
-                      e.accumulate != 0, slot + o.w_off, slot + o.b_off, (int64_t)mdl->b * o.H * o.W, o.C,
-                      mdl->ws + mdl->bn_scratch_bwd_off[sl], st, &mdl->launches, false, true));
-        break;
-    case HPF_OP_RELU:
-        CU(relu_bwd(in0, dout, mdl->grad(q.src0, m), addend, e.accumulate != 0, mdl->numel(i), st, &mdl->launches));
-        break;
-    case HPF_OP_ADD:
-        break;   // its contributions are aliases, on-the-fly addends, or the explicit accumulations above
-    case HPF_OP_MAXPOOL:
-        if (q.src0 >= 0)
-            CU(maxpool_bwd(in0, dout, mdl->grad(q.src0, m), e.accumulate != 0, conv_shape_of(mdl, i), st, &mdl->launches));
-        break;
-    case HPF_OP_HEAD:
-        CU(head_bwd(mdl->params + o.w_off, mdl->cur_labels + (int64_t)m * mdl->b, mdl->act(i, m),
-                    reinterpret_cast<float*>(mdl->ws + mdl->pooled_off[m]), dout, mdl->grad(q.src0, m), slot + o.w_off,
-                    slot + o.b_off, mdl->b, o.iH * o.iW, o.iC, q.c_out, st, &mdl->launches));
-        break;
-    }
-    return HPF_OK;
-}
-
-// phase PH_FWD / PH_BWD / PH_AVG: one phase, forked from and joined into stream 0.  PH_FB: forward and backward as ONE
-// set of dependencies (hpf_forward_backward): the backward cell (p, m) runs on partition p's backward stream as soon as
-// the cell that feeds it has finished - backward (p+1, m), or forward (P-1, m) for the last partition - while the
-// partition's forward stream may still be busy with later micro-batches.  Same kernels on the same data as the two
-// phases, so the results are bit-identical; only the idle slots of the forward drain and the backward fill get used.
 // Cells under way, roughly, while cell (p, m) of the forward (bwd = false) or backward phase runs in the one-graph schedule:
 // the stages busy at its own tick plus those of the other phase at the tick that runs at the same time (the backward
 // pipeline starts when the first micro-batch has passed all P stages).
@@ -762,11 +609,165 @@ int cells_under_way(int P, int M, int p, int m, bool bwd)
     return bwd ? busy(t) + busy(t + P) : busy(t) + busy(t - P);
 }
 
+// Ops of one stage on the micro-batches m .. m + g - 1.  sl: the stream slot (partition, lane) whose side stream is used.
+// Launches that know nothing of micro-batches take the group as one larger batch where its tensors are contiguous.
+int forward_op(hpf_model* mdl, int i, int m, int g, cudaStream_t st, int sl)
+{
+    (void)sl;
+    const OpInfo& o = mdl->ops[i];
+    const hpf_op& q = o.op;
+    if (g > 1 && q.kind != HPF_OP_HEAD && !(mdl->contiguous(i) && mdl->contiguous(q.src0) && (q.kind != HPF_OP_ADD || mdl->contiguous(q.src1)))) {
+        for (int k = 0; k < g; ++k) { int rc = forward_op(mdl, i, m + k, 1, st, sl); if (rc) return rc; }
+        return HPF_OK;
+    }
+    const float* in0 = src_act(mdl, q.src0, m);
+    float* out = mdl->act(i, m);
+    const int64_t rows = (int64_t)mdl->b * o.H * o.W;
+    BnGroup grp;
+    grp.count = g; grp.x = mdl->tensor_stride[i]; grp.stats = 2 * o.C; grp.param = mdl->G; grp.scratch = (int64_t)mdl->bn_scratch_bytes_[o.part];
+    void* bn_scratch = mdl->ws + mdl->bn_scratch_off[o.part] + m * mdl->bn_scratch_bytes_[o.part];
+    ConvShape gs;
+    if (q.kind == HPF_OP_CONV || q.kind == HPF_OP_MAXPOOL) { gs = conv_shape_of(mdl, i); gs.N *= g; }
+    switch (q.kind) {
+    case HPF_OP_CONV: {
+        // with a fused residual ADD, `out` is the ADD's output tensor and the other addend rides in the epilogue
+        const float* residual = nullptr;
+        if (mdl->fused_into[i] >= 0) {
+            const hpf_op& a = mdl->ops[mdl->fused_into[i]].op;
+            residual = mdl->act(a.src0 == i ? a.src1 : a.src0, m);
+        }
+        if (mdl->use_tc[PASS_FWD][i]) {
+            const bool late = cells_under_way(mdl->P, mdl->n_groups(), o.part, m / mdl->group_size(), false) * mdl->lanes() >= mdl->opt_pdl_late_from;
+            const int cell = mdl->cell_of_op[i];
+            if (cell >= 0 && mdl->cell_runs[cell].ready) {
+                // the whole run of convolutions is one resident grid, enqueued where its first convolution stands
+                const hpf_model::CellRun& run = mdl->cell_runs[cell];
+                if (run.convs[0] == i)
+                    CU(conv_pipe_cell_launch(mdl->ws + run.ops_off, (int)run.convs.size(), m, g, mdl->opt_cell, run.smem, run.tmem,
+                                             reinterpret_cast<unsigned int*>(mdl->ws + mdl->cell_bar_off[sl]), mdl->status(), st, &mdl->launches));
+            } else {
+                CU(conv_pipe_launch(&mdl->pipe_plan[PASS_FWD][i], m, g, late, mdl->status(), st, &mdl->launches));
+            }
+        }
+        else CU(conv_fwd_simt(in0, mdl->params + o.w_off, out, residual, gs, st, &mdl->launches));
+        break;
+    }
+    case HPF_OP_BNRELU:
+        if (mdl->bn_into[i] >= 0) break;   // the convolution that reads this BN applies it (and stores `out` and the statistics)
+        if (mdl->bn_fwd_from[i] >= 0) {    // the producing convolution left the moments of its units
+            const int units = mdl->pipe_geom[PASS_FWD][mdl->bn_fwd_from[i]].blocks_per_m;
+            CU(bn_finalize_partials(mdl->moments(i) + (size_t)m * conv_pipe_partial_floats(units, o.C), units, o.C, q.eps, (double)rows, mdl->stats(i, m), g, st,
+                                    &mdl->launches));
+            CU(bnrelu_fwd_apply(in0, mdl->params + o.w_off, mdl->params + o.b_off, mdl->stats(i, m), out, rows, o.C, st, &mdl->launches, grp));
+        } else {
+            CU(bnrelu_fwd(in0, mdl->params + o.w_off, mdl->params + o.b_off, q.eps, out, mdl->stats(i, m), rows, o.C, bn_scratch, st, &mdl->launches, true, grp));
+        }
+        break;
+    case HPF_OP_BN:                        // batch normalisation without the activation
+        CU(bnrelu_fwd(in0, mdl->params + o.w_off, mdl->params + o.b_off, q.eps, out, mdl->stats(i, m), rows, o.C, bn_scratch, st, &mdl->launches, false, grp));
+        break;
+    case HPF_OP_RELU:
+        CU(relu_fwd(in0, out, mdl->numel(i) * g, st, &mdl->launches));
+        break;
+    case HPF_OP_ADD:
+        if (mdl->add_done_by[i] < 0) CU(add_fwd(in0, mdl->act(q.src1, m), out, mdl->numel(i) * g, st, &mdl->launches));
+        break;
+    case HPF_OP_MAXPOOL:
+        CU(maxpool_fwd(in0, out, gs, st, &mdl->launches));
+        break;
+    case HPF_OP_HEAD:
+        for (int k = m; k < m + g; ++k)
+            CU(head_fwd(src_act(mdl, q.src0, k), mdl->params + o.w_off, mdl->params + o.b_off, mdl->cur_labels + (int64_t)k * mdl->b, mdl->act(i, k),
+                        reinterpret_cast<float*>(mdl->ws + mdl->pooled_off[k]), reinterpret_cast<float*>(mdl->ws + mdl->persample_off[k]),
+                        reinterpret_cast<float*>(mdl->ws + mdl->loss_slots_off) + k, mdl->b, o.iH * o.iW, o.iC, q.c_out, st, &mdl->launches));
+        break;
+    }
+    return HPF_OK;
+}
+
+int backward_op(hpf_model* mdl, int i, int m, int g, cudaStream_t st, int sl)
+{
+    const OpInfo& o = mdl->ops[i];
+    const hpf_op& q = o.op;
+    const GradEdge& e = mdl->edge0[i];
+    if (g > 1 && q.kind != HPF_OP_HEAD && !(mdl->contiguous(i) && mdl->contiguous(q.src0) && (q.kind != HPF_OP_ADD || mdl->contiguous(q.src1)))) {
+        for (int k = 0; k < g; ++k) { int rc = backward_op(mdl, i, m + k, 1, st, sl); if (rc) return rc; }
+        return HPF_OK;
+    }
+    // explicit accumulations scheduled at this op
+    for (const AccumAction& a : mdl->accums)
+        if (a.at == i)
+            for (int k = m; k < m + g; ++k)
+                CU(grad_accumulate(mdl->grad(a.dst, k), mdl->grad(a.src, k), mdl->numel(a.dst), a.accumulate != 0, st, &mdl->launches));
+    const float* in0 = src_act(mdl, q.src0, m);
+    float* dout = mdl->grad(i, m);
+    float* slot = mdl->gslots + (int64_t)m * mdl->G;
+    const float* addend = e.addend >= 0 ? mdl->grad(e.addend, m) : nullptr;
+    const int64_t rows = (int64_t)mdl->b * o.H * o.W;
+    BnGroup grp;
+    grp.count = g; grp.x = mdl->tensor_stride[i]; grp.stats = 2 * o.C; grp.param = mdl->G; grp.scratch = (int64_t)mdl->bn_scratch_bytes_[o.part];
+    void* bn_scratch = mdl->ws + mdl->bn_scratch_bwd_off[o.part] + m * mdl->bn_scratch_bytes_[o.part];
+    ConvShape s, gs;
+    if (q.kind == HPF_OP_CONV || q.kind == HPF_OP_MAXPOOL) { s = gs = conv_shape_of(mdl, i); gs.N *= g; }
+    switch (q.kind) {
+    case HPF_OP_CONV: {
+        // The weight gradient feeds nothing but the final average, so it leaves the chain of dependent kernels:
+        // it runs on the partition's side stream once dL/d(output) is ready (everything before this point on st).
+        cudaStream_t wst = st;
+        if (!mdl->side.empty() && !mdl->opt_single) {
+            wst = mdl->side[sl];
+            CU(cudaEventRecord(mdl->ev_side[sl], st));
+            CU(cudaStreamWaitEvent(wst, mdl->ev_side[sl], 0));
+        }
+        if (mdl->use_tc[PASS_WGRAD][i]) {
+            CU(conv_tc_launch(&mdl->wgrad_plan[i], mdl->status(), wst, &mdl->launches, m, g));
+        } else {
+            for (int k = m; k < m + g; ++k)
+                CU(conv_wgrad_simt(src_act(mdl, q.src0, k), mdl->grad(i, k), mdl->gslots + (int64_t)k * mdl->G + o.w_off, s,
+                                   mdl->ws + mdl->conv_scratch_off[o.part] + k * mdl->conv_scratch_ms[o.part], wst, &mdl->launches));
+        }
+        if (q.src0 >= 0) {
+            if (mdl->use_tc[PASS_DGRAD][i]) CU(conv_pipe_launch(&mdl->pipe_plan[PASS_DGRAD][i], m, g, false, mdl->status(), st, &mdl->launches));
+            else CU(conv_dgrad_simt(dout, mdl->params + o.w_off, mdl->grad(q.src0, m), addend, e.accumulate != 0, gs, st, &mdl->launches));
+        }
+        break;
+    }
+    case HPF_OP_BNRELU:
+    case HPF_OP_BN:
+        CU(bnrelu_bwd(in0, dout, mdl->params + o.w_off, mdl->params + o.b_off, mdl->stats(i, m), mdl->grad(q.src0, m), addend,
+                      e.accumulate != 0, slot + o.w_off, slot + o.b_off, rows, o.C, bn_scratch, st, &mdl->launches, q.kind == HPF_OP_BNRELU, true, grp));
+        break;
+    case HPF_OP_RELU:
+        CU(relu_bwd(in0, dout, mdl->grad(q.src0, m), addend, e.accumulate != 0, mdl->numel(i) * g, st, &mdl->launches));
+        break;
+    case HPF_OP_ADD:
+        break;   // its contributions are aliases, on-the-fly addends, or the explicit accumulations above
+    case HPF_OP_MAXPOOL:
+        if (q.src0 >= 0)
+            CU(maxpool_bwd(in0, dout, mdl->grad(q.src0, m), e.accumulate != 0, gs, st, &mdl->launches));
+        break;
+    case HPF_OP_HEAD:
+        for (int k = m; k < m + g; ++k) {
+            float* sl_k = mdl->gslots + (int64_t)k * mdl->G;
+            CU(head_bwd(mdl->params + o.w_off, mdl->cur_labels + (int64_t)k * mdl->b, mdl->act(i, k), reinterpret_cast<float*>(mdl->ws + mdl->pooled_off[k]),
+                        mdl->grad(i, k), mdl->grad(q.src0, k), sl_k + o.w_off, sl_k + o.b_off, mdl->b, o.iH * o.iW, o.iC, q.c_out, st, &mdl->launches));
+        }
+        break;
+    }
+    return HPF_OK;
+}
+
+// phase PH_FWD / PH_BWD / PH_AVG: one phase, forked from and joined into stream 0.  PH_FB: forward and backward as ONE
+// set of dependencies (hpf_forward_backward): the backward cell (p, m) runs on partition p's backward stream as soon as
+// the cell that feeds it has finished - backward (p+1, m), or forward (P-1, m) for the last partition - while the
+// partition's forward stream may still be busy with later micro-batches.  Same kernels on the same data as the two
+// phases, so the results are bit-identical; only the idle slots of the forward drain and the backward fill get used.
 int enqueue_phase(hpf_model* mdl, int phase)
 {
     const PdlScope pdl_scope(mdl->opt_pdl);
     const BnClusterScope bn_cluster_scope(mdl->opt_bn_cluster);
-    const int P = mdl->P, M = mdl->M;
+    const int P = mdl->P, M = mdl->n_groups(), gs = mdl->group_size();          // a cell is a group of micro-batches here
+    auto group = [&](int k) { return std::min(gs, mdl->M - k * gs); };
     cudaStream_t s0 = mdl->streams[0];
     const bool merged = phase == PH_FB;
     const bool do_fwd = phase == PH_FWD || merged, do_bwd = phase == PH_BWD || merged;
@@ -811,7 +812,7 @@ int enqueue_phase(hpf_model* mdl, int phase)
                 }
                 if (mdl->opt_cell_times) CU(stamp_time(mdl->cell_time_slot(PH_FWD, p, m), st, &mdl->launches));
                 for (int i = mdl->part_lo[p]; i < mdl->part_hi[p]; ++i) {
-                    int rc = forward_op(mdl, i, m, st, mdl->slot_of(p, m));
+                    int rc = forward_op(mdl, i, m * gs, group(m), st, mdl->slot_of(p, m));
                     if (rc) return rc;
                 }
                 if (mdl->opt_cell_times) CU(stamp_time(mdl->cell_time_slot(PH_FWD, p, m) + 1, st, &mdl->launches));
@@ -839,7 +840,7 @@ int enqueue_phase(hpf_model* mdl, int phase)
                 }
                 if (mdl->opt_cell_times) CU(stamp_time(mdl->cell_time_slot(PH_BWD, p, m), st, &mdl->launches));
                 for (int i = mdl->part_hi[p] - 1; i >= mdl->part_lo[p]; --i) {
-                    int rc = backward_op(mdl, i, m, st, mdl->slot_of(p, m));
+                    int rc = backward_op(mdl, i, m * gs, group(m), st, mdl->slot_of(p, m));
                     if (rc) return rc;
                 }
                 if (mdl->opt_cell_times) CU(stamp_time(mdl->cell_time_slot(PH_BWD, p, m) + 1, st, &mdl->launches));
@@ -866,9 +867,9 @@ int enqueue_phase(hpf_model* mdl, int phase)
             CU(cudaStreamWaitEvent(s0, mdl->ev_join[k], 0));
         }
     if (do_fwd)
-        CU(loss_average(reinterpret_cast<float*>(mdl->ws + mdl->loss_slots_off), reinterpret_cast<float*>(mdl->ws + mdl->loss_avg_off), M, s0, &mdl->launches));
+        CU(loss_average(reinterpret_cast<float*>(mdl->ws + mdl->loss_slots_off), reinterpret_cast<float*>(mdl->ws + mdl->loss_avg_off), mdl->M, s0, &mdl->launches));
     if (phase == PH_AVG)
-        CU(grad_average(mdl->gslots, mdl->gavg, M, mdl->G, s0, &mdl->launches));
+        CU(grad_average(mdl->gslots, mdl->gavg, mdl->M, mdl->G, s0, &mdl->launches));
     return HPF_OK;
 }
 
@@ -1230,139 +1231,73 @@ int hpf_bind(hpf_model* mdl, float* d_params, float* d_grad_slots, float* d_grad
             if (!mdl->prep_table[p].empty())
                 CU(cudaMemcpyAsync(mdl->ws + mdl->prep_table_off[p], mdl->prep_table[p].data(),
                                    sizeof(WeightPrepEntry) * mdl->prep_table[p].size(), cudaMemcpyHostToDevice, mdl->streams[0]));
-        for (int pass = 0; pass < 3; ++pass) mdl->tc_plan[pass].resize((size_t)n * M);
-        // the forward launch of convolution i on micro-batch m (prepared again when its cell's shared-memory budget changes)
-        auto prepare_fwd = [&](int i, int m) -> int {
+        CU(conv_pipe_init());
+        for (int pass = 0; pass < 2; ++pass) mdl->pipe_plan[pass].assign(n, ConvPipePlan());
+        mdl->wgrad_plan.resize(n);
+        std::vector<char> first_done(mdl->P, 0);
+        for (int i = 0; i < n; ++i) {
             const OpInfo& o = mdl->ops[i];
-            const int src = o.op.src0;
+            if (o.op.kind != HPF_OP_CONV) continue;
+            const int src = o.op.src0, p = o.part;
             const ConvShape s = conv_shape_of(mdl, i);
-            ConvTcPlan* pl = &mdl->tc_plan[PASS_FWD][(size_t)m * n + i];
-            const int sl = mdl->slot_of(o.part, m);
-            void* scratch = mdl->ws + mdl->conv_scratch_off[sl];
-            const int pass = PASS_FWD;
-            const float* residual = nullptr;
-                    if (mdl->fused_into[i] >= 0) {
-                        const hpf_op& a = mdl->ops[mdl->fused_into[i]].op;
-                        residual = mdl->act(a.src0 == i ? a.src1 : a.src0, m);
-                    }
-                    ConvBnFuse fuse;
-                    if (mdl->splitk_bytes[o.part]) { fuse.splitk = mdl->ws + mdl->splitk_off[sl]; fuse.splitk_bytes = mdl->splitk_bytes[o.part]; }
-                    fuse.pdl_late = cells_under_way(mdl->P, M, o.part, m, false) * mdl->lanes() >= mdl->opt_pdl_late_from;
-                    if (mdl->cell_of_op[i] >= 0) {
-                        fuse.cell_ctas = mdl->opt_cell;
-                        fuse.cell_smem = mdl->cell_runs[mdl->cell_of_op[i]].smem_budget;
-                    }
-                    if (mdl->conv_fwd_bn[i] >= 0) {
-                        const int jn = mdl->conv_fwd_bn[i];
-                        const OpInfo& bn = mdl->ops[jn];
-                        fuse.mode = mdl->bn_late[jn] ? 3 : 1;
-                        fuse.ticket = reinterpret_cast<unsigned int*>(mdl->ws + mdl->bn_scratch_off[sl]);
-                        fuse.partials = mdl->bn_partials(jn, m);
-                        fuse.stats_out = mdl->stats(jn, m);
-                        fuse.rows = (long long)mdl->b * bn.H * bn.W;
-                        fuse.eps = bn.op.eps;
-                    }
-                    const float* in = mdl->act(src, m);
-                    const int jb = mdl->conv_in_bn[i];
-                    if (jb >= 0) {
-                        const OpInfo& bn = mdl->ops[jb];
-                        in = mdl->act(bn.op.src0, m);          // the BN's input; its output is a by-product of this kernel
-                        fuse.in_mode = mdl->bn_late[jb] ? 2 : 1;
-                        fuse.in_partials = mdl->bn_partials(jb, m);
-                        fuse.in_tiles = conv_tc_tiles(conv_shape_of(mdl, mdl->bn_fwd_from[jb]), PASS_FWD);
-                        fuse.in_rows = (long long)mdl->b * bn.H * bn.W;
-                        fuse.in_eps = bn.op.eps;
-                        fuse.in_gamma = mdl->params + bn.w_off; fuse.in_beta = mdl->params + bn.b_off;
-                        fuse.in_stats = mdl->stats(jb, m); fuse.in_y = mdl->act(jb, m);
-                    }
-                    CU(conv_tc_prepare(pl, s, pass, passes, in, nullptr, wp + o.w_off, wp + G + o.w_off,
-                                       mdl->act(i, m), residual, false, scratch, &fuse));
-            return HPF_OK;
-        };
-        for (int pass = 0; pass < 3; ++pass) {
-            for (int m = 0; m < M; ++m)
-                for (int i = 0; i < n; ++i) {
-                    if (!mdl->use_tc[pass][i]) continue;
-                    const OpInfo& o = mdl->ops[i];
-                    const int src = o.op.src0;
-                    const ConvShape s = conv_shape_of(mdl, i);
-                    const GradEdge& ed = mdl->edge0[i];
-                    ConvTcPlan* pl = &mdl->tc_plan[pass][(size_t)m * n + i];
-                    const int sl = mdl->slot_of(o.part, m);
-                    void* scratch = mdl->ws + mdl->conv_scratch_off[sl];
-                    if (pass == PASS_FWD) {
-                        int rc = prepare_fwd(i, m);
-                        if (rc) return rc;
-                    }
-                    else if (pass == PASS_DGRAD) {
-                        ConvBnFuse dsplit;
-                        if (mdl->splitk_bytes[o.part]) { dsplit.splitk = mdl->ws + mdl->splitk_bwd_off[sl]; dsplit.splitk_bytes = mdl->splitk_bytes[o.part]; }
-                        CU(conv_tc_prepare(pl, s, pass, passes, mdl->grad(i, m), nullptr, wp + 2 * G + o.w_off, wp + 3 * G + o.w_off,
-                                           mdl->grad(src, m), ed.addend >= 0 ? mdl->grad(ed.addend, m) : nullptr, ed.accumulate != 0, scratch,
-                                           &dsplit));
-                    }
-                    else {
-                        // Weight gradients run on the side streams, beside the stages' chains of dependent kernels and feeding
-                        // nothing but the final average.  With many stages busy the SM time a launch takes counts, not its
-                        // duration: about 32 CTAs is the measured optimum for eight stages (fewer and the weight gradients
-                        // fall behind the chain; with four stages the uncapped launch measured faster).
-                        ConvBnFuse hint;
-                        hint.wgrad_max_ctas = (mdl->n_slots() >= 6 && !mdl->side.empty()) ? 32 : 0;
-                        hint.wgrad_transposing = mdl->opt_wgrad_direct ? 0 : 1;
-                        CU(conv_tc_prepare(pl, s, pass, mdl->opt_conv_path == 2 ? 1 : mdl->opt_wgrad_passes, mdl->grad(i, m), mdl->act(src, m), nullptr, nullptr,
-                                           mdl->gslots + (int64_t)m * mdl->G + o.w_off, nullptr, false, scratch, &hint));
-                    }
+            const GradEdge& ed = mdl->edge0[i];
+            if (mdl->use_tc[PASS_FWD][i]) {
+                const float* in = mdl->act(src, 0);
+                const float* residual = nullptr;
+                if (mdl->fused_into[i] >= 0) {
+                    const hpf_op& a = mdl->ops[mdl->fused_into[i]].op;
+                    residual = mdl->act(a.src0 == i ? a.src1 : a.src0, 0);
                 }
+                ConvPipeBn bn;
+                if (mdl->conv_fwd_bn[i] >= 0) bn.out_partials = mdl->moments(mdl->conv_fwd_bn[i]);
+                const int jb = mdl->conv_in_bn[i];
+                if (jb >= 0) {
+                    const OpInfo& b = mdl->ops[jb];
+                    in = mdl->act(b.op.src0, 0);              // the BN's input; its output is a by-product of this kernel
+                    bn.in_partials = mdl->moments(jb);
+                    bn.in_blocks = mdl->pipe_geom[PASS_FWD][mdl->bn_fwd_from[jb]].blocks_per_m;
+                    bn.in_gamma = mdl->params + b.w_off; bn.in_beta = mdl->params + b.b_off;
+                    bn.in_stats = mdl->stats(jb, 0); bn.in_y = mdl->act(jb, 0); bn.in_eps = b.op.eps;
+                }
+                // the weights are prepared just ahead of the partition's first convolution
+                CU(conv_pipe_prepare(&mdl->pipe_plan[PASS_FWD][i], s, PASS_FWD, passes, M, in, wp + o.w_off, wp + G + o.w_off, mdl->act(i, 0),
+                                     residual, false, &bn, mdl->ws + mdl->splitk_off[p], mdl->splitk_bytes[p], first_done[p] != 0));
+                first_done[p] = 1;
+            }
+            if (mdl->use_tc[PASS_DGRAD][i])
+                CU(conv_pipe_prepare(&mdl->pipe_plan[PASS_DGRAD][i], s, PASS_DGRAD, passes, M, mdl->grad(i, 0), wp + 2 * G + o.w_off,
+                                     wp + 3 * G + o.w_off, mdl->grad(src, 0), ed.addend >= 0 ? mdl->grad(ed.addend, 0) : nullptr,
+                                     ed.accumulate != 0, nullptr, mdl->ws + mdl->splitk_bwd_off[p], mdl->splitk_bytes[p], true));
+            if (mdl->use_tc[PASS_WGRAD][i]) {
+                ConvBnFuse hint;
+                hint.wgrad_transposing = mdl->opt_wgrad_direct ? 0 : 1;
+                hint.micro_batches = M; hint.slot_stride = mdl->G; hint.partial_stride = (long long)(mdl->conv_scratch_ms[p] / sizeof(float));
+                CU(conv_tc_prepare(&mdl->wgrad_plan[i], s, PASS_WGRAD, mdl->opt_conv_path == 2 ? 1 : mdl->opt_wgrad_passes, mdl->grad(i, 0), mdl->act(src, 0),
+                                   nullptr, nullptr, mdl->gslots + o.w_off, nullptr, false, mdl->ws + mdl->conv_scratch_off[p], &hint));
+            }
         }
-        // persistent forward cells: records of every run's launches, per micro-batch
+        // persistent forward cells: the records of every run's launches
+        std::vector<char> runs_in(mdl->P, 0);
         for (auto& run : mdl->cell_runs) {
-            // a launch whose operand pipeline came out shallower than it wants (wide channels: large stages) gets the
-            // shared memory of a whole SM; such a cell's CTAs then sit one per SM
-            bool shallow = false;
-            for (int i : run.convs) {
-                int stages = 0, iters = 0;
-                conv_tc_plan_pipeline(&mdl->tc_plan[PASS_FWD][i], &stages, &iters);
-                if (stages < (iters < 3 ? iters : 3)) shallow = true;
-            }
-            if (shallow) {
-                run.smem_budget = 200u * 1024u;
-                for (int m = 0; m < M; ++m)
-                    for (int i : run.convs) { int rc = prepare_fwd(i, m); if (rc) return rc; }
-            }
-            const size_t rec = conv_tc_cell_op_bytes();
+            const size_t rec = conv_pipe_cell_op_bytes();
             std::vector<unsigned char> host(rec * run.convs.size());
-            bool ok = true;
-            unsigned int most_ctas = 0;
-            for (int m = 0; m < M && ok; ++m) {
-                for (size_t k = 0; k < run.convs.size() && ok; ++k) {
-                    unsigned int smem = 0, tmem = 0, ctas = 0;
-                    cudaError_t e = conv_tc_cell_op(&mdl->tc_plan[PASS_FWD][(size_t)m * n + run.convs[k]], mdl->status(), host.data() + k * rec, &smem, &tmem, &ctas);
-                    if (e == cudaErrorNotSupported) { ok = false; break; }
-                    CU(e);
-                    if (smem > run.smem) run.smem = smem;
-                    if (tmem > run.tmem) run.tmem = tmem;
-                    if (ctas > most_ctas) most_ctas = ctas;
-                }
-                if (ok) CU(cudaMemcpyAsync(mdl->ws + run.ops_off[m], host.data(), host.size(), cudaMemcpyHostToDevice, mdl->streams[0]));
-                CU(cudaStreamSynchronize(mdl->streams[0]));          // `host` is reused for the next micro-batch
+            run.smem = run.tmem = 0;
+            for (size_t k = 0; k < run.convs.size(); ++k) {
+                unsigned int smem = 0, tmem = 0;
+                conv_pipe_cell_op(&mdl->pipe_plan[PASS_FWD][run.convs[k]], mdl->status(), host.data() + k * rec, &smem, &tmem);
+                run.smem = std::max(run.smem, smem); run.tmem = std::max(run.tmem, tmem);
             }
-            run.ctas = (int)most_ctas < mdl->opt_cell ? (int)most_ctas : mdl->opt_cell;
-            run.ready = ok && run.ctas >= 1;
+            CU(cudaMemcpyAsync(mdl->ws + run.ops_off, host.data(), host.size(), cudaMemcpyHostToDevice, mdl->streams[0]));
+            CU(cudaStreamSynchronize(mdl->streams[0]));          // `host` goes out of scope
+            run.ready = true;
+            runs_in[run.part] = 1;
         }
-        // All cells that can run at the same time (one per partition) must be resident together, or their grid barriers
-        // would wait for CTAs that cannot start: the grids have to fit the GPU side by side.
-        {
-            std::vector<double> share(mdl->P, 0.0);
-            for (const auto& run : mdl->cell_runs) {
-                if (!run.ready) continue;
-                const int cap = conv_tc_cell_max_ctas(run.smem);
-                if (cap < run.ctas) return fail(HPF_ERR_UNSUPPORTED, "a persistent cell kernel does not fit the GPU");
-                share[run.part] = std::max(share[run.part], (double)run.ctas / cap);
-            }
-            double total = 0.0;
-            for (double v : share) total += v;
-            if (total > 0.92) return fail(HPF_ERR_UNSUPPORTED, "the persistent cell kernels of all partitions do not fit the GPU together: lower HPF_OPT_CELL_CTAS");
-        }
+        // All cells that can run at the same time (one per partition and lane) must be resident together, or their grid
+        // barriers would wait for CTAs that cannot start: the grids have to fit the GPU side by side.
+        int grids = 0;
+        for (char r : runs_in) grids += r ? mdl->lanes() : 0;
+        if (grids * mdl->opt_cell > 0.92 * conv_pipe_cell_max_ctas())
+            return fail(HPF_ERR_UNSUPPORTED, "the persistent cell kernels of all partitions do not fit the GPU together: lower HPF_OPT_CELL_CTAS");
     }
     CU(cudaStreamSynchronize(mdl->streams[0]));
     mdl->state = ST_BOUND;
@@ -1424,7 +1359,7 @@ int hpf_forward_cell(hpf_model* mdl, int32_t p, int32_t m, const float* d_x, con
     const PdlScope pdl_scope(mdl->opt_pdl);
     const BnClusterScope bn_cluster_scope(mdl->opt_bn_cluster);
     for (int i = mdl->part_lo[p]; i < mdl->part_hi[p]; ++i) {
-        int rc = forward_op(mdl, i, m, mdl->stream_of(p, m), mdl->slot_of(p, m));
+        int rc = forward_op(mdl, i, m, 1, mdl->stream_of(p, m), mdl->slot_of(p, m));
         if (rc) return rc;
     }
     if (mdl->state < ST_FWD) mdl->state = ST_FWD;
@@ -1440,7 +1375,7 @@ int hpf_backward_cell(hpf_model* mdl, int32_t p, int32_t m)
     const PdlScope pdl_scope(mdl->opt_pdl);
     const BnClusterScope bn_cluster_scope(mdl->opt_bn_cluster);
     for (int i = mdl->part_hi[p] - 1; i >= mdl->part_lo[p]; --i) {
-        int rc = backward_op(mdl, i, m, mdl->stream_of(p, m), mdl->slot_of(p, m));
+        int rc = backward_op(mdl, i, m, 1, mdl->stream_of(p, m), mdl->slot_of(p, m));
         if (rc) return rc;
     }
     mdl->state = ST_BWD;
@@ -1704,6 +1639,14 @@ static int check_conv_args(int32_t N, int32_t H, int32_t W, int32_t C, int32_t K
     return HPF_OK;
 }
 
+static size_t single_splitk_bytes(const ConvShape& s)
+{
+    size_t need = 0;
+    for (int pass : {PASS_FWD, PASS_DGRAD})
+        for (int passes : {1, 3}) need = std::max(need, std::max(conv_tc_splitk_bytes(s, pass, passes), conv_pipe_splitk_bytes(s, pass, passes, 1)));
+    return need;
+}
+
 int hpf_conv_scratch_bytes(int32_t N, int32_t H, int32_t W, int32_t C, int32_t K, int32_t R, int32_t stride, int32_t pad, size_t* bytes)
 {
     if (!bytes) return fail(HPF_ERR_INVALID, "null");
@@ -1712,7 +1655,7 @@ int hpf_conv_scratch_bytes(int32_t N, int32_t H, int32_t W, int32_t C, int32_t K
     const ConvShape s = make_conv_shape(N, H, W, C, K, R, stride, pad);
     size_t a = conv_simt_scratch_bytes(s), b = conv_tc_scratch_bytes(s);
     // [weight-gradient partials | K-split tickets and partial tiles | device status (256 bytes)]
-    *bytes = align_up(a > b ? a : b, 256) + align_up(std::max(conv_tc_splitk_bytes(s, PASS_FWD, 3), conv_tc_splitk_bytes(s, PASS_DGRAD, 3)), 256) + 256;
+    *bytes = align_up(a > b ? a : b, 256) + align_up(single_splitk_bytes(s), 256) + 256;
     return HPF_OK;
 }
 
@@ -1750,6 +1693,15 @@ static int conv_single(int pass, const float* in, const float* in2, const float*
     split.wgrad_transposing = transposing ? 1 : 0;
     if (pass != PASS_WGRAD) {
         const size_t a = conv_simt_scratch_bytes(s), b = conv_tc_scratch_bytes(s);
+        ConvPipePlan pipe;
+        CU(conv_pipe_init());
+        const cudaError_t e = conv_pipe_prepare(&pipe, s, pass, path == 2 ? 1 : 3, 1, in, hi, hi + nw, out, nullptr, false, nullptr,
+                                                reinterpret_cast<char*>(d_scratch) + align_up(a > b ? a : b, 256), single_splitk_bytes(s), false);
+        if (e == cudaSuccess) {
+            CU(conv_pipe_launch(&pipe, 0, 1, false, status, st, nullptr));
+            return HPF_OK;
+        }
+        if (e != cudaErrorNotSupported) CU(e);
         split.splitk_bytes = conv_tc_splitk_bytes(s, pass, 3);
         if (split.splitk_bytes) split.splitk = reinterpret_cast<char*>(d_scratch) + align_up(a > b ? a : b, 256);
     }

@@ -85,8 +85,16 @@ bn_reduce_kernel(const float* __restrict__ x, const float* __restrict__ dy, cons
                  const float* __restrict__ beta, const float* __restrict__ stats, float eps, int64_t rows, int C,
                  int cgt, int rl, int passes, int64_t rows_per_blk, unsigned int* ticket,
                  float* __restrict__ partials, float* __restrict__ out_a, float* __restrict__ out_b,
-                 float* __restrict__ coef, float floor)
+                 float* __restrict__ coef, float floor, const BnGroup grp)
 {
+    {   // micro-batch of this block
+        const int64_t gm = blockIdx.y;
+        x += gm * grp.x; if (BWD) { dy += gm * grp.x; stats += gm * grp.stats; }
+        ticket = reinterpret_cast<unsigned int*>(reinterpret_cast<char*>(ticket) + gm * grp.scratch);
+        partials = reinterpret_cast<float*>(reinterpret_cast<char*>(partials) + gm * grp.scratch);
+        if (BWD) coef = reinterpret_cast<float*>(reinterpret_cast<char*>(coef) + gm * grp.scratch);
+        out_a += gm * (BWD ? grp.param : grp.stats); out_b += gm * (BWD ? grp.param : grp.stats);
+    }
     __shared__ double shd[kBnThreads][8];            // 32 KB; the float phase uses it as float[kBnThreads][8]
     float (*sh)[8] = reinterpret_cast<float (*)[8]>(&shd[0][0]);
     pdl_launch_dependents();
@@ -277,8 +285,9 @@ bn_reduce_kernel(const float* __restrict__ x, const float* __restrict__ dy, cons
 __global__ void __launch_bounds__(kBnThreads)
 bn_apply_fwd_kernel(const float4* __restrict__ x, const float* __restrict__ gamma, const float* __restrict__ beta,
                     const float* __restrict__ stats, float4* __restrict__ y, int64_t rows, int C, int cgt, int rl,
-                    int passes, int64_t rows_per_blk, float floor)
+                    int passes, int64_t rows_per_blk, float floor, const BnGroup grp)
 {
+    { const int64_t gm = blockIdx.y; x += gm * grp.x / 4; y += gm * grp.x / 4; stats += gm * grp.stats; }
     pdl_launch_dependents();
     pdl_wait();
     const int t = threadIdx.x, cg_total = C / 4;
@@ -290,8 +299,9 @@ bn_apply_fwd_kernel(const float4* __restrict__ x, const float* __restrict__ gamm
     for (int pass = 0; pass < passes; ++pass) {
         const int cg = pass * cgt + my_cg;
         if (cg >= cg_total) continue;
-        const float4 mu = __ldg(reinterpret_cast<const float4*>(stats) + cg);
-        const float4 rs = __ldg(reinterpret_cast<const float4*>(stats + C) + cg);
+        // (statistics the preceding kernel wrote: not the read-only path)
+        const float4 mu = __ldcg(reinterpret_cast<const float4*>(stats) + cg);
+        const float4 rs = __ldcg(reinterpret_cast<const float4*>(stats + C) + cg);
         const float4 g = __ldg(reinterpret_cast<const float4*>(gamma) + cg);
         const float4 b = __ldg(reinterpret_cast<const float4*>(beta) + cg);
         const int64_t base = (r0 + my_rl) * cg_total + cg, step = (int64_t)rl * cg_total;
@@ -321,8 +331,14 @@ __global__ void __launch_bounds__(kBnThreads)
 bn_apply_bwd_kernel(const float4* __restrict__ x, const float4* __restrict__ dy, const float* __restrict__ gamma,
                     const float* __restrict__ beta, const float* __restrict__ stats, const float* __restrict__ coef,
                     const float4* __restrict__ addend, float4* __restrict__ dx, int64_t rows, int C, int cgt, int rl,
-                    int passes, int64_t rows_per_blk, float floor)
+                    int passes, int64_t rows_per_blk, float floor, const BnGroup grp)
 {
+    {
+        const int64_t gm = blockIdx.y;
+        x += gm * grp.x / 4; dy += gm * grp.x / 4; dx += gm * grp.x / 4; stats += gm * grp.stats;
+        if (ADDEND) addend += gm * grp.x / 4;
+        coef = reinterpret_cast<const float*>(reinterpret_cast<const char*>(coef) + gm * grp.scratch);
+    }
     pdl_launch_dependents();
     pdl_wait();
     const int t = threadIdx.x, cg_total = C / 4;
@@ -376,8 +392,13 @@ __global__ void __launch_bounds__(kBnThreads)
 bn_bwd_cluster_kernel(const float4* __restrict__ x, const float4* __restrict__ dy, const float* __restrict__ gamma,
                       const float* __restrict__ beta, const float* __restrict__ stats, const float4* __restrict__ addend,
                       float4* __restrict__ dx, float* __restrict__ dgamma, float* __restrict__ dbeta, int64_t rows, int C,
-                      int cgc, int64_t rows_per_cta, float floor, int early_x)
+                      int cgc, int64_t rows_per_cta, float floor, int early_x, const BnGroup grp)
 {
+    {
+        const int64_t gm = blockIdx.y;
+        x += gm * grp.x / 4; dy += gm * grp.x / 4; dx += gm * grp.x / 4; stats += gm * grp.stats; dgamma += gm * grp.param; dbeta += gm * grp.param;
+        if (ADDEND) addend += gm * grp.x / 4;
+    }
     namespace cgr = cooperative_groups;
     cgr::cluster_group cluster = cgr::this_cluster();
     __shared__ float wpart[kBnThreads / 32][kBnClusterMaxCgc * 8];
@@ -483,8 +504,9 @@ template <int NV>
 __global__ void __launch_bounds__(kBnThreads)
 bn_fwd_cluster_kernel(const float4* __restrict__ x, const float* __restrict__ gamma, const float* __restrict__ beta, float eps,
                       float4* __restrict__ y, float* __restrict__ stats, int64_t rows, int C, int cgc, int64_t rows_per_cta,
-                      float floor)
+                      float floor, const BnGroup grp)
 {
+    { const int64_t gm = blockIdx.y; x += gm * grp.x / 4; y += gm * grp.x / 4; stats += gm * grp.stats; }
     namespace cgr = cooperative_groups;
     cgr::cluster_group cluster = cgr::this_cluster();
     __shared__ float wpart[kBnThreads / 32][kBnClusterMaxCgc * 8];
@@ -626,8 +648,13 @@ template <bool BWD>
 __global__ void __launch_bounds__(kBnThreads, 2)
 bn_reduce_big_kernel(const float4* __restrict__ x4, const float4* __restrict__ dy4, const float* __restrict__ gamma,
                      const float* __restrict__ beta, const float* __restrict__ stats, int64_t rows, int C, int cgt, int rl,
-                     int64_t rows_per_blk, float* __restrict__ partials, float floor)
+                     int64_t rows_per_blk, float* __restrict__ partials, float floor, const BnGroup grp)
 {
+    {
+        const int64_t gm = blockIdx.y;
+        x4 += gm * grp.x / 4; if (BWD) { dy4 += gm * grp.x / 4; stats += gm * grp.stats; }
+        partials = reinterpret_cast<float*>(reinterpret_cast<char*>(partials) + gm * grp.scratch);
+    }
     namespace cgr = cooperative_groups;
     cgr::cluster_group cluster = cgr::this_cluster();
     __shared__ float sh[kBnThreads][8];
@@ -824,8 +851,13 @@ inline size_t bn_big_apply_smem(int C) { return (size_t)kBnThreads * 8 * sizeof(
 __global__ void __launch_bounds__(kBnThreads, 2)
 bn_apply_big_fwd_kernel(const float4* __restrict__ x, const float* __restrict__ gamma, const float* __restrict__ beta,
                         const float* __restrict__ partials, int n_part, float eps, float* __restrict__ stats,
-                        float4* __restrict__ y, int64_t rows, int C, int cgt, int rl, int64_t rows_per_blk, float floor, int stream_out)
+                        float4* __restrict__ y, int64_t rows, int C, int cgt, int rl, int64_t rows_per_blk, float floor, int stream_out, const BnGroup grp)
 {
+    {
+        const int64_t gm = blockIdx.y;
+        x += gm * grp.x / 4; y += gm * grp.x / 4; stats += gm * grp.stats;
+        partials = reinterpret_cast<const float*>(reinterpret_cast<const char*>(partials) + gm * grp.scratch);
+    }
     extern __shared__ __align__(16) unsigned char bn_big_smem[];
     double (*shd)[8] = reinterpret_cast<double (*)[8]>(bn_big_smem);
     float* fin = reinterpret_cast<float*>(bn_big_smem + (size_t)kBnThreads * 8 * sizeof(double));
@@ -868,8 +900,14 @@ __global__ void __launch_bounds__(kBnThreads, 2)
 bn_apply_big_bwd_kernel(const float4* __restrict__ x, const float4* __restrict__ dy, const float* __restrict__ gamma,
                         const float* __restrict__ beta, const float* __restrict__ stats, const float* __restrict__ partials,
                         int n_part, float* __restrict__ dgamma, float* __restrict__ dbeta, const float4* __restrict__ addend,
-                        float4* __restrict__ dx, int64_t rows, int C, int cgt, int rl, int64_t rows_per_blk, float floor, int stream_out)
+                        float4* __restrict__ dx, int64_t rows, int C, int cgt, int rl, int64_t rows_per_blk, float floor, int stream_out, const BnGroup grp)
 {
+    {
+        const int64_t gm = blockIdx.y;
+        x += gm * grp.x / 4; dy += gm * grp.x / 4; dx += gm * grp.x / 4; stats += gm * grp.stats; dgamma += gm * grp.param; dbeta += gm * grp.param;
+        if (ADDEND) addend += gm * grp.x / 4;
+        partials = reinterpret_cast<const float*>(reinterpret_cast<const char*>(partials) + gm * grp.scratch);
+    }
     extern __shared__ __align__(16) unsigned char bn_big_smem[];
     double (*shd)[8] = reinterpret_cast<double (*)[8]>(bn_big_smem);
     float* fin = reinterpret_cast<float*>(bn_big_smem + (size_t)kBnThreads * 8 * sizeof(double));
@@ -960,10 +998,10 @@ BnBigPlan bn_big_plan(int64_t rows, int C, const BnPlan& p)
 }
 
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_cluster_pdl(void (*kernel)(KArgs...), int grid, int block, int cluster, cudaStream_t st, Args... args)
+inline cudaError_t launch_cluster_pdl(void (*kernel)(KArgs...), dim3 grid, int block, int cluster, cudaStream_t st, Args... args)
 {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid); cfg.blockDim = dim3(block); cfg.dynamicSmemBytes = 0; cfg.stream = st;
+    cfg.gridDim = grid; cfg.blockDim = dim3(block); cfg.dynamicSmemBytes = 0; cfg.stream = st;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = cluster; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
@@ -1572,7 +1610,7 @@ bool big_apply_attributes_set()
 }
 
 cudaError_t bnrelu_fwd(const float* x, const float* gamma, const float* beta, float eps, float* y, float* stats,
-                       int64_t rows, int C, void* scratch, cudaStream_t st, int64_t* n_launch, bool relu)
+                       int64_t rows, int C, void* scratch, cudaStream_t st, int64_t* n_launch, bool relu, const BnGroup& grp)
 {
     const BnPlan p = bn_plan(rows, C);
     const float floor = relu ? 0.f : -INFINITY;
@@ -1582,47 +1620,47 @@ cudaError_t bnrelu_fwd(const float* x, const float* gamma, const float* beta, fl
     if (cp.ok) {
         const float4* x4 = reinterpret_cast<const float4*>(x);
         float4* y4 = reinterpret_cast<float4*>(y);
-        const int grid = cp.n_clusters * kBnCluster;
+        const dim3 grid(cp.n_clusters * kBnCluster, grp.count);
         cudaError_t e;
-        if (cp.nv == 1) e = launch_cluster_pdl(bn_fwd_cluster_kernel<1>, grid, kBnThreads, kBnCluster, st, x4, gamma, beta, eps, y4, stats, rows, C, cp.cgc, cp.rows_per_cta, floor);
-        else if (cp.nv == 2) e = launch_cluster_pdl(bn_fwd_cluster_kernel<2>, grid, kBnThreads, kBnCluster, st, x4, gamma, beta, eps, y4, stats, rows, C, cp.cgc, cp.rows_per_cta, floor);
-        else if (cp.nv == 4) e = launch_cluster_pdl(bn_fwd_cluster_kernel<4>, grid, kBnThreads, kBnCluster, st, x4, gamma, beta, eps, y4, stats, rows, C, cp.cgc, cp.rows_per_cta, floor);
-        else e = launch_cluster_pdl(bn_fwd_cluster_kernel<8>, grid, kBnThreads, kBnCluster, st, x4, gamma, beta, eps, y4, stats, rows, C, cp.cgc, cp.rows_per_cta, floor);
+        if (cp.nv == 1) e = launch_cluster_pdl(bn_fwd_cluster_kernel<1>, grid, kBnThreads, kBnCluster, st, x4, gamma, beta, eps, y4, stats, rows, C, cp.cgc, cp.rows_per_cta, floor, grp);
+        else if (cp.nv == 2) e = launch_cluster_pdl(bn_fwd_cluster_kernel<2>, grid, kBnThreads, kBnCluster, st, x4, gamma, beta, eps, y4, stats, rows, C, cp.cgc, cp.rows_per_cta, floor, grp);
+        else if (cp.nv == 4) e = launch_cluster_pdl(bn_fwd_cluster_kernel<4>, grid, kBnThreads, kBnCluster, st, x4, gamma, beta, eps, y4, stats, rows, C, cp.cgc, cp.rows_per_cta, floor, grp);
+        else e = launch_cluster_pdl(bn_fwd_cluster_kernel<8>, grid, kBnThreads, kBnCluster, st, x4, gamma, beta, eps, y4, stats, rows, C, cp.cgc, cp.rows_per_cta, floor, grp);
         count(n_launch, 1);
         return e;
     }
     const BnBigPlan bp = bn_big_plan<false>(rows, C, p);
     if (bp.ok && big_apply_attributes_set()) {
         const size_t smem = bn_big_apply_smem(C);
-        launch_cluster_pdl(bn_reduce_big_kernel<false>, bp.n_clusters * kBnBigCluster, kBnThreads, kBnBigCluster, st,
+        launch_cluster_pdl(bn_reduce_big_kernel<false>, dim3(bp.n_clusters * kBnBigCluster, grp.count), kBnThreads, kBnBigCluster, st,
                            reinterpret_cast<const float4*>(x), (const float4*)nullptr, gamma, beta, (const float*)nullptr, rows, C,
-                           p.cgt, p.rl, bp.rows_per_blk, partials, floor);
-        launch_pdl(bn_apply_big_fwd_kernel, bp.nblk_apply, kBnThreads, smem, st, reinterpret_cast<const float4*>(x), gamma, beta,
+                           p.cgt, p.rl, bp.rows_per_blk, partials, floor, grp);
+        launch_pdl(bn_apply_big_fwd_kernel, dim3(bp.nblk_apply, grp.count), kBnThreads, smem, st, reinterpret_cast<const float4*>(x), gamma, beta,
                    (const float*)partials, bp.n_clusters, eps, stats, reinterpret_cast<float4*>(y), rows, C, p.cgt, p.rl,
-                   bp.rows_per_blk_apply, floor, bp.stream_out);
+                   bp.rows_per_blk_apply, floor, bp.stream_out, grp);
         count(n_launch, 2);
         return cudaGetLastError();
     }
-    launch_pdl(bn_reduce_kernel<false>, p.nblk, kBnThreads, 0, st, x, (const float*)nullptr, gamma, beta, (const float*)nullptr, eps, rows, C, p.cgt, p.rl,
+    launch_pdl(bn_reduce_kernel<false>, dim3(p.nblk, grp.count), kBnThreads, 0, st, x, (const float*)nullptr, gamma, beta, (const float*)nullptr, eps, rows, C, p.cgt, p.rl,
                                                            p.passes, p.rows_per_blk, ticket, partials, stats, stats + C,
-                                                           (float*)nullptr, floor);
-    launch_pdl(bn_apply_fwd_kernel, p.nblk_apply, kBnThreads, 0, st, reinterpret_cast<const float4*>(x), gamma, beta, stats,
+                                                           (float*)nullptr, floor, grp);
+    launch_pdl(bn_apply_fwd_kernel, dim3(p.nblk_apply, grp.count), kBnThreads, 0, st, reinterpret_cast<const float4*>(x), gamma, beta, stats,
                                                              reinterpret_cast<float4*>(y), rows, C, p.cgt, p.rl, p.passes,
-                                                             p.rows_per_blk_apply, floor);
+                                                             p.rows_per_blk_apply, floor, grp);
     count(n_launch, 2);
     return cudaGetLastError();
 }
 
 cudaError_t bnrelu_bwd(const float* x, const float* dy, const float* gamma, const float* beta, const float* stats,
                        float* dx, const float* addend, bool accumulate, float* dgamma, float* dbeta, int64_t rows,
-                       int C, void* scratch, cudaStream_t st, int64_t* n_launch, bool relu, bool x_is_old)
+                       int C, void* scratch, cudaStream_t st, int64_t* n_launch, bool relu, bool x_is_old, const BnGroup& grp)
 {
     const BnPlan p = bn_plan(rows, C);
     const float floor = relu ? 0.f : -INFINITY;
     const BnClusterPlan cp = g_bn_cluster ? bn_cluster_plan(rows, C) : BnClusterPlan{false, 0, 0, 0, 0};
     if (cp.ok) {
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(cp.n_clusters * kBnCluster); cfg.blockDim = dim3(kBnThreads); cfg.dynamicSmemBytes = 0; cfg.stream = st;
+        cfg.gridDim = dim3(cp.n_clusters * kBnCluster, grp.count); cfg.blockDim = dim3(kBnThreads); cfg.dynamicSmemBytes = 0; cfg.stream = st;
         cudaLaunchAttribute attr[2];
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = kBnCluster; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
@@ -1635,7 +1673,7 @@ cudaError_t bnrelu_bwd(const float* x, const float* dy, const float* gamma, cons
         float4* dx4 = reinterpret_cast<float4*>(dx);
         const int early = x_is_old ? 1 : 0;
         cudaError_t e;
-#define HPF_BN_CL(NV, A, B) e = cudaLaunchKernelEx(&cfg, bn_bwd_cluster_kernel<NV, A, B>, x4, dy4, gamma, beta, stats, ad4, dx4, dgamma, dbeta, rows, C, cp.cgc, cp.rows_per_cta, floor, early)
+#define HPF_BN_CL(NV, A, B) e = cudaLaunchKernelEx(&cfg, bn_bwd_cluster_kernel<NV, A, B>, x4, dy4, gamma, beta, stats, ad4, dx4, dgamma, dbeta, rows, C, cp.cgc, cp.rows_per_cta, floor, early, grp)
 #define HPF_BN_CL_NV(NV) do { if (addend && accumulate) HPF_BN_CL(NV, true, true); else if (addend) HPF_BN_CL(NV, true, false); \
                               else if (accumulate) HPF_BN_CL(NV, false, true); else HPF_BN_CL(NV, false, false); } while (0)
         if (cp.nv == 1) HPF_BN_CL_NV(1); else if (cp.nv == 2) HPF_BN_CL_NV(2); else if (cp.nv == 4) HPF_BN_CL_NV(4); else HPF_BN_CL_NV(8);
@@ -1654,9 +1692,9 @@ cudaError_t bnrelu_bwd(const float* x, const float* dy, const float* gamma, cons
         const float4* dy4 = reinterpret_cast<const float4*>(dy);
         const float4* ad4 = reinterpret_cast<const float4*>(addend);
         float4* dx4 = reinterpret_cast<float4*>(dx);
-        launch_cluster_pdl(bn_reduce_big_kernel<true>, bp.n_clusters * kBnBigCluster, kBnThreads, kBnBigCluster, st, x4, dy4, gamma, beta,
-                           stats, rows, C, p.cgt, p.rl, bp.rows_per_blk, partials, floor);
-#define HPF_BN_BIG(A, B) launch_pdl(bn_apply_big_bwd_kernel<A, B>, bp.nblk_apply, kBnThreads, smem, st, x4, dy4, gamma, beta, stats, (const float*)partials, bp.n_clusters, dgamma, dbeta, ad4, dx4, rows, C, p.cgt, p.rl, bp.rows_per_blk_apply, floor, bp.stream_out)
+        launch_cluster_pdl(bn_reduce_big_kernel<true>, dim3(bp.n_clusters * kBnBigCluster, grp.count), kBnThreads, kBnBigCluster, st, x4, dy4, gamma, beta,
+                           stats, rows, C, p.cgt, p.rl, bp.rows_per_blk, partials, floor, grp);
+#define HPF_BN_BIG(A, B) launch_pdl(bn_apply_big_bwd_kernel<A, B>, dim3(bp.nblk_apply, grp.count), kBnThreads, smem, st, x4, dy4, gamma, beta, stats, (const float*)partials, bp.n_clusters, dgamma, dbeta, ad4, dx4, rows, C, p.cgt, p.rl, bp.rows_per_blk_apply, floor, bp.stream_out, grp)
         if (addend && accumulate) HPF_BN_BIG(true, true);
         else if (addend) HPF_BN_BIG(true, false);
         else if (accumulate) HPF_BN_BIG(false, true);
@@ -1665,14 +1703,14 @@ cudaError_t bnrelu_bwd(const float* x, const float* dy, const float* gamma, cons
         count(n_launch, 2);
         return cudaGetLastError();
     }
-    launch_pdl(bn_reduce_kernel<true>, p.nblk, kBnThreads, 0, st, x, dy, gamma, beta, stats, 0.f, rows, C, p.cgt, p.rl, p.passes,
-                                                          p.rows_per_blk, ticket, partials, dbeta, dgamma, coef, floor);
+    launch_pdl(bn_reduce_kernel<true>, dim3(p.nblk, grp.count), kBnThreads, 0, st, x, dy, gamma, beta, stats, 0.f, rows, C, p.cgt, p.rl, p.passes,
+                                                          p.rows_per_blk, ticket, partials, dbeta, dgamma, coef, floor, grp);
     const float4* x4 = reinterpret_cast<const float4*>(x);
     const float4* dy4 = reinterpret_cast<const float4*>(dy);
     const float4* ad4 = reinterpret_cast<const float4*>(addend);
     float4* dx4 = reinterpret_cast<float4*>(dx);
     const int nb = p.nblk_apply;
-#define HPF_BN_APPLY(A, B) launch_pdl(bn_apply_bwd_kernel<A, B>, nb, kBnThreads, 0, st, x4, dy4, gamma, beta, stats, coef, ad4, dx4, rows, C, p.cgt, p.rl, p.passes, p.rows_per_blk_apply, floor)
+#define HPF_BN_APPLY(A, B) launch_pdl(bn_apply_bwd_kernel<A, B>, dim3(nb, grp.count), kBnThreads, 0, st, x4, dy4, gamma, beta, stats, coef, ad4, dx4, rows, C, p.cgt, p.rl, p.passes, p.rows_per_blk_apply, floor, grp)
     if (addend && accumulate) HPF_BN_APPLY(true, true);
     else if (addend) HPF_BN_APPLY(true, false);
     else if (accumulate) HPF_BN_APPLY(false, true);
@@ -1683,11 +1721,11 @@ cudaError_t bnrelu_bwd(const float* x, const float* dy, const float* gamma, cons
 }
 
 cudaError_t bnrelu_fwd_apply(const float* x, const float* gamma, const float* beta, const float* stats, float* y,
-                             int64_t rows, int C, cudaStream_t st, int64_t* n_launch)
+                             int64_t rows, int C, cudaStream_t st, int64_t* n_launch, const BnGroup& grp)
 {
     const BnPlan p = bn_plan(rows, C);
-    launch_pdl(bn_apply_fwd_kernel, p.nblk_apply, kBnThreads, 0, st, reinterpret_cast<const float4*>(x), gamma, beta, stats,
-               reinterpret_cast<float4*>(y), rows, C, p.cgt, p.rl, p.passes, p.rows_per_blk_apply, 0.f);
+    launch_pdl(bn_apply_fwd_kernel, dim3(p.nblk_apply, grp.count), kBnThreads, 0, st, reinterpret_cast<const float4*>(x), gamma, beta, stats,
+               reinterpret_cast<float4*>(y), rows, C, p.cgt, p.rl, p.passes, p.rows_per_blk_apply, 0.f, grp);
     count(n_launch, 1);
     return cudaGetLastError();
 }
