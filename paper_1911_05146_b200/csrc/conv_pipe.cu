@@ -134,31 +134,42 @@ __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 2, 256;" :::
 
 __host__ __device__ inline size_t partial_floats(int units, int C) { return (size_t)units * 2 * C + (size_t)((units + 3) & ~3); }
 
+__device__ __forceinline__ float4 lane_sum(float4 v, int o)
+{
+    v.x += __shfl_xor_sync(0xffffffffu, v.x, o); v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
+    v.z += __shfl_xor_sync(0xffffffffu, v.z, o); v.w += __shfl_xor_sync(0xffffffffu, v.w, o);
+    return v;
+}
+__device__ __forceinline__ float4 add4(float4 a, float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
+
 // Statistics of a BN's input from the partial moments of one micro-batch: rows of (mean[C], M2[C]) with n values each.
 //   mean = ref + sum n (mean_u - ref) / N,   M2 = sum M2_u + sum n (mean_u - ref)^2 - N (mean - ref)^2,   ref = row 0's mean:
 // no difference of large numbers appears however far a channel's mean is from zero compared with its spread.  Fixed order
-// (every CTA of a launch gets the same bits), fp32 terms, the last combination in fp64.  THREADS threads, which share named barrier 1;
-// tab: mean[C], rstd[C]; red: 3 x THREADS float4.
+// (every CTA of a launch gets the same bits), fp32 terms, the last combination in fp64.  THREADS threads, which share named
+// barrier 1; tab: mean[C], rstd[C]; red: 4 x THREADS float4.  First every thread adds its rows of four channels, then one
+// thread per channel combines: what this costs is latency and instruction fetches, so nothing is unrolled that need not be.
 template <int THREADS>
-__device__ __forceinline__ void merge_moments(const float* partials, int units, int C, double inv_rows, float eps, float* tab, float4* red,
-                                              int tid)
+__device__ __forceinline__ void merge_moments(const float* partials, int rows, int C, double inv_rows, float eps, float* tab, float4* red, int tid)
 {
-    const float* counts = partials + (size_t)units * 2 * C;
+    const float* counts = partials + (size_t)rows * 2 * C;
     const int c4n = C >> 2;
     const int L = c4n <= THREADS ? THREADS / c4n : 1;
+#pragma unroll 1
     for (int c0 = 0; c0 < c4n; c0 += THREADS) {
-        const int col = c0 + (L > 1 ? tid % c4n : tid), ln = L > 1 ? tid / c4n : 0;
-        const bool mine = col < c4n && ln < L;
+        const int width = c4n - c0 < THREADS ? c4n - c0 : THREADS;       // float4 columns of this pass
+        const int ln = L > 1 ? tid / c4n : 0, local = L > 1 ? tid - ln * c4n : tid, col = c0 + local;
+        const bool mine = local < width && ln < L;
         float4 sd = make_float4(0.f, 0.f, 0.f, 0.f), sq = sd, m2 = sd, ref = sd;
         if (mine) {
             ref = __ldcg(reinterpret_cast<const float4*>(partials) + col);
-            for (int k0 = ln; k0 < units; k0 += 4 * L) {
+#pragma unroll 1
+            for (int k0 = ln; k0 < rows; k0 += 4 * L) {
                 float4 a[4], b[4];
                 float n[4];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const int k = k0 + j * L;
-                    const bool have = k < units;
+                    const bool have = k < rows;
                     const float4* row = reinterpret_cast<const float4*>(partials + (size_t)(have ? k : 0) * 2 * C);
                     n[j] = have ? __ldcg(counts + k) : 0.f;
                     a[j] = __ldcg(row + col);
@@ -167,51 +178,39 @@ __device__ __forceinline__ void merge_moments(const float* partials, int units, 
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const float dx = a[j].x - ref.x, dy = a[j].y - ref.y, dz = a[j].z - ref.z, dw = a[j].w - ref.w;
-                    sd.x = fmaf(n[j], dx, sd.x); sd.y = fmaf(n[j], dy, sd.y); sd.z = fmaf(n[j], dz, sd.z); sd.w = fmaf(n[j], dw, sd.w);
-                    sq.x = fmaf(n[j] * dx, dx, sq.x); sq.y = fmaf(n[j] * dy, dy, sq.y); sq.z = fmaf(n[j] * dz, dz, sq.z); sq.w = fmaf(n[j] * dw, dw, sq.w);
-                    m2.x += b[j].x; m2.y += b[j].y; m2.z += b[j].z; m2.w += b[j].w;
+                    const float nx = n[j] * dx, ny = n[j] * dy, nz = n[j] * dz, nw = n[j] * dw;
+                    sd.x += nx; sd.y += ny; sd.z += nz; sd.w += nw;
+                    sq.x = fmaf(nx, dx, sq.x); sq.y = fmaf(ny, dy, sq.y); sq.z = fmaf(nz, dz, sq.z); sq.w = fmaf(nw, dw, sq.w);
+                    m2 = add4(m2, b[j]);
                 }
             }
         }
-        int lanes = L;                               // row lanes left to add, red[l * c4n + col]
+        int lanes = L, at = tid;                      // row lanes left to add: red[lane * width + local]
+        bool put = mine;
         if (c4n <= 16 && (c4n & (c4n - 1)) == 0) {
             // the row lanes of a column inside a warp first: a fixed butterfly
-            for (int o = 16; o >= c4n; o >>= 1) {
-                sd.x += __shfl_xor_sync(0xffffffffu, sd.x, o); sd.y += __shfl_xor_sync(0xffffffffu, sd.y, o);
-                sd.z += __shfl_xor_sync(0xffffffffu, sd.z, o); sd.w += __shfl_xor_sync(0xffffffffu, sd.w, o);
-                sq.x += __shfl_xor_sync(0xffffffffu, sq.x, o); sq.y += __shfl_xor_sync(0xffffffffu, sq.y, o);
-                sq.z += __shfl_xor_sync(0xffffffffu, sq.z, o); sq.w += __shfl_xor_sync(0xffffffffu, sq.w, o);
-                m2.x += __shfl_xor_sync(0xffffffffu, m2.x, o); m2.y += __shfl_xor_sync(0xffffffffu, m2.y, o);
-                m2.z += __shfl_xor_sync(0xffffffffu, m2.z, o); m2.w += __shfl_xor_sync(0xffffffffu, m2.w, o);
-            }
+#pragma unroll 1
+            for (int o = 16; o >= c4n; o >>= 1) { sd = lane_sum(sd, o); sq = lane_sum(sq, o); m2 = lane_sum(m2, o); }
             lanes = THREADS / 32;
-            const int at = (tid >> 5) * c4n + (tid & 31);
-            if ((tid & 31) < c4n) { red[at] = sd; red[THREADS + at] = sq; red[2 * THREADS + at] = m2; }
-        } else if (L > 1) {
-            red[tid] = sd; red[THREADS + tid] = sq; red[2 * THREADS + tid] = m2;
+            at = (tid >> 5) * c4n + (tid & 31);
+            put = (tid & 31) < c4n;
         }
-        if (lanes > 1) {
-            asm volatile("bar.sync 1, %0;" ::"n"(THREADS) : "memory");
-            if (mine && ln == 0)
-                for (int l = 1; l < lanes; ++l) {
-                    const float4 x = red[l * c4n + col], y = red[THREADS + l * c4n + col], z = red[2 * THREADS + l * c4n + col];
-                    sd.x += x.x; sd.y += x.y; sd.z += x.z; sd.w += x.w;
-                    sq.x += y.x; sq.y += y.y; sq.z += y.z; sq.w += y.w;
-                    m2.x += z.x; m2.y += z.y; m2.z += z.z; m2.w += z.w;
-                }
+        if (put) { red[at] = sd; red[THREADS + at] = sq; red[2 * THREADS + at] = m2; }
+        if (mine && ln == 0) red[3 * THREADS + local] = ref;
+        asm volatile("bar.sync 1, %0;" ::"n"(THREADS) : "memory");
+        const float* r = reinterpret_cast<const float*>(red);
+#pragma unroll 1
+        for (int c = tid; c < 4 * width; c += THREADS) {
+            float d = 0.f, q = 0.f, v = 0.f;
+#pragma unroll 2
+            for (int l = 0; l < lanes; ++l) { const int i = 4 * l * width + c; d += r[i]; q += r[4 * THREADS + i]; v += r[8 * THREADS + i]; }
+            const double dm = (double)d * inv_rows;
+            double var = ((double)v + (double)q) * inv_rows - dm * dm;
+            if (var < 0.0) var = 0.0;
+            tab[4 * c0 + c] = (float)((double)r[12 * THREADS + c] + dm);
+            tab[C + 4 * c0 + c] = 1.0f / sqrtf((float)(var + (double)eps));
         }
-        if (mine && ln == 0) {
-            const float d[4] = {sd.x, sd.y, sd.z, sd.w}, q[4] = {sq.x, sq.y, sq.z, sq.w}, v[4] = {m2.x, m2.y, m2.z, m2.w},
-                        r[4] = {ref.x, ref.y, ref.z, ref.w};
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const double dm = (double)d[j] * inv_rows;
-                double var = ((double)v[j] + (double)q[j]) * inv_rows - dm * dm;
-                if (var < 0.0) var = 0.0;
-                tab[4 * col + j] = (float)((double)r[j] + dm);
-                tab[C + 4 * col + j] = 1.0f / sqrtf((float)(var + (double)eps));
-            }
-        }
+        if (c0 + THREADS < c4n) asm volatile("bar.sync 1, %0;" ::"n"(THREADS) : "memory");
     }
 }
 
@@ -270,113 +269,102 @@ __device__ __forceinline__ Span span_of(const PipeScalars& p, const UnitWalk& u)
     return r;
 }
 
+constexpr int kMomentPlane = kEpiWarps * 32 * 2;      // float4: one per thread and column group (two per warp)
+
+// What one warp does with 32 rows x 32 (or 16) columns of a finished tile, which stand in its patch of shared memory.
 struct EmitArgs {
     float* out;                  // this warp's column group
     const float* extra;
-    float4* patch;
+    const float4* patch;
     float4* moments;             // this lane's k, sum (x - k), sum (x - k)^2 of its four columns: three planes of kMomentPlane, or null
     bool accumulate, ok;
-    int fill;
-    bool zero_fill;
-    int dense_h, dense_w;
-    int step;                    // dense rows: floats between rows
+    int zero_fill, dense_h, dense_w;
 };
-constexpr int kMomentPlane = kEpiWarps * 32 * 2;      // two column groups per warp
 
-// One warp's 32 rows x (4 * LPR) columns of a tile: LPR lanes hold a row's 16-byte pieces.  Loads, shared-memory reads and
-// stores are batched by kind, so that a batch's latencies overlap.  DENSE: all 32 rows are stored, one after the other in
-// memory (row 0 at ro of lane 0); otherwise ro is this lane's row offset or -1.
-// Moments are taken about the first value the warp stored for a column: sums of x and x*x themselves would cancel for a
-// channel whose mean is large against its spread.
-template <int LPR, bool DENSE, class Stage>
-__device__ __forceinline__ void emit_rows(const EmitArgs& a, int ro, int lane, bool have_shift, Stage stage)
+// The residuals of four row steps, beginning with step b.
+__device__ __forceinline__ void emit_residuals(const EmitArgs& a, int ro, int lane, int lsh, int b, float4* e)
 {
-    constexpr int RSTEP = 32 / LPR;
-    const int cq = lane & (LPR - 1), rq = lane / LPR;
-    float4 e[4];
-    int so[4];
-    const int base = DENSE ? __shfl_sync(0xffffffffu, ro, 0) + rq * a.step + 4 * cq : 0;
-    auto offsets = [&](int b) {
+    const int cq = lane & ((1 << lsh) - 1), r = (lane >> lsh) + ((32 >> lsh) * b);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            if (DENSE) so[i] = base + (b + i) * RSTEP * a.step;
-            else {
-                const int r = __shfl_sync(0xffffffffu, ro, rq + RSTEP * (b + i));
-                so[i] = r >= 0 ? r + 4 * cq : -1;
-            }
-        }
-        if (a.extra) {
-            // (not the read-only path: the preceding kernel may have written it)
-#pragma unroll
-            for (int i = 0; i < 4; ++i) e[i] = __ldcg(reinterpret_cast<const float4*>(a.extra + (DENSE || so[i] >= 0 ? so[i] : 0)));
-        }
-    };
-    offsets(0);                                       // the first residuals travel while the accumulator is read
-    stage();
-    __syncwarp();
-    const unsigned int who = DENSE ? 0xffffffffu : __ballot_sync(0xffffffffu, ro >= 0);      // lane = row here
+    for (int i = 0; i < 4; ++i) {
+        const int so = __shfl_sync(0xffffffffu, ro, r + (32 >> lsh) * i);
+        // (not the read-only path: the preceding kernel may have written it)
+        e[i] = __ldcg(reinterpret_cast<const float4*>(a.extra + (so >= 0 ? so + 4 * cq : 0)));
+    }
+}
+
+// 1 << lsh lanes hold a row's 16-byte pieces; ro is this lane's row offset or -1.  Loads, shared-memory reads and stores are
+// batched by kind, so that a batch's latencies overlap; there is ONE copy of this code for all widths and forms, since a
+// launch of a few microseconds runs it once or twice and would wait for its instructions otherwise (the kernel had grown to
+// 200 KB with specialised copies: 4000-8000 clocks for the first tile of a launch).
+// Moments are taken about a value of the column: sums of x and x*x themselves would cancel for a channel whose mean is large
+// against its spread.
+__device__ __forceinline__ void emit_rows(const EmitArgs& a, int ro, int fill, int lane, int lsh, bool have_shift, float4* e)
+{
+    const int cq = lane & ((1 << lsh) - 1), rq = lane >> lsh, rstep = 32 >> lsh, steps = 1 << lsh;
+    const unsigned int who = __ballot_sync(0xffffffffu, ro >= 0);        // lane = row here
     float4 k = make_float4(0.f, 0.f, 0.f, 0.f), sd = k, sq = k;
-    if (a.moments && have_shift) k = a.moments[0];
-#pragma unroll
-    for (int b = 0; b < LPR; b += 4) {
-        if (b > 0) offsets(b);
+    const bool moments = a.moments != nullptr && who != 0u;
+    if (moments) {
+        if (have_shift) k = a.moments[0];
+        else {
+            const int r0 = __ffs(who) - 1, so = __shfl_sync(0xffffffffu, ro, r0);
+            k = a.patch[r0 * 8 + (cq ^ (r0 & 7))];
+            if (a.extra) k = add4(k, __ldcg(reinterpret_cast<const float4*>(a.extra + so + 4 * cq)));
+            a.moments[0] = k;
+        }
+    }
+#pragma unroll 1
+    for (int b = 0; b < steps; b += 4) {
+        int so[4];
         float4 v[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) { const int r = rq + RSTEP * (b + i); v[i] = a.patch[r * 8 + (cq ^ (r & 7))]; }
+        for (int i = 0; i < 4; ++i) {
+            const int r = rq + rstep * (b + i);
+            so[i] = __shfl_sync(0xffffffffu, ro, r);
+            v[i] = a.patch[r * 8 + (cq ^ (r & 7))];
+        }
         if (a.extra) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) { v[i].x += e[i].x; v[i].y += e[i].y; v[i].z += e[i].z; v[i].w += e[i].w; }
+            for (int i = 0; i < 4; ++i) v[i] = add4(v[i], e[i]);
+            if (b + 4 < steps) emit_residuals(a, ro, lane, lsh, b + 4, e);
         }
+        float* out = a.out + 4 * cq;
         if (a.accumulate) {
 #pragma unroll
             for (int i = 0; i < 4; ++i)
-                if (DENSE || so[i] >= 0) { const float4 o = __ldcg(reinterpret_cast<const float4*>(a.out + so[i])); v[i].x += o.x; v[i].y += o.y; v[i].z += o.z; v[i].w += o.w; }
+                if (so[i] >= 0) v[i] = add4(v[i], __ldcg(reinterpret_cast<const float4*>(out + so[i])));
         }
         if (a.ok) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) if (DENSE || so[i] >= 0) *reinterpret_cast<float4*>(a.out + so[i]) = v[i];
+            for (int i = 0; i < 4; ++i) if (so[i] >= 0) *reinterpret_cast<float4*>(out + so[i]) = v[i];
         }
-        if (!DENSE && a.zero_fill) {
-            // strided data gradient: the positions between the samples receive no contribution
-            const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (moments) {
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                const int f = __shfl_sync(0xffffffffu, a.fill, rq + RSTEP * (b + i));
-                if (so[i] >= 0 && a.ok) {
-                    if (f & 1) *reinterpret_cast<float4*>(a.out + so[i] + a.dense_w) = zero;
-                    if (f & 2) *reinterpret_cast<float4*>(a.out + so[i] + a.dense_h) = zero;
-                    if (f & 4) *reinterpret_cast<float4*>(a.out + so[i] + a.dense_h + a.dense_w) = zero;
-                }
-            }
-        }
-        if (a.moments && who) {
-            if (!have_shift) {
-                const int r0 = DENSE ? 0 : __ffs(who) - 1, src = (r0 % RSTEP) * LPR + cq, step = r0 / RSTEP - b;
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    if (step == i) {
-                        k.x = __shfl_sync(0xffffffffu, v[i].x, src); k.y = __shfl_sync(0xffffffffu, v[i].y, src);
-                        k.z = __shfl_sync(0xffffffffu, v[i].z, src); k.w = __shfl_sync(0xffffffffu, v[i].w, src);
-                        have_shift = true;
-                        a.moments[0] = k;
-                    }
-            }
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const bool real = DENSE || so[i] >= 0;
+                const bool real = so[i] >= 0;
                 const float d0 = real ? v[i].x - k.x : 0.f, d1 = real ? v[i].y - k.y : 0.f, d2 = real ? v[i].z - k.z : 0.f, d3 = real ? v[i].w - k.w : 0.f;
                 sd.x += d0; sd.y += d1; sd.z += d2; sd.w += d3;
                 sq.x = fmaf(d0, d0, sq.x); sq.y = fmaf(d1, d1, sq.y); sq.z = fmaf(d2, d2, sq.z); sq.w = fmaf(d3, d3, sq.w);
             }
         }
     }
-    if (a.moments && who) {
-        float4 t = a.moments[kMomentPlane];
-        t.x += sd.x; t.y += sd.y; t.z += sd.z; t.w += sd.w;
-        a.moments[kMomentPlane] = t;
-        t = a.moments[2 * kMomentPlane];
-        t.x += sq.x; t.y += sq.y; t.z += sq.z; t.w += sq.w;
-        a.moments[2 * kMomentPlane] = t;
+    if (moments) {
+        a.moments[kMomentPlane] = add4(a.moments[kMomentPlane], sd);
+        a.moments[2 * kMomentPlane] = add4(a.moments[2 * kMomentPlane], sq);
+    }
+    if (a.zero_fill == 2) {
+        // strided data gradient: the positions between the samples receive no contribution
+        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+        for (int i = 0; i < steps; ++i) {
+            const int so = __shfl_sync(0xffffffffu, ro, rq + rstep * i), f = __shfl_sync(0xffffffffu, fill, rq + rstep * i);
+            if (so < 0 || !a.ok) continue;
+            float* out = a.out + so + 4 * cq;
+            if (f & 1) *reinterpret_cast<float4*>(out + a.dense_w) = zero;
+            if (f & 2) *reinterpret_cast<float4*>(out + a.dense_h) = zero;
+            if (f & 4) *reinterpret_cast<float4*>(out + a.dense_h + a.dense_w) = zero;
+        }
     }
     __syncwarp();
 }
@@ -429,6 +417,7 @@ __device__ __forceinline__ void mma_role(const PipeScalars& p, const MmaEnv& e)
         b_it = 1;
         if (!mbar_wait(e.b_full, 0, e.abort_flag)) { report(p.status, 22); return; }
     }
+#pragma unroll 1
     for (UnitWalk u(p, e.m_first, e.u_first, e.u_count); u.left > 0; u.next(p)) {
         const int nt = u.tiles(p), kb = u.kb(p), ke = u.ke(p);
         const uint64_t lead = (uint64_t)(span_of(p, u).lead * 8);
@@ -436,16 +425,19 @@ __device__ __forceinline__ void mma_role(const PipeScalars& p, const MmaEnv& e)
         tc_fence_after();
         const uint32_t acc0 = e.tmem_base + (uint32_t)(buf * T) * acc_cols;
         uint32_t keep = 0u;
+#pragma unroll 1
         for (int c = kb; c < ke; ++c) {
             if (!mbar_wait(e.a_full + 8 * s, apar, e.abort_flag)) { report(p.status, 24); return; }
             uint64_t a = a_first + (uint64_t)((uint32_t)s * a_step) + lead;
             uint64_t b = RESIDENT ? b_first + (uint64_t)((uint32_t)(c * taps) * b_step) : 0;
             int sx = 0;
+#pragma unroll 1
             for (int tap = 0; tap < taps; ++tap) {
                 if (!RESIDENT) {
                     if (!mbar_wait(e.b_full + 8 * bs, bpar, e.abort_flag)) { report(p.status, 25); *e.b_used = b_it; *e.a_used = a_it; return; }
                     b = b_first + (uint64_t)((uint32_t)bs * b_step);
                 }
+#pragma unroll 1
                 for (int t = 0; t < nt; ++t) issue_tile<KIND>(acc0 + (uint32_t)t * acc_cols, a + (uint64_t)(t * 1024), b, b_half, idesc, idesc2, keep);
                 keep = 1u;
                 if (RESIDENT) b += b_step;
@@ -466,8 +458,10 @@ __device__ __forceinline__ void mma_role(const PipeScalars& p, const MmaEnv& e)
         *e.b_used = b_it; *e.a_used = a_it;
     }
     if (e.drain) {
+#pragma unroll 1
         for (int i = 0; i < a_stages && i < a_it; ++i) mbar_wait(e.a_empty + 8 * i, (uint32_t)((a_it - 1 - i) / a_stages) & 1u, e.abort_flag);
         if (!RESIDENT)
+#pragma unroll 1
             for (int i = 0; i < b_stages && i < b_it; ++i) mbar_wait(e.b_empty + 8 * i, (uint32_t)((b_it - 1 - i) / b_stages) & 1u, e.abort_flag);
     }
 }
@@ -519,6 +513,7 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
             int s = 0, it = 0;
             uint32_t par = 1u;
             bool live = true;
+#pragma unroll 1
             for (UnitWalk u(p, m_first, u_first, u_count); u.left > 0 && live; u.next(p)) {
                 const Span sp = span_of(p, u);
                 const uint32_t tx = (uint32_t)sp.rows * 64u;
@@ -530,16 +525,19 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
                     if (p.strips > 1 && img0 >= 0) { const int n = div_magic(img0, p.strips, p.magic_strip); strip0 = img0 - n * p.strips; img0 = n; }
                 }
                 const int first = (int)((long long)u.m * p.pix_ms);
+#pragma unroll 1
                 for (int c = u.kb(p), ce = u.ke(p); c < ce; ++c, ++it) {
                     if (!mbar_wait(a_empty + 8 * s, par, &abort_flag)) { report(p.status, 20); live = false; break; }
                     const uint32_t bar = a_raw + 8 * s;
                     uint32_t dst = smem_base + (uint32_t)s * p.a_stage_bytes;
                     mbar_expect_tx(bar, tx);
                     if (p.flat) {
+#pragma unroll 1
                         for (int k = 0; k < sp.blocks; ++k, dst += kTileM * 128u) tma_load_2d(dst, &gp.tm_a, bar, 16 * c, first + (sp.block0 + k) * kTileM);
                     } else {
                         int img = img0, h = h0, strip = strip0;
                         const uint32_t step = (uint32_t)p.box_pos * 128u;
+#pragma unroll 1
                         for (int k = 0; k < sp.blocks; ++k, dst += step) {
                             // (a block beyond the last row of its map is the zero row: outside the tensor, filled with zeros)
                             tma_load_4d(dst, &gp.tm_a, bar, 16 * c, strip * p.strip_w - p.col0, h * p.box_h, first + (img < 0 ? 0 : img));
@@ -563,7 +561,9 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
                 const int n = p.n_chunks * taps;
                 mbar_expect_tx(b_full, tx * (uint32_t)n);
                 uint32_t dst = dst0;
+#pragma unroll 1
                 for (int c = 0; c < p.n_chunks; ++c)
+#pragma unroll 1
                     for (int tap = 0; tap < taps; ++tap, dst += stage_bytes) {
                         tma_load_2d(dst, &gp.tm_b, b_full, tap * c_in + 16 * c, co0);
                         if (three) tma_load_2d(dst + half, &gp.tm_b_lo, b_full, tap * c_in + 16 * c, co0);
@@ -573,8 +573,11 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
                 int s = 0, it = 0;
                 uint32_t par = 1u;
                 bool live = true;
+#pragma unroll 1
                 for (UnitWalk u(p, m_first, u_first, u_count); u.left > 0 && live; u.next(p))
+#pragma unroll 1
                     for (int c = u.kb(p), ce = u.ke(p); c < ce && live; ++c)
+#pragma unroll 1
                         for (int tap = 0; tap < taps; ++tap, ++it) {
                             if (!mbar_wait(b_empty + 8 * s, par, &abort_flag)) { report(p.status, 21); live = false; break; }
                             const uint32_t bar = b_full + 8 * s, dst = dst0 + (uint32_t)s * stage_bytes;
@@ -616,6 +619,7 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
         const bool three = p.three != 0;
         float* tab = reinterpret_cast<float*>(smem + p.off_bn);
         if (BN_IN) {
+#pragma unroll 1
             for (int i = tid; i < C; i += kSplitThreads) { tab[2 * C + i] = __ldg(p.bn_gamma + i); tab[3 * C + i] = __ldg(p.bn_beta + i); }
             if (!CELL) pdl_wait();
         }
@@ -626,6 +630,7 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
         uint32_t par = 0;
         const bool store_y = BN_IN && slice == 0;
         bool ok = true;
+#pragma unroll 1
         for (UnitWalk cu(p, m_first, u_first, u_count); cu.left > 0; cu.next(p)) {
             const int kb = cu.kb(p), ke = cu.ke(p);
             const Span sp = span_of(p, cu);
@@ -639,8 +644,10 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
                     split_sync();
                 }
                 if (slice == 0 && cu.ul == 0 && cu.z == 0)
+#pragma unroll 1
                     for (int i = tid; i < 2 * C; i += kSplitThreads) p.bn_stats[(size_t)cur_m * 2 * C + i] = tab[i];
             }
+#pragma unroll 1
             for (int c = kb; c < ke; ++c) {
                 if (turn == my_group) {
                     ok = mbar_wait(a_raw + 8 * s, par, &abort_flag) && ok;
@@ -664,6 +671,7 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
                             py = div_magic(pos, p.Wp, p.magic_w); px = pos - py * p.Wp;
                         }
                         // four rows in flight; the block is allocated in whole batches, so the last one needs no bounds
+#pragma unroll 1
                         for (int row = row0; row < sp.rows; row += kRowBatch * row_step, hi += kRowBatch * byte_step, lo += kRowBatch * byte_step) {
                             float4 v[kRowBatch];
 #pragma unroll
@@ -676,10 +684,6 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
                                 if (FLAT) {
                                     inside[j] = own[j] = r < valid;
                                     off[j] = yo; yo += row_step * C;
-                                } else if (p.strips > 1) {
-                                    const Pixel w = locate(p, sp.pos0 + r);
-                                    inside[j] = w.in; own[j] = w.own && r >= own_lo && r < own_hi;
-                                    off[j] = w.n * p.in_sn + w.y * p.in_sh + w.x * p.in_sw;
                                 } else {
                                     inside[j] = px < p.W && py < p.Hv && pn >= 0 && r < valid;
                                     own[j] = inside[j] && r >= own_lo && r < own_hi;
@@ -708,6 +712,7 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
                                 for (int j = 0; j < kRowBatch; ++j) if (own[j]) *reinterpret_cast<float4*>(ydst + off[j]) = v[j];
                         }
                     } else if (three) {
+#pragma unroll 1
                         for (int row = row0; row < sp.rows; row += kRowBatch * row_step, hi += kRowBatch * byte_step, lo += kRowBatch * byte_step) {
                             float4 v[kRowBatch];
 #pragma unroll
@@ -748,36 +753,40 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
         uint32_t par = 0;
         // moments of the block so far: this lane's columns in shared memory, rows counted per warp
         float4* mom = reinterpret_cast<float4*>(smem + p.off_stat) + ew * 64 + lane;
-        unsigned int have_mask = 0;
+        bool have = false;
         int count = 0;
         if (stats)
             for (int gi = 0; gi < 2; ++gi) { mom[gi * 32 + kMomentPlane] = make_float4(0.f, 0.f, 0.f, 0.f); mom[gi * 32 + 2 * kMomentPlane] = make_float4(0.f, 0.f, 0.f, 0.f); }
+#pragma unroll 1
         for (UnitWalk u(p, m_first, u_first, u_count); u.left > 0; u.next(p)) {
             bool finish = true, ok = true;
             if (!alternate || turn == half) {
             const int nt = u.tiles(p);
-            // this lane's row of every tile, and which neighbours of a strided data gradient's sample get zeros
-            int roff[4], fill = 0;
-#pragma unroll
-            for (int t = 0; t < 4; ++t)
-                if (t < nt) {
-                    const int pos = (u.ul * T + t) * kTileM + quad * 32 + lane;
-                    if (FLAT) { roff[t] = pos < p.pos_per_m ? pos * C_out + co0 : -1; continue; }
-                    const Pixel px = locate(p, pos);
-                    roff[t] = px.own ? px.n * p.os_n + px.y * p.os_h + px.x * p.os_w + co0 : -1;
-                    if (p.zero_fill == 2 && px.own) {
-                        const bool right = 2 * px.x + 1 < p.out_w, below = 2 * px.y + 1 < p.out_h;
-                        fill |= ((right ? 1 : 0) | (below ? 2 : 0) | (right && below ? 4 : 0)) << (4 * t);
-                    }
-                }
-            float* out = p.out + (long long)u.m * p.out_ms;
-            const float* extra = p.extra ? p.extra + (long long)u.m * p.out_ms : nullptr;
+            float* out = p.out + (long long)u.m * p.out_ms + co0;
+            const float* extra = p.extra ? p.extra + (long long)u.m * p.out_ms + co0 : nullptr;
+            EmitArgs ea{out, extra, patch, nullptr, p.accumulate != 0, true, p.zero_fill, p.dense_h, p.dense_w};
+            // this lane's row of a tile, and which neighbours of a strided data gradient's sample get zeros
+            int ro = -1, fill = 0;
+            auto place = [&](int t) {
+                const int pos = (u.ul * T + t) * kTileM + quad * 32 + lane;
+                if (FLAT) { ro = pos < p.pos_per_m ? pos * C_out : -1; return; }
+                const Pixel px = locate(p, pos);
+                ro = px.own ? px.n * p.os_n + px.y * p.os_h + px.x * p.os_w : -1;
+                const bool right = 2 * px.x + 1 < p.out_w, below = 2 * px.y + 1 < p.out_h;
+                fill = (right ? 1 : 0) | (below ? 2 : 0) | (right && below ? 4 : 0);
+            };
+            const uint32_t acc0 = tmem_base + (uint32_t)(buf * T) * p.acc_cols + ((uint32_t)(quad * 32) << 16);
+            const size_t sk_tile = (size_t)kTileM * n_chunk;
+            const float* sk_all = nullptr;
+            // the first residuals travel while the accumulator is formed
+            float4 e[4];
+            place(t_first);
+            if (extra && t_first < nt) { ea.extra = extra + 32 * g_first; emit_residuals(ea, ro, lane, n_chunk - 32 * g_first >= 32 ? 3 : 2, 0, e); }
             ok = mbar_wait(acc_full + 8 * buf, par, &abort_flag);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok && lane == 0) report(p.status, 27);
             if (!CELL && p.pdl_late && u.last(p)) pdl_launch_dependents();
             tc_fence_after();
-            const uint32_t acc0 = tmem_base + (uint32_t)(buf * T) * p.acc_cols + ((uint32_t)(quad * 32) << 16);
             // 16 columns of this lane's row, hi and lo products added
             auto accumulator = [&](int t, int col, float* v) {
                 const uint32_t at = acc0 + (uint32_t)t * p.acc_cols + (uint32_t)col;
@@ -792,9 +801,6 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
                     tmem_ld_wait();
                 }
             };
-            finish = true;
-            const float* sk_all = nullptr;
-            const size_t sk_tile = (size_t)kTileM * n_chunk;
             if (ksplit > 1) {
                 // this CTA's partial sums; the CTA that takes the last ticket of the unit adds them in split order
                 const size_t key = (size_t)u.ul * p.slices + slice;
@@ -803,8 +809,11 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
                 float* partials = reinterpret_cast<float*>(base + kSplitKTicketBytes);
                 sk_all = partials + key * ksplit * T * sk_tile;
                 float* mine = partials + (key * ksplit + u.z) * T * sk_tile;
-                for (int g = g_first; g < groups; g += g_step)
-                    for (int t = t_first; t < nt; t += t_step)
+#pragma unroll 1
+                for (int t = t_first; t < nt; t += t_step)
+#pragma unroll 1
+                    for (int g = g_first; g < groups; g += g_step)
+#pragma unroll 1
                         for (int h = 2 * g; h < 2 * g + 2 && 16 * h < n_chunk; ++h) {
                             float v[16];
                             accumulator(t, 16 * h, v);
@@ -820,77 +829,46 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
                 finish = last_of_unit != 0;
                 if (finish) __threadfence();
             }
-            if (finish)
+            ea.ok = ok;
+#pragma unroll 1
+            for (int t = t_first; finish && t < nt; t += t_step) {
+                if (t > t_first) place(t);
+                const int rows = __popc(__ballot_sync(0xffffffffu, ro >= 0));
+                count += rows;
+#pragma unroll 1
                 for (int g = g_first, gi = 0; g < groups; g += g_step, ++gi) {
-                    const bool full = n_chunk - 32 * g >= 32;
-                    for (int t = t_first; t < nt; t += t_step) {
-                        const int ro = t == 0 ? roff[0] : (t == 1 ? roff[1] : (t == 2 ? roff[2] : roff[3]));
-                        // 16 columns of the row into the patch; the next 16 are on their way while these are stored
-                        const uint32_t at = acc0 + (uint32_t)t * p.acc_cols + (uint32_t)(32 * g);
-                        auto to_patch = [&](int h, const float* v) {
+                    const int left = n_chunk - 32 * g, lsh = left >= 32 ? 3 : 2;
+                    ea.out = out + 32 * g;
+                    if (extra) {
+                        ea.extra = extra + 32 * g;
+                        if (t > t_first || gi > 0) emit_residuals(ea, ro, lane, lsh, 0, e);
+                    }
+                    if (stats) ea.moments = mom + gi * 32;
+                    // 16 columns of the row at a time into the patch
+#pragma unroll 1
+                    for (int h = 0; h < 2 && 16 * h < left; ++h) {
+                        float v[16];
+                        if (ksplit > 1) {
 #pragma unroll
-                            for (int j = 0; j < 4; ++j) patch[lane * 8 + ((4 * h + j) ^ (lane & 7))] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
-                        };
-                        auto stage = [&](auto width) {
-                            constexpr int H = decltype(width)::value / 16;
-                            float v[16], w[16];
-                            if (ksplit > 1) {
-                                for (int h = 0; h < H; ++h) {
-#pragma unroll
-                                    for (int j = 0; j < 16; ++j) v[j] = 0.f;
-                                    for (int z = 0; z < ksplit; ++z) {
-                                        load16(sk_all + ((size_t)z * T + t) * sk_tile + ((size_t)(2 * g + h) * kTileM + quad * 32 + lane) * 16, w);
-#pragma unroll
-                                        for (int j = 0; j < 16; ++j) v[j] += w[j];
-                                    }
-                                    to_patch(h, v);
-                                }
-                            } else if (stacked) {
-                                tmem_ld16_nowait(at, v);
-                                tmem_ld16_nowait(at + (uint32_t)n_chunk, w);
-                                tmem_ld_wait();
+                            for (int j = 0; j < 16; ++j) v[j] = 0.f;
+#pragma unroll 1
+                            for (int z = 0; z < ksplit; ++z) {
+                                float w[16];
+                                load16(sk_all + ((size_t)z * T + t) * sk_tile + ((size_t)(2 * g + h) * kTileM + quad * 32 + lane) * 16, w);
 #pragma unroll
                                 for (int j = 0; j < 16; ++j) v[j] += w[j];
-                                if (H == 2) {
-                                    float x[16];
-                                    tmem_ld16_nowait(at + 16u, x);
-                                    tmem_ld16_nowait(at + (uint32_t)n_chunk + 16u, w);
-                                    to_patch(0, v);
-                                    tmem_ld_wait();
-#pragma unroll
-                                    for (int j = 0; j < 16; ++j) v[j] = x[j] + w[j];
-                                    to_patch(1, v);
-                                } else {
-                                    to_patch(0, v);
-                                }
-                            } else {
-                                tmem_ld16_nowait(at, v);
-                                if (H == 2) tmem_ld16_nowait(at + 16u, w);
-                                tmem_ld_wait();
-                                to_patch(0, v);
-                                if (H == 2) to_patch(1, w);
                             }
-                        };
-                        const EmitArgs ea{out + 32 * g, extra ? extra + 32 * g : nullptr, patch, stats ? mom + gi * 32 : nullptr, p.accumulate != 0, ok,
-                                          p.zero_fill == 2 ? fill >> (4 * t) : 0, p.zero_fill == 2, p.dense_h, p.dense_w, C_out};
-                        const bool have = (have_mask >> gi) & 1u;
-                        const auto go32 = [&] { stage(std::integral_constant<int, 32>()); };
-                        const auto go16 = [&] { stage(std::integral_constant<int, 16>()); };
-                        if (FLAT && (u.ul * T + t) * kTileM + quad * 32 + 32 <= p.pos_per_m) {
-                            if (full) emit_rows<8, true>(ea, ro, lane, have, go32);
-                            else emit_rows<4, true>(ea, ro, lane, have, go16);
-                            if (stats) { have_mask |= 1u << gi; if (gi == 0) count += 32; }
                         } else {
-                            if (full) emit_rows<8, false>(ea, ro, lane, have, go32);
-                            else emit_rows<4, false>(ea, ro, lane, have, go16);
-                            if (stats) {
-                                const int n = __popc(__ballot_sync(0xffffffffu, ro >= 0));
-                                if (n) have_mask |= 1u << gi;
-                                if (gi == 0) count += n;
-                            }
+                            accumulator(t, 32 * g + 16 * h, v);
                         }
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) patch[lane * 8 + ((4 * h + j) ^ (lane & 7))] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
                     }
+                    __syncwarp();
+                    emit_rows(ea, ro, fill, lane, lsh, have, e);
                 }
+                if (rows) have = true;
+            }
             // the accumulator is read: the next unit's MMAs may have it
             tc_fence_before();
             __syncwarp();
@@ -902,17 +880,14 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
             if (stats && finish && (ksplit > 1 || u.last_of_block())) {
                 // the block's moments: lanes, then the warps' parts, each about its own shift
                 float* contrib = reinterpret_cast<float*>(smem + p.off_stat + 3u * 16u * kMomentPlane) + (size_t)flip * parts * (3 * n_chunk + 1);
+#pragma unroll 1
                 for (int g = g_first, gi = 0; g < groups; g += g_step, ++gi) {
                     const int lpr = n_chunk - 32 * g >= 32 ? 8 : 4;
                     float4 sd = mom[gi * 32 + kMomentPlane], sq = mom[gi * 32 + 2 * kMomentPlane];
                     const float4 k = mom[gi * 32], zero = make_float4(0.f, 0.f, 0.f, 0.f);
                     mom[gi * 32 + kMomentPlane] = zero; mom[gi * 32 + 2 * kMomentPlane] = zero;
-                    for (int o = 16; o >= lpr; o >>= 1) {
-                        sd.x += __shfl_xor_sync(0xffffffffu, sd.x, o); sd.y += __shfl_xor_sync(0xffffffffu, sd.y, o);
-                        sd.z += __shfl_xor_sync(0xffffffffu, sd.z, o); sd.w += __shfl_xor_sync(0xffffffffu, sd.w, o);
-                        sq.x += __shfl_xor_sync(0xffffffffu, sq.x, o); sq.y += __shfl_xor_sync(0xffffffffu, sq.y, o);
-                        sq.z += __shfl_xor_sync(0xffffffffu, sq.z, o); sq.w += __shfl_xor_sync(0xffffffffu, sq.w, o);
-                    }
+#pragma unroll 1
+                    for (int o = 16; o >= lpr; o >>= 1) { sd = lane_sum(sd, o); sq = lane_sum(sq, o); }
                     if (lane < lpr) {
                         float* c3 = contrib + (size_t)part * 3 * n_chunk + 32 * g + 4 * lane;
                         *reinterpret_cast<float4*>(c3) = k;
@@ -922,24 +897,25 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
                 }
                 float* counts = contrib + (size_t)parts * 3 * n_chunk;
                 if (lane == 0 && (whole || half == 0)) counts[part] = (float)count;
-                count = 0; have_mask = 0;
+                count = 0; have = false;
                 epi_sync();
                 if (tid < n_chunk) {
-                    float N = 0.f, k0 = 0.f, sum = 0.f, m2 = 0.f;
-                    for (int w = 0; w < parts; ++w)
-                        if (counts[w] > 0.f) {
-                            const float k = contrib[(size_t)w * 3 * n_chunk + tid];
-                            if (N == 0.f) k0 = k;
-                            N += counts[w];
-                            sum += fmaf(counts[w], k - k0, contrib[(size_t)w * 3 * n_chunk + n_chunk + tid]);
-                        }
-                    const float dm = N > 0.f ? sum / N : 0.f;
-                    for (int w = 0; w < parts; ++w)
-                        if (counts[w] > 0.f) {
-                            const float n = counts[w], d = contrib[(size_t)w * 3 * n_chunk + n_chunk + tid], e = d / n;
-                            const float away = contrib[(size_t)w * 3 * n_chunk + tid] - k0 + e - dm;
-                            m2 += contrib[(size_t)w * 3 * n_chunk + 2 * n_chunk + tid] - d * e + n * away * away;
-                        }
+                    // parts about their own shifts k_w: sum and squares about the first one's,
+                    //   sum (x - k0) = sum_w [d_w + n_w e],  sum (x - k0)^2 = sum_w [q_w + e (2 d_w + n_w e)],  e = k_w - k0
+                    float N = 0.f, k0 = 0.f, sum = 0.f, sq = 0.f;
+                    const float* c3 = contrib + tid;
+#pragma unroll 1
+                    for (int w = 0; w < parts; ++w, c3 += 3 * n_chunk) {
+                        const float n = counts[w];
+                        if (n == 0.f) continue;
+                        const float d = c3[n_chunk];
+                        if (N == 0.f) k0 = c3[0];
+                        const float e = c3[0] - k0;
+                        N += n;
+                        sum += fmaf(n, e, d);
+                        sq += fmaf(e, fmaf(n, e, 2.f * d), c3[2 * n_chunk]);
+                    }
+                    const float dm = N > 0.f ? sum / N : 0.f, m2 = fmaxf(fmaf(-sum, dm, sq), 0.f);
                     float* dst = p.st_partials + (size_t)u.m * partial_floats(p.blocks_per_m, C_out);
                     const int r = u.ul / p.unit_block;
                     float* row = dst + (size_t)r * 2 * C_out + co0 + tid;
@@ -1117,8 +1093,8 @@ __global__ void __launch_bounds__(kPipeThreads, 1) conv_pipe_cell_kernel(const _
 // Statistics for a BN that runs a kernel of its own although its input came from a convolution that left moments.
 __global__ void __launch_bounds__(256) bn_finalize_kernel(const float* __restrict__ partials, int units, int C, double inv_rows, float eps, float* stats)
 {
-    extern __shared__ float4 dyn[];                   // 3 x 256 float4, then the table
-    float* tab = reinterpret_cast<float*>(dyn + 768);
+    extern __shared__ float4 dyn[];                   // 4 x 256 float4, then the table
+    float* tab = reinterpret_cast<float*>(dyn + 1024);
     const int m = blockIdx.x;
     pdl_launch_dependents();
     pdl_wait();
@@ -1174,7 +1150,7 @@ int sm_count()
 
 constexpr int kPlanSms = 148;                         // the split of the work is planned for a whole B200, with or without a device at hand
 inline unsigned int stat_bytes(int n_chunk) { return 3u * 16u * kMomentPlane + (unsigned int)(2 * (n_chunk <= 64 ? 8 : 4) * (3 * n_chunk + 1) * 4 + 127) & ~127u; }
-inline unsigned int bn_bytes(int c_in) { return (unsigned int)(4 * c_in * 4 + 3 * kSplitThreads * 16); }
+inline unsigned int bn_bytes(int c_in) { return (unsigned int)(4 * c_in * 4 + 4 * kSplitThreads * 16); }
 
 }  // namespace
 
@@ -1288,7 +1264,7 @@ bool conv_pipe_geom(const ConvShape& s, int pass, int passes, int M, ConvPipeGeo
 }
 
 bool conv_pipe_can_fuse_bn_output(const ConvPipeGeom& g) { return g.n_chunk <= 128; }      // a warp keeps the moments of two groups of 32 channels
-bool conv_pipe_can_fuse_bn_input(const ConvShape& s) { return s.stride == 1 && s.C % 16 == 0 && s.C <= 512; }
+bool conv_pipe_can_fuse_bn_input(const ConvShape& s) { return s.stride == 1 && s.C % 16 == 0 && s.C <= 512 && s.W <= 254; }      // (no column strips)
 
 size_t conv_pipe_splitk_bytes(const ConvShape& s, int pass, int passes, int M)
 {
@@ -1387,14 +1363,14 @@ cudaError_t conv_pipe_prepare(ConvPipePlan* plan, const ConvShape& s, int pass, 
     p.off_stage = (p.off_b + (unsigned int)g.b_stages * g.b_stage_bytes + 127u) & ~127u;
     p.off_stat = p.off_stage + kEpiWarps * 4096u;
     p.off_red = p.off_stat + stat_bytes(g.n_chunk);
-    p.off_bn = p.off_red + 3 * kSplitThreads * 16;
+    p.off_bn = p.off_red + 4 * kSplitThreads * 16;
     L->smem = p.off_red + 1024;
     if (bn && bn->out_partials) {
         if (!conv_pipe_can_fuse_bn_output(g)) return cudaErrorNotSupported;
         p.st_partials = bn->out_partials;
     }
     if (bn && bn->in_partials) {
-        if (pass != PASS_FWD || s.stride != 1 || v.c_in > 512 || bn->in_blocks < 1) return cudaErrorNotSupported;
+        if (pass != PASS_FWD || !conv_pipe_can_fuse_bn_input(s) || bn->in_blocks < 1) return cudaErrorNotSupported;
         p.bn_partials = bn->in_partials; p.bn_units = bn->in_blocks; p.bn_gamma = bn->in_gamma; p.bn_beta = bn->in_beta;
         p.bn_stats = bn->in_stats; p.bn_y = bn->in_y; p.bn_eps = bn->in_eps;
         p.bn_inv_rows = 1.0 / ((double)s.N * s.H * s.W);
@@ -1464,7 +1440,7 @@ cudaError_t conv_pipe_cell_launch(const void* d_ops, int n_ops, int m_first, int
 cudaError_t bn_finalize_partials(const float* partials, int units, int C, float eps, double rows, float* stats, int m_count, cudaStream_t st,
                                  int64_t* n_launch)
 {
-    launch_pdl(bn_finalize_kernel, dim3(m_count), dim3(256), (size_t)768 * 16 + 2 * (size_t)C * 4, st, partials, units, C, 1.0 / rows, eps, stats);
+    launch_pdl(bn_finalize_kernel, dim3(m_count), dim3(256), (size_t)1024 * 16 + 2 * (size_t)C * 4, st, partials, units, C, 1.0 / rows, eps, stats);
     if (n_launch) ++*n_launch;
     return cudaGetLastError();
 }
