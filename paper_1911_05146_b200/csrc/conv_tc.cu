@@ -51,33 +51,7 @@ constexpr int kFwdMaxStages = 4;
 #endif
 constexpr int kWgradWantCtas = HPF_WGRAD_WANT;   // CTAs a weight-gradient launch spreads its pixel walk over at least
 constexpr int kMultiTileFrom = 2 * 296;     // CTAs (two per SM) beyond which a forward / data-gradient launch gives each CTA two tiles
-constexpr unsigned int kCellTmemCols = 256;  // tensor-memory columns a persistent cell CTA may hold (two such CTAs share an SM's 512)
-constexpr unsigned int kCellSmemBudget = 100 * 1024;   // dynamic shared memory of a cell CTA (two per SM)
 constexpr unsigned int kWgradSlack = 16384;   // an MMA reads 128 operand rows (16 KB) from a base that may be the last one in use
-
-// Optional timelines for latency studies (debug builds only).  HPF_TC_TIMELINE=2: every CTA of the forward kernel
-// stamps its milestones in shared memory and adds the elapsed times to per-class totals (class = window size and
-// grid size), read back with hpf_debug_timeline.  Otherwise: globaltimer stamps of CTA (0,0) behind the status word.
-#if defined(HPF_TC_TIMELINE) && HPF_TC_TIMELINE == 2
-__device__ unsigned long long g_tl_acc[8][16];
-#define HPF_TL(slot)                                                                                      \
-    do {                                                                                                  \
-        unsigned long long t_;                                                                            \
-        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t_));                                            \
-        tl_s[(slot)] = t_;                                                                                \
-    } while (0)
-#elif defined(HPF_TC_TIMELINE)
-#define HPF_TL(slot)                                                                                      \
-    do {                                                                                                  \
-        if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) {                                      \
-            unsigned long long t_;                                                                        \
-            asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t_));                                        \
-            reinterpret_cast<unsigned long long*>(p.status)[2 + (slot)] = t_;                             \
-        }                                                                                                 \
-    } while (0)
-#else
-#define HPF_TL(slot) do {} while (0)
-#endif
 
 // ------------------------------------------------------------------------------------------------
 // kernel parameters
@@ -104,39 +78,21 @@ struct FwdScalars {
     int zero_fill;               // > 1: the output pixel grid is strided, fill the rest of each patch with zeros
     int out_h, out_w;            // dense output extent (zero fill bounds)
     unsigned int a_bytes, b_bytes, stage_bytes, tx_bytes, tmem_cols, idesc, idesc2, stg_pitch;
-    // batch-norm statistics folded into the write-out (see ConvBnFuse): 0 none, 1 sums of the output and its square
-    int stat_mode;
-    float* stat_partials;        // [tiles][2][c_out] per-tile partial sums
-    unsigned int* stat_ticket;   // counts finished CTAs; zero between launches
-    float* stat_out;             // mean[c_out], rstd[c_out], written by the CTA that finishes last
-    float stat_eps;
-    float stat_inv_tile_rows;    // 1 / (pixels of one tile)
-    double stat_inv_rows;        // 1 / (pixels the statistics run over)
-    // BN+ReLU applied to the activation operand on its way to the tensor core (see ConvBnFuse::in_mode)
     // several tiles per CTA (MULTI kernel; tile j of CTA b is tile b*tiles_per_cta + j): tile j+1's loads, split and MMAs
     // run under tile j's write-out, each tile has its own accumulator columns, and the write-out is staged in a region
     // of its own
     int n_tiles, tiles_per_cta;
     unsigned int acc_cols;       // tensor-memory columns of one tile's accumulator
     unsigned int stg_off;        // byte offset of the write-out staging area (0: it reuses the idle pipeline buffers)
-    int bn_in;
-    int in_w, in_h;              // extent of the input pixel grid (the padding mask)
-    const float* bn_in_gamma;
-    const float* bn_in_beta;
-    const float* bn_in_stats;    // bn_in 1: mean[c_in], rstd[c_in] (left by the kernel that produced x)
-    // bn_in 2: the statistics are derived here from the producer's per-tile sums and stored by the first CTA
-    const float* bn_in_partials; // [bn_in_tiles][2][c_in]
-    float* bn_in_stats_out;
-    int bn_in_tiles;
-    float bn_in_eps;
-    double bn_in_inv_rows;
-    float* bn_in_y;              // relu(bn(x)), dense [N][in_h][in_w][c_in], written by the CTAs of the first channel slice
     // K loop split over gridDim.z CTAs (launches of a few tiles with a long K loop): every CTA stores its partial tile, the
     // one that takes the last ticket of its (tile, channel slice) adds them in split order and writes the output
     int pdl_late;                // see the kernel's first statement
     int ksplit;
     float* splitk_partials;      // [(tile * slices + slice) * ksplit + z][128][n_chunk]
     unsigned int* splitk_ticket; // one per (tile, slice); zero between launches
+    // micro-batches: a launch covers several, each of ctas_per_m CTAs along x
+    int ctas_per_m;
+    long long out_ms, sk_ms;     // floats between their outputs, bytes between their split-K scratch
 };
 struct alignas(64) FwdParams {
     CUtensorMap tm_a;            // activations {C, Wv, Hv, N}
@@ -192,105 +148,25 @@ struct alignas(64) WgradDirectParams {
     WgradDirectScalars s;
 };
 
-// BN statistics from per-tile moments [n_tiles][2][C]: per tile and channel the mean of the tile's values and the sum
-// of their squared deviations from that mean (M2).  Every tile holds the same number of values (the host fuses only
-// launches whose tiles are all full), so the total is
-//     mean = average of the tile means,   M2 = sum of the tile M2 + n_tile * sum (tile mean - mean)^2,
-// evaluated about tile 0's mean so that no difference of large numbers appears anywhere: the result stays accurate
-// however far a channel's mean is from zero compared with its spread.  What is added up are small differences of tile
-// means, their squares and the non-negative tile M2, at most a few hundred terms: fp32 sums in a fixed order (every
-// caller gets the same bits), the final combination in fp64.  Called by 256 threads (tid 0..255) that share named
-// barrier 1; C is a power of two in 16..256; bn_ws: 8 x 32 x 8 floats of shared memory.  On return thread tid < C holds
-// its channel's mean and 1/sqrt(var + eps).
-// Consecutive threads read consecutive float4 of a tile's row (coalesced: every CTA of a launch reads these same few
-// lines); the lanes of a warp that share a column are added by a butterfly, the warps through shared memory.
-__device__ __forceinline__ void bn_combine_partials(const float* partials, int n_tiles, int C, double inv_rows, float eps,
-                                                    float (*bn_ws)[32][8], int tid, float* mean, float* rstd)
-{
-    const int ncol4 = C >> 1;                          // float4 columns of one tile's [2][C] moments: 8..128
-    const int col4 = tid % ncol4, ln = tid / ncol4, L = 256 / ncol4;
-    const float4* part = reinterpret_cast<const float4*>(partials);
-    // the first C/4 columns are tile means: accumulated as differences from tile 0's mean (and their squares)
-    const bool mean_col = col4 < (C >> 2);
-    const float4 ref = mean_col ? __ldcg(part + col4) : make_float4(0.f, 0.f, 0.f, 0.f);
-    float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f, b0 = 0.f, b1 = 0.f, b2 = 0.f, b3 = 0.f;
-    // eight rows per batch, all eight loads in flight together (a loop that used each load before issuing the next would
-    // pay an L2 round trip per row); rows beyond the last add zero
-    for (int k0 = ln; k0 < n_tiles; k0 += 8 * L) {
-        float4 v[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const int k = k0 + j * L;
-            v[j] = k < n_tiles ? __ldcg(part + (size_t)k * ncol4 + col4) : ref;
-        }
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const float f0 = v[j].x - ref.x, f1 = v[j].y - ref.y, f2 = v[j].z - ref.z, f3 = v[j].w - ref.w;
-            a0 += f0; a1 += f1; a2 += f2; a3 += f3;
-            b0 = fmaf(f0, f0, b0); b1 = fmaf(f1, f1, b1); b2 = fmaf(f2, f2, b2); b3 = fmaf(f3, f3, b3);
-        }
-    }
-    // lanes of one warp that share a column (fewer than 32 columns): a fixed butterfly
-    for (int off = 16; off >= ncol4; off >>= 1) {
-        a0 += __shfl_xor_sync(0xffffffffu, a0, off); a1 += __shfl_xor_sync(0xffffffffu, a1, off);
-        a2 += __shfl_xor_sync(0xffffffffu, a2, off); a3 += __shfl_xor_sync(0xffffffffu, a3, off);
-        b0 += __shfl_xor_sync(0xffffffffu, b0, off); b1 += __shfl_xor_sync(0xffffffffu, b1, off);
-        b2 += __shfl_xor_sync(0xffffffffu, b2, off); b3 += __shfl_xor_sync(0xffffffffu, b3, off);
-    }
-    const int warp = tid >> 5, lane = tid & 31;
-    if (lane < ncol4) {
-        float* d = bn_ws[warp][lane];
-        *reinterpret_cast<float4*>(d) = make_float4(a0, a1, a2, a3);
-        if (mean_col) *reinterpret_cast<float4*>(d + 4) = make_float4(b0, b1, b2, b3);
-    }
-    // tile 0's means travel in the half of an M2 column's slot that nothing else uses (that of the channel's M2 column in
-    // the first warp that holds it), so that nothing has to be fetched again after the barrier
-    if (mean_col && ln == 0) {
-        const int qv0 = (C >> 2) + col4;
-        *reinterpret_cast<float4*>(bn_ws[ncol4 > 32 ? qv0 >> 5 : 0][qv0 & 31] + 4) = ref;
-    }
-    asm volatile("bar.sync 1, 256;" ::: "memory");
-    if (tid < C) {
-        // column q sits in lane q % 32 of the warps q / 32, q / 32 + ncol4 / 32, ... (of every warp when there are at most
-        // 32 columns): added in ascending warp order
-        const int qm = tid >> 2, qv = (C >> 2) + (tid >> 2), comp = tid & 3;
-        const int wstep = ncol4 > 32 ? ncol4 >> 5 : 1;
-        float sd = 0.f, sq = 0.f, m2 = 0.f;
-        for (int w = (ncol4 > 32 ? qm >> 5 : 0); w < 8; w += wstep) { sd += bn_ws[w][qm & 31][comp]; sq += bn_ws[w][qm & 31][4 + comp]; }
-        for (int w = (ncol4 > 32 ? qv >> 5 : 0); w < 8; w += wstep) m2 += bn_ws[w][qv & 31][comp];
-        // (no fp64 division: mean = ref + sd / T and var = M2 / rows + (sq - sd^2 / T) / T with 1 / T in fp32-exact steps)
-        const double inv_tiles = (double)(1.0f / (float)n_tiles);
-        const double dsd = (double)sd;
-        const double m = (double)bn_ws[ncol4 > 32 ? qv >> 5 : 0][qv & 31][4 + comp] + dsd * inv_tiles;
-        double var = (double)m2 * inv_rows + ((double)sq - dsd * dsd * inv_tiles) * inv_tiles;
-        if (var < 0.0) var = 0.0;
-        *mean = (float)m;
-        *rstd = 1.0f / sqrtf((float)(var + (double)eps));          // correctly rounded fp32 operations: within an ulp or two of the fp64 result
-    }
-}
-
 // ------------------------------------------------------------------------------------------------
 // forward / data-gradient kernel: 10 warps = TMA producer, MMA issuer, 8 splitter / epilogue warps
 // ------------------------------------------------------------------------------------------------
-// One CTA's share of a forward / data-gradient launch: `vb` of `vg` (block index and grid size of the launch as a stand-alone
-// launch has them).  MODE 0: one 128-pixel tile per CTA (the shortest launch; what a launch of up to one wave wants).
-// MODE 1: p.tiles_per_cta tiles per CTA for launches of several waves: fewer CTAs, and a tile's write-out hides the next
-// tile's loads, split and MMAs.  MODE 2: the K loop split over vg.z CTAs.  MODE 3: inside the persistent cell kernel, which
-// runs many launches one after the other in one resident grid: tiles per CTA and K split are read from the parameters,
-// tensor memory is allocated once by the caller, the mbarriers are set up again for every call, and nothing of the
-// programmatic-launch protocol applies.  `p` (shared memory) holds gp->s.
-template <int MODE>
-__device__ __forceinline__ int conv_fwd_cta(const FwdParams* gpp, FwdScalars& p, const uint3 vb, const uint3 vg, const uint32_t cell_tmem_base,
-                                             const bool cell_first)
+// MULTI: p.tiles_per_cta tiles per CTA for launches of several waves: fewer CTAs, and a tile's write-out hides the next tile's
+// loads, split and MMAs; otherwise one 128-pixel tile per CTA (the shortest launch; what a launch of up to one wave wants).
+// KSPLIT: the K loop split over gridDim.z CTAs.
+template <bool MULTI, bool KSPLIT>
+__global__ void __launch_bounds__(320, 2) conv_tc_fwd_kernel(const __grid_constant__ FwdParams gp, const int m_first)
 {
-    const FwdParams& gp = *gpp;
-    constexpr bool CELL = MODE == 3;
-    const bool MULTI = CELL ? p.tiles_per_cta > 1 : MODE == 1;
-    const bool KSPLIT = CELL ? p.ksplit > 1 : MODE == 2;
-#if defined(HPF_TC_TIMELINE) && HPF_TC_TIMELINE == 2
-    __shared__ unsigned long long tl_s[16];
-    if (threadIdx.x < 16) tl_s[threadIdx.x] = 0;
-#endif
+    __shared__ FwdScalars p;                 // scalar parameters, see load_scalars
+    // Programmatic launch: the next kernel of the stream may be scheduled once every CTA of this one has said so.  Early (here):
+    // the successor's set-up hides under this kernel, which shortens a lone stage's chain of kernels.  Late (when the first
+    // accumulator is complete, see below): the successor's CTAs do not sit in SM slots for the whole life of this kernel,
+    // which is what counts when every stage is busy and slots are what the stages compete for.  The host chooses per launch.
+    if (!gp.s.pdl_late) pdl_launch_dependents();
+    load_scalars(&p, &gp.s);
+    __syncthreads();
+    const int micro = m_first + (int)blockIdx.x / p.ctas_per_m;
+    const uint3 vb = make_uint3(blockIdx.x % p.ctas_per_m, blockIdx.y, blockIdx.z);
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint64_t bars[3 * 8 + 4];       // full[8], empty[8], split[8], accum[4] (one per tile of this CTA)
     __shared__ uint32_t tmem_slot;
@@ -323,7 +199,6 @@ __device__ __forceinline__ int conv_fwd_cta(const FwdParams* gpp, FwdScalars& p,
         q0 = tw__ * p.box_w; p0 = (t__ % p.tiles_h) * p.box_h; n0 = (t__ / p.tiles_h) * p.box_n; \
     }
 
-    if (threadIdx.x == 0) HPF_TL(0);
     const int total = p.R * p.R * p.n_kchunks;
     // this CTA's share of the K loop (all of it unless the launch splits K over gridDim.z)
     const int kb = KSPLIT ? (int)(((long long)total * vb.z) / p.ksplit) : 0;
@@ -338,23 +213,21 @@ __device__ __forceinline__ int conv_fwd_cta(const FwdParams* gpp, FwdScalars& p,
         if (KSPLIT) { f_tap = kb / p.n_kchunks; f_kc = kb % p.n_kchunks; f_r = f_tap / p.R; f_sx = f_tap % p.R; }
     }
     if (threadIdx.x == 0) {
-        if (CELL && !cell_first)       // the barriers of the call before are retired first
-            for (int j = 0; j < 3 * 8 + 4; ++j) mbar_inval(full0 + 8 * j);
         for (int s = 0; s < p.stages; ++s) { mbar_init(full0 + 8 * s, 1); mbar_init(empty0 + 8 * s, 1); mbar_init(split0 + 8 * s, 8); }
         for (int j = 0; j < 4; ++j) mbar_init(accum_bar + 8 * j, 1);
         abort_flag = 0; issued = 0; consumed = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (threadIdx.x == 32) { prefetch_tmap(&gp.tm_a); prefetch_tmap(&gp.tm_b); if (p.passes == 3) prefetch_tmap(&gp.tm_b_lo); }
-    if (!CELL && warp == 0) tmem_alloc(smem_u32(&tmem_slot), p.tmem_cols);
+    if (warp == 0) tmem_alloc(smem_u32(&tmem_slot), p.tmem_cols);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     // Everything above touched only parameters, shared and tensor memory.  The TMA producer (warp 0) first works out
     // its first tile's coordinates - a chain of dependent shared-memory reads and integer divisions of most of a
     // microsecond - and waits for the preceding kernel only then, right before its first copy.
-    if (!CELL && warp != 0) pdl_wait();
-    const uint32_t tmem_base = CELL ? cell_tmem_base : tmem_slot;
+    if (warp != 0) pdl_wait();
+    const uint32_t tmem_base = tmem_slot;
 
     if (warp == 0) {
         if (elect_one()) {
@@ -366,6 +239,7 @@ __device__ __forceinline__ int conv_fwd_cta(const FwdParams* gpp, FwdScalars& p,
             const int stages = p.stages, nkc = p.n_kchunks, R = p.R, pad = p.pad, kchunk = p.kchunk, c_in = p.c_in;
             const uint32_t tx = p.tx_bytes, stage_bytes = p.stage_bytes;
             const bool three = p.passes == 3;
+            const int n_base = micro * p.N;      // (a ragged last box reaches into the next micro-batch: rows nobody stores)
             for (int j = 0; j < my_tiles && live; ++j) {
                 int q0 = f_q0, p0 = f_p0, n0 = f_n0;
                 if (j > 0) {
@@ -378,26 +252,16 @@ __device__ __forceinline__ int conv_fwd_cta(const FwdParams* gpp, FwdScalars& p,
                     if (!mbar_wait(empty0 + 8 * st, par, &abort_flag)) { report(p.status, 1); live = false; break; }
                     const uint32_t dst = smem_base + st * stage_bytes;
                     const int cx = kc * kchunk, cq = q0 + sx - pad, cp = p0 + r - pad, cb = tap * c_in + cx;
-                    if (!CELL && it == 0) { pdl_wait(); HPF_TL(1); }
+                    if (it == 0) pdl_wait();
                     mbar_expect_tx(full0 + 8 * st, tx);
-                    tma_load_4d(dst, &gp.tm_a, full0 + 8 * st, cx, cq, cp, n0);
+                    tma_load_4d(dst, &gp.tm_a, full0 + 8 * st, cx, cq, cp, n_base + n0);
                     tma_load_2d(dst + off_b, &gp.tm_b, full0 + 8 * st, cb, co0);
                     if (three) tma_load_2d(dst + off_blo, &gp.tm_b_lo, full0 + 8 * st, cb, co0);
-                    if (it == 0) HPF_TL(2);
                     if (++kc == nkc) { kc = 0; ++tap; if (++sx == R) { sx = 0; ++r; } }
                     if (++st == stages) { st = 0; par ^= 1u; }
                 }
             }
-            if (!CELL && it == 0) pdl_wait();         // nothing to copy: still ordered behind the preceding kernel
-            if (CELL && live) {
-                // The MMA issuer's last commits on the `empty` barriers are awaited by nobody in a stand-alone launch.  Here
-                // the barriers are set up again for the next call, so every arrival still on its way has to land first.
-                const int left = it < stages ? it : stages;
-                for (int j = 0; j < left; ++j) {
-                    if (!mbar_wait(empty0 + 8 * st, par, &abort_flag)) { report(p.status, 8); break; }
-                    if (++st == stages) { st = 0; par ^= 1u; }
-                }
-            }
+            if (it == 0) pdl_wait();         // nothing to copy: still ordered behind the preceding kernel
             issued = it;
         }
     } else if (warp == 1) {
@@ -411,10 +275,10 @@ __device__ __forceinline__ int conv_fwd_cta(const FwdParams* gpp, FwdScalars& p,
             const bool stacked = p.stacked != 0;
             const int stages = p.stages, k8n = p.kchunk / 8;
             const bool three = p.passes == 3;
-            // the splitter warps write the lo part (and with BN+ReLU on the way in rewrite the tile) before the MMAs of the
+            // the splitter warps write the lo part before the MMAs of the
             // stage are issued.  (Issuing the MMAs that read only the tile as copied ahead of the splitters' barrier was
             // measured: the step got 1.7 ms slower.)
-            const bool split_first = three || p.bn_in != 0;
+            const bool split_first = three;
             int it = 0, s = 0;
             uint32_t par = 0;
             bool live = true;
@@ -424,7 +288,6 @@ __device__ __forceinline__ int conv_fwd_cta(const FwdParams* gpp, FwdScalars& p,
                 if (!mbar_wait(full0 + 8 * s, par, &abort_flag)) { report(p.status, 2); live = false; break; }
                 if (split_first && !mbar_wait(split0 + 8 * s, par, &abort_flag)) { report(p.status, 6); live = false; break; }
                 tc_fence_after();
-                if (it == 0) HPF_TL(5);
                 const uint32_t st = smem_base + s * stage_bytes;
                 const uint64_t a0 = desc_hi | (uint64_t)((st & 0x3FFFFu) >> 4);
                 const uint64_t b0 = desc_hi | (uint64_t)(((st + off_b) & 0x3FFFFu) >> 4);
@@ -455,112 +318,12 @@ __device__ __forceinline__ int conv_fwd_cta(const FwdParams* gpp, FwdScalars& p,
               if (live) umma_commit(accum_bar + 8 * j);      // tile j's accumulator is complete once these MMAs retire
             }
             consumed = it;
-            HPF_TL(6);
         }
     } else {
         // ---- warps 2..9: split the activation tile into hi / lo, then the epilogue ----
         const int tid = threadIdx.x - 64;               // 0..255
         bool ok = true;
-        if (p.bn_in) {
-            // ---- BN+ReLU on the way in: the tile holds the BN's input x; the operand is relu(gamma*xhat+beta) ----
-            __shared__ __align__(16) float bn_par[4][256];      // mean, rstd, gamma, beta per input channel
-            const int C = p.c_in;
-            if (p.bn_in == 2) {
-                // The producer left only its per-tile sums (few enough that adding them here, under the first copy's
-                // latency, is cheaper than a ticket at the producer's end): every CTA adds them in the same fixed order,
-                // so all CTAs hold identical statistics; the first CTA stores them for the backward pass.
-                __shared__ __align__(16) float bn_red[8][32][8];
-                float gam = 0.f, bet = 0.f, mu = 0.f, rs = 0.f;
-                if (tid < C) { gam = __ldg(p.bn_in_gamma + tid); bet = __ldg(p.bn_in_beta + tid); }   // travel with the sums
-                bn_combine_partials(p.bn_in_partials, p.bn_in_tiles, C, p.bn_in_inv_rows, p.bn_in_eps, bn_red, tid, &mu, &rs);
-                if (tid < C) {
-                    bn_par[0][tid] = mu; bn_par[1][tid] = rs; bn_par[2][tid] = gam; bn_par[3][tid] = bet;
-                    if (vb.x == 0 && vb.y == 0) { p.bn_in_stats_out[tid] = mu; p.bn_in_stats_out[C + tid] = rs; }
-                }
-            }
-            // the statistics written by the kernel before (not the read-only path) and the parameters: fetched now, used
-            // after the index arithmetic below, which runs under their latency
-            float ld_mu = 0.f, ld_rs = 0.f, ld_g = 0.f, ld_b = 0.f;
-            if (p.bn_in != 2 && tid < C) {
-                ld_mu = __ldcg(p.bn_in_stats + tid); ld_rs = __ldcg(p.bn_in_stats + C + tid);
-                ld_g = __ldg(p.bn_in_gamma + tid); ld_b = __ldg(p.bn_in_beta + tid);
-            }
-            // A thread owns one 16-byte column of the (swizzled) tile rows tid/f4row + j*(256/f4row): its four
-            // channels within the K chunk are fixed, and so are the pixels of its rows.
-            const int f4row = p.kchunk >> 2;                    // 4 or 8 float4 per tile row
-            const int per = (int)(p.a_bytes >> 12);             // rows per thread: 2 or 4
-            const int row0 = tid / f4row, rstep = 256 / f4row;
-            const int cph = tid % f4row;
-            const int clog = p.kchunk == 32 ? (cph ^ (row0 & 7)) : (cph ^ ((row0 >> 1) & 3));
-            const bool three = p.passes == 3;
-            const bool writer = vb.y == 0;
-            const int stages = p.stages, nkc = p.n_kchunks, R = p.R, pad = p.pad;
-            // position of row r of the pixel box (the same for every tile)
-            int rw[4], rh[4], rn[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int r = row0 + j * rstep;
-                rw[j] = r % p.box_w; rh[j] = (r / p.box_w) % p.box_h; rn[j] = r / (p.box_w * p.box_h);
-            }
-            const int tap_b = kb / nkc, kc_b = kb - tap_b * nkc, ry_b = tap_b / R, sx_b = tap_b - ry_b * R;
-            if (p.bn_in != 2 && tid < C) { bn_par[0][tid] = ld_mu; bn_par[1][tid] = ld_rs; bn_par[2][tid] = ld_g; bn_par[3][tid] = ld_b; }
-            asm volatile("bar.sync 1, 256;" ::: "memory");
-            int it = 0, s = 0;
-            uint32_t par = 0;
-            for (int tj = 0; tj < my_tiles && ok; ++tj) {
-              HPF_TILE_ORIGIN(tile0 + tj);
-              int px[4], py[4], pn[4];
-#pragma unroll
-              for (int j = 0; j < 4; ++j) {
-                px[j] = q0 + rw[j]; py[j] = p0 + rh[j];
-                pn[j] = (j < per && rn[j] < p.box_n && n0 + rn[j] < p.N) ? n0 + rn[j] : -1;
-              }
-              int kc = kc_b, ry = ry_b, sx = sx_b;
-              for (int k = kb; k < ke; ++k, ++it) {
-                ok = mbar_wait(full0 + 8 * s, par, &abort_flag);
-                ok = __all_sync(0xffffffffu, ok);
-                if (!ok) { if (lane == 0) report(p.status, 7); break; }
-                if (it == 0 && tid == 0) HPF_TL(3);
-                const int dyy = ry - pad, dxx = sx - pad;
-                const int ch = kc * p.kchunk + 4 * clog;
-                const float4 mu = *reinterpret_cast<const float4*>(&bn_par[0][ch]);
-                const float4 rs = *reinterpret_cast<const float4*>(&bn_par[1][ch]);
-                const float4 g = *reinterpret_cast<const float4*>(&bn_par[2][ch]);
-                const float4 b = *reinterpret_cast<const float4*>(&bn_par[3][ch]);
-                float4* a = reinterpret_cast<float4*>(smem + s * p.stage_bytes);
-                float4* alo = reinterpret_cast<float4*>(smem + s * p.stage_bytes + off_alo);
-                float4 v[4];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) if (j < per) v[j] = a[tid + 256 * j];
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    if (j < per) {
-                        const int xx = px[j] + dxx, yy = py[j] + dyy;
-                        const bool inside = pn[j] >= 0 && (unsigned)xx < (unsigned)p.in_w && (unsigned)yy < (unsigned)p.in_h;
-                        float4 y;       // the padding ring is zero AFTER the activation
-                        y.x = inside ? fmaxf(fmaf(g.x, (v[j].x - mu.x) * rs.x, b.x), 0.f) : 0.f;
-                        y.y = inside ? fmaxf(fmaf(g.y, (v[j].y - mu.y) * rs.y, b.y), 0.f) : 0.f;
-                        y.z = inside ? fmaxf(fmaf(g.z, (v[j].z - mu.z) * rs.z, b.z), 0.f) : 0.f;
-                        y.w = inside ? fmaxf(fmaf(g.w, (v[j].w - mu.w) * rs.w, b.w), 0.f) : 0.f;
-                        if (writer && inside && dxx == 0 && dyy == 0)     // each pixel is some tile's centre tap exactly once
-                            *reinterpret_cast<float4*>(p.bn_in_y + (((size_t)pn[j] * p.in_h + yy) * p.in_w + xx) * C + ch) = y;
-                        if (three) {
-                            const float4 h = make_float4(tf32_hi(y.x), tf32_hi(y.y), tf32_hi(y.z), tf32_hi(y.w));
-                            a[tid + 256 * j] = h;
-                            alo[tid + 256 * j] = make_float4(y.x - h.x, y.y - h.y, y.z - h.z, y.w - h.w);
-                        } else {
-                            a[tid + 256 * j] = y;
-                        }
-                    }
-                fence_async_smem();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(split0 + 8 * s);
-                if (it == 0 && tid == 0) HPF_TL(4);
-                if (++kc == nkc) { kc = 0; if (++sx == R) { sx = 0; ++ry; } }
-                if (++s == stages) { s = 0; par ^= 1u; }
-              }
-            }
-        } else if (p.passes == 3) {
+if (p.passes == 3) {
             const int per = (int)(p.a_bytes >> 12);     // float4 per thread: a_bytes / 16 / 256 = 2 or 4
             const int all = my_tiles * (ke - kb);
             const int stages = p.stages;
@@ -570,7 +333,6 @@ __device__ __forceinline__ int conv_fwd_cta(const FwdParams* gpp, FwdScalars& p,
                 ok = mbar_wait(full0 + 8 * s, par, &abort_flag);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) { if (lane == 0) report(p.status, 7); break; }
-                if (it == 0 && tid == 0) HPF_TL(3);
                 float4* a = reinterpret_cast<float4*>(smem + s * p.stage_bytes);
                 float4* alo = reinterpret_cast<float4*>(smem + s * p.stage_bytes + off_alo);
                 float4 v[4];
@@ -587,7 +349,6 @@ __device__ __forceinline__ int conv_fwd_cta(const FwdParams* gpp, FwdScalars& p,
                 fence_async_smem();               // generic-proxy writes -> tensor-core reads
                 __syncwarp();
                 if (lane == 0) mbar_arrive(split0 + 8 * s);
-                if (it == 0 && tid == 0) HPF_TL(4);
                 if (++s == stages) { s = 0; par ^= 1u; }
             }
         }
@@ -596,11 +357,9 @@ __device__ __forceinline__ int conv_fwd_cta(const FwdParams* gpp, FwdScalars& p,
         // stores would touch 32 lines each).  With one tile per CTA the staging area is the pipeline itself, idle once
         // the accumulator is complete; with several tiles it is a region of its own, because the next tile's loads and
         // MMAs are in flight while this tile is written out.
-        __shared__ float4 shift_s[64];                 // per group of 4 output channels: the shift of the tile's statistics
         __shared__ int row_off[kTileM];                // offset (floats) of the pixel's channel row in the output, or -1
         __shared__ int row_fill[kTileM];               // strided data gradient: which neighbours of the sample exist
         float* const stg = reinterpret_cast<float*>(smem + stg_off);
-        bool all_done = true;
         for (int tj = 0; tj < my_tiles; ++tj) {
         HPF_TILE_ORIGIN(tile0 + tj);
         // the row tables do not depend on the accumulator: they are built while the MMAs still run
@@ -616,13 +375,11 @@ __device__ __forceinline__ int conv_fwd_cta(const FwdParams* gpp, FwdScalars& p,
             row_fill[tid] = (valid && p.zero_fill > 1 && p.zero_fill <= 4) ? fill : 0;
         }
         mbar_wait(accum_bar + 8 * tj, 0, &abort_flag);
-        if (!CELL && tj == 0 && p.pdl_late) pdl_launch_dependents();
+        if (tj == 0 && p.pdl_late) pdl_launch_dependents();
         asm volatile("bar.sync 1, 256;" ::: "memory");
         const bool done = abort_flag == 0;             // uniform over the 8 warps after the barrier
-        all_done = all_done && done;
         if (done) {
             tc_fence_after();
-            if (tid == 0 && tj == 0) HPF_TL(7);
             // TMEM lane = pixel within the tile.  Two warps share each group of 32 lanes (a warp reaches lanes
             // 32*(warp%4) ..): they take alternate groups of 16 output channels.
             const int row = (warp & 3) * 32 + lane;
@@ -644,9 +401,7 @@ __device__ __forceinline__ int conv_fwd_cta(const FwdParams* gpp, FwdScalars& p,
 #pragma unroll
                 for (int j = 0; j < 4; ++j) dst[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
             }
-            if (tid == 0 && tj == 0) HPF_TL(10);
             asm volatile("bar.sync 1, 256;" ::: "memory");
-            if (tid == 0 && tj == 0) HPF_TL(11);
             bool write_out = true;
             if (KSPLIT) {
                 // split K: the staged tile is this CTA's partial sum.  Store it; the CTA that takes the last ticket of this
@@ -654,20 +409,22 @@ __device__ __forceinline__ int conv_fwd_cta(const FwdParams* gpp, FwdScalars& p,
                 // is) and goes on to the write-out; the others are done.
                 __shared__ int last_of_unit;
                 const int c4n_ = p.n_chunk >> 2, tile_f4 = kTileM * c4n_;
-                const unsigned int unit = vb.x * vg.y + vb.y;
-                float4* mine = reinterpret_cast<float4*>(p.splitk_partials) + ((size_t)unit * p.ksplit + vb.z) * tile_f4;
+                const unsigned int unit = vb.x * gridDim.y + vb.y;
+                float* const sk_partials = reinterpret_cast<float*>(reinterpret_cast<char*>(p.splitk_partials) + micro * p.sk_ms);
+                unsigned int* const sk_ticket = reinterpret_cast<unsigned int*>(reinterpret_cast<char*>(p.splitk_ticket) + micro * p.sk_ms);
+                float4* mine = reinterpret_cast<float4*>(sk_partials) + ((size_t)unit * p.ksplit + vb.z) * tile_f4;
                 for (int idx = tid; idx < tile_f4; idx += 256) {
                     const int r = idx / c4n_, c4 = idx - r * c4n_;
                     mine[idx] = *reinterpret_cast<const float4*>(stg + (size_t)r * p.stg_pitch + 4 * c4);
                 }
                 __threadfence();
                 asm volatile("bar.sync 1, 256;" ::: "memory");
-                if (tid == 0) last_of_unit = atomicAdd(p.splitk_ticket + unit, 1u) == (unsigned int)p.ksplit - 1u;
+                if (tid == 0) last_of_unit = atomicAdd(sk_ticket + unit, 1u) == (unsigned int)p.ksplit - 1u;
                 asm volatile("bar.sync 1, 256;" ::: "memory");
                 write_out = last_of_unit != 0;
                 if (write_out) {
                     __threadfence();
-                    const float4* all = reinterpret_cast<const float4*>(p.splitk_partials) + (size_t)unit * p.ksplit * tile_f4;
+                    const float4* all = reinterpret_cast<const float4*>(sk_partials) + (size_t)unit * p.ksplit * tile_f4;
                     for (int idx = tid; idx < tile_f4; idx += 256) {
                         float4 a4 = __ldcg(all + idx);
                         for (int z = 1; z < p.ksplit; ++z) {
@@ -677,35 +434,21 @@ __device__ __forceinline__ int conv_fwd_cta(const FwdParams* gpp, FwdScalars& p,
                         const int r = idx / c4n_, c4 = idx - r * c4n_;
                         *reinterpret_cast<float4*>(stg + (size_t)r * p.stg_pitch + 4 * c4) = a4;
                     }
-                    if (tid == 0) p.splitk_ticket[unit] = 0u;
+                    if (tid == 0) sk_ticket[unit] = 0u;
                     asm volatile("bar.sync 1, 256;" ::: "memory");
                 }
             }
-            float4 sa = make_float4(0.f, 0.f, 0.f, 0.f), sb = sa, sk = sa;
             if (write_out) {
             // write-out: consecutive threads write consecutive float4 of a pixel's channel row.  Eight warps cannot
             // hide latency by occupancy, so four independent float4 are in flight per thread and nothing is re-read.
             const int c4n = p.n_chunk >> 2;
             const int total4 = kTileM * c4n;
             const int sh = (c4n & (c4n - 1)) == 0 ? 31 - __clz(c4n) : -1;
-            const float* extra = p.extra;
-            float* outp = p.out;
+            const float* extra = p.extra ? p.extra + micro * p.out_ms : nullptr;
+            float* outp = p.out + micro * p.out_ms;
             const bool accumulate = p.accumulate != 0;
             const unsigned int pitch = p.stg_pitch;
             const long long dense_h = p.dense_h, dense_w = p.dense_w;
-            const int stat_mode = p.stat_mode;
-            if (stat_mode) {
-                // The statistics are accumulated as deviations from the tile's first pixel (what the kernel stores for it,
-                // so residual included): sums of x and x*x themselves would cancel catastrophically in var = E[x^2] - mean^2
-                // for a channel whose mean is large compared with its spread.  A thread keeps one group of 4 channels
-                // throughout (256 is a multiple of c4n), so one shift per thread does.
-                const int c4k = tid % c4n;
-                sk = *reinterpret_cast<const float4*>(stg + 4 * c4k);
-                if (extra) { const float4 e = __ldcg(reinterpret_cast<const float4*>(extra + row_off[0] + 4 * c4k)); sk.x += e.x; sk.y += e.y; sk.z += e.z; sk.w += e.w; }
-                if (accumulate) { const float4 e = *reinterpret_cast<const float4*>(outp + row_off[0] + 4 * c4k); sk.x += e.x; sk.y += e.y; sk.z += e.z; sk.w += e.w; }
-                if (tid < c4n) shift_s[tid] = sk;          // read again when the tile's moments are formed
-            }
-            if (tid == 0 && tj == 0) HPF_TL(12);
             for (int base = tid; base < total4; base += 1024) {
                 float4 o[4];
                 int off[4];
@@ -740,12 +483,6 @@ __device__ __forceinline__ int conv_fwd_cta(const FwdParams* gpp, FwdScalars& p,
                     if (off[u] < 0) continue;
                     float* optr = outp + off[u];
                     *reinterpret_cast<float4*>(optr) = o[u];
-                    if (stat_mode) {
-                        const float dx_ = o[u].x - sk.x, dy_ = o[u].y - sk.y, dz_ = o[u].z - sk.z, dw_ = o[u].w - sk.w;
-                        sa.x += dx_; sa.y += dy_; sa.z += dz_; sa.w += dw_;
-                        sb.x = fmaf(dx_, dx_, sb.x); sb.y = fmaf(dy_, dy_, sb.y);
-                        sb.z = fmaf(dz_, dz_, sb.z); sb.w = fmaf(dw_, dw_, sb.w);
-                    }
                     if (fill[u]) {
                         // strided data gradient: the positions between the samples receive no contribution
                         const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -756,88 +493,11 @@ __device__ __forceinline__ int conv_fwd_cta(const FwdParams* gpp, FwdScalars& p,
                 }
             }
             }   // write_out
-            if (tid == 0 && tj == 0) HPF_TL(13);
-            if (p.stat_mode) {
-                const int c4n = p.n_chunk >> 2;
-                const int stat_mode = p.stat_mode;
-                // a thread kept one group of 4 channels throughout (256 is a multiple of c4n): add the 256 / c4n
-                // threads of each group in ascending order and store this tile's partial sums
-                asm volatile("bar.sync 1, 256;" ::: "memory");          // the staging area is free again
-                float4* red = reinterpret_cast<float4*>(stg);
-                int n_rows = 256;                                       // rows of `red` per group stride c4n
-                if (c4n <= 16) {
-                    // the 32 / c4n threads of a group inside a warp first: a fixed butterfly, then one row per warp
-                    for (int off = 16; off >= c4n; off >>= 1) {
-                        sa.x += __shfl_xor_sync(0xffffffffu, sa.x, off); sa.y += __shfl_xor_sync(0xffffffffu, sa.y, off);
-                        sa.z += __shfl_xor_sync(0xffffffffu, sa.z, off); sa.w += __shfl_xor_sync(0xffffffffu, sa.w, off);
-                        sb.x += __shfl_xor_sync(0xffffffffu, sb.x, off); sb.y += __shfl_xor_sync(0xffffffffu, sb.y, off);
-                        sb.z += __shfl_xor_sync(0xffffffffu, sb.z, off); sb.w += __shfl_xor_sync(0xffffffffu, sb.w, off);
-                    }
-                    if (lane < c4n) { const int r = (tid >> 5) * c4n + lane; red[2 * r] = sa; red[2 * r + 1] = sb; }
-                    n_rows = 8 * c4n;
-                } else {
-                    red[2 * tid] = sa; red[2 * tid + 1] = sb;
-                }
-                asm volatile("bar.sync 1, 256;" ::: "memory");
-                if (tid == 0 && tj == 0) HPF_TL(14);
-                if (tid < ((c4n * 2 + 31) & ~31)) {          // whole warps: the swap below is a warp shuffle
-                    // threads 2g and 2g+1 add group g's rows of shifted sums and of shifted squares, swap the totals, and store
-                    // the tile's mean (from the sums and the group's shift, which thread g keeps: fetched through shared memory)
-                    // and the sum of squared deviations from it
-                    const int g = tid >> 1, which = tid & 1;
-                    const bool mine = tid < c4n * 2;
-                    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {                       // n_rows / c4n <= 8
-                        const int t2 = g + j * c4n;
-                        if (mine && t2 < n_rows) { const float4 v2 = red[2 * t2 + which]; acc.x += v2.x; acc.y += v2.y; acc.z += v2.z; acc.w += v2.w; }
-                    }
-                    float4 oth;
-                    oth.x = __shfl_xor_sync(0xffffffffu, acc.x, 1); oth.y = __shfl_xor_sync(0xffffffffu, acc.y, 1);
-                    oth.z = __shfl_xor_sync(0xffffffffu, acc.z, 1); oth.w = __shfl_xor_sync(0xffffffffu, acc.w, 1);
-                    const float4 s1 = which ? oth : acc, s2 = which ? acc : oth;
-                    const float4 kg = shift_s[mine ? g : 0];
-                    const float inv_n = p.stat_inv_tile_rows;       // every tile of a fused launch is full
-                    float4 r;
-                    if (which == 0) r = make_float4(kg.x + s1.x * inv_n, kg.y + s1.y * inv_n, kg.z + s1.z * inv_n, kg.w + s1.w * inv_n);
-                    else r = make_float4(s2.x - s1.x * s1.x * inv_n, s2.y - s1.y * s1.y * inv_n, s2.z - s1.z * s1.z * inv_n, s2.w - s1.w * s1.w * inv_n);
-                    if (mine) {
-                        float* dstp = p.stat_partials + ((size_t)(tile0 + tj) * 2 + which) * p.c_out + co0 + 4 * g;
-                        *reinterpret_cast<float4*>(dstp) = r;
-                        if (stat_mode == 1) __threadfence();
-                    }
-                }
-            }
         }
         if (MULTI) asm volatile("bar.sync 1, 256;" ::: "memory");      // the staging area and the row tables serve the next tile
         }   // tiles of this CTA
-        {
-            const int stat_mode = p.stat_mode;
-            if (stat_mode && all_done) {
-                // stat_mode 1: the CTA that finishes last turns the per-tile sums into mean and 1/sigma (tiles are added in
-                // a fixed order in fp64, so the result does not depend on which CTA that is).  stat_mode 3: the reading
-                // convolution adds the few per-tile sums itself, and this kernel ends without a ticket.
-                __shared__ int is_last;
-                if (stat_mode == 1) asm volatile("bar.sync 1, 256;" ::: "memory");
-                if (stat_mode == 1 && tid == 0) {
-                    const unsigned int done_before = atomicAdd(p.stat_ticket, 1u);
-                    is_last = done_before == vg.x * vg.y - 1;
-                }
-                if (stat_mode == 1) asm volatile("bar.sync 1, 256;" ::: "memory");
-                if (stat_mode == 1 && is_last) {
-                    __threadfence();
-                    float mu = 0.f, rs = 0.f;
-                    // every tile is written out and the pipeline buffers are idle: they hold the reduction
-                    bn_combine_partials(p.stat_partials, p.n_tiles, p.c_out, p.stat_inv_rows, p.stat_eps,
-                                        reinterpret_cast<float (*)[32][8]>(smem), tid, &mu, &rs);
-                    if (tid < p.c_out) { p.stat_out[tid] = mu; p.stat_out[p.c_out + tid] = rs; }
-                    if (tid == 0) *p.stat_ticket = 0u;
-                }
-            }
-        }
     }
 
-    if (threadIdx.x == 64) HPF_TL(8);
     // ---- teardown ----
     tc_fence_before();
     __syncthreads();
@@ -850,138 +510,7 @@ __device__ __forceinline__ int conv_fwd_cta(const FwdParams* gpp, FwdScalars& p,
         }
     }
     __syncthreads();
-    if (!CELL && warp == 0) tmem_dealloc(tmem_base, p.tmem_cols);
-    if (threadIdx.x == 0) HPF_TL(9);
-#if defined(HPF_TC_TIMELINE) && HPF_TC_TIMELINE == 2
-    __syncthreads();
-    if (threadIdx.x < 16) {
-        const int tiles = vg.x;
-        const int cls = (p.R == 3 ? 1 : 0) + 2 * (tiles >= 128 ? 0 : (tiles >= 32 ? 1 : 2)) + (p.bn_in ? 0 : 0);
-        if (threadIdx.x == 0) atomicAdd(&g_tl_acc[cls][0], 1ull);
-        else if (tl_s[threadIdx.x] > tl_s[0]) atomicAdd(&g_tl_acc[cls][threadIdx.x], tl_s[threadIdx.x] - tl_s[0]);
-    }
-#endif
-    return abort_flag;          // uniform: nobody writes it between the barrier above and the next call's set-up
-}
-
-template <bool MULTI, bool KSPLIT = false>
-__global__ void __launch_bounds__(320, 2) conv_tc_fwd_kernel(const __grid_constant__ FwdParams gp)
-{
-    __shared__ FwdScalars p;                 // scalar parameters, see load_scalars
-    // Programmatic launch: the next kernel of the stream may be scheduled once every CTA of this one has said so.  Early (here):
-    // the successor's set-up hides under this kernel, which shortens a lone stage's chain of kernels.  Late (when the first
-    // accumulator is complete, see below): the successor's CTAs do not sit in SM slots for the whole life of this kernel,
-    // which is what counts when every stage is busy and slots are what the stages compete for.  The host chooses per launch.
-    if (!gp.s.pdl_late) pdl_launch_dependents();
-    load_scalars(&p, &gp.s);
-    __syncthreads();
-    conv_fwd_cta<MULTI ? 1 : (KSPLIT ? 2 : 0)>(&gp, p, make_uint3(blockIdx.x, blockIdx.y, blockIdx.z), make_uint3(gridDim.x, gridDim.y, gridDim.z), 0u, true);
-}
-
-// ------------------------------------------------------------------------------------------------
-// persistent cell kernel: the forward convolutions of one (partition, micro-batch) cell in ONE resident grid
-// ------------------------------------------------------------------------------------------------
-// A cell of the pipeline is a chain of a hundred and more small dependent convolutions.  As separate launches each pays
-// the launch-to-launch latency, and eight stages' worth of them compete for SM slots in which their CTAs mostly wait.
-// Here a fixed, small grid stays resident for the whole cell and walks the list of launches: the CTAs share out the
-// CTAs of each launch (virtual CTAs: block index and grid size of the stand-alone launch), run them with the same code,
-// and meet at a grid-wide barrier before the next launch, whose input the whole grid has just produced.  Every CTA of
-// the grid must be resident at the same time; the host sizes the grids so that all cells that can run concurrently fit
-// the GPU together.  The barrier wait is bounded like every other wait here.
-struct alignas(64) CellOp {
-    FwdParams p;                 // exactly what the stand-alone launch would receive
-    unsigned int gx, gy, gz;     // its grid
-    unsigned int reserved;
-};
-struct CellParams {
-    const CellOp* ops;           // device memory, written before the launch and read-only for the kernel
-    int n_ops;
-    unsigned int* barrier;       // {arrivals, generation}: zero before the first use, left with arrivals at zero
-    DeviceStatus* status;
-    unsigned int tmem_cols;      // the largest accumulator of the list
-};
-
-__device__ __forceinline__ unsigned int ld_acquire_gpu(const unsigned int* ptr)
-{
-    unsigned int v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(ptr) : "memory");
-    return v;
-}
-__device__ __forceinline__ void st_release_gpu(unsigned int* ptr, unsigned int v)
-{
-    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(ptr), "r"(v) : "memory");
-}
-
-// All CTAs of the grid arrive; the last one opens the next generation.  What the CTAs wrote before the barrier is
-// visible to all of them after it, also to copies issued through the async proxy (TMA).  Returns false when the wait ran
-// out or another kernel already reported a failure.
-__device__ __forceinline__ bool cell_grid_barrier(unsigned int* bar, DeviceStatus* status, int* stop_flag)
-{
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        const unsigned int gen = ld_acquire_gpu(bar + 1);      // cannot advance before this CTA has arrived
-        __threadfence();
-        int stop = 0;
-        if (atomicAdd(bar, 1u) == gridDim.x - 1) {
-            bar[0] = 0u;
-            __threadfence();
-            st_release_gpu(bar + 1, gen + 1u);
-        } else {
-            const long long t0 = clock64();
-            int polls = 0;
-            while (ld_acquire_gpu(bar + 1) == gen) {
-                if ((++polls & 63) == 0 && (clock64() - t0 > kWaitLimit || ld_acquire_gpu(&status->code) != 0u)) { report(status, 9); stop = 1; break; }
-            }
-        }
-        *stop_flag = stop;
-    }
-    __syncthreads();
-    asm volatile("fence.proxy.async;" ::: "memory");
-    return *stop_flag == 0;
-}
-
-__global__ void __launch_bounds__(320, 2) conv_tc_cell_kernel(const __grid_constant__ CellParams cp)
-{
-    __shared__ FwdScalars p;
-    __shared__ unsigned int vgrid[4];
-    __shared__ uint32_t cell_tmem;
-    __shared__ int cell_stop;
-    constexpr int kWords = (int)(sizeof(FwdScalars) / 4);
-    static_assert(sizeof(FwdScalars) % 4 == 0 && kWords + 3 <= 320, "one parameter word per thread");
-    const int tid = threadIdx.x;
-    if ((tid >> 5) == 0) tmem_alloc(smem_u32(&cell_tmem), cp.tmem_cols);
-    if (tid == 0) cell_stop = 0;
-    // one word of the parameters per thread: the first launch's now, the next one's while the current one runs
-    auto fetch = [&](int op) -> uint32_t {
-        const CellOp* o = cp.ops + op;
-        if (tid < kWords) return __ldg(reinterpret_cast<const uint32_t*>(&o->p.s) + tid);
-        if (tid < kWords + 3) return __ldg(&o->gx + (tid - kWords));
-        return 0u;
-    };
-    uint32_t nxt = fetch(0);
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem_base = cell_tmem;
-    bool first = true;
-    int stop = 0;
-    for (int op = 0; op < cp.n_ops && !stop; ++op) {
-        if (tid < kWords) reinterpret_cast<uint32_t*>(&p)[tid] = nxt;
-        else if (tid < kWords + 3) vgrid[tid - kWords] = nxt;
-        if (op + 1 < cp.n_ops) nxt = fetch(op + 1);
-        __syncthreads();
-        const unsigned int gx = vgrid[0], gy = vgrid[1], gz = vgrid[2], V = gx * gy * gz;
-        for (unsigned int v = blockIdx.x; v < V && !stop; v += gridDim.x) {
-            const uint3 vb = make_uint3(v % gx, (v / gx) % gy, v / (gx * gy));
-            stop = conv_fwd_cta<3>(&cp.ops[op].p, p, vb, make_uint3(gx, gy, gz), tmem_base, first);
-            first = false;
-        }
-        if (stop) break;
-        if (op + 1 < cp.n_ops && !cell_grid_barrier(cp.barrier, cp.status, &cell_stop)) stop = 1;
-    }
-    tc_fence_before();
-    __syncthreads();
-    if ((tid >> 5) == 0) tmem_dealloc(tmem_base, cp.tmem_cols);
+    if (warp == 0) tmem_dealloc(tmem_base, p.tmem_cols);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1821,36 +1350,6 @@ bool conv_tc_supported(const ConvShape& s, int pass)
     return choose_box(v.Q, v.P, v.N, kTileM, 1, &b);
 }
 
-int conv_tc_tiles(const ConvShape& s, int pass)
-{
-    FwdView v;
-    PixelBox b;
-    if (pass == PASS_WGRAD || !fwd_view(s, pass, &v) || !choose_box(v.Q, v.P, v.N, kTileM, 1, &b)) return 0;
-    return ((v.Q + b.w - 1) / b.w) * ((v.P + b.h - 1) / b.h) * ((v.N + b.n - 1) / b.n);
-}
-
-bool conv_tc_can_fuse_bn(const ConvShape& s, int pass)
-{
-    FwdView v;
-    if (pass == PASS_WGRAD || !fwd_view(s, pass, &v)) return false;
-    // the write-out keeps one group of 4 channels per thread and the last CTA combines 2*C columns with 256 threads:
-    // a power of two between 16 and 256 channels, all in one channel slice
-    const int C = v.c_out;
-    if (!(C >= 16 && C <= 256 && (C & (C - 1)) == 0 && conv_tc_tiles(s, pass) > 0)) return false;
-    // the per-tile moments are merged as equal-sized groups: every tile must be full
-    PixelBox b;
-    if (!choose_box(v.Q, v.P, v.N, kTileM, 1, &b)) return false;
-    return v.Q % b.w == 0 && v.P % b.h == 0 && v.N % b.n == 0;
-}
-
-bool conv_tc_can_fuse_bn_input(const ConvShape& s)
-{
-    FwdView v;
-    if (!fwd_view(s, PASS_FWD, &v) || s.stride != 1) return false;
-    const int C = s.C;
-    return C >= 16 && C <= 256 && (C & (C - 1)) == 0 && conv_tc_tiles(s, PASS_FWD) > 0;
-}
-
 cudaError_t conv_tc_init()
 {
     if (g_encode) return cudaSuccess;
@@ -1859,13 +1358,11 @@ cudaError_t conv_tc_init()
     cudaError_t e = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &q);
     if (e != cudaSuccess) return e;
     if (q != cudaDriverEntryPointSuccess || !fn) return cudaErrorNotSupported;
-    e = cudaFuncSetAttribute(conv_tc_fwd_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget + 2048);
+    e = cudaFuncSetAttribute(conv_tc_fwd_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget + 2048);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(conv_tc_fwd_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget + 2048);
+    e = cudaFuncSetAttribute(conv_tc_fwd_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget + 2048);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(conv_tc_fwd_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget + 2048);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(conv_tc_cell_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget + 2048);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(conv_tc_wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWgradSmemBudget + 2048);
     if (e != cudaSuccess) return e;
@@ -1943,14 +1440,14 @@ static_assert(sizeof(ConvTcFwdLaunch) <= sizeof(((ConvTcPlan*)0)->storage) && si
 
 cudaError_t conv_tc_prepare(ConvTcPlan* plan, const ConvShape& s, int pass, int passes, const float* in, const float* in2,
                             const float* w_hi, const float* w_lo, float* out, const float* extra, bool accumulate, void* scratch,
-                            const ConvBnFuse* fuse)
+                            const ConvTcHints* hints)
 {
     plan->valid = 0; plan->s = s; plan->pass = pass; plan->direct = 0;
-    const int M = fuse && fuse->micro_batches > 1 ? fuse->micro_batches : 1;
-    const long long dw_ms = fuse ? fuse->slot_stride : 0;
+    const int M = hints && hints->micro_batches > 1 ? hints->micro_batches : 1;
+    const long long dw_ms = hints ? hints->slot_stride : 0;
     if (passes != 1 && passes != 3) return cudaErrorInvalidValue;
     WgradDirectGeom dg;
-    if (pass == PASS_WGRAD && !(fuse && fuse->wgrad_transposing) && wgrad_direct_geom(s, passes, &dg, M)) {
+    if (pass == PASS_WGRAD && !(hints && hints->wgrad_transposing) && wgrad_direct_geom(s, passes, &dg, M)) {
         ConvTcWgradDirectLaunch* L = reinterpret_cast<ConvTcWgradDirectLaunch*>(plan->storage);
         WgradDirectParams& P = L->p;
         memset(&P, 0, sizeof P);
@@ -1986,7 +1483,7 @@ cudaError_t conv_tc_prepare(ConvTcPlan* plan, const ConvShape& s, int pass, int 
         p.taps_per_mma = 256 / slot < dg.taps_per_cta ? 256 / slot : dg.taps_per_cta;
         p.idesc = instr_desc(slot * p.taps_per_mma, true, true);
         p.idesc_tail = instr_desc(slot * (dg.taps_per_cta % p.taps_per_mma ? dg.taps_per_cta % p.taps_per_mma : p.taps_per_mma), true, true);
-        p.split_stride = n_out; p.splits = dg.splits; p.out_ms = dg.splits > 1 ? (fuse && fuse->partial_stride ? fuse->partial_stride : n_out * dg.splits) : dw_ms; L->dw_ms = dw_ms;
+        p.split_stride = n_out; p.splits = dg.splits; p.out_ms = dg.splits > 1 ? (hints && hints->partial_stride ? hints->partial_stride : n_out * dg.splits) : dw_ms; L->dw_ms = dw_ms;
         L->grid = dim3(dg.splits, dg.tap_groups, (s.K / dg.m_chunk) * (s.C / dg.n_cols));
         L->smem = (unsigned int)dg.stages * dg.stage_bytes + dg.slack + 1024;
         L->splits = dg.splits; L->dw = out; L->n_out = n_out;
@@ -2033,7 +1530,7 @@ cudaError_t conv_tc_prepare(ConvTcPlan* plan, const ConvShape& s, int pass, int 
         p.taps_per_mma = 256 / g.n_cols < g.taps_per_cta ? 256 / g.n_cols : g.taps_per_cta;
         p.idesc = instr_desc(g.n_cols * p.taps_per_mma, false, false);
         p.idesc_tail = instr_desc(g.n_cols * (g.taps_per_cta % p.taps_per_mma ? g.taps_per_cta % p.taps_per_mma : p.taps_per_mma), false, false);
-        p.split_stride = n_out; p.splits = g.splits; p.out_ms = g.splits > 1 ? (fuse && fuse->partial_stride ? fuse->partial_stride : n_out * g.splits) : dw_ms; L->dw_ms = dw_ms;
+        p.split_stride = n_out; p.splits = g.splits; p.out_ms = g.splits > 1 ? (hints && hints->partial_stride ? hints->partial_stride : n_out * g.splits) : dw_ms; L->dw_ms = dw_ms;
         L->grid = dim3(g.splits, g.tap_groups, (s.K / g.m_chunk) * (s.C / g.n_cols));
         L->smem = (unsigned int)g.raw_stages * g.raw_bytes + (unsigned int)g.t_stages * g.t_bytes + (g.m_chunk < 128 ? kWgradSlack : 0u) + 1024;
         L->splits = g.splits; L->dw = out; L->n_out = n_out;
@@ -2051,15 +1548,12 @@ cudaError_t conv_tc_prepare(ConvTcPlan* plan, const ConvShape& s, int pass, int 
     int n_chunk = v.c_out < 256 ? v.c_out : 256;
     {
         // A launch with few pixel tiles leaves most SMs idle: twice as many channel slices of 128 (two MMAs of the stacked
-        // width per K step instead of three) fill them.  When BN work rides in the kernel every slice repeats the BN on its
-        // copy of the activation tile, which only pays when the K loop is long (the wide convolutions of the ImageNet layout).
+        // width per K step instead of three) fill them.
         const int tiles = ((v.Q + b.w - 1) / b.w) * ((v.P + b.h - 1) / b.h) * ((v.N + b.n - 1) / b.n);
-        const bool fused = fuse && (fuse->mode || fuse->in_mode);
-        const int ksteps = v.R * v.R * v.c_in / 8;
-        if ((!fused || ksteps >= 64) && v.c_out % 256 == 0 && tiles * (v.c_out / 256) <= 74) n_chunk = 128;
+        if (v.c_out % 256 == 0 && tiles * (v.c_out / 256) <= 74) n_chunk = 128;
     }
     {
-        cuuint64_t dims[4] = {(cuuint64_t)v.c_in, (cuuint64_t)v.in_w, (cuuint64_t)v.in_h, (cuuint64_t)v.N};
+        cuuint64_t dims[4] = {(cuuint64_t)v.c_in, (cuuint64_t)v.in_w, (cuuint64_t)v.in_h, (cuuint64_t)v.N * M};
         cuuint64_t str[3] = {(cuuint64_t)v.in_sw * 4, (cuuint64_t)v.in_sh * 4, (cuuint64_t)v.in_sn * 4};
         cuuint32_t box[4] = {(cuuint32_t)kchunk, (cuuint32_t)b.w, (cuuint32_t)b.h, (cuuint32_t)b.n};
         cudaError_t e = encode(&P.tm_a, in, 4, dims, str, box, kchunk * 4);
@@ -2098,28 +1592,7 @@ cudaError_t conv_tc_prepare(ConvTcPlan* plan, const ConvShape& s, int pass, int 
     // one more where two CTAs still fit an SM: nine taps then take two rounds of the ring instead of three
     if (total > kFwdMaxStages && (unsigned int)(kFwdMaxStages + 1) * p.stage_bytes <= 92u * 1024u) stages = kFwdMaxStages + 1;
     if (stages > total) stages = total;
-    const int cell_ctas = fuse ? fuse->cell_ctas : 0;
-    const unsigned int cell_budget = cell_ctas > 0 ? (fuse->cell_smem ? fuse->cell_smem : kCellSmemBudget) : 0u;
-    if (cell_ctas > 0)
-        while (stages > 1 && (unsigned int)stages * p.stage_bytes > cell_budget) --stages;
     p.stages = stages;
-    if (fuse && fuse->mode) {
-        if (256 % (n_chunk / 4)) return cudaErrorNotSupported;
-        if ((fuse->mode != 1 && fuse->mode != 3) || pass != PASS_FWD || !conv_tc_can_fuse_bn(s, pass) || fuse->rows < 1) return cudaErrorNotSupported;
-        p.stat_mode = fuse->mode; p.stat_partials = fuse->partials;
-        p.stat_ticket = fuse->ticket; p.stat_out = fuse->stats_out; p.stat_eps = fuse->eps; p.stat_inv_rows = 1.0 / (double)fuse->rows;
-        p.stat_inv_tile_rows = 1.0f / (float)b.rows;
-    }
-    if (fuse && fuse->in_mode) {
-        if (pass != PASS_FWD || !conv_tc_can_fuse_bn_input(s)) return cudaErrorNotSupported;
-        if (fuse->in_mode != 1 && fuse->in_mode != 2) return cudaErrorInvalidValue;
-        if (fuse->in_mode == 2 && (fuse->in_tiles < 1 || fuse->in_rows < 1 || !fuse->in_partials)) return cudaErrorInvalidValue;
-        p.bn_in = fuse->in_mode; p.in_w = v.in_w; p.in_h = v.in_h;
-        p.bn_in_gamma = fuse->in_gamma; p.bn_in_beta = fuse->in_beta;
-        p.bn_in_stats = fuse->in_stats; p.bn_in_y = fuse->in_y;
-        p.bn_in_partials = fuse->in_partials; p.bn_in_stats_out = fuse->in_stats; p.bn_in_tiles = fuse->in_tiles;
-        p.bn_in_eps = fuse->in_eps; p.bn_in_inv_rows = fuse->in_rows > 0 ? 1.0 / (double)fuse->in_rows : 0.0;
-    }
     p.stacked = (passes == 3 && 2 * n_chunk <= 256) ? 1 : 0;
     p.acc_cols = (unsigned int)(p.stacked ? 2 * n_chunk : n_chunk);
     p.idesc = instr_desc(n_chunk, false, false);
@@ -2133,29 +1606,20 @@ cudaError_t conv_tc_prepare(ConvTcPlan* plan, const ConvShape& s, int pass, int 
     // the 512 columns of an SM) and a staging area beside the pipeline.  A launch of about a wave keeps one tile per
     // CTA: there the duration of the launch is one CTA's own chain.
     p.tiles_per_cta = 1;
-    if (cell_ctas > 0) {
-        // inside a persistent cell kernel of cell_ctas CTAs: as many tiles per CTA as bring the launch down to one round of
-        // the grid, within four accumulator barriers, the cell's tensor-memory columns and its shared memory
-        int t = (p.n_tiles * (v.c_out / n_chunk) + cell_ctas - 1) / cell_ctas;
-        if (t > 4) t = 4;
-        while (t > 1 && (unsigned int)t * p.acc_cols > kCellTmemCols) --t;
-        if (t > 1 && pipe_bytes + stg_bytes > cell_budget) t = 1;
-        p.tiles_per_cta = t < 1 ? 1 : t;
-    } else if (p.n_tiles * (v.c_out / n_chunk) >= kMultiTileFrom && 2 * p.acc_cols <= 256 && pipe_bytes + stg_bytes <= 110u * 1024u) {
+    if (p.n_tiles * (v.c_out / n_chunk) >= kMultiTileFrom && 2 * p.acc_cols <= 256 && pipe_bytes + stg_bytes <= 110u * 1024u) {
         int t = (p.n_tiles * (v.c_out / n_chunk) + 295) / 296;            // tiles per CTA that bring the launch down to one wave
         if (t > 4) t = 4;                                                 // accumulator barriers
         while (t > 2 && (unsigned int)t * p.acc_cols > 256u) --t;
         p.tiles_per_cta = t < 2 ? 2 : t;
     }
-    p.pdl_late = fuse && fuse->pdl_late ? 1 : 0;
     p.ksplit = 1;
-    if (fuse && fuse->splitk && !fuse->mode && !fuse->in_mode && p.tiles_per_cta == 1) {
+    if (hints && hints->splitk && p.tiles_per_cta == 1) {
         const int S = splitk_factor(p.n_tiles, v.c_out / n_chunk, total, kchunk / 8);
         const size_t need = kSplitKTicketBytes + (size_t)p.n_tiles * (v.c_out / n_chunk) * S * kTileM * n_chunk * sizeof(float);
-        if (S > 1 && need <= fuse->splitk_bytes) {
-            p.ksplit = S;
-            p.splitk_ticket = reinterpret_cast<unsigned int*>(fuse->splitk);
-            p.splitk_partials = reinterpret_cast<float*>(reinterpret_cast<char*>(fuse->splitk) + kSplitKTicketBytes);
+        if (S > 1 && need <= hints->splitk_bytes) {
+            p.ksplit = S; p.sk_ms = (long long)hints->splitk_bytes;
+            p.splitk_ticket = reinterpret_cast<unsigned int*>(hints->splitk);
+            p.splitk_partials = reinterpret_cast<float*>(reinterpret_cast<char*>(hints->splitk) + kSplitKTicketBytes);
             const int per_cta = total / S;                   // the shortest share of the K loop
             if (p.stages > per_cta) p.stages = per_cta < 1 ? 1 : per_cta;
         }
@@ -2165,12 +1629,12 @@ cudaError_t conv_tc_prepare(ConvTcPlan* plan, const ConvShape& s, int pass, int 
     L->grid = dim3((p.n_tiles + p.tiles_per_cta - 1) / p.tiles_per_cta, v.c_out / n_chunk, p.ksplit);
     L->smem = p.tiles_per_cta > 1 ? pipe_bytes + stg_bytes : (pipe_bytes > stg_bytes ? pipe_bytes : stg_bytes);
     L->smem += 1024;
-    if (p.stat_mode == 1 && L->smem < 8192u + 1024u) L->smem = 8192u + 1024u;      // the last CTA's reduction: 8 x 32 x 8 floats
+    p.ctas_per_m = (int)L->grid.x; p.out_ms = v.N * v.os_n;
     plan->valid = 1;
     return cudaSuccess;
 }
 
-cudaError_t conv_tc_launch(const ConvTcPlan* plan, DeviceStatus* status, cudaStream_t st, int64_t* n_launch, int m_first, int m_count)
+cudaError_t conv_tc_launch(const ConvTcPlan* plan, DeviceStatus* status, cudaStream_t st, int64_t* n_launch, int m_first, int m_count, bool pdl_late)
 {
     if (!plan->valid) return cudaErrorInvalidValue;
     if (plan->pass == PASS_WGRAD && plan->direct) {
@@ -2198,55 +1662,11 @@ cudaError_t conv_tc_launch(const ConvTcPlan* plan, DeviceStatus* status, cudaStr
         return cudaGetLastError();
     }
     ConvTcFwdLaunch L = *reinterpret_cast<const ConvTcFwdLaunch*>(plan->storage);
-    L.p.s.status = status;
-    if (L.p.s.ksplit > 1) launch_pdl(conv_tc_fwd_kernel<false, true>, L.grid, dim3(320), L.smem, st, L.p);
-    else if (L.p.s.tiles_per_cta > 1) launch_pdl(conv_tc_fwd_kernel<true>, L.grid, dim3(320), L.smem, st, L.p);
-    else launch_pdl(conv_tc_fwd_kernel<false>, L.grid, dim3(320), L.smem, st, L.p);
-    count(n_launch, 1);
-    return cudaGetLastError();
-}
-
-size_t conv_tc_cell_op_bytes() { return sizeof(CellOp); }
-
-cudaError_t conv_tc_cell_op(const ConvTcPlan* plan, DeviceStatus* status, void* dst_host, unsigned int* smem, unsigned int* tmem_cols,
-                            unsigned int* ctas)
-{
-    if (!plan->valid || plan->pass == PASS_WGRAD) return cudaErrorInvalidValue;
-    const ConvTcFwdLaunch* L = reinterpret_cast<const ConvTcFwdLaunch*>(plan->storage);
-    CellOp op;
-    memset(&op, 0, sizeof op);
-    op.p = L->p;
-    op.p.s.status = status;
-    op.gx = L->grid.x; op.gy = L->grid.y; op.gz = L->grid.z;
-    memcpy(dst_host, &op, sizeof op);
-    if (L->p.s.tmem_cols > kCellTmemCols) return cudaErrorNotSupported;
-    *smem = L->smem; *tmem_cols = L->p.s.tmem_cols; *ctas = L->grid.x * L->grid.y * L->grid.z;
-    return cudaSuccess;
-}
-
-void conv_tc_plan_pipeline(const ConvTcPlan* plan, int* stages, int* k_iterations)
-{
-    const ConvTcFwdLaunch* L = reinterpret_cast<const ConvTcFwdLaunch*>(plan->storage);
-    *stages = L->p.s.stages; *k_iterations = L->p.s.R * L->p.s.R * L->p.s.n_kchunks;
-}
-
-int conv_tc_cell_max_ctas(unsigned int smem)
-{
-    int dev = 0, sms = 0, per_sm = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, conv_tc_cell_kernel, 320, smem) != cudaSuccess) { (void)cudaGetLastError(); return 0; }
-    if (per_sm > 2) per_sm = 2;          // two cell CTAs hold an SM's 512 tensor-memory columns between them
-    return per_sm * sms;
-}
-
-cudaError_t conv_tc_cell_launch(const void* d_ops, int n_ops, int ctas, unsigned int smem, unsigned int tmem_cols, unsigned int* d_barrier,
-                                DeviceStatus* status, cudaStream_t st, int64_t* n_launch)
-{
-    if (n_ops < 1 || ctas < 1 || tmem_cols < 32 || tmem_cols > kCellTmemCols) return cudaErrorInvalidValue;
-    CellParams cp;
-    cp.ops = reinterpret_cast<const CellOp*>(d_ops); cp.n_ops = n_ops; cp.barrier = d_barrier; cp.status = status; cp.tmem_cols = tmem_cols;
-    // a plain stream-ordered launch: a resident grid that started early would only hold SM slots while it waits
-    conv_tc_cell_kernel<<<dim3(ctas), dim3(320), smem, st>>>(cp);
+    L.p.s.status = status; L.p.s.pdl_late = pdl_late ? 1 : 0;
+    const dim3 grid(L.grid.x * m_count, L.grid.y, L.grid.z);
+    if (L.p.s.ksplit > 1) launch_pdl(conv_tc_fwd_kernel<false, true>, grid, dim3(320), L.smem, st, L.p, m_first);
+    else if (L.p.s.tiles_per_cta > 1) launch_pdl(conv_tc_fwd_kernel<true, false>, grid, dim3(320), L.smem, st, L.p, m_first);
+    else launch_pdl(conv_tc_fwd_kernel<false, false>, grid, dim3(320), L.smem, st, L.p, m_first);
     count(n_launch, 1);
     return cudaGetLastError();
 }
@@ -2277,16 +1697,3 @@ cudaError_t conv_weight_prep_single(const float* w, float* w_hi, float* w_lo, fl
 }
 
 }  // namespace hpf
-
-#if defined(HPF_TC_TIMELINE) && HPF_TC_TIMELINE == 2
-extern "C" int hpf_debug_timeline(unsigned long long* h_out, int reset)
-{
-    cudaDeviceSynchronize();
-    if (h_out && cudaMemcpyFromSymbol(h_out, hpf::g_tl_acc, sizeof(unsigned long long) * 8 * 16) != cudaSuccess) return -1;
-    if (reset) {
-        static unsigned long long zeros[8 * 16];
-        if (cudaMemcpyToSymbol(hpf::g_tl_acc, zeros, sizeof zeros) != cudaSuccess) return -1;
-    }
-    return 0;
-}
-#endif

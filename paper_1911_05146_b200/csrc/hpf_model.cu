@@ -93,6 +93,14 @@ struct hpf_model {
     std::vector<int> conv_fwd_bn;              // the inverse map
     std::vector<int> bn_into, conv_in_bn;      // BN -> the convolution that applies it to its own input operand (no BN kernel), and the inverse
     std::vector<size_t> bn_moments_off;        // BN -> per-unit moments of its input left by the producing convolution, all micro-batches
+    // Forward / data-gradient launches of networks with batch norm are the pipelined kernel's wherever it covers the shape.
+    // Without batch norm nothing re-scales the activations: the last bits of a convolution's sum move ReLU and max-pool
+    // decisions and, over a few updates, the whole trajectory (1-2 % of VGG-16's gradient after two steps, for sums that differ
+    // by 3e-6).  Such networks keep the tile kernel's order of summation; on their wide, small maps (256 channels and more on
+    // 8 x 8 and less, where a padded grid of positions wastes a quarter and more of the MMA rows) it is no slower.
+    bool has_bn = false;
+    std::vector<char> use_pipe[2];
+    std::vector<ConvTcPlan> tile_plan[2];      // conv -> its launch on the tile kernel
     std::vector<ConvPipeGeom> pipe_geom[2];    // conv -> split of its forward / data-gradient launches
     bool opt_pdl = true;       // programmatic dependent launch for this model's kernels
     bool opt_bn_cluster = true; // BN backward of micro-batch sized tensors as one thread-block-cluster launch
@@ -416,7 +424,9 @@ int passes_of(const hpf_model* mdl) { return mdl->opt_conv_path == 2 ? 1 : 3; }
 void build_kernel_plan(hpf_model* mdl)
 {
     const int n = mdl->n_ops;
-    for (int pass = 0; pass < 2; ++pass) mdl->pipe_geom[pass].assign(n, ConvPipeGeom());
+    mdl->has_bn = false;
+    for (const OpInfo& o : mdl->ops) mdl->has_bn = mdl->has_bn || o.op.kind == HPF_OP_BN || o.op.kind == HPF_OP_BNRELU;
+    for (int pass = 0; pass < 2; ++pass) { mdl->pipe_geom[pass].assign(n, ConvPipeGeom()); mdl->use_pipe[pass].assign(n, 0); }
     for (int pass = 0; pass < 3; ++pass) {
         mdl->use_tc[pass].assign(n, 0);
         for (int i = 0; i < n; ++i) mdl->use_tc[pass][i] = op_uses_tc(mdl, i, pass) ? 1 : 0;
@@ -432,7 +442,7 @@ void build_kernel_plan(hpf_model* mdl)
         int t = bn.op.src0, prod = -1;
         if (mdl->ops[t].op.kind == HPF_OP_CONV && mdl->fused_into[t] < 0) prod = t;
         else if (mdl->ops[t].op.kind == HPF_OP_ADD && mdl->add_done_by[t] >= 0) prod = mdl->add_done_by[t];
-        if (prod < 0 || !mdl->use_tc[PASS_FWD][prod] || mdl->ops[prod].part != bn.part || mdl->conv_fwd_bn[prod] >= 0 ||
+        if (prod < 0 || !mdl->use_pipe[PASS_FWD][prod] || mdl->ops[prod].part != bn.part || mdl->conv_fwd_bn[prod] >= 0 ||
             !conv_pipe_can_fuse_bn_output(mdl->pipe_geom[PASS_FWD][prod])) continue;
         bool adjacent = true;
         for (int k = prod + 1; k < j; ++k)
@@ -442,7 +452,7 @@ void build_kernel_plan(hpf_model* mdl)
         // the BN+ReLU itself: applied by its only reader, the next op, a stride-1 tensor-core convolution
         if ((mdl->opt_fuse_bn & 2) && bn.consumers.size() == 1 && bn.consumers[0] == j + 1) {
             const int i = j + 1;
-            if (mdl->ops[i].op.kind == HPF_OP_CONV && mdl->ops[i].op.src0 == j && mdl->use_tc[PASS_FWD][i] && mdl->ops[i].part == bn.part &&
+            if (mdl->ops[i].op.kind == HPF_OP_CONV && mdl->ops[i].op.src0 == j && mdl->use_pipe[PASS_FWD][i] && mdl->ops[i].part == bn.part &&
                 conv_pipe_can_fuse_bn_input(conv_shape_of(mdl, i))) {
                 mdl->bn_into[j] = i; mdl->conv_in_bn[i] = j;
             }
@@ -470,7 +480,7 @@ void build_cell_runs(hpf_model* mdl)
         };
         for (int i = mdl->part_lo[p]; i < mdl->part_hi[p]; ++i) {
             const int kind = mdl->ops[i].op.kind;
-            if (kind == HPF_OP_CONV && mdl->use_tc[PASS_FWD][i]) run.convs.push_back(i);
+            if (kind == HPF_OP_CONV && mdl->use_pipe[PASS_FWD][i]) run.convs.push_back(i);
             else if (kind == HPF_OP_BNRELU && mdl->bn_into[i] >= 0) continue;
             else if (kind == HPF_OP_ADD && mdl->add_done_by[i] >= 0) continue;
             else close();
@@ -502,7 +512,8 @@ void build_memory_plan(hpf_model* mdl)
             if (o.op.kind == HPF_OP_BNRELU || o.op.kind == HPF_OP_BN) bn = std::max(bn, bn_scratch_bytes((int64_t)mdl->b * o.H * o.W, o.C));
             if (o.op.kind == HPF_OP_CONV && mdl->opt_conv_path != 1)
                 for (int pass : {PASS_FWD, PASS_DGRAD})
-                    if (mdl->use_tc[pass][i]) sk = std::max(sk, conv_pipe_splitk_bytes(conv_shape_of(mdl, i), pass, passes_of(mdl), M));
+                    if (mdl->use_tc[pass][i]) sk = std::max(sk, mdl->use_pipe[pass][i] ? conv_pipe_splitk_bytes(conv_shape_of(mdl, i), pass, passes_of(mdl), M)
+                                                                        : conv_tc_splitk_bytes(conv_shape_of(mdl, i), pass, 3));
         }
         mdl->bn_scratch_bytes_[p] = align_up(bn, 256);
         mdl->splitk_bytes[p] = sk;
@@ -580,7 +591,9 @@ bool op_uses_tc(hpf_model* mdl, int i, int pass)
     // a strided data gradient zero-fills between its samples, so it cannot also add to what is there
     if (pass == PASS_DGRAD && mdl->ops[i].op.stride > 1 && (mdl->edge0[i].accumulate || mdl->edge0[i].addend >= 0)) return false;
     if (pass == PASS_WGRAD) return conv_tc_supported(conv_shape_of(mdl, i), pass);
-    return conv_pipe_geom(conv_shape_of(mdl, i), pass, passes_of(mdl), mdl->M, &mdl->pipe_geom[pass][i]);
+    const ConvShape s = conv_shape_of(mdl, i);
+    mdl->use_pipe[pass][i] = mdl->has_bn && conv_pipe_geom(s, pass, passes_of(mdl), mdl->M, &mdl->pipe_geom[pass][i]);
+    return mdl->use_pipe[pass][i] || conv_tc_supported(s, pass);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -645,8 +658,10 @@ int forward_op(hpf_model* mdl, int i, int m, int g, cudaStream_t st, int sl)
                 if (run.convs[0] == i)
                     CU(conv_pipe_cell_launch(mdl->ws + run.ops_off, (int)run.convs.size(), m, g, mdl->opt_cell, run.smem, run.tmem,
                                              reinterpret_cast<unsigned int*>(mdl->ws + mdl->cell_bar_off[sl]), mdl->status(), st, &mdl->launches));
-            } else {
+            } else if (mdl->use_pipe[PASS_FWD][i]) {
                 CU(conv_pipe_launch(&mdl->pipe_plan[PASS_FWD][i], m, g, late, mdl->status(), st, &mdl->launches));
+            } else {
+                CU(conv_tc_launch(&mdl->tile_plan[PASS_FWD][i], mdl->status(), st, &mdl->launches, m, g, late));
             }
         }
         else CU(conv_fwd_simt(in0, mdl->params + o.w_off, out, residual, gs, st, &mdl->launches));
@@ -727,7 +742,8 @@ int backward_op(hpf_model* mdl, int i, int m, int g, cudaStream_t st, int sl)
                                    mdl->ws + mdl->conv_scratch_off[o.part] + k * mdl->conv_scratch_ms[o.part], wst, &mdl->launches));
         }
         if (q.src0 >= 0) {
-            if (mdl->use_tc[PASS_DGRAD][i]) CU(conv_pipe_launch(&mdl->pipe_plan[PASS_DGRAD][i], m, g, false, mdl->status(), st, &mdl->launches));
+            if (mdl->use_pipe[PASS_DGRAD][i]) CU(conv_pipe_launch(&mdl->pipe_plan[PASS_DGRAD][i], m, g, false, mdl->status(), st, &mdl->launches));
+            else if (mdl->use_tc[PASS_DGRAD][i]) CU(conv_tc_launch(&mdl->tile_plan[PASS_DGRAD][i], mdl->status(), st, &mdl->launches, m, g));
             else CU(conv_dgrad_simt(dout, mdl->params + o.w_off, mdl->grad(q.src0, m), addend, e.accumulate != 0, gs, st, &mdl->launches));
         }
         break;
@@ -1232,7 +1248,7 @@ int hpf_bind(hpf_model* mdl, float* d_params, float* d_grad_slots, float* d_grad
                 CU(cudaMemcpyAsync(mdl->ws + mdl->prep_table_off[p], mdl->prep_table[p].data(),
                                    sizeof(WeightPrepEntry) * mdl->prep_table[p].size(), cudaMemcpyHostToDevice, mdl->streams[0]));
         CU(conv_pipe_init());
-        for (int pass = 0; pass < 2; ++pass) mdl->pipe_plan[pass].assign(n, ConvPipePlan());
+        for (int pass = 0; pass < 2; ++pass) { mdl->pipe_plan[pass].assign(n, ConvPipePlan()); mdl->tile_plan[pass].assign(n, ConvTcPlan()); }
         mdl->wgrad_plan.resize(n);
         std::vector<char> first_done(mdl->P, 0);
         for (int i = 0; i < n; ++i) {
@@ -1241,6 +1257,8 @@ int hpf_bind(hpf_model* mdl, float* d_params, float* d_grad_slots, float* d_grad
             const int src = o.op.src0, p = o.part;
             const ConvShape s = conv_shape_of(mdl, i);
             const GradEdge& ed = mdl->edge0[i];
+            ConvTcHints tile;                     // launches on the tile kernel
+            tile.micro_batches = M; tile.splitk_bytes = mdl->splitk_bytes[p];
             if (mdl->use_tc[PASS_FWD][i]) {
                 const float* in = mdl->act(src, 0);
                 const float* residual = nullptr;
@@ -1260,16 +1278,26 @@ int hpf_bind(hpf_model* mdl, float* d_params, float* d_grad_slots, float* d_grad
                     bn.in_stats = mdl->stats(jb, 0); bn.in_y = mdl->act(jb, 0); bn.in_eps = b.op.eps;
                 }
                 // the weights are prepared just ahead of the partition's first convolution
-                CU(conv_pipe_prepare(&mdl->pipe_plan[PASS_FWD][i], s, PASS_FWD, passes, M, in, wp + o.w_off, wp + G + o.w_off, mdl->act(i, 0),
+                if (mdl->use_pipe[PASS_FWD][i]) CU(conv_pipe_prepare(&mdl->pipe_plan[PASS_FWD][i], s, PASS_FWD, passes, M, in, wp + o.w_off, wp + G + o.w_off, mdl->act(i, 0),
                                      residual, false, &bn, mdl->ws + mdl->splitk_off[p], mdl->splitk_bytes[p], first_done[p] != 0));
+                else {
+                    tile.splitk = mdl->splitk_bytes[p] ? mdl->ws + mdl->splitk_off[p] : nullptr;
+                    CU(conv_tc_prepare(&mdl->tile_plan[PASS_FWD][i], s, PASS_FWD, passes, in, nullptr, wp + o.w_off, wp + G + o.w_off, mdl->act(i, 0), residual,
+                                       false, nullptr, &tile));
+                }
                 first_done[p] = 1;
             }
-            if (mdl->use_tc[PASS_DGRAD][i])
+            if (mdl->use_pipe[PASS_DGRAD][i])
                 CU(conv_pipe_prepare(&mdl->pipe_plan[PASS_DGRAD][i], s, PASS_DGRAD, passes, M, mdl->grad(i, 0), wp + 2 * G + o.w_off,
                                      wp + 3 * G + o.w_off, mdl->grad(src, 0), ed.addend >= 0 ? mdl->grad(ed.addend, 0) : nullptr,
                                      ed.accumulate != 0, nullptr, mdl->ws + mdl->splitk_bwd_off[p], mdl->splitk_bytes[p], true));
+            else if (mdl->use_tc[PASS_DGRAD][i]) {
+                tile.splitk = mdl->splitk_bytes[p] ? mdl->ws + mdl->splitk_bwd_off[p] : nullptr;
+                CU(conv_tc_prepare(&mdl->tile_plan[PASS_DGRAD][i], s, PASS_DGRAD, passes, mdl->grad(i, 0), nullptr, wp + 2 * G + o.w_off, wp + 3 * G + o.w_off,
+                                   mdl->grad(src, 0), ed.addend >= 0 ? mdl->grad(ed.addend, 0) : nullptr, ed.accumulate != 0, nullptr, &tile));
+            }
             if (mdl->use_tc[PASS_WGRAD][i]) {
-                ConvBnFuse hint;
+                ConvTcHints hint;
                 hint.wgrad_transposing = mdl->opt_wgrad_direct ? 0 : 1;
                 hint.micro_batches = M; hint.slot_stride = mdl->G; hint.partial_stride = (long long)(mdl->conv_scratch_ms[p] / sizeof(float));
                 CU(conv_tc_prepare(&mdl->wgrad_plan[i], s, PASS_WGRAD, mdl->opt_conv_path == 2 ? 1 : mdl->opt_wgrad_passes, mdl->grad(i, 0), mdl->act(src, 0),
@@ -1689,7 +1717,7 @@ static int conv_single(int pass, const float* in, const float* in2, const float*
     DeviceStatus* status = reinterpret_cast<DeviceStatus*>(reinterpret_cast<char*>(d_scratch) + sb - 256);
     const int64_t nw = (int64_t)K * R * R * C;
     const float* hi = wprep ? wprep + (pass == PASS_DGRAD ? 2 * nw : 0) : nullptr;
-    ConvBnFuse split;
+    ConvTcHints split;
     split.wgrad_transposing = transposing ? 1 : 0;
     if (pass != PASS_WGRAD) {
         const size_t a = conv_simt_scratch_bytes(s), b = conv_tc_scratch_bytes(s);
