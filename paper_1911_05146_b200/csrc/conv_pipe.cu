@@ -38,7 +38,7 @@ constexpr int kSplitThreads = 32 * kSplitWarps, kRowStep = 8 * kSplitWarps;
 constexpr int kPipeThreads = 32 * (kFirstSplit + kSplitWarps + kEpiWarps);
 constexpr int kMaxBlockRows = 768, kRowBatch = 4;     // operand rows of a block at most; rows a splitter thread has in flight
 constexpr uint32_t kPipeSmem = 222 * 1024;            // dynamic shared memory of a CTA
-constexpr int kMaxA = 4, kMaxB = 8;
+constexpr int kMaxA = 8, kMaxB = 8;
 
 struct PipeScalars {
     const float* in;
@@ -53,12 +53,12 @@ struct PipeScalars {
     uint32_t magic_w, magic_img, magic_strip;
     int in_sw, in_sh, in_sn, os_w, os_h, os_n;
     int zero_fill, out_h, out_w, dense_h, dense_w;
-    int a_stages, b_stages, b_resident, acc_bufs, split_groups, epi_alternate;
+    int a_stages, b_stages, b_taps, b_resident, acc_bufs, split_groups, epi_alternate;
     // how the operand is copied: flat (128 consecutive pixels per box) or blocks of box_h padded rows of one map
     int flat, box_h, box_pos, blocks_per_img;
     uint32_t magic_box, magic_bpi;
     long long pix_ms;                                 // flat: pixels per micro-batch; else maps per micro-batch
-    uint32_t a_stage_bytes, b_stage_bytes, acc_cols, tmem_cols, idesc, idesc2;
+    uint32_t a_stage_bytes, b_stage_bytes, b_tap_bytes, acc_cols, tmem_cols, idesc, idesc2;
     uint32_t off_b, off_bn, off_red, off_stat, off_stage;
     int three, stacked, pdl_late, w_ready;
     // BN+ReLU on the way in
@@ -269,14 +269,13 @@ __device__ __forceinline__ Span span_of(const PipeScalars& p, const UnitWalk& u)
     return r;
 }
 
-constexpr int kMomentPlane = kEpiWarps * 32 * 2;      // float4: one per thread and column group (two per warp)
-
 // What one warp does with 32 rows x 32 (or 16) columns of a finished tile, which stand in its patch of shared memory.
 struct EmitArgs {
     float* out;                  // this warp's column group
     const float* extra;
     const float4* patch;
-    float4* moments;             // this lane's k, sum (x - k), sum (x - k)^2 of its four columns: three planes of kMomentPlane, or null
+    float* moments;              // the warp's k, sum (x - k), sum (x - k)^2 of its columns: three rows of mom_pitch floats, or null
+    int mom_pitch;
     bool accumulate, ok;
     int zero_fill, dense_h, dense_w;
 };
@@ -306,12 +305,11 @@ __device__ __forceinline__ void emit_rows(const EmitArgs& a, int ro, int fill, i
     float4 k = make_float4(0.f, 0.f, 0.f, 0.f), sd = k, sq = k;
     const bool moments = a.moments != nullptr && who != 0u;
     if (moments) {
-        if (have_shift) k = a.moments[0];
+        if (have_shift) k = *reinterpret_cast<const float4*>(a.moments + 4 * cq);
         else {
             const int r0 = __ffs(who) - 1, so = __shfl_sync(0xffffffffu, ro, r0);
             k = a.patch[r0 * 8 + (cq ^ (r0 & 7))];
             if (a.extra) k = add4(k, __ldcg(reinterpret_cast<const float4*>(a.extra + so + 4 * cq)));
-            a.moments[0] = k;
         }
     }
 #pragma unroll 1
@@ -350,8 +348,15 @@ __device__ __forceinline__ void emit_rows(const EmitArgs& a, int ro, int fill, i
         }
     }
     if (moments) {
-        a.moments[kMomentPlane] = add4(a.moments[kMomentPlane], sd);
-        a.moments[2 * kMomentPlane] = add4(a.moments[2 * kMomentPlane], sq);
+        // the lanes that share a column, then one lane per four columns adds to the block's sums
+#pragma unroll 1
+        for (int o = 16; o >= steps; o >>= 1) { sd = lane_sum(sd, o); sq = lane_sum(sq, o); }
+        if (lane < steps) {
+            float4 *pk = reinterpret_cast<float4*>(a.moments + 4 * cq), *pd = reinterpret_cast<float4*>(a.moments + a.mom_pitch + 4 * cq),
+                   *pq = reinterpret_cast<float4*>(a.moments + 2 * a.mom_pitch + 4 * cq);
+            if (have_shift) { *pd = add4(*pd, sd); *pq = add4(*pq, sq); }
+            else { *pk = k; *pd = sd; *pq = sq; }
+        }
     }
     if (a.zero_fill == 2) {
         // strided data gradient: the positions between the samples receive no contribution
@@ -406,9 +411,9 @@ template <bool RESIDENT, int KIND>
 __device__ __forceinline__ void mma_role(const PipeScalars& p, const MmaEnv& e)
 {
     const uint64_t a_desc = smem_desc(0, 16, 1024, 128), b_desc = smem_desc(0, 16, 512, 64);
-    const uint32_t idesc = p.idesc, idesc2 = p.idesc2, acc_cols = p.acc_cols, a_step = p.a_stage_bytes >> 4, b_step = p.b_stage_bytes >> 4;
+    const uint32_t idesc = p.idesc, idesc2 = p.idesc2, acc_cols = p.acc_cols, a_step = p.a_stage_bytes >> 4, b_step = p.b_stage_bytes >> 4, b_tap = p.b_tap_bytes >> 4;
     const uint64_t b_half = ((uint32_t)p.n_chunk * 64u) >> 4;
-    const int taps = p.taps, R = p.R, a_stages = p.a_stages, b_stages = p.b_stages, acc_bufs = p.acc_bufs, T = p.T;
+    const int taps = p.taps, group = RESIDENT ? p.taps : p.b_taps, R = p.R, a_stages = p.a_stages, b_stages = p.b_stages, acc_bufs = p.acc_bufs, T = p.T;
     const uint64_t row_step = (uint64_t)((p.Wp - (R - 1)) * 8);      // from a window row's last tap to the next row's first
     const uint64_t a_first = a_desc | (uint64_t)(e.smem_base >> 4), b_first = b_desc | (uint64_t)((e.smem_base + p.off_b) >> 4);
     int s = 0, bs = 0, buf = 0, b_it = 0, a_it = 0;
@@ -429,25 +434,28 @@ __device__ __forceinline__ void mma_role(const PipeScalars& p, const MmaEnv& e)
         for (int c = kb; c < ke; ++c) {
             if (!mbar_wait(e.a_full + 8 * s, apar, e.abort_flag)) { report(p.status, 24); return; }
             uint64_t a = a_first + (uint64_t)((uint32_t)s * a_step) + lead;
-            uint64_t b = RESIDENT ? b_first + (uint64_t)((uint32_t)(c * taps) * b_step) : 0;
+            uint64_t b = RESIDENT ? b_first + (uint64_t)((uint32_t)(c * taps) * b_tap) : 0;
             int sx = 0;
 #pragma unroll 1
-            for (int tap = 0; tap < taps; ++tap) {
+            for (int left = taps; left > 0; left -= group) {
                 if (!RESIDENT) {
                     if (!mbar_wait(e.b_full + 8 * bs, bpar, e.abort_flag)) { report(p.status, 25); *e.b_used = b_it; *e.a_used = a_it; return; }
                     b = b_first + (uint64_t)((uint32_t)bs * b_step);
                 }
 #pragma unroll 1
-                for (int t = 0; t < nt; ++t) issue_tile<KIND>(acc0 + (uint32_t)t * acc_cols, a + (uint64_t)(t * 1024), b, b_half, idesc, idesc2, keep);
-                keep = 1u;
-                if (RESIDENT) b += b_step;
-                else {
+                for (int k = 0; k < group; ++k) {
+#pragma unroll 1
+                    for (int t = 0; t < nt; ++t) issue_tile<KIND>(acc0 + (uint32_t)t * acc_cols, a + (uint64_t)(t * 1024), b, b_half, idesc, idesc2, keep);
+                    keep = 1u;
+                    b += b_tap;
+                    a += 8;
+                    if (++sx == R) { sx = 0; a += row_step - 8; }
+                }
+                if (!RESIDENT) {
                     umma_commit(e.b_empty + 8 * bs);
                     ++b_it;
                     if (++bs == b_stages) { bs = 0; bpar ^= 1u; }
                 }
-                a += 8;
-                if (++sx == R) { sx = 0; a += row_step - 8; }
             }
             umma_commit(e.a_empty + 8 * s);
             ++a_it;
@@ -553,7 +561,7 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
         if (elect_one()) {
             // ---- weights ----
             if (!CELL && !p.w_ready) pdl_wait();
-            const uint32_t half = (uint32_t)p.n_chunk * 64u, stage_bytes = p.b_stage_bytes, dst0 = smem_base + p.off_b;
+            const uint32_t half = (uint32_t)p.n_chunk * 64u, tap_bytes = p.b_tap_bytes, dst0 = smem_base + p.off_b;
             const bool three = p.three != 0;
             const uint32_t tx = three ? 2u * half : half;
             const int taps = p.taps, c_in = p.c_in;
@@ -564,7 +572,7 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
 #pragma unroll 1
                 for (int c = 0; c < p.n_chunks; ++c)
 #pragma unroll 1
-                    for (int tap = 0; tap < taps; ++tap, dst += stage_bytes) {
+                    for (int tap = 0; tap < taps; ++tap, dst += tap_bytes) {
                         tma_load_2d(dst, &gp.tm_b, b_full, tap * c_in + 16 * c, co0);
                         if (three) tma_load_2d(dst + half, &gp.tm_b_lo, b_full, tap * c_in + 16 * c, co0);
                     }
@@ -578,12 +586,16 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
 #pragma unroll 1
                     for (int c = u.kb(p), ce = u.ke(p); c < ce && live; ++c)
 #pragma unroll 1
-                        for (int tap = 0; tap < taps; ++tap, ++it) {
+                        for (int tap = 0; tap < taps; ++it) {
                             if (!mbar_wait(b_empty + 8 * s, par, &abort_flag)) { report(p.status, 21); live = false; break; }
-                            const uint32_t bar = b_full + 8 * s, dst = dst0 + (uint32_t)s * stage_bytes;
-                            mbar_expect_tx(bar, tx);
-                            tma_load_2d(dst, &gp.tm_b, bar, tap * c_in + 16 * c, co0);
-                            if (three) tma_load_2d(dst + half, &gp.tm_b_lo, bar, tap * c_in + 16 * c, co0);
+                            const uint32_t bar = b_full + 8 * s;
+                            uint32_t dst = dst0 + (uint32_t)s * p.b_stage_bytes;
+                            mbar_expect_tx(bar, tx * (uint32_t)p.b_taps);
+#pragma unroll 1
+                            for (int e = tap + p.b_taps; tap < e; ++tap, dst += tap_bytes) {
+                                tma_load_2d(dst, &gp.tm_b, bar, tap * c_in + 16 * c, co0);
+                                if (three) tma_load_2d(dst + half, &gp.tm_b_lo, bar, tap * c_in + 16 * c, co0);
+                            }
                             if (++s == p.b_stages) { s = 0; par ^= 1u; }
                         }
                 b_issued = it;
@@ -605,8 +617,10 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
         }
     } else if (warp >= kFirstSplit && warp < kFirstSplit + kSplitWarps) {
         // ---- the operand: normalise, split ----
-        // The warps work on `split_groups` blocks at a time (as many as the ring holds, up to four): what a block costs is a
-        // chain of latencies - copy, shared-memory reads, arithmetic, stores, fence, hand-over - and not instructions.
+        // The warps work on `split_groups` blocks at a time: what a block costs is a chain of latencies - copy, shared-memory
+        // reads, arithmetic, stores, fence, hand-over - and not instructions.  The ring is a multiple of the groups, so that a
+        // stage is always the same group's: one that came back to a stage after another group's turn could take the parity of
+        // the round before last for this round's.
         const int tid = threadIdx.x - 32 * kFirstSplit;
         const int groups = p.split_groups, wpg = kSplitWarps / groups, my_group = (tid >> 5) / wpg, gw = (tid >> 5) - my_group * wpg;
         // a thread owns one 16-byte quarter of the rows row0 + row_step * j; the eight rows of a warp are taken so that a
@@ -626,7 +640,8 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
         // a step of row_step positions in maps, rows and columns of the padded grid
         const int dn = BN_IN && !FLAT ? row_step / p.img_pos : 0, drem = row_step - dn * p.img_pos;
         const int dy = BN_IN && !FLAT ? drem / p.Wp : 0, dx = drem - dy * p.Wp, Hp = BN_IN && !FLAT ? p.img_pos / p.Wp : 1;
-        int s = 0, turn = 0, cur_m = -1;
+        // this group's next block: its chunk within the unit, its place in the ring
+        int s = my_group, ahead = my_group, cur_m = -1;
         uint32_t par = 0;
         const bool store_y = BN_IN && slice == 0;
         bool ok = true;
@@ -648,8 +663,8 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
                     for (int i = tid; i < 2 * C; i += kSplitThreads) p.bn_stats[(size_t)cur_m * 2 * C + i] = tab[i];
             }
 #pragma unroll 1
-            for (int c = kb; c < ke; ++c) {
-                if (turn == my_group) {
+            for (int c = kb + ahead; c < ke; c += groups) {
+                {
                     ok = mbar_wait(a_raw + 8 * s, par, &abort_flag) && ok;
                     // (after a wait that gave up the warps run through the rest without waiting: they still have to meet at
                     // the named barriers)
@@ -727,9 +742,11 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
                     __syncwarp();
                     if (lane == 0) mbar_arrive(a_full + 8 * s);
                 }
-                if (++turn == groups) turn = 0;
-                if (++s == S) { s = 0; par ^= 1u; }
+                s += groups;
+                if (s >= S) { s -= S; par ^= 1u; }
+                ahead += groups;
             }
+            ahead -= ke - kb;
         }
     } else if (warp >= kFirstSplit + kSplitWarps) {
         // ---- write-out: tensor memory -> registers -> a 32 x 32 patch of shared memory -> global memory ----
@@ -751,12 +768,11 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
         if (!CELL) pdl_wait();
         int buf = alternate ? half : 0, flip = 0;
         uint32_t par = 0;
-        // moments of the block so far: this lane's columns in shared memory, rows counted per warp
-        float4* mom = reinterpret_cast<float4*>(smem + p.off_stat) + ew * 64 + lane;
+        // the warps' moments of the block so far, twice: those of the block before may still be read
+        float* const mom0 = reinterpret_cast<float*>(smem + p.off_stat);
+        const int mom_size = parts * (3 * n_chunk + 1);
         bool have = false;
         int count = 0;
-        if (stats)
-            for (int gi = 0; gi < 2; ++gi) { mom[gi * 32 + kMomentPlane] = make_float4(0.f, 0.f, 0.f, 0.f); mom[gi * 32 + 2 * kMomentPlane] = make_float4(0.f, 0.f, 0.f, 0.f); }
 #pragma unroll 1
         for (UnitWalk u(p, m_first, u_first, u_count); u.left > 0; u.next(p)) {
             bool finish = true, ok = true;
@@ -764,7 +780,7 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
             const int nt = u.tiles(p);
             float* out = p.out + (long long)u.m * p.out_ms + co0;
             const float* extra = p.extra ? p.extra + (long long)u.m * p.out_ms + co0 : nullptr;
-            EmitArgs ea{out, extra, patch, nullptr, p.accumulate != 0, true, p.zero_fill, p.dense_h, p.dense_w};
+            EmitArgs ea{out, extra, patch, nullptr, n_chunk, p.accumulate != 0, true, p.zero_fill, p.dense_h, p.dense_w};
             // this lane's row of a tile, and which neighbours of a strided data gradient's sample get zeros
             int ro = -1, fill = 0;
             auto place = [&](int t) {
@@ -843,7 +859,7 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
                         ea.extra = extra + 32 * g;
                         if (t > t_first || gi > 0) emit_residuals(ea, ro, lane, lsh, 0, e);
                     }
-                    if (stats) ea.moments = mom + gi * 32;
+                    if (stats) ea.moments = mom0 + flip * mom_size + part * 3 * n_chunk + 32 * g;
                     // 16 columns of the row at a time into the patch
 #pragma unroll 1
                     for (int h = 0; h < 2 && 16 * h < left; ++h) {
@@ -879,22 +895,7 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
             turn ^= 1;
             if (stats && finish && (ksplit > 1 || u.last_of_block())) {
                 // the block's moments: lanes, then the warps' parts, each about its own shift
-                float* contrib = reinterpret_cast<float*>(smem + p.off_stat + 3u * 16u * kMomentPlane) + (size_t)flip * parts * (3 * n_chunk + 1);
-#pragma unroll 1
-                for (int g = g_first, gi = 0; g < groups; g += g_step, ++gi) {
-                    const int lpr = n_chunk - 32 * g >= 32 ? 8 : 4;
-                    float4 sd = mom[gi * 32 + kMomentPlane], sq = mom[gi * 32 + 2 * kMomentPlane];
-                    const float4 k = mom[gi * 32], zero = make_float4(0.f, 0.f, 0.f, 0.f);
-                    mom[gi * 32 + kMomentPlane] = zero; mom[gi * 32 + 2 * kMomentPlane] = zero;
-#pragma unroll 1
-                    for (int o = 16; o >= lpr; o >>= 1) { sd = lane_sum(sd, o); sq = lane_sum(sq, o); }
-                    if (lane < lpr) {
-                        float* c3 = contrib + (size_t)part * 3 * n_chunk + 32 * g + 4 * lane;
-                        *reinterpret_cast<float4*>(c3) = k;
-                        *reinterpret_cast<float4*>(c3 + n_chunk) = sd;
-                        *reinterpret_cast<float4*>(c3 + 2 * n_chunk) = sq;
-                    }
-                }
+                float* contrib = mom0 + flip * mom_size;
                 float* counts = contrib + (size_t)parts * 3 * n_chunk;
                 if (lane == 0 && (whole || half == 0)) counts[part] = (float)count;
                 count = 0; have = false;
@@ -1149,7 +1150,8 @@ int sm_count()
 }
 
 constexpr int kPlanSms = 148;                         // the split of the work is planned for a whole B200, with or without a device at hand
-inline unsigned int stat_bytes(int n_chunk) { return 3u * 16u * kMomentPlane + (unsigned int)(2 * (n_chunk <= 64 ? 8 : 4) * (3 * n_chunk + 1) * 4 + 127) & ~127u; }
+inline unsigned int stat_bytes(int n_chunk) { return (unsigned int)(2 * (n_chunk <= 64 ? 8 : 4) * (3 * n_chunk + 1) * 4 + 127) & ~127u; }
+inline int split_groups_of(int a_stages) { return a_stages % 4 == 0 ? 4 : (a_stages % 2 == 0 ? 2 : 1); }
 inline unsigned int bn_bytes(int c_in) { return (unsigned int)(4 * c_in * 4 + 4 * kSplitThreads * 16); }
 
 }  // namespace
@@ -1186,13 +1188,16 @@ bool conv_pipe_geom(const ConvShape& s, int pass, int passes, int M, ConvPipeGeo
     g->pos_per_m = (int)pos;
     g->tiles_per_m = (g->pos_per_m + kTileM - 1) / kTileM;
     const int taps = s.R * s.R, chunks = v.c_in / 16, n = g->n_chunk;
-    g->b_stage_bytes = (unsigned int)(three ? 2 : 1) * (unsigned int)n * 64u;
-    const unsigned int all_b = g->b_stage_bytes * (unsigned int)(taps * chunks);
-    const unsigned int fixed = kEpiWarps * 4096u + stat_bytes(n) + (pass == PASS_FWD ? bn_bytes(v.c_in <= 512 ? v.c_in : 0) : 0u);
-    // Tiles per unit, stacked weights (hi*hi and hi*lo from one MMA over [B_hi; B_lo]) and accumulator sets: the combination
-    // with the least modelled time for the busiest CTA.  Clocks per MMA (K = 8) as measured alone; at 128 columns an unstacked
-    // MMA reads 128 bytes of shared memory per clock, all there is, and pays for every other access; operand and weight
-    // bytes at 20 and 28 per clock and SM; about 350 clocks per 128 x 32 outputs written.
+    g->b_tap_bytes = (unsigned int)(three ? 2 : 1) * (unsigned int)n * 64u;
+    const unsigned int all_b = g->b_tap_bytes * (unsigned int)(taps * chunks);
+    // (the data gradient forms no moments and applies no BN)
+    const unsigned int fixed = kEpiWarps * 4096u + (pass == PASS_FWD ? stat_bytes(n) + bn_bytes(v.c_in <= 512 ? v.c_in : 0) : 0u);
+    // Tiles per unit, stacked weights (hi*hi and hi*lo from one MMA over [B_hi; B_lo]), accumulator sets and the two rings:
+    // the combination with the least modelled time for the busiest CTA, from clocks measured stage by stage.  A chunk takes
+    // the longest of: its MMAs (K = 8; at 128 columns an unstacked MMA reads 128 bytes of shared memory per clock, all there
+    // is, and pays for every other access) and the waits between them; an operand stage's life (copy, split, MMAs) over the
+    // stages of the ring - with two stages of 32 KB a 1x1 convolution waited for that, 1640 clocks a chunk against 870 of
+    // MMAs; the same for the weights; the bytes at 20 (operand, mostly from HBM) and 28 (weights, L2) per clock and SM.
     auto clk = [](int c) { return c <= 32 ? 40.0 : (c <= 64 ? 48.0 : (c <= 96 ? 58.0 : (c <= 128 ? 68.0 : 0.5 * c))); };
     double best = 0.0;
     g->T = 0;
@@ -1205,22 +1210,38 @@ bool conv_pipe_geom(const ConvShape& s, int pass, int passes, int M, ConvPipeGeo
                 const int nj = (rows + kRowStep * kRowBatch - 1) / (kRowStep * kRowBatch) * kRowBatch;
                 if (nj * kRowStep > kMaxBlockRows) continue;
                 const unsigned int a_stage = (unsigned int)(nj * kRowStep) * 128u;
-                // room for two operand blocks beside the weights: all of them, or a ring of at least three stages
-                const bool resident = all_b <= 100u * 1024u && all_b + fixed + 2 * a_stage <= kPipeSmem;
-                if (!resident && 3 * g->b_stage_bytes + fixed + 2 * a_stage > kPipeSmem) continue;
                 const int units = (g->tiles_per_m + T - 1) / T;
                 const int per_slice = kPlanSms / g->slices > 0 ? kPlanSms / g->slices : 1;
                 const double rounds = (double)(((long long)M * units + per_slice - 1) / per_slice);
                 const double step = !three ? clk(n) : (stacked ? clk(2 * n) + clk(n) : 3.0 * (n == 128 ? 80.0 : clk(n)));
-                double mma = (double)T * 2.0 * taps * chunks * step;
-                if (!resident) mma = std::max(mma, (double)all_b / 28.0);
-                const double load = (double)rows * v.c_in * 4.0 / 20.0, epi = 350.0 * T * ((n + 31) / 32);
-                const double body = bufs == 2 ? std::max(std::max(mma, load), epi) : std::max(mma, load) + epi;
-                const double cost = rounds * body + std::max(mma, load) * 0.3 + epi;
-                if (g->T == 0 || cost < best * 0.999) {
-                    best = cost;
-                    g->T = T; g->units_per_m = units; g->a_rows = nj * kRowStep; g->a_stage_bytes = a_stage; g->b_resident = resident ? 1 : 0;
-                    g->stacked = stacked; g->acc_cols = (unsigned int)cols; g->acc_bufs = bufs;
+                const double tap_mma = 2.0 * T * step, epi = 1100.0 * T * ((n + 31) / 32) / 2.0;
+                // weights: resident, or a ring whose stage holds the taps of a window row (fewer waits) or one tap
+                for (int bt = s.R; bt >= 0; bt = bt == 3 ? 1 : bt - 1) {
+                    const bool resident = bt == 0;
+                    if (resident && all_b > 100u * 1024u) continue;
+                    const unsigned int b_stage = resident ? all_b : (unsigned int)bt * g->b_tap_bytes;
+                    for (int bs = resident ? 1 : 2; bs <= (resident ? 1 : kMaxB); ++bs) {
+                        const unsigned int b_all = (unsigned int)bs * b_stage;
+                        if (b_all + fixed + 2 * a_stage > kPipeSmem) break;
+                        int as = (int)((kPipeSmem - fixed - b_all) / a_stage);
+                        if (as > kMaxA) as = kMaxA;
+                        for (; as >= 2; --as) {
+                        const int groups = split_groups_of(as);
+                        const double split = three ? 250.0 + 5.6 * rows * groups / 4.0 : 100.0;
+                        const double mma = resident ? taps * tap_mma + 100.0
+                                                    : (double)(taps / bt) * std::max({bt * tap_mma + 100.0, (1000.0 + b_stage / 40.0 + bt * tap_mma) / bs, b_stage / 28.0});
+                        const double chunk = std::max({mma, (1200.0 + rows * 1.6 + split + mma) / as, split / groups, rows * 64.0 / 20.0});
+                        const double k_loop = chunk * chunks, body = bufs == 2 ? std::max(k_loop, epi) : k_loop + epi;
+                        const double cost = rounds * body + chunk + 1000.0 + epi;
+                        if (g->T == 0 || cost < best * 0.999) {
+                            best = cost;
+                            g->T = T; g->units_per_m = units; g->a_rows = nj * kRowStep; g->a_stage_bytes = a_stage; g->a_stages = as;
+                            g->b_resident = resident ? 1 : 0; g->b_taps = resident ? taps : bt; g->b_stages = resident ? taps * chunks : bs;
+                            g->b_stage_bytes = resident ? g->b_tap_bytes : b_stage;
+                            g->stacked = stacked; g->acc_cols = (unsigned int)cols; g->acc_bufs = bufs;
+                        }
+                        }
+                    }
                 }
             }
     if (!g->T) return false;
@@ -1234,7 +1255,6 @@ bool conv_pipe_geom(const ConvShape& s, int pass, int passes, int M, ConvPipeGeo
         if (S > chunks) S = chunks;
         if (S > 1) g->ksplit = S;
     }
-    if (g->ksplit > 1) g->b_resident = 0;
     // Blocks of units: the reader of the BN moments merges one row per block, so as few as leave the busiest CTA with at most
     // a tenth more work.
     g->unit_block = 1;
@@ -1247,20 +1267,7 @@ bool conv_pipe_geom(const ConvShape& s, int pass, int passes, int M, ConvPipeGeo
         }
     }
     g->blocks_per_m = (g->units_per_m + g->unit_block - 1) / g->unit_block;
-    if (!g->b_resident && 3 * g->b_stage_bytes + fixed + 2 * g->a_stage_bytes > kPipeSmem) return false;
-    unsigned int left = kPipeSmem - fixed;
-    if (g->b_resident) { g->b_stages = taps * chunks; left -= all_b; }
-    else {
-        // the operand ring first gets two stages; the weights up to eight of what is left, the operand the rest
-        int bs = (int)((left - 2 * g->a_stage_bytes) / g->b_stage_bytes);
-        if (bs > kMaxB) bs = kMaxB;
-        if (bs > taps * chunks) bs = taps * chunks;
-        g->b_stages = bs;
-        left -= (unsigned int)bs * g->b_stage_bytes;
-    }
-    g->a_stages = (int)(left / g->a_stage_bytes);
-    if (g->a_stages > kMaxA) g->a_stages = kMaxA;
-    return g->a_stages >= 2;
+    return true;
 }
 
 bool conv_pipe_can_fuse_bn_output(const ConvPipeGeom& g) { return g.n_chunk <= 128; }      // a warp keeps the moments of two groups of 32 channels
@@ -1350,19 +1357,19 @@ cudaError_t conv_pipe_prepare(ConvPipePlan* plan, const ConvShape& s, int pass, 
         e = g.flat ? encode_map(tm, in, 2, fd, fs, fb, CU_TENSOR_MAP_SWIZZLE_128B) : encode_map(tm, in, 4, rd, rs, rb, CU_TENSOR_MAP_SWIZZLE_128B);
         if (e != cudaSuccess) return e;
     }
-    p.a_stages = g.a_stages; p.b_stages = g.b_stages; p.b_resident = g.b_resident; p.acc_bufs = g.acc_bufs;
-    p.a_stage_bytes = g.a_stage_bytes; p.b_stage_bytes = g.b_stage_bytes; p.acc_cols = g.acc_cols;
+    p.a_stages = g.a_stages; p.b_stages = g.b_stages; p.b_taps = g.b_taps; p.b_resident = g.b_resident; p.acc_bufs = g.acc_bufs;
+    p.a_stage_bytes = g.a_stage_bytes; p.b_stage_bytes = g.b_stage_bytes; p.b_tap_bytes = g.b_tap_bytes; p.acc_cols = g.acc_cols;
     p.tmem_cols = columns_pow2((unsigned int)(g.acc_bufs * g.T) * g.acc_cols);
     p.idesc = instr_desc(g.n_chunk, false, false);
     p.idesc2 = instr_desc(g.stacked ? 2 * g.n_chunk : g.n_chunk, false, false);
-    p.split_groups = g.a_stages >= 4 ? 4 : 2;
+    p.split_groups = split_groups_of(g.a_stages);
     p.epi_alternate = g.acc_bufs == 2 && g.n_chunk <= 64 && g.ksplit == 1 ? 1 : 0;
     p.three = passes == 3 ? 1 : 0; p.stacked = g.stacked; p.w_ready = w_ready ? 1 : 0;
     const unsigned int a_bytes = (unsigned int)g.a_stages * g.a_stage_bytes;
     p.off_b = a_bytes;
     p.off_stage = (p.off_b + (unsigned int)g.b_stages * g.b_stage_bytes + 127u) & ~127u;
     p.off_stat = p.off_stage + kEpiWarps * 4096u;
-    p.off_red = p.off_stat + stat_bytes(g.n_chunk);
+    p.off_red = p.off_stat + (pass == PASS_FWD ? stat_bytes(g.n_chunk) : 0u);
     p.off_bn = p.off_red + 4 * kSplitThreads * 16;
     L->smem = p.off_red + 1024;
     if (bn && bn->out_partials) {

@@ -15,8 +15,8 @@ struct ConvPipeGeom {
     int unit_block, blocks_per_m; // consecutive units one CTA takes; blocks of a micro-batch = rows of its BN partial moments
     int slices, n_chunk;         // output channels: slices of n_chunk
     int ksplit;                  // CTAs that share one unit's K loop
-    int a_rows, a_stages, b_stages, b_resident, acc_bufs;
-    unsigned int acc_cols, a_stage_bytes, b_stage_bytes;
+    int a_rows, a_stages, b_stages, b_taps, b_resident, acc_bufs;      // b_taps: taps per stage of the weight ring
+    unsigned int acc_cols, a_stage_bytes, b_stage_bytes, b_tap_bytes;
     int stacked;
     int flat, box_h;             // operand copies: 128 consecutive pixels, or box_h padded map rows each
     int pos_per_m, Wp, Hp, halo, strips, strip_w, col0;
