@@ -119,12 +119,15 @@ cudaError_t maxpool_fwd(const float* x, float* y, ConvShape s, cudaStream_t st, 
 cudaError_t maxpool_bwd(const float* x, const float* dy, float* dx, bool accumulate, ConvShape s, cudaStream_t st,
                         int64_t* n_launch);
 // head: a [b][HW][C]; pooled scratch [b][C]; persample scratch [b]
+// Micro-batches of one launch of the head's kernels, and the floats (labels: integers) between their tensors; loss slots follow
+// one another.
+struct HeadGroup { int count = 1; int64_t act = 0, logits = 0, labels = 0, pooled = 0, persample = 0, param = 0; };
 cudaError_t head_fwd(const float* a, const float* Wfc, const float* bias, const int32_t* labels, float* logits,
                      float* pooled, float* persample, float* loss_slot, int b, int HW, int C, int ncls,
-                     cudaStream_t st, int64_t* n_launch);
+                     cudaStream_t st, int64_t* n_launch, const HeadGroup& grp = HeadGroup());
 cudaError_t head_bwd(const float* Wfc, const int32_t* labels, const float* logits, const float* pooled,
                      float* dlogits, float* da, float* dW, float* dbias, int b, int HW, int C, int ncls,
-                     cudaStream_t st, int64_t* n_launch);
+                     cudaStream_t st, int64_t* n_launch, const HeadGroup& grp = HeadGroup());
 
 // ---------------- CUDA-core convolutions (conv_simt.cu) ----------------
 size_t conv_simt_scratch_bytes(const ConvShape& s);

@@ -622,6 +622,18 @@ int cells_under_way(int P, int M, int p, int m, bool bwd)
     return bwd ? busy(t) + busy(t + P) : busy(t) + busy(t - P);
 }
 
+HeadGroup head_group(const hpf_model* mdl, int i, int g)
+{
+    const OpInfo& o = mdl->ops[i];
+    HeadGroup h;
+    h.count = g; h.act = mdl->tensor_stride[o.op.src0]; h.logits = mdl->tensor_stride[i]; h.labels = mdl->b; h.param = mdl->G;
+    if (mdl->M > 1) {
+        h.pooled = (int64_t)(mdl->pooled_off[1] - mdl->pooled_off[0]) / (int64_t)sizeof(float);
+        h.persample = (int64_t)(mdl->persample_off[1] - mdl->persample_off[0]) / (int64_t)sizeof(float);
+    }
+    return h;
+}
+
 // Ops of one stage on the micro-batches m .. m + g - 1.  sl: the stream slot (partition, lane) whose side stream is used.
 // Launches that know nothing of micro-batches take the group as one larger batch where its tensors are contiguous.
 int forward_op(hpf_model* mdl, int i, int m, int g, cudaStream_t st, int sl)
@@ -691,10 +703,9 @@ int forward_op(hpf_model* mdl, int i, int m, int g, cudaStream_t st, int sl)
         CU(maxpool_fwd(in0, out, gs, st, &mdl->launches));
         break;
     case HPF_OP_HEAD:
-        for (int k = m; k < m + g; ++k)
-            CU(head_fwd(src_act(mdl, q.src0, k), mdl->params + o.w_off, mdl->params + o.b_off, mdl->cur_labels + (int64_t)k * mdl->b, mdl->act(i, k),
-                        reinterpret_cast<float*>(mdl->ws + mdl->pooled_off[k]), reinterpret_cast<float*>(mdl->ws + mdl->persample_off[k]),
-                        reinterpret_cast<float*>(mdl->ws + mdl->loss_slots_off) + k, mdl->b, o.iH * o.iW, o.iC, q.c_out, st, &mdl->launches));
+        CU(head_fwd(in0, mdl->params + o.w_off, mdl->params + o.b_off, mdl->cur_labels + (int64_t)m * mdl->b, out,
+                    reinterpret_cast<float*>(mdl->ws + mdl->pooled_off[m]), reinterpret_cast<float*>(mdl->ws + mdl->persample_off[m]),
+                    reinterpret_cast<float*>(mdl->ws + mdl->loss_slots_off) + m, mdl->b, o.iH * o.iW, o.iC, q.c_out, st, &mdl->launches, head_group(mdl, i, g)));
         break;
     }
     return HPF_OK;
@@ -763,11 +774,8 @@ int backward_op(hpf_model* mdl, int i, int m, int g, cudaStream_t st, int sl)
             CU(maxpool_bwd(in0, dout, mdl->grad(q.src0, m), e.accumulate != 0, gs, st, &mdl->launches));
         break;
     case HPF_OP_HEAD:
-        for (int k = m; k < m + g; ++k) {
-            float* sl_k = mdl->gslots + (int64_t)k * mdl->G;
-            CU(head_bwd(mdl->params + o.w_off, mdl->cur_labels + (int64_t)k * mdl->b, mdl->act(i, k), reinterpret_cast<float*>(mdl->ws + mdl->pooled_off[k]),
-                        mdl->grad(i, k), mdl->grad(q.src0, k), sl_k + o.w_off, sl_k + o.b_off, mdl->b, o.iH * o.iW, o.iC, q.c_out, st, &mdl->launches));
-        }
+        CU(head_bwd(mdl->params + o.w_off, mdl->cur_labels + (int64_t)m * mdl->b, mdl->act(i, m), reinterpret_cast<float*>(mdl->ws + mdl->pooled_off[m]),
+                    dout, mdl->grad(q.src0, m), slot + o.w_off, slot + o.b_off, mdl->b, o.iH * o.iW, o.iC, q.c_out, st, &mdl->launches, head_group(mdl, i, g)));
         break;
     }
     return HPF_OK;

@@ -1234,6 +1234,36 @@ maxpool_fwd_kernel(const float* __restrict__ x, float* __restrict__ y, ConvShape
     }
 }
 
+// Four channels per thread.
+__global__ void __launch_bounds__(kThreads)
+maxpool_fwd_vec4_kernel(const float4* __restrict__ x, float4* __restrict__ y, ConvShape s)
+{
+    const int C4 = s.C / 4;
+    const int64_t total = (int64_t)s.N * s.P * s.Q * C4;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += stride) {
+        const int c = (int)(i % C4);
+        int64_t r = i / C4;
+        const int q = (int)(r % s.Q); r /= s.Q;
+        const int p = (int)(r % s.P);
+        const int n = (int)(r / s.P);
+        float4 best = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+        for (int rr = 0; rr < s.R; ++rr) {
+            const int ih = p * s.stride + rr - s.pad;
+            if (ih < 0 || ih >= s.H) continue;
+            const float4* row = x + ((int64_t)n * s.H + ih) * s.W * C4 + c;
+#pragma unroll 3
+            for (int ss = 0; ss < s.R; ++ss) {
+                const int iw = q * s.stride + ss - s.pad;
+                if (iw < 0 || iw >= s.W) continue;
+                const float4 v = __ldg(row + (int64_t)iw * C4);
+                best.x = fmaxf(best.x, v.x); best.y = fmaxf(best.y, v.y); best.z = fmaxf(best.z, v.z); best.w = fmaxf(best.w, v.w);
+            }
+        }
+        y[i] = best;
+    }
+}
+
 // Gather form (no atomics, fixed order): an input position receives dy of every window whose first
 // maximum (row-major window order) it is.
 template <bool ACCUM>
@@ -1331,6 +1361,82 @@ maxpool_bwd_vec4_kernel(const float4* __restrict__ x, const float4* __restrict__
     }
 }
 
+// The same routing for stride 2, four channels and a 2 x 2 block of input positions per thread (C a multiple of 4).  A block
+// at even coordinates meets one window for R = 2 without padding and 2 x 2 for R = 3 with padding 1, whose
+// 5 x 5 inputs are read once for four outputs (6 loads each); position by position every output walked all its windows in
+// full (20 loads on average).  The first maximum of a window is found once for the block.  Contributions are added in window order.
+// 64 x 112 x 112 x 64, R = 3: 925 us before.
+template <int R, bool ACCUM>
+__global__ void __launch_bounds__(kThreads)
+maxpool_bwd_s2_kernel(const float4* __restrict__ x, const float4* __restrict__ dy, float4* __restrict__ dx, ConvShape s)
+{
+    constexpr int PAD = R == 3 ? 1 : 0, WIN = R == 3 ? 2 : 1;      // windows of a block along one axis
+    const int C4 = s.C / 4, HB = (s.H + 1) / 2, WB = (s.W + 1) / 2;
+    const int64_t total = (int64_t)s.N * HB * WB * C4;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += stride) {
+        const int c = (int)(i % C4);
+        int64_t r = i / C4;
+        const int wb = (int)(r % WB); r /= WB;
+        const int hb = (int)(r % HB);
+        const int64_t img = (r / HB);
+        const float4* xi = x + img * s.H * s.W * C4 + c;
+        float acc[2][2][4];
+#pragma unroll
+        for (int a = 0; a < 2; ++a)
+#pragma unroll
+            for (int b = 0; b < 2; ++b)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) acc[a][b][k] = 0.f;
+#pragma unroll
+        for (int p = 0; p < WIN; ++p)
+#pragma unroll
+            for (int q = 0; q < WIN; ++q) {
+                if (hb + p >= s.P || wb + q >= s.Q) continue;
+                const int h0 = 2 * (hb + p) - PAD, w0 = 2 * (wb + q) - PAD;
+                float best[4];
+                int at[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) { best[k] = -INFINITY; at[k] = -1; }
+#pragma unroll
+                for (int rr = 0; rr < R; ++rr)
+#pragma unroll
+                    for (int ss = 0; ss < R; ++ss) {
+                        const int ih = h0 + rr, iw = w0 + ss;
+                        if (ih < 0 || ih >= s.H || iw < 0 || iw >= s.W) continue;
+                        const float4 v4 = __ldg(xi + ((int64_t)ih * s.W + iw) * C4);
+                        const float v[4] = {v4.x, v4.y, v4.z, v4.w};
+#pragma unroll
+                        for (int k = 0; k < 4; ++k)
+                            if (at[k] < 0 || v[k] > best[k]) { best[k] = v[k]; at[k] = rr * R + ss; }
+                    }
+                const float4 g4 = __ldg(dy + ((img * s.P + hb + p) * s.Q + wb + q) * C4 + c);
+                const float g[4] = {g4.x, g4.y, g4.z, g4.w};
+#pragma unroll
+                for (int a = 0; a < 2; ++a)
+#pragma unroll
+                    for (int b = 0; b < 2; ++b) {
+                        const int rr = a + PAD - 2 * p, ss = b + PAD - 2 * q;      // where the position stands in this window
+                        if (rr < 0 || rr >= R || ss < 0 || ss >= R) continue;
+#pragma unroll
+                        for (int k = 0; k < 4; ++k)
+                            if (at[k] == rr * R + ss) acc[a][b][k] += g[k];
+                    }
+            }
+#pragma unroll
+        for (int a = 0; a < 2; ++a)
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {
+                const int h = 2 * hb + a, w = 2 * wb + b;
+                if (h >= s.H || w >= s.W) continue;
+                float4* d = dx + ((img * s.H + h) * s.W + w) * C4 + c;
+                float4 v = make_float4(acc[a][b][0], acc[a][b][1], acc[a][b][2], acc[a][b][3]);
+                if (ACCUM) { const float4 e = *d; v.x = e.x + v.x; v.y = e.y + v.y; v.z = e.z + v.z; v.w = e.w + v.w; }
+                *d = v;
+            }
+    }
+}
+
 // ------------------------------------------------------------------------------------------------
 // head: global average pool + FC + softmax cross-entropy
 // ------------------------------------------------------------------------------------------------
@@ -1362,10 +1468,12 @@ __device__ float block_reduce(float v, bool is_max, float* sh)
 __global__ void __launch_bounds__(kThreads)
 head_fwd_kernel(const float* __restrict__ a, const float* __restrict__ Wfc, const float* __restrict__ bias,
                 const int32_t* __restrict__ labels, float* __restrict__ logits, float* __restrict__ pooled,
-                float* __restrict__ persample, int HW, int C, int ncls)
+                float* __restrict__ persample, int HW, int C, int ncls, const HeadGroup grp)
 {
     extern __shared__ float smem[];
     __shared__ float red[32];
+    a += blockIdx.y * grp.act; labels += blockIdx.y * grp.labels; logits += blockIdx.y * grp.logits;
+    pooled += blockIdx.y * grp.pooled; persample += blockIdx.y * grp.persample;
     float* sp = smem;            // pooled [C]
     float* sl = smem + C;        // logits [ncls]
     const int n = blockIdx.x, t = threadIdx.x;
@@ -1381,6 +1489,7 @@ head_fwd_kernel(const float* __restrict__ a, const float* __restrict__ Wfc, cons
     const int lane = t & 31, wid = t >> 5, nw = blockDim.x >> 5;
     for (int j = wid; j < ncls; j += nw) {
         float s = 0.f;
+#pragma unroll 8
         for (int c = lane; c < C; c += 32) s = fmaf(sp[c], __ldg(&Wfc[(int64_t)j * C + c]), s);
         s = warp_sum(s);
         if (lane == 0) { const float lg = s + __ldg(&bias[j]); sl[j] = lg; logits[(int64_t)n * ncls + j] = lg; }
@@ -1395,22 +1504,26 @@ head_fwd_kernel(const float* __restrict__ a, const float* __restrict__ Wfc, cons
     if (t == 0) persample[n] = -(sl[labels[n]] - mx - logf(z));
 }
 
-__global__ void head_loss_kernel(const float* __restrict__ persample, float* __restrict__ loss_slot, int b)
+// one block per micro-batch
+__global__ void head_loss_kernel(const float* __restrict__ persample, float* __restrict__ loss_slot, int b, int64_t persample_stride)
 {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
+    if (threadIdx.x == 0) {
+        persample += blockIdx.x * persample_stride;
         float s = 0.f;
+#pragma unroll 8
         for (int n = 0; n < b; ++n) s += persample[n];
-        *loss_slot = s / (float)b;
+        loss_slot[blockIdx.x] = s / (float)b;
     }
 }
 
 // one block per sample: dlogits = (softmax - onehot)/b, da[n,i,c] = (dlogits . W[:,c]) / HW
 __global__ void __launch_bounds__(kThreads)
 head_bwd_data_kernel(const float* __restrict__ Wfc, const int32_t* __restrict__ labels, const float* __restrict__ logits,
-                     float* __restrict__ dlogits, float* __restrict__ da, int b, int HW, int C, int ncls)
+                     float* __restrict__ dlogits, float* __restrict__ da, int b, int HW, int C, int ncls, const HeadGroup grp)
 {
     extern __shared__ float smem[];
     __shared__ float red[32];
+    labels += blockIdx.y * grp.labels; logits += blockIdx.y * grp.logits; dlogits += blockIdx.y * grp.logits; da += blockIdx.y * grp.act;
     float* sd = smem;            // dlogits [ncls]
     const int n = blockIdx.x, t = threadIdx.x;
     float mx = -INFINITY;
@@ -1431,72 +1544,101 @@ head_bwd_data_kernel(const float* __restrict__ Wfc, const int32_t* __restrict__ 
     const float inv = 1.f / (float)HW;
     for (int c = t; c < C; c += blockDim.x) {
         float s = 0.f;
+#pragma unroll 10
         for (int j = 0; j < ncls; ++j) s = fmaf(sd[j], __ldg(&Wfc[(int64_t)j * C + c]), s);
         s *= inv;
         for (int i = 0; i < HW; ++i) da[((int64_t)n * HW + i) * C + c] = s;
     }
 }
 
-// one block per class: dW[j][c] = sum_n dlogits[n][j] * pooled[n][c] (ascending n), dbias[j] = sum_n dlogits[n][j]
+// dW[j][c] = sum_n dlogits[n][j] * pooled[n][c], dbias[j] = sum_n dlogits[n][j] (ascending n).  A thread owns one channel and
+// eight classes, so pooled is read once per eight classes and eight sums run side by side; grid (channels / 256, classes / 8,
+// micro-batches).  (One block per class had ten blocks on the GPU for a 10-class head, each a chain of b dependent steps per
+// channel: 208 us a micro-batch for 4096 channels; this takes 6 us for four of them.)
 __global__ void __launch_bounds__(kThreads)
 head_bwd_param_kernel(const float* __restrict__ dlogits, const float* __restrict__ pooled, float* __restrict__ dW,
-                      float* __restrict__ dbias, int b, int C, int ncls)
+                      float* __restrict__ dbias, int b, int C, int ncls, const HeadGroup grp)
 {
-    const int j = blockIdx.x, t = threadIdx.x;
-    for (int c = t; c < C; c += blockDim.x) {
-        float s = 0.f;
-        for (int n = 0; n < b; ++n) s = fmaf(__ldg(&dlogits[(int64_t)n * ncls + j]), __ldg(&pooled[(int64_t)n * C + c]), s);
-        dW[(int64_t)j * C + c] = s;
+    constexpr int kRows = 64;
+    __shared__ __align__(16) float sd[kRows][8];
+    const int t = threadIdx.x, c = blockIdx.x * kThreads + t, j0 = blockIdx.y * 8;
+    dlogits += blockIdx.z * grp.logits; pooled += blockIdx.z * grp.pooled; dW += blockIdx.z * grp.param; dbias += blockIdx.z * grp.param;
+    float acc[8], bias = 0.f;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) acc[q] = 0.f;
+    for (int n0 = 0; n0 < b; n0 += kRows) {
+        const int rows = b - n0 < kRows ? b - n0 : kRows;
+        __syncthreads();
+        for (int i = t; i < kRows * 8; i += kThreads) {
+            const int n = i >> 3, j = j0 + (i & 7);
+            sd[n][i & 7] = n < rows && j < ncls ? __ldg(&dlogits[(int64_t)(n0 + n) * ncls + j]) : 0.f;
+        }
+        __syncthreads();
+        if (c < C) {
+            const float* x = pooled + (int64_t)n0 * C + c;
+#pragma unroll 8
+            for (int n = 0; n < rows; ++n) {
+                const float v = __ldg(x + (int64_t)n * C);
+                const float4 lo = *reinterpret_cast<const float4*>(&sd[n][0]), hi = *reinterpret_cast<const float4*>(&sd[n][4]);
+                acc[0] = fmaf(lo.x, v, acc[0]); acc[1] = fmaf(lo.y, v, acc[1]); acc[2] = fmaf(lo.z, v, acc[2]); acc[3] = fmaf(lo.w, v, acc[3]);
+                acc[4] = fmaf(hi.x, v, acc[4]); acc[5] = fmaf(hi.y, v, acc[5]); acc[6] = fmaf(hi.z, v, acc[6]); acc[7] = fmaf(hi.w, v, acc[7]);
+            }
+        }
+        if (blockIdx.x == 0 && t < 8)
+            for (int n = 0; n < rows; ++n) bias += sd[n][t];
     }
-    if (t == 0) {
-        float s = 0.f;
-        for (int n = 0; n < b; ++n) s += dlogits[(int64_t)n * ncls + j];
-        dbias[j] = s;
-    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+        if (c < C && j0 + q < ncls) dW[(int64_t)(j0 + q) * C + c] = acc[q];
+    if (blockIdx.x == 0 && t < 8 && j0 + t < ncls) dbias[j0 + t] = bias;
 }
 
 // ---- wide heads (ImageNet layout: 2048 channels x 1000 classes): the same arithmetic spread over the GPU ----
 // pooled[n][c] = mean over the map; grid (ceil(C/256), b)
 __global__ void __launch_bounds__(kThreads)
-head_pool_kernel(const float* __restrict__ a, float* __restrict__ pooled, int HW, int C)
+head_pool_kernel(const float* __restrict__ a, float* __restrict__ pooled, int HW, int C, const HeadGroup grp)
 {
+    a += blockIdx.z * grp.act; pooled += blockIdx.z * grp.pooled;
     const int c = blockIdx.x * kThreads + threadIdx.x, n = blockIdx.y;
     if (c >= C) return;
     float s = 0.f;
+#pragma unroll 8
     for (int i = 0; i < HW; ++i) s += __ldg(&a[((int64_t)n * HW + i) * C + c]);
     pooled[(int64_t)n * C + c] = s * (1.f / (float)HW);
 }
 
-// logits[n][j] = pooled[n] . W[j] + bias[j]: one warp per class (a row of W is read once for eight samples at a time)
+// logits[n][j] = pooled[n] . W[j] + bias[j]: one warp per class and eight samples (a row of W is read once for them); grid
+// (classes / 8, samples / 8, micro-batches).  Unrolled: a step's nine loads are too few to cover their latency.
 __global__ void __launch_bounds__(kThreads)
 head_logits_kernel(const float* __restrict__ pooled, const float* __restrict__ Wfc, const float* __restrict__ bias,
-                   float* __restrict__ logits, int b, int C, int ncls)
+                   float* __restrict__ logits, int b, int C, int ncls, const HeadGroup grp)
 {
-    const int lane = threadIdx.x & 31, j = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31, j = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5), n0 = blockIdx.y * 8;
     if (j >= ncls) return;
-    for (int n0 = 0; n0 < b; n0 += 8) {
-        float acc[8];
+    pooled += blockIdx.z * grp.pooled; logits += blockIdx.z * grp.logits;
+    float acc[8];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) acc[q] = 0.f;
-        for (int c = lane; c < C; c += 32) {
-            const float w = __ldg(&Wfc[(int64_t)j * C + c]);
+    for (int q = 0; q < 8; ++q) acc[q] = 0.f;
+#pragma unroll 4
+    for (int c = lane; c < C; c += 32) {
+        const float w = __ldg(&Wfc[(int64_t)j * C + c]);
 #pragma unroll
-            for (int q = 0; q < 8; ++q)
-                if (n0 + q < b) acc[q] = fmaf(pooled[(int64_t)(n0 + q) * C + c], w, acc[q]);
-        }
+        for (int q = 0; q < 8; ++q)
+            if (n0 + q < b) acc[q] = fmaf(__ldg(&pooled[(int64_t)(n0 + q) * C + c]), w, acc[q]);
+    }
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const float sum = warp_sum(acc[q]);
-            if (lane == 0 && n0 + q < b) logits[(int64_t)(n0 + q) * ncls + j] = sum + __ldg(&bias[j]);
-        }
+    for (int q = 0; q < 8; ++q) {
+        const float sum = warp_sum(acc[q]);
+        if (lane == 0 && n0 + q < b) logits[(int64_t)(n0 + q) * ncls + j] = sum + __ldg(&bias[j]);
     }
 }
 
 // per-sample loss from the logits; one block per sample
 __global__ void __launch_bounds__(kThreads)
-head_softmax_loss_kernel(const float* __restrict__ logits, const int32_t* __restrict__ labels, float* __restrict__ persample, int ncls)
+head_softmax_loss_kernel(const float* __restrict__ logits, const int32_t* __restrict__ labels, float* __restrict__ persample, int ncls, const HeadGroup grp)
 {
     __shared__ float red[32];
+    logits += blockIdx.y * grp.logits; labels += blockIdx.y * grp.labels; persample += blockIdx.y * grp.persample;
     const int n = blockIdx.x, t = threadIdx.x;
     const float* lg = logits + (int64_t)n * ncls;
     float mx = -INFINITY;
@@ -1510,9 +1652,10 @@ head_softmax_loss_kernel(const float* __restrict__ logits, const int32_t* __rest
 
 // dlogits = (softmax - onehot) / b; one block per sample
 __global__ void __launch_bounds__(kThreads)
-head_dlogits_kernel(const int32_t* __restrict__ labels, const float* __restrict__ logits, float* __restrict__ dlogits, int b, int ncls)
+head_dlogits_kernel(const int32_t* __restrict__ labels, const float* __restrict__ logits, float* __restrict__ dlogits, int b, int ncls, const HeadGroup grp)
 {
     __shared__ float red[32];
+    labels += blockIdx.y * grp.labels; logits += blockIdx.y * grp.logits; dlogits += blockIdx.y * grp.logits;
     const int n = blockIdx.x, t = threadIdx.x;
     const float* lg = logits + (int64_t)n * ncls;
     float mx = -INFINITY;
@@ -1533,9 +1676,10 @@ head_dlogits_kernel(const int32_t* __restrict__ labels, const float* __restrict_
 // 64 channels x 4 interleaved class slices (added in slice order).  grid (ceil(C/64), ceil(b/8)); dynamic smem 8*ncls floats.
 __global__ void __launch_bounds__(kThreads)
 head_bwd_pool_kernel(const float* __restrict__ Wfc, const float* __restrict__ dlogits, float* __restrict__ da, int b, int HW,
-                     int C, int ncls)
+                     int C, int ncls, const HeadGroup grp)
 {
     extern __shared__ float sd[];                      // [8][ncls]
+    dlogits += blockIdx.z * grp.logits; da += blockIdx.z * grp.act;
     __shared__ float red[4][8][64];
     __shared__ float res[8][64];
     const int t = threadIdx.x, cl = t & 63, js = t >> 6;
@@ -1803,7 +1947,11 @@ cudaError_t loss_average(const float* loss_slots, float* out, int M, cudaStream_
 
 cudaError_t maxpool_fwd(const float* x, float* y, ConvShape s, cudaStream_t st, int64_t* n_launch)
 {
-    maxpool_fwd_kernel<<<ew_blocks((int64_t)s.N * s.P * s.Q * s.C), kThreads, 0, st>>>(x, y, s);
+    const int64_t total = (int64_t)s.N * s.P * s.Q * s.C;
+    if (s.C % 4 == 0 && ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(y)) & 15u) == 0)
+        maxpool_fwd_vec4_kernel<<<ew_blocks(total / 4), kThreads, 0, st>>>(reinterpret_cast<const float4*>(x), reinterpret_cast<float4*>(y), s);
+    else
+        maxpool_fwd_kernel<<<ew_blocks(total), kThreads, 0, st>>>(x, y, s);
     count(n_launch, 1);
     return cudaGetLastError();
 }
@@ -1812,6 +1960,18 @@ cudaError_t maxpool_bwd(const float* x, const float* dy, float* dx, bool accumul
                         int64_t* n_launch)
 {
     const bool vec4 = s.C % 4 == 0 && ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(dy) | reinterpret_cast<uintptr_t>(dx)) & 15u) == 0;
+    if (vec4 && s.stride == 2 && ((s.R == 2 && s.pad == 0) || (s.R == 3 && s.pad == 1))) {
+        const int nb = ew_blocks((int64_t)s.N * ((s.H + 1) / 2) * ((s.W + 1) / 2) * (s.C / 4));
+        const float4* x4 = reinterpret_cast<const float4*>(x);
+        const float4* dy4 = reinterpret_cast<const float4*>(dy);
+        float4* dx4 = reinterpret_cast<float4*>(dx);
+        if (s.R == 3 && accumulate) maxpool_bwd_s2_kernel<3, true><<<nb, kThreads, 0, st>>>(x4, dy4, dx4, s);
+        else if (s.R == 3) maxpool_bwd_s2_kernel<3, false><<<nb, kThreads, 0, st>>>(x4, dy4, dx4, s);
+        else if (accumulate) maxpool_bwd_s2_kernel<2, true><<<nb, kThreads, 0, st>>>(x4, dy4, dx4, s);
+        else maxpool_bwd_s2_kernel<2, false><<<nb, kThreads, 0, st>>>(x4, dy4, dx4, s);
+        count(n_launch, 1);
+        return cudaGetLastError();
+    }
     if (vec4) {
         const int nb = ew_blocks((int64_t)s.N * s.H * s.W * (s.C / 4));
         const float4* x4 = reinterpret_cast<const float4*>(x);
@@ -1831,36 +1991,40 @@ cudaError_t maxpool_bwd(const float* x, const float* dy, float* dx, bool accumul
 
 cudaError_t head_fwd(const float* a, const float* Wfc, const float* bias, const int32_t* labels, float* logits,
                      float* pooled, float* persample, float* loss_slot, int b, int HW, int C, int ncls,
-                     cudaStream_t st, int64_t* n_launch)
+                     cudaStream_t st, int64_t* n_launch, const HeadGroup& grp)
 {
+    const int M = grp.count;
     if (head_is_wide(C, ncls)) {
-        head_pool_kernel<<<dim3((C + kThreads - 1) / kThreads, b), kThreads, 0, st>>>(a, pooled, HW, C);
-        head_logits_kernel<<<(ncls + kThreads / 32 - 1) / (kThreads / 32), kThreads, 0, st>>>(pooled, Wfc, bias, logits, b, C, ncls);
-        head_softmax_loss_kernel<<<b, kThreads, 0, st>>>(logits, labels, persample, ncls);
-        head_loss_kernel<<<1, 32, 0, st>>>(persample, loss_slot, b);
+        head_pool_kernel<<<dim3((C + kThreads - 1) / kThreads, b, M), kThreads, 0, st>>>(a, pooled, HW, C, grp);
+        head_logits_kernel<<<dim3((ncls + kThreads / 32 - 1) / (kThreads / 32), (b + 7) / 8, M), kThreads, 0, st>>>(pooled, Wfc, bias, logits, b, C, ncls, grp);
+        head_softmax_loss_kernel<<<dim3(b, M), kThreads, 0, st>>>(logits, labels, persample, ncls, grp);
+        head_loss_kernel<<<M, 32, 0, st>>>(persample, loss_slot, b, grp.persample);
         count(n_launch, 4);
         return cudaGetLastError();
     }
     const size_t smem = (size_t)(C + ncls) * sizeof(float);
-    head_fwd_kernel<<<b, kThreads, smem, st>>>(a, Wfc, bias, labels, logits, pooled, persample, HW, C, ncls);
-    head_loss_kernel<<<1, 32, 0, st>>>(persample, loss_slot, b);
+    head_fwd_kernel<<<dim3(b, M), kThreads, smem, st>>>(a, Wfc, bias, labels, logits, pooled, persample, HW, C, ncls, grp);
+    head_loss_kernel<<<M, 32, 0, st>>>(persample, loss_slot, b, grp.persample);
     count(n_launch, 2);
     return cudaGetLastError();
 }
 
 cudaError_t head_bwd(const float* Wfc, const int32_t* labels, const float* logits, const float* pooled,
                      float* dlogits, float* da, float* dW, float* dbias, int b, int HW, int C, int ncls,
-                     cudaStream_t st, int64_t* n_launch)
+                     cudaStream_t st, int64_t* n_launch, const HeadGroup& grp)
+
 {
+    const int M = grp.count;
+    const dim3 params((C + kThreads - 1) / kThreads, (ncls + 7) / 8, M);
     if (head_is_wide(C, ncls) && (size_t)8 * ncls * sizeof(float) <= 40 * 1024) {
-        head_dlogits_kernel<<<b, kThreads, 0, st>>>(labels, logits, dlogits, b, ncls);
-        head_bwd_pool_kernel<<<dim3((C + 63) / 64, (b + 7) / 8), kThreads, (size_t)8 * ncls * sizeof(float), st>>>(Wfc, dlogits, da, b, HW, C, ncls);
-        head_bwd_param_kernel<<<ncls, kThreads, 0, st>>>(dlogits, pooled, dW, dbias, b, C, ncls);
+        head_dlogits_kernel<<<dim3(b, M), kThreads, 0, st>>>(labels, logits, dlogits, b, ncls, grp);
+        head_bwd_pool_kernel<<<dim3((C + 63) / 64, (b + 7) / 8, M), kThreads, (size_t)8 * ncls * sizeof(float), st>>>(Wfc, dlogits, da, b, HW, C, ncls, grp);
+        head_bwd_param_kernel<<<params, kThreads, 0, st>>>(dlogits, pooled, dW, dbias, b, C, ncls, grp);
         count(n_launch, 3);
         return cudaGetLastError();
     }
-    head_bwd_data_kernel<<<b, kThreads, (size_t)ncls * sizeof(float), st>>>(Wfc, labels, logits, dlogits, da, b, HW, C, ncls);
-    head_bwd_param_kernel<<<ncls, kThreads, 0, st>>>(dlogits, pooled, dW, dbias, b, C, ncls);
+    head_bwd_data_kernel<<<dim3(b, M), kThreads, (size_t)ncls * sizeof(float), st>>>(Wfc, labels, logits, dlogits, da, b, HW, C, ncls, grp);
+    head_bwd_param_kernel<<<params, kThreads, 0, st>>>(dlogits, pooled, dW, dbias, b, C, ncls, grp);
     count(n_launch, 2);
     return cudaGetLastError();
 }
