@@ -537,7 +537,7 @@ void build_memory_plan(hpf_model* mdl)
         for (int i = mdl->part_lo[p]; i < mdl->part_hi[p]; ++i)
             if (mdl->ops[i].op.kind == HPF_OP_CONV) {
                 const ConvShape s = conv_shape_of(mdl, i);
-                cv = std::max(cv, std::max(conv_simt_scratch_bytes(s), conv_tc_scratch_bytes(s, M)));
+                cv = std::max(cv, std::max(conv_simt_scratch_bytes(s, M), conv_tc_scratch_bytes(s, M)));
             }
         mdl->conv_scratch_ms[p] = align_up(cv, 256);
         mdl->conv_scratch_off[p] = take(mdl->conv_scratch_ms[p] * M);
@@ -748,9 +748,8 @@ int backward_op(hpf_model* mdl, int i, int m, int g, cudaStream_t st, int sl)
         if (mdl->use_tc[PASS_WGRAD][i]) {
             CU(conv_tc_launch(&mdl->wgrad_plan[i], mdl->status(), wst, &mdl->launches, m, g));
         } else {
-            for (int k = m; k < m + g; ++k)
-                CU(conv_wgrad_simt(src_act(mdl, q.src0, k), mdl->grad(i, k), mdl->gslots + (int64_t)k * mdl->G + o.w_off, s,
-                                   mdl->ws + mdl->conv_scratch_off[o.part] + k * mdl->conv_scratch_ms[o.part], wst, &mdl->launches));
+            CU(conv_wgrad_simt(in0, dout, slot + o.w_off, s, mdl->ws + mdl->conv_scratch_off[o.part] + m * mdl->conv_scratch_ms[o.part], wst, &mdl->launches,
+                               mdl->M, g, (long long)(mdl->conv_scratch_ms[o.part] / sizeof(float)), mdl->G));
         }
         if (q.src0 >= 0) {
             if (mdl->use_pipe[PASS_DGRAD][i]) CU(conv_pipe_launch(&mdl->pipe_plan[PASS_DGRAD][i], m, g, false, mdl->status(), st, &mdl->launches));
