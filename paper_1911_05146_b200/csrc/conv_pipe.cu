@@ -70,8 +70,9 @@ struct PipeScalars {
     int bn_units;
     float bn_eps;
     double bn_inv_rows;
-    // BN moments of the output
+    // BN moments of the output; bn_x (data gradient): the sums of a BN+ReLU's backward instead, whose input bn_x is laid out like out
     float* st_partials;
+    const float* bn_x;
     // split K
     char* sk_base;                                    // per micro-batch: tickets, then partial tiles
     long long sk_ms;                                  // bytes between micro-batches
@@ -278,6 +279,12 @@ struct EmitArgs {
     int mom_pitch;
     bool accumulate, ok;
     int zero_fill, dense_h, dense_w;
+    // not null: `extra` is the input x of a BN+ReLU whose output gradient this is: it is not added; the sums are those of
+    // dz = dy where the activation was positive, and of dz * xhat
+    const float* bn_mean;        // this column group's: mean, rstd (bn_c floats further on), gamma, beta
+    const float* bn_gamma;
+    const float* bn_beta;
+    int bn_c;
 };
 
 // The residuals of four row steps, beginning with step b.
@@ -298,13 +305,18 @@ __device__ __forceinline__ void emit_residuals(const EmitArgs& a, int ro, int la
 // 200 KB with specialised copies: 4000-8000 clocks for the first tile of a launch).
 // Moments are taken about a value of the column: sums of x and x*x themselves would cancel for a channel whose mean is large
 // against its spread.
+template <bool BNB>
 __device__ __forceinline__ void emit_rows(const EmitArgs& a, int ro, int fill, int lane, int lsh, bool have_shift, float4* e)
 {
     const int cq = lane & ((1 << lsh) - 1), rq = lane >> lsh, rstep = 32 >> lsh, steps = 1 << lsh;
     const unsigned int who = __ballot_sync(0xffffffffu, ro >= 0);        // lane = row here
     float4 k = make_float4(0.f, 0.f, 0.f, 0.f), sd = k, sq = k;
     const bool moments = a.moments != nullptr && who != 0u;
-    if (moments) {
+    float4 rs = k, g = k, bt = k;
+    if (BNB) {
+        k = __ldg(reinterpret_cast<const float4*>(a.bn_mean + 4 * cq)); rs = __ldg(reinterpret_cast<const float4*>(a.bn_mean + a.bn_c + 4 * cq));
+        g = __ldg(reinterpret_cast<const float4*>(a.bn_gamma + 4 * cq)); bt = __ldg(reinterpret_cast<const float4*>(a.bn_beta + 4 * cq));
+    } else if (moments) {
         if (have_shift) k = *reinterpret_cast<const float4*>(a.moments + 4 * cq);
         else {
             const int r0 = __ffs(who) - 1, so = __shfl_sync(0xffffffffu, ro, r0);
@@ -322,7 +334,18 @@ __device__ __forceinline__ void emit_rows(const EmitArgs& a, int ro, int fill, i
             so[i] = __shfl_sync(0xffffffffu, ro, r);
             v[i] = a.patch[r * 8 + (cq ^ (r & 7))];
         }
-        if (a.extra) {
+        if (BNB) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const bool real = so[i] >= 0;
+                const float x0 = (e[i].x - k.x) * rs.x, x1 = (e[i].y - k.y) * rs.y, x2 = (e[i].z - k.z) * rs.z, x3 = (e[i].w - k.w) * rs.w;
+                const float d0 = real && fmaf(g.x, x0, bt.x) > 0.f ? v[i].x : 0.f, d1 = real && fmaf(g.y, x1, bt.y) > 0.f ? v[i].y : 0.f,
+                            d2 = real && fmaf(g.z, x2, bt.z) > 0.f ? v[i].z : 0.f, d3 = real && fmaf(g.w, x3, bt.w) > 0.f ? v[i].w : 0.f;
+                sd.x += d0; sd.y += d1; sd.z += d2; sd.w += d3;
+                sq.x = fmaf(d0, x0, sq.x); sq.y = fmaf(d1, x1, sq.y); sq.z = fmaf(d2, x2, sq.z); sq.w = fmaf(d3, x3, sq.w);
+            }
+            if (b + 4 < steps) emit_residuals(a, ro, lane, lsh, b + 4, e);
+        } else if (a.extra) {
 #pragma unroll
             for (int i = 0; i < 4; ++i) v[i] = add4(v[i], e[i]);
             if (b + 4 < steps) emit_residuals(a, ro, lane, lsh, b + 4, e);
@@ -337,7 +360,7 @@ __device__ __forceinline__ void emit_rows(const EmitArgs& a, int ro, int fill, i
 #pragma unroll
             for (int i = 0; i < 4; ++i) if (so[i] >= 0) *reinterpret_cast<float4*>(out + so[i]) = v[i];
         }
-        if (moments) {
+        if (moments && !BNB) {
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const bool real = so[i] >= 0;
@@ -493,8 +516,9 @@ __device__ __forceinline__ void pipe_init_barriers(const PipeScalars& p, PipeSha
 
 // The work of one CTA (number bid of nblk) of a launch: the barriers are initialised, tensor memory is allocated.
 // FLAT: the operand's positions and the output's pixels are the same consecutive rows (1x1 windows without a stride).
+// BNB: a data gradient that forms the sums of a BN+ReLU's backward.
 // CELL: inside the persistent cell kernel, which keeps its tensor memory and has no successor to trigger.
-template <bool BN_IN, bool FLAT, bool CELL>
+template <bool BN_IN, bool FLAT, bool BNB, bool CELL>
 __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars& p, PipeShared& sh, uint8_t* smem, const uint32_t tmem_base,
                                          const int m_first, const int m_count, const int bid, const int nblk)
 {
@@ -779,8 +803,10 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
             if (!alternate || turn == half) {
             const int nt = u.tiles(p);
             float* out = p.out + (long long)u.m * p.out_ms + co0;
-            const float* extra = p.extra ? p.extra + (long long)u.m * p.out_ms + co0 : nullptr;
-            EmitArgs ea{out, extra, patch, nullptr, n_chunk, p.accumulate != 0, true, p.zero_fill, p.dense_h, p.dense_w};
+            const float* addend = BNB ? p.bn_x : p.extra;
+            const float* extra = addend ? addend + (long long)u.m * p.out_ms + co0 : nullptr;
+            const float* bnb = BNB ? p.bn_stats + (long long)u.m * 2 * C_out + co0 : nullptr;
+            EmitArgs ea{out, extra, patch, nullptr, n_chunk, p.accumulate != 0, true, p.zero_fill, p.dense_h, p.dense_w, nullptr, nullptr, nullptr, C_out};
             // this lane's row of a tile, and which neighbours of a strided data gradient's sample get zeros
             int ro = -1, fill = 0;
             auto place = [&](int t) {
@@ -855,6 +881,7 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
                 for (int g = g_first, gi = 0; g < groups; g += g_step, ++gi) {
                     const int left = n_chunk - 32 * g, lsh = left >= 32 ? 3 : 2;
                     ea.out = out + 32 * g;
+                    if (BNB) { ea.bn_mean = bnb + 32 * g; ea.bn_gamma = p.bn_gamma + co0 + 32 * g; ea.bn_beta = p.bn_beta + co0 + 32 * g; }
                     if (extra) {
                         ea.extra = extra + 32 * g;
                         if (t > t_first || gi > 0) emit_residuals(ea, ro, lane, lsh, 0, e);
@@ -881,7 +908,7 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
                         for (int j = 0; j < 4; ++j) patch[lane * 8 + ((4 * h + j) ^ (lane & 7))] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
                     }
                     __syncwarp();
-                    emit_rows(ea, ro, fill, lane, lsh, have, e);
+                    emit_rows<BNB>(ea, ro, fill, lane, lsh, have, e);
                 }
                 if (rows) have = true;
             }
@@ -900,7 +927,15 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
                 if (lane == 0 && (whole || half == 0)) counts[part] = (float)count;
                 count = 0; have = false;
                 epi_sync();
-                if (tid < n_chunk) {
+                if (BNB && tid < n_chunk) {
+                    float sum = 0.f, sq = 0.f;
+                    const float* c3 = contrib + tid;
+#pragma unroll 1
+                    for (int w = 0; w < parts; ++w, c3 += 3 * n_chunk)
+                        if (counts[w] > 0.f) { sum += c3[n_chunk]; sq += c3[2 * n_chunk]; }
+                    float* row = p.st_partials + (size_t)u.m * partial_floats(p.blocks_per_m, C_out) + (size_t)(u.ul / p.unit_block) * 2 * C_out + co0 + tid;
+                    if (ok) { row[0] = sum; row[C_out] = sq; }
+                } else if (tid < n_chunk) {
                     // parts about their own shifts k_w: sum and squares about the first one's,
                     //   sum (x - k0) = sum_w [d_w + n_w e],  sum (x - k0)^2 = sum_w [q_w + e (2 d_w + n_w e)],  e = k_w - k0
                     float N = 0.f, k0 = 0.f, sum = 0.f, sq = 0.f;
@@ -947,7 +982,7 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
     __syncthreads();
 }
 
-template <bool BN_IN, bool FLAT>
+template <bool BN_IN, bool FLAT, bool BNB>
 __global__ void __launch_bounds__(kPipeThreads, 1) conv_pipe_kernel(const __grid_constant__ PipeParams gp, const int m_first, const int m_count)
 {
     const PipeScalars& p = gp.s;
@@ -973,7 +1008,7 @@ __global__ void __launch_bounds__(kPipeThreads, 1) conv_pipe_kernel(const __grid
     // take the columns this one needs and wait for this one to finish.
     if (!p.pdl_late) pdl_launch_dependents();
     const uint32_t tmem_base = sh.tmem_slot;
-    pipe_cta<BN_IN, FLAT, false>(gp, p, sh, smem, tmem_base, m_first, m_count, (int)blockIdx.x, (int)gridDim.x);
+    pipe_cta<BN_IN, FLAT, BNB, false>(gp, p, sh, smem, tmem_base, m_first, m_count, (int)blockIdx.x, (int)gridDim.x);
     if (warp_index() == 0) tmem_dealloc(tmem_base, p.tmem_cols);
 }
 
@@ -1076,11 +1111,11 @@ __global__ void __launch_bounds__(kPipeThreads, 1) conv_pipe_cell_kernel(const _
             __syncthreads();
             tc_fence_after();
             if (bn_in) {
-                if (flat) pipe_cta<true, true, true>(gp, p, sh, smem, tmem_base, m_first, m_count, v, V);
-                else pipe_cta<true, false, true>(gp, p, sh, smem, tmem_base, m_first, m_count, v, V);
+                if (flat) pipe_cta<true, true, false, true>(gp, p, sh, smem, tmem_base, m_first, m_count, v, V);
+                else pipe_cta<true, false, false, true>(gp, p, sh, smem, tmem_base, m_first, m_count, v, V);
             } else {
-                if (flat) pipe_cta<false, true, true>(gp, p, sh, smem, tmem_base, m_first, m_count, v, V);
-                else pipe_cta<false, false, true>(gp, p, sh, smem, tmem_base, m_first, m_count, v, V);
+                if (flat) pipe_cta<false, true, false, true>(gp, p, sh, smem, tmem_base, m_first, m_count, v, V);
+                else pipe_cta<false, false, false, true>(gp, p, sh, smem, tmem_base, m_first, m_count, v, V);
             }
             if (sh.abort_flag) { if (tid == 0) cell_stop = 1; break; }
         }
@@ -1190,8 +1225,8 @@ bool conv_pipe_geom(const ConvShape& s, int pass, int passes, int M, ConvPipeGeo
     const int taps = s.R * s.R, chunks = v.c_in / 16, n = g->n_chunk;
     g->b_tap_bytes = (unsigned int)(three ? 2 : 1) * (unsigned int)n * 64u;
     const unsigned int all_b = g->b_tap_bytes * (unsigned int)(taps * chunks);
-    // (the data gradient forms no moments and applies no BN)
-    const unsigned int fixed = kEpiWarps * 4096u + (pass == PASS_FWD ? stat_bytes(n) + bn_bytes(v.c_in <= 512 ? v.c_in : 0) : 0u);
+    // (the data gradient applies no BN)
+    const unsigned int fixed = kEpiWarps * 4096u + stat_bytes(n) + (pass == PASS_FWD ? bn_bytes(v.c_in <= 512 ? v.c_in : 0) : 0u);
     // Tiles per unit, stacked weights (hi*hi and hi*lo from one MMA over [B_hi; B_lo]), accumulator sets and the two rings:
     // the combination with the least modelled time for the busiest CTA, from clocks measured stage by stage.  A chunk takes
     // the longest of: its MMAs (K = 8; at 128 columns an unstacked MMA reads 128 bytes of shared memory per clock, all there
@@ -1288,7 +1323,8 @@ cudaError_t conv_pipe_init()
     static bool done = false;
     if (done) return cudaSuccess;
     cudaError_t e = cudaSuccess;
-    for (auto kernel : {conv_pipe_kernel<false, false>, conv_pipe_kernel<false, true>, conv_pipe_kernel<true, false>, conv_pipe_kernel<true, true>})
+    for (auto kernel : {conv_pipe_kernel<false, false, false>, conv_pipe_kernel<false, true, false>, conv_pipe_kernel<true, false, false>, conv_pipe_kernel<true, true, false>,
+                        conv_pipe_kernel<false, false, true>, conv_pipe_kernel<false, true, true>})
         if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPipeSmem + 1024);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(conv_pipe_cell_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPipeSmem + 1024);
     done = e == cudaSuccess;
@@ -1369,12 +1405,17 @@ cudaError_t conv_pipe_prepare(ConvPipePlan* plan, const ConvShape& s, int pass, 
     p.off_b = a_bytes;
     p.off_stage = (p.off_b + (unsigned int)g.b_stages * g.b_stage_bytes + 127u) & ~127u;
     p.off_stat = p.off_stage + kEpiWarps * 4096u;
-    p.off_red = p.off_stat + (pass == PASS_FWD ? stat_bytes(g.n_chunk) : 0u);
+    p.off_red = p.off_stat + stat_bytes(g.n_chunk);
     p.off_bn = p.off_red + 4 * kSplitThreads * 16;
     L->smem = p.off_red + 1024;
     if (bn && bn->out_partials) {
         if (!conv_pipe_can_fuse_bn_output(g)) return cudaErrorNotSupported;
         p.st_partials = bn->out_partials;
+    }
+    if (bn && bn->bwd_partials) {
+        if (pass != PASS_DGRAD || s.stride != 1 || extra || accumulate || !conv_pipe_can_fuse_bn_output(g)) return cudaErrorNotSupported;
+        p.st_partials = bn->bwd_partials; p.bn_x = bn->bwd_x; p.bn_stats = const_cast<float*>(bn->bwd_stats);
+        p.bn_gamma = bn->in_gamma; p.bn_beta = bn->in_beta;
     }
     if (bn && bn->in_partials) {
         if (pass != PASS_FWD || !conv_pipe_can_fuse_bn_input(s) || bn->in_blocks < 1) return cudaErrorNotSupported;
@@ -1406,8 +1447,9 @@ cudaError_t conv_pipe_launch(const ConvPipePlan* plan, int m_first, int m_count,
     if (per_slice < 1) per_slice = 1;
     if (per_slice > tasks) per_slice = tasks;
     const bool flat = p.flat && p.zero_fill == 1;
-    auto kernel = L.bn_in ? (flat ? conv_pipe_kernel<true, true> : conv_pipe_kernel<true, false>)
-                          : (flat ? conv_pipe_kernel<false, true> : conv_pipe_kernel<false, false>);
+    auto kernel = L.bn_in ? (flat ? conv_pipe_kernel<true, true, false> : conv_pipe_kernel<true, false, false>)
+                          : (p.bn_x ? (flat ? conv_pipe_kernel<false, true, true> : conv_pipe_kernel<false, false, true>)
+                                    : (flat ? conv_pipe_kernel<false, true, false> : conv_pipe_kernel<false, false, false>));
     launch_pdl(kernel, dim3(per_slice * p.slices), dim3(kPipeThreads), L.smem, st, L.p, m_first, m_count);
     if (n_launch) ++*n_launch;
     return cudaGetLastError();

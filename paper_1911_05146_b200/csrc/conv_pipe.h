@@ -30,6 +30,9 @@ bool conv_pipe_geom(const ConvShape& s, int pass, int passes, int M, ConvPipeGeo
 //   in_partials: the input x is the input of a BN+ReLU that only this convolution reads: it merges the producer's moments
 //     (in_blocks rows), applies y = relu(gamma*(x-mean)*rstd+beta) to its operand, stores y (in_y) and the statistics
 //     (in_stats: mean[C], rstd[C] per micro-batch) for the backward pass.
+//   bwd_partials (data gradient): the output is the gradient of a BN+ReLU's output that no other kernel adds to: per block of
+//     units and channel the sums of dz and of dz * xhat, [blocks_per_m][2][channels] floats in conv_pipe_partial_floats() per
+//     micro-batch, from the BN's input (bwd_x), statistics (bwd_stats) and parameters (in_gamma, in_beta).
 struct ConvPipeBn {
     float* out_partials = nullptr;
     const float* in_partials = nullptr;
@@ -39,6 +42,9 @@ struct ConvPipeBn {
     float* in_stats = nullptr;
     float* in_y = nullptr;
     float in_eps = 0.f;
+    float* bwd_partials = nullptr;
+    const float* bwd_x = nullptr;
+    const float* bwd_stats = nullptr;
 };
 size_t conv_pipe_partial_floats(int blocks_per_m, int channels);
 bool conv_pipe_can_fuse_bn_output(const ConvPipeGeom& g);

@@ -92,6 +92,8 @@ struct hpf_model {
     std::vector<int> bn_fwd_from;              // BN -> conv whose forward kernel also produces the statistics of the BN (its input), or -1
     std::vector<int> conv_fwd_bn;              // the inverse map
     std::vector<int> bn_into, conv_in_bn;      // BN -> the convolution that applies it to its own input operand (no BN kernel), and the inverse
+    std::vector<int> bn_bwd_from, conv_bwd_bn;  // BN+ReLU -> the convolution whose data gradient also forms the sums of its backward, or -1, and the inverse map
+    std::vector<size_t> bn_sums_off;           // where it leaves them, all micro-batches
     std::vector<size_t> bn_moments_off;        // BN -> per-unit moments of its input left by the producing convolution, all micro-batches
     // Forward / data-gradient launches of networks with batch norm are the pipelined kernel's wherever it covers the shape.
     // Without batch norm nothing re-scales the activations: the last bits of a convolution's sum move ReLU and max-pool
@@ -434,10 +436,22 @@ void build_kernel_plan(hpf_model* mdl)
     mdl->bn_fwd_from.assign(n, -1);
     mdl->conv_fwd_bn.assign(n, -1);
     mdl->bn_into.assign(n, -1); mdl->conv_in_bn.assign(n, -1);
+    mdl->bn_bwd_from.assign(n, -1); mdl->conv_bwd_bn.assign(n, -1);
     if (!(mdl->opt_fuse_bn & 1)) return;
     for (int j = 0; j < n; ++j) {
         const OpInfo& bn = mdl->ops[j];
         if (bn.op.kind != HPF_OP_BNRELU) continue;
+        // Backward: the only kernel that writes the gradient of the BN's output forms its sums where the BN would read
+        // everything twice.  (A BN that one launch of clusters handles from registers is faster left alone: the sums cost the
+        // data gradient's write-out about a microsecond of latency, resnet11 took 395 us instead of 355.)
+        if (bn.consumers.size() == 1 && !(mdl->opt_bn_cluster && bn_bwd_is_one_launch((int64_t)mdl->b * bn.H * bn.W, bn.C))) {
+            const int i = bn.consumers[0];
+            const OpInfo& c = mdl->ops[i];
+            if (i == j + 1 && c.op.kind == HPF_OP_CONV && c.op.stride == 1 && bn.C <= 2048 && c.part == bn.part && mdl->use_pipe[PASS_DGRAD][i] && !mdl->edge0[i].accumulate &&
+                mdl->edge0[i].addend < 0 && conv_pipe_can_fuse_bn_output(mdl->pipe_geom[PASS_DGRAD][i])) {
+                mdl->bn_bwd_from[j] = i; mdl->conv_bwd_bn[i] = j;
+            }
+        }
         // forward: the kernel that writes the BN's input
         int t = bn.op.src0, prod = -1;
         if (mdl->ops[t].op.kind == HPF_OP_CONV && mdl->fused_into[t] < 0) prod = t;
@@ -527,6 +541,10 @@ void build_memory_plan(hpf_model* mdl)
     mdl->zero_hi = at;
     build_cell_runs(mdl);
     for (auto& run : mdl->cell_runs) run.ops_off = take(conv_pipe_cell_op_bytes() * run.convs.size());
+    mdl->bn_sums_off.assign(n, 0);
+    for (int j = 0; j < n; ++j)
+        if (mdl->bn_bwd_from[j] >= 0)
+            mdl->bn_sums_off[j] = take(sizeof(float) * M * conv_pipe_partial_floats(mdl->pipe_geom[PASS_DGRAD][mdl->bn_bwd_from[j]].blocks_per_m, mdl->ops[j].C));
     mdl->bn_moments_off.assign(n, 0);
     for (int j = 0; j < n; ++j)
         if (mdl->bn_fwd_from[j] >= 0)
@@ -760,6 +778,13 @@ int backward_op(hpf_model* mdl, int i, int m, int g, cudaStream_t st, int sl)
     }
     case HPF_OP_BNRELU:
     case HPF_OP_BN:
+        if (mdl->bn_bwd_from[i] >= 0) {
+            const int blocks = mdl->pipe_geom[PASS_DGRAD][mdl->bn_bwd_from[i]].blocks_per_m;
+            const int64_t ms = (int64_t)conv_pipe_partial_floats(blocks, o.C);
+            CU(bnrelu_bwd_apply(in0, dout, mdl->params + o.w_off, mdl->params + o.b_off, mdl->stats(i, m), reinterpret_cast<const float*>(mdl->ws + mdl->bn_sums_off[i]) + m * ms,
+                                blocks, ms, mdl->grad(q.src0, m), addend, e.accumulate != 0, slot + o.w_off, slot + o.b_off, rows, o.C, st, &mdl->launches, grp));
+            break;
+        }
         CU(bnrelu_bwd(in0, dout, mdl->params + o.w_off, mdl->params + o.b_off, mdl->stats(i, m), mdl->grad(q.src0, m), addend,
                       e.accumulate != 0, slot + o.w_off, slot + o.b_off, rows, o.C, bn_scratch, st, &mdl->launches, q.kind == HPF_OP_BNRELU, true, grp));
         break;
@@ -1294,10 +1319,18 @@ int hpf_bind(hpf_model* mdl, float* d_params, float* d_grad_slots, float* d_grad
                 }
                 first_done[p] = 1;
             }
+            ConvPipeBn sums;
+            if (mdl->conv_bwd_bn[i] >= 0) {
+                const int jb = mdl->conv_bwd_bn[i];
+                const OpInfo& b = mdl->ops[jb];
+                sums.bwd_partials = reinterpret_cast<float*>(mdl->ws + mdl->bn_sums_off[jb]);
+                sums.bwd_x = mdl->act(b.op.src0, 0); sums.bwd_stats = mdl->stats(jb, 0);
+                sums.in_gamma = mdl->params + b.w_off; sums.in_beta = mdl->params + b.b_off;
+            }
             if (mdl->use_pipe[PASS_DGRAD][i])
                 CU(conv_pipe_prepare(&mdl->pipe_plan[PASS_DGRAD][i], s, PASS_DGRAD, passes, M, mdl->grad(i, 0), wp + 2 * G + o.w_off,
                                      wp + 3 * G + o.w_off, mdl->grad(src, 0), ed.addend >= 0 ? mdl->grad(ed.addend, 0) : nullptr,
-                                     ed.accumulate != 0, nullptr, mdl->ws + mdl->splitk_bwd_off[p], mdl->splitk_bytes[p], true));
+                                     ed.accumulate != 0, &sums, mdl->ws + mdl->splitk_bwd_off[p], mdl->splitk_bytes[p], true));
             else if (mdl->use_tc[PASS_DGRAD][i]) {
                 tile.splitk = mdl->splitk_bytes[p] ? mdl->ws + mdl->splitk_bwd_off[p] : nullptr;
                 CU(conv_tc_prepare(&mdl->tile_plan[PASS_DGRAD][i], s, PASS_DGRAD, passes, mdl->grad(i, 0), nullptr, wp + 2 * G + o.w_off, wp + 3 * G + o.w_off,

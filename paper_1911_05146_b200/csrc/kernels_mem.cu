@@ -375,6 +375,83 @@ bn_apply_bwd_kernel(const float4* __restrict__ x, const float4* __restrict__ dy,
     }
 }
 
+// BN+ReLU backward after a data gradient that left the sums of dz and dz * xhat per block of its work (`sums`: n_sums rows of
+// [2][C]): every block adds the few rows in order (fp64), then writes its rows of dx.  One read of x and dy instead of two, and one
+// launch instead of a reduction and this, or instead of a cluster's exchange.  What bounds it is memory: grids of a few
+// blocks per SM over all micro-batches, since every block adds the same rows first.
+template <bool ADDEND, bool ACCUM>
+__global__ void __launch_bounds__(kBnThreads)
+bn_apply_sums_bwd_kernel(const float4* __restrict__ x, const float4* __restrict__ dy, const float* __restrict__ gamma,
+                         const float* __restrict__ beta, const float* __restrict__ stats, const float* __restrict__ sums, int n_sums,
+                         int64_t sums_ms, float* __restrict__ dgamma, float* __restrict__ dbeta, const float4* __restrict__ addend,
+                         float4* __restrict__ dx, int64_t rows, int C, int cgt, int rl, int passes, int64_t rows_per_blk, const BnGroup grp)
+{
+    extern __shared__ float coef[];                    // [2][C]
+    __shared__ double red[kBnThreads * 4];
+    {
+        const int64_t gm = blockIdx.y;
+        x += gm * grp.x / 4; dy += gm * grp.x / 4; dx += gm * grp.x / 4; stats += gm * grp.stats; sums += gm * sums_ms;
+        dgamma += gm * grp.param; dbeta += gm * grp.param;
+        if (ADDEND) addend += gm * grp.x / 4;
+    }
+    pdl_launch_dependents();
+    pdl_wait();
+    const int t = threadIdx.x, cols = C / 2;           // float4 columns of a row of sums
+    const double inv_rows = 1.0 / (double)rows;
+    for (int c0 = 0; c0 < cols; c0 += kBnThreads) {
+        const int width = cols - c0 < kBnThreads ? cols - c0 : kBnThreads, L = kBnThreads / width;
+        const int ln = t / width, col = c0 + t - ln * width;
+        double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
+        if (ln < L) {
+#pragma unroll 4
+            for (int k = ln; k < n_sums; k += L) {
+                const float4 v = __ldcg(reinterpret_cast<const float4*>(sums + (int64_t)k * 2 * C) + col);
+                a0 += v.x; a1 += v.y; a2 += v.z; a3 += v.w;
+            }
+        }
+        red[4 * t] = a0; red[4 * t + 1] = a1; red[4 * t + 2] = a2; red[4 * t + 3] = a3;
+        __syncthreads();
+        for (int c = t; c < 4 * width; c += kBnThreads) {
+            double a = 0.0;
+            for (int l = 0; l < L; ++l) a += red[4 * l * width + c];
+            const int at = 4 * c0 + c;                 // below C: sum of dz, from C on: sum of dz * xhat
+            coef[at] = (float)(a * inv_rows);
+            if (blockIdx.x == 0) { if (at < C) dbeta[at] = (float)a; else dgamma[at - C] = (float)a; }
+        }
+        __syncthreads();
+    }
+    const int cg_total = C / 4, my_rl = t / cgt, my_cg = t % cgt;
+    const int64_t r0 = (int64_t)blockIdx.x * rows_per_blk;
+    const int64_t r1 = r0 + rows_per_blk < rows ? r0 + rows_per_blk : rows;
+    if (my_rl >= rl) return;
+    for (int pass = 0; pass < passes; ++pass) {
+        const int cg = pass * cgt + my_cg;
+        if (cg >= cg_total) continue;
+        const float4 mu = __ldg(reinterpret_cast<const float4*>(stats) + cg);
+        const float4 rs = __ldg(reinterpret_cast<const float4*>(stats + C) + cg);
+        const float4 g = __ldg(reinterpret_cast<const float4*>(gamma) + cg);
+        const float4 b = __ldg(reinterpret_cast<const float4*>(beta) + cg);
+        const float4 ca = *reinterpret_cast<const float4*>(coef + 4 * cg);
+        const float4 cb = *reinterpret_cast<const float4*>(coef + C + 4 * cg);
+        const int64_t base = (r0 + my_rl) * cg_total + cg, step = (int64_t)rl * cg_total;
+        const int n = (int)((r1 - r0 - my_rl + rl - 1) / rl);
+#pragma unroll 4
+        for (int k = 0; k < n; ++k) {
+            const int64_t i = base + k * step;
+            const float4 v = __ldg(x + i);
+            const float4 d = __ldcg(dy + i);
+            float4 o;
+            o.x = bn_dx1(v.x, d.x, mu.x, rs.x, g.x, b.x, ca.x, cb.x, 0.f);
+            o.y = bn_dx1(v.y, d.y, mu.y, rs.y, g.y, b.y, ca.y, cb.y, 0.f);
+            o.z = bn_dx1(v.z, d.z, mu.z, rs.z, g.z, b.z, ca.z, cb.z, 0.f);
+            o.w = bn_dx1(v.w, d.w, mu.w, rs.w, g.w, b.w, ca.w, cb.w, 0.f);
+            if (ADDEND) { const float4 e = __ldg(addend + i); o.x += e.x; o.y += e.y; o.z += e.z; o.w += e.w; }
+            if (ACCUM) { const float4 e = dx[i]; o.x += e.x; o.y += e.y; o.z += e.z; o.w += e.w; }
+            dx[i] = o;
+        }
+    }
+}
+
 // BN(+ReLU) backward of a micro-batch sized tensor in ONE launch: thread-block clusters instead of the reduce / apply pair.
 // A cluster of kBnCluster CTAs owns cgc float4 column groups (channels never mix, so clusters are independent); its CTAs
 // split the rows.  Every thread keeps its NV rows of x and dy in registers, the CTA reduces sum dz and sum dz*xhat per
@@ -1861,6 +1938,33 @@ cudaError_t bnrelu_bwd(const float* x, const float* dy, const float* gamma, cons
     else HPF_BN_APPLY(false, false);
 #undef HPF_BN_APPLY
     count(n_launch, 2);
+    return cudaGetLastError();
+}
+
+bool bn_bwd_is_one_launch(int64_t rows, int C) { return bn_cluster_plan(rows, C).ok; }
+
+cudaError_t bnrelu_bwd_apply(const float* x, const float* dy, const float* gamma, const float* beta, const float* stats, const float* sums, int n_sums,
+                             int64_t sums_ms, float* dx, const float* addend, bool accumulate, float* dgamma, float* dbeta, int64_t rows, int C,
+                             cudaStream_t st, int64_t* n_launch, const BnGroup& grp)
+{
+    const BnPlan p = bn_plan(rows, C);
+    // four rows a thread at least, six blocks an SM at most
+    int64_t nb = rows / ((int64_t)p.rl * 4), most = 148 * 6 / grp.count;
+    if (nb > most) nb = most;
+    if (nb < 1) nb = 1;
+    const int64_t rpb = ceil_div64(rows, nb);
+    const dim3 grid((unsigned int)ceil_div64(rows, rpb), grp.count);
+    const float4* x4 = reinterpret_cast<const float4*>(x);
+    const float4* dy4 = reinterpret_cast<const float4*>(dy);
+    const float4* ad4 = reinterpret_cast<const float4*>(addend);
+    float4* dx4 = reinterpret_cast<float4*>(dx);
+#define HPF_BN_SUMS(A, B) launch_pdl(bn_apply_sums_bwd_kernel<A, B>, grid, dim3(kBnThreads), (size_t)2 * C * sizeof(float), st, x4, dy4, gamma, beta, stats, sums, n_sums, sums_ms, dgamma, dbeta, ad4, dx4, rows, C, p.cgt, p.rl, p.passes, rpb, grp)
+    if (addend && accumulate) HPF_BN_SUMS(true, true);
+    else if (addend) HPF_BN_SUMS(true, false);
+    else if (accumulate) HPF_BN_SUMS(false, true);
+    else HPF_BN_SUMS(false, false);
+#undef HPF_BN_SUMS
+    count(n_launch, 1);
     return cudaGetLastError();
 }
 
