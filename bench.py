@@ -283,7 +283,7 @@ def kernel_roofline(torch, hpf, cfg, pk):
             # proportion to the pixels (the input is read once, nothing is re-read); null when no capture covers the shape
             "traffic": traffic,
             "peak_source": pk["source"],
-            "kernel": "conv_tc_fwd_kernel (tcgen05 implicit GEMM, three-pass TF32), %dx%d stride %d, %d->%d channels, %dx%d "
+            "kernel": "conv_pipe_kernel (tcgen05 implicit GEMM, three-pass TF32), %dx%d stride %d, %d->%d channels, %dx%d "
                       "pixels, micro-batch %d; %d rotating operand sets, kernel nodes only, launched with programmatic dependent launch as in the step"
                       % (ks, ks, st, ci, co, H, H, b, nset),
             "algorithmic_bytes_per_launch": alg, "us_per_launch": sec * 1e6,

@@ -101,11 +101,11 @@ int hpf_model_destroy(hpf_model *model);
  *                          nothing but the average, so its rounding error (about 8e-4 relative with one pass) does not
  *                          compound with depth the way forward and data-gradient errors do; those always follow
  *                          HPF_OPT_CONV_PATH.
- *   HPF_OPT_FUSE_BN        bit 0: the per-channel sums of a BN's forward statistics are formed in the write-out of the
- *                          tensor-core convolution kernel that produces the BN's input, when both run back to back on
- *                          one stream; the BN forward is then one kernel.  bit 1 (needs bit 0): a BN+ReLU whose output
+ *   HPF_OPT_FUSE_BN        bit 0: the moments of a BN's input are formed in the write-out of the tensor-core
+ *                          convolution that produces it, when both run back to back on one stream; the sums of a large
+ *                          BN+ReLU's backward in that of the data gradient which writes its output's gradient.  bit 1 (needs bit 0): a BN+ReLU whose output
  *                          only the next op reads, a stride-1 tensor-core convolution of the same partition, has no
- *                          kernel of its own: that convolution derives the statistics from the per-tile sums, applies
+ *                          kernel of its own: that convolution derives the statistics from the moments, applies
  *                          the BN+ReLU to its input tile on the way to the tensor core and stores the BN's output and
  *                          statistics as a by-product.  0: every BN runs its own kernels.  Default 3.
  *   HPF_OPT_CELL_TIMES     1: a one-thread kernel stores the device's nanosecond timer at the start and at the end of
@@ -136,7 +136,7 @@ int hpf_model_destroy(hpf_model *model);
  *                          resident for the cell, walks the list of convolutions and meets at a grid-wide barrier between
  *                          them (Section 5.3's stage as one resident grid instead of a chain of launches).  The cells of
  *                          all partitions must fit the GPU together (hpf_bind: HPF_ERR_UNSUPPORTED otherwise).  Results
- *                          are bit-identical to N = 0 when the tile assignment is the same.  0: one launch per convolution. */
+ *                          are bit-identical to N = 0.  0: one launch per convolution. */
 typedef enum { HPF_OPT_GRAPH = 1, HPF_OPT_CONV_PATH = 2, HPF_OPT_SINGLE_STREAM = 3, HPF_OPT_KEEP_MESSAGES = 4,
                HPF_OPT_FUSE_ADD = 5, HPF_OPT_PDL = 6, HPF_OPT_WGRAD_PASSES = 7, HPF_OPT_FUSE_BN = 8, HPF_OPT_CELL_TIMES = 9,
                HPF_OPT_BN_CLUSTER = 10, HPF_OPT_CELL_CTAS = 11, HPF_OPT_PDL_LATE_FROM = 12,
