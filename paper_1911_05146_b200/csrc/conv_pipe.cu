@@ -1474,6 +1474,12 @@ cudaError_t conv_pipe_launch(const ConvPipePlan* plan, int m_first, int m_count,
     auto kernel = L.bn_in ? (flat ? conv_pipe_kernel<true, true, false> : conv_pipe_kernel<true, false, false>)
                           : (p.bn_x ? (flat ? conv_pipe_kernel<false, true, true> : conv_pipe_kernel<false, false, true>)
                                     : (flat ? conv_pipe_kernel<false, true, false> : conv_pipe_kernel<false, false, false>));
+    // What a CTA has to do decides how its warps share it (the sums are the same either way).  A block of the operand takes one
+    // splitter warp about 2000 clocks and all four of them 850, so with one or two blocks in all they share each; with a single unit
+    // both halves of the write-out's warps take it.
+    const int units = (tasks + per_slice - 1) / per_slice * p.unit_block, blocks = units * ((p.n_chunks + p.ksplit - 1) / p.ksplit);
+    if (blocks < 4) L.p.s.split_groups = blocks < 2 || p.split_groups == 1 ? 1 : 2;
+    if (units == 1 && p.n_chunk > 32) L.p.s.epi_alternate = 0;      // (each half a group of columns: the partial sums of the moments stay the same)
     launch_pdl(kernel, dim3(per_slice * p.slices), dim3(kPipeThreads), L.smem, st, L.p, m_first, m_count);
     if (n_launch) ++*n_launch;
     return cudaGetLastError();
