@@ -144,7 +144,24 @@ __device__ __forceinline__ float4 lane_sum(float4 v, int o)
     v.z += __shfl_xor_sync(0xffffffffu, v.z, o); v.w += __shfl_xor_sync(0xffffffffu, v.w, o);
     return v;
 }
-__device__ __forceinline__ float4 add4(float4 a, float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
+// Four values at a time with the two-wide fp32 instructions: the same rounding, half the instructions - what the write-out
+// and the operand rewrite of a tile cost is instructions issued and fetched.
+__device__ __forceinline__ uint64_t pair(float x, float y) { uint64_t r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y)); return r; }
+__device__ __forceinline__ void unpair(uint64_t v, float& x, float& y) { asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v)); }
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) { uint64_t r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
+__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) { uint64_t r; asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) { uint64_t r; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) { uint64_t r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }
+__device__ __forceinline__ float4 unpair4(uint64_t lo, uint64_t hi) { float4 r; unpair(lo, r.x, r.y); unpair(hi, r.z, r.w); return r; }
+__device__ __forceinline__ float4 add4(float4 a, float4 b) { return unpair4(add2(pair(a.x, a.y), pair(b.x, b.y)), add2(pair(a.z, a.w), pair(b.z, b.w))); }
+__device__ __forceinline__ float4 sub4(float4 a, float4 b) { return unpair4(sub2(pair(a.x, a.y), pair(b.x, b.y)), sub2(pair(a.z, a.w), pair(b.z, b.w))); }
+__device__ __forceinline__ float4 mul4(float4 a, float4 b) { return unpair4(mul2(pair(a.x, a.y), pair(b.x, b.y)), mul2(pair(a.z, a.w), pair(b.z, b.w))); }
+__device__ __forceinline__ float4 fma4(float4 a, float4 b, float4 c)
+{
+    return unpair4(fma2(pair(a.x, a.y), pair(b.x, b.y), pair(c.x, c.y)), fma2(pair(a.z, a.w), pair(b.z, b.w), pair(c.z, c.w)));
+}
+// what the tensor core ignores of a value
+__device__ __forceinline__ float4 lo_part(float4 v) { return sub4(v, make_float4(tf32_hi(v.x), tf32_hi(v.y), tf32_hi(v.z), tf32_hi(v.w))); }
 
 // Statistics of a BN's input from the partial moments of one micro-batch: rows of (mean[C], M2[C]) with n values each.
 //   mean = ref + sum n (mean_u - ref) / N,   M2 = sum M2_u + sum n (mean_u - ref)^2 - N (mean - ref)^2,   ref = row 0's mean:
@@ -341,11 +358,11 @@ __device__ __forceinline__ void emit_rows(const EmitArgs& a, int ro, int fill, i
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const bool real = so[i] >= 0;
-                const float x0 = (e[i].x - k.x) * rs.x, x1 = (e[i].y - k.y) * rs.y, x2 = (e[i].z - k.z) * rs.z, x3 = (e[i].w - k.w) * rs.w;
-                const float d0 = real && fmaf(g.x, x0, bt.x) > 0.f ? v[i].x : 0.f, d1 = real && fmaf(g.y, x1, bt.y) > 0.f ? v[i].y : 0.f,
-                            d2 = real && fmaf(g.z, x2, bt.z) > 0.f ? v[i].z : 0.f, d3 = real && fmaf(g.w, x3, bt.w) > 0.f ? v[i].w : 0.f;
-                sd.x += d0; sd.y += d1; sd.z += d2; sd.w += d3;
-                sq.x = fmaf(d0, x0, sq.x); sq.y = fmaf(d1, x1, sq.y); sq.z = fmaf(d2, x2, sq.z); sq.w = fmaf(d3, x3, sq.w);
+                const float4 xh = mul4(sub4(e[i], k), rs), z = fma4(g, xh, bt);
+                const float4 d = make_float4(real && z.x > 0.f ? v[i].x : 0.f, real && z.y > 0.f ? v[i].y : 0.f, real && z.z > 0.f ? v[i].z : 0.f,
+                                             real && z.w > 0.f ? v[i].w : 0.f);
+                sd = add4(sd, d);
+                sq = fma4(d, xh, sq);
             }
             if (b + 4 < steps) emit_residuals(a, ro, lane, lsh, b + 4, e);
         } else if (a.extra) {
@@ -366,10 +383,9 @@ __device__ __forceinline__ void emit_rows(const EmitArgs& a, int ro, int fill, i
         if (moments && !BNB) {
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                const bool real = so[i] >= 0;
-                const float d0 = real ? v[i].x - k.x : 0.f, d1 = real ? v[i].y - k.y : 0.f, d2 = real ? v[i].z - k.z : 0.f, d3 = real ? v[i].w - k.w : 0.f;
-                sd.x += d0; sd.y += d1; sd.z += d2; sd.w += d3;
-                sq.x = fmaf(d0, d0, sq.x); sq.y = fmaf(d1, d1, sq.y); sq.z = fmaf(d2, d2, sq.z); sq.w = fmaf(d3, d3, sq.w);
+                const float4 d = sub4(so[i] >= 0 ? v[i] : k, k);
+                sd = add4(sd, d);
+                sq = fma4(d, d, sq);
             }
         }
     }
@@ -737,10 +753,8 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
                             }
 #pragma unroll
                             for (int j = 0; j < kRowBatch; ++j) {
-                                v[j].x = fmaxf(fmaf(g.x, (v[j].x - mu.x) * rs.x, b.x), 0.f);
-                                v[j].y = fmaxf(fmaf(g.y, (v[j].y - mu.y) * rs.y, b.y), 0.f);
-                                v[j].z = fmaxf(fmaf(g.z, (v[j].z - mu.z) * rs.z, b.z), 0.f);
-                                v[j].w = fmaxf(fmaf(g.w, (v[j].w - mu.w) * rs.w, b.w), 0.f);
+                                const float4 z = fma4(g, mul4(sub4(v[j], mu), rs), b);
+                                v[j] = make_float4(fmaxf(z.x, 0.f), fmaxf(z.y, 0.f), fmaxf(z.z, 0.f), fmaxf(z.w, 0.f));
                                 if (!inside[j]) v[j] = make_float4(0.f, 0.f, 0.f, 0.f);      // the padding is zero AFTER the activation
                                 *reinterpret_cast<float4*>(hi + byte_step * j) = v[j];
                             }
@@ -748,7 +762,7 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
 #pragma unroll
                                 for (int j = 0; j < kRowBatch; ++j)
                                     *reinterpret_cast<float4*>(lo + byte_step * j) =
-                                        make_float4(v[j].x - tf32_hi(v[j].x), v[j].y - tf32_hi(v[j].y), v[j].z - tf32_hi(v[j].z), v[j].w - tf32_hi(v[j].w));
+                                        lo_part(v[j]);
                             if (store_y)
 #pragma unroll
                                 for (int j = 0; j < kRowBatch; ++j) if (own[j]) *reinterpret_cast<float4*>(ydst + off[j]) = v[j];
@@ -762,7 +776,7 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
 #pragma unroll
                             for (int j = 0; j < kRowBatch; ++j)
                                 *reinterpret_cast<float4*>(lo + byte_step * j) =
-                                    make_float4(v[j].x - tf32_hi(v[j].x), v[j].y - tf32_hi(v[j].y), v[j].z - tf32_hi(v[j].z), v[j].w - tf32_hi(v[j].w));
+                                    lo_part(v[j]);
                         }
                     }
                     fence_async_smem();               // generic-proxy writes -> tensor-core reads
@@ -841,7 +855,7 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
                     tmem_ld16_nowait(at + (uint32_t)n_chunk, w);
                     tmem_ld_wait();
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) v[j] += w[j];
+                    for (int j = 0; j < 16; j += 2) unpair(add2(pair(v[j], v[j + 1]), pair(w[j], w[j + 1])), v[j], v[j + 1]);
                 } else {
                     tmem_ld_wait();
                 }
@@ -902,7 +916,7 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
                                 float w[16];
                                 load16(sk_all + ((size_t)z * T + t) * sk_tile + ((size_t)(2 * g + h) * kTileM + quad * 32 + lane) * 16, w);
 #pragma unroll
-                                for (int j = 0; j < 16; ++j) v[j] += w[j];
+                                for (int j = 0; j < 16; j += 2) unpair(add2(pair(v[j], v[j + 1]), pair(w[j], w[j + 1])), v[j], v[j + 1]);
                             }
                         } else {
                             accumulator(t, 32 * g + 16 * h, v);
