@@ -1189,8 +1189,10 @@ void wgrad_splits(const ConvShape& s, int n_tiles, int ctas_per_split, int M, in
     if (splits > cap) splits = cap;
     if (splits > 296) splits = 296;          // two CTAs per SM
     if (M > 1) {
-        // the launch covers the model's M micro-batches, each with its own sums: two waves of two CTAs per SM between them
-        int ms = 592 / (ctas_per_split * M);
+        // The launch covers the model's M micro-batches, each with its own sums.  It runs beside the chain of data gradients,
+        // which wants whole SMs, and its partial sums are written and read again: one and a half CTAs per SM in all.
+        // 592 / 296 / 222 / 148 / 74 CTAs: resnet152 39.2 / 37.9 / 36.6 / 36.8 / 36.9 ms, resnet110 6.71 / 6.61 / 6.53 / 6.50 / 6.71.
+        int ms = 222 / (ctas_per_split * M);
         if (ms < 1) ms = 1;
         if (splits > ms) splits = ms;
     }
