@@ -441,10 +441,15 @@ void build_kernel_plan(hpf_model* mdl)
     for (int j = 0; j < n; ++j) {
         const OpInfo& bn = mdl->ops[j];
         if (bn.op.kind != HPF_OP_BNRELU) continue;
-        // Backward: the only kernel that writes the gradient of the BN's output forms its sums where the BN would read
-        // everything twice.  (A BN that one launch of clusters handles from registers is faster left alone: the sums cost the
-        // data gradient's write-out about a microsecond of latency, resnet11 took 395 us instead of 355.)
-        if (bn.consumers.size() == 1 && !(mdl->opt_bn_cluster && bn_bwd_is_one_launch((int64_t)mdl->b * bn.H * bn.W, bn.C))) {
+        // Backward: the only kernel that writes the gradient of the BN's output forms its sums, unless one launch of clusters
+        // does it all from registers and is the better one: below a million values over all micro-batches (its clusters are
+        // resident at once; the sums cost the data gradient's write-out about a microsecond of latency, resnet11 took 395 us
+        // instead of 355), and beyond 128 channels (several channel slices repeat the work, and those data gradients are
+        // bound by their MMAs: resnet152 36.7 ms against 37.2 with the sums everywhere; resnet1001 63.7 ms with clusters
+        // wherever they fit, 61.3 so).
+        const bool clusters = mdl->opt_bn_cluster && bn_bwd_is_one_launch((int64_t)mdl->b * bn.H * bn.W, bn.C) &&
+                              (bn.C > 128 || (int64_t)mdl->B * bn.H * bn.W * bn.C < 1000000);
+        if (bn.consumers.size() == 1 && !clusters) {
             const int i = bn.consumers[0];
             const OpInfo& c = mdl->ops[i];
             if (i == j + 1 && c.op.kind == HPF_OP_CONV && c.op.stride == 1 && bn.C <= 2048 && c.part == bn.part && mdl->use_pipe[PASS_DGRAD][i] && !mdl->edge0[i].accumulate &&
