@@ -1143,17 +1143,45 @@ __global__ void __launch_bounds__(kPipeThreads, 1) conv_pipe_cell_kernel(const _
     if (warp_index() == 0) tmem_dealloc(tmem_base, cp.tmem_cols);
 }
 
-// Statistics for a BN that runs a kernel of its own although its input came from a convolution that left moments.
-__global__ void __launch_bounds__(256) bn_finalize_kernel(const float* __restrict__ partials, int units, int C, double inv_rows, float eps, float* stats)
+// Statistics for a BN that runs a kernel of its own although its input came from a convolution that left moments (the formulas
+// of merge_moments).  A block takes 128 channels with eight row lanes, grid (channels / 128, micro-batches): latency bound, so the
+// rows are spread (one block per micro-batch took 16 us at 1024 channels).
+__global__ void __launch_bounds__(256) bn_finalize_kernel(const float* __restrict__ partials, int rows, int C, double inv_rows, float eps, float* stats)
 {
-    extern __shared__ float4 dyn[];                   // 4 x 256 float4, then the table
-    float* tab = reinterpret_cast<float*>(dyn + 1024);
-    const int m = blockIdx.x;
+    __shared__ float4 red[3][8][32];
+    __shared__ float4 refs[32];
     pdl_launch_dependents();
     pdl_wait();
-    merge_moments<256>(partials + (size_t)m * partial_floats(units, C), units, C, inv_rows, eps, tab, dyn, threadIdx.x);
+    const int t = threadIdx.x, lane = t & 31, ln = t >> 5, c4n = C >> 2, col = blockIdx.x * 32 + lane;
+    partials += (size_t)blockIdx.y * partial_floats(rows, C); stats += (size_t)blockIdx.y * 2 * C;
+    const float* counts = partials + (size_t)rows * 2 * C;
+    float4 sd = make_float4(0.f, 0.f, 0.f, 0.f), sq = sd, m2 = sd, ref = sd;
+    if (col < c4n) {
+        ref = __ldcg(reinterpret_cast<const float4*>(partials) + col);
+#pragma unroll 4
+        for (int k = ln; k < rows; k += 8) {
+            const float4* row = reinterpret_cast<const float4*>(partials + (size_t)k * 2 * C);
+            const float n = __ldcg(counts + k);
+            const float4 d = sub4(__ldcg(row + col), ref), nd = mul4(make_float4(n, n, n, n), d);
+            sd = add4(sd, nd);
+            sq = fma4(nd, d, sq);
+            m2 = add4(m2, __ldcg(row + c4n + col));
+        }
+    }
+    red[0][ln][lane] = sd; red[1][ln][lane] = sq; red[2][ln][lane] = m2;
+    if (ln == 0) refs[lane] = ref;
     __syncthreads();
-    for (int i = threadIdx.x; i < 2 * C; i += 256) stats[(size_t)m * 2 * C + i] = tab[i];
+    const int c = blockIdx.x * 128 + t;
+    if (t >= 128 || c >= C) return;
+    const float* r = reinterpret_cast<const float*>(&red[0][0][0]) + t;
+    float d = 0.f, q = 0.f, v = 0.f;
+#pragma unroll
+    for (int l = 0; l < 8; ++l) { d += r[128 * l]; q += r[128 * (8 + l)]; v += r[128 * (16 + l)]; }
+    const double dm = (double)d * inv_rows;
+    double var = ((double)v + (double)q) * inv_rows - dm * dm;
+    if (var < 0.0) var = 0.0;
+    stats[c] = (float)((double)reinterpret_cast<const float*>(refs)[t] + dm);
+    stats[C + c] = 1.0f / sqrtf((float)(var + (double)eps));
 }
 
 // Forward pass, or the data gradient seen as a forward problem.
@@ -1533,7 +1561,7 @@ cudaError_t conv_pipe_cell_launch(const void* d_ops, int n_ops, int m_first, int
 cudaError_t bn_finalize_partials(const float* partials, int units, int C, float eps, double rows, float* stats, int m_count, cudaStream_t st,
                                  int64_t* n_launch)
 {
-    launch_pdl(bn_finalize_kernel, dim3(m_count), dim3(256), (size_t)1024 * 16 + 2 * (size_t)C * 4, st, partials, units, C, 1.0 / rows, eps, stats);
+    launch_pdl(bn_finalize_kernel, dim3((C + 127) / 128, m_count), dim3(256), 0, st, partials, units, C, 1.0 / rows, eps, stats);
     if (n_launch) ++*n_launch;
     return cudaGetLastError();
 }
