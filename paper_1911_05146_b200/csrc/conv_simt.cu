@@ -43,10 +43,11 @@ struct SimtArgs {
     Div dC, dK, dR, dQ, dP, dW, dH;
 };
 
-template <int MODE, int BM, int BN, int BK, int KS>
+// TM x 4 outputs per thread
+template <int MODE, int BM, int BN, int BK, int KS, int TM>
 __global__ void __launch_bounds__(THREADS) conv_simt_kernel(const __grid_constant__ SimtArgs g)
 {
-    static_assert((BM / 4) * (BN / 4) * KS == THREADS && BK % KS == 0, "256 threads");
+    static_assert((BM / TM) * (BN / 4) * KS == THREADS && BK % KS == 0, "256 threads");
     constexpr int EA = BM * BK / THREADS, EB = BN * BK / THREADS;
     constexpr int TILE = (BM + 4) * BK + (BN + 4) * BK, RED = KS > 1 ? KS * BM * BN : 0;
     __shared__ __align__(16) float sm[TILE > RED ? TILE : RED];
@@ -145,9 +146,9 @@ __global__ void __launch_bounds__(THREADS) conv_simt_kernel(const __grid_constan
     };
     constexpr int TX = BN / 4, SLICE = THREADS / KS;
     const int ks = tid / SLICE, lt = tid - ks * SLICE, ty = lt / TX, tx = lt - ty * TX;
-    float acc[4][4];
+    float acc[TM][4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < TM; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
 
@@ -169,10 +170,16 @@ __global__ void __launch_bounds__(THREADS) conv_simt_kernel(const __grid_constan
 #pragma unroll
         for (int k = 0; k < BK / KS; ++k) {
             const int kk = ks * (BK / KS) + k;
-            const float4 a4 = *reinterpret_cast<const float4*>(&As[kk][ty * 4]), b4 = *reinterpret_cast<const float4*>(&Bs[kk][tx * 4]);
-            const float av[4] = {a4.x, a4.y, a4.z, a4.w}, bv[4] = {b4.x, b4.y, b4.z, b4.w};
+            const float4 b4 = *reinterpret_cast<const float4*>(&Bs[kk][tx * 4]);
+            const float bv[4] = {b4.x, b4.y, b4.z, b4.w};
+            float av[TM];
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int i = 0; i < TM; i += 4) {
+                const float4 a4 = *reinterpret_cast<const float4*>(&As[kk][ty * TM + i]);
+                av[i] = a4.x; av[i + 1] = a4.y; av[i + 2] = a4.z; av[i + 3] = a4.w;
+            }
+#pragma unroll
+            for (int i = 0; i < TM; ++i)
 #pragma unroll
                 for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
         }
@@ -181,9 +188,9 @@ __global__ void __launch_bounds__(THREADS) conv_simt_kernel(const __grid_constan
         // the slices of the k steps, in order
         __syncthreads();
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < TM; ++i)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) sm[(ks * BM + ty * 4 + i) * BN + tx * 4 + j] = acc[i][j];
+            for (int j = 0; j < 4; ++j) sm[(ks * BM + ty * TM + i) * BN + tx * 4 + j] = acc[i][j];
         __syncthreads();
         for (int i = tid; i < BM * BN; i += THREADS) {
             float v = 0.f;
@@ -195,8 +202,8 @@ __global__ void __launch_bounds__(THREADS) conv_simt_kernel(const __grid_constan
         return;
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int m = m0 + ty * 4 + i;
+    for (int i = 0; i < TM; ++i) {
+        const int m = m0 + ty * TM + i;
         if (m >= Md) continue;
         int64_t row = m;
         if (MODE == MODE_DGRAD && s.stride > 1) {
@@ -268,16 +275,18 @@ SimtArgs make_args(const float* a, const float* b, float* out, const float* extr
     return g;
 }
 
-template <int MODE, int BM, int BN, int BK, int KS>
+template <int MODE, int BM, int BN, int BK, int KS, int TM = 4>
 void launch_tiles(const SimtArgs& g, int z, cudaStream_t st)
 {
-    conv_simt_kernel<MODE, BM, BN, BK, KS><<<dim3((g.Md + BM - 1) / BM, (g.Nd + BN - 1) / BN, z), THREADS, 0, st>>>(g);
+    conv_simt_kernel<MODE, BM, BN, BK, KS, TM><<<dim3((g.Md + BM - 1) / BM, (g.Nd + BN - 1) / BN, z), THREADS, 0, st>>>(g);
 }
 template <int MODE>
 void launch_by_width(const SimtArgs& g, int z, cudaStream_t st)
 {
     if (g.Nd <= 16) launch_tiles<MODE, 256, 16, 16, 1>(g, z, st);
     else if (g.Nd <= 32) launch_tiles<MODE, 128, 32, 16, 1>(g, z, st);
+    // (eight rows a thread take three shared-memory loads per 32 products instead of four; from two such tiles per SM on)
+    else if ((long long)g.Md * ((g.Nd + 63) / 64) * z >= 2 * 148 * 128) launch_tiles<MODE, 128, 64, 16, 1, 8>(g, z, st);
     else launch_tiles<MODE, 64, 64, 16, 1>(g, z, st);
 }
 
