@@ -131,10 +131,10 @@ struct hpf_model {
     int slot_of(int p, int m) const { return p * lanes() + m % lanes(); }
     int opt_pdl_late_from = 8;   // forward cells that run while at least this many cells are under way trigger their successors late
     // Groups: on one GPU the stages share the same SMs, and a micro-batch's launches are too small to fill them, so one launch
-    // covers `group_size()` micro-batches of a stage wherever nothing asks for cells of their own.  Every micro-batch keeps
+    // covers all micro-batches of a stage wherever nothing asks for cells of their own (then one micro-batch).  Every micro-batch keeps
     // its own statistics, losses and gradient slot, formed in the same order whatever the size of the group.
-    int group_size() const;
-    int n_groups() const { const int g = group_size(); return (M + g - 1) / g; }
+    int group_size() const { return opt_messages || opt_cell_times || lanes() > 1 ? 1 : M; }
+    int n_groups() const { return M / group_size(); }
     int opt_fuse_bn = 3;       // bit 0: BN statistics in the producing convolution's write-out, bit 1: BN+ReLU applied by the reading convolution
     std::vector<GradEdge> edge0;              // per op: contribution to src0
     std::vector<AccumAction> accums;
@@ -201,14 +201,6 @@ struct hpf_model {
     cudaStream_t stream_of(int p, int m = 0) const { return opt_single ? streams[0] : streams[slot_of(p, m)]; }
     DeviceStatus* status() const { return reinterpret_cast<DeviceStatus*>(ws + status_off); }
 };
-
-int hpf_model::group_size() const
-{
-    if (opt_messages || opt_cell_times || lanes() > 1) return 1;
-    const char* v = getenv("HPF_GROUP");
-    int g = v ? atoi(v) : M;
-    return g < 1 ? 1 : (g > M ? M : g);
-}
 
 namespace {
 
@@ -820,7 +812,6 @@ int enqueue_phase(hpf_model* mdl, int phase)
     const PdlScope pdl_scope(mdl->opt_pdl);
     const BnClusterScope bn_cluster_scope(mdl->opt_bn_cluster);
     const int P = mdl->P, M = mdl->n_groups(), gs = mdl->group_size();          // a cell is a group of micro-batches here
-    auto group = [&](int k) { return std::min(gs, mdl->M - k * gs); };
     cudaStream_t s0 = mdl->streams[0];
     const bool merged = phase == PH_FB;
     const bool do_fwd = phase == PH_FWD || merged, do_bwd = phase == PH_BWD || merged;
@@ -865,7 +856,7 @@ int enqueue_phase(hpf_model* mdl, int phase)
                 }
                 if (mdl->opt_cell_times) CU(stamp_time(mdl->cell_time_slot(PH_FWD, p, m), st, &mdl->launches));
                 for (int i = mdl->part_lo[p]; i < mdl->part_hi[p]; ++i) {
-                    int rc = forward_op(mdl, i, m * gs, group(m), st, mdl->slot_of(p, m));
+                    int rc = forward_op(mdl, i, m * gs, gs, st, mdl->slot_of(p, m));
                     if (rc) return rc;
                 }
                 if (mdl->opt_cell_times) CU(stamp_time(mdl->cell_time_slot(PH_FWD, p, m) + 1, st, &mdl->launches));
@@ -893,7 +884,7 @@ int enqueue_phase(hpf_model* mdl, int phase)
                 }
                 if (mdl->opt_cell_times) CU(stamp_time(mdl->cell_time_slot(PH_BWD, p, m), st, &mdl->launches));
                 for (int i = mdl->part_hi[p] - 1; i >= mdl->part_lo[p]; --i) {
-                    int rc = backward_op(mdl, i, m * gs, group(m), st, mdl->slot_of(p, m));
+                    int rc = backward_op(mdl, i, m * gs, gs, st, mdl->slot_of(p, m));
                     if (rc) return rc;
                 }
                 if (mdl->opt_cell_times) CU(stamp_time(mdl->cell_time_slot(PH_BWD, p, m) + 1, st, &mdl->launches));

@@ -336,6 +336,23 @@ def test_stage_lanes_give_the_same_bits_and_fill_the_bubble(lanes, one_graph):
     assert fwd[0][1][0] < fwd[0][0][1]
 
 
+def test_the_environment_changes_nothing_between_two_steps_of_a_bound_model(monkeypatch):
+    """How many micro-batches a launch covers follows from the model's options alone: a variable that once set it, changed
+    after hpf_bind, leaves the launches of the next step as they were."""
+    c = wl.config("r11")
+    x, labels, theta = seeded(c["ops"], c["in_hwc"], c["B"])
+    bd = Bound(c["ops"], c["in_hwc"], c["B"], c["M"], c["cuts"], theta, {hpf.OPT_GRAPH: 0})
+    bd.upload(x, labels)
+
+    def launches():
+        before = bd.model.launch_count()
+        bd.step()
+        return bd.model.launch_count() - before
+    n = launches()
+    monkeypatch.setenv("HPF_GROUP", "1")
+    assert launches() == n
+
+
 def test_too_few_streams_for_the_lanes_are_refused():
     ops = wl.resnet_v2_cifar(1)
     model = hpf.Model(ops, (4, 32, 32, 3), wl.default_cuts(len(ops), 2), 2)
