@@ -421,24 +421,26 @@ struct ResidentPlan { bool ok; int grid, iters; long long per_cta; size_t smem; 
 // shared memory); 0 otherwise.  Asked once per device.
 int resident_sm_count()
 {
-    static int cached[64] = {0};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-    if (!cached[dev]) {
-        int n = 0, coop = 0, per_sm = 0;
+    static PerDevice<int> sms;
+    int count = 0;
+    const cudaError_t e = sms.get(&count, [](int dev, int* n) {
+        int coop = 0, per_sm = 0;
         const int max_dyn = kResSmemV * kResThreads * (int)sizeof(float4);
-        bool ok = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
-                  cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop != 0;
-        ok = ok && cudaFuncSetAttribute(bn_fwd_resident_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, max_dyn) == cudaSuccess;
-        ok = ok && cudaFuncSetAttribute(bn_bwd_resident_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_dyn) == cudaSuccess;
-        ok = ok && cudaFuncSetAttribute(bn_bwd_resident_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_dyn) == cudaSuccess;
-        ok = ok && cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bn_fwd_resident_kernel, kResThreads, max_dyn) == cudaSuccess && per_sm >= 1;
-        ok = ok && cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bn_bwd_resident_kernel<false>, kResThreads, max_dyn) == cudaSuccess && per_sm >= 1;
-        ok = ok && cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bn_bwd_resident_kernel<true>, kResThreads, max_dyn) == cudaSuccess && per_sm >= 1;
-        if (!ok) { (void)cudaGetLastError(); return 0; }
-        cached[dev] = n;
-    }
-    return cached[dev];
+        cudaError_t err = cudaDeviceGetAttribute(n, cudaDevAttrMultiProcessorCount, dev);
+        if (err == cudaSuccess) err = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+        if (err == cudaSuccess && !coop) err = cudaErrorNotSupported;
+        if (err == cudaSuccess) err = cudaFuncSetAttribute(bn_fwd_resident_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, max_dyn);
+        for (auto kernel : {bn_bwd_resident_kernel<false>, bn_bwd_resident_kernel<true>})
+            if (err == cudaSuccess) err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, max_dyn);
+        if (err == cudaSuccess) err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bn_fwd_resident_kernel, kResThreads, max_dyn);
+        for (auto kernel : {bn_bwd_resident_kernel<false>, bn_bwd_resident_kernel<true>}) {
+            if (err == cudaSuccess && per_sm < 1) err = cudaErrorNotSupported;
+            if (err == cudaSuccess) err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kResThreads, max_dyn);
+        }
+        return err == cudaSuccess && per_sm < 1 ? cudaErrorNotSupported : err;
+    });
+    if (e != cudaSuccess) { (void)cudaGetLastError(); return 0; }
+    return count;
 }
 
 // nreg iterations of a thread stay in registers, the others take `slots` float4 of shared memory each.

@@ -1221,11 +1221,10 @@ bool pipe_view(const ConvShape& s, int pass, PipeView* v)
 
 int sm_count()
 {
-    static const int n = [] {
-        int dev = 0, v = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) { (void)cudaGetLastError(); return 148; }
-        return v;
-    }();
+    static PerDevice<int> sms;
+    int n = 0;
+    const cudaError_t e = sms.get(&n, [](int dev, int* v) { return cudaDeviceGetAttribute(v, cudaDevAttrMultiProcessorCount, dev); });
+    if (e != cudaSuccess) { (void)cudaGetLastError(); return 148; }
     return n;
 }
 
@@ -1386,15 +1385,17 @@ static_assert(sizeof(ConvPipeLaunch) <= sizeof(((ConvPipePlan*)0)->storage), "pl
 
 cudaError_t conv_pipe_init()
 {
-    static bool done = false;
-    if (done) return cudaSuccess;
-    cudaError_t e = cudaSuccess;
-    for (auto kernel : {conv_pipe_kernel<false, false, false>, conv_pipe_kernel<false, true, false>, conv_pipe_kernel<true, false, false>, conv_pipe_kernel<true, true, false>,
-                        conv_pipe_kernel<false, false, true>, conv_pipe_kernel<false, true, true>})
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPipeSmem + 1024);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(conv_pipe_cell_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPipeSmem + 1024);
-    done = e == cudaSuccess;
-    return e;
+    static PerDevice<bool> attributes;
+    bool set = false;
+    return attributes.get(&set, [](int, bool* done) {
+        cudaError_t e = cudaSuccess;
+        for (auto kernel : {conv_pipe_kernel<false, false, false>, conv_pipe_kernel<false, true, false>, conv_pipe_kernel<true, false, false>, conv_pipe_kernel<true, true, false>,
+                            conv_pipe_kernel<false, false, true>, conv_pipe_kernel<false, true, true>})
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPipeSmem + 1024);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(conv_pipe_cell_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPipeSmem + 1024);
+        *done = true;
+        return e;
+    });
 }
 
 namespace {

@@ -1354,24 +1354,23 @@ bool conv_tc_supported(const ConvShape& s, int pass)
 
 cudaError_t conv_tc_init()
 {
-    if (g_encode) return cudaSuccess;
-    void* fn = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    cudaError_t e = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &q);
-    if (e != cudaSuccess) return e;
-    if (q != cudaDriverEntryPointSuccess || !fn) return cudaErrorNotSupported;
-    e = cudaFuncSetAttribute(conv_tc_fwd_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget + 2048);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(conv_tc_fwd_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget + 2048);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(conv_tc_fwd_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget + 2048);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(conv_tc_wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWgradSmemBudget + 2048);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(conv_tc_wgrad_direct_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWgradSmemBudget + 2048);
-    if (e != cudaSuccess) return e;
-    g_encode = reinterpret_cast<EncodeTiledFn>(fn);
-    return cudaSuccess;
+    // (the lock also orders the entry point's address before its first use by whichever thread comes next)
+    static PerDevice<bool> attributes;
+    bool set = false;
+    return attributes.get(&set, [](int, bool* done) {
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        cudaError_t e = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &q);
+        if (e != cudaSuccess) return e;
+        if (q != cudaDriverEntryPointSuccess || !fn) return cudaErrorNotSupported;
+        for (auto kernel : {conv_tc_fwd_kernel<false, false>, conv_tc_fwd_kernel<true, false>, conv_tc_fwd_kernel<false, true>})
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget + 2048);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(conv_tc_wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWgradSmemBudget + 2048);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(conv_tc_wgrad_direct_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWgradSmemBudget + 2048);
+        if (e == cudaSuccess && !g_encode) g_encode = reinterpret_cast<EncodeTiledFn>(fn);
+        *done = true;
+        return e;
+    });
 }
 
 namespace {

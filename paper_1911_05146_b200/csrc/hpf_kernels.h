@@ -6,6 +6,8 @@
 #include <stdint.h>
 #include <stddef.h>
 
+#include <mutex>
+
 namespace hpf {
 
 struct ConvShape {
@@ -18,6 +20,35 @@ inline ConvShape make_conv_shape(int N, int H, int W, int C, int K, int R, int s
     ConvShape s{N, H, W, C, K, R, stride, pad, (H + 2 * pad - R) / stride + 1, (W + 2 * pad - R) / stride + 1};
     return s;
 }
+
+// What is asked or set once per device: a kernel's attributes and the number of SMs belong to one device, and a process may
+// drive several, from several threads.
+template <typename T>
+class PerDevice {
+    static constexpr int kDevices = 64;
+    std::mutex lock;
+    bool have[kDevices] = {};
+    T value[kDevices] = {};
+
+public:
+    // make(device, &value) runs with the current device; a failure is returned and tried again by the next call
+    template <typename F>
+    cudaError_t get(T* out, F&& make)
+    {
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e != cudaSuccess) return e;
+        if (dev < 0 || dev >= kDevices) return make(dev, out);
+        std::lock_guard<std::mutex> hold(lock);
+        if (!have[dev]) {
+            e = make(dev, &value[dev]);
+            if (e != cudaSuccess) return e;
+            have[dev] = true;
+        }
+        *out = value[dev];
+        return cudaSuccess;
+    }
+};
 
 // Programmatic dependent launch.  The step is a long chain of small dependent kernels, so the gap between the end
 // of one and the start of the next is a sizeable part of the critical path.  Hot kernels are launched with the

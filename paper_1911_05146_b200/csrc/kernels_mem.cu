@@ -1032,21 +1032,19 @@ struct BnBigPlan { bool ok; int n_clusters, nblk_apply, stream_out; int64_t rows
 template <bool BWD>
 int bn_big_max_clusters()
 {
-    // per device: a process may drive several GPUs, and the answer (like the attributes set below) belongs to one of them
-    static int cached_by_device[64];
-    static bool have[64];
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) { (void)cudaGetLastError(); return 0; }
-    if (have[dev]) return cached_by_device[dev];
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(kBnBigCluster * kBnBigMaxPartials); cfg.blockDim = dim3(kBnThreads);
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = kBnBigCluster; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
+    static PerDevice<int> clusters;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, bn_reduce_big_kernel<BWD>, &cfg) != cudaSuccess) { (void)cudaGetLastError(); n = 0; }
-    cached_by_device[dev] = n; have[dev] = true;
+    const cudaError_t e = clusters.get(&n, [](int, int* v) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(kBnBigCluster * kBnBigMaxPartials); cfg.blockDim = dim3(kBnThreads);
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = kBnBigCluster; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr; cfg.numAttrs = 1;
+        if (cudaOccupancyMaxActiveClusters(v, bn_reduce_big_kernel<BWD>, &cfg) != cudaSuccess) { (void)cudaGetLastError(); *v = 0; }
+        return cudaSuccess;
+    });
+    if (e != cudaSuccess) { (void)cudaGetLastError(); return 0; }
     return n;
 }
 
@@ -1814,20 +1812,19 @@ size_t bn_scratch_bytes(int64_t rows, int C)
 // The attribute is set once per device; if that fails the callers stay on the ticket path, which needs none.
 bool big_apply_attributes_set()
 {
-    static signed char state[64];        // 0 not tried, 1 set, -1 failed
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) { (void)cudaGetLastError(); return false; }
-    if (state[dev] == 0) {
+    static PerDevice<bool> attributes;
+    bool set = false;
+    const cudaError_t e = attributes.get(&set, [](int, bool* ok) {
         const int mx = (int)bn_big_apply_smem(2048);
-        bool ok = cudaFuncSetAttribute(bn_apply_big_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, mx) == cudaSuccess;
-        ok = ok && cudaFuncSetAttribute(bn_apply_big_bwd_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx) == cudaSuccess;
-        ok = ok && cudaFuncSetAttribute(bn_apply_big_bwd_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx) == cudaSuccess;
-        ok = ok && cudaFuncSetAttribute(bn_apply_big_bwd_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx) == cudaSuccess;
-        ok = ok && cudaFuncSetAttribute(bn_apply_big_bwd_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx) == cudaSuccess;
-        if (!ok) (void)cudaGetLastError();
-        state[dev] = ok ? 1 : -1;
-    }
-    return state[dev] == 1;
+        *ok = cudaFuncSetAttribute(bn_apply_big_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, mx) == cudaSuccess;
+        for (auto kernel : {bn_apply_big_bwd_kernel<false, false>, bn_apply_big_bwd_kernel<false, true>, bn_apply_big_bwd_kernel<true, false>,
+                            bn_apply_big_bwd_kernel<true, true>})
+            *ok = *ok && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, mx) == cudaSuccess;
+        if (!*ok) (void)cudaGetLastError();
+        return cudaSuccess;
+    });
+    if (e != cudaSuccess) { (void)cudaGetLastError(); return false; }
+    return set;
 }
 
 cudaError_t bnrelu_fwd(const float* x, const float* gamma, const float* beta, float eps, float* y, float* stats,
