@@ -238,8 +238,8 @@ bn_fwd_resident_kernel(const float4* __restrict__ x4, const float* __restrict__ 
         const long long i = base + (long long)j * kResThreads;
         if (i < cta_end) res_cp_async16(&held[(j - kResRegV) * kResThreads + t], x4 + i);
     }
-    const float4 sh = __ldg(x4 + q);                 // shift = row 0 (shifted sums avoid cancellation)
-    const float shift_c = t < C ? __ldg(reinterpret_cast<const float*>(x4) + t) : 0.f;   // for the finalisation of channel t
+    const float4 sh = __ldcg(x4 + q);                 // shift = row 0 (shifted sums avoid cancellation)
+    const float shift_c = t < C ? __ldcg(reinterpret_cast<const float*>(x4) + t) : 0.f;   // for the finalisation of channel t
     float4 r[kResRegV];
 #pragma unroll
     for (int j = 0; j < kResRegV; ++j) {
@@ -331,8 +331,8 @@ bn_bwd_resident_kernel(const float4* __restrict__ x4, const float4* __restrict__
             if (HOLD_X) res_cp_async16(&held[((j - NREG) * SL + 1) * kResThreads + t], x4 + i);
         }
     }
-    const float4 mu = __ldg(reinterpret_cast<const float4*>(stats) + q);
-    const float4 rs = __ldg(reinterpret_cast<const float4*>(stats + C) + q);
+    const float4 mu = __ldcg(reinterpret_cast<const float4*>(stats) + q);
+    const float4 rs = __ldcg(reinterpret_cast<const float4*>(stats + C) + q);
     const float4 gm = __ldg(reinterpret_cast<const float4*>(gamma) + q);
     const float4 bt = __ldg(reinterpret_cast<const float4*>(beta) + q);
     float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
@@ -343,7 +343,7 @@ bn_bwd_resident_kernel(const float4* __restrict__ x4, const float4* __restrict__
         for (int j = 0; j < NREG; ++j) {
             const long long i = base + (long long)j * kResThreads;
             const bool in = i < cta_end;
-            v[j] = in ? __ldg(x4 + i) : mu;
+            v[j] = in ? __ldcg(x4 + i) : mu;
             d[j] = in ? __ldcs(dy4 + i) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
 #pragma unroll
@@ -361,7 +361,7 @@ bn_bwd_resident_kernel(const float4* __restrict__ x4, const float4* __restrict__
         if (i < cta_end) {
             float4* slot = &held[((j - NREG) * SL) * kResThreads + t];
             const float4 d = slot[0];
-            const float4 v = HOLD_X ? slot[kResThreads] : __ldg(x4 + i);
+            const float4 v = HOLD_X ? slot[kResThreads] : __ldcg(x4 + i);
             float4 xh, dz;
             res_dz(v, d, mu, rs, gm, bt, floor, xh, dz);
             res_acc_bwd(a, b, dz, xh);
@@ -392,9 +392,9 @@ bn_bwd_resident_kernel(const float4* __restrict__ x4, const float4* __restrict__
         if (i < cta_end) {
             float4 xh;
             if (HOLD_X) xh = rx[j];
-            else { const float4 v = __ldg(x4 + i); xh = res_xhat4(v, mu, rs); }
+            else { const float4 v = __ldcg(x4 + i); xh = res_xhat4(v, mu, rs); }
             float4 o = res_dx(rz[j], xh, sc, ca, cb);
-            if (addend) { const float4 e = __ldg(addend + i); o.x += e.x; o.y += e.y; o.z += e.z; o.w += e.w; }
+            if (addend) { const float4 e = __ldcg(addend + i); o.x += e.x; o.y += e.y; o.z += e.z; o.w += e.w; }
             if (accumulate) { const float4 e = dx4[i]; o.x += e.x; o.y += e.y; o.z += e.z; o.w += e.w; }
             __stcs(dx4 + i, o);
         }
@@ -406,9 +406,9 @@ bn_bwd_resident_kernel(const float4* __restrict__ x4, const float4* __restrict__
             const float4* slot = &held[((j - NREG) * SL) * kResThreads + t];
             float4 xh;
             if (HOLD_X) xh = slot[kResThreads];
-            else { const float4 v = __ldg(x4 + i); xh = res_xhat4(v, mu, rs); }
+            else { const float4 v = __ldcg(x4 + i); xh = res_xhat4(v, mu, rs); }
             float4 o = res_dx(slot[0], xh, sc, ca, cb);
-            if (addend) { const float4 e = __ldg(addend + i); o.x += e.x; o.y += e.y; o.z += e.z; o.w += e.w; }
+            if (addend) { const float4 e = __ldcg(addend + i); o.x += e.x; o.y += e.y; o.z += e.z; o.w += e.w; }
             if (accumulate) { const float4 e = dx4[i]; o.x += e.x; o.y += e.y; o.z += e.z; o.w += e.w; }
             __stcs(dx4 + i, o);
         }

@@ -334,7 +334,8 @@ __device__ __forceinline__ void emit_rows(const EmitArgs& a, int ro, int fill, i
     const bool moments = a.moments != nullptr && who != 0u;
     float4 rs = k, g = k, bt = k;
     if (BNB) {
-        k = __ldg(reinterpret_cast<const float4*>(a.bn_mean + 4 * cq)); rs = __ldg(reinterpret_cast<const float4*>(a.bn_mean + a.bn_c + 4 * cq));
+        // (statistics are results of the step: not the read-only path)
+        k = __ldcg(reinterpret_cast<const float4*>(a.bn_mean + 4 * cq)); rs = __ldcg(reinterpret_cast<const float4*>(a.bn_mean + a.bn_c + 4 * cq));
         g = __ldg(reinterpret_cast<const float4*>(a.bn_gamma + 4 * cq)); bt = __ldg(reinterpret_cast<const float4*>(a.bn_beta + 4 * cq));
     } else if (moments) {
         if (have_shift) k = *reinterpret_cast<const float4*>(a.moments + 4 * cq);

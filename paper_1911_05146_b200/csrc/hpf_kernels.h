@@ -55,7 +55,9 @@ public:
 // programmatic-serialisation attribute: such a kernel may be scheduled while its predecessor in the stream is
 // still running, executes its prologue (barrier and tensor-memory set-up, parameter and descriptor fetches), and
 // blocks in pdl_wait() until the predecessor has completed and its writes are visible.  Every kernel launched
-// this way calls pdl_wait() before its first read or write of global data.
+// this way calls pdl_wait() before its first read or write of global data.  What the step itself computes (activations,
+// gradients, statistics, partial sums) such a kernel reads with __ldcg, never with __ldg: the compiler takes a read-only load
+// for independent of everything and may move it above the wait.  Parameters, which change between steps only, may be __ldg.
 // Per host thread: the model whose phase is being enqueued sets it for the duration of the enqueue (PdlScope).
 extern thread_local bool g_pdl_enabled;
 struct PdlScope {

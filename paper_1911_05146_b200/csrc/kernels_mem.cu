@@ -117,12 +117,12 @@ bn_reduce_kernel(const float* __restrict__ x, const float* __restrict__ dy, cons
         if (my_rl < rl && cg < cg_total) {
             float4 p0, p1, gm, bt;
             if (BWD) {
-                p0 = __ldg(reinterpret_cast<const float4*>(stats) + cg);              // mean
-                p1 = __ldg(reinterpret_cast<const float4*>(stats + C) + cg);          // rstd
+                p0 = __ldcg(reinterpret_cast<const float4*>(stats) + cg);              // mean
+                p1 = __ldcg(reinterpret_cast<const float4*>(stats + C) + cg);          // rstd
                 gm = __ldg(reinterpret_cast<const float4*>(gamma) + cg);
                 bt = __ldg(reinterpret_cast<const float4*>(beta) + cg);
             } else {
-                p0 = __ldg(x4 + cg);                                                  // shift = first row
+                p0 = __ldcg(x4 + cg);                                                  // shift = first row
             }
             const float4* xp = x4 + (r0 + my_rl) * cg_total + cg;
             const float4* dp = dy4 + (r0 + my_rl) * cg_total + cg;
@@ -130,9 +130,9 @@ bn_reduce_kernel(const float* __restrict__ x, const float* __restrict__ dy, cons
             const int n = (int)((r1 - r0 - my_rl + rl - 1) / rl);
 #pragma unroll 4
             for (int k = 0; k < n; ++k) {
-                const float4 v = __ldg(xp + k * step);
+                const float4 v = __ldcg(xp + k * step);
                 if (BWD) {
-                    const float4 g = __ldg(dp + k * step);
+                    const float4 g = __ldcg(dp + k * step);
                     float xh, dz;
                     xh = bn_xhat(v.x, p0.x, p1.x); dz = bn_z(xh, gm.x, bt.x) > floor ? g.x : 0.f; a.x += dz; b.x = fmaf(dz, xh, b.x);
                     xh = bn_xhat(v.y, p0.y, p1.y); dz = bn_z(xh, gm.y, bt.y) > floor ? g.y : 0.f; a.y += dz; b.y = fmaf(dz, xh, b.y);
@@ -269,7 +269,7 @@ bn_reduce_kernel(const float* __restrict__ x, const float* __restrict__ dy, cons
                 coef[c] = (float)(sa * inv_rows);
                 coef[C + c] = (float)(sb * inv_rows);
             } else {
-                const double shift = (double)__ldg(x + c);
+                const double shift = (double)__ldcg(x + c);
                 const double ms = sa * inv_rows;
                 double var = sb * inv_rows - ms * ms;
                 if (var < 0.0) var = 0.0;
@@ -306,15 +306,21 @@ bn_apply_fwd_kernel(const float4* __restrict__ x, const float* __restrict__ gamm
         const float4 b = __ldg(reinterpret_cast<const float4*>(beta) + cg);
         const int64_t base = (r0 + my_rl) * cg_total + cg, step = (int64_t)rl * cg_total;
         const int n = (int)((r1 - r0 - my_rl + rl - 1) / rl);
-#pragma unroll 4
-        for (int k = 0; k < n; ++k) {
-            const float4 v = __ldg(x + base + k * step);
-            float4 o;
-            o.x = fmaxf(bn_z(bn_xhat(v.x, mu.x, rs.x), g.x, b.x), floor);
-            o.y = fmaxf(bn_z(bn_xhat(v.y, mu.y, rs.y), g.y, b.y), floor);
-            o.z = fmaxf(bn_z(bn_xhat(v.z, mu.z, rs.z), g.z, b.z), floor);
-            o.w = fmaxf(bn_z(bn_xhat(v.w, mu.w, rs.w), g.w, b.w), floor);
-            y[base + k * step] = o;
+        // (ordered loads are not moved over stores: a batch's loads are written ahead of them)
+        for (int k0 = 0; k0 < n; k0 += 4) {
+            float4 v[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) if (k0 + j < n) v[j] = __ldcg(x + base + (k0 + j) * step);
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (k0 + j < n) {
+                    float4 o;
+                    o.x = fmaxf(bn_z(bn_xhat(v[j].x, mu.x, rs.x), g.x, b.x), floor);
+                    o.y = fmaxf(bn_z(bn_xhat(v[j].y, mu.y, rs.y), g.y, b.y), floor);
+                    o.z = fmaxf(bn_z(bn_xhat(v[j].z, mu.z, rs.z), g.z, b.z), floor);
+                    o.w = fmaxf(bn_z(bn_xhat(v[j].w, mu.w, rs.w), g.w, b.w), floor);
+                    y[base + (k0 + j) * step] = o;
+                }
         }
     }
 }
@@ -324,6 +330,37 @@ __device__ __forceinline__ float bn_dx1(float x, float dy, float mu, float rs, f
     const float xh = bn_xhat(x, mu, rs);
     const float dz = bn_z(xh, g, b) > floor ? dy : 0.f;
     return g * rs * (dz - ca - xh * cb);
+}
+
+// dx of a thread's rows, four at a time: the loads of a batch are in flight together (ordered loads are not moved over stores).
+template <bool ADDEND, bool ACCUM>
+__device__ __forceinline__ void bn_dx_rows(const float4* x, const float4* dy, const float4* addend, float4* dx, int n, int64_t step, float4 mu, float4 rs,
+                                           float4 g, float4 b, float4 ca, float4 cb, float floor)
+{
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int k0 = 0; k0 < n; k0 += 4, x += 4 * step, dy += 4 * step, addend += ADDEND ? 4 * step : 0, dx += 4 * step) {
+        float4 v[4], d[4], e[4], a[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const bool in = k0 + j < n;
+            v[j] = in ? __ldcg(x + j * step) : zero;
+            d[j] = in ? __ldcg(dy + j * step) : zero;
+            if (ADDEND) e[j] = in ? __ldcg(addend + j * step) : zero;
+            if (ACCUM) a[j] = in ? dx[j * step] : zero;
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (k0 + j < n) {
+                float4 o;
+                o.x = bn_dx1(v[j].x, d[j].x, mu.x, rs.x, g.x, b.x, ca.x, cb.x, floor);
+                o.y = bn_dx1(v[j].y, d[j].y, mu.y, rs.y, g.y, b.y, ca.y, cb.y, floor);
+                o.z = bn_dx1(v[j].z, d[j].z, mu.z, rs.z, g.z, b.z, ca.z, cb.z, floor);
+                o.w = bn_dx1(v[j].w, d[j].w, mu.w, rs.w, g.w, b.w, ca.w, cb.w, floor);
+                if (ADDEND) { o.x += e[j].x; o.y += e[j].y; o.z += e[j].z; o.w += e[j].w; }
+                if (ACCUM) { o.x += a[j].x; o.y += a[j].y; o.z += a[j].z; o.w += a[j].w; }
+                dx[j * step] = o;
+            }
+    }
 }
 
 template <bool ADDEND, bool ACCUM>
@@ -350,28 +387,15 @@ bn_apply_bwd_kernel(const float4* __restrict__ x, const float4* __restrict__ dy,
     for (int pass = 0; pass < passes; ++pass) {
         const int cg = pass * cgt + my_cg;
         if (cg >= cg_total) continue;
-        const float4 mu = __ldg(reinterpret_cast<const float4*>(stats) + cg);
-        const float4 rs = __ldg(reinterpret_cast<const float4*>(stats + C) + cg);
+        const float4 mu = __ldcg(reinterpret_cast<const float4*>(stats) + cg);
+        const float4 rs = __ldcg(reinterpret_cast<const float4*>(stats + C) + cg);
         const float4 g = __ldg(reinterpret_cast<const float4*>(gamma) + cg);
         const float4 b = __ldg(reinterpret_cast<const float4*>(beta) + cg);
         const float4 ca = __ldcg(reinterpret_cast<const float4*>(coef) + cg);
         const float4 cb = __ldcg(reinterpret_cast<const float4*>(coef + C) + cg);
         const int64_t base = (r0 + my_rl) * cg_total + cg, step = (int64_t)rl * cg_total;
         const int n = (int)((r1 - r0 - my_rl + rl - 1) / rl);
-#pragma unroll 4
-        for (int k = 0; k < n; ++k) {
-            const int64_t i = base + k * step;
-            const float4 v = __ldg(x + i);
-            const float4 d = __ldg(dy + i);
-            float4 o;
-            o.x = bn_dx1(v.x, d.x, mu.x, rs.x, g.x, b.x, ca.x, cb.x, floor);
-            o.y = bn_dx1(v.y, d.y, mu.y, rs.y, g.y, b.y, ca.y, cb.y, floor);
-            o.z = bn_dx1(v.z, d.z, mu.z, rs.z, g.z, b.z, ca.z, cb.z, floor);
-            o.w = bn_dx1(v.w, d.w, mu.w, rs.w, g.w, b.w, ca.w, cb.w, floor);
-            if (ADDEND) { const float4 e = __ldg(addend + i); o.x += e.x; o.y += e.y; o.z += e.z; o.w += e.w; }
-            if (ACCUM) { const float4 e = dx[i]; o.x += e.x; o.y += e.y; o.z += e.z; o.w += e.w; }
-            dx[i] = o;
-        }
+        bn_dx_rows<ADDEND, ACCUM>(x + base, dy + base, ADDEND ? addend + base : nullptr, dx + base, n, step, mu, rs, g, b, ca, cb, floor);
     }
 }
 
@@ -427,28 +451,15 @@ bn_apply_sums_bwd_kernel(const float4* __restrict__ x, const float4* __restrict_
     for (int pass = 0; pass < passes; ++pass) {
         const int cg = pass * cgt + my_cg;
         if (cg >= cg_total) continue;
-        const float4 mu = __ldg(reinterpret_cast<const float4*>(stats) + cg);
-        const float4 rs = __ldg(reinterpret_cast<const float4*>(stats + C) + cg);
+        const float4 mu = __ldcg(reinterpret_cast<const float4*>(stats) + cg);
+        const float4 rs = __ldcg(reinterpret_cast<const float4*>(stats + C) + cg);
         const float4 g = __ldg(reinterpret_cast<const float4*>(gamma) + cg);
         const float4 b = __ldg(reinterpret_cast<const float4*>(beta) + cg);
         const float4 ca = *reinterpret_cast<const float4*>(coef + 4 * cg);
         const float4 cb = *reinterpret_cast<const float4*>(coef + C + 4 * cg);
         const int64_t base = (r0 + my_rl) * cg_total + cg, step = (int64_t)rl * cg_total;
         const int n = (int)((r1 - r0 - my_rl + rl - 1) / rl);
-#pragma unroll 4
-        for (int k = 0; k < n; ++k) {
-            const int64_t i = base + k * step;
-            const float4 v = __ldg(x + i);
-            const float4 d = __ldcg(dy + i);
-            float4 o;
-            o.x = bn_dx1(v.x, d.x, mu.x, rs.x, g.x, b.x, ca.x, cb.x, 0.f);
-            o.y = bn_dx1(v.y, d.y, mu.y, rs.y, g.y, b.y, ca.y, cb.y, 0.f);
-            o.z = bn_dx1(v.z, d.z, mu.z, rs.z, g.z, b.z, ca.z, cb.z, 0.f);
-            o.w = bn_dx1(v.w, d.w, mu.w, rs.w, g.w, b.w, ca.w, cb.w, 0.f);
-            if (ADDEND) { const float4 e = __ldg(addend + i); o.x += e.x; o.y += e.y; o.z += e.z; o.w += e.w; }
-            if (ACCUM) { const float4 e = dx[i]; o.x += e.x; o.y += e.y; o.z += e.z; o.w += e.w; }
-            dx[i] = o;
-        }
+        bn_dx_rows<ADDEND, ACCUM>(x + base, dy + base, ADDEND ? addend + base : nullptr, dx + base, n, step, mu, rs, g, b, ca, cb, 0.f);
     }
 }
 
@@ -497,13 +508,13 @@ bn_bwd_cluster_kernel(const float4* __restrict__ x, const float4* __restrict__ d
     const int64_t base = (r0 + my_rl) * cg_total + cg, step = (int64_t)rl * cg_total;
 
     if (!early_x) pdl_wait();
-    const float4 mu = __ldg(reinterpret_cast<const float4*>(stats) + cg);
-    const float4 rs = __ldg(reinterpret_cast<const float4*>(stats + C) + cg);
+    const float4 mu = __ldcg(reinterpret_cast<const float4*>(stats) + cg);
+    const float4 rs = __ldcg(reinterpret_cast<const float4*>(stats + C) + cg);
     const float4 gm = __ldg(reinterpret_cast<const float4*>(gamma) + cg);
     const float4 bt = __ldg(reinterpret_cast<const float4*>(beta) + cg);
     float4 xv[NV], dv[NV];
 #pragma unroll
-    for (int k = 0; k < NV; ++k) if (k < n) xv[k] = __ldg(x + base + k * step);
+    for (int k = 0; k < NV; ++k) if (k < n) xv[k] = __ldcg(x + base + k * step);
     if (early_x) pdl_wait();
 #pragma unroll
     for (int k = 0; k < NV; ++k) if (k < n) dv[k] = __ldcg(dy + base + k * step);   // not the read-only path: such a load may be moved above the wait
@@ -748,12 +759,12 @@ bn_reduce_big_kernel(const float4* __restrict__ x4, const float4* __restrict__ d
     {
         float4 p0, p1, gm, bt;
         if (BWD) {
-            p0 = __ldg(reinterpret_cast<const float4*>(stats) + my_cg);
-            p1 = __ldg(reinterpret_cast<const float4*>(stats + C) + my_cg);
+            p0 = __ldcg(reinterpret_cast<const float4*>(stats) + my_cg);
+            p1 = __ldcg(reinterpret_cast<const float4*>(stats + C) + my_cg);
             gm = __ldg(reinterpret_cast<const float4*>(gamma) + my_cg);
             bt = __ldg(reinterpret_cast<const float4*>(beta) + my_cg);
         } else {
-            p0 = __ldg(x4 + my_cg);                                                   // shift = first row
+            p0 = __ldcg(x4 + my_cg);                                                   // shift = first row
         }
         const float4* xp = x4 + (r0 + my_rl) * cg_total + my_cg;
         const float4* dp = dy4 + (r0 + my_rl) * cg_total + my_cg;
@@ -765,10 +776,10 @@ bn_reduce_big_kernel(const float4* __restrict__ x4, const float4* __restrict__ d
         for (int k0 = 0; k0 < n; k0 += NB) {
             float4 v[NB], g[BWD ? NB : 1];
 #pragma unroll
-            for (int j = 0; j < NB; ++j) if (k0 + j < n) v[j] = __ldg(xp + (k0 + j) * step);
+            for (int j = 0; j < NB; ++j) if (k0 + j < n) v[j] = __ldcg(xp + (k0 + j) * step);
             if (BWD) {
 #pragma unroll
-                for (int j = 0; j < NB; ++j) if (k0 + j < n) g[j] = __ldg(dp + (k0 + j) * step);
+                for (int j = 0; j < NB; ++j) if (k0 + j < n) g[j] = __ldcg(dp + (k0 + j) * step);
             }
 #pragma unroll
             for (int j = 0; j < NB; ++j) {
@@ -910,7 +921,7 @@ __device__ __forceinline__ void bn_big_finalise(const float* __restrict__ partia
             fin[C + cl] = (float)(sb * inv_rows);
             if (write_out) { out_a[cl] = (float)sa; out_b[cl] = (float)sb; }        // dbeta, dgamma
         } else {
-            const double shift = (double)__ldg(x + cl);
+            const double shift = (double)__ldcg(x + cl);
             const double ms = sa * inv_rows;
             double var = sb * inv_rows - ms * ms;
             if (var < 0.0) var = 0.0;
@@ -957,7 +968,7 @@ bn_apply_big_fwd_kernel(const float4* __restrict__ x, const float* __restrict__ 
     for (int k0 = n - 1; k0 >= 0; k0 -= NB) {              // from the end of the slab, in batches of predicated loads
         float4 v[NB];
 #pragma unroll
-        for (int j = 0; j < NB; ++j) if (k0 - j >= 0) v[j] = __ldg(x + base + (k0 - j) * step);
+        for (int j = 0; j < NB; ++j) if (k0 - j >= 0) v[j] = __ldcg(x + base + (k0 - j) * step);
 #pragma unroll
         for (int j = 0; j < NB; ++j) {
             if (k0 - j >= 0) {
@@ -998,8 +1009,8 @@ bn_apply_big_bwd_kernel(const float4* __restrict__ x, const float4* __restrict__
     if (r1 > rows) r1 = rows;
     const float4 ca = *reinterpret_cast<const float4*>(fin + my_cg * 4);
     const float4 cb = *reinterpret_cast<const float4*>(fin + C + my_cg * 4);
-    const float4 mu = __ldg(reinterpret_cast<const float4*>(stats) + my_cg);
-    const float4 rs = __ldg(reinterpret_cast<const float4*>(stats + C) + my_cg);
+    const float4 mu = __ldcg(reinterpret_cast<const float4*>(stats) + my_cg);
+    const float4 rs = __ldcg(reinterpret_cast<const float4*>(stats + C) + my_cg);
     const float4 g = __ldg(reinterpret_cast<const float4*>(gamma) + my_cg);
     const float4 b = __ldg(reinterpret_cast<const float4*>(beta) + my_cg);
     const int64_t base = (r0 + my_rl) * cg_total + my_cg, step = (int64_t)rl * cg_total;
@@ -1008,7 +1019,7 @@ bn_apply_big_bwd_kernel(const float4* __restrict__ x, const float4* __restrict__
     for (int k0 = n - 1; k0 >= 0; k0 -= NB) {
         float4 v[NB], d[NB];
 #pragma unroll
-        for (int j = 0; j < NB; ++j) if (k0 - j >= 0) { v[j] = __ldg(x + base + (k0 - j) * step); d[j] = __ldg(dy + base + (k0 - j) * step); }
+        for (int j = 0; j < NB; ++j) if (k0 - j >= 0) { v[j] = __ldcg(x + base + (k0 - j) * step); d[j] = __ldcg(dy + base + (k0 - j) * step); }
 #pragma unroll
         for (int j = 0; j < NB; ++j) {
             if (k0 - j >= 0) {
@@ -1018,7 +1029,7 @@ bn_apply_big_bwd_kernel(const float4* __restrict__ x, const float4* __restrict__
                 o.y = bn_dx1(v[j].y, d[j].y, mu.y, rs.y, g.y, b.y, ca.y, cb.y, floor);
                 o.z = bn_dx1(v[j].z, d[j].z, mu.z, rs.z, g.z, b.z, ca.z, cb.z, floor);
                 o.w = bn_dx1(v[j].w, d[j].w, mu.w, rs.w, g.w, b.w, ca.w, cb.w, floor);
-                if (ADDEND) { const float4 e = __ldg(addend + i); o.x += e.x; o.y += e.y; o.z += e.z; o.w += e.w; }
+                if (ADDEND) { const float4 e = __ldcg(addend + i); o.x += e.x; o.y += e.y; o.z += e.z; o.w += e.w; }
                 if (ACCUM) { const float4 e = dx[i]; o.x += e.x; o.y += e.y; o.z += e.z; o.w += e.w; }
                 if (stream_out) __stcs(dx + i, o); else dx[i] = o;
             }
@@ -1106,10 +1117,10 @@ add_kernel(const float* __restrict__ a, const float* __restrict__ b, float* __re
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     for (int64_t i = t0; i < n4; i += stride) {
-        const float4 u = __ldg(reinterpret_cast<const float4*>(a) + i), v = __ldg(reinterpret_cast<const float4*>(b) + i);
+        const float4 u = __ldcg(reinterpret_cast<const float4*>(a) + i), v = __ldcg(reinterpret_cast<const float4*>(b) + i);
         reinterpret_cast<float4*>(out)[i] = make_float4(u.x + v.x, u.y + v.y, u.z + v.z, u.w + v.w);
     }
-    for (int64_t i = n4 * 4 + t0; i < n; i += stride) out[i] = a[i] + b[i];
+    for (int64_t i = n4 * 4 + t0; i < n; i += stride) out[i] = __ldcg(a + i) + __ldcg(b + i);
 }
 
 // Stand-alone ReLU (the post-activation residual block ends in one): y = max(x, 0); dx = dy * [x > 0] (+ addend) (+= dx).
@@ -1122,10 +1133,10 @@ relu_fwd_kernel(const float* __restrict__ x, float* __restrict__ y, int64_t n)
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     for (int64_t i = t0; i < n4; i += stride) {
-        const float4 v = __ldg(reinterpret_cast<const float4*>(x) + i);
+        const float4 v = __ldcg(reinterpret_cast<const float4*>(x) + i);
         reinterpret_cast<float4*>(y)[i] = make_float4(fmaxf(v.x, 0.f), fmaxf(v.y, 0.f), fmaxf(v.z, 0.f), fmaxf(v.w, 0.f));
     }
-    for (int64_t i = n4 * 4 + t0; i < n; i += stride) y[i] = fmaxf(x[i], 0.f);
+    for (int64_t i = n4 * 4 + t0; i < n; i += stride) y[i] = fmaxf(__ldcg(x + i), 0.f);
 }
 
 template <bool ADDEND, bool ACCUM>
@@ -1139,15 +1150,15 @@ relu_bwd_kernel(const float* __restrict__ x, const float* __restrict__ dy, const
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     for (int64_t i = t0; i < n4; i += stride) {
-        const float4 v = __ldg(reinterpret_cast<const float4*>(x) + i), d = __ldg(reinterpret_cast<const float4*>(dy) + i);
+        const float4 v = __ldcg(reinterpret_cast<const float4*>(x) + i), d = __ldcg(reinterpret_cast<const float4*>(dy) + i);
         float4 o = make_float4(v.x > 0.f ? d.x : 0.f, v.y > 0.f ? d.y : 0.f, v.z > 0.f ? d.z : 0.f, v.w > 0.f ? d.w : 0.f);
-        if (ADDEND) { const float4 e = __ldg(reinterpret_cast<const float4*>(addend) + i); o.x += e.x; o.y += e.y; o.z += e.z; o.w += e.w; }
+        if (ADDEND) { const float4 e = __ldcg(reinterpret_cast<const float4*>(addend) + i); o.x += e.x; o.y += e.y; o.z += e.z; o.w += e.w; }
         if (ACCUM) { const float4 e = reinterpret_cast<const float4*>(dx)[i]; o.x += e.x; o.y += e.y; o.z += e.z; o.w += e.w; }
         reinterpret_cast<float4*>(dx)[i] = o;
     }
     for (int64_t i = n4 * 4 + t0; i < n; i += stride) {
-        float o = x[i] > 0.f ? dy[i] : 0.f;
-        if (ADDEND) o += addend[i];
+        float o = __ldcg(x + i) > 0.f ? __ldcg(dy + i) : 0.f;
+        if (ADDEND) o += __ldcg(addend + i);
         if (ACCUM) o += dx[i];
         dx[i] = o;
     }
@@ -1163,11 +1174,11 @@ accumulate_kernel(float* __restrict__ dst, const float* __restrict__ src, int64_
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     for (int64_t i = t0; i < n4; i += stride) {
-        float4 v = __ldg(reinterpret_cast<const float4*>(src) + i);
+        float4 v = __ldcg(reinterpret_cast<const float4*>(src) + i);
         if (ACCUM) { const float4 e = reinterpret_cast<float4*>(dst)[i]; v.x += e.x; v.y += e.y; v.z += e.z; v.w += e.w; }
         reinterpret_cast<float4*>(dst)[i] = v;
     }
-    for (int64_t i = n4 * 4 + t0; i < n; i += stride) dst[i] = ACCUM ? dst[i] + src[i] : src[i];
+    for (int64_t i = n4 * 4 + t0; i < n; i += stride) dst[i] = ACCUM ? dst[i] + __ldcg(src + i) : __ldcg(src + i);
 }
 
 // out[j] = (slots[0][j] + slots[1][j] + ... + slots[M-1][j]) / M, ascending m.  Reads M*G floats,

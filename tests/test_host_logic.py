@@ -189,3 +189,28 @@ def test_microbatch_tuner_search_order():
     assert halving_candidates(1) == [1]
     for b in (7, 30, 128):
         assert all(b % m == 0 for m in halving_candidates(b))
+
+
+def test_kernels_that_start_early_read_the_steps_results_with_ordered_loads():
+    """A kernel launched with programmatic dependent launch may not read what the step computes through the read-only path: the
+    compiler is free to move such a load above the wait on the preceding kernel.  Parameters are all it may read that way."""
+    csrc = os.path.join(os.path.dirname(hpf.__file__), "csrc")
+    text = {f: open(os.path.join(csrc, f)).read() for f in sorted(os.listdir(csrc)) if f.endswith((".cu", ".cuh"))}
+    # device functions by name; what an early kernel calls counts as its own
+    bodies = {}
+    for t in text.values():
+        t = re.sub(r"//[^\n]*", "", t)
+        for m in re.finditer(r"\n((?:[^\n{}]+\n)+)\{\n(.*?)\n\}\n", t, re.S):
+            names = [n for n in re.findall(r"(\w+)\s*\(", m.group(1)) if n != "__launch_bounds__"]
+            bodies[names[0] if names else ""] = m.group(2)
+    early = [k for k, body in bodies.items() if "pdl_wait()" in body and k != "pdl_wait"]
+    assert {"pipe_cta", "bn_apply_sums_bwd_kernel", "bn_bwd_cluster_kernel", "relu_fwd_kernel"} <= set(early), early
+    todo, seen = list(early), set()
+    while todo:
+        k = todo.pop()
+        if k in seen:
+            continue
+        seen.add(k)
+        todo += [c for c in re.findall(r"\b(\w+)\s*(?:<[^;()<>]*>)?\(", bodies[k]) if c in bodies]
+        for arg in re.findall(r"__ldg\((?:reinterpret_cast<[^>]*>\()?&?([\w.]+)", bodies[k]):
+            assert arg.split(".")[-1] in ("gamma", "beta", "bn_gamma", "bn_beta"), (k, arg)
