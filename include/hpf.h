@@ -131,6 +131,12 @@ int hpf_model_destroy(hpf_model *model);
  *                          innermost) to the tensor core as MN-major operands, as they land in shared memory; 0: the earlier
  *                          kernel, which transposes every tile in shared memory first (kept as a cross-check; also used for
  *                          channel counts that are neither 16 nor a multiple of 32).
+ *   HPF_OPT_GROUP_LAUNCHES 1 (default): a step's launches cover all micro-batches of a stage, and their work is split for that;
+ *                          0: they cover one, split like those of hpf_forward_cell / hpf_backward_cell.  How the work of a
+ *                          convolution is split decides in which order the moments of a BN and the slices of a weight
+ *                          gradient are added: within one setting every way to run a step gives the same bits, between the two
+ *                          the results agree to fp32 rounding.  A step with 0 is the one-GPU counterpart of a stage-per-GPU run,
+ *                          bit for bit.
  *   HPF_OPT_CELL_CTAS      N > 0: the forward tensor-core convolutions of a (partition, micro-batch) cell that follow each
  *                          other with no other kernel between them run as ONE persistent kernel of N CTAs that stays
  *                          resident for the cell, walks the list of convolutions and meets at a grid-wide barrier between
@@ -140,7 +146,7 @@ int hpf_model_destroy(hpf_model *model);
 typedef enum { HPF_OPT_GRAPH = 1, HPF_OPT_CONV_PATH = 2, HPF_OPT_SINGLE_STREAM = 3, HPF_OPT_KEEP_MESSAGES = 4,
                HPF_OPT_FUSE_ADD = 5, HPF_OPT_PDL = 6, HPF_OPT_WGRAD_PASSES = 7, HPF_OPT_FUSE_BN = 8, HPF_OPT_CELL_TIMES = 9,
                HPF_OPT_BN_CLUSTER = 10, HPF_OPT_CELL_CTAS = 11, HPF_OPT_PDL_LATE_FROM = 12,
-               HPF_OPT_STAGE_LANES = 13, HPF_OPT_WGRAD_DIRECT = 14 } hpf_option;
+               HPF_OPT_STAGE_LANES = 13, HPF_OPT_WGRAD_DIRECT = 14, HPF_OPT_GROUP_LAUNCHES = 15 } hpf_option;
 int hpf_set_option(hpf_model *model, int32_t option, int32_t value);
 
 /* ---- integer bookkeeping (Section 5.1 lists, Section 5.3 pipelining) ----------------------------- */
@@ -213,6 +219,7 @@ int hpf_forward_backward(hpf_model *model, const float *d_x, const int32_t *d_la
  *                          for micro-batch m (hpf_boundary_desc), which must be in place.
  *   hpf_backward_cell      reverse sweep of partition p on micro-batch m; for p < P-1 the gradient buffers listed by
  *                          hpf_backward_message_desc(cut p) must hold what the partition above computed (Eq. 7).
+ *                          The launches of both cover one micro-batch and are planned for that (HPF_OPT_GROUP_LAUNCHES).
  *   hpf_join_partition     orders partition p's weight-gradient side stream before what follows on its stream.
  *   hpf_partition_param_range   partition p's contiguous slice of the flat parameter / gradient vectors: the message
  *                          of the per-partition allreduce across replicas (Section 5.3, one communicator per partition).

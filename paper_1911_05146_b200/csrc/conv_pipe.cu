@@ -1238,7 +1238,7 @@ inline unsigned int bn_bytes(int c_in) { return (unsigned int)(4 * c_in * 4 + 4 
 
 size_t conv_pipe_partial_floats(int units_per_m, int channels) { return partial_floats(units_per_m, channels); }
 
-static bool plan_geom(const ConvShape& s, int pass, int passes, int M, ConvPipeGeom* g)
+static bool plan_geom(const ConvShape& s, int pass, int passes, int launched, ConvPipeGeom* g)
 {
     PipeView v;
     if (pass == PASS_WGRAD || !pipe_view(s, pass, &v)) return false;
@@ -1292,7 +1292,7 @@ static bool plan_geom(const ConvShape& s, int pass, int passes, int M, ConvPipeG
                 const unsigned int a_stage = (unsigned int)(nj * kRowStep) * 128u;
                 const int units = (g->tiles_per_m + T - 1) / T;
                 const int per_slice = kPlanSms / g->slices > 0 ? kPlanSms / g->slices : 1;
-                const double rounds = (double)(((long long)M * units + per_slice - 1) / per_slice);
+                const double rounds = (double)(((long long)launched * units + per_slice - 1) / per_slice);
                 const double step = !three ? clk(n) : (stacked ? clk(2 * n) + clk(n) : 3.0 * (n == 128 ? 80.0 : clk(n)));
                 const double tap_mma = 2.0 * T * step, epi = 1100.0 * T * ((n + 31) / 32) / 2.0;
                 // weights: resident, or a ring whose stage holds the taps of a window row (fewer waits) or one tap
@@ -1327,7 +1327,7 @@ static bool plan_geom(const ConvShape& s, int pass, int passes, int M, ConvPipeG
     if (!g->T) return false;
     // Few units with a long K loop: several CTAs share it (partial tiles in L2, added in order by the last to finish).
     g->ksplit = 1;
-    const int tasks = M * g->units_per_m * g->slices, ksteps = 2 * taps * chunks;
+    const int tasks = launched * g->units_per_m * g->slices, ksteps = 2 * taps * chunks;
     if (2 * tasks <= kPlanSms && ksteps >= 128) {
         int S = kPlanSms / tasks;
         if (S > 8) S = 8;
@@ -1340,9 +1340,9 @@ static bool plan_geom(const ConvShape& s, int pass, int passes, int M, ConvPipeG
     g->unit_block = 1;
     if (g->ksplit == 1) {
         const int per_slice = kPlanSms / g->slices > 0 ? kPlanSms / g->slices : 1;
-        const int most = (M * g->units_per_m + per_slice - 1) / per_slice;
+        const int most = (launched * g->units_per_m + per_slice - 1) / per_slice;
         for (int u = 2; u <= 16 && u <= most; ++u) {
-            const int blocks = M * ((g->units_per_m + u - 1) / u);
+            const int blocks = launched * ((g->units_per_m + u - 1) / u);
             if (10 * u * ((blocks + per_slice - 1) / per_slice) <= 11 * most) g->unit_block = u;
         }
     }
@@ -1353,18 +1353,18 @@ static bool plan_geom(const ConvShape& s, int pass, int passes, int M, ConvPipeG
 // The search takes several microseconds and a single convolution's call asks for its plan and its scratch sizes: as long as the
 // convolution itself for a small one (1x1 on 4 x 4 maps, forward and both gradients: 64 us, 32 with the last plans kept).
 // Each thread keeps a fixed number of them.
-bool conv_pipe_geom(const ConvShape& s, int pass, int passes, int M, ConvPipeGeom* g)
+bool conv_pipe_geom(const ConvShape& s, int pass, int passes, int launched, ConvPipeGeom* g)
 {
     struct Kept { int key[11]; bool used, ok; ConvPipeGeom g; };
     constexpr int kKept = 64;
     static thread_local Kept kept[kKept];
-    const int key[11] = {s.N, s.H, s.W, s.C, s.K, s.R, s.stride, s.pad, pass, passes, M};
+    const int key[11] = {s.N, s.H, s.W, s.C, s.K, s.R, s.stride, s.pad, pass, passes, launched};
     unsigned int h = 2166136261u;
     for (int k : key) h = (h ^ (unsigned int)k) * 16777619u;
     Kept& e = kept[(h >> 16) % kKept];
     if (!e.used || memcmp(e.key, key, sizeof key) != 0) {
         memcpy(e.key, key, sizeof key);
-        e.ok = plan_geom(s, pass, passes, M, &e.g);
+        e.ok = plan_geom(s, pass, passes, launched, &e.g);
         e.used = true;
     }
     *g = e.g;
@@ -1374,11 +1374,15 @@ bool conv_pipe_geom(const ConvShape& s, int pass, int passes, int M, ConvPipeGeo
 bool conv_pipe_can_fuse_bn_output(const ConvPipeGeom& g) { return g.n_chunk <= 128; }      // a warp keeps the moments of two groups of 32 channels
 bool conv_pipe_can_fuse_bn_input(const ConvShape& s) { return s.stride == 1 && s.C % 16 == 0 && s.C <= 512 && s.W <= 254; }      // (no column strips)
 
-size_t conv_pipe_splitk_bytes(const ConvShape& s, int pass, int passes, int M)
+size_t conv_pipe_splitk_bytes(const ConvPipeGeom& g)
+{
+    if (g.ksplit < 2) return 0;
+    return (kSplitKTicketBytes + (size_t)g.units_per_m * g.slices * g.ksplit * g.T * kTileM * g.n_chunk * sizeof(float) + 255) & ~(size_t)255;
+}
+size_t conv_pipe_splitk_bytes(const ConvShape& s, int pass, int passes, int launched)
 {
     ConvPipeGeom g;
-    if (!conv_pipe_geom(s, pass, passes, M, &g) || g.ksplit < 2) return 0;
-    return (kSplitKTicketBytes + (size_t)g.units_per_m * g.slices * g.ksplit * g.T * kTileM * g.n_chunk * sizeof(float) + 255) & ~(size_t)255;
+    return conv_pipe_geom(s, pass, passes, launched, &g) ? conv_pipe_splitk_bytes(g) : 0;
 }
 
 struct ConvPipeLaunch { PipeParams p; unsigned int smem; int bn_in; };
@@ -1423,14 +1427,14 @@ unsigned int columns_pow2(unsigned int need)
 }
 }  // namespace
 
-cudaError_t conv_pipe_prepare(ConvPipePlan* plan, const ConvShape& s, int pass, int passes, int M, const float* in, const float* w_hi,
+cudaError_t conv_pipe_prepare(ConvPipePlan* plan, const ConvShape& s, int pass, int passes, int M, int launched, const float* in, const float* w_hi,
                               const float* w_lo, float* out, const float* extra, bool accumulate, const ConvPipeBn* bn, void* splitk,
                               size_t splitk_bytes, bool w_ready)
 {
     plan->valid = 0;
     ConvPipeGeom g;
     PipeView v;
-    if ((passes != 1 && passes != 3) || !conv_pipe_geom(s, pass, passes, M, &g) || !pipe_view(s, pass, &v)) return cudaErrorNotSupported;
+    if ((passes != 1 && passes != 3) || !conv_pipe_geom(s, pass, passes, launched, &g) || !pipe_view(s, pass, &v)) return cudaErrorNotSupported;
     ConvPipeLaunch* L = reinterpret_cast<ConvPipeLaunch*>(plan->storage);
     memset(L, 0, sizeof *L);
     const long long kdim = (long long)s.R * s.R * v.c_in;
@@ -1494,7 +1498,7 @@ cudaError_t conv_pipe_prepare(ConvPipePlan* plan, const ConvShape& s, int pass, 
         L->bn_in = 1;
     }
     if (g.ksplit > 1) {
-        if (!splitk || conv_pipe_splitk_bytes(s, pass, passes, M) > splitk_bytes) return cudaErrorInvalidValue;
+        if (!splitk || conv_pipe_splitk_bytes(g) > splitk_bytes) return cudaErrorInvalidValue;
         p.sk_base = reinterpret_cast<char*>(splitk); p.sk_ms = (long long)splitk_bytes;
     }
     if (L->smem > kPipeSmem + 1024) return cudaErrorNotSupported;

@@ -6,8 +6,8 @@
 namespace hpf {
 
 // Work split of one convolution.  It depends on the shape of ONE micro-batch, on the precision and on how many micro-batches
-// the model has - never on how many of them a launch covers - so that every sum is formed in the same order whichever
-// micro-batches share a launch.
+// the launches it is planned for cover - never on which of them share a launch - so that every sum is formed in the same order
+// whichever micro-batches a planned launch is given.
 struct ConvPipeGeom {
     int tiles_per_m;             // tiles of 128 positions of one micro-batch
     int T;                       // tiles per unit (they share every weight tile)
@@ -21,7 +21,7 @@ struct ConvPipeGeom {
     int flat, box_h;             // operand copies: 128 consecutive pixels, or box_h padded map rows each
     int pos_per_m, Wp, Hp, halo, strips, strip_w, col0;
 };
-bool conv_pipe_geom(const ConvShape& s, int pass, int passes, int M, ConvPipeGeom* g);
+bool conv_pipe_geom(const ConvShape& s, int pass, int passes, int launched, ConvPipeGeom* g);
 
 // BN work that rides in the forward kernel.
 //   out_partials: the output is the input of a BN: per block of units and output channel the mean and the sum of squared
@@ -51,7 +51,8 @@ bool conv_pipe_can_fuse_bn_output(const ConvPipeGeom& g);
 // Whether a BN+ReLU may be applied to this convolution's operand on its way to the tensor core.
 bool conv_pipe_can_fuse_bn_input(const ConvShape& s);
 // Scratch of one micro-batch for launches that split their K loop (0: none does); zeroed once, successive micro-batches follow.
-size_t conv_pipe_splitk_bytes(const ConvShape& s, int pass, int passes, int M);
+size_t conv_pipe_splitk_bytes(const ConvPipeGeom& g);
+size_t conv_pipe_splitk_bytes(const ConvShape& s, int pass, int passes, int launched);
 
 // A prepared launch; the pointers are those of micro-batch 0, whose successors follow contiguously.
 struct ConvPipePlan {
@@ -59,9 +60,10 @@ struct ConvPipePlan {
     alignas(64) unsigned char storage[960];
 };
 cudaError_t conv_pipe_init();
-// s.N = samples of one micro-batch.  in / out / extra as conv_tc_prepare; w_ready: the prepared weights were complete before
-// the kernel that precedes this one in its stream was enqueued.
-cudaError_t conv_pipe_prepare(ConvPipePlan* plan, const ConvShape& s, int pass, int passes, int M, const float* in, const float* w_hi,
+// s.N = samples of one micro-batch, M micro-batches in the tensors, `launched` of them in the launches this is planned for.
+// in / out / extra as conv_tc_prepare; w_ready: the prepared weights were complete before the kernel that precedes this one in
+// its stream was enqueued.
+cudaError_t conv_pipe_prepare(ConvPipePlan* plan, const ConvShape& s, int pass, int passes, int M, int launched, const float* in, const float* w_hi,
                               const float* w_lo, float* out, const float* extra, bool accumulate, const ConvPipeBn* bn,
                               void* splitk, size_t splitk_bytes, bool w_ready);
 // Micro-batches m_first .. m_first + m_count - 1 in one launch.

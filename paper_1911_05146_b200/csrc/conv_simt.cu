@@ -242,15 +242,15 @@ wgrad_reduce_kernel(const float* __restrict__ partials, float* __restrict__ dw, 
 }
 
 // Slices of the pixels of one micro-batch.  Few output tiles (a stem convolution: one to three) leave it to the slices to
-// fill the GPU, two blocks per SM over the M micro-batches of a launch, down to 128 pixels each.
+// fill the GPU, two blocks per SM over the micro-batches of a launch, down to 128 pixels each.
 struct WgradSplit { int splits, k_per_split; };
-WgradSplit wgrad_split(const ConvShape& s, int M)
+WgradSplit wgrad_split(const ConvShape& s, int launched)
 {
     constexpr int kStep = 64;
     const int64_t pixels = (int64_t)s.N * s.P * s.Q;
     const int64_t outs = (int64_t)s.K * s.R * s.R * s.C;
     int64_t splits = pixels / 1024;                       // >= 1024 pixels per slice
-    const int64_t out_tiles = (int64_t)((s.K + 63) / 64) * ((s.R * s.R * s.C + 63) / 64) * M;
+    const int64_t out_tiles = (int64_t)((s.K + 63) / 64) * ((s.R * s.R * s.C + 63) / 64) * launched;
     if (splits * out_tiles < 296) splits = (296 + out_tiles - 1) / out_tiles;
     if (splits * out_tiles > 1184) splits = (1184 + out_tiles - 1) / out_tiles;
     if (splits > pixels / 128) splits = pixels / 128;
@@ -294,9 +294,9 @@ inline void count(int64_t* n_launch, int k) { if (n_launch) *n_launch += k; }
 
 }  // namespace
 
-size_t conv_simt_scratch_bytes(const ConvShape& s, int M)
+size_t conv_simt_scratch_bytes(const ConvShape& s, int launched)
 {
-    const WgradSplit w = wgrad_split(s, M);
+    const WgradSplit w = wgrad_split(s, launched);
     return (size_t)w.splits * s.K * s.R * s.R * s.C * sizeof(float);
 }
 
@@ -321,9 +321,9 @@ cudaError_t conv_dgrad_simt(const float* dy, const float* w, float* dx, const fl
 }
 
 cudaError_t conv_wgrad_simt(const float* x, const float* dy, float* dw, const ConvShape& s, void* scratch,
-                            cudaStream_t st, int64_t* n_launch, int M, int m_count, long long scratch_ms, long long dw_ms)
+                            cudaStream_t st, int64_t* n_launch, int launched, int m_count, long long scratch_ms, long long dw_ms)
 {
-    const WgradSplit ws = wgrad_split(s, M);
+    const WgradSplit ws = wgrad_split(s, launched);
     SimtArgs g = make_args(dy, x, reinterpret_cast<float*>(scratch), nullptr, false, s);
     g.Md = s.K; g.Nd = s.R * s.R * s.C; g.Kd = s.N * s.P * s.Q; g.k_per_split = ws.k_per_split; g.splits = ws.splits;
     g.a_ms = (long long)s.N * s.P * s.Q * s.K; g.b_ms = (long long)s.N * s.H * s.W * s.C; g.out_ms = scratch_ms;

@@ -1175,7 +1175,7 @@ cudaError_t encode(CUtensorMap* tm, const float* base, int rank, const cuuint64_
 }
 
 // How many pixel splits (CTAs along x) a weight-gradient launch of n_tiles pixel tiles gets.
-void wgrad_splits(const ConvShape& s, int n_tiles, int ctas_per_split, int M, int* splits_out, int* tiles_per_split_out)
+void wgrad_splits(const ConvShape& s, int n_tiles, int ctas_per_split, int launched, int* splits_out, int* tiles_per_split_out)
 {
     const int taps = s.R * s.R;
     // enough CTAs to spread the pixel walk, few enough that the partials stay a fraction of the operand bytes
@@ -1188,11 +1188,11 @@ void wgrad_splits(const ConvShape& s, int n_tiles, int ctas_per_split, int M, in
     if (cap < want) cap = want;
     if (splits > cap) splits = cap;
     if (splits > 296) splits = 296;          // two CTAs per SM
-    if (M > 1) {
-        // The launch covers the model's M micro-batches, each with its own sums.  It runs beside the chain of data gradients,
+    if (launched > 1) {
+        // The launch covers several micro-batches, each with its own sums.  It runs beside the chain of data gradients,
         // which wants whole SMs, and its partial sums are written and read again: one and a half CTAs per SM in all.
         // 592 / 296 / 222 / 148 / 74 CTAs: resnet152 39.2 / 37.9 / 36.6 / 36.8 / 36.9 ms, resnet110 6.71 / 6.61 / 6.53 / 6.50 / 6.71.
-        int ms = 222 / (ctas_per_split * M);
+        int ms = 222 / (ctas_per_split * launched);
         if (ms < 1) ms = 1;
         if (splits > ms) splits = ms;
     }
@@ -1208,7 +1208,7 @@ struct WgradGeom {
     unsigned int raw_bytes, t_bytes, tmem_cols;
 };
 
-bool wgrad_geom(const ConvShape& s, int passes, WgradGeom* g, int M = 1)
+bool wgrad_geom(const ConvShape& s, int passes, WgradGeom* g, int launched)
 {
     if (s.C % 16 || s.K % 16) return false;
     if (s.R != 1 && s.R != 3) return false;
@@ -1255,7 +1255,7 @@ bool wgrad_geom(const ConvShape& s, int passes, WgradGeom* g, int M = 1)
     g->tmem_cols = pow2_cols(g->taps_per_cta * g->n_cols);
     const int tiles_w = (s.Q + g->box.w - 1) / g->box.w, tiles_h = (s.P + g->box.h - 1) / g->box.h, tiles_n = (s.N + g->box.n - 1) / g->box.n;
     g->n_tiles = tiles_w * tiles_h * tiles_n;
-    wgrad_splits(s, g->n_tiles, g->tap_groups * (s.K / g->m_chunk) * (s.C / g->n_cols), M, &g->splits, &g->tiles_per_split);
+    wgrad_splits(s, g->n_tiles, g->tap_groups * (s.K / g->m_chunk) * (s.C / g->n_cols), launched, &g->splits, &g->tiles_per_split);
     return true;
 }
 
@@ -1270,7 +1270,7 @@ struct WgradDirectGeom {
 // the first combination whose accumulators take at most half of an SM's tensor memory (other kernels' CTAs share the
 // SM) and that gets at least three pipeline stages into 100 KB of shared memory - failing that two stages, failing
 // that two stages into 200 KB with all of the tensor memory.
-bool wgrad_direct_geom(const ConvShape& s, int passes, WgradDirectGeom* g, int M = 1)
+bool wgrad_direct_geom(const ConvShape& s, int passes, WgradDirectGeom* g, int launched)
 {
     if (s.C % 16 || s.K % 16) return false;
     if ((s.C > 16 && s.C % 32) || (s.K > 16 && s.K % 32)) return false;
@@ -1332,7 +1332,7 @@ bool wgrad_direct_geom(const ConvShape& s, int passes, WgradDirectGeom* g, int M
     g->tmem_cols = pow2_cols(g->taps_per_cta * g->n_blocks * 32);
     const int tiles_w = (s.Q + g->box.w - 1) / g->box.w, tiles_h = (s.P + g->box.h - 1) / g->box.h, tiles_n = (s.N + g->box.n - 1) / g->box.n;
     g->n_tiles = tiles_w * tiles_h * tiles_n;
-    wgrad_splits(s, g->n_tiles, g->tap_groups * (s.K / g->m_chunk) * (s.C / g->n_cols), M, &g->splits, &g->tiles_per_split);
+    wgrad_splits(s, g->n_tiles, g->tap_groups * (s.K / g->m_chunk) * (s.C / g->n_cols), launched, &g->splits, &g->tiles_per_split);
     return true;
 }
 
@@ -1345,7 +1345,7 @@ inline void count(int64_t* n_launch, int k) { if (n_launch) *n_launch += k; }
 // ------------------------------------------------------------------------------------------------
 bool conv_tc_supported(const ConvShape& s, int pass)
 {
-    if (pass == PASS_WGRAD) { WgradGeom g; return wgrad_geom(s, 3, &g); }
+    if (pass == PASS_WGRAD) { WgradGeom g; return wgrad_geom(s, 3, &g, 1); }
     FwdView v;
     if (!fwd_view(s, pass, &v)) return false;
     PixelBox b;
@@ -1416,16 +1416,16 @@ size_t conv_tc_splitk_bytes(const ConvShape& s, int pass, int passes)
     return kSplitKTicketBytes + (size_t)tiles * (v.c_out / n_chunk) * S * kTileM * n_chunk * sizeof(float);
 }
 
-size_t conv_tc_scratch_bytes(const ConvShape& s, int M)
+size_t conv_tc_scratch_bytes(const ConvShape& s, int launched)
 {
     size_t need = 0;
     for (int passes = 1; passes <= 3; passes += 2) {
         WgradGeom g;
-        if (!wgrad_geom(s, passes, &g, M)) continue;
+        if (!wgrad_geom(s, passes, &g, launched)) continue;
         const size_t b = g.splits > 1 ? (size_t)g.splits * s.K * s.R * s.R * s.C * sizeof(float) : 0;
         if (b > need) need = b;
         WgradDirectGeom d;
-        if (!wgrad_direct_geom(s, passes, &d, M)) continue;
+        if (!wgrad_direct_geom(s, passes, &d, launched)) continue;
         const size_t bd = d.splits > 1 ? (size_t)d.splits * s.K * s.R * s.R * s.C * sizeof(float) : 0;
         if (bd > need) need = bd;
     }
@@ -1444,11 +1444,11 @@ cudaError_t conv_tc_prepare(ConvTcPlan* plan, const ConvShape& s, int pass, int 
                             const ConvTcHints* hints)
 {
     plan->valid = 0; plan->s = s; plan->pass = pass; plan->direct = 0;
-    const int M = hints && hints->micro_batches > 1 ? hints->micro_batches : 1;
+    const int M = hints && hints->micro_batches > 1 ? hints->micro_batches : 1, launched = hints ? hints->launched : 1;
     const long long dw_ms = hints ? hints->slot_stride : 0;
     if (passes != 1 && passes != 3) return cudaErrorInvalidValue;
     WgradDirectGeom dg;
-    if (pass == PASS_WGRAD && !(hints && hints->wgrad_transposing) && wgrad_direct_geom(s, passes, &dg, M)) {
+    if (pass == PASS_WGRAD && !(hints && hints->wgrad_transposing) && wgrad_direct_geom(s, passes, &dg, launched)) {
         ConvTcWgradDirectLaunch* L = reinterpret_cast<ConvTcWgradDirectLaunch*>(plan->storage);
         WgradDirectParams& P = L->p;
         memset(&P, 0, sizeof P);
@@ -1494,7 +1494,7 @@ cudaError_t conv_tc_prepare(ConvTcPlan* plan, const ConvShape& s, int pass, int 
     }
     if (pass == PASS_WGRAD) {
         WgradGeom g;
-        if (!wgrad_geom(s, passes, &g, M)) return cudaErrorNotSupported;
+        if (!wgrad_geom(s, passes, &g, launched)) return cudaErrorNotSupported;
         ConvTcWgradLaunch* L = reinterpret_cast<ConvTcWgradLaunch*>(plan->storage);
         WgradParams& P = L->p;
         memset(&P, 0, sizeof P);

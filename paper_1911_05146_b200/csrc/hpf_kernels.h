@@ -169,8 +169,8 @@ cudaError_t head_bwd(const float* Wfc, const int32_t* labels, const float* logit
                      cudaStream_t st, int64_t* n_launch, const HeadGroup& grp = HeadGroup());
 
 // ---------------- CUDA-core convolutions (conv_simt.cu) ----------------
-// partial sums of a weight gradient of one micro-batch, of a model with M of them
-size_t conv_simt_scratch_bytes(const ConvShape& s, int M = 1);
+// partial sums of a weight gradient of one micro-batch; launched: micro-batches of the launches it is planned for
+size_t conv_simt_scratch_bytes(const ConvShape& s, int launched = 1);
 // y = conv(x, w) (+ residual)
 cudaError_t conv_fwd_simt(const float* x, const float* w, float* y, const float* residual, const ConvShape& s,
                           cudaStream_t st, int64_t* n_launch);
@@ -179,6 +179,6 @@ cudaError_t conv_dgrad_simt(const float* dy, const float* w, float* dx, const fl
                             const ConvShape& s, cudaStream_t st, int64_t* n_launch);
 // x, dy: micro-batch 0 of m_count contiguous ones of s.N samples; floats between their partial sums and between their dw
 cudaError_t conv_wgrad_simt(const float* x, const float* dy, float* dw, const ConvShape& s, void* scratch, cudaStream_t st, int64_t* n_launch,
-                            int M = 1, int m_count = 1, long long scratch_ms = 0, long long dw_ms = 0);
+                            int launched = 1, int m_count = 1, long long scratch_ms = 0, long long dw_ms = 0);
 
 }  // namespace hpf

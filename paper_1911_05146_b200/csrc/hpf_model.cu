@@ -89,21 +89,35 @@ struct hpf_model {
     std::vector<int> grad_alias;              // tensor -> ADD op whose gradient buffer it shares, or -1
     std::vector<int> fused_into;              // conv -> residual ADD computed in its epilogue (its own output is not stored), or -1
     std::vector<int> add_done_by;             // ADD -> the conv that computes it, or -1
-    std::vector<int> bn_fwd_from;              // BN -> conv whose forward kernel also produces the statistics of the BN (its input), or -1
-    std::vector<int> conv_fwd_bn;              // the inverse map
-    std::vector<int> bn_into, conv_in_bn;      // BN -> the convolution that applies it to its own input operand (no BN kernel), and the inverse
-    std::vector<int> bn_bwd_from, conv_bwd_bn;  // BN+ReLU -> the convolution whose data gradient also forms the sums of its backward, or -1, and the inverse map
-    std::vector<size_t> bn_sums_off;           // where it leaves them, all micro-batches
-    std::vector<size_t> bn_moments_off;        // BN -> per-unit moments of its input left by the producing convolution, all micro-batches
+    // Which kernels the convolutions run on and what BN work rides in them, planned for launches that cover `launched`
+    // micro-batches of a stage.  The first set is the step's, whose launches cover all micro-batches; the second that of the
+    // calls which run one cell (hpf_forward_cell, hpf_backward_cell), where a launch has one micro-batch and a GPU to itself:
+    // with the step's blocks of work a 3x3 convolution of 16 channels on 16 maps of 32 x 32 filled 18 SMs instead of 137.
+    struct KernelPlan {
+        int launched = 1;
+        bool prepared = false;
+        std::vector<int> bn_fwd_from, conv_fwd_bn;  // BN -> conv whose forward kernel also produces the statistics of the BN (its input), or -1, and the inverse map
+        std::vector<int> bn_into, conv_in_bn;       // BN -> the convolution that applies it to its own input operand (no BN kernel), and the inverse
+        std::vector<int> bn_bwd_from, conv_bwd_bn;  // BN+ReLU -> the convolution whose data gradient also forms the sums of its backward, or -1, and the inverse map
+        std::vector<char> use_pipe[2];
+        std::vector<ConvPipeGeom> pipe_geom[2];     // conv -> split of its forward / data-gradient launches
+        std::vector<ConvPipePlan> pipe_plan[2];
+        std::vector<ConvTcPlan> wgrad_plan;
+    };
+    KernelPlan kernels[2];
+    // (the persistent cell kernels hold the step's launches: with them everything keeps to the step's plan)
+    bool has_cell_plan() const { return kernels[0].launched > 1 && opt_cell == 0; }
+    KernelPlan& cell_kernels() { return kernels[has_cell_plan() ? 1 : 0]; }
+    int kernel_plans() const { return has_cell_plan() ? 2 : 1; }
+    std::vector<size_t> bn_sums_off;           // where a data gradient leaves the sums of a BN+ReLU's backward, all micro-batches
+    std::vector<size_t> bn_moments_off;        // BN -> per-block moments of its input left by the producing convolution, all micro-batches
     // Forward / data-gradient launches of networks with batch norm are the pipelined kernel's wherever it covers the shape.
     // Without batch norm nothing re-scales the activations: the last bits of a convolution's sum move ReLU and max-pool
     // decisions and, over a few updates, the whole trajectory (1-2 % of VGG-16's gradient after two steps, for sums that differ
     // by 3e-6).  Such networks keep the tile kernel's order of summation; on their wide, small maps (256 channels and more on
     // 8 x 8 and less, where a padded grid of positions wastes a quarter and more of the MMA rows) it is no slower.
     bool has_bn = false;
-    std::vector<char> use_pipe[2];
     std::vector<ConvTcPlan> tile_plan[2];      // conv -> its launch on the tile kernel
-    std::vector<ConvPipeGeom> pipe_geom[2];    // conv -> split of its forward / data-gradient launches
     bool opt_pdl = true;       // programmatic dependent launch for this model's kernels
     bool opt_bn_cluster = true; // BN backward of micro-batch sized tensors as one thread-block-cluster launch
     int opt_cell_times = 0;    // record a device timestamp at the start and end of every (partition, micro-batch) cell
@@ -133,7 +147,8 @@ struct hpf_model {
     // Groups: on one GPU the stages share the same SMs, and a micro-batch's launches are too small to fill them, so one launch
     // covers all micro-batches of a stage wherever nothing asks for cells of their own (then one micro-batch).  Every micro-batch keeps
     // its own statistics, losses and gradient slot, formed in the same order whatever the size of the group.
-    int group_size() const { return opt_messages || opt_cell_times || lanes() > 1 ? 1 : M; }
+    int opt_group = 1;         // 0: launches of one micro-batch, planned as such
+    int group_size() const { return !opt_group || opt_messages || opt_cell_times || lanes() > 1 ? 1 : M; }
     int n_groups() const { return M / group_size(); }
     int opt_fuse_bn = 3;       // bit 0: BN statistics in the producing convolution's write-out, bit 1: BN+ReLU applied by the reading convolution
     std::vector<GradEdge> edge0;              // per op: contribution to src0
@@ -169,9 +184,6 @@ struct hpf_model {
     std::vector<cudaEvent_t> ev_fdone, ev_bjoin;   // forward (P-1, m) done; backward stream p done
     std::vector<cudaEvent_t> ev_side, ev_side_join;   // per partition: gradient ready -> side stream; side stream done
     cudaEvent_t ev_fork = nullptr, ev_sync = nullptr;
-    // tensor-core plans per op: forward / data gradient, weight gradient
-    std::vector<ConvPipePlan> pipe_plan[2];
-    std::vector<ConvTcPlan> wgrad_plan;
     std::vector<char> use_tc[3];              // per op
     // graphs
     struct FwdGraph { const float* x = nullptr; const int32_t* labels = nullptr; cudaGraphExec_t exec = nullptr; int64_t nodes = 0; };
@@ -401,7 +413,7 @@ void build_fusion_plan(hpf_model* mdl)
 
 ConvShape conv_shape_of(const hpf_model* mdl, int i);
 int passes_of(const hpf_model* mdl);
-bool op_uses_tc(hpf_model* mdl, int i, int pass);
+bool op_uses_tc(hpf_model* mdl, hpf_model::KernelPlan* k, int i, int pass);
 
 ConvShape conv_shape_of(const hpf_model* mdl, int i)
 {
@@ -415,57 +427,57 @@ int passes_of(const hpf_model* mdl) { return mdl->opt_conv_path == 2 ? 1 : 3; }
 // forward kernel that produces its input (only when producer and BN run back to back on the same stream: same
 // partition, nothing but a fused residual add between them), and the BN+ReLU itself on the operand path of the convolution
 // that reads it.
-void build_kernel_plan(hpf_model* mdl)
+void build_kernel_plan(hpf_model* mdl, hpf_model::KernelPlan* kp)
 {
     const int n = mdl->n_ops;
     mdl->has_bn = false;
     for (const OpInfo& o : mdl->ops) mdl->has_bn = mdl->has_bn || o.op.kind == HPF_OP_BN || o.op.kind == HPF_OP_BNRELU;
-    for (int pass = 0; pass < 2; ++pass) { mdl->pipe_geom[pass].assign(n, ConvPipeGeom()); mdl->use_pipe[pass].assign(n, 0); }
+    for (int pass = 0; pass < 2; ++pass) { kp->pipe_geom[pass].assign(n, ConvPipeGeom()); kp->use_pipe[pass].assign(n, 0); }
     for (int pass = 0; pass < 3; ++pass) {
         mdl->use_tc[pass].assign(n, 0);
-        for (int i = 0; i < n; ++i) mdl->use_tc[pass][i] = op_uses_tc(mdl, i, pass) ? 1 : 0;
+        for (int i = 0; i < n; ++i) mdl->use_tc[pass][i] = op_uses_tc(mdl, kp, i, pass) ? 1 : 0;      // (the same for every plan)
     }
-    mdl->bn_fwd_from.assign(n, -1);
-    mdl->conv_fwd_bn.assign(n, -1);
-    mdl->bn_into.assign(n, -1); mdl->conv_in_bn.assign(n, -1);
-    mdl->bn_bwd_from.assign(n, -1); mdl->conv_bwd_bn.assign(n, -1);
+    kp->bn_fwd_from.assign(n, -1);
+    kp->conv_fwd_bn.assign(n, -1);
+    kp->bn_into.assign(n, -1); kp->conv_in_bn.assign(n, -1);
+    kp->bn_bwd_from.assign(n, -1); kp->conv_bwd_bn.assign(n, -1);
     if (!(mdl->opt_fuse_bn & 1)) return;
     for (int j = 0; j < n; ++j) {
         const OpInfo& bn = mdl->ops[j];
         if (bn.op.kind != HPF_OP_BNRELU) continue;
         // Backward: the only kernel that writes the gradient of the BN's output forms its sums, unless one launch of clusters
-        // does it all from registers and is the better one: below a million values over all micro-batches (its clusters are
+        // does it all from registers and is the better one: below a million values over the micro-batches of a launch (its clusters are
         // resident at once; the sums cost the data gradient's write-out about a microsecond of latency, resnet11 took 395 us
         // instead of 355), and beyond 128 channels (several channel slices repeat the work, and those data gradients are
         // bound by their MMAs: resnet152 36.7 ms against 37.2 with the sums everywhere; resnet1001 63.7 ms with clusters
         // wherever they fit, 61.3 so).
         const bool clusters = mdl->opt_bn_cluster && bn_bwd_is_one_launch((int64_t)mdl->b * bn.H * bn.W, bn.C) &&
-                              (bn.C > 128 || (int64_t)mdl->B * bn.H * bn.W * bn.C < 1000000);
+                              (bn.C > 128 || (int64_t)kp->launched * mdl->b * bn.H * bn.W * bn.C < 1000000);
         if (bn.consumers.size() == 1 && !clusters) {
             const int i = bn.consumers[0];
             const OpInfo& c = mdl->ops[i];
-            if (i == j + 1 && c.op.kind == HPF_OP_CONV && c.op.stride == 1 && bn.C <= 2048 && c.part == bn.part && mdl->use_pipe[PASS_DGRAD][i] && !mdl->edge0[i].accumulate &&
-                mdl->edge0[i].addend < 0 && conv_pipe_can_fuse_bn_output(mdl->pipe_geom[PASS_DGRAD][i])) {
-                mdl->bn_bwd_from[j] = i; mdl->conv_bwd_bn[i] = j;
+            if (i == j + 1 && c.op.kind == HPF_OP_CONV && c.op.stride == 1 && bn.C <= 2048 && c.part == bn.part && kp->use_pipe[PASS_DGRAD][i] && !mdl->edge0[i].accumulate &&
+                mdl->edge0[i].addend < 0 && conv_pipe_can_fuse_bn_output(kp->pipe_geom[PASS_DGRAD][i])) {
+                kp->bn_bwd_from[j] = i; kp->conv_bwd_bn[i] = j;
             }
         }
         // forward: the kernel that writes the BN's input
         int t = bn.op.src0, prod = -1;
         if (mdl->ops[t].op.kind == HPF_OP_CONV && mdl->fused_into[t] < 0) prod = t;
         else if (mdl->ops[t].op.kind == HPF_OP_ADD && mdl->add_done_by[t] >= 0) prod = mdl->add_done_by[t];
-        if (prod < 0 || !mdl->use_pipe[PASS_FWD][prod] || mdl->ops[prod].part != bn.part || mdl->conv_fwd_bn[prod] >= 0 ||
-            !conv_pipe_can_fuse_bn_output(mdl->pipe_geom[PASS_FWD][prod])) continue;
+        if (prod < 0 || !kp->use_pipe[PASS_FWD][prod] || mdl->ops[prod].part != bn.part || kp->conv_fwd_bn[prod] >= 0 ||
+            !conv_pipe_can_fuse_bn_output(kp->pipe_geom[PASS_FWD][prod])) continue;
         bool adjacent = true;
         for (int k = prod + 1; k < j; ++k)
             if (!(mdl->ops[k].op.kind == HPF_OP_ADD && mdl->add_done_by[k] >= 0)) adjacent = false;
         if (!adjacent) continue;
-        mdl->bn_fwd_from[j] = prod; mdl->conv_fwd_bn[prod] = j;
+        kp->bn_fwd_from[j] = prod; kp->conv_fwd_bn[prod] = j;
         // the BN+ReLU itself: applied by its only reader, the next op, a stride-1 tensor-core convolution
         if ((mdl->opt_fuse_bn & 2) && bn.consumers.size() == 1 && bn.consumers[0] == j + 1) {
             const int i = j + 1;
-            if (mdl->ops[i].op.kind == HPF_OP_CONV && mdl->ops[i].op.src0 == j && mdl->use_pipe[PASS_FWD][i] && mdl->ops[i].part == bn.part &&
+            if (mdl->ops[i].op.kind == HPF_OP_CONV && mdl->ops[i].op.src0 == j && kp->use_pipe[PASS_FWD][i] && mdl->ops[i].part == bn.part &&
                 conv_pipe_can_fuse_bn_input(conv_shape_of(mdl, i))) {
-                mdl->bn_into[j] = i; mdl->conv_in_bn[i] = j;
+                kp->bn_into[j] = i; kp->conv_in_bn[i] = j;
             }
         }
     }
@@ -491,8 +503,8 @@ void build_cell_runs(hpf_model* mdl)
         };
         for (int i = mdl->part_lo[p]; i < mdl->part_hi[p]; ++i) {
             const int kind = mdl->ops[i].op.kind;
-            if (kind == HPF_OP_CONV && mdl->use_pipe[PASS_FWD][i]) run.convs.push_back(i);
-            else if (kind == HPF_OP_BNRELU && mdl->bn_into[i] >= 0) continue;
+            if (kind == HPF_OP_CONV && mdl->kernels[0].use_pipe[PASS_FWD][i]) run.convs.push_back(i);
+            else if (kind == HPF_OP_BNRELU && mdl->kernels[0].bn_into[i] >= 0) continue;
             else if (kind == HPF_OP_ADD && mdl->add_done_by[i] >= 0) continue;
             else close();
         }
@@ -507,7 +519,9 @@ void build_cell_runs(hpf_model* mdl)
 void build_memory_plan(hpf_model* mdl)
 {
     build_fusion_plan(mdl);
-    build_kernel_plan(mdl);
+    mdl->kernels[0].launched = mdl->opt_group ? mdl->M : 1;
+    mdl->kernels[1].launched = 1;
+    for (int k = 0; k < mdl->kernel_plans(); ++k) build_kernel_plan(mdl, &mdl->kernels[k]);
     const int n = mdl->n_ops, M = mdl->M, P = mdl->P;
     size_t at = 0;
     auto take = [&](size_t bytes) { size_t o = at; at = align_up(at + bytes, 256); return o; };
@@ -523,8 +537,11 @@ void build_memory_plan(hpf_model* mdl)
             if (o.op.kind == HPF_OP_BNRELU || o.op.kind == HPF_OP_BN) bn = std::max(bn, bn_scratch_bytes((int64_t)mdl->b * o.H * o.W, o.C));
             if (o.op.kind == HPF_OP_CONV && mdl->opt_conv_path != 1)
                 for (int pass : {PASS_FWD, PASS_DGRAD})
-                    if (mdl->use_tc[pass][i]) sk = std::max(sk, mdl->use_pipe[pass][i] ? conv_pipe_splitk_bytes(conv_shape_of(mdl, i), pass, passes_of(mdl), M)
-                                                                        : conv_tc_splitk_bytes(conv_shape_of(mdl, i), pass, 3));
+                    for (int k = 0; k < mdl->kernel_plans(); ++k)
+                        if (mdl->use_tc[pass][i])
+                            sk = std::max(sk, mdl->kernels[k].use_pipe[pass][i]
+                                                  ? conv_pipe_splitk_bytes(mdl->kernels[k].pipe_geom[pass][i])
+                                                  : conv_tc_splitk_bytes(conv_shape_of(mdl, i), pass, 3));
         }
         mdl->bn_scratch_bytes_[p] = align_up(bn, 256);
         mdl->splitk_bytes[p] = sk;
@@ -538,21 +555,25 @@ void build_memory_plan(hpf_model* mdl)
     mdl->zero_hi = at;
     build_cell_runs(mdl);
     for (auto& run : mdl->cell_runs) run.ops_off = take(conv_pipe_cell_op_bytes() * run.convs.size());
-    mdl->bn_sums_off.assign(n, 0);
-    for (int j = 0; j < n; ++j)
-        if (mdl->bn_bwd_from[j] >= 0)
-            mdl->bn_sums_off[j] = take(sizeof(float) * M * conv_pipe_partial_floats(mdl->pipe_geom[PASS_DGRAD][mdl->bn_bwd_from[j]].blocks_per_m, mdl->ops[j].C));
-    mdl->bn_moments_off.assign(n, 0);
-    for (int j = 0; j < n; ++j)
-        if (mdl->bn_fwd_from[j] >= 0)
-            mdl->bn_moments_off[j] = take(sizeof(float) * M * conv_pipe_partial_floats(mdl->pipe_geom[PASS_FWD][mdl->bn_fwd_from[j]].blocks_per_m, mdl->ops[j].C));
+    mdl->bn_sums_off.assign(n, 0); mdl->bn_moments_off.assign(n, 0);
+    for (int j = 0; j < n; ++j) {
+        size_t sums = 0, moments = 0;
+        for (int k = 0; k < mdl->kernel_plans(); ++k) {
+            const hpf_model::KernelPlan& kp = mdl->kernels[k];
+            if (kp.bn_bwd_from[j] >= 0) sums = std::max(sums, conv_pipe_partial_floats(kp.pipe_geom[PASS_DGRAD][kp.bn_bwd_from[j]].blocks_per_m, mdl->ops[j].C));
+            if (kp.bn_fwd_from[j] >= 0) moments = std::max(moments, conv_pipe_partial_floats(kp.pipe_geom[PASS_FWD][kp.bn_fwd_from[j]].blocks_per_m, mdl->ops[j].C));
+        }
+        if (sums) mdl->bn_sums_off[j] = take(sizeof(float) * M * sums);
+        if (moments) mdl->bn_moments_off[j] = take(sizeof(float) * M * moments);
+    }
     mdl->conv_scratch_off.assign(P, 0); mdl->conv_scratch_ms.assign(P, 0);
     for (int p = 0; p < P; ++p) {
         size_t cv = 256;
         for (int i = mdl->part_lo[p]; i < mdl->part_hi[p]; ++i)
             if (mdl->ops[i].op.kind == HPF_OP_CONV) {
                 const ConvShape s = conv_shape_of(mdl, i);
-                cv = std::max(cv, std::max(conv_simt_scratch_bytes(s, M), conv_tc_scratch_bytes(s, M)));
+                for (int k = 0; k < mdl->kernel_plans(); ++k)
+                    cv = std::max(cv, std::max(conv_simt_scratch_bytes(s, mdl->kernels[k].launched), conv_tc_scratch_bytes(s, mdl->kernels[k].launched)));
             }
         mdl->conv_scratch_ms[p] = align_up(cv, 256);
         mdl->conv_scratch_off[p] = take(mdl->conv_scratch_ms[p] * M);
@@ -597,7 +618,7 @@ void build_memory_plan(hpf_model* mdl)
     mdl->planned = true;
 }
 
-bool op_uses_tc(hpf_model* mdl, int i, int pass)
+bool op_uses_tc(hpf_model* mdl, hpf_model::KernelPlan* k, int i, int pass)
 {
     if (mdl->opt_conv_path == 1) return false;
     if (mdl->ops[i].op.kind != HPF_OP_CONV) return false;
@@ -607,8 +628,88 @@ bool op_uses_tc(hpf_model* mdl, int i, int pass)
     if (pass == PASS_DGRAD && mdl->ops[i].op.stride > 1 && (mdl->edge0[i].accumulate || mdl->edge0[i].addend >= 0)) return false;
     if (pass == PASS_WGRAD) return conv_tc_supported(conv_shape_of(mdl, i), pass);
     const ConvShape s = conv_shape_of(mdl, i);
-    mdl->use_pipe[pass][i] = mdl->has_bn && conv_pipe_geom(s, pass, passes_of(mdl), mdl->M, &mdl->pipe_geom[pass][i]);
-    return mdl->use_pipe[pass][i] || conv_tc_supported(s, pass);
+    k->use_pipe[pass][i] = mdl->has_bn && conv_pipe_geom(s, pass, passes_of(mdl), k->launched, &k->pipe_geom[pass][i]);
+    return k->use_pipe[pass][i] || conv_tc_supported(s, pass);
+}
+
+// The launches of one set of plans: tensor maps and parameters over the bound buffers.  The step's are prepared by hpf_bind,
+// the cells' by the first call that runs one (a program that only makes steps does not wait for them).
+int prepare_kernels(hpf_model* mdl, hpf_model::KernelPlan& kp)
+{
+    if (kp.prepared) return HPF_OK;
+    bool any_tc = false;
+    for (int pass = 0; pass < 3; ++pass)
+        for (char use : mdl->use_tc[pass]) any_tc = any_tc || use;
+    if (!any_tc) { kp.prepared = true; return HPF_OK; }
+    const int n = mdl->n_ops, M = mdl->M, passes = passes_of(mdl);
+    float* wp = reinterpret_cast<float*>(mdl->ws + mdl->wprep_off);
+    const int64_t G = (mdl->G + 3) / 4 * 4;       // stride between the four prepared-weight arrays
+    for (int pass = 0; pass < 2; ++pass) kp.pipe_plan[pass].assign(n, ConvPipePlan());
+    kp.wgrad_plan.assign(n, ConvTcPlan());
+    std::vector<char> first_done(mdl->P, 0);
+    for (int i = 0; i < n; ++i) {
+        const OpInfo& o = mdl->ops[i];
+        if (o.op.kind != HPF_OP_CONV) continue;
+        const int src = o.op.src0, p = o.part;
+        const ConvShape s = conv_shape_of(mdl, i);
+        const GradEdge& ed = mdl->edge0[i];
+        ConvTcHints tile;                     // launches on the tile kernel
+        tile.micro_batches = M; tile.splitk_bytes = mdl->splitk_bytes[p];
+        if (mdl->use_tc[PASS_FWD][i]) {
+            const float* in = mdl->act(src, 0);
+            const float* residual = nullptr;
+            if (mdl->fused_into[i] >= 0) {
+                const hpf_op& a = mdl->ops[mdl->fused_into[i]].op;
+                residual = mdl->act(a.src0 == i ? a.src1 : a.src0, 0);
+            }
+            ConvPipeBn bn;
+            if (kp.conv_fwd_bn[i] >= 0) bn.out_partials = mdl->moments(kp.conv_fwd_bn[i]);
+            const int jb = kp.conv_in_bn[i];
+            if (jb >= 0) {
+                const OpInfo& b = mdl->ops[jb];
+                in = mdl->act(b.op.src0, 0);              // the BN's input; its output is a by-product of this kernel
+                bn.in_partials = mdl->moments(jb);
+                bn.in_blocks = kp.pipe_geom[PASS_FWD][kp.bn_fwd_from[jb]].blocks_per_m;
+                bn.in_gamma = mdl->params + b.w_off; bn.in_beta = mdl->params + b.b_off;
+                bn.in_stats = mdl->stats(jb, 0); bn.in_y = mdl->act(jb, 0); bn.in_eps = b.op.eps;
+            }
+            // the weights are prepared just ahead of the partition's first convolution
+            if (kp.use_pipe[PASS_FWD][i]) CU(conv_pipe_prepare(&kp.pipe_plan[PASS_FWD][i], s, PASS_FWD, passes, M, kp.launched, in, wp + o.w_off, wp + G + o.w_off, mdl->act(i, 0),
+                                 residual, false, &bn, mdl->ws + mdl->splitk_off[p], mdl->splitk_bytes[p], first_done[p] != 0));
+            else {
+                tile.splitk = mdl->splitk_bytes[p] ? mdl->ws + mdl->splitk_off[p] : nullptr;
+                CU(conv_tc_prepare(&mdl->tile_plan[PASS_FWD][i], s, PASS_FWD, passes, in, nullptr, wp + o.w_off, wp + G + o.w_off, mdl->act(i, 0), residual,
+                                   false, nullptr, &tile));
+            }
+            first_done[p] = 1;
+        }
+        ConvPipeBn sums;
+        if (kp.conv_bwd_bn[i] >= 0) {
+            const int jb = kp.conv_bwd_bn[i];
+            const OpInfo& b = mdl->ops[jb];
+            sums.bwd_partials = reinterpret_cast<float*>(mdl->ws + mdl->bn_sums_off[jb]);
+            sums.bwd_x = mdl->act(b.op.src0, 0); sums.bwd_stats = mdl->stats(jb, 0);
+            sums.in_gamma = mdl->params + b.w_off; sums.in_beta = mdl->params + b.b_off;
+        }
+        if (kp.use_pipe[PASS_DGRAD][i])
+            CU(conv_pipe_prepare(&kp.pipe_plan[PASS_DGRAD][i], s, PASS_DGRAD, passes, M, kp.launched, mdl->grad(i, 0), wp + 2 * G + o.w_off,
+                                 wp + 3 * G + o.w_off, mdl->grad(src, 0), ed.addend >= 0 ? mdl->grad(ed.addend, 0) : nullptr,
+                                 ed.accumulate != 0, &sums, mdl->ws + mdl->splitk_bwd_off[p], mdl->splitk_bytes[p], true));
+        else if (mdl->use_tc[PASS_DGRAD][i]) {
+            tile.splitk = mdl->splitk_bytes[p] ? mdl->ws + mdl->splitk_bwd_off[p] : nullptr;
+            CU(conv_tc_prepare(&mdl->tile_plan[PASS_DGRAD][i], s, PASS_DGRAD, passes, mdl->grad(i, 0), nullptr, wp + 2 * G + o.w_off, wp + 3 * G + o.w_off,
+                               mdl->grad(src, 0), ed.addend >= 0 ? mdl->grad(ed.addend, 0) : nullptr, ed.accumulate != 0, nullptr, &tile));
+        }
+        if (mdl->use_tc[PASS_WGRAD][i]) {
+            ConvTcHints hint;
+            hint.wgrad_transposing = mdl->opt_wgrad_direct ? 0 : 1;
+            hint.micro_batches = M; hint.launched = kp.launched; hint.slot_stride = mdl->G; hint.partial_stride = (long long)(mdl->conv_scratch_ms[p] / sizeof(float));
+            CU(conv_tc_prepare(&kp.wgrad_plan[i], s, PASS_WGRAD, mdl->opt_conv_path == 2 ? 1 : mdl->opt_wgrad_passes, mdl->grad(i, 0), mdl->act(src, 0),
+                               nullptr, nullptr, mdl->gslots + o.w_off, nullptr, false, mdl->ws + mdl->conv_scratch_off[p], &hint));
+        }
+    }
+    kp.prepared = true;
+    return HPF_OK;
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -651,13 +752,12 @@ HeadGroup head_group(const hpf_model* mdl, int i, int g)
 
 // Ops of one stage on the micro-batches m .. m + g - 1.  sl: the stream slot (partition, lane) whose side stream is used.
 // Launches that know nothing of micro-batches take the group as one larger batch where its tensors are contiguous.
-int forward_op(hpf_model* mdl, int i, int m, int g, cudaStream_t st, int sl)
+int forward_op(hpf_model* mdl, const hpf_model::KernelPlan& kp, int i, int m, int g, cudaStream_t st, int sl)
 {
-    (void)sl;
     const OpInfo& o = mdl->ops[i];
     const hpf_op& q = o.op;
     if (g > 1 && q.kind != HPF_OP_HEAD && !(mdl->contiguous(i) && mdl->contiguous(q.src0) && (q.kind != HPF_OP_ADD || mdl->contiguous(q.src1)))) {
-        for (int k = 0; k < g; ++k) { int rc = forward_op(mdl, i, m + k, 1, st, sl); if (rc) return rc; }
+        for (int k = 0; k < g; ++k) { int rc = forward_op(mdl, kp, i, m + k, 1, st, sl); if (rc) return rc; }
         return HPF_OK;
     }
     const float* in0 = src_act(mdl, q.src0, m);
@@ -685,8 +785,8 @@ int forward_op(hpf_model* mdl, int i, int m, int g, cudaStream_t st, int sl)
                 if (run.convs[0] == i)
                     CU(conv_pipe_cell_launch(mdl->ws + run.ops_off, (int)run.convs.size(), m, g, mdl->opt_cell, run.smem, run.tmem,
                                              reinterpret_cast<unsigned int*>(mdl->ws + mdl->cell_bar_off[sl]), mdl->status(), st, &mdl->launches));
-            } else if (mdl->use_pipe[PASS_FWD][i]) {
-                CU(conv_pipe_launch(&mdl->pipe_plan[PASS_FWD][i], m, g, late, mdl->status(), st, &mdl->launches));
+            } else if (kp.use_pipe[PASS_FWD][i]) {
+                CU(conv_pipe_launch(&kp.pipe_plan[PASS_FWD][i], m, g, late, mdl->status(), st, &mdl->launches));
             } else {
                 CU(conv_tc_launch(&mdl->tile_plan[PASS_FWD][i], mdl->status(), st, &mdl->launches, m, g, late));
             }
@@ -695,9 +795,9 @@ int forward_op(hpf_model* mdl, int i, int m, int g, cudaStream_t st, int sl)
         break;
     }
     case HPF_OP_BNRELU:
-        if (mdl->bn_into[i] >= 0) break;   // the convolution that reads this BN applies it (and stores `out` and the statistics)
-        if (mdl->bn_fwd_from[i] >= 0) {    // the producing convolution left the moments of its units
-            const int units = mdl->pipe_geom[PASS_FWD][mdl->bn_fwd_from[i]].blocks_per_m;
+        if (kp.bn_into[i] >= 0) break;   // the convolution that reads this BN applies it (and stores `out` and the statistics)
+        if (kp.bn_fwd_from[i] >= 0) {    // the producing convolution left the moments of its units
+            const int units = kp.pipe_geom[PASS_FWD][kp.bn_fwd_from[i]].blocks_per_m;
             CU(bn_finalize_partials(mdl->moments(i) + (size_t)m * conv_pipe_partial_floats(units, o.C), units, o.C, q.eps, (double)rows, mdl->stats(i, m), g, st,
                                     &mdl->launches));
             CU(bnrelu_fwd_apply(in0, mdl->params + o.w_off, mdl->params + o.b_off, mdl->stats(i, m), out, rows, o.C, st, &mdl->launches, grp));
@@ -726,13 +826,13 @@ int forward_op(hpf_model* mdl, int i, int m, int g, cudaStream_t st, int sl)
     return HPF_OK;
 }
 
-int backward_op(hpf_model* mdl, int i, int m, int g, cudaStream_t st, int sl)
+int backward_op(hpf_model* mdl, const hpf_model::KernelPlan& kp, int i, int m, int g, cudaStream_t st, int sl)
 {
     const OpInfo& o = mdl->ops[i];
     const hpf_op& q = o.op;
     const GradEdge& e = mdl->edge0[i];
     if (g > 1 && q.kind != HPF_OP_HEAD && !(mdl->contiguous(i) && mdl->contiguous(q.src0) && (q.kind != HPF_OP_ADD || mdl->contiguous(q.src1)))) {
-        for (int k = 0; k < g; ++k) { int rc = backward_op(mdl, i, m + k, 1, st, sl); if (rc) return rc; }
+        for (int k = 0; k < g; ++k) { int rc = backward_op(mdl, kp, i, m + k, 1, st, sl); if (rc) return rc; }
         return HPF_OK;
     }
     // explicit accumulations scheduled at this op
@@ -761,13 +861,13 @@ int backward_op(hpf_model* mdl, int i, int m, int g, cudaStream_t st, int sl)
             CU(cudaStreamWaitEvent(wst, mdl->ev_side[sl], 0));
         }
         if (mdl->use_tc[PASS_WGRAD][i]) {
-            CU(conv_tc_launch(&mdl->wgrad_plan[i], mdl->status(), wst, &mdl->launches, m, g));
+            CU(conv_tc_launch(&kp.wgrad_plan[i], mdl->status(), wst, &mdl->launches, m, g));
         } else {
             CU(conv_wgrad_simt(in0, dout, slot + o.w_off, s, mdl->ws + mdl->conv_scratch_off[o.part] + m * mdl->conv_scratch_ms[o.part], wst, &mdl->launches,
-                               mdl->M, g, (long long)(mdl->conv_scratch_ms[o.part] / sizeof(float)), mdl->G));
+                               kp.launched, g, (long long)(mdl->conv_scratch_ms[o.part] / sizeof(float)), mdl->G));
         }
         if (q.src0 >= 0) {
-            if (mdl->use_pipe[PASS_DGRAD][i]) CU(conv_pipe_launch(&mdl->pipe_plan[PASS_DGRAD][i], m, g, false, mdl->status(), st, &mdl->launches));
+            if (kp.use_pipe[PASS_DGRAD][i]) CU(conv_pipe_launch(&kp.pipe_plan[PASS_DGRAD][i], m, g, false, mdl->status(), st, &mdl->launches));
             else if (mdl->use_tc[PASS_DGRAD][i]) CU(conv_tc_launch(&mdl->tile_plan[PASS_DGRAD][i], mdl->status(), st, &mdl->launches, m, g));
             else CU(conv_dgrad_simt(dout, mdl->params + o.w_off, mdl->grad(q.src0, m), addend, e.accumulate != 0, gs, st, &mdl->launches));
         }
@@ -775,8 +875,8 @@ int backward_op(hpf_model* mdl, int i, int m, int g, cudaStream_t st, int sl)
     }
     case HPF_OP_BNRELU:
     case HPF_OP_BN:
-        if (mdl->bn_bwd_from[i] >= 0) {
-            const int blocks = mdl->pipe_geom[PASS_DGRAD][mdl->bn_bwd_from[i]].blocks_per_m;
+        if (kp.bn_bwd_from[i] >= 0) {
+            const int blocks = kp.pipe_geom[PASS_DGRAD][kp.bn_bwd_from[i]].blocks_per_m;
             const int64_t ms = (int64_t)conv_pipe_partial_floats(blocks, o.C);
             CU(bnrelu_bwd_apply(in0, dout, mdl->params + o.w_off, mdl->params + o.b_off, mdl->stats(i, m), reinterpret_cast<const float*>(mdl->ws + mdl->bn_sums_off[i]) + m * ms,
                                 blocks, ms, mdl->grad(q.src0, m), addend, e.accumulate != 0, slot + o.w_off, slot + o.b_off, rows, o.C, st, &mdl->launches, grp));
@@ -856,7 +956,7 @@ int enqueue_phase(hpf_model* mdl, int phase)
                 }
                 if (mdl->opt_cell_times) CU(stamp_time(mdl->cell_time_slot(PH_FWD, p, m), st, &mdl->launches));
                 for (int i = mdl->part_lo[p]; i < mdl->part_hi[p]; ++i) {
-                    int rc = forward_op(mdl, i, m * gs, gs, st, mdl->slot_of(p, m));
+                    int rc = forward_op(mdl, mdl->kernels[0], i, m * gs, gs, st, mdl->slot_of(p, m));
                     if (rc) return rc;
                 }
                 if (mdl->opt_cell_times) CU(stamp_time(mdl->cell_time_slot(PH_FWD, p, m) + 1, st, &mdl->launches));
@@ -884,7 +984,7 @@ int enqueue_phase(hpf_model* mdl, int phase)
                 }
                 if (mdl->opt_cell_times) CU(stamp_time(mdl->cell_time_slot(PH_BWD, p, m), st, &mdl->launches));
                 for (int i = mdl->part_hi[p] - 1; i >= mdl->part_lo[p]; --i) {
-                    int rc = backward_op(mdl, i, m * gs, gs, st, mdl->slot_of(p, m));
+                    int rc = backward_op(mdl, mdl->kernels[0], i, m * gs, gs, st, mdl->slot_of(p, m));
                     if (rc) return rc;
                 }
                 if (mdl->opt_cell_times) CU(stamp_time(mdl->cell_time_slot(PH_BWD, p, m) + 1, st, &mdl->launches));
@@ -1046,6 +1146,7 @@ int hpf_set_option(hpf_model* mdl, int32_t option, int32_t value)
     case HPF_OPT_WGRAD_DIRECT: mdl->opt_wgrad_direct = value != 0; break;
     case HPF_OPT_STAGE_LANES: if (value < 1 || value > 64) return fail(HPF_ERR_INVALID, "1..64 lanes"); mdl->opt_lanes = value; break;
     case HPF_OPT_PDL_LATE_FROM: if (value < 0) return fail(HPF_ERR_INVALID, ">= 0"); mdl->opt_pdl_late_from = value; break;
+    case HPF_OPT_GROUP_LAUNCHES: mdl->opt_group = value != 0; break;
     case HPF_OPT_CELL_CTAS: if (value < 0 || value > 148) return fail(HPF_ERR_INVALID, "0..148 CTAs"); mdl->opt_cell = value; break;
     case HPF_OPT_WGRAD_PASSES: if (value != 1 && value != 3) return fail(HPF_ERR_INVALID, "1 or 3 passes"); mdl->opt_wgrad_passes = value; break;
     default: return fail(HPF_ERR_INVALID, "unknown option");
@@ -1263,9 +1364,6 @@ int hpf_bind(hpf_model* mdl, float* d_params, float* d_grad_slots, float* d_grad
     mdl->prep_table.assign(mdl->P, {});
     if (any_tc) {
         CU(conv_tc_init());
-        const int passes = mdl->opt_conv_path == 2 ? 1 : 3;
-        float* wp = reinterpret_cast<float*>(mdl->ws + mdl->wprep_off);
-        const int64_t G = (mdl->G + 3) / 4 * 4;       // stride between the four prepared-weight arrays
         for (int i = 0; i < n; ++i)
             if (mdl->use_tc[PASS_FWD][i] || mdl->use_tc[PASS_DGRAD][i]) {
                 const OpInfo& o = mdl->ops[i];
@@ -1276,70 +1374,9 @@ int hpf_bind(hpf_model* mdl, float* d_params, float* d_grad_slots, float* d_grad
                 CU(cudaMemcpyAsync(mdl->ws + mdl->prep_table_off[p], mdl->prep_table[p].data(),
                                    sizeof(WeightPrepEntry) * mdl->prep_table[p].size(), cudaMemcpyHostToDevice, mdl->streams[0]));
         CU(conv_pipe_init());
-        for (int pass = 0; pass < 2; ++pass) { mdl->pipe_plan[pass].assign(n, ConvPipePlan()); mdl->tile_plan[pass].assign(n, ConvTcPlan()); }
-        mdl->wgrad_plan.resize(n);
-        std::vector<char> first_done(mdl->P, 0);
-        for (int i = 0; i < n; ++i) {
-            const OpInfo& o = mdl->ops[i];
-            if (o.op.kind != HPF_OP_CONV) continue;
-            const int src = o.op.src0, p = o.part;
-            const ConvShape s = conv_shape_of(mdl, i);
-            const GradEdge& ed = mdl->edge0[i];
-            ConvTcHints tile;                     // launches on the tile kernel
-            tile.micro_batches = M; tile.splitk_bytes = mdl->splitk_bytes[p];
-            if (mdl->use_tc[PASS_FWD][i]) {
-                const float* in = mdl->act(src, 0);
-                const float* residual = nullptr;
-                if (mdl->fused_into[i] >= 0) {
-                    const hpf_op& a = mdl->ops[mdl->fused_into[i]].op;
-                    residual = mdl->act(a.src0 == i ? a.src1 : a.src0, 0);
-                }
-                ConvPipeBn bn;
-                if (mdl->conv_fwd_bn[i] >= 0) bn.out_partials = mdl->moments(mdl->conv_fwd_bn[i]);
-                const int jb = mdl->conv_in_bn[i];
-                if (jb >= 0) {
-                    const OpInfo& b = mdl->ops[jb];
-                    in = mdl->act(b.op.src0, 0);              // the BN's input; its output is a by-product of this kernel
-                    bn.in_partials = mdl->moments(jb);
-                    bn.in_blocks = mdl->pipe_geom[PASS_FWD][mdl->bn_fwd_from[jb]].blocks_per_m;
-                    bn.in_gamma = mdl->params + b.w_off; bn.in_beta = mdl->params + b.b_off;
-                    bn.in_stats = mdl->stats(jb, 0); bn.in_y = mdl->act(jb, 0); bn.in_eps = b.op.eps;
-                }
-                // the weights are prepared just ahead of the partition's first convolution
-                if (mdl->use_pipe[PASS_FWD][i]) CU(conv_pipe_prepare(&mdl->pipe_plan[PASS_FWD][i], s, PASS_FWD, passes, M, in, wp + o.w_off, wp + G + o.w_off, mdl->act(i, 0),
-                                     residual, false, &bn, mdl->ws + mdl->splitk_off[p], mdl->splitk_bytes[p], first_done[p] != 0));
-                else {
-                    tile.splitk = mdl->splitk_bytes[p] ? mdl->ws + mdl->splitk_off[p] : nullptr;
-                    CU(conv_tc_prepare(&mdl->tile_plan[PASS_FWD][i], s, PASS_FWD, passes, in, nullptr, wp + o.w_off, wp + G + o.w_off, mdl->act(i, 0), residual,
-                                       false, nullptr, &tile));
-                }
-                first_done[p] = 1;
-            }
-            ConvPipeBn sums;
-            if (mdl->conv_bwd_bn[i] >= 0) {
-                const int jb = mdl->conv_bwd_bn[i];
-                const OpInfo& b = mdl->ops[jb];
-                sums.bwd_partials = reinterpret_cast<float*>(mdl->ws + mdl->bn_sums_off[jb]);
-                sums.bwd_x = mdl->act(b.op.src0, 0); sums.bwd_stats = mdl->stats(jb, 0);
-                sums.in_gamma = mdl->params + b.w_off; sums.in_beta = mdl->params + b.b_off;
-            }
-            if (mdl->use_pipe[PASS_DGRAD][i])
-                CU(conv_pipe_prepare(&mdl->pipe_plan[PASS_DGRAD][i], s, PASS_DGRAD, passes, M, mdl->grad(i, 0), wp + 2 * G + o.w_off,
-                                     wp + 3 * G + o.w_off, mdl->grad(src, 0), ed.addend >= 0 ? mdl->grad(ed.addend, 0) : nullptr,
-                                     ed.accumulate != 0, &sums, mdl->ws + mdl->splitk_bwd_off[p], mdl->splitk_bytes[p], true));
-            else if (mdl->use_tc[PASS_DGRAD][i]) {
-                tile.splitk = mdl->splitk_bytes[p] ? mdl->ws + mdl->splitk_bwd_off[p] : nullptr;
-                CU(conv_tc_prepare(&mdl->tile_plan[PASS_DGRAD][i], s, PASS_DGRAD, passes, mdl->grad(i, 0), nullptr, wp + 2 * G + o.w_off, wp + 3 * G + o.w_off,
-                                   mdl->grad(src, 0), ed.addend >= 0 ? mdl->grad(ed.addend, 0) : nullptr, ed.accumulate != 0, nullptr, &tile));
-            }
-            if (mdl->use_tc[PASS_WGRAD][i]) {
-                ConvTcHints hint;
-                hint.wgrad_transposing = mdl->opt_wgrad_direct ? 0 : 1;
-                hint.micro_batches = M; hint.slot_stride = mdl->G; hint.partial_stride = (long long)(mdl->conv_scratch_ms[p] / sizeof(float));
-                CU(conv_tc_prepare(&mdl->wgrad_plan[i], s, PASS_WGRAD, mdl->opt_conv_path == 2 ? 1 : mdl->opt_wgrad_passes, mdl->grad(i, 0), mdl->act(src, 0),
-                                   nullptr, nullptr, mdl->gslots + o.w_off, nullptr, false, mdl->ws + mdl->conv_scratch_off[p], &hint));
-            }
-        }
+        for (int pass = 0; pass < 2; ++pass) mdl->tile_plan[pass].assign(n, ConvTcPlan());
+        const int rc = prepare_kernels(mdl, mdl->kernels[0]);
+        if (rc) return rc;
         // persistent forward cells: the records of every run's launches
         std::vector<char> runs_in(mdl->P, 0);
         for (auto& run : mdl->cell_runs) {
@@ -1348,7 +1385,7 @@ int hpf_bind(hpf_model* mdl, float* d_params, float* d_grad_slots, float* d_grad
             run.smem = run.tmem = 0;
             for (size_t k = 0; k < run.convs.size(); ++k) {
                 unsigned int smem = 0, tmem = 0;
-                conv_pipe_cell_op(&mdl->pipe_plan[PASS_FWD][run.convs[k]], mdl->status(), host.data() + k * rec, &smem, &tmem);
+                conv_pipe_cell_op(&mdl->kernels[0].pipe_plan[PASS_FWD][run.convs[k]], mdl->status(), host.data() + k * rec, &smem, &tmem);
                 run.smem = std::max(run.smem, smem); run.tmem = std::max(run.tmem, tmem);
             }
             CU(cudaMemcpyAsync(mdl->ws + run.ops_off, host.data(), host.size(), cudaMemcpyHostToDevice, mdl->streams[0]));
@@ -1420,10 +1457,12 @@ int hpf_forward_cell(hpf_model* mdl, int32_t p, int32_t m, const float* d_x, con
     if (p == mdl->P - 1 && !d_labels) return fail(HPF_ERR_INVALID, "the last partition reads the labels");
     if (d_x) mdl->cur_x = d_x;
     if (d_labels) mdl->cur_labels = d_labels;
+    const int prepared = prepare_kernels(mdl, mdl->cell_kernels());
+    if (prepared) return prepared;
     const PdlScope pdl_scope(mdl->opt_pdl);
     const BnClusterScope bn_cluster_scope(mdl->opt_bn_cluster);
     for (int i = mdl->part_lo[p]; i < mdl->part_hi[p]; ++i) {
-        int rc = forward_op(mdl, i, m, 1, mdl->stream_of(p, m), mdl->slot_of(p, m));
+        int rc = forward_op(mdl, mdl->cell_kernels(), i, m, 1, mdl->stream_of(p, m), mdl->slot_of(p, m));
         if (rc) return rc;
     }
     if (mdl->state < ST_FWD) mdl->state = ST_FWD;
@@ -1436,10 +1475,12 @@ int hpf_backward_cell(hpf_model* mdl, int32_t p, int32_t m)
     if (mdl->state < ST_FWD) return fail(HPF_ERR_STATE, "the cell's forward has not run");
     if (p < 0 || p >= mdl->P || m < 0 || m >= mdl->M) return fail(HPF_ERR_INVALID, "cell out of range");
     if (p == mdl->P - 1 && !mdl->cur_labels) return fail(HPF_ERR_STATE, "the last partition needs the labels of its forward cell");
+    const int prepared = prepare_kernels(mdl, mdl->cell_kernels());
+    if (prepared) return prepared;
     const PdlScope pdl_scope(mdl->opt_pdl);
     const BnClusterScope bn_cluster_scope(mdl->opt_bn_cluster);
     for (int i = mdl->part_hi[p] - 1; i >= mdl->part_lo[p]; --i) {
-        int rc = backward_op(mdl, i, m, 1, mdl->stream_of(p, m), mdl->slot_of(p, m));
+        int rc = backward_op(mdl, mdl->cell_kernels(), i, m, 1, mdl->stream_of(p, m), mdl->slot_of(p, m));
         if (rc) return rc;
     }
     mdl->state = ST_BWD;
@@ -1647,14 +1688,14 @@ int hpf_step_bytes(const hpf_model* mdl_c, double* fused_bytes)
             conv_weights += w;
             f = read_in + w + out_el;
             if (mdl->fused_into[i] >= 0) f += out_el;                       // the residual rides in the write-out
-            if (mdl->conv_in_bn[i] >= 0) f += in_el;                        // the BN+ReLU output is stored as a by-product
+            if (mdl->kernels[0].conv_in_bn[i] >= 0) f += in_el;                        // the BN+ReLU output is stored as a by-product
             if (q.src0 >= 0) bw += out_el + w + in_el + extra_in;           // data gradient
             bw += read_in + out_el + w;                                     // weight gradient
             break;
         }
         case HPF_OP_BNRELU:
         case HPF_OP_BN:
-            f = mdl->bn_into[i] >= 0 ? 0.0 : 2.0 * out_el;                 // applied by the reading convolution: no traffic of its own
+            f = mdl->kernels[0].bn_into[i] >= 0 ? 0.0 : 2.0 * out_el;                 // applied by the reading convolution: no traffic of its own
             bw = 3.0 * out_el + extra_in;
             break;
         case HPF_OP_RELU: f = 2.0 * out_el; bw = 3.0 * out_el + extra_in; break;
@@ -1759,7 +1800,7 @@ static int conv_single(int pass, const float* in, const float* in2, const float*
         const size_t a = conv_simt_scratch_bytes(s), b = conv_tc_scratch_bytes(s);
         ConvPipePlan pipe;
         CU(conv_pipe_init());
-        const cudaError_t e = conv_pipe_prepare(&pipe, s, pass, path == 2 ? 1 : 3, 1, in, hi, hi + nw, out, nullptr, false, nullptr,
+        const cudaError_t e = conv_pipe_prepare(&pipe, s, pass, path == 2 ? 1 : 3, 1, 1, in, hi, hi + nw, out, nullptr, false, nullptr,
                                                 reinterpret_cast<char*>(d_scratch) + align_up(a > b ? a : b, 256), single_splitk_bytes(s), false);
         if (e == cudaSuccess) {
             CU(conv_pipe_launch(&pipe, 0, 1, false, status, st, nullptr));

@@ -1,14 +1,10 @@
 // Host code of the library that has no entry point of its own, without a GPU: linked with the library's objects, the runtime
 // calls that need a device replaced (-Wl,--wrap).  Usage: host_checks NAME; exit status 0 and a line of figures, or 1.
-#include "conv_pipe.h"
+#include "hpf_model.cu"          // the model's plans are its own: this file takes the place of its object
 
 #include <cstdio>
 #include <cstring>
 #include <map>
-#include <thread>
-#include <vector>
-
-using namespace hpf;
 
 static thread_local int g_device = 0;
 static std::mutex g_lock;
@@ -57,8 +53,68 @@ static int attributes_per_device()
     return 0;
 }
 
+// Two pre-activation bottleneck blocks on H x H maps behind a 3 -> c stem, and a head.
+static hpf_model* bottlenecks(int H, int c, int w, int co, int B, int M)
+{
+    std::vector<hpf_op> ops;
+    auto add = [&](int kind, int s0, int s1, int ci, int k, int ks) {
+        ops.push_back(hpf_op{kind, s0, s1, ci, k, ks, kind == HPF_OP_CONV || kind == HPF_OP_HEAD ? 1 : 0, kind == HPF_OP_CONV ? ks / 2 : 0, kind == HPF_OP_BNRELU ? 1e-5f : 0.f});
+        return (int)ops.size() - 1;
+    };
+    int t = add(HPF_OP_CONV, -1, -1, 3, c, 3);
+    for (int b = 0; b < 2; ++b) {
+        int v = add(HPF_OP_CONV, add(HPF_OP_BNRELU, t, -1, c, c, 0), -1, c, w, 1);
+        v = add(HPF_OP_CONV, add(HPF_OP_BNRELU, v, -1, w, w, 0), -1, w, w, 3);
+        v = add(HPF_OP_CONV, add(HPF_OP_BNRELU, v, -1, w, w, 0), -1, w, co, 1);
+        const int shortcut = b ? t : add(HPF_OP_CONV, t, -1, c, co, 1);
+        t = add(HPF_OP_ADD, v, shortcut, co, co, 0);
+        c = co;
+    }
+    add(HPF_OP_HEAD, add(HPF_OP_BNRELU, t, -1, c, c, 0), -1, c, 10, 0);
+    const int32_t shape[4] = {B, H, H, 3};
+    hpf_model* mdl = nullptr;
+    size_t bytes = 0;
+    if (hpf_model_create(ops.data(), (int32_t)ops.size(), shape, nullptr, 0, M, &mdl) != HPF_OK || hpf_workspace_bytes(mdl, &bytes) != HPF_OK) return nullptr;
+    return mdl;
+}
+
+// A cell's launches cover one micro-batch: their work is split for that, not for the M micro-batches of a step's launches.
+// The busiest CTA has at most a tenth more units than an even split over the GPU leaves it.
+static int cells_are_planned_for_one_micro_batch()
+{
+    const struct { int H, c, w, co, B, M; } nets[] = {{32, 16, 16, 64, 128, 8}, {32, 16, 16, 64, 128, 4}, {16, 64, 32, 128, 128, 4}, {56, 64, 64, 256, 64, 4},
+                                                      {14, 512, 256, 1024, 64, 4}, {27, 16, 16, 64, 42, 3}};
+    int finer = 0, seen = 0;
+    for (const auto& net : nets) {
+        hpf_model* mdl = bottlenecks(net.H, net.c, net.w, net.co, net.B, net.M);
+        CHECK(mdl);
+        const hpf_model::KernelPlan &step = mdl->kernels[0], &cell = mdl->cell_kernels();
+        CHECK(step.launched == net.M && cell.launched == 1);
+        for (int pass = 0; pass < 2; ++pass)
+            for (int i = 0; i < mdl->n_ops; ++i) {
+                CHECK(step.use_pipe[pass][i] == cell.use_pipe[pass][i]);
+                if (!cell.use_pipe[pass][i] || (pass == PASS_DGRAD && mdl->ops[i].op.src0 < 0)) continue;
+                const ConvPipeGeom& g = cell.pipe_geom[pass][i];
+                const int ctas = 148 / g.slices > 0 ? 148 / g.slices : 1;
+                const int busiest = (g.blocks_per_m * g.ksplit + ctas - 1) / ctas * g.unit_block, even = (g.units_per_m * g.ksplit + ctas - 1) / ctas;
+                CHECK(10 * busiest <= 11 * even);
+                finer += g.blocks_per_m * g.ksplit > step.pipe_geom[pass][i].blocks_per_m * step.pipe_geom[pass][i].ksplit;
+                ++seen;
+            }
+        hpf_model_destroy(mdl);
+    }
+    CHECK(seen > 60 && finer > 20);
+    // one plan where the step's launches cover one micro-batch anyway
+    hpf_model* one = bottlenecks(32, 16, 16, 64, 16, 1);
+    CHECK(one && &one->cell_kernels() == &one->kernels[0] && one->kernels[0].launched == 1);
+    hpf_model_destroy(one);
+    printf("%d launches, %d of them split finer than the step's\n", seen, finer);
+    return 0;
+}
+
 int main(int argc, char** argv)
 {
+    if (argc > 1 && !strcmp(argv[1], "cells_are_planned_for_one_micro_batch")) return cells_are_planned_for_one_micro_batch();
     if (argc > 1 && !strcmp(argv[1], "attributes_per_device")) return attributes_per_device();
     printf("unknown check\n");
     return 1;

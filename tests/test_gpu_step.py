@@ -412,6 +412,33 @@ def test_stage_per_gpu_hand_offs_emulated_on_one_gpu(P, R, cuts):
                 assert rel_l2(full[off:off + cnt], g_ref[off:off + cnt]) <= TOL_TENSOR, ("op", i)
 
 
+def test_cells_are_the_step_of_one_micro_batch_launches_bit_for_bit():
+    """Micro-batches of 16 images, where the work of a launch that covers one is split otherwise than that of a step's launches:
+    the cells equal the step with HPF_OPT_GROUP_LAUNCHES = 0 bit for bit, and the ordinary step to the rounding of its sums."""
+    from paper_1911_05146_b200.hybrid import HybridLayout, Stage, emulate_step
+    ops, B, M, hwc, cuts = wl.resnet_v2_cifar(1), 64, 4, (32, 32, 3), [9]
+    x, labels, theta = seeded(ops, hwc, B, seed=21, bn_jitter=0.2)
+    dev = torch.device("cuda:0")
+    layout = HybridLayout(2, 2)
+    stages = [Stage(ops, (B,) + hwc, cuts, M, torch.from_numpy(theta), p, dev) for p in range(2)]
+    slices = emulate_step(stages, layout, [(torch.from_numpy(x).to(dev), torch.from_numpy(labels).to(dev))])
+    cells = torch.cat([slices[rank] for rank in range(2)])
+    out = {}
+    for grouped in (0, 1):
+        bd = Bound(ops, hwc, B, M, cuts, theta, {hpf.OPT_GROUP_LAUNCHES: grouped})
+        bd.upload(x, labels)
+        bd.step()
+        out[grouped] = bd.avg.clone()
+        one_graph = Bound(ops, hwc, B, M, cuts, theta, {hpf.OPT_GROUP_LAUNCHES: grouped, hpf.OPT_CELL_TIMES: 1}, backward_streams=True)
+        one_graph.upload(x, labels)
+        one_graph.step(one_graph=True)
+        assert torch.equal(one_graph.avg, out[grouped])
+    assert torch.equal(cells, out[0])
+    ref = ora.step(ops, hwc, theta, x, labels, M, cuts=cuts)["g_avg"]
+    for g in out.values():
+        assert rel_l2(g.cpu().numpy(), ref) <= TOL_TENSOR
+
+
 def test_one_rank_of_the_hybrid_step_is_the_ordinary_step():
     """hybrid.run_step on a world of one rank (one replica, one partition): the same cells, the library's average, no
     neighbour and no allreduce; bit for bit the ordinary step without a CUDA graph."""
