@@ -126,7 +126,10 @@ int hpf_model_destroy(hpf_model *model);
  *                          the same SMs, so nothing forces that order: with L > 1 the cells (p, m) and (p, m + 1) may run side
  *                          by side, the hand-offs between stages are unchanged, and the idle slots of the pipeline's fill and
  *                          drain get used.  Every cell computes on the same data with the same kernels: results are
- *                          bit-identical for every L.  hpf_bind then wants its streams per (partition, lane).
+ *                          bit-identical for every L.  hpf_bind then wants its streams per (partition, lane).  Where a launch
+ *                          covers all micro-batches of a stage (the default: HPF_OPT_GROUP_LAUNCHES) they are all under way
+ *                          at once whatever L is; lanes matter with launches of one (that option 0, HPF_OPT_CELL_TIMES,
+ *                          HPF_OPT_KEEP_MESSAGES).
  *   HPF_OPT_WGRAD_DIRECT   1 (default): the tensor-core weight gradient hands its TMA tiles (pixels x channels, channels
  *                          innermost) to the tensor core as MN-major operands, as they land in shared memory; 0: the earlier
  *                          kernel, which transposes every tile in shared memory first (kept as a cross-check; also used for

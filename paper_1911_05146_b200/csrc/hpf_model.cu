@@ -137,7 +137,8 @@ struct hpf_model {
     std::vector<size_t> cell_bar_off;         // per stream of cells: the grid barrier's two words (zeroed at bind)
     // Stage lanes: a stage keeps up to `lanes` of its micro-batches under way at once, micro-batch m on lane m % lanes; every
     // lane has its own streams and its own scratch, so cells of different lanes share nothing but the parameters.  One
-    // lane is the paper's schedule (a stage works through its micro-batches one after the other).
+    // lane is the paper's schedule (a stage works through its micro-batches one after the other).  Launches that cover all
+    // micro-batches have them all under way anyway: lanes only matter where a step's launches cover one.
     int opt_wgrad_direct = 1;   // weight gradients read their TMA tiles as MN-major operands (0: the kernel that transposes them)
     int opt_lanes = 1;
     int lanes() const { return opt_lanes < M ? opt_lanes : M; }
@@ -148,7 +149,7 @@ struct hpf_model {
     // covers all micro-batches of a stage wherever nothing asks for cells of their own (then one micro-batch).  Every micro-batch keeps
     // its own statistics, losses and gradient slot, formed in the same order whatever the size of the group.
     int opt_group = 1;         // 0: launches of one micro-batch, planned as such
-    int group_size() const { return !opt_group || opt_messages || opt_cell_times || lanes() > 1 ? 1 : M; }
+    int group_size() const { return !opt_group || opt_messages || opt_cell_times ? 1 : M; }
     int n_groups() const { return M / group_size(); }
     int opt_fuse_bn = 3;       // bit 0: BN statistics in the producing convolution's write-out, bit 1: BN+ReLU applied by the reading convolution
     std::vector<GradEdge> edge0;              // per op: contribution to src0

@@ -112,8 +112,26 @@ static int cells_are_planned_for_one_micro_batch()
     return 0;
 }
 
+// What asks for cells of their own makes a step's launches cover one micro-batch; stage lanes, which only order them, do not.
+static int launches_cover_all_micro_batches()
+{
+    const struct { int option, value, covered; } cases[] = {{HPF_OPT_STAGE_LANES, 1, 4}, {HPF_OPT_STAGE_LANES, 2, 4}, {HPF_OPT_STAGE_LANES, 8, 4},
+                                                            {HPF_OPT_CELL_TIMES, 1, 1}, {HPF_OPT_KEEP_MESSAGES, 1, 1}, {HPF_OPT_GROUP_LAUNCHES, 0, 1}};
+    for (const auto& c : cases) {
+        hpf_model* mdl = bottlenecks(32, 16, 16, 64, 128, 4);
+        CHECK(mdl && hpf_set_option(mdl, c.option, c.value) == HPF_OK);
+        CHECK(mdl->group_size() == c.covered);
+        int32_t slots = 0;
+        CHECK(hpf_num_stream_slots(mdl, &slots) == HPF_OK && slots == (c.option == HPF_OPT_STAGE_LANES ? std::min(c.value, 4) : 1));
+        hpf_model_destroy(mdl);
+    }
+    printf("ok\n");
+    return 0;
+}
+
 int main(int argc, char** argv)
 {
+    if (argc > 1 && !strcmp(argv[1], "launches_cover_all_micro_batches")) return launches_cover_all_micro_batches();
     if (argc > 1 && !strcmp(argv[1], "cells_are_planned_for_one_micro_batch")) return cells_are_planned_for_one_micro_batch();
     if (argc > 1 && !strcmp(argv[1], "attributes_per_device")) return attributes_per_device();
     printf("unknown check\n");

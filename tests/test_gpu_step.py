@@ -336,6 +336,21 @@ def test_stage_lanes_give_the_same_bits_and_fill_the_bubble(lanes, one_graph):
     assert fwd[0][1][0] < fwd[0][0][1]
 
 
+@pytest.mark.parametrize("lanes,one_graph", [(2, True), (4, False), (8, True)])
+def test_stage_lanes_add_no_launches_to_a_step_that_covers_all_micro_batches(lanes, one_graph):
+    ops = wl.resnet_v2_cifar(1)
+    x, labels, theta = seeded(ops, (32, 32, 3), 8, seed=6, bn_jitter=0.1)
+    out = []
+    for L in (1, lanes):
+        bd = Bound(ops, (32, 32, 3), 8, 4, wl.default_cuts(len(ops), 3), theta, {hpf.OPT_STAGE_LANES: L}, backward_streams=one_graph)
+        bd.upload(x, labels)
+        for _ in range(2):
+            loss = bd.step(one_graph=one_graph)
+        out.append((loss, bd.model.launch_count(), bd.slots.clone(), bd.avg.clone()))
+    assert out[0][:2] == out[1][:2]
+    assert torch.equal(out[0][2], out[1][2]) and torch.equal(out[0][3], out[1][3])
+
+
 def test_the_environment_changes_nothing_between_two_steps_of_a_bound_model(monkeypatch):
     """How many micro-batches a launch covers follows from the model's options alone: a variable that once set it, changed
     after hpf_bind, leaves the launches of the next step as they were."""
