@@ -9,6 +9,10 @@ enum ConvPass { PASS_FWD = 0, PASS_DGRAD = 1, PASS_WGRAD = 2 };
 // Whether the tensor-core kernels cover this shape for this pass.
 bool conv_tc_supported(const ConvShape& s, int pass);
 
+// Whether a forward or data-gradient convolution without BN work of its own is faster here than as a pipelined launch
+// (conv_pipe.h), which covers the same shapes.
+bool conv_tc_faster_alone(const ConvShape& s, int pass, int passes);
+
 // Resolves the driver entry point used to encode tensor maps.  Needs a CUDA driver.
 cudaError_t conv_tc_init();
 

@@ -1801,8 +1801,10 @@ static int conv_single(int pass, const float* in, const float* in2, const float*
         const size_t a = conv_simt_scratch_bytes(s), b = conv_tc_scratch_bytes(s);
         ConvPipePlan pipe;
         CU(conv_pipe_init());
-        const cudaError_t e = conv_pipe_prepare(&pipe, s, pass, path == 2 ? 1 : 3, 1, 1, in, hi, hi + nw, out, nullptr, false, nullptr,
-                                                reinterpret_cast<char*>(d_scratch) + align_up(a > b ? a : b, 256), single_splitk_bytes(s), false);
+        const cudaError_t e = conv_tc_faster_alone(s, pass, path == 2 ? 1 : 3)
+                                  ? cudaErrorNotSupported
+                                  : conv_pipe_prepare(&pipe, s, pass, path == 2 ? 1 : 3, 1, 1, in, hi, hi + nw, out, nullptr, false, nullptr,
+                                                      reinterpret_cast<char*>(d_scratch) + align_up(a > b ? a : b, 256), single_splitk_bytes(s), false);
         if (e == cudaSuccess) {
             CU(conv_pipe_launch(&pipe, 0, 1, false, status, st, nullptr));
             return HPF_OK;

@@ -129,8 +129,27 @@ static int launches_cover_all_micro_batches()
     return 0;
 }
 
+// Which kernel a convolution that is called by itself runs on.
+static int calls_by_themselves()
+{
+    auto tile = [](int N, int H, int C, int K, int R, int stride, int pass, int passes) {
+        return conv_tc_faster_alone(make_conv_shape(N, H, H, C, K, R, stride, R / 2), pass, passes);
+    };
+    CHECK(tile(16, 32, 64, 16, 1, 1, PASS_FWD, 3) && tile(10, 17, 512, 32, 1, 2, PASS_FWD, 3));
+    CHECK(tile(37, 32, 64, 16, 1, 1, PASS_FWD, 3) && !tile(38, 32, 64, 16, 1, 1, PASS_FWD, 3));            // 296 tiles
+    CHECK(tile(74, 16, 16, 64, 1, 1, PASS_FWD, 3) && !tile(75, 16, 16, 64, 1, 1, PASS_FWD, 3));            // 148 x 64 outputs
+    CHECK(!tile(75, 16, 16, 256, 1, 1, PASS_FWD, 3) && tile(75, 16, 16, 256, 1, 1, PASS_DGRAD, 3));        // the two ways differ
+    CHECK(!tile(75, 16, 96, 96, 1, 1, PASS_FWD, 3) && tile(75, 16, 96, 96, 1, 1, PASS_FWD, 1));            // one pass, and not widening
+    CHECK(!tile(75, 16, 64, 96, 1, 1, PASS_FWD, 1));
+    CHECK(tile(37, 15, 64, 48, 1, 2, PASS_FWD, 3) && tile(74, 15, 48, 64, 1, 2, PASS_FWD, 3) && !tile(74, 15, 128, 48, 1, 2, PASS_DGRAD, 3));
+    CHECK(!tile(64, 56, 64, 256, 1, 1, PASS_FWD, 1) && !tile(4, 8, 64, 64, 3, 1, PASS_FWD, 3));
+    printf("ok\n");
+    return 0;
+}
+
 int main(int argc, char** argv)
 {
+    if (argc > 1 && !strcmp(argv[1], "calls_by_themselves")) return calls_by_themselves();
     if (argc > 1 && !strcmp(argv[1], "launches_cover_all_micro_batches")) return launches_cover_all_micro_batches();
     if (argc > 1 && !strcmp(argv[1], "cells_are_planned_for_one_micro_batch")) return cells_are_planned_for_one_micro_batch();
     if (argc > 1 && !strcmp(argv[1], "attributes_per_device")) return attributes_per_device();

@@ -28,6 +28,20 @@ def test_convolutions_at_the_edges_of_the_tiling(N, ks, st, ci, co, H, path):
 
 
 @pytest.mark.parametrize("N,ks,st,ci,co,H", [
+    (37, 1, 1, 32, 16, 32),      # 296 tiles: the most the tile kernel takes; its data gradient is as wide as it may be
+    (38, 1, 1, 32, 16, 32),      # 304: pipelined
+    (37, 1, 1, 48, 64, 16),      # 74 tiles of 64 channels, 48 the other way
+    (75, 1, 1, 16, 256, 16),     # pipelined forward, the tile kernel's data gradient
+    (75, 1, 1, 96, 96, 16),      # one pass on the tile kernel, three pipelined
+    (37, 1, 2, 64, 48, 15),      # strided, ragged tiles: the data gradient beyond its quarter of the line
+    (2, 1, 2, 16, 32, 9)], ids=str)
+@pytest.mark.parametrize("path", [0, 2])
+def test_one_by_one_windows_on_either_side_of_the_kernels_line(N, ks, st, ci, co, H, path):
+    e = _conv_case(ks, st, ci, co, H, N, path)
+    assert max(e) <= (2e-5 if path == 0 else TOL_TENSOR), e
+
+
+@pytest.mark.parametrize("N,ks,st,ci,co,H", [
     (1, 3, 1, 3, 16, 5),         # a stem: 16-wide tiles, the k steps shared by the block's warps
     (3, 7, 2, 3, 64, 17),
     (2, 3, 2, 16, 32, 9),        # strided: four classes of input positions of unequal size
