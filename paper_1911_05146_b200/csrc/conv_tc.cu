@@ -1188,10 +1188,12 @@ void wgrad_splits(const ConvShape& s, int n_tiles, int ctas_per_split, int launc
     if (cap < want) cap = want;
     if (splits > cap) splits = cap;
     if (splits > 296) splits = 296;          // two CTAs per SM
-    if (launched > 1) {
-        // The launch covers several micro-batches, each with its own sums.  It runs beside the chain of data gradients,
-        // which wants whole SMs, and its partial sums are written and read again: one and a half CTAs per SM in all.
-        // 592 / 296 / 222 / 148 / 74 CTAs: resnet152 39.2 / 37.9 / 36.6 / 36.8 / 36.9 ms, resnet110 6.71 / 6.61 / 6.53 / 6.50 / 6.71.
+    if (launched > 0) {
+        // Inside a step the launch covers all micro-batches of a stage, each with its own sums, and runs beside the chain of data
+        // gradients, which wants whole SMs; its partial sums are written and read again: one and a half CTAs per SM in all.
+        // 592 / 296 / 222 / 148 / 74 CTAs: resnet152 39.2 / 37.9 / 36.6 / 36.8 / 36.9 ms, resnet110 6.71 / 6.61 / 6.53 / 6.50 / 6.71,
+        // resnet1001 - / - / 60.2 / 60.9 / -; one micro-batch: resnet110 of 128 images 6.83 (296) / 6.60 (222) / 6.62 (148), wide
+        // resnet182 of 64 8.88 / 8.77 / 8.81.
         int ms = 222 / (ctas_per_split * launched);
         if (ms < 1) ms = 1;
         if (splits > ms) splits = ms;
@@ -1462,7 +1464,7 @@ cudaError_t conv_tc_prepare(ConvTcPlan* plan, const ConvShape& s, int pass, int 
                             const ConvTcHints* hints)
 {
     plan->valid = 0; plan->s = s; plan->pass = pass; plan->direct = 0;
-    const int M = hints && hints->micro_batches > 1 ? hints->micro_batches : 1, launched = hints ? hints->launched : 1;
+    const int M = hints && hints->micro_batches > 1 ? hints->micro_batches : 1, launched = hints ? hints->launched : 0;
     const long long dw_ms = hints ? hints->slot_stride : 0;
     if (passes != 1 && passes != 3) return cudaErrorInvalidValue;
     WgradDirectGeom dg;

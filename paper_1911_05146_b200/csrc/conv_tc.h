@@ -16,8 +16,8 @@ bool conv_tc_faster_alone(const ConvShape& s, int pass, int passes);
 // Resolves the driver entry point used to encode tensor maps.  Needs a CUDA driver.
 cudaError_t conv_tc_init();
 
-// weight-gradient partials of one micro-batch; launched: micro-batches a launch covers (ConvTcHints)
-size_t conv_tc_scratch_bytes(const ConvShape& s, int launched = 1);
+// weight-gradient partials of one micro-batch; launched: as in ConvTcHints
+size_t conv_tc_scratch_bytes(const ConvShape& s, int launched = 0);
 
 // A prepared launch: tensor maps are encoded once (they bake in the device pointers) and the kernel
 // parameters are kept ready in `storage`.
@@ -34,7 +34,7 @@ struct ConvTcHints {
     // the model's micro-batches, contiguous in every tensor; for a weight gradient the floats between their outputs and
     // between their partial sums (0: packed)
     int micro_batches = 1;
-    int launched = 1;            // how many of them the launches this is planned for cover
+    int launched = 0;            // how many of them the launches this is planned for cover; 0: a call by itself, not part of a step
     long long slot_stride = 0;
     long long partial_stride = 0;
     // weight gradient only: 1 keeps the kernel that transposes its tiles in shared memory (a cross-check)

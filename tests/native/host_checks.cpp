@@ -147,8 +147,22 @@ static int calls_by_themselves()
     return 0;
 }
 
+// A step's weight gradients run beside its chain of data gradients whether it has one micro-batch or several: the same limit
+// on their CTAs (and so on their partial sums); a call by itself has the GPU.
+static int weight_gradients_of_a_step()
+{
+    const ConvShape s = make_conv_shape(128, 32, 32, 64, 16, 1, 1, 0);
+    const size_t slice = (size_t)s.K * s.C * sizeof(float);
+    CHECK(conv_tc_scratch_bytes(s, 1) <= 222 * slice && conv_tc_scratch_bytes(s, 1) > 148 * slice);
+    CHECK(conv_tc_scratch_bytes(s, 2) <= 111 * slice);
+    CHECK(conv_tc_scratch_bytes(s) > 222 * slice);
+    printf("ok\n");
+    return 0;
+}
+
 int main(int argc, char** argv)
 {
+    if (argc > 1 && !strcmp(argv[1], "weight_gradients_of_a_step")) return weight_gradients_of_a_step();
     if (argc > 1 && !strcmp(argv[1], "calls_by_themselves")) return calls_by_themselves();
     if (argc > 1 && !strcmp(argv[1], "launches_cover_all_micro_batches")) return launches_cover_all_micro_batches();
     if (argc > 1 && !strcmp(argv[1], "cells_are_planned_for_one_micro_batch")) return cells_are_planned_for_one_micro_batch();

@@ -25,7 +25,8 @@ def checks(tmp_path_factory):
     return exe
 
 
-@pytest.mark.parametrize("name", ["attributes_per_device", "cells_are_planned_for_one_micro_batch", "launches_cover_all_micro_batches", "calls_by_themselves"])
+@pytest.mark.parametrize("name", ["attributes_per_device", "cells_are_planned_for_one_micro_batch", "launches_cover_all_micro_batches", "calls_by_themselves",
+                                  "weight_gradients_of_a_step"])
 def test_host(checks, name):
     r = subprocess.run([checks, name], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0, r.stdout + r.stderr
