@@ -1305,11 +1305,14 @@ static bool plan_geom(const ConvShape& s, int pass, int passes, int launched, Co
                         if (b_all + fixed + 2 * a_stage > kPipeSmem) break;
                         int as = (int)((kPipeSmem - fixed - b_all) / a_stage);
                         if (as > kMaxA) as = kMaxA;
-                        for (; as >= 2; --as) {
-                        const int groups = split_groups_of(as);
-                        const double split = three ? 250.0 + 5.6 * rows * groups / 4.0 : 100.0;
                         const double mma = resident ? taps * tap_mma + 100.0
                                                     : (double)(taps / bt) * std::max({bt * tap_mma + 100.0, (1000.0 + b_stage / 40.0 + bt * tap_mma) / bs, b_stage / 28.0});
+                        // (of the rings that serve the same number of groups the deepest is the best)
+                        for (int tried = 0; as >= 2 && tried != 7; --as) {
+                        const int groups = split_groups_of(as);
+                        if (tried & groups) continue;
+                        tried |= groups;
+                        const double split = three ? 250.0 + 5.6 * rows * groups / 4.0 : 100.0;
                         const double chunk = std::max({mma, (1200.0 + rows * 1.6 + split + mma) / as, split / groups, rows * 64.0 / 20.0});
                         const double k_loop = chunk * chunks, body = bufs == 2 ? std::max(k_loop, epi) : k_loop + epi;
                         const double cost = rounds * body + chunk + 1000.0 + epi;
