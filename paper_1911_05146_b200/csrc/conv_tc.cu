@@ -1406,7 +1406,9 @@ int unfused_n_chunk(int c_out, int tiles)
 // A small 1x1 window: two of its CTAs fit an SM, so the whole launch is resident at once, one tile each, and starts under the
 // one before it, while a pipelined CTA takes an SM to itself and works through its 16-channel chunks one after the other.  Small is
 // up to 128 x 64 outputs per SM; twice that for one pass over at least as many channels as come out, where those chunks are the
-// longer chain; a quarter for the strided data gradient, which writes four times the pixels it computes.
+// longer chain; a quarter for the strided data gradient, which writes four times the pixels it computes.  Beyond 512 channels
+// in, the pipelined kernel's finer split of the K loop wins (4096 -> 4096 on 128 pixels 48 us against 64, 2048 -> 512 on 16 maps of
+// 7 x 7 31 / 44, 1024 -> 1024 on 4 of 7 x 7 23.5 / 26.4).
 // Measured on 136 drawn 1x1 shapes both ways (16..512 channels, maps of 4..56, batch 4..128, one and three passes, calls back to
 // back): inside the line 0.61 of the pipelined launch's time (geometric mean of 189, one of them above 1.05: 9.6 us against 8.8;
 // 512 -> 32 channels on 10 maps of 17 x 17 12 us against 29, 64 -> 16 on 16 maps of 32 x 32 5.0 against 9.1), outside 1.15
@@ -1418,7 +1420,7 @@ bool conv_tc_faster_alone(const ConvShape& s, int pass, int passes)
     long long line = 148 * 64;
     if (passes == 1 && c_in >= c_out) line *= 2;
     if (pass == PASS_DGRAD && s.stride > 1) line /= 4;
-    return s.R == 1 && tiles <= 2 * 148 && tiles * c_out <= line;
+    return s.R == 1 && c_in <= 512 && tiles <= 2 * 148 && tiles * c_out <= line;
 }
 
 size_t conv_tc_splitk_bytes(const ConvShape& s, int pass, int passes)

@@ -142,6 +142,7 @@ static int calls_by_themselves()
     CHECK(!tile(75, 16, 96, 96, 1, 1, PASS_FWD, 3) && tile(75, 16, 96, 96, 1, 1, PASS_FWD, 1));            // one pass, and not widening
     CHECK(!tile(75, 16, 64, 96, 1, 1, PASS_FWD, 1));
     CHECK(tile(37, 15, 64, 48, 1, 2, PASS_FWD, 3) && tile(74, 15, 48, 64, 1, 2, PASS_FWD, 3) && !tile(74, 15, 128, 48, 1, 2, PASS_DGRAD, 3));
+    CHECK(tile(16, 7, 512, 64, 1, 1, PASS_FWD, 3) && !tile(16, 7, 528, 64, 1, 1, PASS_FWD, 3) && tile(16, 7, 528, 64, 1, 1, PASS_DGRAD, 3));
     CHECK(!tile(64, 56, 64, 256, 1, 1, PASS_FWD, 1) && !tile(4, 8, 64, 64, 3, 1, PASS_FWD, 3));
     printf("ok\n");
     return 0;
