@@ -80,10 +80,10 @@ def measure_tf32_peak(torch, seconds=2.0):
 
 
 def dram_traffic_table():
-    """DRAM bytes of the convolution kernel per launch as ncu counted them, from the tracked summary
-    profiles/conv_tc_fwd_dram_traffic.txt: rows `ksize stride c_in c_out H batch read_bytes write_bytes`."""
+    """DRAM bytes of the pipelined convolution kernel per launch as ncu counted them, from the tracked summary
+    profiles/conv_pipe_dram_traffic.txt: rows `ksize stride c_in c_out H batch read_bytes write_bytes`."""
     table = {}
-    path = os.path.join(ROOT, "profiles", "conv_tc_fwd_dram_traffic.txt")
+    path = os.path.join(ROOT, "profiles", "conv_pipe_dram_traffic.txt")
     if os.path.exists(path):
         for line in open(path):
             f = line.split("#")[0].split()
@@ -230,10 +230,11 @@ def aggregate_throughput(world, batch_per_rank, ms_per_step):
 def kernel_roofline(torch, hpf, cfg, pk):
     """The dominant kernel of the step (the tensor-core convolution forward / data-gradient kernel: a third of the
     summed kernel time in the ncu launch list, profiles/) timed alone through the C ABI on the workload's heaviest
-    convolution shape at the micro-batch size, cycling through operand sets that together exceed L2.  The calls are
-    captured once into a CUDA graph and the replay is timed with CUDA events on the launching stream, so that the
-    figure is the kernel's launch-to-launch duration and not the host's call overhead."""
-    b = cfg["B"] // cfg["M"]
+    convolution shape, one launch over all images of the batch, as many as a launch of the step covers (its micro-batches
+    together; there the BN on either side rides in it, here it does not), cycling through operand sets that together exceed L2.
+    The calls are captured once into a CUDA graph and the replay is timed with CUDA events on the launching stream, so that
+    the figure is the kernel's launch-to-launch duration and not the host's call overhead."""
+    b = cfg["B"]
     shapes = wl.tensor_shapes(cfg["ops"], cfg["in_hwc"])
     weight = {}
     for i, o in enumerate(cfg["ops"]):
@@ -277,18 +278,17 @@ def kernel_roofline(torch, hpf, cfg, pk):
     achieved = alg / sec / 1e9
     cap = dram_traffic_table().get((ks, st, ci, co, H))
     traffic = cap[1] * b / cap[0] if cap else None
+    pipelined = ks == 3 or ci > 512 or (b * P * P + 127) // 128 * co > 148 * 64      # (a small 1x1 call by itself takes the other kernel)
     return {"bound": "hbm", "achieved": achieved, "peak": pk["hbm_gbs"], "unit": "GB/s", "frac": achieved / pk["hbm_gbs"],
             # dram__bytes_read + dram__bytes_write of this kernel in the ncu capture of the same shape (tracked table under
-            # profiles/, captured at a batch whose operands exceed L2), scaled by the pixels per launch: traffic grows in
-            # proportion to the pixels (the input is read once, nothing is re-read); null when no capture covers the shape
-            "traffic": traffic,
+            # profiles/, captured at batch 128), scaled by the pixels per launch: traffic grows in proportion to the pixels (the
+            # input is read once, nothing is re-read); null when no capture covers the shape or the launch is small
+            "traffic": traffic if pipelined else None,
             "peak_source": pk["source"],
-            "kernel": "conv_pipe_kernel (tcgen05 implicit GEMM, three-pass TF32), %dx%d stride %d, %d->%d channels, %dx%d "
-                      "pixels, micro-batch %d; %d rotating operand sets, kernel nodes only, launched with programmatic dependent launch as in the step"
-                      % (ks, ks, st, ci, co, H, H, b, nset),
-            "algorithmic_bytes_per_launch": alg, "us_per_launch": sec * 1e6,
-            "note": "at the micro-batch size the kernel is latency bound (one 128-pixel tile per CTA, %d CTAs); "
-                    "the batch-128 sweep (--workload conv_sweep) gives the bandwidth-bound figures" % ((b * P * P + 127) // 128)}
+            "kernel": "%s (tcgen05 implicit GEMM, three-pass TF32), %dx%d stride %d, %d->%d channels, %dx%d "
+                      "pixels, %d images; %d rotating operand sets, kernel nodes only, launched with programmatic dependent launch"
+                      % ("conv_pipe_kernel" if pipelined else "conv_tc_fwd_kernel", ks, ks, st, ci, co, H, H, b, nset),
+            "algorithmic_bytes_per_launch": alg, "us_per_launch": sec * 1e6}
 
 
 def run_hybrid(args, cfg, torch, hpf, dist, rank, local, world, dev):

@@ -31,7 +31,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     procs = []
     for src in _sources():
         obj = os.path.join(CSRC, os.path.basename(src)[:-3] + ".o")
-        extra = os.environ.get("HPF_NVCC_EXTRA", "").split()          # e.g. -DHPF_TC_TIMELINE for latency studies
+        extra = os.environ.get("HPF_NVCC_EXTRA", "").split()          # e.g. -DHPF_RES_TIMELINE for latency studies
         cmd = [nvcc] + [f for f in NVCC_FLAGS if not f.startswith("--use_fast_math")] + extra + (["-Xptxas", "-v"] if verbose else []) + ["-c", src, "-o", obj]
         procs.append((cmd, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
         objs.append(obj)

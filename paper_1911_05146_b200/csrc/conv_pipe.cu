@@ -22,8 +22,9 @@
 // fit), warp 2 issues the MMAs, warps 4-7 rewrite the operand in place (BN+ReLU, lo part), warps 8-15 read finished
 // accumulators from tensor memory, add the residual, store and form the BN moments.
 //
-// Measured alone, batch 128, three passes (before: one 128-pixel tile per CTA, nine copies per 3x3 tile): 3x3 16->16 @32
-// 45 -> 19 us, 64->64 @32 107 -> 65, 128->128 @16 61 -> 45; 1x1 64->64 @32 31 -> 22, 16->64 @32 23 -> 17 (2.5 TB/s).
+// Measured alone, batch 128, three passes, against the tile kernel's one 128-pixel tile per CTA and nine copies per 3x3 tile:
+// 3x3 16->16 @32 45 -> 20 us, 64->64 @32 107 -> 68, 128->128 @16 58 -> 48; 1x1 64->64 @32 31 -> 25, 16->64 @32 23 -> 18 (2.3 TB/s),
+// but 64->16 @32 18 -> 22 (profiles/conv_sweep_batch128.md).
 #include "conv_pipe.h"
 #include "tc_ptx.cuh"
 

@@ -10,6 +10,9 @@ pipeline, reads how long every (partition, micro-batch) cell really took while t
 (`hpf_cell_times`), apportions each partition's measured time to its ops in proportion to their modelled cost, asks
 `hpf_balance_cuts` for the cuts that even out those costs, and repeats; the fastest cut list seen wins.  Cuts change
 nothing in the arithmetic (the oracle's partition-count invariance), only which stage runs what.
+Reading cell times makes every launch cover one micro-batch (OPT_CELL_TIMES); an ordinary step on one GPU has launches that
+cover all of them, for which cuts hardly matter.  What the measurement balances is the pipeline of single cells, whose shares
+carry over to a run with a GPU per partition; "ms" in the history is the step measured that way.
 """
 import torch
 
