@@ -805,7 +805,10 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
         // channels, or alternate tiles where there is one group.
         const bool alternate = p.epi_alternate != 0, by_tile = !alternate && groups == 1, whole = alternate || by_tile;
         const int g_first = whole ? 0 : half, g_step = whole ? 1 : 2, t_first = by_tile ? half : 0, t_step = by_tile ? 2 : 1;
-        const int parts = whole ? 8 : 4, part = whole ? ew : quad;
+        // (alternating sets: a block's first unit always counts as part 0..3, whichever set's turn it is, so that its moments are
+        // added in the same order wherever in a CTA's work the block stands)
+        const int parts = whole ? 8 : 4;
+        int part = whole ? ew : quad;
         int turn = 0;
         float4* patch = reinterpret_cast<float4*>(smem + p.off_stage) + ew * 256;
         if (!CELL) pdl_wait();
@@ -945,6 +948,7 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
                 float* counts = contrib + (size_t)parts * 3 * n_chunk;
                 if (lane == 0 && (whole || half == 0)) counts[part] = (float)count;
                 count = 0; have = false;
+                if (alternate) part = ew ^ (turn << 2);
                 epi_sync();
                 if (BNB && tid < n_chunk) {
                     float sum = 0.f, sq = 0.f;

@@ -427,6 +427,20 @@ def test_stage_per_gpu_hand_offs_emulated_on_one_gpu(P, R, cuts):
                 assert rel_l2(full[off:off + cnt], g_ref[off:off + cnt]) <= TOL_TENSOR, ("op", i)
 
 
+def test_launches_of_one_micro_batch_and_of_all_add_in_the_same_order():
+    """Eight micro-batches of 32 images: a CTA of a launch over all of them takes several blocks of seven units, so that a block
+    may begin on either set of the write-out's warps; in a launch of one it takes a single block.  The moments of a BN, and all
+    that follows, are the same bits."""
+    ops, B, M, hwc = wl.resnet_v2_cifar(1), 256, 8, (32, 32, 3)
+    x, labels, theta = seeded(ops, hwc, B, seed=22, bn_jitter=0.2)
+    out = []
+    for opts in ({}, {hpf.OPT_CELL_TIMES: 1}):
+        bd = Bound(ops, hwc, B, M, [], theta, opts)
+        bd.upload(x, labels)
+        out.append((bd.step(), bd.slots.clone()))
+    assert out[0][0] == out[1][0] and torch.equal(out[0][1], out[1][1])
+
+
 def test_cells_are_the_step_of_one_micro_batch_launches_bit_for_bit():
     """Micro-batches of 16 images, where the work of a launch that covers one is split otherwise than that of a step's launches:
     the cells equal the step with HPF_OPT_GROUP_LAUNCHES = 0 bit for bit, and the ordinary step to the rounding of its sums."""
