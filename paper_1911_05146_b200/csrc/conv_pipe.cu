@@ -18,13 +18,15 @@
 // Operand rows.  A chunk is 16 channels: bytes 0-63 of the 128-byte row hold the value (the tensor core ignores the low 13
 // mantissa bits: that is the hi part), bytes 64-127 the lo part of the three-pass form, in the 128-byte swizzle.
 //
-// Roles (16 warps): warp 0 copies the operand, warp 1 the weights (TMA; kept in shared memory for the whole launch when they
-// fit), warp 2 issues the MMAs, warps 4-7 rewrite the operand in place (BN+ReLU, lo part), warps 8-15 read finished
-// accumulators from tensor memory, add the residual, store and form the BN moments.
+// Roles (16 warps): warp 0 copies the operand (a 1x1 window's without a stride: warps 0 and 3, 16 bytes a lane), warp 1 the
+// weights (TMA; kept in shared memory for the whole launch when they fit), warp 2 issues the MMAs, warps 4-7 rewrite the operand
+// in place (BN+ReLU, lo part), warps 8-15 read finished accumulators from tensor memory, add the residual, store and form
+// the BN moments.
 //
-// Measured alone, batch 128, three passes, against the tile kernel's one 128-pixel tile per CTA and nine copies per 3x3 tile:
-// 3x3 16->16 @32 45 -> 20 us, 64->64 @32 107 -> 68, 128->128 @16 58 -> 48; 1x1 64->64 @32 31 -> 25, 16->64 @32 23 -> 18 (2.3 TB/s),
-// but 64->16 @32 18 -> 22 (profiles/conv_sweep_batch128.md).
+// Measured alone, batch 128, three passes (graph of ten launches), before and since the write-out reads rows (write_out), the MMAs are
+// issued in straight lines (mma_role) and the operand of a 1x1 window is copied by lanes: 3x3 16->16 @32 19.8 -> 15.5 us,
+// 64->64 @8 15.1 -> 11.6; 1x1 64->16 @32 21.8 -> 13.7, 16->64 @32 17.8 -> 14.3; batch 64: 3x3 64->64 @56 90 -> 74, 256->256 @14 82 -> 73;
+// 1x1 64->256 @56 70 -> 73, 256->64 @56 86 -> 69, 512->128 @28 54 -> 43, 1024->256 @14 56 -> 41.
 #include "conv_pipe.h"
 #include "tc_ptx.cuh"
 
@@ -54,7 +56,7 @@ struct PipeScalars {
     int units_per_m, unit_block, blocks_per_m, tiles_per_m, T, slices, n_chunk, ksplit;
     int R, taps, n_chunks, c_in, c_out;
     int pos_per_m, Wp, img_pos, Hv, W, halo, strips, strip_w, col0;
-    uint32_t magic_w, magic_img, magic_strip;
+    uint32_t magic_w, magic_img, magic_strip, magic_blocks, magic_ksplit;
     int in_sw, in_sh, in_sn, os_w, os_h, os_n;
     int zero_fill, out_h, out_w, dense_h, dense_w;
     int a_stages, b_stages, b_taps, b_resident, acc_bufs, split_groups, epi_alternate;
@@ -63,7 +65,8 @@ struct PipeScalars {
     uint32_t magic_box, magic_bpi;
     long long pix_ms;                                 // flat: pixels per micro-batch; else maps per micro-batch
     uint32_t a_stage_bytes, b_stage_bytes, b_tap_bytes, acc_cols, tmem_cols, idesc, idesc2;
-    uint32_t off_b, off_bn, off_red, off_stat, off_stage;
+    uint32_t off_b, off_bn, off_red, off_stat, off_slots, off_ring, off_bnb, slot_bytes;
+    int wide;                                         // a write-out lane has 8 channels of a row (else 4)
     int three, stacked, pdl_late, w_ready;
     // BN+ReLU on the way in
     const float* bn_partials;
@@ -118,22 +121,45 @@ __device__ __forceinline__ Pixel locate(const PipeScalars& p, int pos)
     return r;
 }
 
-// 16 consecutive floats of one thread: two full sectors
-__device__ __forceinline__ void store16(float* d, const float* v)
+// W = 4 or 8 consecutive floats of one thread (16 or 32 bytes, aligned).  Reads are ordered ones: the preceding kernel may have
+// written what they fetch.
+template <int W>
+__device__ __forceinline__ void store_vec(float* d, const float* v)
 {
-    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(d), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]),
-                 "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]) : "memory");
-    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(d + 8), "f"(v[8]), "f"(v[9]), "f"(v[10]), "f"(v[11]),
-                 "f"(v[12]), "f"(v[13]), "f"(v[14]), "f"(v[15]) : "memory");
+    if constexpr (W == 8)
+        asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(d), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]),
+                     "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]) : "memory");
+    else *reinterpret_cast<float4*>(d) = make_float4(v[0], v[1], v[2], v[3]);
 }
-__device__ __forceinline__ void load16(const float* s, float* v)
+template <int W>
+__device__ __forceinline__ void load_vec(const float* s, float* v)
 {
 #pragma unroll
-    for (int j = 0; j < 16; j += 4) {
+    for (int j = 0; j < W; j += 4) {
         const float4 t = __ldcg(reinterpret_cast<const float4*>(s + j));
         v[j] = t.x; v[j + 1] = t.y; v[j + 2] = t.z; v[j + 3] = t.w;
     }
 }
+// the same in shared memory
+template <int W>
+__device__ __forceinline__ void read_vec(const float* s, float* v)
+{
+#pragma unroll
+    for (int j = 0; j < W; j += 4) {
+        const float4 t = *reinterpret_cast<const float4*>(s + j);
+        v[j] = t.x; v[j + 1] = t.y; v[j + 2] = t.z; v[j + 3] = t.w;
+    }
+}
+__device__ __forceinline__ void cp_async16(uint32_t dst, const float* src) { asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory"); }
+__device__ __forceinline__ void cp_async16_zfill(uint32_t dst, const float* src, bool real)
+{
+    asm volatile("cp.async.cg.shared.global.L2::256B [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(real ? 16 : 0) : "memory");
+}
+// arrives (once a lane) when this lane's copies so far have landed
+__device__ __forceinline__ void cp_async_arrive(uint32_t bar) { asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar) : "memory"); }
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int LEFT>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(LEFT) : "memory"); }
 __device__ __forceinline__ void split_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kSplitThreads) : "memory"); }
 __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 2, 256;" ::: "memory"); }
 
@@ -161,6 +187,13 @@ __device__ __forceinline__ float4 fma4(float4 a, float4 b, float4 c)
 {
     return unpair4(fma2(pair(a.x, a.y), pair(b.x, b.y), pair(c.x, c.y)), fma2(pair(a.z, a.w), pair(b.z, b.w), pair(c.z, c.w)));
 }
+// acc[0..W) op= ..., two at a time
+template <int W>
+__device__ __forceinline__ void add_to(float* acc, const float* v)
+{
+#pragma unroll
+    for (int j = 0; j < W; j += 2) unpair(add2(pair(acc[j], acc[j + 1]), pair(v[j], v[j + 1])), acc[j], acc[j + 1]);
+}
 // what the tensor core ignores of a value
 __device__ __forceinline__ float4 lo_part(float4 v) { return sub4(v, make_float4(tf32_hi(v.x), tf32_hi(v.y), tf32_hi(v.z), tf32_hi(v.w))); }
 
@@ -183,7 +216,7 @@ __device__ __forceinline__ void merge_moments(const float* partials, int rows, i
         const bool mine = local < width && ln < L;
         float4 sd = make_float4(0.f, 0.f, 0.f, 0.f), sq = sd, m2 = sd, ref = sd;
         if (mine) {
-            ref = __ldcg(reinterpret_cast<const float4*>(partials) + col);
+            if (rows > 0) ref = __ldcg(reinterpret_cast<const float4*>(partials) + col);
 #pragma unroll 1
             for (int k0 = ln; k0 < rows; k0 += 4 * L) {
                 float4 a[4], b[4];
@@ -241,12 +274,14 @@ __device__ __forceinline__ void merge_moments(const float* partials, int rows, i
 struct UnitWalk {
     int m, ul, z, left;          // left: blocks, the current one included
     int end;                     // first unit beyond the current block
+    int row;                     // first block's number within its micro-batch
     __device__ __forceinline__ UnitWalk(const PipeScalars& p, int m_first, int first, int count) : left(count)
     {
         z = 0;
-        if (p.ksplit > 1) { z = first % p.ksplit; first /= p.ksplit; }
-        m = first / p.blocks_per_m;
-        ul = (first - m * p.blocks_per_m) * p.unit_block;
+        if (p.ksplit > 1) { const int whole = div_magic(first, p.ksplit, p.magic_ksplit); z = first - whole * p.ksplit; first = whole; }
+        m = div_magic(first, p.blocks_per_m, p.magic_blocks);
+        row = first - m * p.blocks_per_m;
+        ul = row * p.unit_block;
         m += m_first;
         set_end(p);
     }
@@ -265,8 +300,6 @@ struct UnitWalk {
         if (ul == p.units_per_m) { ul = 0; ++m; }
         set_end(p);
     }
-    __device__ __forceinline__ bool last_of_block() const { return ul + 1 == end; }
-    __device__ __forceinline__ bool last(const PipeScalars& p) const { return left == 1 && (p.ksplit > 1 || last_of_block()); }
     __device__ __forceinline__ int tiles(const PipeScalars& p) const { const int n = p.tiles_per_m - ul * p.T; return n < p.T ? n : p.T; }
     __device__ __forceinline__ int kb(const PipeScalars& p) const { return p.ksplit > 1 ? z * p.n_chunks / p.ksplit : 0; }
     __device__ __forceinline__ int ke(const PipeScalars& p) const { return p.ksplit > 1 ? (z + 1) * p.n_chunks / p.ksplit : p.n_chunks; }
@@ -291,175 +324,51 @@ __device__ __forceinline__ Span span_of(const PipeScalars& p, const UnitWalk& u)
     return r;
 }
 
-// What one warp does with 32 rows x 32 (or 16) columns of a finished tile, which stand in its patch of shared memory.
-struct EmitArgs {
-    float* out;                  // this warp's column group
-    const float* extra;
-    const float4* patch;
-    float* moments;              // the warp's k, sum (x - k), sum (x - k)^2 of its columns: three rows of mom_pitch floats, or null
-    int mom_pitch;
-    bool accumulate, ok;
-    int zero_fill, dense_h, dense_w;
-    // not null: `extra` is the input x of a BN+ReLU whose output gradient this is: it is not added; the sums are those of
-    // dz = dy where the activation was positive, and of dz * xhat
-    const float* bn_mean;        // this column group's: mean, rstd (bn_c floats further on), gamma, beta
-    const float* bn_gamma;
-    const float* bn_beta;
-    int bn_c;
-};
-
-// The residuals of four row steps, beginning with step b.
-__device__ __forceinline__ void emit_residuals(const EmitArgs& a, int ro, int lane, int lsh, int b, float4* e)
-{
-    const int cq = lane & ((1 << lsh) - 1), r = (lane >> lsh) + ((32 >> lsh) * b);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int so = __shfl_sync(0xffffffffu, ro, r + (32 >> lsh) * i);
-        // (not the read-only path: the preceding kernel may have written it)
-        e[i] = __ldcg(reinterpret_cast<const float4*>(a.extra + (so >= 0 ? so + 4 * cq : 0)));
-    }
-}
-
-// 1 << lsh lanes hold a row's 16-byte pieces; ro is this lane's row offset or -1.  Loads, shared-memory reads and stores are
-// batched by kind, so that a batch's latencies overlap; there is ONE copy of this code for all widths and forms, since a
-// launch of a few microseconds runs it once or twice and would wait for its instructions otherwise (the kernel had grown to
-// 200 KB with specialised copies: 4000-8000 clocks for the first tile of a launch).
-// Moments are taken about a value of the column: sums of x and x*x themselves would cancel for a channel whose mean is large
-// against its spread.
-template <bool BNB>
-__device__ __forceinline__ void emit_rows(const EmitArgs& a, int ro, int fill, int lane, int lsh, bool have_shift, float4* e)
-{
-    const int cq = lane & ((1 << lsh) - 1), rq = lane >> lsh, rstep = 32 >> lsh, steps = 1 << lsh;
-    const unsigned int who = __ballot_sync(0xffffffffu, ro >= 0);        // lane = row here
-    float4 k = make_float4(0.f, 0.f, 0.f, 0.f), sd = k, sq = k;
-    const bool moments = a.moments != nullptr && who != 0u;
-    float4 rs = k, g = k, bt = k;
-    if (BNB) {
-        // (statistics are results of the step: not the read-only path)
-        k = __ldcg(reinterpret_cast<const float4*>(a.bn_mean + 4 * cq)); rs = __ldcg(reinterpret_cast<const float4*>(a.bn_mean + a.bn_c + 4 * cq));
-        g = __ldg(reinterpret_cast<const float4*>(a.bn_gamma + 4 * cq)); bt = __ldg(reinterpret_cast<const float4*>(a.bn_beta + 4 * cq));
-    } else if (moments) {
-        if (have_shift) k = *reinterpret_cast<const float4*>(a.moments + 4 * cq);
-        else {
-            const int r0 = __ffs(who) - 1, so = __shfl_sync(0xffffffffu, ro, r0);
-            k = a.patch[r0 * 8 + (cq ^ (r0 & 7))];
-            if (a.extra) k = add4(k, __ldcg(reinterpret_cast<const float4*>(a.extra + so + 4 * cq)));
-        }
-    }
-#pragma unroll 1
-    for (int b = 0; b < steps; b += 4) {
-        int so[4];
-        float4 v[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int r = rq + rstep * (b + i);
-            so[i] = __shfl_sync(0xffffffffu, ro, r);
-            v[i] = a.patch[r * 8 + (cq ^ (r & 7))];
-        }
-        if (BNB) {
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const bool real = so[i] >= 0;
-                const float4 xh = mul4(sub4(e[i], k), rs), z = fma4(g, xh, bt);
-                const float4 d = make_float4(real && z.x > 0.f ? v[i].x : 0.f, real && z.y > 0.f ? v[i].y : 0.f, real && z.z > 0.f ? v[i].z : 0.f,
-                                             real && z.w > 0.f ? v[i].w : 0.f);
-                sd = add4(sd, d);
-                sq = fma4(d, xh, sq);
-            }
-            if (b + 4 < steps) emit_residuals(a, ro, lane, lsh, b + 4, e);
-        } else if (a.extra) {
-#pragma unroll
-            for (int i = 0; i < 4; ++i) v[i] = add4(v[i], e[i]);
-            if (b + 4 < steps) emit_residuals(a, ro, lane, lsh, b + 4, e);
-        }
-        float* out = a.out + 4 * cq;
-        if (a.accumulate) {
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-                if (so[i] >= 0) v[i] = add4(v[i], __ldcg(reinterpret_cast<const float4*>(out + so[i])));
-        }
-        if (a.ok) {
-#pragma unroll
-            for (int i = 0; i < 4; ++i) if (so[i] >= 0) *reinterpret_cast<float4*>(out + so[i]) = v[i];
-        }
-        if (moments && !BNB) {
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const float4 d = sub4(so[i] >= 0 ? v[i] : k, k);
-                sd = add4(sd, d);
-                sq = fma4(d, d, sq);
-            }
-        }
-    }
-    if (moments) {
-        // the lanes that share a column, then one lane per four columns adds to the block's sums
-#pragma unroll 1
-        for (int o = 16; o >= steps; o >>= 1) { sd = lane_sum(sd, o); sq = lane_sum(sq, o); }
-        if (lane < steps) {
-            float4 *pk = reinterpret_cast<float4*>(a.moments + 4 * cq), *pd = reinterpret_cast<float4*>(a.moments + a.mom_pitch + 4 * cq),
-                   *pq = reinterpret_cast<float4*>(a.moments + 2 * a.mom_pitch + 4 * cq);
-            if (have_shift) { *pd = add4(*pd, sd); *pq = add4(*pq, sq); }
-            else { *pk = k; *pd = sd; *pq = sq; }
-        }
-    }
-    if (a.zero_fill == 2) {
-        // strided data gradient: the positions between the samples receive no contribution
-        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 1
-        for (int i = 0; i < steps; ++i) {
-            const int so = __shfl_sync(0xffffffffu, ro, rq + rstep * i), f = __shfl_sync(0xffffffffu, fill, rq + rstep * i);
-            if (so < 0 || !a.ok) continue;
-            float* out = a.out + so + 4 * cq;
-            if (f & 1) *reinterpret_cast<float4*>(out + a.dense_w) = zero;
-            if (f & 2) *reinterpret_cast<float4*>(out + a.dense_h) = zero;
-            if (f & 4) *reinterpret_cast<float4*>(out + a.dense_h + a.dense_w) = zero;
-        }
-    }
-    __syncwarp();
-}
-
-// The MMA issuer (one thread).  RESIDENT: the weights of all chunks and taps stand in shared memory; otherwise a ring.
+// The MMA issuer (one thread).
 // KIND 0: one pass; 1: hi*hi and hi*lo from one MMA over [B_hi; B_lo]; 2: three MMAs.  Everything that does not change is
 // taken out of the loops and nothing in the tap loop waits or branches on loaded values: with the modes told apart inside it
 // an MMA took 115 clocks to issue, against 40 (N = 32) the tensor core needs.
 struct MmaEnv {
     volatile int* abort_flag;
     uint32_t smem_base, tmem_base, a_full, a_empty, b_full, b_empty, acc_full, acc_empty;
-    int m_first, u_first, u_count;
     int *a_used, *b_used;
-    bool drain;                  // wait until every barrier has seen its last arrival (they are used again)
 };
+// (Only the low words of the descriptors ever change.)
+__device__ __forceinline__ uint64_t desc_at(uint32_t lo, uint32_t hi) { uint64_t r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(lo), "r"(hi)); return r; }
 template <int KIND>
-__device__ __forceinline__ void issue_tile(uint32_t acc, uint64_t a, uint64_t b, uint64_t b_half, uint32_t idesc, uint32_t idesc2, uint32_t keep)
+__device__ __forceinline__ void issue_tile(uint32_t acc, uint32_t a, uint32_t a_hi, uint32_t b, uint32_t b_hi, uint32_t b_half, uint32_t idesc, uint32_t idesc2, uint32_t keep)
 {
     // (a: value or hi part, +4: lo part; +2: the chunk's second K step)
+    auto A = [&](uint32_t d) { return desc_at(a + d, a_hi); };
+    auto B = [&](uint32_t d) { return desc_at(b + d, b_hi); };
     if (KIND == 0) {
-        umma_tf32(acc, a, b, idesc, keep);
-        umma_tf32(acc, a + 2, b + 2, idesc, 1u);
+        umma_tf32(acc, A(0), B(0), idesc, keep);
+        umma_tf32(acc, A(2), B(2), idesc, 1u);
     } else if (KIND == 1) {
-        umma_tf32(acc, a, b, idesc2, keep);
-        umma_tf32(acc, a + 4, b, idesc, 1u);
-        umma_tf32(acc, a + 2, b + 2, idesc2, 1u);
-        umma_tf32(acc, a + 6, b + 2, idesc, 1u);
+        umma_tf32(acc, A(0), B(0), idesc2, keep);
+        umma_tf32(acc, A(4), B(0), idesc, 1u);
+        umma_tf32(acc, A(2), B(2), idesc2, 1u);
+        umma_tf32(acc, A(6), B(2), idesc, 1u);
     } else {
-        const uint64_t bl = b + b_half;
-        umma_tf32(acc, a, b, idesc, keep);
-        umma_tf32(acc, a + 4, b, idesc, 1u);
-        umma_tf32(acc, a, bl, idesc, 1u);
-        umma_tf32(acc, a + 2, b + 2, idesc, 1u);
-        umma_tf32(acc, a + 6, b + 2, idesc, 1u);
-        umma_tf32(acc, a + 2, bl + 2, idesc, 1u);
+        umma_tf32(acc, A(0), B(0), idesc, keep);
+        umma_tf32(acc, A(4), B(0), idesc, 1u);
+        umma_tf32(acc, A(0), B(b_half), idesc, 1u);
+        umma_tf32(acc, A(2), B(2), idesc, 1u);
+        umma_tf32(acc, A(6), B(2), idesc, 1u);
+        umma_tf32(acc, A(2), B(b_half + 2), idesc, 1u);
     }
 }
-template <bool RESIDENT, int KIND>
-__device__ __forceinline__ void mma_role(const PipeScalars& p, const MmaEnv& e)
+// WINDOW: 3 or 1.  What one MMA of 16 columns costs is 40 clocks; every branch between two of them in this one-thread code about 50 more.
+template <bool RESIDENT, int KIND, int WINDOW, bool CELL>
+__device__ __forceinline__ void mma_role(const PipeScalars& p, const MmaEnv& e, UnitWalk u)
 {
-    const uint64_t a_desc = smem_desc(0, 16, 1024, 128), b_desc = smem_desc(0, 16, 512, 64);
+    const uint64_t a_desc = smem_desc(e.smem_base, 16, 1024, 128), b_desc = smem_desc(e.smem_base + p.off_b, 16, 512, 64);
+    const uint32_t a_hi = (uint32_t)(a_desc >> 32), b_hi = (uint32_t)(b_desc >> 32), a_first = (uint32_t)a_desc, b_first = (uint32_t)b_desc;
     const uint32_t idesc = p.idesc, idesc2 = p.idesc2, acc_cols = p.acc_cols, a_step = p.a_stage_bytes >> 4, b_step = p.b_stage_bytes >> 4, b_tap = p.b_tap_bytes >> 4;
-    const uint64_t b_half = ((uint32_t)p.n_chunk * 64u) >> 4;
-    const int taps = p.taps, group = RESIDENT ? p.taps : p.b_taps, R = p.R, a_stages = p.a_stages, b_stages = p.b_stages, acc_bufs = p.acc_bufs, T = p.T;
-    const uint64_t row_step = (uint64_t)((p.Wp - (R - 1)) * 8);      // from a window row's last tap to the next row's first
-    const uint64_t a_first = a_desc | (uint64_t)(e.smem_base >> 4), b_first = b_desc | (uint64_t)((e.smem_base + p.off_b) >> 4);
+    const uint32_t b_half = ((uint32_t)p.n_chunk * 64u) >> 4;
+    const int a_stages = p.a_stages, b_stages = p.b_stages, acc_bufs = p.acc_bufs, T = p.T;
+    const bool by_tap = !RESIDENT && WINDOW > 1 && p.b_taps == 1;    // a stage of the weight ring is one tap, not a window row
+    const uint32_t next_row = (uint32_t)p.Wp * 8u;                   // from a window row to the next
     int s = 0, bs = 0, buf = 0, b_it = 0, a_it = 0;
     uint32_t apar = 0, bpar = 0, cpar = 1u;
     if (RESIDENT) {
@@ -467,38 +376,37 @@ __device__ __forceinline__ void mma_role(const PipeScalars& p, const MmaEnv& e)
         if (!mbar_wait(e.b_full, 0, e.abort_flag)) { report(p.status, 22); return; }
     }
 #pragma unroll 1
-    for (UnitWalk u(p, e.m_first, e.u_first, e.u_count); u.left > 0; u.next(p)) {
+    for (; u.left > 0; u.next(p)) {
         const int nt = u.tiles(p), kb = u.kb(p), ke = u.ke(p);
-        const uint64_t lead = (uint64_t)(span_of(p, u).lead * 8);
+        const uint32_t skipped = p.flat ? 0u : (uint32_t)(span_of(p, u).lead * 8);
         if (!mbar_wait(e.acc_empty + 8 * buf, cpar, e.abort_flag)) { report(p.status, 23); return; }
         tc_fence_after();
         const uint32_t acc0 = e.tmem_base + (uint32_t)(buf * T) * acc_cols;
         uint32_t keep = 0u;
+        uint32_t b = b_first + (uint32_t)(kb * WINDOW * WINDOW) * b_tap;      // RESIDENT: the taps of all chunks stand in a row
 #pragma unroll 1
         for (int c = kb; c < ke; ++c) {
             if (!mbar_wait(e.a_full + 8 * s, apar, e.abort_flag)) { report(p.status, 24); return; }
-            uint64_t a = a_first + (uint64_t)((uint32_t)s * a_step) + lead;
-            uint64_t b = RESIDENT ? b_first + (uint64_t)((uint32_t)(c * taps) * b_tap) : 0;
-            int sx = 0;
+            uint32_t row = a_first + (uint32_t)s * a_step + skipped;
 #pragma unroll 1
-            for (int left = taps; left > 0; left -= group) {
-                if (!RESIDENT) {
-                    if (!mbar_wait(e.b_full + 8 * bs, bpar, e.abort_flag)) { report(p.status, 25); *e.b_used = b_it; *e.a_used = a_it; return; }
-                    b = b_first + (uint64_t)((uint32_t)bs * b_step);
-                }
+            for (int r = 0; r < WINDOW; ++r, row += next_row) {
+#pragma unroll
+                for (int x = 0; x < WINDOW; ++x) {
+                    if (!RESIDENT && (by_tap || x == 0)) {
+                        if (!mbar_wait(e.b_full + 8 * bs, bpar, e.abort_flag)) { report(p.status, 25); *e.b_used = b_it; *e.a_used = a_it; return; }
+                        b = b_first + (uint32_t)bs * b_step;
+                    }
+                    issue_tile<KIND>(acc0, row + 8u * x, a_hi, b, b_hi, b_half, idesc, idesc2, keep);
+                    if (T > 1)
 #pragma unroll 1
-                for (int k = 0; k < group; ++k) {
-#pragma unroll 1
-                    for (int t = 0; t < nt; ++t) issue_tile<KIND>(acc0 + (uint32_t)t * acc_cols, a + (uint64_t)(t * 1024), b, b_half, idesc, idesc2, keep);
+                        for (int t = 1; t < nt; ++t) issue_tile<KIND>(acc0 + (uint32_t)t * acc_cols, row + 8u * x + (uint32_t)(t * 1024), a_hi, b, b_hi, b_half, idesc, idesc2, keep);
                     keep = 1u;
                     b += b_tap;
-                    a += 8;
-                    if (++sx == R) { sx = 0; a += row_step - 8; }
-                }
-                if (!RESIDENT) {
-                    umma_commit(e.b_empty + 8 * bs);
-                    ++b_it;
-                    if (++bs == b_stages) { bs = 0; bpar ^= 1u; }
+                    if (!RESIDENT && (by_tap || x == WINDOW - 1)) {
+                        umma_commit(e.b_empty + 8 * bs);
+                        ++b_it;
+                        if (++bs == b_stages) { bs = 0; bpar ^= 1u; }
+                    }
                 }
             }
             umma_commit(e.a_empty + 8 * s);
@@ -509,12 +417,25 @@ __device__ __forceinline__ void mma_role(const PipeScalars& p, const MmaEnv& e)
         if (++buf == acc_bufs) { buf = 0; cpar ^= 1u; }
         *e.b_used = b_it; *e.a_used = a_it;
     }
-    if (e.drain) {
+    if (CELL) {                  // wait until every barrier has seen its last arrival: they are used again
 #pragma unroll 1
         for (int i = 0; i < a_stages && i < a_it; ++i) mbar_wait(e.a_empty + 8 * i, (uint32_t)((a_it - 1 - i) / a_stages) & 1u, e.abort_flag);
         if (!RESIDENT)
 #pragma unroll 1
             for (int i = 0; i < b_stages && i < b_it; ++i) mbar_wait(e.b_empty + 8 * i, (uint32_t)((b_it - 1 - i) / b_stages) & 1u, e.abort_flag);
+    }
+}
+template <int WINDOW, bool CELL>
+__device__ __forceinline__ void mma_roles(const PipeScalars& p, const MmaEnv& e, const UnitWalk& u)
+{
+    if (p.b_resident) {
+        if (!p.three) mma_role<true, 0, WINDOW, CELL>(p, e, u);
+        else if (p.stacked) mma_role<true, 1, WINDOW, CELL>(p, e, u);
+        else mma_role<true, 2, WINDOW, CELL>(p, e, u);
+    } else {
+        if (!p.three) mma_role<false, 0, WINDOW, CELL>(p, e, u);
+        else if (p.stacked) mma_role<false, 1, WINDOW, CELL>(p, e, u);
+        else mma_role<false, 2, WINDOW, CELL>(p, e, u);
     }
 }
 
@@ -533,24 +454,392 @@ __device__ __forceinline__ void pipe_init_barriers(const PipeScalars& p, PipeSha
 #pragma unroll
     for (int s = lane; s < 3 * kMaxA + 2 * kMaxB + 4; s += 32) {
         const bool full = s >= kMaxA && s < 2 * kMaxA, acc_empty = s >= 3 * kMaxA + 2 && s < 3 * kMaxA + 4;
-        mbar_init(bar + 8 * s, full ? split : (acc_empty ? emit : 1u));
+        mbar_init(bar + 8 * s, full ? split : (acc_empty ? emit : (s < kMaxA && p.flat ? 32u : 1u)));
     }
     if (lane == 0) { sh.abort_flag = 0; sh.b_issued = 0; sh.b_used = 0; sh.a_issued = 0; sh.a_used = 0; }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+}
+
+// ---- write-out: tensor memory -> registers -> global memory ----
+// A 16x256b load gives four lanes of a warp a row of the accumulator, two columns of every eight each.  The weights' rows are copied
+// in an order (the dimensions of their tensor map) that makes a lane's columns of a group of 4 W output channels W consecutive
+// ones: the four lanes have a row of the group between them, residuals are read the same way, and a lane keeps the sums of its
+// own channels from row to row, with no transposition and no exchange between lanes until a block of units ends.
+// A warp's 32 rows x 32 channels with residual and moments took 3600 clocks through a patch of shared memory, 300 instructions with
+// their latencies; now 2000 without and up to 4300 with a residual, which is then the memory's rate (18 bytes a clock and SM).
+//
+// What a launch of a few microseconds pays here is the first execution of every instruction: 100-150 clocks per 128 bytes of
+// code, a first patch took 8600 clocks against 2400 of the following ones.  So there is one loop over patches (32 rows x
+// one group of channels), every part of which stands in the code once, and its first, dry round - no rows, nothing waited
+// for, nothing stored - runs ahead of the first accumulator.  Everything together: ResNet-110 5.96 -> 5.62 ms, ResNet-11 0.327 -> 0.299.
+template <int W, bool FLAT, bool BNB, bool CELL>
+__device__ __forceinline__ void write_out(const PipeScalars& p, PipeShared& sh, uint8_t* smem, const uint32_t tmem_base,
+                                          const uint32_t acc_full, const uint32_t acc_empty, const UnitWalk& u0, const int slice)
+{
+    constexpr int kCols = 4 * W, H = 2 * W;           // channels of a group; values a lane holds of 16 rows
+    const int warp = warp_index(), lane = threadIdx.x & 31;
+    const int tid = threadIdx.x - 32 * (kFirstSplit + kSplitWarps), ew = warp - kFirstSplit - kSplitWarps;
+    const int quad = warp & 3, half = ew >> 2;        // a warp reads the 32 lanes of its quadrant; two warps share one
+    const int q = lane & 3, r8 = lane >> 2;           // this lane's quarter of a row; its rows are r8 + 8 i
+    const int n_chunk = p.n_chunk, groups = n_chunk / kCols, T = p.T, C_out = p.c_out, ksplit = p.ksplit, co0 = slice * n_chunk;
+    const bool stacked = p.stacked != 0, stats = p.st_partials != nullptr;
+    // Two sets of four warps.  Where there is one group of channels they take alternate units (with two accumulator sets) or
+    // alternate tiles of a unit; otherwise alternate groups.
+    const bool alternate = p.epi_alternate != 0, whole = groups == 1;
+    const int g_first = whole ? 0 : half, g_step = whole ? 1 : 2, t_first = whole && !alternate ? half : 0, t_step = whole && !alternate ? 2 : 1;
+    const int parts = whole ? 8 : 4;
+    int part = whole ? ew : quad;
+    float4* const slots = reinterpret_cast<float4*>(smem + p.off_slots + (uint32_t)ew * p.slot_bytes);      // the lanes' sums of the block so far, W / 2 float4 a lane and group
+    // residuals of two times 16 rows; 8 (or 4) lanes copy a row's line (piece l % W of row l / W), so that no sector is fetched twice
+    uint8_t* const ring = smem + p.off_ring + ew * (W * 512);
+    const int copy_row = lane / W, copy_piece = lane % W, copy_step = 32 / W;
+    float* const bn_tab = reinterpret_cast<float*>(smem + p.off_bnb) + ew * 256;    // BNB: mean, rstd, gamma, beta of this warp's groups
+    float* const mom0 = reinterpret_cast<float*>(smem + p.off_stat);                // the warps' moments of a block, twice: those of the block before may still be read
+    const int mom_size = parts * (3 * n_chunk + 1);
+    const float* const addend = BNB ? p.bn_x : p.extra;
+    const size_t sk_tile = (size_t)kTileM * n_chunk;
+    int bn_m = -1, buf = alternate ? half : 0, flip = 0, count = 0;
+    uint32_t par = 0;
+    bool have = false, ok = true, finish = true, dry = true;
+    // blocks of units: the current one's micro-batch, row of partial moments, the number of its first unit within the CTA's work
+    const int blocks = u0.left;
+    int bm = u0.m, br = u0.row, first_unit = 0;
+
+    // the patch under way and the one after it: unit, tile, group, offsets of this lane's four rows (-1: none), which of the
+    // warp's 32 there are, and, three bits a row, which neighbours of a strided data gradient's sample get zeros
+    UnitWalk u = u0, nu = u0;
+    if (alternate && half == 1) nu.next(p);
+    int t = 0, g = g_first, nt = t_first, ng = g_first;
+    int off[4], noff[4], fill = 0, nfill = 0;
+    unsigned int who = 0, nwho = 0;
+    int nrow = -1;                                    // offset of the next patch's row `lane`
+    bool first = false, nfirst = true;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) off[i] = noff[i] = -1;
+    bool place = true;
+#pragma unroll 1
+    while (true) {
+        const bool more = nu.left > 0;
+        if (place && more) {
+            // (a set that shares the tiles of a unit may find none left: no rows then)
+            const int pos0 = (nu.ul * T + nt) * kTileM + quad * 32;
+            const bool some = nt < nu.tiles(p);
+            if (FLAT) {
+                const int n = some ? p.pos_per_m - pos0 : 0;
+                nwho = n >= 32 ? 0xffffffffu : (n > 0 ? (1u << n) - 1u : 0u);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) noff[i] = r8 + 8 * i < n ? (pos0 + r8 + 8 * i) * C_out : -1;
+                nrow = lane < n ? (pos0 + lane) * C_out : -1;
+            } else {
+                const Pixel px = locate(p, pos0 + lane);
+                const int ro = some && px.own ? px.n * p.os_n + px.y * p.os_h + px.x * p.os_w : -1;
+                const bool right = 2 * px.x + 1 < p.out_w, below = 2 * px.y + 1 < p.out_h;
+                const int f = (right ? 1 : 0) | (below ? 2 : 0) | (right && below ? 4 : 0);
+                nwho = __ballot_sync(0xffffffffu, ro >= 0);
+                nrow = ro;
+                nfill = 0;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    noff[i] = __shfl_sync(0xffffffffu, ro, r8 + 8 * i);
+                    nfill |= __shfl_sync(0xffffffffu, f, r8 + 8 * i) << (3 * i);
+                }
+            }
+        }
+        if (!dry && first) {
+            ok = mbar_wait(acc_full + 8 * buf, par, &sh.abort_flag);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok && lane == 0) report(p.status, 27);
+            if (!CELL && p.pdl_late && nu.left <= 0) pdl_launch_dependents();
+            tc_fence_after();
+        }
+        const uint32_t acc0 = tmem_base + (uint32_t)(buf * T) * p.acc_cols + ((uint32_t)(quad * 32) << 16);
+        // 16 rows of a group, hi and lo products added
+        auto accumulator = [&](int at_t, int at_g, int h, float* v) {
+            const uint32_t at = acc0 + (uint32_t)at_t * p.acc_cols + (uint32_t)(kCols * at_g) + ((uint32_t)(16 * h) << 16);
+            tmem_ld_rows<W>(at, v);
+            if (stacked) {
+                float w[H];
+                tmem_ld_rows<W>(at + (uint32_t)n_chunk, w);
+                tmem_ld_wait();
+                add_to<H>(v, w);
+            } else {
+                tmem_ld_wait();
+            }
+        };
+        float* const sk_all = ksplit > 1 ? reinterpret_cast<float*>(p.sk_base + u.m * p.sk_ms + kSplitKTicketBytes) + ((size_t)u.ul * p.slices + slice) * ksplit * T * sk_tile : nullptr;
+        if (ksplit > 1 && !dry && first) {
+            // this CTA's partial sums; the CTA that takes the last ticket of the unit adds them in split order
+            unsigned int* ticket = reinterpret_cast<unsigned int*>(p.sk_base + u.m * p.sk_ms) + (size_t)u.ul * p.slices + slice;
+            float* mine = sk_all + u.z * T * sk_tile;
+#pragma unroll 1
+            for (int t1 = t_first; t1 < u.tiles(p); t1 += t_step)
+#pragma unroll 1
+                for (int g1 = g_first; g1 < groups; g1 += g_step)
+#pragma unroll 1
+                    for (int h = 0; h < 2; ++h) {
+                        float v[H];
+                        accumulator(t1, g1, h, v);
+                        float* d = mine + t1 * sk_tile + ((size_t)((2 * g1 + h) * 4 + quad) * 32 + lane) * H;
+                        if (ok) { store_vec<W>(d, v); store_vec<W>(d + W, v + W); }
+                    }
+            __threadfence();
+            epi_sync();
+            if (tid == 0) {
+                sh.last_of_unit = atomicAdd(ticket, 1u) == (unsigned int)ksplit - 1u;
+                if (sh.last_of_unit) *ticket = 0u;
+            }
+            epi_sync();
+            finish = sh.last_of_unit != 0;
+            if (finish) __threadfence();
+            else {
+                who = 0;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) off[i] = -1;
+            }
+        }
+        if (BNB && !dry && u.m != bn_m) {
+            // statistics and parameters of this warp's columns (statistics are results of the step: not the read-only path)
+            bn_m = u.m;
+            const float* st = p.bn_stats + (long long)u.m * 2 * C_out + co0;
+            __syncwarp();
+#pragma unroll 1
+            for (int g1 = g_first, gi = 0; g1 < groups; g1 += g_step, ++gi)
+                if (lane < 4 * W) {
+                    const int kind = lane / W;
+                    const float* from = kind < 2 ? st + kind * C_out : (kind == 2 ? p.bn_gamma : p.bn_beta) + co0;
+                    reinterpret_cast<float4*>(bn_tab + gi * 4 * kCols)[lane] = __ldcg(reinterpret_cast<const float4*>(from + kCols * g1) + lane % W);
+                }
+            __syncwarp();
+        }
+        const int gi = whole ? 0 : g >> 1;
+        if (g == g_first) count += __popc(who);
+        float* const sums = mom0 + flip * mom_size + part * 3 * n_chunk + kCols * g + W * q;      // k, then the block's results
+        float4* const slot = slots + gi * (W / 2) * 32 + lane;
+        float* const dst = p.out + (long long)u.m * p.out_ms + co0 + kCols * g + W * q;
+        const float* const src = addend + (long long)nu.m * p.out_ms + co0 + kCols * ng + 4 * copy_piece;
+        float k[W], sd[W], sq[W];
+        bool have_k = have;
+#pragma unroll
+        for (int j = 0; j < W; ++j) k[j] = sd[j] = sq[j] = 0.f;
+        if (stats && have) {
+            if (!BNB) read_vec<W>(sums, k);
+#pragma unroll
+            for (int j = 0; j < W; j += 4) { read_vec<4>(reinterpret_cast<const float*>(slot + 8 * j), sd + j); read_vec<4>(reinterpret_cast<const float*>(slot + 8 * (W + j)), sq + j); }
+        }
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h) {
+            const int o[2] = {h ? off[2] : off[0], h ? off[3] : off[1]};
+            float v[H];
+            if (ksplit > 1 && finish && !dry) {
+#pragma unroll
+                for (int j = 0; j < H; ++j) v[j] = 0.f;
+#pragma unroll 1
+                for (int z = 0; z < ksplit; ++z) {
+                    float w[H];
+                    load_vec<H>(sk_all + ((size_t)z * T + t) * sk_tile + ((size_t)((2 * g + h) * 4 + quad) * 32 + lane) * H, w);
+                    add_to<H>(v, w);
+                }
+            } else {
+                accumulator(t, g, h, v);
+            }
+            // in the order of the rows: tensor memory gives two columns of row 0, two of row 1, the next two of row 0, ...
+            float x[2][W], e[H];
+#pragma unroll
+            for (int j = 0; j < W; ++j) { x[0][j] = v[(j >> 1) * 4 + (j & 1)]; x[1][j] = v[(j >> 1) * 4 + 2 + (j & 1)]; }
+            if (addend) {
+                if (!dry) { cp_async_wait<1>(); __syncwarp(); }
+#pragma unroll
+                for (int r = 0; r < 2; ++r)
+#pragma unroll
+                    for (int j = 0; j < W; j += 4)
+                        read_vec<4>(reinterpret_cast<const float*>(ring + h * (W * 256) + (r8 + 8 * r) * (W * 16) + (((q * (W / 4) + j / 4) ^ (W == 8 ? r8 : 0)) << 4)), e + W * r + j);
+                if (!BNB) { add_to<W>(x[0], e); add_to<W>(x[1], e + W); }
+            }
+            if (dry && h == 0 && !CELL) pdl_wait();
+            if (addend) {
+                // the residual (BNB: the BN's input) of the next patch travels while this one is written out
+                __syncwarp();
+                if (more) {
+                    uint32_t to = smem_u32(ring + h * (W * 256)) + (uint32_t)(copy_row * (W * 16));
+#pragma unroll
+                    for (int i = 0; i < W / 2; ++i, to += (uint32_t)(copy_step * W * 16)) {
+                        const int r = copy_row + copy_step * i;
+                        const int no = __shfl_sync(0xffffffffu, nrow, 16 * h + r);
+                        cp_async16(to + (uint32_t)((copy_piece ^ (W == 8 ? r & 7 : 0)) << 4), src + (no >= 0 ? no : 0));
+                    }
+                }
+                cp_async_commit();
+            }
+            if (p.accumulate) {
+#pragma unroll
+                for (int r = 0; r < 2; ++r)
+                    if (o[r] >= 0) { float w[W]; load_vec<W>(dst + o[r], w); add_to<W>(x[r], w); }
+            }
+            if (BNB) {
+                const float* tab = bn_tab + gi * 4 * kCols + W * q;
+#pragma unroll
+                for (int j = 0; j < W; j += 4) {
+                    const float4 mu = *reinterpret_cast<const float4*>(tab + j), rs = *reinterpret_cast<const float4*>(tab + kCols + j),
+                                 ga = *reinterpret_cast<const float4*>(tab + 2 * kCols + j), be = *reinterpret_cast<const float4*>(tab + 3 * kCols + j);
+#pragma unroll
+                    for (int r = 0; r < 2; ++r) {
+                        const float* xe = e + W * r + j;
+                        const bool real = o[r] >= 0;
+                        const float4 xh = mul4(sub4(make_float4(xe[0], xe[1], xe[2], xe[3]), mu), rs), z = fma4(ga, xh, be);
+                        const float4 d = make_float4(real && z.x > 0.f ? x[r][j] : 0.f, real && z.y > 0.f ? x[r][j + 1] : 0.f,
+                                                     real && z.z > 0.f ? x[r][j + 2] : 0.f, real && z.w > 0.f ? x[r][j + 3] : 0.f);
+                        const float4 a = add4(make_float4(sd[j], sd[j + 1], sd[j + 2], sd[j + 3]), d),
+                                     b = fma4(d, xh, make_float4(sq[j], sq[j + 1], sq[j + 2], sq[j + 3]));
+                        sd[j] = a.x; sd[j + 1] = a.y; sd[j + 2] = a.z; sd[j + 3] = a.w;
+                        sq[j] = b.x; sq[j + 1] = b.y; sq[j + 2] = b.z; sq[j + 3] = b.w;
+                    }
+                }
+            } else if (stats) {
+                // moments are taken about a value of the column (the first one): sums of x and x * x themselves would cancel for
+                // a channel whose mean is large against its spread
+                if (!have_k && (((who >> (16 * h)) & 0xffffu) || dry)) {
+                    const int r0 = __ffs(who) - 1, from = (r0 & 7) * 4 + q;
+#pragma unroll
+                    for (int j = 0; j < W; ++j) k[j] = __shfl_sync(0xffffffffu, r0 & 8 ? x[1][j] : x[0][j], from);
+                    have_k = true;
+                    if (lane < 4)
+#pragma unroll
+                        for (int j = 0; j < W; j += 4) *reinterpret_cast<float4*>(sums + j) = make_float4(k[j], k[j + 1], k[j + 2], k[j + 3]);
+                }
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    const bool real = o[r] >= 0;
+#pragma unroll
+                    for (int j = 0; j < W; j += 2) {
+                        const uint64_t kk = pair(k[j], k[j + 1]), d = sub2(real ? pair(x[r][j], x[r][j + 1]) : kk, kk);
+                        unpair(add2(pair(sd[j], sd[j + 1]), d), sd[j], sd[j + 1]);
+                        unpair(fma2(d, d, pair(sq[j], sq[j + 1])), sq[j], sq[j + 1]);
+                    }
+                }
+            }
+#pragma unroll
+            for (int r = 0; r < 2; ++r)
+                if (o[r] >= 0 && ok) store_vec<W>(dst + o[r], x[r]);
+            if (!FLAT && p.zero_fill == 2) {
+                // strided data gradient: the positions between the samples receive no contribution
+                float zero[W];
+#pragma unroll
+                for (int j = 0; j < W; ++j) zero[j] = 0.f;
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    const int f = o[r] >= 0 && ok ? fill >> (3 * (2 * h + r)) : 0;
+                    if (f & 1) store_vec<W>(dst + o[r] + p.dense_w, zero);
+                    if (f & 2) store_vec<W>(dst + o[r] + p.dense_h, zero);
+                    if (f & 4) store_vec<W>(dst + o[r] + p.dense_h + p.dense_w, zero);
+                }
+            }
+        }
+        if (stats) {
+#pragma unroll
+            for (int j = 0; j < W; j += 4) {
+                slot[8 * j] = make_float4(sd[j], sd[j + 1], sd[j + 2], sd[j + 3]);
+                slot[8 * (W + j)] = make_float4(sq[j], sq[j + 1], sq[j + 2], sq[j + 3]);
+            }
+            __syncwarp();                             // k is read by the next patch, the sums by the lanes that add them up
+        }
+        if (nfirst && !dry) {
+            // the accumulator is read: the next unit's MMAs may have it
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(acc_empty + 8 * buf);
+            if (alternate) par ^= 1u;                 // (a set of warps always meets its own accumulator set)
+            else if (++buf == p.acc_bufs) { buf = 0; par ^= 1u; }
+        }
+        if (g + g_step >= groups && who) have = true;
+        // Ends of blocks between this patch and the next (alternating sets: also of blocks in which this set has no unit): the moments
+        // of the lanes, then the warps' parts, each about its own shift.
+        const int at_block = blocks - (more ? nu.left : 0);
+#pragma unroll 1
+        for (int b = dry ? -1 : blocks - u.left; stats && b < at_block; ++b) {
+            float* contrib = mom0 + flip * mom_size;
+            float* counts = contrib + (size_t)parts * 3 * n_chunk;
+            // a lane adds what eight lanes have of its column
+            const float* from = reinterpret_cast<const float*>(slots) + ((lane % W) >> 2) * 128 + (lane / W) * 4 + (lane & 3);
+#pragma unroll 1
+            for (int g1 = g_first; g1 < groups; g1 += g_step, from += W * 64) {
+                float sum = 0.f, sq1 = 0.f;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) { sum += from[16 * j]; sq1 += from[W * 32 + 16 * j]; }
+                float* to = contrib + part * 3 * n_chunk + kCols * g1 + lane;
+                if (lane < kCols) { to[n_chunk] = sum; to[2 * n_chunk] = sq1; }
+            }
+            if (lane == 0 && (whole || half == 0)) counts[part] = (float)count;
+            epi_sync();
+            if (tid < n_chunk) {
+                // parts about their own shifts k_w: sum and squares about the first one's,
+                //   sum (x - k0) = sum_w [d_w + n_w e],  sum (x - k0)^2 = sum_w [q_w + e (2 d_w + n_w e)],  e = k_w - k0
+                // (BNB: no shifts, the sums themselves)
+                float N = 0.f, k0 = 0.f, sum = 0.f, sq1 = 0.f;
+                const float* c3 = contrib + tid;
+#pragma unroll 1
+                for (int w = 0; w < parts; ++w, c3 += 3 * n_chunk) {
+                    const float cnt = counts[w];
+                    if (cnt == 0.f) continue;
+                    const float d = c3[n_chunk];
+                    if (N == 0.f && !BNB) k0 = c3[0];
+                    const float ek = BNB ? 0.f : c3[0] - k0;
+                    N += cnt;
+                    sum += fmaf(cnt, ek, d);
+                    sq1 += fmaf(ek, fmaf(cnt, ek, 2.f * d), c3[2 * n_chunk]);
+                }
+                const float dm = N > 0.f ? sum / N : 0.f, m2 = fmaxf(fmaf(-sum, dm, sq1), 0.f);
+                float* all = p.st_partials + (size_t)bm * partial_floats(p.blocks_per_m, C_out);
+                float* row = all + (size_t)br * 2 * C_out + co0 + tid;
+                if (ok && finish && b >= 0) {
+                    row[0] = BNB ? sum : k0 + dm; row[C_out] = BNB ? sq1 : m2;
+                    if (!BNB && tid == 0 && slice == 0) all[(size_t)p.blocks_per_m * 2 * C_out + br] = N;
+                }
+            }
+            flip ^= 1;
+            count = 0; have = false;
+            if (b >= 0 && ksplit == 1) {
+                const int start = br * p.unit_block, left = p.units_per_m - start;
+                first_unit += left < p.unit_block ? left : p.unit_block;
+                if (++br == p.blocks_per_m) { br = 0; ++bm; }
+                // (alternating sets: a block's first unit counts as part 0..3, whichever set's turn it is, so that its moments are added in
+                // the same order wherever in a CTA's work the block stands)
+                if (alternate) part = quad + 4 * (half ^ (first_unit & 1));
+            }
+        }
+        if (!more) break;
+        // the next patch is the current one, and what follows it
+        u = nu; t = nt < T ? nt : T - 1; g = ng; who = nwho; fill = nfill; first = nfirst;
+        if (first) finish = true;
+        if (ksplit > 1) { bm = u.m; br = u.ul; }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) off[i] = finish ? noff[i] : -1;
+        if (!finish) who = 0;
+        dry = false;
+        place = nfirst = false;
+        if ((ng += g_step) >= groups) {
+            ng = g_first; place = true;
+            if ((nt += t_step) >= nu.tiles(p)) {
+                nt = t_first; nfirst = true;
+                nu.next(p);
+                if (alternate && nu.left > 0) nu.next(p);
+            }
+        }
+    }
 }
 
 // The work of one CTA (number bid of nblk) of a launch: the barriers are initialised, tensor memory is allocated.
 // FLAT: the operand's positions and the output's pixels are the same consecutive rows (1x1 windows without a stride).
 // BNB: a data gradient that forms the sums of a BN+ReLU's backward.
 // CELL: inside the persistent cell kernel, which keeps its tensor memory and has no successor to trigger.
-template <bool BN_IN, bool FLAT, bool BNB, bool CELL>
+// W: channels of a row that a write-out lane has.
+template <bool BN_IN, bool FLAT, bool BNB, int W, bool CELL>
 __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars& p, PipeShared& sh, uint8_t* smem, const uint32_t tmem_base,
                                          const int m_first, const int m_count, const int bid, const int nblk)
 {
     const uint32_t smem_base = smem_u32(smem);
     const int warp = warp_index(), lane = threadIdx.x & 31;
     uint64_t* bars = sh.bars;
-    int &abort_flag = sh.abort_flag, &b_issued = sh.b_issued, &b_used = sh.b_used, &a_issued = sh.a_issued, &a_used = sh.a_used, &last_of_unit = sh.last_of_unit;
+    int &abort_flag = sh.abort_flag, &b_issued = sh.b_issued, &b_used = sh.b_used, &a_issued = sh.a_issued, &a_used = sh.a_used;
     const uint32_t a_raw = smem_u32(&bars[0]), a_full = smem_u32(&bars[kMaxA]), a_empty = smem_u32(&bars[2 * kMaxA]),
                    acc_full = smem_u32(&bars[3 * kMaxA]), acc_empty = smem_u32(&bars[3 * kMaxA + 2]), b_full = smem_u32(&bars[3 * kMaxA + 4]),
                    b_empty = smem_u32(&bars[3 * kMaxA + 4 + kMaxB]);
@@ -561,22 +850,51 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
     const int each = total / ctas, more = total - each * ctas;
     const int u_first = cta * each + (cta < more ? cta : more), u_count = each + (cta < more ? 1 : 0);
     const int co0 = slice * p.n_chunk;
+    const UnitWalk u0(p, m_first, u_first, u_count);
 
-    if (warp == 0) {
+    if (p.flat && (warp == 0 || warp == 3)) {
+        // ---- operand copies, consecutive pixels ----
+        // Two warps take alternate blocks, 16 bytes a lane straight to their place in the swizzled rows.  A tensor copy takes an SM 6.7
+        // clocks for every 64-byte row of its box (copies alone on all SMs: 9.6 bytes a clock and SM, 15 in rows of 128 bytes).
+        const int S = p.a_stages, C = p.c_in, row0 = lane >> 2, mine = warp == 0 ? 0 : 1;
+        const uint32_t at = smem_base + (uint32_t)row0 * 128u + (uint32_t)(((lane & 3) ^ row0) << 4);
+        int s = mine % S, it = 0;
+        uint32_t par = mine < S ? 1u : 0u;
+        bool live = true, waited = CELL;
+#pragma unroll 1
+        for (UnitWalk u = u0; u.left > 0 && live; u.next(p)) {
+            const int start = u.ul * p.T * kTileM, rows = u.tiles(p) * kTileM, valid = p.pos_per_m - start;
+            const float* const unit = p.in + (long long)u.m * p.in_ms + (long long)(start + row0) * C + 4 * (lane & 3);
+#pragma unroll 1
+            for (int c = u.kb(p), ce = u.ke(p); c < ce; ++c, ++it) {
+                if ((it & 1) != mine) continue;
+                live = __all_sync(0xffffffffu, mbar_wait(a_empty + 8 * s, par, &abort_flag));
+                if (!live) { if (lane == 0) report(p.status, 20); break; }
+                if (!waited) { pdl_wait(); waited = true; }
+                const float* src = unit + 16 * c;
+                uint32_t dst = at + (uint32_t)s * p.a_stage_bytes;
+#pragma unroll 4
+                for (int row = row0; row < rows; row += 8, src += 8 * C, dst += 1024u) cp_async16_zfill(dst, row < valid ? src : p.in, row < valid);
+                cp_async_arrive(a_raw + 8 * s);
+                s += 2;
+                if (s >= S) { s -= S; par ^= 1u; }
+            }
+        }
+        cp_async_wait<0>();                           // (also after a wait that gave up: nothing may land in shared memory that was given back)
+    } else if (warp == 0) {
         if (elect_one()) {
-            // ---- operand copies ----
-            if (!CELL) pdl_wait();
+            // ---- operand copies ---- (the first one's coordinates are worked out while the predecessor still runs)
             const int S = p.a_stages;
             int s = 0, it = 0;
             uint32_t par = 1u;
             bool live = true;
 #pragma unroll 1
-            for (UnitWalk u(p, m_first, u_first, u_count); u.left > 0 && live; u.next(p)) {
+            for (UnitWalk u = u0; u.left > 0 && live; u.next(p)) {
                 const Span sp = span_of(p, u);
                 const uint32_t tx = (uint32_t)sp.rows * 64u;
                 // first block: map, row within it
                 int img0 = 0, h0 = 0, strip0 = 0;
-                if (!p.flat) {
+                {
                     if (sp.block0 < 0) { img0 = -1; h0 = p.blocks_per_img + sp.block0; if (h0 < 0) h0 = 0; }
                     else { img0 = div_magic(sp.block0, p.blocks_per_img, p.magic_bpi); h0 = sp.block0 - img0 * p.blocks_per_img; }
                     if (p.strips > 1 && img0 >= 0) { const int n = div_magic(img0, p.strips, p.magic_strip); strip0 = img0 - n * p.strips; img0 = n; }
@@ -588,10 +906,8 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
                     const uint32_t bar = a_raw + 8 * s;
                     uint32_t dst = smem_base + (uint32_t)s * p.a_stage_bytes;
                     mbar_expect_tx(bar, tx);
-                    if (p.flat) {
-#pragma unroll 1
-                        for (int k = 0; k < sp.blocks; ++k, dst += kTileM * 128u) tma_load_2d(dst, &gp.tm_a, bar, 16 * c, first + (sp.block0 + k) * kTileM);
-                    } else {
+                    if (!CELL && it == 0) pdl_wait();
+                    {
                         int img = img0, h = h0, strip = strip0;
                         const uint32_t step = (uint32_t)p.box_pos * 128u;
 #pragma unroll 1
@@ -613,7 +929,7 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
             const uint32_t half = (uint32_t)p.n_chunk * 64u, tap_bytes = p.b_tap_bytes, dst0 = smem_base + p.off_b;
             const bool three = p.three != 0;
             const uint32_t tx = three ? 2u * half : half;
-            const int taps = p.taps, c_in = p.c_in;
+            const int taps = p.taps, c_in = p.c_in, block0 = p.wide ? co0 >> 5 : co0 >> 4;
             if (p.b_resident) {
                 const int n = p.n_chunks * taps;
                 mbar_expect_tx(b_full, tx * (uint32_t)n);
@@ -622,8 +938,8 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
                 for (int c = 0; c < p.n_chunks; ++c)
 #pragma unroll 1
                     for (int tap = 0; tap < taps; ++tap, dst += tap_bytes) {
-                        tma_load_2d(dst, &gp.tm_b, b_full, tap * c_in + 16 * c, co0);
-                        if (three) tma_load_2d(dst + half, &gp.tm_b_lo, b_full, tap * c_in + 16 * c, co0);
+                        tma_load_5d(dst, &gp.tm_b, b_full, tap * c_in + 16 * c, 0, 0, 0, block0);
+                        if (three) tma_load_5d(dst + half, &gp.tm_b_lo, b_full, tap * c_in + 16 * c, 0, 0, 0, block0);
                     }
                 b_issued = 1;
             } else {
@@ -631,7 +947,7 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
                 uint32_t par = 1u;
                 bool live = true;
 #pragma unroll 1
-                for (UnitWalk u(p, m_first, u_first, u_count); u.left > 0 && live; u.next(p))
+                for (UnitWalk u = u0; u.left > 0 && live; u.next(p))
 #pragma unroll 1
                     for (int c = u.kb(p), ce = u.ke(p); c < ce && live; ++c)
 #pragma unroll 1
@@ -642,8 +958,8 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
                             mbar_expect_tx(bar, tx * (uint32_t)p.b_taps);
 #pragma unroll 1
                             for (int e = tap + p.b_taps; tap < e; ++tap, dst += tap_bytes) {
-                                tma_load_2d(dst, &gp.tm_b, bar, tap * c_in + 16 * c, co0);
-                                if (three) tma_load_2d(dst + half, &gp.tm_b_lo, bar, tap * c_in + 16 * c, co0);
+                                tma_load_5d(dst, &gp.tm_b, bar, tap * c_in + 16 * c, 0, 0, 0, block0);
+                                if (three) tma_load_5d(dst + half, &gp.tm_b_lo, bar, tap * c_in + 16 * c, 0, 0, 0, block0);
                             }
                             if (++s == p.b_stages) { s = 0; par ^= 1u; }
                         }
@@ -653,16 +969,9 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
     } else if (warp == 2) {
         if (elect_one()) {
             // ---- MMAs ----
-            const MmaEnv env{&abort_flag, smem_base, tmem_base, a_full, a_empty, b_full, b_empty, acc_full, acc_empty, m_first, u_first, u_count, &a_used, &b_used, CELL};
-            if (p.b_resident) {
-                if (!p.three) mma_role<true, 0>(p, env);
-                else if (p.stacked) mma_role<true, 1>(p, env);
-                else mma_role<true, 2>(p, env);
-            } else {
-                if (!p.three) mma_role<false, 0>(p, env);
-                else if (p.stacked) mma_role<false, 1>(p, env);
-                else mma_role<false, 2>(p, env);
-            }
+            const MmaEnv env{&abort_flag, smem_base, tmem_base, a_full, a_empty, b_full, b_empty, acc_full, acc_empty, &a_used, &b_used};
+            if (FLAT || p.R == 1) mma_roles<1, CELL>(p, env, u0);
+            else mma_roles<3, CELL>(p, env, u0);
         }
     } else if (warp >= kFirstSplit && warp < kFirstSplit + kSplitWarps) {
         // ---- the operand: normalise, split ----
@@ -677,14 +986,12 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
         const int row_step = 8 * wpg;
         const int cph = lane & 3, r8 = ((lane >> 2) & 1) * 4 + (lane >> 3), row0 = gw * 8 + r8;
         const uint32_t at_hi = (uint32_t)row0 * 128u + (uint32_t)((cph ^ r8) << 4), at_lo = (uint32_t)row0 * 128u + (uint32_t)(((cph + 4) ^ r8) << 4);
-        const uint32_t byte_step = (uint32_t)row_step * 128u;
         const int S = p.a_stages, C = p.c_in, halo = p.halo;
         const bool three = p.three != 0;
         float* tab = reinterpret_cast<float*>(smem + p.off_bn);
         if (BN_IN) {
 #pragma unroll 1
             for (int i = tid; i < C; i += kSplitThreads) { tab[2 * C + i] = __ldg(p.bn_gamma + i); tab[3 * C + i] = __ldg(p.bn_beta + i); }
-            if (!CELL) pdl_wait();
         }
         // a step of row_step positions in maps, rows and columns of the padded grid
         const int dn = BN_IN && !FLAT ? row_step / p.img_pos : 0, drem = row_step - dn * p.img_pos;
@@ -694,37 +1001,42 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
         uint32_t par = 0;
         const bool store_y = BN_IN && slice == 0;
         bool ok = true;
+        UnitWalk cu = u0;
+        // The first round is a dry one (see write_out): no rows to merge, one row a thread, in the scratch of the merge.
+        bool dry = BN_IN;
 #pragma unroll 1
-        for (UnitWalk cu(p, m_first, u_first, u_count); cu.left > 0; cu.next(p)) {
-            const int kb = cu.kb(p), ke = cu.ke(p);
+        while (cu.left > 0) {
+            const int kb = cu.kb(p), ke = dry ? kb + ahead + 1 : cu.ke(p);
             const Span sp = span_of(p, cu);
-            const int own_lo = sp.lead + halo, own_hi = own_lo + cu.tiles(p) * kTileM, valid = p.pos_per_m - sp.pos0;
+            const int own_lo = sp.lead + halo, own_hi = own_lo + cu.tiles(p) * kTileM, valid = p.pos_per_m - sp.pos0, n_rows = dry ? 1 : sp.rows;
             if (BN_IN) {
-                if (cu.m != cur_m) {
-                    cur_m = cu.m;
+                if (dry || cu.m != cur_m) {
+                    if (!dry) cur_m = cu.m;
                     split_sync();                     // everybody is done with the table of the micro-batch before
-                    merge_moments<kSplitThreads>(p.bn_partials + (size_t)cur_m * partial_floats(p.bn_units, C), p.bn_units, C, p.bn_inv_rows, p.bn_eps, tab,
+                    merge_moments<kSplitThreads>(p.bn_partials + (size_t)cu.m * partial_floats(p.bn_units, C), dry ? 0 : p.bn_units, C, p.bn_inv_rows, p.bn_eps, tab,
                                   reinterpret_cast<float4*>(smem + p.off_red), tid);
                     split_sync();
                 }
-                if (slice == 0 && cu.ul == 0 && cu.z == 0)
+                if (!dry && slice == 0 && cu.ul == 0 && cu.z == 0)
 #pragma unroll 1
                     for (int i = tid; i < 2 * C; i += kSplitThreads) p.bn_stats[(size_t)cur_m * 2 * C + i] = tab[i];
             }
 #pragma unroll 1
             for (int c = kb + ahead; c < ke; c += groups) {
                 {
-                    ok = mbar_wait(a_raw + 8 * s, par, &abort_flag) && ok;
+                    if (!dry) ok = mbar_wait(a_raw + 8 * s, par, &abort_flag) && ok;
                     // (after a wait that gave up the warps run through the rest without waiting: they still have to meet at
                     // the named barriers)
                     if (!ok && lane == 0) report(p.status, 26);
-                    uint8_t* hi = smem + (uint32_t)s * p.a_stage_bytes + at_hi;
-                    uint8_t* lo = smem + (uint32_t)s * p.a_stage_bytes + at_lo;
+                    // (dry: every row step of the one batch at the same place, in the merge's scratch)
+                    uint8_t* const stage = smem + (dry ? p.off_red : (uint32_t)s * p.a_stage_bytes);
+                    uint8_t *hi = stage + (dry ? 16 * lane : at_hi), *lo = stage + (dry ? 16 * lane : at_lo);
+                    const uint32_t byte_step = dry ? 0u : (uint32_t)row_step * 128u;
                     if (BN_IN) {
                         const int ch = 16 * c + 4 * cph;
                         const float4 mu = *reinterpret_cast<const float4*>(tab + ch), rs = *reinterpret_cast<const float4*>(tab + C + ch);
                         const float4 g = *reinterpret_cast<const float4*>(tab + 2 * C + ch), b = *reinterpret_cast<const float4*>(tab + 3 * C + ch);
-                        float* ydst = p.bn_y + (long long)cur_m * p.in_ms + 16 * c + 4 * cph;
+                        float* ydst = p.bn_y + (long long)cu.m * p.in_ms + 16 * c + 4 * cph;
                         int yo = (sp.pos0 + row0) * C;                   // FLAT: offset of this thread's first row
                         int pn = 0, py = 0, px = 0;                      // otherwise its map, row and column
                         if (!FLAT) {
@@ -736,7 +1048,7 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
                         }
                         // four rows in flight; the block is allocated in whole batches, so the last one needs no bounds
 #pragma unroll 1
-                        for (int row = row0; row < sp.rows; row += kRowBatch * row_step, hi += kRowBatch * byte_step, lo += kRowBatch * byte_step) {
+                        for (int row = dry ? 0 : row0; row < n_rows; row += kRowBatch * row_step, hi += kRowBatch * byte_step, lo += kRowBatch * byte_step) {
                             float4 v[kRowBatch];
 #pragma unroll
                             for (int j = 0; j < kRowBatch; ++j) v[j] = *reinterpret_cast<const float4*>(hi + byte_step * j);
@@ -746,11 +1058,12 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
                             for (int j = 0; j < kRowBatch; ++j) {
                                 const int r = row + row_step * j;
                                 if (FLAT) {
-                                    inside[j] = own[j] = r < valid;
+                                    inside[j] = r < valid;
+                                    own[j] = inside[j] && !dry;
                                     off[j] = yo; yo += row_step * C;
                                 } else {
                                     inside[j] = px < p.W && py < p.Hv && pn >= 0 && r < valid;
-                                    own[j] = inside[j] && r >= own_lo && r < own_hi;
+                                    own[j] = inside[j] && r >= own_lo && r < own_hi && !dry;
                                     off[j] = pn * p.in_sn + py * p.in_sh + px * p.in_sw;
                                     px += dx; py += dy; pn += dn;
                                     if (px >= p.Wp) { px -= p.Wp; ++py; }
@@ -775,7 +1088,7 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
                         }
                     } else if (three) {
 #pragma unroll 1
-                        for (int row = row0; row < sp.rows; row += kRowBatch * row_step, hi += kRowBatch * byte_step, lo += kRowBatch * byte_step) {
+                        for (int row = dry ? 0 : row0; row < n_rows; row += kRowBatch * row_step, hi += kRowBatch * byte_step, lo += kRowBatch * byte_step) {
                             float4 v[kRowBatch];
 #pragma unroll
                             for (int j = 0; j < kRowBatch; ++j) v[j] = *reinterpret_cast<const float4*>(hi + byte_step * j);
@@ -787,207 +1100,23 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
                     }
                     fence_async_smem();               // generic-proxy writes -> tensor-core reads
                     __syncwarp();
+                    if (dry) break;
                     if (lane == 0) mbar_arrive(a_full + 8 * s);
                 }
                 s += groups;
                 if (s >= S) { s -= S; par ^= 1u; }
                 ahead += groups;
             }
+            if (dry) {
+                dry = false;
+                if (!CELL) pdl_wait();
+                continue;
+            }
             ahead -= ke - kb;
+            cu.next(p);
         }
     } else if (warp >= kFirstSplit + kSplitWarps) {
-        // ---- write-out: tensor memory -> registers -> a 32 x 32 patch of shared memory -> global memory ----
-        // A TMEM lane is a position, so stores straight from the registers touch 32 lines per instruction (measured: half a
-        // sector per clock and SM); through a warp's own patch eight lanes write a row's 128 bytes, and a thread that keeps
-        // four columns forms their moments without crossing lanes.
-        const int tid = threadIdx.x - 32 * (kFirstSplit + kSplitWarps), ew = warp - kFirstSplit - kSplitWarps;
-        const int quad = warp & 3, half = ew >> 2;    // a warp reads the 32 lanes of its quadrant; two warps share one
-        const int n_chunk = p.n_chunk, groups = (n_chunk + 31) >> 5, T = p.T, C_out = p.c_out, ksplit = p.ksplit;
-        const bool stacked = p.stacked != 0, stats = p.st_partials != nullptr;
-        // Two sets of four warps.  With two accumulator sets and at most 64 channels each takes every other unit, so that the
-        // latencies of one unit's write-out run beside the other's; otherwise they share a unit: alternate groups of 32
-        // channels, or alternate tiles where there is one group.
-        const bool alternate = p.epi_alternate != 0, by_tile = !alternate && groups == 1, whole = alternate || by_tile;
-        const int g_first = whole ? 0 : half, g_step = whole ? 1 : 2, t_first = by_tile ? half : 0, t_step = by_tile ? 2 : 1;
-        // (alternating sets: a block's first unit always counts as part 0..3, whichever set's turn it is, so that its moments are
-        // added in the same order wherever in a CTA's work the block stands)
-        const int parts = whole ? 8 : 4;
-        int part = whole ? ew : quad;
-        int turn = 0;
-        float4* patch = reinterpret_cast<float4*>(smem + p.off_stage) + ew * 256;
-        if (!CELL) pdl_wait();
-        int buf = alternate ? half : 0, flip = 0;
-        uint32_t par = 0;
-        // the warps' moments of the block so far, twice: those of the block before may still be read
-        float* const mom0 = reinterpret_cast<float*>(smem + p.off_stat);
-        const int mom_size = parts * (3 * n_chunk + 1);
-        bool have = false;
-        int count = 0;
-#pragma unroll 1
-        for (UnitWalk u(p, m_first, u_first, u_count); u.left > 0; u.next(p)) {
-            bool finish = true, ok = true;
-            if (!alternate || turn == half) {
-            const int nt = u.tiles(p);
-            float* out = p.out + (long long)u.m * p.out_ms + co0;
-            const float* addend = BNB ? p.bn_x : p.extra;
-            const float* extra = addend ? addend + (long long)u.m * p.out_ms + co0 : nullptr;
-            const float* bnb = BNB ? p.bn_stats + (long long)u.m * 2 * C_out + co0 : nullptr;
-            EmitArgs ea{out, extra, patch, nullptr, n_chunk, p.accumulate != 0, true, p.zero_fill, p.dense_h, p.dense_w, nullptr, nullptr, nullptr, C_out};
-            // this lane's row of a tile, and which neighbours of a strided data gradient's sample get zeros
-            int ro = -1, fill = 0;
-            auto place = [&](int t) {
-                const int pos = (u.ul * T + t) * kTileM + quad * 32 + lane;
-                if (FLAT) { ro = pos < p.pos_per_m ? pos * C_out : -1; return; }
-                const Pixel px = locate(p, pos);
-                ro = px.own ? px.n * p.os_n + px.y * p.os_h + px.x * p.os_w : -1;
-                const bool right = 2 * px.x + 1 < p.out_w, below = 2 * px.y + 1 < p.out_h;
-                fill = (right ? 1 : 0) | (below ? 2 : 0) | (right && below ? 4 : 0);
-            };
-            const uint32_t acc0 = tmem_base + (uint32_t)(buf * T) * p.acc_cols + ((uint32_t)(quad * 32) << 16);
-            const size_t sk_tile = (size_t)kTileM * n_chunk;
-            const float* sk_all = nullptr;
-            // the first residuals travel while the accumulator is formed
-            float4 e[4];
-            place(t_first);
-            if (extra && t_first < nt) { ea.extra = extra + 32 * g_first; emit_residuals(ea, ro, lane, n_chunk - 32 * g_first >= 32 ? 3 : 2, 0, e); }
-            ok = mbar_wait(acc_full + 8 * buf, par, &abort_flag);
-            ok = __all_sync(0xffffffffu, ok);
-            if (!ok && lane == 0) report(p.status, 27);
-            if (!CELL && p.pdl_late && u.last(p)) pdl_launch_dependents();
-            tc_fence_after();
-            // 16 columns of this lane's row, hi and lo products added
-            auto accumulator = [&](int t, int col, float* v) {
-                const uint32_t at = acc0 + (uint32_t)t * p.acc_cols + (uint32_t)col;
-                tmem_ld16_nowait(at, v);
-                if (stacked) {
-                    float w[16];
-                    tmem_ld16_nowait(at + (uint32_t)n_chunk, w);
-                    tmem_ld_wait();
-#pragma unroll
-                    for (int j = 0; j < 16; j += 2) unpair(add2(pair(v[j], v[j + 1]), pair(w[j], w[j + 1])), v[j], v[j + 1]);
-                } else {
-                    tmem_ld_wait();
-                }
-            };
-            if (ksplit > 1) {
-                // this CTA's partial sums; the CTA that takes the last ticket of the unit adds them in split order
-                const size_t key = (size_t)u.ul * p.slices + slice;
-                char* base = p.sk_base + u.m * p.sk_ms;
-                unsigned int* ticket = reinterpret_cast<unsigned int*>(base) + key;
-                float* partials = reinterpret_cast<float*>(base + kSplitKTicketBytes);
-                sk_all = partials + key * ksplit * T * sk_tile;
-                float* mine = partials + (key * ksplit + u.z) * T * sk_tile;
-#pragma unroll 1
-                for (int t = t_first; t < nt; t += t_step)
-#pragma unroll 1
-                    for (int g = g_first; g < groups; g += g_step)
-#pragma unroll 1
-                        for (int h = 2 * g; h < 2 * g + 2 && 16 * h < n_chunk; ++h) {
-                            float v[16];
-                            accumulator(t, 16 * h, v);
-                            if (ok) store16(mine + t * sk_tile + ((size_t)h * kTileM + quad * 32 + lane) * 16, v);
-                        }
-                __threadfence();
-                epi_sync();
-                if (tid == 0) {
-                    last_of_unit = atomicAdd(ticket, 1u) == (unsigned int)ksplit - 1u;
-                    if (last_of_unit) *ticket = 0u;
-                }
-                epi_sync();
-                finish = last_of_unit != 0;
-                if (finish) __threadfence();
-            }
-            ea.ok = ok;
-#pragma unroll 1
-            for (int t = t_first; finish && t < nt; t += t_step) {
-                if (t > t_first) place(t);
-                const int rows = __popc(__ballot_sync(0xffffffffu, ro >= 0));
-                count += rows;
-#pragma unroll 1
-                for (int g = g_first, gi = 0; g < groups; g += g_step, ++gi) {
-                    const int left = n_chunk - 32 * g, lsh = left >= 32 ? 3 : 2;
-                    ea.out = out + 32 * g;
-                    if (BNB) { ea.bn_mean = bnb + 32 * g; ea.bn_gamma = p.bn_gamma + co0 + 32 * g; ea.bn_beta = p.bn_beta + co0 + 32 * g; }
-                    if (extra) {
-                        ea.extra = extra + 32 * g;
-                        if (t > t_first || gi > 0) emit_residuals(ea, ro, lane, lsh, 0, e);
-                    }
-                    if (stats) ea.moments = mom0 + flip * mom_size + part * 3 * n_chunk + 32 * g;
-                    // 16 columns of the row at a time into the patch
-#pragma unroll 1
-                    for (int h = 0; h < 2 && 16 * h < left; ++h) {
-                        float v[16];
-                        if (ksplit > 1) {
-#pragma unroll
-                            for (int j = 0; j < 16; ++j) v[j] = 0.f;
-#pragma unroll 1
-                            for (int z = 0; z < ksplit; ++z) {
-                                float w[16];
-                                load16(sk_all + ((size_t)z * T + t) * sk_tile + ((size_t)(2 * g + h) * kTileM + quad * 32 + lane) * 16, w);
-#pragma unroll
-                                for (int j = 0; j < 16; j += 2) unpair(add2(pair(v[j], v[j + 1]), pair(w[j], w[j + 1])), v[j], v[j + 1]);
-                            }
-                        } else {
-                            accumulator(t, 32 * g + 16 * h, v);
-                        }
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) patch[lane * 8 + ((4 * h + j) ^ (lane & 7))] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
-                    }
-                    __syncwarp();
-                    emit_rows<BNB>(ea, ro, fill, lane, lsh, have, e);
-                }
-                if (rows) have = true;
-            }
-            // the accumulator is read: the next unit's MMAs may have it
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(acc_empty + 8 * buf);
-            if (alternate) par ^= 1u;                 // (a set of warps always meets its own accumulator set)
-            else if (++buf == p.acc_bufs) { buf = 0; par ^= 1u; }
-            }
-            turn ^= 1;
-            if (stats && finish && (ksplit > 1 || u.last_of_block())) {
-                // the block's moments: lanes, then the warps' parts, each about its own shift
-                float* contrib = mom0 + flip * mom_size;
-                float* counts = contrib + (size_t)parts * 3 * n_chunk;
-                if (lane == 0 && (whole || half == 0)) counts[part] = (float)count;
-                count = 0; have = false;
-                if (alternate) part = ew ^ (turn << 2);
-                epi_sync();
-                if (BNB && tid < n_chunk) {
-                    float sum = 0.f, sq = 0.f;
-                    const float* c3 = contrib + tid;
-#pragma unroll 1
-                    for (int w = 0; w < parts; ++w, c3 += 3 * n_chunk)
-                        if (counts[w] > 0.f) { sum += c3[n_chunk]; sq += c3[2 * n_chunk]; }
-                    float* row = p.st_partials + (size_t)u.m * partial_floats(p.blocks_per_m, C_out) + (size_t)(u.ul / p.unit_block) * 2 * C_out + co0 + tid;
-                    if (ok) { row[0] = sum; row[C_out] = sq; }
-                } else if (tid < n_chunk) {
-                    // parts about their own shifts k_w: sum and squares about the first one's,
-                    //   sum (x - k0) = sum_w [d_w + n_w e],  sum (x - k0)^2 = sum_w [q_w + e (2 d_w + n_w e)],  e = k_w - k0
-                    float N = 0.f, k0 = 0.f, sum = 0.f, sq = 0.f;
-                    const float* c3 = contrib + tid;
-#pragma unroll 1
-                    for (int w = 0; w < parts; ++w, c3 += 3 * n_chunk) {
-                        const float n = counts[w];
-                        if (n == 0.f) continue;
-                        const float d = c3[n_chunk];
-                        if (N == 0.f) k0 = c3[0];
-                        const float e = c3[0] - k0;
-                        N += n;
-                        sum += fmaf(n, e, d);
-                        sq += fmaf(e, fmaf(n, e, 2.f * d), c3[2 * n_chunk]);
-                    }
-                    const float dm = N > 0.f ? sum / N : 0.f, m2 = fmaxf(fmaf(-sum, dm, sq), 0.f);
-                    float* dst = p.st_partials + (size_t)u.m * partial_floats(p.blocks_per_m, C_out);
-                    const int r = u.ul / p.unit_block;
-                    float* row = dst + (size_t)r * 2 * C_out + co0 + tid;
-                    if (ok) { row[0] = k0 + dm; row[C_out] = m2; }
-                    if (tid == 0 && slice == 0 && ok) dst[(size_t)p.blocks_per_m * 2 * C_out + r] = N;
-                }
-                flip ^= 1;
-            }
-        }
+        write_out<W, FLAT, BNB, CELL>(p, sh, smem, tmem_base, acc_full, acc_empty, u0, slice);
     }
 
     // ---- teardown ----
@@ -1009,7 +1138,7 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
     __syncthreads();
 }
 
-template <bool BN_IN, bool FLAT, bool BNB>
+template <bool BN_IN, bool FLAT, bool BNB, int W>
 __global__ void __launch_bounds__(kPipeThreads, 1) conv_pipe_kernel(const __grid_constant__ PipeParams gp, const int m_first, const int m_count)
 {
     const PipeScalars& p = gp.s;
@@ -1023,7 +1152,7 @@ __global__ void __launch_bounds__(kPipeThreads, 1) conv_pipe_kernel(const __grid
     __shared__ PipeShared sh;
     uint8_t* smem = smem_raw + (((smem_u32(smem_raw) + 1023u) & ~1023u) - smem_u32(smem_raw));
     if (warp_index() == 3) pipe_init_barriers(p, sh, threadIdx.x & 31);
-    if (threadIdx.x == 32) { prefetch_tmap(&gp.tm_a); prefetch_tmap(&gp.tm_b); prefetch_tmap(&gp.tm_b_lo); }
+    if (threadIdx.x == 32) { if (!p.flat) prefetch_tmap(&gp.tm_a); prefetch_tmap(&gp.tm_b); prefetch_tmap(&gp.tm_b_lo); }
     if (warp_index() == 0) tmem_alloc(smem_u32(&sh.tmem_slot), p.tmem_cols);
     tc_fence_before();
     __syncthreads();
@@ -1032,7 +1161,7 @@ __global__ void __launch_bounds__(kPipeThreads, 1) conv_pipe_kernel(const __grid
     // take the columns this one needs and wait for this one to finish.
     if (!p.pdl_late) pdl_launch_dependents();
     const uint32_t tmem_base = sh.tmem_slot;
-    pipe_cta<BN_IN, FLAT, BNB, false>(gp, p, sh, smem, tmem_base, m_first, m_count, (int)blockIdx.x, (int)gridDim.x);
+    pipe_cta<BN_IN, FLAT, BNB, W, false>(gp, p, sh, smem, tmem_base, m_first, m_count, (int)blockIdx.x, (int)gridDim.x);
     if (warp_index() == 0) tmem_dealloc(tmem_base, p.tmem_cols);
 }
 
@@ -1136,11 +1265,11 @@ __global__ void __launch_bounds__(kPipeThreads, 1) conv_pipe_cell_kernel(const _
             __syncthreads();
             tc_fence_after();
             if (bn_in) {
-                if (flat) pipe_cta<true, true, false, true>(gp, p, sh, smem, tmem_base, m_first, m_count, v, V);
-                else pipe_cta<true, false, false, true>(gp, p, sh, smem, tmem_base, m_first, m_count, v, V);
+                if (flat) { if (p.wide) pipe_cta<true, true, false, 8, true>(gp, p, sh, smem, tmem_base, m_first, m_count, v, V); else pipe_cta<true, true, false, 4, true>(gp, p, sh, smem, tmem_base, m_first, m_count, v, V); }
+                else { if (p.wide) pipe_cta<true, false, false, 8, true>(gp, p, sh, smem, tmem_base, m_first, m_count, v, V); else pipe_cta<true, false, false, 4, true>(gp, p, sh, smem, tmem_base, m_first, m_count, v, V); }
             } else {
-                if (flat) pipe_cta<false, true, false, true>(gp, p, sh, smem, tmem_base, m_first, m_count, v, V);
-                else pipe_cta<false, false, false, true>(gp, p, sh, smem, tmem_base, m_first, m_count, v, V);
+                if (flat) { if (p.wide) pipe_cta<false, true, false, 8, true>(gp, p, sh, smem, tmem_base, m_first, m_count, v, V); else pipe_cta<false, true, false, 4, true>(gp, p, sh, smem, tmem_base, m_first, m_count, v, V); }
+                else { if (p.wide) pipe_cta<false, false, false, 8, true>(gp, p, sh, smem, tmem_base, m_first, m_count, v, V); else pipe_cta<false, false, false, 4, true>(gp, p, sh, smem, tmem_base, m_first, m_count, v, V); }
             }
             if (sh.abort_flag) { if (tid == 0) cell_stop = 1; break; }
         }
@@ -1237,7 +1366,14 @@ int sm_count()
 }
 
 constexpr int kPlanSms = 148;                         // the split of the work is planned for a whole B200, with or without a device at hand
-inline unsigned int stat_bytes(int n_chunk) { return (unsigned int)(2 * (n_chunk <= 64 ? 8 : 4) * (3 * n_chunk + 1) * 4 + 127) & ~127u; }
+inline unsigned int stat_bytes(int n_chunk) { return (unsigned int)(2 * (n_chunk <= 32 ? 8 : 4) * (3 * n_chunk + 1) * 4 + 127) & ~127u; }
+// sums a write-out warp's lanes keep: two values of 32 lanes a channel of its groups (no launch of more than 128 channels forms any)
+inline unsigned int slot_bytes(int n_chunk)
+{
+    if (n_chunk > 128) return 0;
+    return n_chunk % 32 == 0 ? (unsigned int)(n_chunk / 32 + 1) / 2 * 2048u : (unsigned int)(n_chunk / 16 + 1) / 2 * 1024u;
+}
+constexpr unsigned int kBnbBytes = kEpiWarps * 1024u;  // statistics and parameters of a write-out warp's channels (data gradient)
 inline int split_groups_of(int a_stages) { return a_stages % 4 == 0 ? 4 : (a_stages % 2 == 0 ? 2 : 1); }
 inline unsigned int bn_bytes(int c_in) { return (unsigned int)(4 * c_in * 4 + 4 * kSplitThreads * 16); }
 
@@ -1245,7 +1381,7 @@ inline unsigned int bn_bytes(int c_in) { return (unsigned int)(4 * c_in * 4 + 4 
 
 size_t conv_pipe_partial_floats(int units_per_m, int channels) { return partial_floats(units_per_m, channels); }
 
-static bool plan_geom(const ConvShape& s, int pass, int passes, int launched, ConvPipeGeom* g)
+static bool plan_geom(const ConvShape& s, int pass, int passes, int launched, ConvPipeUse use, ConvPipeGeom* g)
 {
     PipeView v;
     if (pass == PASS_WGRAD || !pipe_view(s, pass, &v)) return false;
@@ -1278,7 +1414,9 @@ static bool plan_geom(const ConvShape& s, int pass, int passes, int launched, Co
     g->b_tap_bytes = (unsigned int)(three ? 2 : 1) * (unsigned int)n * 64u;
     const unsigned int all_b = g->b_tap_bytes * (unsigned int)(taps * chunks);
     // (the data gradient applies no BN)
-    const unsigned int fixed = kEpiWarps * 4096u + stat_bytes(n) + (pass == PASS_FWD ? bn_bytes(v.c_in <= 512 ? v.c_in : 0) : 0u);
+    g->use = use;
+    const unsigned int fixed = (use.addend ? kEpiWarps * (n % 32 == 0 ? 4096u : 2048u) : 0u) + (use.moments ? kEpiWarps * slot_bytes(n) + stat_bytes(n) : 0u) + 128u +
+                               (pass == PASS_DGRAD ? (use.moments ? kBnbBytes : 0u) : (use.bn_in ? bn_bytes(v.c_in) : 0u));
     // Tiles per unit, stacked weights (hi*hi and hi*lo from one MMA over [B_hi; B_lo]), accumulator sets and the two rings:
     // the combination with the least modelled time for the busiest CTA, from clocks measured stage by stage.  A chunk takes
     // the longest of: its MMAs (K = 8; at 128 columns an unstacked MMA reads 128 bytes of shared memory per clock, all there
@@ -1301,7 +1439,7 @@ static bool plan_geom(const ConvShape& s, int pass, int passes, int launched, Co
                 const int per_slice = kPlanSms / g->slices > 0 ? kPlanSms / g->slices : 1;
                 const double rounds = (double)(((long long)launched * units + per_slice - 1) / per_slice);
                 const double step = !three ? clk(n) : (stacked ? clk(2 * n) + clk(n) : 3.0 * (n == 128 ? 80.0 : clk(n)));
-                const double tap_mma = 2.0 * T * step, epi = 1100.0 * T * ((n + 31) / 32) / 2.0;
+                const double tap_mma = 2.0 * T * step, epi = T * (use.addend ? 3600.0 : 2000.0) * (n <= 32 ? 0.5 : (n + 63) / 64);
                 // weights: resident, or a ring whose stage holds the taps of a window row (fewer waits) or one tap
                 for (int bt = s.R; bt >= 0; bt = bt == 3 ? 1 : bt - 1) {
                     const bool resident = bt == 0;
@@ -1319,10 +1457,11 @@ static bool plan_geom(const ConvShape& s, int pass, int passes, int launched, Co
                         const int groups = split_groups_of(as);
                         if (tried & groups) continue;
                         tried |= groups;
-                        const double split = three ? 250.0 + 5.6 * rows * groups / 4.0 : 100.0;
+                        const double split = use.bn_in ? 1200.0 + 8.0 * rows * groups / 4.0 : (three ? 250.0 + 5.6 * rows * groups / 4.0 : 100.0);
                         const double chunk = std::max({mma, (1200.0 + rows * 1.6 + split + mma) / as, split / groups, rows * 64.0 / 20.0});
                         const double k_loop = chunk * chunks, body = bufs == 2 ? std::max(k_loop, epi) : k_loop + epi;
-                        const double cost = rounds * body + chunk + 1000.0 + epi;
+                        // (weights that stay leave the memory system to the rest)
+                        const double cost = (rounds * body + chunk + 1000.0 + epi) * (resident ? 1.0 : 1.03);
                         if (g->T == 0 || cost < best * 0.999) {
                             best = cost;
                             g->T = T; g->units_per_m = units; g->a_rows = nj * kRowStep; g->a_stage_bytes = a_stage; g->a_stages = as;
@@ -1363,18 +1502,18 @@ static bool plan_geom(const ConvShape& s, int pass, int passes, int launched, Co
 // The search takes several microseconds and a single convolution's call asks for its plan and its scratch sizes: as long as the
 // convolution itself for a small one (1x1 on 4 x 4 maps, forward and both gradients: 64 us, 32 with the last plans kept).
 // Each thread keeps a fixed number of them.
-bool conv_pipe_geom(const ConvShape& s, int pass, int passes, int launched, ConvPipeGeom* g)
+bool conv_pipe_geom(const ConvShape& s, int pass, int passes, int launched, ConvPipeUse use, ConvPipeGeom* g)
 {
-    struct Kept { int key[11]; bool used, ok; ConvPipeGeom g; };
+    struct Kept { int key[12]; bool used, ok; ConvPipeGeom g; };
     constexpr int kKept = 64;
     static thread_local Kept kept[kKept];
-    const int key[11] = {s.N, s.H, s.W, s.C, s.K, s.R, s.stride, s.pad, pass, passes, launched};
+    const int key[12] = {s.N, s.H, s.W, s.C, s.K, s.R, s.stride, s.pad, pass, passes, launched, (use.addend ? 1 : 0) | (use.moments ? 2 : 0) | (use.bn_in ? 4 : 0)};
     unsigned int h = 2166136261u;
     for (int k : key) h = (h ^ (unsigned int)k) * 16777619u;
     Kept& e = kept[(h >> 16) % kKept];
     if (!e.used || memcmp(e.key, key, sizeof key) != 0) {
         memcpy(e.key, key, sizeof key);
-        e.ok = plan_geom(s, pass, passes, launched, &e.g);
+        e.ok = plan_geom(s, pass, passes, launched, use, &e.g);
         e.used = true;
     }
     *g = e.g;
@@ -1392,11 +1531,22 @@ size_t conv_pipe_splitk_bytes(const ConvPipeGeom& g)
 size_t conv_pipe_splitk_bytes(const ConvShape& s, int pass, int passes, int launched)
 {
     ConvPipeGeom g;
-    return conv_pipe_geom(s, pass, passes, launched, &g) ? conv_pipe_splitk_bytes(g) : 0;
+    return conv_pipe_geom(s, pass, passes, launched, ConvPipeUse(), &g) ? conv_pipe_splitk_bytes(g) : 0;
 }
 
 struct ConvPipeLaunch { PipeParams p; unsigned int smem; int bn_in; };
 static_assert(sizeof(ConvPipeLaunch) <= sizeof(((ConvPipePlan*)0)->storage), "plan storage too small");
+
+namespace {
+using PipeKernel = void (*)(PipeParams, int, int);
+template <int W>
+PipeKernel pipe_kernel(bool bn_in, bool flat, bool bnb)
+{
+    if (bn_in) return flat ? conv_pipe_kernel<true, true, false, W> : conv_pipe_kernel<true, false, false, W>;
+    if (bnb) return flat ? conv_pipe_kernel<false, true, true, W> : conv_pipe_kernel<false, false, true, W>;
+    return flat ? conv_pipe_kernel<false, true, false, W> : conv_pipe_kernel<false, false, false, W>;
+}
+}  // namespace
 
 cudaError_t conv_pipe_init()
 {
@@ -1404,9 +1554,9 @@ cudaError_t conv_pipe_init()
     bool set = false;
     return attributes.get(&set, [](int, bool* done) {
         cudaError_t e = cudaSuccess;
-        for (auto kernel : {conv_pipe_kernel<false, false, false>, conv_pipe_kernel<false, true, false>, conv_pipe_kernel<true, false, false>, conv_pipe_kernel<true, true, false>,
-                            conv_pipe_kernel<false, false, true>, conv_pipe_kernel<false, true, true>})
-            if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPipeSmem + 1024);
+        for (int k = 0; k < 6; ++k)
+            for (PipeKernel kernel : {pipe_kernel<8>(k >= 4, k & 1, k == 2 || k == 3), pipe_kernel<4>(k >= 4, k & 1, k == 2 || k == 3)})
+                if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPipeSmem + 1024);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(conv_pipe_cell_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPipeSmem + 1024);
         *done = true;
         return e;
@@ -1418,16 +1568,19 @@ cudaError_t encode_map(CUtensorMap* tm, const float* base, int rank, const cuuin
                        CUtensorMapSwizzle swizzle)
 {
     if (!g_encode) return cudaErrorNotReady;
-    const cuuint32_t ones[4] = {1, 1, 1, 1};
+    const cuuint32_t ones[5] = {1, 1, 1, 1, 1};
     const CUresult r = g_encode(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, (cuuint32_t)rank, const_cast<float*>(base), dims, strides, box, ones,
                                 CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
-cudaError_t encode_weights(CUtensorMap* tm, const float* base, long long kdim, int c_out, int n_chunk)
+// Rows in the order the write-out wants the accumulator's columns in (write_out): of a group of 4 W channels, columns 2 i and 2 i + 1
+// of the c-th eight are channels W i + 2 c and the next.
+cudaError_t encode_weights(CUtensorMap* tm, const float* base, long long kdim, int c_out, int n_chunk, int W)
 {
-    const cuuint64_t dims[2] = {(cuuint64_t)kdim, (cuuint64_t)c_out}, strides[1] = {(cuuint64_t)kdim * 4};
-    const cuuint32_t box[2] = {16, (cuuint32_t)n_chunk};
-    return encode_map(tm, base, 2, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_64B);
+    const cuuint64_t row = (cuuint64_t)kdim * 4;
+    const cuuint64_t dims[5] = {(cuuint64_t)kdim, 2, 4, (cuuint64_t)W / 2, (cuuint64_t)(c_out / (4 * W))}, strides[4] = {row, W * row, 2 * row, 4 * W * row};
+    const cuuint32_t box[5] = {16, 2, 4, (cuuint32_t)W / 2, (cuuint32_t)(n_chunk / (4 * W))};
+    return encode_map(tm, base, 5, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_64B);
 }
 unsigned int columns_pow2(unsigned int need)
 {
@@ -1439,17 +1592,20 @@ unsigned int columns_pow2(unsigned int need)
 
 cudaError_t conv_pipe_prepare(ConvPipePlan* plan, const ConvShape& s, int pass, int passes, int M, int launched, const float* in, const float* w_hi,
                               const float* w_lo, float* out, const float* extra, bool accumulate, const ConvPipeBn* bn, void* splitk,
-                              size_t splitk_bytes, bool w_ready)
+                              size_t splitk_bytes, bool w_ready, ConvPipeUse use)
 {
     plan->valid = 0;
     ConvPipeGeom g;
     PipeView v;
-    if ((passes != 1 && passes != 3) || !conv_pipe_geom(s, pass, passes, launched, &g) || !pipe_view(s, pass, &v)) return cudaErrorNotSupported;
+    if ((passes != 1 && passes != 3) || !conv_pipe_geom(s, pass, passes, launched, use, &g) || !pipe_view(s, pass, &v)) return cudaErrorNotSupported;
     ConvPipeLaunch* L = reinterpret_cast<ConvPipeLaunch*>(plan->storage);
     memset(L, 0, sizeof *L);
     const long long kdim = (long long)s.R * s.R * v.c_in;
-    cudaError_t e = encode_weights(&L->p.tm_b, w_hi, kdim, v.c_out, g.n_chunk);
-    if (e == cudaSuccess) e = encode_weights(&L->p.tm_b_lo, passes == 3 ? w_lo : w_hi, kdim, v.c_out, g.n_chunk);
+    // 32-byte pieces of a row where the buffers allow them (a caller's own may start at any 16 bytes)
+    const uintptr_t at = reinterpret_cast<uintptr_t>(out) | reinterpret_cast<uintptr_t>(splitk) | (splitk_bytes & 31);
+    const bool wide = g.n_chunk % 32 == 0 && at % 32 == 0;
+    cudaError_t e = encode_weights(&L->p.tm_b, w_hi, kdim, v.c_out, g.n_chunk, wide ? 8 : 4);
+    if (e == cudaSuccess) e = encode_weights(&L->p.tm_b_lo, passes == 3 ? w_lo : w_hi, kdim, v.c_out, g.n_chunk, wide ? 8 : 4);
     if (e != cudaSuccess) return e;
     PipeScalars& p = L->p.s;
     p.in = in; p.out = out; p.extra = extra; p.in_ms = v.in_ms; p.out_ms = v.out_ms;
@@ -1458,21 +1614,18 @@ cudaError_t conv_pipe_prepare(ConvPipePlan* plan, const ConvShape& s, int pass, 
     p.R = s.R; p.taps = s.R * s.R; p.n_chunks = v.c_in / 16; p.c_in = v.c_in; p.c_out = v.c_out;
     p.pos_per_m = g.pos_per_m; p.Wp = g.Wp; p.img_pos = g.Wp * g.Hp; p.Hv = v.P; p.W = v.Q; p.halo = g.halo;
     p.strips = g.strips; p.strip_w = g.strip_w; p.col0 = g.col0;
-    p.magic_w = magic_of(g.Wp); p.magic_img = magic_of(p.img_pos); p.magic_strip = magic_of(g.strips);
+    p.magic_w = magic_of(g.Wp); p.magic_img = magic_of(p.img_pos); p.magic_strip = magic_of(g.strips); p.magic_blocks = magic_of(g.blocks_per_m); p.magic_ksplit = magic_of(g.ksplit);
     p.in_sw = v.in_sw; p.in_sh = v.in_sh; p.in_sn = v.in_sn; p.os_w = v.os_w; p.os_h = v.os_h; p.os_n = v.os_n;
     p.zero_fill = v.zero_fill; p.out_h = v.out_h; p.out_w = v.out_w; p.dense_h = v.dense_h; p.dense_w = v.dense_w;
     p.flat = g.flat; p.box_h = g.box_h; p.box_pos = g.box_h * g.Wp; p.blocks_per_img = g.Hp / g.box_h;
     p.magic_box = magic_of(p.box_pos); p.magic_bpi = magic_of(p.blocks_per_img);
     p.pix_ms = g.flat ? (long long)s.N * v.P * v.Q : s.N;
     if ((long long)M * p.pix_ms >= (1LL << 31)) return cudaErrorNotSupported;
-    {
-        CUtensorMap* tm = &L->p.tm_a;
-        const cuuint64_t fd[2] = {(cuuint64_t)v.c_in, (cuuint64_t)(M * p.pix_ms)}, fs[1] = {(cuuint64_t)v.c_in * 4};
-        const cuuint32_t fb[2] = {16, kTileM};
+    if (!g.flat) {
         const cuuint64_t rd[4] = {(cuuint64_t)v.c_in, (cuuint64_t)v.in_W, (cuuint64_t)v.in_H, (cuuint64_t)M * s.N};
         const cuuint64_t rs[3] = {(cuuint64_t)v.in_sw * 4, (cuuint64_t)v.in_sh * 4, (cuuint64_t)v.in_sn * 4};
         const cuuint32_t rb[4] = {16, (cuuint32_t)g.Wp, (cuuint32_t)g.box_h, 1};
-        e = g.flat ? encode_map(tm, in, 2, fd, fs, fb, CU_TENSOR_MAP_SWIZZLE_128B) : encode_map(tm, in, 4, rd, rs, rb, CU_TENSOR_MAP_SWIZZLE_128B);
+        e = encode_map(&L->p.tm_a, in, 4, rd, rs, rb, CU_TENSOR_MAP_SWIZZLE_128B);
         if (e != cudaSuccess) return e;
     }
     p.a_stages = g.a_stages; p.b_stages = g.b_stages; p.b_taps = g.b_taps; p.b_resident = g.b_resident; p.acc_bufs = g.acc_bufs;
@@ -1481,15 +1634,20 @@ cudaError_t conv_pipe_prepare(ConvPipePlan* plan, const ConvShape& s, int pass, 
     p.idesc = instr_desc(g.n_chunk, false, false);
     p.idesc2 = instr_desc(g.stacked ? 2 * g.n_chunk : g.n_chunk, false, false);
     p.split_groups = split_groups_of(g.a_stages);
-    p.epi_alternate = g.acc_bufs == 2 && g.n_chunk <= 64 && g.ksplit == 1 ? 1 : 0;
+    p.wide = wide ? 1 : 0;
+    p.epi_alternate = g.acc_bufs == 2 && g.n_chunk == (wide ? 32 : 16) && g.ksplit == 1 ? 1 : 0;
+    p.slot_bytes = slot_bytes(g.n_chunk);
     p.three = passes == 3 ? 1 : 0; p.stacked = g.stacked; p.w_ready = w_ready ? 1 : 0;
     const unsigned int a_bytes = (unsigned int)g.a_stages * g.a_stage_bytes;
     p.off_b = a_bytes;
-    p.off_stage = (p.off_b + (unsigned int)g.b_stages * g.b_stage_bytes + 127u) & ~127u;
-    p.off_stat = p.off_stage + kEpiWarps * 4096u;
-    p.off_red = p.off_stat + stat_bytes(g.n_chunk);
+    p.off_ring = (p.off_b + (unsigned int)g.b_stages * g.b_stage_bytes + 127u) & ~127u;
+    p.off_slots = p.off_ring + (g.use.addend ? kEpiWarps * (wide ? 4096u : 2048u) : 0u);
+    p.off_stat = p.off_slots + (g.use.moments ? kEpiWarps * p.slot_bytes : 0u);
+    p.off_red = p.off_bnb = p.off_stat + (g.use.moments ? stat_bytes(g.n_chunk) : 0u);
     p.off_bn = p.off_red + 4 * kSplitThreads * 16;
-    L->smem = p.off_red + 1024;
+    const bool sums = bn && (bn->out_partials || bn->bwd_partials);
+    if (((extra || (bn && bn->bwd_partials)) && !use.addend) || (sums && !use.moments) || (bn && bn->in_partials && !use.bn_in)) return cudaErrorInvalidValue;
+    L->smem = p.off_red + (pass == PASS_DGRAD && use.moments ? kBnbBytes : 0u) + 1024;
     if (bn && bn->out_partials) {
         if (!conv_pipe_can_fuse_bn_output(g)) return cudaErrorNotSupported;
         p.st_partials = bn->out_partials;
@@ -1529,15 +1687,12 @@ cudaError_t conv_pipe_launch(const ConvPipePlan* plan, int m_first, int m_count,
     if (per_slice < 1) per_slice = 1;
     if (per_slice > tasks) per_slice = tasks;
     const bool flat = p.flat && p.zero_fill == 1;
-    auto kernel = L.bn_in ? (flat ? conv_pipe_kernel<true, true, false> : conv_pipe_kernel<true, false, false>)
-                          : (p.bn_x ? (flat ? conv_pipe_kernel<false, true, true> : conv_pipe_kernel<false, false, true>)
-                                    : (flat ? conv_pipe_kernel<false, true, false> : conv_pipe_kernel<false, false, false>));
+    auto kernel = p.wide ? pipe_kernel<8>(L.bn_in, flat, p.bn_x != nullptr) : pipe_kernel<4>(L.bn_in, flat, p.bn_x != nullptr);
     // What a CTA has to do decides how its warps share it (the sums are the same either way).  A block of the operand takes one
     // splitter warp about 2000 clocks and all four of them 850, so with one or two blocks in all they share each; with a single unit
     // both halves of the write-out's warps take it.
     const int units = (tasks + per_slice - 1) / per_slice * p.unit_block, blocks = units * ((p.n_chunks + p.ksplit - 1) / p.ksplit);
     if (blocks < 4) L.p.s.split_groups = blocks < 2 || p.split_groups == 1 ? 1 : 2;
-    if (units == 1 && p.n_chunk > 32) L.p.s.epi_alternate = 0;      // (each half a group of columns: the partial sums of the moments stay the same)
     launch_pdl(kernel, dim3(per_slice * p.slices), dim3(kPipeThreads), L.smem, st, L.p, m_first, m_count);
     if (n_launch) ++*n_launch;
     return cudaGetLastError();

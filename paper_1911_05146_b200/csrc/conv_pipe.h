@@ -5,6 +5,13 @@
 
 namespace hpf {
 
+// What a launch may be asked to do besides the convolution: shared memory is planned for it.
+struct ConvPipeUse {
+    bool addend = false;         // the write-out reads a residual (or, for the sums of a BN+ReLU's backward, its input) beside the accumulator
+    bool moments = false;        // it forms BN moments or the sums of a BN+ReLU's backward
+    bool bn_in = false;          // a BN+ReLU is applied to the operand
+};
+
 // Work split of one convolution.  It depends on the shape of ONE micro-batch, on the precision and on how many micro-batches
 // the launches it is planned for cover - never on which of them share a launch - so that every sum is formed in the same order
 // whichever micro-batches a planned launch is given.
@@ -18,10 +25,11 @@ struct ConvPipeGeom {
     int a_rows, a_stages, b_stages, b_taps, b_resident, acc_bufs;      // b_taps: taps per stage of the weight ring
     unsigned int acc_cols, a_stage_bytes, b_stage_bytes, b_tap_bytes;
     int stacked;
+    ConvPipeUse use;
     int flat, box_h;             // operand copies: 128 consecutive pixels, or box_h padded map rows each
     int pos_per_m, Wp, Hp, halo, strips, strip_w, col0;
 };
-bool conv_pipe_geom(const ConvShape& s, int pass, int passes, int launched, ConvPipeGeom* g);
+bool conv_pipe_geom(const ConvShape& s, int pass, int passes, int launched, ConvPipeUse use, ConvPipeGeom* g);
 
 // BN work that rides in the forward kernel.
 //   out_partials: the output is the input of a BN: per block of units and output channel the mean and the sum of squared
@@ -65,7 +73,7 @@ cudaError_t conv_pipe_init();
 // its stream was enqueued.
 cudaError_t conv_pipe_prepare(ConvPipePlan* plan, const ConvShape& s, int pass, int passes, int M, int launched, const float* in, const float* w_hi,
                               const float* w_lo, float* out, const float* extra, bool accumulate, const ConvPipeBn* bn,
-                              void* splitk, size_t splitk_bytes, bool w_ready);
+                              void* splitk, size_t splitk_bytes, bool w_ready, ConvPipeUse use);
 // Micro-batches m_first .. m_first + m_count - 1 in one launch.
 // pdl_late: the successor may be scheduled when the last accumulator of a CTA is complete, not at its start.
 cudaError_t conv_pipe_launch(const ConvPipePlan* plan, int m_first, int m_count, bool pdl_late, DeviceStatus* status, cudaStream_t st, int64_t* n_launch);

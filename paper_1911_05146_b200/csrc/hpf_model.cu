@@ -632,7 +632,19 @@ bool op_uses_tc(hpf_model* mdl, hpf_model::KernelPlan* k, int i, int pass)
     if (pass == PASS_DGRAD && mdl->ops[i].op.stride > 1 && (mdl->edge0[i].accumulate || mdl->edge0[i].addend >= 0)) return false;
     if (pass == PASS_WGRAD) return conv_tc_supported(conv_shape_of(mdl, i), pass);
     const ConvShape s = conv_shape_of(mdl, i);
-    k->use_pipe[pass][i] = mdl->has_bn && conv_pipe_geom(s, pass, passes_of(mdl), k->launched, &k->pipe_geom[pass][i]);
+    // what may ride in the launch (what does is decided with the plans at hand)
+    auto is_bn = [&](int op) { return mdl->ops[op].op.kind == HPF_OP_BNRELU; };
+    ConvPipeUse use;
+    if (pass == PASS_FWD) {
+        const int out = mdl->fused_into[i] >= 0 ? mdl->fused_into[i] : i;
+        use.addend = out != i;
+        for (int c : mdl->ops[out].consumers) use.moments = use.moments || is_bn(c);
+        use.bn_in = is_bn(mdl->ops[i].op.src0) && conv_pipe_can_fuse_bn_input(s);
+    } else {
+        use.moments = is_bn(mdl->ops[i].op.src0) && mdl->ops[i].op.stride == 1;
+        use.addend = mdl->edge0[i].addend >= 0 || use.moments;
+    }
+    k->use_pipe[pass][i] = mdl->has_bn && conv_pipe_geom(s, pass, passes_of(mdl), k->launched, use, &k->pipe_geom[pass][i]);
     return k->use_pipe[pass][i] || conv_tc_supported(s, pass);
 }
 
@@ -679,7 +691,7 @@ int prepare_kernels(hpf_model* mdl, hpf_model::KernelPlan& kp)
             }
             // the weights are prepared just ahead of the partition's first convolution
             if (kp.use_pipe[PASS_FWD][i]) CU(conv_pipe_prepare(&kp.pipe_plan[PASS_FWD][i], s, PASS_FWD, passes, M, kp.launched, in, wp + o.w_off, wp + G + o.w_off, mdl->act(i, 0),
-                                 residual, false, &bn, mdl->ws + mdl->splitk_off[p], mdl->splitk_bytes[p], first_done[p] != 0));
+                                 residual, false, &bn, mdl->ws + mdl->splitk_off[p], mdl->splitk_bytes[p], first_done[p] != 0, kp.pipe_geom[PASS_FWD][i].use));
             else {
                 tile.splitk = mdl->splitk_bytes[p] ? mdl->ws + mdl->splitk_off[p] : nullptr;
                 CU(conv_tc_prepare(&mdl->tile_plan[PASS_FWD][i], s, PASS_FWD, passes, in, nullptr, wp + o.w_off, wp + G + o.w_off, mdl->act(i, 0), residual,
@@ -698,7 +710,7 @@ int prepare_kernels(hpf_model* mdl, hpf_model::KernelPlan& kp)
         if (kp.use_pipe[PASS_DGRAD][i])
             CU(conv_pipe_prepare(&kp.pipe_plan[PASS_DGRAD][i], s, PASS_DGRAD, passes, M, kp.launched, mdl->grad(i, 0), wp + 2 * G + o.w_off,
                                  wp + 3 * G + o.w_off, mdl->grad(src, 0), ed.addend >= 0 ? mdl->grad(ed.addend, 0) : nullptr,
-                                 ed.accumulate != 0, &sums, mdl->ws + mdl->splitk_bwd_off[p], mdl->splitk_bytes[p], true));
+                                 ed.accumulate != 0, &sums, mdl->ws + mdl->splitk_bwd_off[p], mdl->splitk_bytes[p], true, kp.pipe_geom[PASS_DGRAD][i].use));
         else if (mdl->use_tc[PASS_DGRAD][i]) {
             tile.splitk = mdl->splitk_bytes[p] ? mdl->ws + mdl->splitk_bwd_off[p] : nullptr;
             CU(conv_tc_prepare(&mdl->tile_plan[PASS_DGRAD][i], s, PASS_DGRAD, passes, mdl->grad(i, 0), nullptr, wp + 2 * G + o.w_off, wp + 3 * G + o.w_off,
@@ -1807,7 +1819,7 @@ static int conv_single(int pass, const float* in, const float* in2, const float*
         const cudaError_t e = conv_tc_faster_alone(s, pass, path == 2 ? 1 : 3)
                                   ? cudaErrorNotSupported
                                   : conv_pipe_prepare(&pipe, s, pass, path == 2 ? 1 : 3, 1, 1, in, hi, hi + nw, out, nullptr, false, nullptr,
-                                                      reinterpret_cast<char*>(d_scratch) + align_up(a > b ? a : b, 256), single_splitk_bytes(s), false);
+                                                      reinterpret_cast<char*>(d_scratch) + align_up(a > b ? a : b, 256), single_splitk_bytes(s), false, ConvPipeUse());
         if (e == cudaSuccess) {
             CU(conv_pipe_launch(&pipe, 0, 1, false, status, st, nullptr));
             return HPF_OK;
