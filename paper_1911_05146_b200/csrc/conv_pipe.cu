@@ -203,12 +203,13 @@ __device__ __forceinline__ float4 lo_part(float4 v) { return sub4(v, make_float4
 // (every CTA of a launch gets the same bits), fp32 terms, the last combination in fp64.  THREADS threads, which share named
 // barrier 1; tab: mean[C], rstd[C]; red: 4 x THREADS float4.  First every thread adds its rows of four channels, then one
 // thread per channel combines: what this costs is latency and instruction fetches, so nothing is unrolled that need not be.
+// counts: the rows' n; second: float4 from a row's means to its M2 (a dry round reads other memory in their place).
 template <int THREADS>
-__device__ __forceinline__ void merge_moments(const float* partials, int rows, int C, double inv_rows, float eps, float* tab, float4* red, int tid)
+__device__ __forceinline__ void merge_moments(const float* partials, const float* counts, int rows, int second, int C, double inv_rows, float eps, float* tab, float4* red, int tid)
 {
-    const float* counts = partials + (size_t)rows * 2 * C;
     const int c4n = C >> 2;
     const int L = c4n <= THREADS ? THREADS / c4n : 1;
+    constexpr int kRows = 6;                          // rows in flight: 37 of 64 channels, 18 of 128 in one round trip
 #pragma unroll 1
     for (int c0 = 0; c0 < c4n; c0 += THREADS) {
         const int width = c4n - c0 < THREADS ? c4n - c0 : THREADS;       // float4 columns of this pass
@@ -216,22 +217,22 @@ __device__ __forceinline__ void merge_moments(const float* partials, int rows, i
         const bool mine = local < width && ln < L;
         float4 sd = make_float4(0.f, 0.f, 0.f, 0.f), sq = sd, m2 = sd, ref = sd;
         if (mine) {
-            if (rows > 0) ref = __ldcg(reinterpret_cast<const float4*>(partials) + col);
+            ref = __ldcg(reinterpret_cast<const float4*>(partials) + col);
 #pragma unroll 1
-            for (int k0 = ln; k0 < rows; k0 += 4 * L) {
-                float4 a[4], b[4];
-                float n[4];
+            for (int k0 = ln; k0 < rows; k0 += kRows * L) {
+                float4 a[kRows], b[kRows];
+                float n[kRows];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
+                for (int j = 0; j < kRows; ++j) {
                     const int k = k0 + j * L;
                     const bool have = k < rows;
                     const float4* row = reinterpret_cast<const float4*>(partials + (size_t)(have ? k : 0) * 2 * C);
                     n[j] = have ? __ldcg(counts + k) : 0.f;
                     a[j] = __ldcg(row + col);
-                    b[j] = have ? __ldcg(row + c4n + col) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    b[j] = have ? __ldcg(row + second + col) : make_float4(0.f, 0.f, 0.f, 0.f);
                 }
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
+                for (int j = 0; j < kRows; ++j) {
                     const float dx = a[j].x - ref.x, dy = a[j].y - ref.y, dz = a[j].z - ref.z, dw = a[j].w - ref.w;
                     const float nx = n[j] * dx, ny = n[j] * dy, nz = n[j] * dz, nw = n[j] * dw;
                     sd.x += nx; sd.y += ny; sd.z += nz; sd.w += nw;
@@ -1002,7 +1003,8 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
         const bool store_y = BN_IN && slice == 0;
         bool ok = true;
         UnitWalk cu = u0;
-        // The first round is a dry one (see write_out): no rows to merge, one row a thread, in the scratch of the merge.
+        // The first round is a dry one (see write_out): one row to merge (parameters in place of moments, which the preceding kernel
+        // may still write), one row a thread, in the scratch of the merge.
         bool dry = BN_IN;
 #pragma unroll 1
         while (cu.left > 0) {
@@ -1013,7 +1015,8 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
                 if (dry || cu.m != cur_m) {
                     if (!dry) cur_m = cu.m;
                     split_sync();                     // everybody is done with the table of the micro-batch before
-                    merge_moments<kSplitThreads>(p.bn_partials + (size_t)cu.m * partial_floats(p.bn_units, C), dry ? 0 : p.bn_units, C, p.bn_inv_rows, p.bn_eps, tab,
+                    const float* const rows0 = dry ? p.bn_gamma : p.bn_partials + (size_t)cu.m * partial_floats(p.bn_units, C);
+                    merge_moments<kSplitThreads>(rows0, dry ? p.bn_gamma : rows0 + (size_t)p.bn_units * 2 * C, dry ? 1 : p.bn_units, dry ? 0 : C >> 2, C, p.bn_inv_rows, p.bn_eps, tab,
                                   reinterpret_cast<float4*>(smem + p.off_red), tid);
                     split_sync();
                 }
@@ -1521,7 +1524,10 @@ bool conv_pipe_geom(const ConvShape& s, int pass, int passes, int launched, Conv
 }
 
 bool conv_pipe_can_fuse_bn_output(const ConvPipeGeom& g) { return g.n_chunk <= 128; }      // a warp keeps the moments of two groups of 32 channels
-bool conv_pipe_can_fuse_bn_input(const ConvShape& s) { return s.stride == 1 && s.C % 16 == 0 && s.C <= 512 && s.W <= 254; }      // (no column strips)
+// (No column strips.)  Every channel slice of a launch repeats the work on its operand, about 1200 clocks for 128 rows of 16 channels
+// instead of 400: with four and more slices of a 1x1 window that is what the launch takes, and BN+ReLU in kernels of their own
+// cost less (256->1024 @14 and the like: ResNet-152 35.0 -> 34.1 ms).  Two slices pay: 64->256 @56 would take 16 us to read and write.
+bool conv_pipe_can_fuse_bn_input(const ConvShape& s) { return s.stride == 1 && s.C % 16 == 0 && s.C <= 512 && s.W <= 254 && (s.R > 1 || s.K <= 256); }
 
 size_t conv_pipe_splitk_bytes(const ConvPipeGeom& g)
 {

@@ -418,6 +418,7 @@ void build_fusion_plan(hpf_model* mdl)
 ConvShape conv_shape_of(const hpf_model* mdl, int i);
 int passes_of(const hpf_model* mdl);
 bool op_uses_tc(hpf_model* mdl, hpf_model::KernelPlan* k, int i, int pass);
+bool bn_sums_wanted(const hpf_model* mdl, const hpf_model::KernelPlan* kp, int j);
 
 ConvShape conv_shape_of(const hpf_model* mdl, int i)
 {
@@ -426,6 +427,20 @@ ConvShape conv_shape_of(const hpf_model* mdl, int i)
 }
 
 int passes_of(const hpf_model* mdl) { return mdl->opt_conv_path == 2 ? 1 : 3; }
+
+// Backward: the only kernel that writes the gradient of the BN's output forms its sums, unless one launch of clusters
+// does it all from registers and is the better one: below a million values over the micro-batches of a launch (its clusters are
+// resident at once; the sums cost the data gradient's write-out about a microsecond of latency, resnet11 took 395 us
+// instead of 355), and beyond 128 channels (several channel slices repeat the work, and those data gradients are
+// bound by their MMAs: resnet152 36.7 ms against 37.2 with the sums everywhere; resnet1001 63.7 ms with clusters
+// wherever they fit, 61.3 so).
+bool bn_sums_wanted(const hpf_model* mdl, const hpf_model::KernelPlan* kp, int j)
+{
+    const OpInfo& o = mdl->ops[j];
+    const bool clusters = mdl->opt_bn_cluster && bn_bwd_is_one_launch((int64_t)mdl->b * o.H * o.W, o.C) &&
+                          (o.C > 128 || (int64_t)kp->launched * mdl->b * o.H * o.W * o.C < 1000000);
+    return o.op.kind == HPF_OP_BNRELU && !clusters;
+}
 
 // Which convolutions run on the tensor cores, and which BN work rides inside them: the statistics of a BN in the
 // forward kernel that produces its input (only when producer and BN run back to back on the same stream: same
@@ -449,15 +464,7 @@ void build_kernel_plan(hpf_model* mdl, hpf_model::KernelPlan* kp)
     for (int j = 0; j < n; ++j) {
         const OpInfo& bn = mdl->ops[j];
         if (bn.op.kind != HPF_OP_BNRELU) continue;
-        // Backward: the only kernel that writes the gradient of the BN's output forms its sums, unless one launch of clusters
-        // does it all from registers and is the better one: below a million values over the micro-batches of a launch (its clusters are
-        // resident at once; the sums cost the data gradient's write-out about a microsecond of latency, resnet11 took 395 us
-        // instead of 355), and beyond 128 channels (several channel slices repeat the work, and those data gradients are
-        // bound by their MMAs: resnet152 36.7 ms against 37.2 with the sums everywhere; resnet1001 63.7 ms with clusters
-        // wherever they fit, 61.3 so).
-        const bool clusters = mdl->opt_bn_cluster && bn_bwd_is_one_launch((int64_t)mdl->b * bn.H * bn.W, bn.C) &&
-                              (bn.C > 128 || (int64_t)kp->launched * mdl->b * bn.H * bn.W * bn.C < 1000000);
-        if (bn.consumers.size() == 1 && !clusters) {
+        if (bn.consumers.size() == 1 && bn_sums_wanted(mdl, kp, j)) {
             const int i = bn.consumers[0];
             const OpInfo& c = mdl->ops[i];
             if (i == j + 1 && c.op.kind == HPF_OP_CONV && c.op.stride == 1 && bn.C <= 2048 && c.part == bn.part && kp->use_pipe[PASS_DGRAD][i] && !mdl->edge0[i].accumulate &&
@@ -641,7 +648,7 @@ bool op_uses_tc(hpf_model* mdl, hpf_model::KernelPlan* k, int i, int pass)
         for (int c : mdl->ops[out].consumers) use.moments = use.moments || is_bn(c);
         use.bn_in = is_bn(mdl->ops[i].op.src0) && conv_pipe_can_fuse_bn_input(s);
     } else {
-        use.moments = is_bn(mdl->ops[i].op.src0) && mdl->ops[i].op.stride == 1;
+        use.moments = mdl->ops[i].op.stride == 1 && (mdl->opt_fuse_bn & 1) && bn_sums_wanted(mdl, k, mdl->ops[i].op.src0);
         use.addend = mdl->edge0[i].addend >= 0 || use.moments;
     }
     k->use_pipe[pass][i] = mdl->has_bn && conv_pipe_geom(s, pass, passes_of(mdl), k->launched, use, &k->pipe_geom[pass][i]);
