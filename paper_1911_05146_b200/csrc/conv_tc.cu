@@ -863,6 +863,7 @@ __global__ void __launch_bounds__(192) conv_tc_wgrad_direct_kernel(const __grid_
             const int stages = p.stages, k8n = p.rows >> 3;
             const bool three = p.passes == 3;
             const uint32_t ready0 = three ? split0 : full0;
+            const uint64_t lo = (uint64_t)(p.lo_off >> 4);
             int it = 0, s = 0;
             uint32_t par = 0;
             for (; it < total; ++it) {
@@ -874,16 +875,32 @@ __global__ void __launch_bounds__(192) conv_tc_wgrad_direct_kernel(const __grid_
                     const int nt = ntaps - tg < p.taps_per_mma ? ntaps - tg : p.taps_per_mma;
                     const uint32_t idesc = nt == p.taps_per_mma ? p.idesc : p.idesc_tail;
                     const uint32_t acc = tmem_base + (uint32_t)(tg * slot);
-                    const uint32_t b_tg = b_src + (uint32_t)tg * tap_bytes;
-                    for (int k8 = 0; k8 < k8n; ++k8) {
-                        const uint64_t ad = smem_desc_mn(a_src + 1024u * k8, block_bytes);
-                        const uint64_t bd = smem_desc_mn(b_tg + 1024u * k8, block_bytes);
-                        umma_tf32(acc, ad, bd, idesc, (it | k8) ? 1u : 0u);
+                    // (8 pixels are 1024 bytes, 64 units of a descriptor)
+                    uint64_t ad = smem_desc_mn(a_src, block_bytes), bd = smem_desc_mn(b_src + (uint32_t)tg * tap_bytes, block_bytes);
+                    uint32_t keep = it ? 1u : 0u;
+                    int k8 = 0;
+                    // Four K steps a round: one MMA of up to 64 columns takes 40-50 clocks, a branch of this one-thread loop between
+                    // two of them as much again (an MMA a round: 100 clocks).
+#pragma unroll 1
+                    for (; k8 + 4 <= k8n; k8 += 4, ad += 256, bd += 256, keep = 1u) {
                         if (three) {
-                            const uint64_t adl = smem_desc_mn(a_src + p.lo_off + 1024u * k8, block_bytes);
-                            const uint64_t bdl = smem_desc_mn(b_tg + p.lo_off + 1024u * k8, block_bytes);
-                            umma_tf32(acc, adl, bd, idesc, 1u);
-                            umma_tf32(acc, ad, bdl, idesc, 1u);
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                umma_tf32(acc, ad + 64 * j, bd + 64 * j, idesc, j ? 1u : keep);
+                                umma_tf32(acc, ad + lo + 64 * j, bd + 64 * j, idesc, 1u);
+                                umma_tf32(acc, ad + 64 * j, bd + lo + 64 * j, idesc, 1u);
+                            }
+                        } else {
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) umma_tf32(acc, ad + 64 * j, bd + 64 * j, idesc, j ? 1u : keep);
+                        }
+                    }
+#pragma unroll 1
+                    for (; k8 < k8n; ++k8, ad += 64, bd += 64, keep = 1u) {
+                        umma_tf32(acc, ad, bd, idesc, keep);
+                        if (three) {
+                            umma_tf32(acc, ad + lo, bd, idesc, 1u);
+                            umma_tf32(acc, ad, bd + lo, idesc, 1u);
                         }
                     }
                 }
@@ -936,24 +953,33 @@ __global__ void __launch_bounds__(192) conv_tc_wgrad_direct_kernel(const __grid_
         done = __all_sync(0xffffffffu, done);
         if (done) {
             tc_fence_after();
-            const int row = (warp & 3) * 32 + lane;          // TMEM lane = output channel within the chunk
-            const bool valid = row < p.m_chunk;
-            const uint32_t lane_addr = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
-            float* obase = p.out + (long long)micro * p.out_ms + (long long)split * p.split_stride + ((long long)(m0 + row) * p.R * p.R) * p.c_in + cn0;
-            if ((warp & 3) * 32 < p.m_chunk)                 // a whole warp of lanes beyond the chunk has nothing to read
+            // Four lanes have a row (an output channel) and store 8 bytes each, whole sectors of 8 rows: with a lane per row an instruction
+            // touched 32 lines, and a gradient slot that starts at an odd multiple of 8 bytes took 4-byte stores (VGG-16's 4096 x
+            // 4096 layer, 268 MB over four micro-batches, 266 us).
+            const int quad = warp & 3, q = lane & 3, row0 = quad * 32 + (lane >> 2);
+            const uint32_t lane_addr = tmem_base + ((uint32_t)(quad * 32) << 16);
+            const long long row_stride = (long long)p.R * p.R * p.c_in;
+            float* obase = p.out + (long long)micro * p.out_ms + (long long)split * p.split_stride + (m0 + row0) * row_stride + cn0 + 2 * q;
+            const bool pairs = (reinterpret_cast<uintptr_t>(obase) & 7u) == 0;      // (every other term is a whole number of 16-byte pieces)
+            if (quad * 32 < p.m_chunk)                       // a whole warp of lanes beyond the chunk has nothing to read
+#pragma unroll 1
                 for (int tp = 0; tp < ntaps; ++tp)
+#pragma unroll 1
                     for (int c0 = 0; c0 < p.n_cols; c0 += 16) {
-                        float v[16];
-                        tmem_ld16(lane_addr + (uint32_t)(tp * slot + c0), v);
-                        if (valid) {
-                            // a gradient slot starts at m*G floats: 16-byte aligned only if G is a multiple of 4
-                            float* o = obase + (long long)(tap0 + tp) * p.c_in + c0;
-                            if ((reinterpret_cast<uintptr_t>(o) & 15u) == 0) {
+                        float v[2][8];
+                        tmem_ld_rows<4>(lane_addr + (uint32_t)(tp * slot + c0), v[0]);
+                        tmem_ld_rows<4>(lane_addr + (16u << 16) + (uint32_t)(tp * slot + c0), v[1]);
+                        tmem_ld_wait();
+                        float* o = obase + (long long)(tap0 + tp) * p.c_in + c0;
 #pragma unroll
-                                for (int j = 0; j < 16; j += 4) *reinterpret_cast<float4*>(o + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+                        for (int i = 0; i < 4; ++i, o += 8 * row_stride) {
+                            if (row0 + 8 * i >= p.m_chunk) continue;
+                            const float* x = &v[i >> 1][2 * (i & 1)];
+                            if (pairs) {
+                                *reinterpret_cast<float2*>(o) = make_float2(x[0], x[1]);
+                                *reinterpret_cast<float2*>(o + 8) = make_float2(x[4], x[5]);
                             } else {
-#pragma unroll
-                                for (int j = 0; j < 16; ++j) o[j] = v[j];
+                                o[0] = x[0]; o[1] = x[1]; o[8] = x[4]; o[9] = x[5];
                             }
                         }
                     }
