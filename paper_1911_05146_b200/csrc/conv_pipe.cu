@@ -31,6 +31,7 @@
 #include "tc_ptx.cuh"
 
 #include <algorithm>
+#include <math.h>
 #include <string.h>
 #include <type_traits>
 
@@ -1283,45 +1284,67 @@ __global__ void __launch_bounds__(kPipeThreads, 1) conv_pipe_cell_kernel(const _
     if (warp_index() == 0) tmem_dealloc(tmem_base, cp.tmem_cols);
 }
 
-// Statistics for a BN that runs a kernel of its own although its input came from a convolution that left moments (the formulas
-// of merge_moments).  A block takes 128 channels with eight row lanes, grid (channels / 128, micro-batches): latency bound, so the
-// rows are spread (one block per micro-batch took 16 us at 1024 channels).
-__global__ void __launch_bounds__(256) bn_finalize_kernel(const float* __restrict__ partials, int rows, int C, double inv_rows, float eps, float* stats)
+// A BN that no convolution applies, from the moments the producing convolution left: every block merges them (merge_moments, the same
+// bits in each) and normalises its rows, one launch and one reading of x instead of a launch for the statistics and one for
+// the rest.  sum, act: the residual sum and the ReLU that follow a plain BN in a post-activation block, sum = y + add, act = max(sum, 0),
+// two launches and three trips through memory less.  Bound by memory; grid (blocks, micro-batches).
+constexpr int kMergeThreads = 256;
+struct BnMergeApply {
+    const float *partials, *gamma, *beta;
+    float* stats;
+    const float4 *x, *add;
+    float4 *y, *sum, *act;       // add, sum, act: null without
+    int units, C;
+    double inv_rows;
+    float eps, floor;
+    long long n4, per_block, ms4;   // float4 of a micro-batch, of a block; between micro-batches
+};
+__global__ void __launch_bounds__(kMergeThreads) bn_merge_apply_kernel(const BnMergeApply a)
 {
-    __shared__ float4 red[3][8][32];
-    __shared__ float4 refs[32];
+    extern __shared__ float tab[];                    // mean, rstd
+    __shared__ float4 red[4 * kMergeThreads];
     pdl_launch_dependents();
     pdl_wait();
-    const int t = threadIdx.x, lane = t & 31, ln = t >> 5, c4n = C >> 2, col = blockIdx.x * 32 + lane;
-    partials += (size_t)blockIdx.y * partial_floats(rows, C); stats += (size_t)blockIdx.y * 2 * C;
-    const float* counts = partials + (size_t)rows * 2 * C;
-    float4 sd = make_float4(0.f, 0.f, 0.f, 0.f), sq = sd, m2 = sd, ref = sd;
-    if (col < c4n) {
-        ref = __ldcg(reinterpret_cast<const float4*>(partials) + col);
-#pragma unroll 4
-        for (int k = ln; k < rows; k += 8) {
-            const float4* row = reinterpret_cast<const float4*>(partials + (size_t)k * 2 * C);
-            const float n = __ldcg(counts + k);
-            const float4 d = sub4(__ldcg(row + col), ref), nd = mul4(make_float4(n, n, n, n), d);
-            sd = add4(sd, nd);
-            sq = fma4(nd, d, sq);
-            m2 = add4(m2, __ldcg(row + c4n + col));
-        }
-    }
-    red[0][ln][lane] = sd; red[1][ln][lane] = sq; red[2][ln][lane] = m2;
-    if (ln == 0) refs[lane] = ref;
+    const int t = threadIdx.x, C = a.C, c4n = C >> 2;
+    const float* partials = a.partials + (size_t)blockIdx.y * partial_floats(a.units, C);
+    merge_moments<kMergeThreads>(partials, partials + (size_t)a.units * 2 * C, a.units, c4n, C, a.inv_rows, a.eps, tab, red, t);
     __syncthreads();
-    const int c = blockIdx.x * 128 + t;
-    if (t >= 128 || c >= C) return;
-    const float* r = reinterpret_cast<const float*>(&red[0][0][0]) + t;
-    float d = 0.f, q = 0.f, v = 0.f;
+    if (blockIdx.x == 0)
+        for (int i = t; i < 2 * C; i += kMergeThreads) a.stats[(size_t)blockIdx.y * 2 * C + i] = tab[i];
+    const long long first = blockIdx.x * a.per_block + t, end = (blockIdx.x + 1) * a.per_block < a.n4 ? (blockIdx.x + 1) * a.per_block : a.n4;
+    const long long ms = blockIdx.y * a.ms4;
+    int col = (int)(first % c4n);
+    const int step = kMergeThreads % c4n;             // 0: a thread keeps its channels
+    const float4 *mean4 = reinterpret_cast<const float4*>(tab), *rstd4 = mean4 + c4n;
+    float4 mu = mean4[col], rs = rstd4[col], g = __ldg(reinterpret_cast<const float4*>(a.gamma) + col), b = __ldg(reinterpret_cast<const float4*>(a.beta) + col);
+#pragma unroll 1
+    for (long long i = first; i < end; i += 4 * kMergeThreads) {
+        float4 v[4], e[4];
 #pragma unroll
-    for (int l = 0; l < 8; ++l) { d += r[128 * l]; q += r[128 * (8 + l)]; v += r[128 * (16 + l)]; }
-    const double dm = (double)d * inv_rows;
-    double var = ((double)v + (double)q) * inv_rows - dm * dm;
-    if (var < 0.0) var = 0.0;
-    stats[c] = (float)((double)reinterpret_cast<const float*>(refs)[t] + dm);
-    stats[C + c] = 1.0f / sqrtf((float)(var + (double)eps));
+        for (int j = 0; j < 4; ++j)
+            if (i + j * kMergeThreads < end) {
+                v[j] = __ldcg(a.x + ms + i + j * kMergeThreads);
+                if (a.add) e[j] = __ldcg(a.add + ms + i + j * kMergeThreads);
+            }
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (i + j * kMergeThreads < end) {
+                const long long at = ms + i + j * kMergeThreads;
+                float4 z = fma4(g, mul4(sub4(v[j], mu), rs), b);
+                z = make_float4(fmaxf(z.x, a.floor), fmaxf(z.y, a.floor), fmaxf(z.z, a.floor), fmaxf(z.w, a.floor));
+                a.y[at] = z;
+                if (a.add) {
+                    z = add4(z, e[j]);
+                    a.sum[at] = z;
+                    if (a.act) a.act[at] = make_float4(fmaxf(z.x, 0.f), fmaxf(z.y, 0.f), fmaxf(z.z, 0.f), fmaxf(z.w, 0.f));
+                }
+                if (step) {
+                    col += step;
+                    if (col >= c4n) col -= c4n;
+                    mu = mean4[col]; rs = rstd4[col]; g = __ldg(reinterpret_cast<const float4*>(a.gamma) + col); b = __ldg(reinterpret_cast<const float4*>(a.beta) + col);
+                }
+            }
+    }
 }
 
 // Forward pass, or the data gradient seen as a forward problem.
@@ -1738,10 +1761,23 @@ cudaError_t conv_pipe_cell_launch(const void* d_ops, int n_ops, int m_first, int
     return cudaGetLastError();
 }
 
-cudaError_t bn_finalize_partials(const float* partials, int units, int C, float eps, double rows, float* stats, int m_count, cudaStream_t st,
-                                 int64_t* n_launch)
+cudaError_t bn_merge_apply(const float* partials, int units, const float* gamma, const float* beta, float eps, bool relu, const float* x, float* y, const float* add,
+                           float* sum, float* act, float* stats, long long rows, int C, int m_count, cudaStream_t st, int64_t* n_launch)
 {
-    launch_pdl(bn_finalize_kernel, dim3((C + 127) / 128, m_count), dim3(256), 0, st, partials, units, C, 1.0 / rows, eps, stats);
+    BnMergeApply a{};
+    a.partials = partials; a.gamma = gamma; a.beta = beta; a.stats = stats; a.units = units; a.C = C;
+    a.x = reinterpret_cast<const float4*>(x); a.add = reinterpret_cast<const float4*>(add);
+    a.y = reinterpret_cast<float4*>(y); a.sum = reinterpret_cast<float4*>(sum); a.act = reinterpret_cast<float4*>(act);
+    a.inv_rows = 1.0 / (double)rows; a.eps = eps; a.floor = relu ? 0.f : -INFINITY;
+    a.n4 = a.ms4 = rows * C / 4;
+    // Every block merges the moments first: eight float4 a thread at least, twice as much of the tensor as of moments, four blocks an SM
+    // at most.
+    long long blocks = (a.n4 + 8 * kMergeThreads - 1) / (8 * kMergeThreads), most = 4 * kPlanSms / m_count, share = a.n4 / ((long long)units * C);
+    if (blocks > share) blocks = share;
+    if (blocks > most) blocks = most;
+    if (blocks < 1) blocks = 1;
+    a.per_block = (a.n4 + blocks - 1) / blocks;
+    launch_pdl(bn_merge_apply_kernel, dim3((unsigned int)((a.n4 + a.per_block - 1) / a.per_block), m_count), dim3(kMergeThreads), (size_t)2 * C * sizeof(float), st, a);
     if (n_launch) ++*n_launch;
     return cudaGetLastError();
 }

@@ -89,8 +89,9 @@ int conv_pipe_cell_max_ctas();
 cudaError_t conv_pipe_cell_launch(const void* d_ops, int n_ops, int m_first, int m_count, int ctas, unsigned int smem, unsigned int tmem_cols,
                                   unsigned int* d_barrier, DeviceStatus* status, cudaStream_t st, int64_t* n_launch);
 
-// mean[C], rstd[C] of m_count micro-batches from the partial moments a forward kernel left (for a BN that runs its own kernel).
-cudaError_t bn_finalize_partials(const float* partials, int units, int C, float eps, double rows, float* stats, int m_count, cudaStream_t st,
-                                 int64_t* n_launch);
+// y = BN(x) (+ ReLU) and the statistics of m_count micro-batches of `rows` rows, which follow one another, from the partial moments a
+// forward kernel left; with add: sum = y + add and, unless null, act = max(sum, 0) beside it.
+cudaError_t bn_merge_apply(const float* partials, int units, const float* gamma, const float* beta, float eps, bool relu, const float* x, float* y, const float* add,
+                           float* sum, float* act, float* stats, long long rows, int C, int m_count, cudaStream_t st, int64_t* n_launch);
 
 }  // namespace hpf

@@ -135,15 +135,12 @@ struct BnClusterScope {
 cudaError_t relu_fwd(const float* x, float* y, int64_t n, cudaStream_t st, int64_t* n_launch);
 cudaError_t relu_bwd(const float* x, const float* dy, float* dx, const float* addend, bool accumulate, int64_t n, cudaStream_t st,
                      int64_t* n_launch);
-// The forward's second half alone: the statistics (mean[C], rstd[C]) were left by the convolution kernel that produced x.
 // Whether the backward of a BN of this size is one launch of clusters that keep their rows in registers.
 bool bn_bwd_is_one_launch(int64_t rows, int C);
 // dx, dgamma, dbeta from sums of dz and dz * xhat that the kernel which wrote dy left: n_sums rows of [2][C], sums_ms floats between micro-batches
 cudaError_t bnrelu_bwd_apply(const float* x, const float* dy, const float* gamma, const float* beta, const float* stats, const float* sums, int n_sums,
                              int64_t sums_ms, float* dx, const float* addend, bool accumulate, float* dgamma, float* dbeta, int64_t rows, int C,
                              cudaStream_t st, int64_t* n_launch, const BnGroup& grp = BnGroup());
-cudaError_t bnrelu_fwd_apply(const float* x, const float* gamma, const float* beta, const float* stats, float* y,
-                             int64_t rows, int C, cudaStream_t st, int64_t* n_launch, const BnGroup& grp = BnGroup());
 cudaError_t add_fwd(const float* a, const float* b, float* out, int64_t n, cudaStream_t st, int64_t* n_launch);
 // dst (+)= src
 cudaError_t grad_accumulate(float* dst, const float* src, int64_t n, bool accumulate, cudaStream_t st, int64_t* n_launch);

@@ -99,6 +99,7 @@ struct hpf_model {
         std::vector<int> bn_fwd_from, conv_fwd_bn;  // BN -> conv whose forward kernel also produces the statistics of the BN (its input), or -1, and the inverse map
         std::vector<int> bn_into, conv_in_bn;       // BN -> the convolution that applies it to its own input operand (no BN kernel), and the inverse
         std::vector<int> bn_bwd_from, conv_bwd_bn;  // BN+ReLU -> the convolution whose data gradient also forms the sums of its backward, or -1, and the inverse map
+        std::vector<char> bn_tail;                  // BN -> ops behind it that its kernel does as well: 1 the residual sum, 2 and the ReLU after it
         std::vector<char> use_pipe[2];
         std::vector<ConvPipeGeom> pipe_geom[2];     // conv -> split of its forward / data-gradient launches
         std::vector<ConvPipePlan> pipe_plan[2];
@@ -208,6 +209,7 @@ struct hpf_model {
     float* grad(int op, int m) const { return reinterpret_cast<float*>(ws + grad_off[op]) + m * tensor_stride[op]; }
     float* stats(int op, int m) const { return reinterpret_cast<float*>(ws + stats_off[op]) + (int64_t)m * 2 * ops[op].C; }
     float* moments(int bn) const { return reinterpret_cast<float*>(ws + bn_moments_off[bn]); }
+    int64_t tensor_stride_of(int op) const { const int64_t e = numel(op); return e % 16 == 0 ? e : (e + 63) / 64 * 64; }      // whole micro-batches side by side: one launch, one tensor map
     bool contiguous(int op) const { return op < 0 || tensor_stride[op] == numel(op); }
     unsigned long long* cell_time_slot(int phase, int p, int m) const
     {
@@ -460,10 +462,11 @@ void build_kernel_plan(hpf_model* mdl, hpf_model::KernelPlan* kp)
     kp->conv_fwd_bn.assign(n, -1);
     kp->bn_into.assign(n, -1); kp->conv_in_bn.assign(n, -1);
     kp->bn_bwd_from.assign(n, -1); kp->conv_bwd_bn.assign(n, -1);
+    kp->bn_tail.assign(n, 0);
     if (!(mdl->opt_fuse_bn & 1)) return;
     for (int j = 0; j < n; ++j) {
         const OpInfo& bn = mdl->ops[j];
-        if (bn.op.kind != HPF_OP_BNRELU) continue;
+        if (bn.op.kind != HPF_OP_BNRELU && bn.op.kind != HPF_OP_BN) continue;
         if (bn.consumers.size() == 1 && bn_sums_wanted(mdl, kp, j)) {
             const int i = bn.consumers[0];
             const OpInfo& c = mdl->ops[i];
@@ -483,6 +486,16 @@ void build_kernel_plan(hpf_model* mdl, hpf_model::KernelPlan* kp)
             if (!(mdl->ops[k].op.kind == HPF_OP_ADD && mdl->add_done_by[k] >= 0)) adjacent = false;
         if (!adjacent) continue;
         kp->bn_fwd_from[j] = prod; kp->conv_fwd_bn[prod] = j;
+        if (bn.op.kind == HPF_OP_BN) {
+            // the end of a post-activation block: the sum with an earlier tensor of the BN's result, which nothing else reads, and its ReLU
+            const bool whole = mdl->tensor_stride_of(j) == mdl->numel(j);
+            if (whole && bn.consumers.size() == 1 && bn.consumers[0] == j + 1 && mdl->ops[j + 1].op.kind == HPF_OP_ADD && mdl->add_done_by[j + 1] < 0 &&
+                mdl->ops[j + 1].op.src0 != mdl->ops[j + 1].op.src1 && mdl->ops[j + 1].part == bn.part) {
+                kp->bn_tail[j] = 1;
+                if (j + 2 < n && mdl->ops[j + 2].op.kind == HPF_OP_RELU && mdl->ops[j + 2].op.src0 == j + 1 && mdl->ops[j + 2].part == bn.part) kp->bn_tail[j] = 2;
+            }
+            continue;
+        }
         // the BN+ReLU itself: applied by its only reader, the next op, a stride-1 tensor-core convolution
         if ((mdl->opt_fuse_bn & 2) && bn.consumers.size() == 1 && bn.consumers[0] == j + 1) {
             const int i = j + 1;
@@ -605,8 +618,7 @@ void build_memory_plan(hpf_model* mdl)
     }
     mdl->act_off.assign(n, 0); mdl->grad_off.assign(n, 0); mdl->stats_off.assign(n, 0); mdl->tensor_stride.assign(n, 0);
     for (int i = 0; i < n; ++i) {
-        const int64_t e = mdl->numel(i);
-        mdl->tensor_stride[i] = e % 16 == 0 ? e : (e + 63) / 64 * 64;       // whole micro-batches side by side: one launch, one tensor map
+        mdl->tensor_stride[i] = mdl->tensor_stride_of(i);
     }
     for (int i = n - 1; i >= 0; --i) {
         const int f = mdl->fused_into[i], a = mdl->grad_alias[i];              // f, a > i: already placed
@@ -641,11 +653,12 @@ bool op_uses_tc(hpf_model* mdl, hpf_model::KernelPlan* k, int i, int pass)
     const ConvShape s = conv_shape_of(mdl, i);
     // what may ride in the launch (what does is decided with the plans at hand)
     auto is_bn = [&](int op) { return mdl->ops[op].op.kind == HPF_OP_BNRELU; };
+    auto is_plain_bn = [&](int op) { return mdl->ops[op].op.kind == HPF_OP_BN; };
     ConvPipeUse use;
     if (pass == PASS_FWD) {
         const int out = mdl->fused_into[i] >= 0 ? mdl->fused_into[i] : i;
         use.addend = out != i;
-        for (int c : mdl->ops[out].consumers) use.moments = use.moments || is_bn(c);
+        for (int c : mdl->ops[out].consumers) use.moments = use.moments || is_bn(c) || is_plain_bn(c);
         use.bn_in = is_bn(mdl->ops[i].op.src0) && conv_pipe_can_fuse_bn_input(s);
     } else {
         use.moments = mdl->ops[i].op.stride == 1 && (mdl->opt_fuse_bn & 1) && bn_sums_wanted(mdl, k, mdl->ops[i].op.src0);
@@ -818,24 +831,26 @@ int forward_op(hpf_model* mdl, const hpf_model::KernelPlan& kp, int i, int m, in
         break;
     }
     case HPF_OP_BNRELU:
+    case HPF_OP_BN:                        // batch normalisation without the activation
         if (kp.bn_into[i] >= 0) break;   // the convolution that reads this BN applies it (and stores `out` and the statistics)
         if (kp.bn_fwd_from[i] >= 0) {    // the producing convolution left the moments of its units
-            const int units = kp.pipe_geom[PASS_FWD][kp.bn_fwd_from[i]].blocks_per_m;
-            CU(bn_finalize_partials(mdl->moments(i) + (size_t)m * conv_pipe_partial_floats(units, o.C), units, o.C, q.eps, (double)rows, mdl->stats(i, m), g, st,
-                                    &mdl->launches));
-            CU(bnrelu_fwd_apply(in0, mdl->params + o.w_off, mdl->params + o.b_off, mdl->stats(i, m), out, rows, o.C, st, &mdl->launches, grp));
+            const int units = kp.pipe_geom[PASS_FWD][kp.bn_fwd_from[i]].blocks_per_m, tail = kp.bn_tail[i];
+            const float* add = nullptr;
+            if (tail > 0) { const hpf_op& sum = mdl->ops[i + 1].op; add = mdl->act(sum.src0 == i ? sum.src1 : sum.src0, m); }
+            CU(bn_merge_apply(mdl->moments(i) + (size_t)m * conv_pipe_partial_floats(units, o.C), units, mdl->params + o.w_off, mdl->params + o.b_off, q.eps,
+                              q.kind == HPF_OP_BNRELU, in0, out, add, tail > 0 ? mdl->act(i + 1, m) : nullptr, tail > 1 ? mdl->act(i + 2, m) : nullptr, mdl->stats(i, m),
+                              rows, o.C, g, st, &mdl->launches));
         } else {
-            CU(bnrelu_fwd(in0, mdl->params + o.w_off, mdl->params + o.b_off, q.eps, out, mdl->stats(i, m), rows, o.C, bn_scratch, st, &mdl->launches, true, grp));
+            CU(bnrelu_fwd(in0, mdl->params + o.w_off, mdl->params + o.b_off, q.eps, out, mdl->stats(i, m), rows, o.C, bn_scratch, st, &mdl->launches,
+                          q.kind == HPF_OP_BNRELU, grp));
         }
         break;
-    case HPF_OP_BN:                        // batch normalisation without the activation
-        CU(bnrelu_fwd(in0, mdl->params + o.w_off, mdl->params + o.b_off, q.eps, out, mdl->stats(i, m), rows, o.C, bn_scratch, st, &mdl->launches, false, grp));
-        break;
     case HPF_OP_RELU:
+        if (i >= 2 && kp.bn_tail[i - 2] > 1) break;      // (done with the BN two ops before)
         CU(relu_fwd(in0, out, mdl->numel(i) * g, st, &mdl->launches));
         break;
     case HPF_OP_ADD:
-        if (mdl->add_done_by[i] < 0) CU(add_fwd(in0, mdl->act(q.src1, m), out, mdl->numel(i) * g, st, &mdl->launches));
+        if (mdl->add_done_by[i] < 0 && !(i >= 1 && kp.bn_tail[i - 1] > 0)) CU(add_fwd(in0, mdl->act(q.src1, m), out, mdl->numel(i) * g, st, &mdl->launches));
         break;
     case HPF_OP_MAXPOOL:
         CU(maxpool_fwd(in0, out, gs, st, &mdl->launches));

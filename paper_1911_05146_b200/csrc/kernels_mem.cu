@@ -1976,16 +1976,6 @@ cudaError_t bnrelu_bwd_apply(const float* x, const float* dy, const float* gamma
     return cudaGetLastError();
 }
 
-cudaError_t bnrelu_fwd_apply(const float* x, const float* gamma, const float* beta, const float* stats, float* y,
-                             int64_t rows, int C, cudaStream_t st, int64_t* n_launch, const BnGroup& grp)
-{
-    const BnPlan p = bn_plan(rows, C);
-    launch_pdl(bn_apply_fwd_kernel, dim3(p.nblk_apply, grp.count), kBnThreads, 0, st, reinterpret_cast<const float4*>(x), gamma, beta, stats,
-               reinterpret_cast<float4*>(y), rows, C, p.cgt, p.rl, p.passes, p.rows_per_blk_apply, 0.f, grp);
-    count(n_launch, 1);
-    return cudaGetLastError();
-}
-
 cudaError_t relu_fwd(const float* x, float* y, int64_t n, cudaStream_t st, int64_t* n_launch)
 {
     launch_pdl(relu_fwd_kernel, ew_blocks(n / 4 + 1), kThreads, 0, st, x, y, n);
