@@ -204,13 +204,13 @@ __device__ __forceinline__ float4 lo_part(float4 v) { return sub4(v, make_float4
 // (every CTA of a launch gets the same bits), fp32 terms, the last combination in fp64.  THREADS threads, which share named
 // barrier 1; tab: mean[C], rstd[C]; red: 4 x THREADS float4.  First every thread adds its rows of four channels, then one
 // thread per channel combines: what this costs is latency and instruction fetches, so nothing is unrolled that need not be.
-// counts: the rows' n; second: float4 from a row's means to its M2 (a dry round reads other memory in their place).
 template <int THREADS>
-__device__ __forceinline__ void merge_moments(const float* partials, const float* counts, int rows, int second, int C, double inv_rows, float eps, float* tab, float4* red, int tid)
+__device__ __forceinline__ void merge_moments(const float* partials, int rows, int C, double inv_rows, float eps, float* tab, float4* red, int tid)
 {
+    const float* counts = partials + (size_t)rows * 2 * C;
     const int c4n = C >> 2;
     const int L = c4n <= THREADS ? THREADS / c4n : 1;
-    constexpr int kRows = 6;                          // rows in flight: 37 of 64 channels, 18 of 128 in one round trip
+    constexpr int kRows = 4;                          // rows in flight (six: no faster)
 #pragma unroll 1
     for (int c0 = 0; c0 < c4n; c0 += THREADS) {
         const int width = c4n - c0 < THREADS ? c4n - c0 : THREADS;       // float4 columns of this pass
@@ -230,7 +230,7 @@ __device__ __forceinline__ void merge_moments(const float* partials, const float
                     const float4* row = reinterpret_cast<const float4*>(partials + (size_t)(have ? k : 0) * 2 * C);
                     n[j] = have ? __ldcg(counts + k) : 0.f;
                     a[j] = __ldcg(row + col);
-                    b[j] = have ? __ldcg(row + second + col) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    b[j] = have ? __ldcg(row + c4n + col) : make_float4(0.f, 0.f, 0.f, 0.f);
                 }
 #pragma unroll
                 for (int j = 0; j < kRows; ++j) {
@@ -988,6 +988,7 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
         const int row_step = 8 * wpg;
         const int cph = lane & 3, r8 = ((lane >> 2) & 1) * 4 + (lane >> 3), row0 = gw * 8 + r8;
         const uint32_t at_hi = (uint32_t)row0 * 128u + (uint32_t)((cph ^ r8) << 4), at_lo = (uint32_t)row0 * 128u + (uint32_t)(((cph + 4) ^ r8) << 4);
+        const uint32_t byte_step = (uint32_t)row_step * 128u;
         const int S = p.a_stages, C = p.c_in, halo = p.halo;
         const bool three = p.three != 0;
         float* tab = reinterpret_cast<float*>(smem + p.off_bn);
@@ -1004,38 +1005,35 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
         const bool store_y = BN_IN && slice == 0;
         bool ok = true;
         UnitWalk cu = u0;
-        // The first round is a dry one (see write_out): one row to merge (parameters in place of moments, which the preceding kernel
-        // may still write), one row a thread, in the scratch of the merge.
-        bool dry = BN_IN;
+        // (No dry round here: the merge and the first block are bound by their own latencies, and what the round costs in conditions made
+        // ResNet-110 5.46 -> 5.59 ms, scoring ResNet-182 6.03 -> 6.29.)
+        if (BN_IN && !CELL) pdl_wait();
 #pragma unroll 1
-        while (cu.left > 0) {
-            const int kb = cu.kb(p), ke = dry ? kb + ahead + 1 : cu.ke(p);
+        for (; cu.left > 0; cu.next(p)) {
+            const int kb = cu.kb(p), ke = cu.ke(p);
             const Span sp = span_of(p, cu);
-            const int own_lo = sp.lead + halo, own_hi = own_lo + cu.tiles(p) * kTileM, valid = p.pos_per_m - sp.pos0, n_rows = dry ? 1 : sp.rows;
+            const int own_lo = sp.lead + halo, own_hi = own_lo + cu.tiles(p) * kTileM, valid = p.pos_per_m - sp.pos0;
             if (BN_IN) {
-                if (dry || cu.m != cur_m) {
-                    if (!dry) cur_m = cu.m;
+                if (cu.m != cur_m) {
+                    cur_m = cu.m;
                     split_sync();                     // everybody is done with the table of the micro-batch before
-                    const float* const rows0 = dry ? p.bn_gamma : p.bn_partials + (size_t)cu.m * partial_floats(p.bn_units, C);
-                    merge_moments<kSplitThreads>(rows0, dry ? p.bn_gamma : rows0 + (size_t)p.bn_units * 2 * C, dry ? 1 : p.bn_units, dry ? 0 : C >> 2, C, p.bn_inv_rows, p.bn_eps, tab,
-                                  reinterpret_cast<float4*>(smem + p.off_red), tid);
+                    const float* const rows0 = p.bn_partials + (size_t)cur_m * partial_floats(p.bn_units, C);
+                    merge_moments<kSplitThreads>(rows0, p.bn_units, C, p.bn_inv_rows, p.bn_eps, tab, reinterpret_cast<float4*>(smem + p.off_red), tid);
                     split_sync();
                 }
-                if (!dry && slice == 0 && cu.ul == 0 && cu.z == 0)
+                if (slice == 0 && cu.ul == 0 && cu.z == 0)
 #pragma unroll 1
                     for (int i = tid; i < 2 * C; i += kSplitThreads) p.bn_stats[(size_t)cur_m * 2 * C + i] = tab[i];
             }
 #pragma unroll 1
             for (int c = kb + ahead; c < ke; c += groups) {
                 {
-                    if (!dry) ok = mbar_wait(a_raw + 8 * s, par, &abort_flag) && ok;
+                    ok = mbar_wait(a_raw + 8 * s, par, &abort_flag) && ok;
                     // (after a wait that gave up the warps run through the rest without waiting: they still have to meet at
                     // the named barriers)
                     if (!ok && lane == 0) report(p.status, 26);
-                    // (dry: every row step of the one batch at the same place, in the merge's scratch)
-                    uint8_t* const stage = smem + (dry ? p.off_red : (uint32_t)s * p.a_stage_bytes);
-                    uint8_t *hi = stage + (dry ? 16 * lane : at_hi), *lo = stage + (dry ? 16 * lane : at_lo);
-                    const uint32_t byte_step = dry ? 0u : (uint32_t)row_step * 128u;
+                    uint8_t* hi = smem + (uint32_t)s * p.a_stage_bytes + at_hi;
+                    uint8_t* lo = smem + (uint32_t)s * p.a_stage_bytes + at_lo;
                     if (BN_IN) {
                         const int ch = 16 * c + 4 * cph;
                         const float4 mu = *reinterpret_cast<const float4*>(tab + ch), rs = *reinterpret_cast<const float4*>(tab + C + ch);
@@ -1052,7 +1050,7 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
                         }
                         // four rows in flight; the block is allocated in whole batches, so the last one needs no bounds
 #pragma unroll 1
-                        for (int row = dry ? 0 : row0; row < n_rows; row += kRowBatch * row_step, hi += kRowBatch * byte_step, lo += kRowBatch * byte_step) {
+                        for (int row = row0; row < sp.rows; row += kRowBatch * row_step, hi += kRowBatch * byte_step, lo += kRowBatch * byte_step) {
                             float4 v[kRowBatch];
 #pragma unroll
                             for (int j = 0; j < kRowBatch; ++j) v[j] = *reinterpret_cast<const float4*>(hi + byte_step * j);
@@ -1062,12 +1060,11 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
                             for (int j = 0; j < kRowBatch; ++j) {
                                 const int r = row + row_step * j;
                                 if (FLAT) {
-                                    inside[j] = r < valid;
-                                    own[j] = inside[j] && !dry;
+                                    inside[j] = own[j] = r < valid;
                                     off[j] = yo; yo += row_step * C;
                                 } else {
                                     inside[j] = px < p.W && py < p.Hv && pn >= 0 && r < valid;
-                                    own[j] = inside[j] && r >= own_lo && r < own_hi && !dry;
+                                    own[j] = inside[j] && r >= own_lo && r < own_hi;
                                     off[j] = pn * p.in_sn + py * p.in_sh + px * p.in_sw;
                                     px += dx; py += dy; pn += dn;
                                     if (px >= p.Wp) { px -= p.Wp; ++py; }
@@ -1092,7 +1089,7 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
                         }
                     } else if (three) {
 #pragma unroll 1
-                        for (int row = dry ? 0 : row0; row < n_rows; row += kRowBatch * row_step, hi += kRowBatch * byte_step, lo += kRowBatch * byte_step) {
+                        for (int row = row0; row < sp.rows; row += kRowBatch * row_step, hi += kRowBatch * byte_step, lo += kRowBatch * byte_step) {
                             float4 v[kRowBatch];
 #pragma unroll
                             for (int j = 0; j < kRowBatch; ++j) v[j] = *reinterpret_cast<const float4*>(hi + byte_step * j);
@@ -1104,20 +1101,13 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
                     }
                     fence_async_smem();               // generic-proxy writes -> tensor-core reads
                     __syncwarp();
-                    if (dry) break;
                     if (lane == 0) mbar_arrive(a_full + 8 * s);
                 }
                 s += groups;
                 if (s >= S) { s -= S; par ^= 1u; }
                 ahead += groups;
             }
-            if (dry) {
-                dry = false;
-                if (!CELL) pdl_wait();
-                continue;
-            }
             ahead -= ke - kb;
-            cu.next(p);
         }
     } else if (warp >= kFirstSplit + kSplitWarps) {
         write_out<W, FLAT, BNB, CELL>(p, sh, smem, tmem_base, acc_full, acc_empty, u0, slice);
@@ -1307,7 +1297,7 @@ __global__ void __launch_bounds__(kMergeThreads) bn_merge_apply_kernel(const BnM
     pdl_wait();
     const int t = threadIdx.x, C = a.C, c4n = C >> 2;
     const float* partials = a.partials + (size_t)blockIdx.y * partial_floats(a.units, C);
-    merge_moments<kMergeThreads>(partials, partials + (size_t)a.units * 2 * C, a.units, c4n, C, a.inv_rows, a.eps, tab, red, t);
+    merge_moments<kMergeThreads>(partials, a.units, C, a.inv_rows, a.eps, tab, red, t);
     __syncthreads();
     if (blockIdx.x == 0)
         for (int i = t; i < 2 * C; i += kMergeThreads) a.stats[(size_t)blockIdx.y * 2 * C + i] = tab[i];
