@@ -43,7 +43,7 @@ constexpr int kSplitWarps = 4, kEpiWarps = 8;
 constexpr int kFirstSplit = 4;                        // warps 0..2: operand copies, weight copies, MMAs; 3 idle
 constexpr int kSplitThreads = 32 * kSplitWarps, kRowStep = 8 * kSplitWarps;
 constexpr int kPipeThreads = 32 * (kFirstSplit + kSplitWarps + kEpiWarps);
-constexpr int kMaxBlockRows = 768, kRowBatch = 4;     // operand rows of a block at most; rows a splitter thread has in flight
+constexpr int kMaxBlockRows = 768, kRowBatch = 2;     // operand rows of a block at most; rows a splitter thread has in flight (code counts: 1 / 2 / 4 / 8: ResNet-110 5.47 / 5.44 / 5.46 / 5.59 ms)
 constexpr uint32_t kPipeSmem = 222 * 1024;            // dynamic shared memory of a CTA
 constexpr int kMaxA = 8, kMaxB = 8;
 
@@ -1048,7 +1048,7 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
                             pn += q; pos -= q * p.img_pos;
                             py = div_magic(pos, p.Wp, p.magic_w); px = pos - py * p.Wp;
                         }
-                        // four rows in flight; the block is allocated in whole batches, so the last one needs no bounds
+                        // two rows in flight; the block is allocated in whole batches, so the last one needs no bounds
 #pragma unroll 1
                         for (int row = row0; row < sp.rows; row += kRowBatch * row_step, hi += kRowBatch * byte_step, lo += kRowBatch * byte_step) {
                             float4 v[kRowBatch];
