@@ -1524,11 +1524,13 @@ static bool plan_geom(const ConvShape& s, int pass, int passes, int launched, Co
 bool conv_pipe_geom(const ConvShape& s, int pass, int passes, int launched, ConvPipeUse use, ConvPipeGeom* g)
 {
     struct Kept { int key[12]; bool used, ok; ConvPipeGeom g; };
-    constexpr int kKept = 64;
+    constexpr int kKept = 256;
     static thread_local Kept kept[kKept];
     const int key[12] = {s.N, s.H, s.W, s.C, s.K, s.R, s.stride, s.pad, pass, passes, launched, (use.addend ? 1 : 0) | (use.moments ? 2 : 0) | (use.bn_in ? 4 : 0)};
     unsigned int h = 2166136261u;
     for (int k : key) h = (h ^ (unsigned int)k) * 16777619u;
+    // (keys that differ in the last word only must not share a place: the convolutions of a block take turns)
+    h = (h ^ (h >> 15)) * 2246822519u;
     Kept& e = kept[(h >> 16) % kKept];
     if (!e.used || memcmp(e.key, key, sizeof key) != 0) {
         memcpy(e.key, key, sizeof key);
@@ -1623,6 +1625,8 @@ cudaError_t conv_pipe_prepare(ConvPipePlan* plan, const ConvShape& s, int pass, 
     ConvPipeLaunch* L = reinterpret_cast<ConvPipeLaunch*>(plan->storage);
     memset(L, 0, sizeof *L);
     const long long kdim = (long long)s.R * s.R * v.c_in;
+    // (16-byte copies and stores; a tensor map refuses other addresses itself)
+    if ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(out) | reinterpret_cast<uintptr_t>(extra)) & 15) return cudaErrorInvalidValue;
     // 32-byte pieces of a row where the buffers allow them (a caller's own may start at any 16 bytes)
     const uintptr_t at = reinterpret_cast<uintptr_t>(out) | reinterpret_cast<uintptr_t>(splitk) | (splitk_bytes & 31);
     const bool wide = g.n_chunk % 32 == 0 && at % 32 == 0;

@@ -1,6 +1,8 @@
 """Sizes at the edges of the kernels' tiles and of the rules that choose between them, against the oracle."""
 import pytest
+import torch
 
+import paper_1911_05146_b200 as hpf
 import workloads as wl
 from test_gpu_kernels import TOL_TENSOR, _conv_case
 from test_gpu_step import check_step
@@ -68,3 +70,47 @@ def test_batch_norm_backward_from_the_sums_of_the_data_gradient(batch):
     channels), the shortcut adds on the way; ragged last tiles."""
     ops = wl.resnet_v2_cifar(1, widths=(64,), outs=(64,))
     check_step(ops, (33, 33, 3), batch, 1, [5], seed=22, bn_jitter=0.2)
+
+
+@pytest.mark.parametrize("N,ks,st,ci,co,H", [
+    (75, 1, 1, 16, 256, 16),     # two slices of 128 channels, each of a lane's eight in two pieces of four
+    (38, 1, 1, 32, 16, 32),      # 16 channels forward, 32 the other way
+    (3, 3, 1, 64, 96, 9),        # padded grid, three groups of 32 channels
+    (2, 3, 1, 512, 512, 2),      # split over CTAs
+    (5, 1, 2, 64, 64, 15)], ids=str)      # zeros between the samples
+@pytest.mark.parametrize("path", [0, 2])
+def test_results_that_start_at_any_sixteen_bytes(N, ks, st, ci, co, H, path):
+    """The write-out stores 32 bytes a lane where the buffer allows it and 16 otherwise: the same bits."""
+    P, dev = (H - 1) // st + 1, "cuda:0"
+    g = torch.Generator(device=dev)
+    g.manual_seed(N)
+    x, dy = torch.randn(N, H, H, ci, generator=g, device=dev), torch.randn(N, P, P, co, generator=g, device=dev)
+    w = torch.randn(co, ks, ks, ci, generator=g, device=dev) * (2.0 / (ci * ks * ks)) ** 0.5
+    args = (N, H, H, ci, co, ks, st, ks // 2, path)
+    wprep, scratch = torch.empty(4 * w.numel(), device=dev), torch.zeros(hpf.conv_scratch_bytes(*args[:8]), dtype=torch.uint8, device=dev)
+    hpf.conv_prepare_weights(w, wprep, ci, co, ks)
+    out = []
+    for skip in (0, 4):
+        y, dx = (torch.full((t.numel() + 4,), float("nan"), device=dev)[skip:skip + t.numel()] for t in (dy, x))
+        hpf.conv_fwd(x, w, wprep, y, *args, scratch)
+        hpf.conv_dgrad(dy, w, wprep, dx, *args, scratch)
+        out.append((y, dx))
+    torch.cuda.synchronize()
+    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+    assert not torch.isnan(out[1][0]).any() and not torch.isnan(out[1][1]).any()
+
+
+@pytest.mark.parametrize("C,ks,size", [(48, 3, 9), (64, 1, 7), (1040, 1, 3)], ids=str)      # a lane's channels change from row to row; stay; more than a block's threads
+@pytest.mark.parametrize("cuts", [[], [2], [3], [4]], ids=str)
+def test_a_plain_batch_norm_ends_its_block(C, ks, size, cuts):
+    """BN, residual sum and ReLU in one launch, as far as they stand in one partition."""
+    ops = [wl.Op(wl.CONV, -1, -1, 3, C, 3, 1, 1, 0.0), wl.Op(wl.CONV, 0, -1, C, C, ks, 1, ks // 2, 0.0), wl.Op(wl.BN, 1, -1, C, C, 0, 1, 0, 1e-5),
+           wl.Op(wl.ADD, 2, 0, C, C, 0, 1, 0, 0.0), wl.Op(wl.RELU, 3, -1, C, C, 0, 1, 0, 0.0), wl.Op(wl.HEAD, 4, -1, C, 10, 0, 1, 0, 0.0)]
+    check_step(ops, (size, size, 3), 6, 3, cuts, seed=23, bn_jitter=0.2)
+
+
+def test_a_plain_batch_norm_and_its_sum_without_an_activation():
+    """(No BN may follow the sum: it would remove what the first one's shift adds, whose gradient would be zero plus rounding.)"""
+    ops = [wl.Op(wl.CONV, -1, -1, 3, 32, 3, 1, 1, 0.0), wl.Op(wl.CONV, 0, -1, 32, 32, 3, 1, 1, 0.0), wl.Op(wl.BN, 1, -1, 32, 32, 0, 1, 0, 1e-5),
+           wl.Op(wl.ADD, 0, 2, 32, 32, 0, 1, 0, 0.0), wl.Op(wl.HEAD, 3, -1, 32, 10, 0, 1, 0, 0.0)]
+    check_step(ops, (8, 8, 3), 4, 2, [], seed=24, bn_jitter=0.2)
