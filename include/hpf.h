@@ -121,7 +121,7 @@ int hpf_model_destroy(hpf_model *model);
  *                          but costs throughput once every stage is busy.  0: always late; a large N: always early.
  *                          Only launches of one micro-batch run many cells at once: with the default grouped launches two
  *                          cells at most are under way and N matters from 2 down.  0 against the default there: ResNet-11
- *                          0.328 / 0.334 ms, ResNet-110 6.28 / 6.24, ResNet-152 35.4 / 35.5, ResNet-1001 60.1 / 59.7.
+ *                          0.328 / 0.334 ms, ResNet-110 6.28 / 6.24, ResNet-152 35.4 / 35.5, ResNet-1001 60.1 / 59.7 (before the write-out was rewritten).
  *   HPF_OPT_STAGE_LANES    L (default 1): a stage keeps up to L of its micro-batches under way at once, micro-batch m on lane
  *                          m mod L, every lane with its own streams and scratch memory.  L = 1 is the schedule of Section 5.3
  *                          as the paper's one-process-per-partition runs it: a stage works through its micro-batches one
@@ -150,7 +150,7 @@ int hpf_model_destroy(hpf_model *model);
  *                          all partitions must fit the GPU together (hpf_bind: HPF_ERR_UNSUPPORTED otherwise).  Results
  *                          are bit-identical to N = 0.  0: one launch per convolution, and the faster one: a step with the
  *                          most CTAs that fit against the default, ResNet-11 0.50 / 0.33 ms, ResNet-110 9.4 (one partition) and
- *                          15.0 (four) / 6.2, ResNet-152 45.7 and 87.5 / 35.5, ResNet-1001 87 and 249 / 59.7. */
+ *                          15.0 (four) / 6.2, ResNet-152 45.7 and 87.5 / 35.5, ResNet-1001 87 and 249 / 59.7 (both from before the write-out was rewritten). */
 typedef enum { HPF_OPT_GRAPH = 1, HPF_OPT_CONV_PATH = 2, HPF_OPT_SINGLE_STREAM = 3, HPF_OPT_KEEP_MESSAGES = 4,
                HPF_OPT_FUSE_ADD = 5, HPF_OPT_PDL = 6, HPF_OPT_WGRAD_PASSES = 7, HPF_OPT_FUSE_BN = 8, HPF_OPT_CELL_TIMES = 9,
                HPF_OPT_BN_CLUSTER = 10, HPF_OPT_CELL_CTAS = 11, HPF_OPT_PDL_LATE_FROM = 12,

@@ -473,7 +473,7 @@ __device__ __forceinline__ void pipe_init_barriers(const PipeScalars& p, PipeSha
 // What a launch of a few microseconds pays here is the first execution of every instruction: 100-150 clocks per 128 bytes of
 // code, a first patch took 8600 clocks against 2400 of the following ones.  So there is one loop over patches (32 rows x
 // one group of channels), every part of which stands in the code once, and its first, dry round - no rows, nothing waited
-// for, nothing stored - runs ahead of the first accumulator.  Everything together: ResNet-110 5.96 -> 5.62 ms, ResNet-11 0.327 -> 0.299.
+// for, nothing stored; what it reads from tensor and shared memory is discarded - runs ahead of the first accumulator.  Everything together: ResNet-110 5.96 -> 5.62 ms, ResNet-11 0.327 -> 0.299.
 template <int W, bool FLAT, bool BNB, bool CELL>
 __device__ __forceinline__ void write_out(const PipeScalars& p, PipeShared& sh, uint8_t* smem, const uint32_t tmem_base,
                                           const uint32_t acc_full, const uint32_t acc_empty, const UnitWalk& u0, const int slice)

@@ -962,27 +962,33 @@ __global__ void __launch_bounds__(192) conv_tc_wgrad_direct_kernel(const __grid_
             float* obase = p.out + (long long)micro * p.out_ms + (long long)split * p.split_stride + (m0 + row0) * row_stride + cn0 + 2 * q;
             const bool pairs = (reinterpret_cast<uintptr_t>(obase) & 7u) == 0;      // (every other term is a whole number of 16-byte pieces)
             if (quad * 32 < p.m_chunk)                       // a whole warp of lanes beyond the chunk has nothing to read
+{
+                // W / 2 groups of eight columns a round: 32 columns where the slot is a multiple of them
+                auto write_out = [&](auto width) {
+                    constexpr int W = decltype(width)::value;
 #pragma unroll 1
-                for (int tp = 0; tp < ntaps; ++tp)
+                    for (int tp = 0; tp < ntaps; ++tp)
 #pragma unroll 1
-                    for (int c0 = 0; c0 < p.n_cols; c0 += 16) {
-                        float v[2][8];
-                        tmem_ld_rows<4>(lane_addr + (uint32_t)(tp * slot + c0), v[0]);
-                        tmem_ld_rows<4>(lane_addr + (16u << 16) + (uint32_t)(tp * slot + c0), v[1]);
-                        tmem_ld_wait();
-                        float* o = obase + (long long)(tap0 + tp) * p.c_in + c0;
+                        for (int c0 = 0; c0 < p.n_cols; c0 += 4 * W) {
+                            float v[2][2 * W];
+                            tmem_ld_rows<W>(lane_addr + (uint32_t)(tp * slot + c0), v[0]);
+                            tmem_ld_rows<W>(lane_addr + (16u << 16) + (uint32_t)(tp * slot + c0), v[1]);
+                            tmem_ld_wait();
+                            float* o = obase + (long long)(tap0 + tp) * p.c_in + c0;
 #pragma unroll
-                        for (int i = 0; i < 4; ++i, o += 8 * row_stride) {
-                            if (row0 + 8 * i >= p.m_chunk) continue;
-                            const float* x = &v[i >> 1][2 * (i & 1)];
-                            if (pairs) {
-                                *reinterpret_cast<float2*>(o) = make_float2(x[0], x[1]);
-                                *reinterpret_cast<float2*>(o + 8) = make_float2(x[4], x[5]);
-                            } else {
-                                o[0] = x[0]; o[1] = x[1]; o[8] = x[4]; o[9] = x[5];
+                            for (int i = 0; i < 4; ++i, o += 8 * row_stride) {
+                                if (row0 + 8 * i >= p.m_chunk) continue;
+                                const float* x = &v[i >> 1][2 * (i & 1)];
+#pragma unroll
+                                for (int c = 0; c < W / 2; ++c) {
+                                    if (pairs) *reinterpret_cast<float2*>(o + 8 * c) = make_float2(x[4 * c], x[4 * c + 1]);
+                                    else { o[8 * c] = x[4 * c]; o[8 * c + 1] = x[4 * c + 1]; }
+                                }
                             }
                         }
-                    }
+                };
+                if (p.n_cols % 32 == 0) write_out(std::integral_constant<int, 8>()); else write_out(std::integral_constant<int, 4>());
+            }
         }
     }
 
@@ -1438,7 +1444,9 @@ int unfused_n_chunk(int c_out, int tiles)
 // Measured on 136 drawn 1x1 shapes both ways (16..512 channels, maps of 4..56, batch 4..128, one and three passes, calls back to
 // back): inside the line 0.61 of the pipelined launch's time (geometric mean of 189, one of them above 1.05: 9.6 us against 8.8;
 // 512 -> 32 channels on 10 maps of 17 x 17 12 us against 29, 64 -> 16 on 16 maps of 32 x 32 5.0 against 9.1), outside 1.15
-// (83).  3x3 windows: 1.25 of its time (248).  For a 1x1 window both add the products in the same order.
+// (83).  3x3 windows: 1.25 of its time (248).  For a 1x1 window both add the products in the same order.  Since the pipelined kernel's
+// write-out and MMA issue were rewritten the line still holds but closely: 28 calls of 14 shapes inside it, 0.96 (512 -> 16 on 60
+// maps of 10 x 10 9.5 against 13.2 us, 16 -> 64 on 128 of 16 x 16 both 7.0, 256 -> 512 on 16 of 7 x 7 10.7 against 9.0).
 bool conv_tc_faster_alone(const ConvShape& s, int pass, int passes)
 {
     const long long tiles = ((long long)s.N * s.P * s.Q + kTileM - 1) / kTileM;
