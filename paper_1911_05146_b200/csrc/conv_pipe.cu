@@ -419,6 +419,11 @@ __device__ __forceinline__ void mma_role(const PipeScalars& p, const MmaEnv& e, 
         if (++buf == acc_bufs) { buf = 0; cpar ^= 1u; }
         *e.b_used = b_it; *e.a_used = a_it;
     }
+    // The late trigger.  Here, where a CTA has one last unit whatever its patches and sets of write-out warps are: tied to the write-out's
+    // walk it missed every launch with several patches a unit.  Ten launches in a row, late from the write-out where it could / now:
+    // 3x3 128 -> 128 @16, batch 128, 44.2 / 43.4 us, 1x1 128 -> 512 @28, batch 64, 47.1 / 45.0, 256 -> 64 @8, batch 128, dgrad 8.0 / 7.4, 64 -> 256 @56,
+    // batch 64, 72.8 / 70.7; the one slower one is 3x3 16 -> 16 @32 in one pass, 11.8 / 12.1.
+    if (!CELL && p.pdl_late) pdl_launch_dependents();
     if (CELL) {                  // wait until every barrier has seen its last arrival: they are used again
 #pragma unroll 1
         for (int i = 0; i < a_stages && i < a_it; ++i) mbar_wait(e.a_empty + 8 * i, (uint32_t)((a_it - 1 - i) / a_stages) & 1u, e.abort_flag);
@@ -551,7 +556,6 @@ __device__ __forceinline__ void write_out(const PipeScalars& p, PipeShared& sh, 
             ok = mbar_wait(acc_full + 8 * buf, par, &sh.abort_flag);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok && lane == 0) report(p.status, 27);
-            if (!CELL && p.pdl_late && nu.left <= 0) pdl_launch_dependents();
             tc_fence_after();
         }
         const uint32_t acc0 = tmem_base + (uint32_t)(buf * T) * p.acc_cols + ((uint32_t)(quad * 32) << 16);

@@ -75,7 +75,7 @@ cudaError_t conv_pipe_prepare(ConvPipePlan* plan, const ConvShape& s, int pass, 
                               const float* w_lo, float* out, const float* extra, bool accumulate, const ConvPipeBn* bn,
                               void* splitk, size_t splitk_bytes, bool w_ready, ConvPipeUse use);
 // Micro-batches m_first .. m_first + m_count - 1 in one launch.
-// pdl_late: the successor may be scheduled when the last accumulator of a CTA is complete, not at its start.
+// pdl_late: the successor may be scheduled when a CTA has issued its last MMAs (their operands have arrived), not at its start.
 cudaError_t conv_pipe_launch(const ConvPipePlan* plan, int m_first, int m_count, bool pdl_late, DeviceStatus* status, cudaStream_t st, int64_t* n_launch);
 
 // Persistent cells: prepared launches run one after the other by ONE resident grid of `ctas` CTAs with a grid-wide barrier

@@ -214,3 +214,17 @@ def test_kernels_that_start_early_read_the_steps_results_with_ordered_loads():
         todo += [c for c in re.findall(r"\b(\w+)\s*(?:<[^;()<>]*>)?\(", bodies[k]) if c in bodies]
         for arg in re.findall(r"__ldg\((?:reinterpret_cast<[^>]*>\()?&?([\w.]+)", bodies[k]):
             assert arg.split(".")[-1] in ("gamma", "beta", "bn_gamma", "bn_beta"), (k, arg)
+
+
+def test_every_pipelined_convolution_triggers_its_successor_early_or_late():
+    """A launch that may not trigger at its start (it waits for its weights, or the option asks for it) does so once its CTA has
+    issued all its MMAs: behind the loop over its units, for every number of patches a unit has and of units a CTA has."""
+    text = open(os.path.join(os.path.dirname(hpf.__file__), "csrc", "conv_pipe.cu")).read()
+    text = re.sub(r"//[^\n]*", "", text)
+    body = re.search(r"void mma_role\(.*?\n\{\n(.*?)\n\}\n", text, re.S).group(1)
+    loop = re.search(r"\n    for \(; u\.left > 0; u\.next\(p\)\) \{\n(.*?)\n    \}\n(.*)", body, re.S)
+    assert "umma_commit(e.acc_full" in loop.group(1) and "pdl_launch_dependents" not in loop.group(1)
+    assert re.search(r"^    if \(!CELL && p\.pdl_late\) pdl_launch_dependents\(\);$", loop.group(2), re.M)
+    # the early ones at their start, the late ones there and nowhere else
+    calls = re.findall(r"[^\n;]*pdl_launch_dependents\(\);", text)
+    assert len([c for c in calls if "pdl_late" in c]) == 2 and sum("!p.pdl_late" in c for c in calls) == 1
