@@ -1283,6 +1283,7 @@ __global__ void __launch_bounds__(kPipeThreads, 1) conv_pipe_cell_kernel(const _
 // the rest.  sum, act: the residual sum and the ReLU that follow a plain BN in a post-activation block, sum = y + add, act = max(sum, 0),
 // two launches and three trips through memory less.  Bound by memory; grid (blocks, micro-batches).
 constexpr int kMergeThreads = 256;
+constexpr int kMergeMaxChannels = 24576;              // mean and rstd of every channel in shared memory: 192 KB
 struct BnMergeApply {
     const float *partials, *gamma, *beta;
     float* stats;
@@ -1586,6 +1587,7 @@ cudaError_t conv_pipe_init()
             for (PipeKernel kernel : {pipe_kernel<8>(k >= 4, k & 1, k == 2 || k == 3), pipe_kernel<4>(k >= 4, k & 1, k == 2 || k == 3)})
                 if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPipeSmem + 1024);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(conv_pipe_cell_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPipeSmem + 1024);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(bn_merge_apply_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * kMergeMaxChannels * (int)sizeof(float));
         *done = true;
         return e;
     });
@@ -1758,6 +1760,8 @@ cudaError_t conv_pipe_cell_launch(const void* d_ops, int n_ops, int m_first, int
     if (n_launch) ++*n_launch;
     return cudaGetLastError();
 }
+
+bool bn_merge_apply_takes(int C) { return C <= kMergeMaxChannels; }
 
 cudaError_t bn_merge_apply(const float* partials, int units, const float* gamma, const float* beta, float eps, bool relu, const float* x, float* y, const float* add,
                            float* sum, float* act, float* stats, long long rows, int C, int m_count, cudaStream_t st, int64_t* n_launch)

@@ -91,6 +91,8 @@ cudaError_t conv_pipe_cell_launch(const void* d_ops, int n_ops, int m_first, int
 
 // y = BN(x) (+ ReLU) and the statistics of m_count micro-batches of `rows` rows, which follow one another, from the partial moments a
 // forward kernel left; with add: sum = y + add and, unless null, act = max(sum, 0) beside it.
+// (channels beyond what it takes: the BN forms its statistics itself)
+bool bn_merge_apply_takes(int C);
 cudaError_t bn_merge_apply(const float* partials, int units, const float* gamma, const float* beta, float eps, bool relu, const float* x, float* y, const float* add,
                            float* sum, float* act, float* stats, long long rows, int C, int m_count, cudaStream_t st, int64_t* n_launch);
 

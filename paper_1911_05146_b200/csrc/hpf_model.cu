@@ -479,7 +479,7 @@ void build_kernel_plan(hpf_model* mdl, hpf_model::KernelPlan* kp)
         int t = bn.op.src0, prod = -1;
         if (mdl->ops[t].op.kind == HPF_OP_CONV && mdl->fused_into[t] < 0) prod = t;
         else if (mdl->ops[t].op.kind == HPF_OP_ADD && mdl->add_done_by[t] >= 0) prod = mdl->add_done_by[t];
-        if (prod < 0 || !kp->use_pipe[PASS_FWD][prod] || mdl->ops[prod].part != bn.part || kp->conv_fwd_bn[prod] >= 0 ||
+        if (prod < 0 || !kp->use_pipe[PASS_FWD][prod] || mdl->ops[prod].part != bn.part || kp->conv_fwd_bn[prod] >= 0 || !bn_merge_apply_takes(bn.C) ||
             !conv_pipe_can_fuse_bn_output(kp->pipe_geom[PASS_FWD][prod])) continue;
         bool adjacent = true;
         for (int k = prod + 1; k < j; ++k)

@@ -114,3 +114,11 @@ def test_a_plain_batch_norm_and_its_sum_without_an_activation():
     ops = [wl.Op(wl.CONV, -1, -1, 3, 32, 3, 1, 1, 0.0), wl.Op(wl.CONV, 0, -1, 32, 32, 3, 1, 1, 0.0), wl.Op(wl.BN, 1, -1, 32, 32, 0, 1, 0, 1e-5),
            wl.Op(wl.ADD, 0, 2, 32, 32, 0, 1, 0, 0.0), wl.Op(wl.HEAD, 3, -1, 32, 10, 0, 1, 0, 0.0)]
     check_step(ops, (8, 8, 3), 4, 2, [], seed=24, bn_jitter=0.2)
+
+
+@pytest.mark.parametrize("kind", [wl.BN, wl.BNRELU], ids=["BN", "BNRELU"])
+@pytest.mark.parametrize("C", [4096, 4224, 24576, 24704])      # 48 KB of shared memory and the next; the most channels that fit and the next
+def test_a_batch_norm_of_very_many_channels_behind_a_convolution(C, kind):
+    ops = [wl.Op(wl.CONV, -1, -1, 3, 16, 3, 1, 1, 0.0), wl.Op(wl.CONV, 0, -1, 16, C, 1, 1, 0, 0.0), wl.Op(kind, 1, -1, C, C, 0, 1, 0, 1e-5),
+           wl.Op(wl.CONV, 2, -1, C, 16, 1, 1, 0, 0.0), wl.Op(wl.HEAD, 3, -1, 16, 10, 0, 1, 0, 0.0)]
+    check_step(ops, (4, 4, 3), 4, 2, [], seed=25, bn_jitter=0.2)
