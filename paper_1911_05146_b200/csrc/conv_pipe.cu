@@ -80,6 +80,7 @@ struct PipeScalars {
     double bn_inv_rows;
     // BN moments of the output; bn_x (data gradient): the sums of a BN+ReLU's backward instead, whose input bn_x is laid out like out
     float* st_partials;
+    int st_plain;                                     // of a plain BN's input: added up in fp64, with the lower parts of the means
     const float* bn_x;
     // split K
     char* sk_base;                                    // per micro-batch: tickets, then partial tiles
@@ -164,7 +165,9 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 __device__ __forceinline__ void split_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kSplitThreads) : "memory"); }
 __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 2, 256;" ::: "memory"); }
 
-__host__ __device__ inline size_t partial_floats(int units, int C) { return (size_t)units * 2 * C + (size_t)((units + 3) & ~3); }
+// partial moments of a micro-batch: rows of [2][C], a count a row, and what rounding takes off the rows' means ([C] a row)
+__host__ __device__ inline size_t partial_lo(int units, int C) { return (size_t)units * 2 * C + (size_t)((units + 3) & ~3); }
+__host__ __device__ inline size_t partial_floats(int units, int C) { return partial_lo(units, C) + (size_t)units * C; }
 
 __device__ __forceinline__ float4 lane_sum(float4 v, int o)
 {
@@ -467,6 +470,38 @@ __device__ __forceinline__ void pipe_init_barriers(const PipeScalars& p, PipeSha
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
 
+// The end of a block of units in the write-out, for a plain BN: what eight lanes have of a column and what the warps have of it added up in
+// fp64, as the kernels that form a BN's statistics themselves add their threads' sums.
+__device__ __forceinline__ void lanes_fp64(const float* from, int step, float& sum, float& sq)
+{
+    double s = 0.0, q = 0.0;
+#pragma unroll 1
+    for (int j = 0; j < 8; ++j) { s += (double)from[16 * j]; q += (double)from[step + 16 * j]; }
+    sum = (float)s; sq = (float)q;
+}
+__device__ __forceinline__ void parts_fp64(const PipeScalars& p, const float* c3, const float* counts, int parts, int bm, int br, int c)
+{
+    const int n_chunk = p.n_chunk, C = p.c_out;
+    double n = 0.0, k0 = 0.0, sum = 0.0, sq = 0.0;
+#pragma unroll 1
+    for (int w = 0; w < parts; ++w, c3 += 3 * n_chunk) {
+        const double cnt = counts[w];
+        if (cnt == 0.0) continue;
+        const double d = c3[n_chunk];
+        if (n == 0.0) k0 = c3[0];
+        const double ek = (double)c3[0] - k0;
+        n += cnt;
+        sum += fma(cnt, ek, d);
+        sq += fma(ek, fma(cnt, ek, 2.0 * d), (double)c3[2 * n_chunk]);
+    }
+    const double dm = n > 0.0 ? sum / n : 0.0, mean = k0 + dm;
+    float* all = p.st_partials + (size_t)bm * partial_floats(p.blocks_per_m, C);
+    float* row = all + (size_t)br * 2 * C + c;
+    row[0] = (float)mean; row[C] = fmaxf((float)fma(-sum, dm, sq), 0.f);
+    all[partial_lo(p.blocks_per_m, C) + (size_t)br * C + c] = (float)(mean - (double)(float)mean);
+    if (c == 0) all[(size_t)p.blocks_per_m * 2 * C + br] = (float)n;
+}
+
 // ---- write-out: tensor memory -> registers -> global memory ----
 // A 16x256b load gives four lanes of a warp a row of the accumulator, two columns of every eight each.  The weights' rows are copied
 // in an order (the dimensions of their tensor map) that makes a lane's columns of a group of 4 W output channels W consecutive
@@ -479,7 +514,7 @@ __device__ __forceinline__ void pipe_init_barriers(const PipeScalars& p, PipeSha
 // code, a first patch took 8600 clocks against 2400 of the following ones.  So there is one loop over patches (32 rows x
 // one group of channels), every part of which stands in the code once, and its first, dry round - no rows, nothing waited
 // for, nothing stored; what it reads from tensor and shared memory is discarded - runs ahead of the first accumulator.  Everything together: ResNet-110 5.96 -> 5.62 ms, ResNet-11 0.327 -> 0.299.
-template <int W, bool FLAT, bool BNB, bool CELL>
+template <int W, bool FLAT, bool BNB, bool PLAIN, bool CELL>
 __device__ __forceinline__ void write_out(const PipeScalars& p, PipeShared& sh, uint8_t* smem, const uint32_t tmem_base,
                                           const uint32_t acc_full, const uint32_t acc_empty, const UnitWalk& u0, const int slice)
 {
@@ -489,7 +524,7 @@ __device__ __forceinline__ void write_out(const PipeScalars& p, PipeShared& sh, 
     const int quad = warp & 3, half = ew >> 2;        // a warp reads the 32 lanes of its quadrant; two warps share one
     const int q = lane & 3, r8 = lane >> 2;           // this lane's quarter of a row; its rows are r8 + 8 i
     const int n_chunk = p.n_chunk, groups = n_chunk / kCols, T = p.T, C_out = p.c_out, ksplit = p.ksplit, co0 = slice * n_chunk;
-    const bool stacked = p.stacked != 0, stats = p.st_partials != nullptr;
+    const bool stacked = p.stacked != 0, stats = p.st_partials != nullptr, plain = CELL ? p.st_plain != 0 : PLAIN;
     // Two sets of four warps.  Where there is one group of channels they take alternate units (with two accumulator sets) or
     // alternate tiles of a unit; otherwise alternate groups.
     const bool alternate = p.epi_alternate != 0, whole = groups == 1;
@@ -762,21 +797,25 @@ __device__ __forceinline__ void write_out(const PipeScalars& p, PipeShared& sh, 
         const int at_block = blocks - (more ? nu.left : 0);
 #pragma unroll 1
         for (int b = dry ? -1 : blocks - u.left; stats && b < at_block; ++b) {
-            float* contrib = mom0 + flip * mom_size;
-            float* counts = contrib + (size_t)parts * 3 * n_chunk;
+            float* const contrib = mom0 + flip * mom_size;
+            float* const counts = contrib + (size_t)parts * 3 * n_chunk;
             // a lane adds what eight lanes have of its column
             const float* from = reinterpret_cast<const float*>(slots) + ((lane % W) >> 2) * 128 + (lane / W) * 4 + (lane & 3);
 #pragma unroll 1
             for (int g1 = g_first; g1 < groups; g1 += g_step, from += W * 64) {
                 float sum = 0.f, sq1 = 0.f;
+                if (plain) lanes_fp64(from, W * 32, sum, sq1);
+                else
 #pragma unroll
-                for (int j = 0; j < 8; ++j) { sum += from[16 * j]; sq1 += from[W * 32 + 16 * j]; }
+                    for (int j = 0; j < 8; ++j) { sum += from[16 * j]; sq1 += from[W * 32 + 16 * j]; }
                 float* to = contrib + part * 3 * n_chunk + kCols * g1 + lane;
                 if (lane < kCols) { to[n_chunk] = sum; to[2 * n_chunk] = sq1; }
             }
             if (lane == 0 && (whole || half == 0)) counts[part] = (float)count;
             epi_sync();
-            if (tid < n_chunk) {
+            if (plain) {
+                if (tid < n_chunk && ok && finish && b >= 0) parts_fp64(p, contrib + tid, counts, parts, bm, br, co0 + tid);
+            } else if (tid < n_chunk) {
                 // parts about their own shifts k_w: sum and squares about the first one's,
                 //   sum (x - k0) = sum_w [d_w + n_w e],  sum (x - k0)^2 = sum_w [q_w + e (2 d_w + n_w e)],  e = k_w - k0
                 // (BNB: no shifts, the sums themselves)
@@ -838,7 +877,9 @@ __device__ __forceinline__ void write_out(const PipeScalars& p, PipeShared& sh, 
 // BNB: a data gradient that forms the sums of a BN+ReLU's backward.
 // CELL: inside the persistent cell kernel, which keeps its tensor memory and has no successor to trigger.
 // W: channels of a row that a write-out lane has.
-template <bool BN_IN, bool FLAT, bool BNB, int W, bool CELL>
+// PLAIN: the moments it forms are a plain BN's (a kernel of its own: as a branch of the write-out the fp64 sums cost every launch, ResNet-11
+// 286 -> 290 us); a persistent cell has the branch.
+template <bool BN_IN, bool FLAT, bool BNB, bool PLAIN, int W, bool CELL>
 __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars& p, PipeShared& sh, uint8_t* smem, const uint32_t tmem_base,
                                          const int m_first, const int m_count, const int bid, const int nblk)
 {
@@ -1114,7 +1155,7 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
             ahead -= ke - kb;
         }
     } else if (warp >= kFirstSplit + kSplitWarps) {
-        write_out<W, FLAT, BNB, CELL>(p, sh, smem, tmem_base, acc_full, acc_empty, u0, slice);
+        write_out<W, FLAT, BNB, PLAIN, CELL>(p, sh, smem, tmem_base, acc_full, acc_empty, u0, slice);
     }
 
     // ---- teardown ----
@@ -1136,7 +1177,7 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
     __syncthreads();
 }
 
-template <bool BN_IN, bool FLAT, bool BNB, int W>
+template <bool BN_IN, bool FLAT, bool BNB, bool PLAIN, int W>
 __global__ void __launch_bounds__(kPipeThreads, 1) conv_pipe_kernel(const __grid_constant__ PipeParams gp, const int m_first, const int m_count)
 {
     const PipeScalars& p = gp.s;
@@ -1159,7 +1200,7 @@ __global__ void __launch_bounds__(kPipeThreads, 1) conv_pipe_kernel(const __grid
     // take the columns this one needs and wait for this one to finish.
     if (!p.pdl_late) pdl_launch_dependents();
     const uint32_t tmem_base = sh.tmem_slot;
-    pipe_cta<BN_IN, FLAT, BNB, W, false>(gp, p, sh, smem, tmem_base, m_first, m_count, (int)blockIdx.x, (int)gridDim.x);
+    pipe_cta<BN_IN, FLAT, BNB, PLAIN, W, false>(gp, p, sh, smem, tmem_base, m_first, m_count, (int)blockIdx.x, (int)gridDim.x);
     if (warp_index() == 0) tmem_dealloc(tmem_base, p.tmem_cols);
 }
 
@@ -1263,11 +1304,11 @@ __global__ void __launch_bounds__(kPipeThreads, 1) conv_pipe_cell_kernel(const _
             __syncthreads();
             tc_fence_after();
             if (bn_in) {
-                if (flat) { if (p.wide) pipe_cta<true, true, false, 8, true>(gp, p, sh, smem, tmem_base, m_first, m_count, v, V); else pipe_cta<true, true, false, 4, true>(gp, p, sh, smem, tmem_base, m_first, m_count, v, V); }
-                else { if (p.wide) pipe_cta<true, false, false, 8, true>(gp, p, sh, smem, tmem_base, m_first, m_count, v, V); else pipe_cta<true, false, false, 4, true>(gp, p, sh, smem, tmem_base, m_first, m_count, v, V); }
+                if (flat) { if (p.wide) pipe_cta<true, true, false, false, 8, true>(gp, p, sh, smem, tmem_base, m_first, m_count, v, V); else pipe_cta<true, true, false, false, 4, true>(gp, p, sh, smem, tmem_base, m_first, m_count, v, V); }
+                else { if (p.wide) pipe_cta<true, false, false, false, 8, true>(gp, p, sh, smem, tmem_base, m_first, m_count, v, V); else pipe_cta<true, false, false, false, 4, true>(gp, p, sh, smem, tmem_base, m_first, m_count, v, V); }
             } else {
-                if (flat) { if (p.wide) pipe_cta<false, true, false, 8, true>(gp, p, sh, smem, tmem_base, m_first, m_count, v, V); else pipe_cta<false, true, false, 4, true>(gp, p, sh, smem, tmem_base, m_first, m_count, v, V); }
-                else { if (p.wide) pipe_cta<false, false, false, 8, true>(gp, p, sh, smem, tmem_base, m_first, m_count, v, V); else pipe_cta<false, false, false, 4, true>(gp, p, sh, smem, tmem_base, m_first, m_count, v, V); }
+                if (flat) { if (p.wide) pipe_cta<false, true, false, false, 8, true>(gp, p, sh, smem, tmem_base, m_first, m_count, v, V); else pipe_cta<false, true, false, false, 4, true>(gp, p, sh, smem, tmem_base, m_first, m_count, v, V); }
+                else { if (p.wide) pipe_cta<false, false, false, false, 8, true>(gp, p, sh, smem, tmem_base, m_first, m_count, v, V); else pipe_cta<false, false, false, false, 4, true>(gp, p, sh, smem, tmem_base, m_first, m_count, v, V); }
             }
             if (sh.abort_flag) { if (tid == 0) cell_stop = 1; break; }
         }
@@ -1278,12 +1319,87 @@ __global__ void __launch_bounds__(kPipeThreads, 1) conv_pipe_cell_kernel(const _
     if (warp_index() == 0) tmem_dealloc(tmem_base, cp.tmem_cols);
 }
 
-// A BN that no convolution applies, from the moments the producing convolution left: every block merges them (merge_moments, the same
-// bits in each) and normalises its rows, one launch and one reading of x instead of a launch for the statistics and one for
+// A BN that no convolution applies, from the moments the producing convolution left: every block merges them (the same bits in each)
+// and normalises its rows, one launch and one reading of x instead of a launch for the statistics and one for
 // the rest.  sum, act: the residual sum and the ReLU that follow a plain BN in a post-activation block, sum = y + add, act = max(sum, 0),
 // two launches and three trips through memory less.  Bound by memory; grid (blocks, micro-batches).
 constexpr int kMergeThreads = 256;
 constexpr int kMergeMaxChannels = 24576;              // mean and rstd of every channel in shared memory: 192 KB
+constexpr int kMergeStep = kMergeThreads + 4;         // doubles between the values of a thread: the combining threads' banks
+// merge_moments in fp64 and with the lower parts of the rows' means: a plain BN is no less precise here than where it forms its
+// statistics itself (fp64 sums of fp32 partial sums, a root in fp64).  Mean, in sigma, and 1/sigma, in units of the last place, against fp64
+// statistics of the stored values, root mean square over the channels, itself / here: 64 channels @8, 4 maps, 1.7e-8, 0.56 / 1.1e-8, 0.38;
+// 32 @16, 32 maps, 1.4e-8, 0.39 / 0.9e-8, 0.27; 64 @56, 16 maps, 1.1e-8, 0.35 / 0.8e-8, 0.31.  In fp32 (as for BN+ReLU) 3.5e-8, 0.88; 1.2e-8,
+// 0.58; 1.0e-8, 0.56.  A step of ResNet-110 with post-activation blocks takes 6.06 ms with it and 6.03 in fp32.
+// red: 8 x kMergeStep.
+__device__ __forceinline__ void merge_moments_fp64(const float* partials, int rows, int C, double inv_rows, float eps, float* tab, double* red, int t)
+{
+    constexpr int T = kMergeThreads, kRows = 2;
+    const float *counts = partials + (size_t)rows * 2 * C, *lower = partials + partial_lo(rows, C);
+    const int c4n = C >> 2, L = c4n <= T ? T / c4n : 1;
+#pragma unroll 1
+    for (int c0 = 0; c0 < c4n; c0 += T) {
+        const int width = c4n - c0 < T ? c4n - c0 : T;
+        const int ln = L > 1 ? t / c4n : 0, local = L > 1 ? t - ln * c4n : t, col = c0 + local;
+        const bool mine = local < width && ln < L;
+        double s[8] = {};                             // of four channels sum n (mean_u - ref), sum M2_u + n (mean_u - ref)^2
+        if (mine) {
+            const float4 r4 = __ldcg(reinterpret_cast<const float4*>(partials) + col);
+            const float ref[4] = {r4.x, r4.y, r4.z, r4.w};
+#pragma unroll 1
+            for (int k0 = ln; k0 < rows; k0 += kRows * L) {
+                float mean[kRows][4], lo[kRows][4], m2[kRows][4], n[kRows];
+#pragma unroll
+                for (int j = 0; j < kRows; ++j) {
+                    const bool have = k0 + j * L < rows;
+                    const size_t k = have ? k0 + j * L : 0;
+                    n[j] = have ? __ldcg(counts + k) : 0.f;
+                    load_vec<4>(partials + k * 2 * C + 4 * col, mean[j]);
+                    load_vec<4>(partials + (k * 2 + 1) * C + 4 * col, m2[j]);
+                    load_vec<4>(lower + k * C + 4 * col, lo[j]);
+                }
+#pragma unroll
+                for (int j = 0; j < kRows; ++j)
+                    if (k0 + j * L < rows)
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            const double d = (double)mean[j][e] - (double)ref[e] + (double)lo[j][e], nd = (double)n[j] * d;
+                            s[e] += nd;
+                            s[4 + e] += fma(nd, d, (double)m2[j][e]);
+                        }
+            }
+        }
+        int lanes = L, at = t;                        // row lanes left to add
+        bool put = mine;
+        if (c4n <= 16 && (c4n & (c4n - 1)) == 0) {
+            // the row lanes of a column inside a warp first: a fixed butterfly
+#pragma unroll 1
+            for (int o = 16; o >= c4n; o >>= 1)
+#pragma unroll
+                for (int e = 0; e < 8; ++e) s[e] += __shfl_xor_sync(0xffffffffu, s[e], o);
+            lanes = T / 32;
+            at = (t >> 5) * c4n + (t & 31);
+            put = (t & 31) < c4n;
+        }
+        if (put)
+#pragma unroll
+            for (int e = 0; e < 8; ++e) red[e * kMergeStep + at] = s[e];
+        __syncthreads();
+#pragma unroll 1
+        for (int c = t; c < 4 * width; c += T) {
+            const double* r = red + (c & 3) * kMergeStep + (c >> 2);
+            double d = 0.0, q = 0.0;
+#pragma unroll 4
+            for (int l = 0; l < lanes; ++l, r += width) { d += r[0]; q += r[4 * kMergeStep]; }
+            const double dm = d * inv_rows;
+            double var = q * inv_rows - dm * dm;
+            if (var < 0.0) var = 0.0;
+            tab[4 * c0 + c] = (float)((double)__ldcg(partials + 4 * c0 + c) + dm);
+            tab[C + 4 * c0 + c] = (float)rsqrt(var + (double)eps);
+        }
+        __syncthreads();
+    }
+}
 struct BnMergeApply {
     const float *partials, *gamma, *beta;
     float* stats;
@@ -1291,19 +1407,23 @@ struct BnMergeApply {
     float4 *y, *sum, *act;       // add, sum, act: null without
     int units, C;
     double inv_rows;
-    float eps, floor;
+    float eps;
     long long n4, per_block, ms4;   // float4 of a micro-batch, of a block; between micro-batches
 };
-__global__ void __launch_bounds__(kMergeThreads) bn_merge_apply_kernel(const BnMergeApply a)
+template <bool RELU>
+__global__ void __launch_bounds__(kMergeThreads, 3) bn_merge_apply_kernel(const BnMergeApply a)
 {
+    constexpr float floor = RELU ? 0.f : -INFINITY;
     extern __shared__ float tab[];                    // mean, rstd
-    __shared__ float4 red[4 * kMergeThreads];
+    __shared__ __align__(16) double red[8 * kMergeStep];
     pdl_launch_dependents();
     pdl_wait();
     const int t = threadIdx.x, C = a.C, c4n = C >> 2;
     const float* partials = a.partials + (size_t)blockIdx.y * partial_floats(a.units, C);
-    merge_moments<kMergeThreads>(partials, a.units, C, a.inv_rows, a.eps, tab, red, t);
-    __syncthreads();
+    if constexpr (RELU) {
+        merge_moments<kMergeThreads>(partials, a.units, C, a.inv_rows, a.eps, tab, reinterpret_cast<float4*>(red), t);
+        __syncthreads();
+    } else merge_moments_fp64(partials, a.units, C, a.inv_rows, a.eps, tab, red, t);
     if (blockIdx.x == 0)
         for (int i = t; i < 2 * C; i += kMergeThreads) a.stats[(size_t)blockIdx.y * 2 * C + i] = tab[i];
     const long long first = blockIdx.x * a.per_block + t, end = (blockIdx.x + 1) * a.per_block < a.n4 ? (blockIdx.x + 1) * a.per_block : a.n4;
@@ -1326,7 +1446,7 @@ __global__ void __launch_bounds__(kMergeThreads) bn_merge_apply_kernel(const BnM
             if (i + j * kMergeThreads < end) {
                 const long long at = ms + i + j * kMergeThreads;
                 float4 z = fma4(g, mul4(sub4(v[j], mu), rs), b);
-                z = make_float4(fmaxf(z.x, a.floor), fmaxf(z.y, a.floor), fmaxf(z.z, a.floor), fmaxf(z.w, a.floor));
+                z = make_float4(fmaxf(z.x, floor), fmaxf(z.y, floor), fmaxf(z.z, floor), fmaxf(z.w, floor));
                 a.y[at] = z;
                 if (a.add) {
                     z = add4(z, e[j]);
@@ -1569,11 +1689,13 @@ static_assert(sizeof(ConvPipeLaunch) <= sizeof(((ConvPipePlan*)0)->storage), "pl
 namespace {
 using PipeKernel = void (*)(PipeParams, int, int);
 template <int W>
-PipeKernel pipe_kernel(bool bn_in, bool flat, bool bnb)
+PipeKernel pipe_kernel(bool bn_in, bool flat, bool bnb, bool plain)
 {
-    if (bn_in) return flat ? conv_pipe_kernel<true, true, false, W> : conv_pipe_kernel<true, false, false, W>;
-    if (bnb) return flat ? conv_pipe_kernel<false, true, true, W> : conv_pipe_kernel<false, false, true, W>;
-    return flat ? conv_pipe_kernel<false, true, false, W> : conv_pipe_kernel<false, false, false, W>;
+    if (bnb) return flat ? conv_pipe_kernel<false, true, true, false, W> : conv_pipe_kernel<false, false, true, false, W>;
+    if (plain && bn_in) return flat ? conv_pipe_kernel<true, true, false, true, W> : conv_pipe_kernel<true, false, false, true, W>;
+    if (plain) return flat ? conv_pipe_kernel<false, true, false, true, W> : conv_pipe_kernel<false, false, false, true, W>;
+    if (bn_in) return flat ? conv_pipe_kernel<true, true, false, false, W> : conv_pipe_kernel<true, false, false, false, W>;
+    return flat ? conv_pipe_kernel<false, true, false, false, W> : conv_pipe_kernel<false, false, false, false, W>;
 }
 }  // namespace
 
@@ -1583,11 +1705,12 @@ cudaError_t conv_pipe_init()
     bool set = false;
     return attributes.get(&set, [](int, bool* done) {
         cudaError_t e = cudaSuccess;
-        for (int k = 0; k < 6; ++k)
-            for (PipeKernel kernel : {pipe_kernel<8>(k >= 4, k & 1, k == 2 || k == 3), pipe_kernel<4>(k >= 4, k & 1, k == 2 || k == 3)})
+        for (int k = 0; k < 16; ++k)
+            for (PipeKernel kernel : {pipe_kernel<8>(k & 1, k & 2, k & 4, k & 8), pipe_kernel<4>(k & 1, k & 2, k & 4, k & 8)})
                 if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPipeSmem + 1024);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(conv_pipe_cell_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPipeSmem + 1024);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(bn_merge_apply_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * kMergeMaxChannels * (int)sizeof(float));
+        for (auto kernel : {bn_merge_apply_kernel<true>, bn_merge_apply_kernel<false>})
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * kMergeMaxChannels * (int)sizeof(float));
         *done = true;
         return e;
     });
@@ -1682,7 +1805,7 @@ cudaError_t conv_pipe_prepare(ConvPipePlan* plan, const ConvShape& s, int pass, 
     L->smem = p.off_red + (pass == PASS_DGRAD && use.moments ? kBnbBytes : 0u) + 1024;
     if (bn && bn->out_partials) {
         if (!conv_pipe_can_fuse_bn_output(g)) return cudaErrorNotSupported;
-        p.st_partials = bn->out_partials;
+        p.st_partials = bn->out_partials; p.st_plain = bn->out_plain ? 1 : 0;
     }
     if (bn && bn->bwd_partials) {
         if (pass != PASS_DGRAD || s.stride != 1 || extra || accumulate || !conv_pipe_can_fuse_bn_output(g)) return cudaErrorNotSupported;
@@ -1719,7 +1842,7 @@ cudaError_t conv_pipe_launch(const ConvPipePlan* plan, int m_first, int m_count,
     if (per_slice < 1) per_slice = 1;
     if (per_slice > tasks) per_slice = tasks;
     const bool flat = p.flat && p.zero_fill == 1;
-    auto kernel = p.wide ? pipe_kernel<8>(L.bn_in, flat, p.bn_x != nullptr) : pipe_kernel<4>(L.bn_in, flat, p.bn_x != nullptr);
+    auto kernel = p.wide ? pipe_kernel<8>(L.bn_in, flat, p.bn_x != nullptr, p.st_plain) : pipe_kernel<4>(L.bn_in, flat, p.bn_x != nullptr, p.st_plain);
     // What a CTA has to do decides how its warps share it (the sums are the same either way).  A block of the operand takes one
     // splitter warp about 2000 clocks and all four of them 850, so with one or two blocks in all they share each; with a single unit
     // both halves of the write-out's warps take it.
@@ -1770,7 +1893,7 @@ cudaError_t bn_merge_apply(const float* partials, int units, const float* gamma,
     a.partials = partials; a.gamma = gamma; a.beta = beta; a.stats = stats; a.units = units; a.C = C;
     a.x = reinterpret_cast<const float4*>(x); a.add = reinterpret_cast<const float4*>(add);
     a.y = reinterpret_cast<float4*>(y); a.sum = reinterpret_cast<float4*>(sum); a.act = reinterpret_cast<float4*>(act);
-    a.inv_rows = 1.0 / (double)rows; a.eps = eps; a.floor = relu ? 0.f : -INFINITY;
+    a.inv_rows = 1.0 / (double)rows; a.eps = eps;
     a.n4 = a.ms4 = rows * C / 4;
     // Every block merges the moments first: eight float4 a thread at least, twice as much of the tensor as of moments, four blocks an SM
     // at most.
@@ -1779,7 +1902,7 @@ cudaError_t bn_merge_apply(const float* partials, int units, const float* gamma,
     if (blocks > most) blocks = most;
     if (blocks < 1) blocks = 1;
     a.per_block = (a.n4 + blocks - 1) / blocks;
-    launch_pdl(bn_merge_apply_kernel, dim3((unsigned int)((a.n4 + a.per_block - 1) / a.per_block), m_count), dim3(kMergeThreads), (size_t)2 * C * sizeof(float), st, a);
+    launch_pdl(relu ? bn_merge_apply_kernel<true> : bn_merge_apply_kernel<false>, dim3((unsigned int)((a.n4 + a.per_block - 1) / a.per_block), m_count), dim3(kMergeThreads), (size_t)2 * C * sizeof(float), st, a);
     if (n_launch) ++*n_launch;
     return cudaGetLastError();
 }

@@ -33,8 +33,8 @@ bool conv_pipe_geom(const ConvShape& s, int pass, int passes, int launched, Conv
 
 // BN work that rides in the forward kernel.
 //   out_partials: the output is the input of a BN: per block of units and output channel the mean and the sum of squared
-//     deviations of the stored values, [blocks_per_m][2][c_out] floats and then [blocks_per_m] counts, conv_pipe_partial_floats() per
-//     micro-batch;
+//     deviations of the stored values, [blocks_per_m][2][c_out] floats, then [blocks_per_m] counts and, of a BN without a
+//     ReLU (out_plain), [blocks_per_m][c_out] lower parts of the means, conv_pipe_partial_floats() per micro-batch;
 //   in_partials: the input x is the input of a BN+ReLU that only this convolution reads: it merges the producer's moments
 //     (in_blocks rows), applies y = relu(gamma*(x-mean)*rstd+beta) to its operand, stores y (in_y) and the statistics
 //     (in_stats: mean[C], rstd[C] per micro-batch) for the backward pass.
@@ -43,6 +43,7 @@ bool conv_pipe_geom(const ConvShape& s, int pass, int passes, int launched, Conv
 //     micro-batch, from the BN's input (bwd_x), statistics (bwd_stats) and parameters (in_gamma, in_beta).
 struct ConvPipeBn {
     float* out_partials = nullptr;
+    bool out_plain = false;
     const float* in_partials = nullptr;
     int in_blocks = 0;
     const float* in_gamma = nullptr;

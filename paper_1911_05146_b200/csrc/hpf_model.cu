@@ -699,7 +699,10 @@ int prepare_kernels(hpf_model* mdl, hpf_model::KernelPlan& kp)
                 residual = mdl->act(a.src0 == i ? a.src1 : a.src0, 0);
             }
             ConvPipeBn bn;
-            if (kp.conv_fwd_bn[i] >= 0) bn.out_partials = mdl->moments(kp.conv_fwd_bn[i]);
+            if (kp.conv_fwd_bn[i] >= 0) {
+                bn.out_partials = mdl->moments(kp.conv_fwd_bn[i]);
+                bn.out_plain = mdl->ops[kp.conv_fwd_bn[i]].op.kind == HPF_OP_BN;
+            }
             const int jb = kp.conv_in_bn[i];
             if (jb >= 0) {
                 const OpInfo& b = mdl->ops[jb];

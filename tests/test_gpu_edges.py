@@ -1,10 +1,12 @@
 """Sizes at the edges of the kernels' tiles and of the rules that choose between them, against the oracle."""
+import numpy as np
 import pytest
 import torch
 
 import paper_1911_05146_b200 as hpf
 import workloads as wl
 from test_gpu_kernels import TOL_TENSOR, _conv_case
+from hpf_testlib import Bound, seeded
 from test_gpu_step import check_step
 
 pytestmark = pytest.mark.gpu
@@ -122,3 +124,25 @@ def test_a_batch_norm_of_very_many_channels_behind_a_convolution(C, kind):
     ops = [wl.Op(wl.CONV, -1, -1, 3, 16, 3, 1, 1, 0.0), wl.Op(wl.CONV, 0, -1, 16, C, 1, 1, 0, 0.0), wl.Op(kind, 1, -1, C, C, 0, 1, 0, 1e-5),
            wl.Op(wl.CONV, 2, -1, C, 16, 1, 1, 0, 0.0), wl.Op(wl.HEAD, 3, -1, 16, 10, 0, 1, 0, 0.0)]
     check_step(ops, (4, 4, 3), 4, 2, [], seed=25, bn_jitter=0.2)
+
+
+@pytest.mark.parametrize("C,ks,size,batch,micro,shift", [(64, 1, 8, 8, 2, 0), (64, 3, 8, 4, 1, 0), (256, 1, 9, 5, 1, 0), (16, 3, 32, 16, 2, 30)], ids=str)
+def test_statistics_of_a_plain_batch_norm_behind_a_convolution(C, ks, size, batch, micro, shift):
+    """Mean and 1/sigma as fp64 statistics of the stored values give them.  y = (x - mean) / sigma is a straight line in x, so
+    both come out of a fit far more precisely than one value of y has them.  The mean is off by its own rounding and the fp32 sums
+    of a lane's few rows, values of about sigma: together less than 2^-24 sigma.  1/sigma: its own rounding, half a unit in the
+    last place, and half the relative error of the sum of squares, some 2^-24: less than 1.25 units."""
+    ops = [wl.Op(wl.CONV, -1, -1, 3, 16, 3, 1, 1, 0.0), wl.Op(wl.CONV, 0, -1, 16, C, ks, 1, ks // 2, 0.0), wl.Op(wl.BN, 1, -1, C, C, 0, 1, 0, 1e-5),
+           wl.Op(wl.HEAD, 2, -1, C, 10, 0, 1, 0, 0.0)]
+    x, labels, theta = seeded(ops, (size, size, 3), batch, 31)
+    bd = Bound(ops, (size, size, 3), batch, micro, [], theta)
+    bd.upload(x + np.float32(shift), labels)
+    bd.step()
+    for m in range(micro):
+        v, y = (bd.tensor(i, m).astype(np.float64).reshape(-1, C) for i in (1, 2))
+        mean, sigma = v.mean(0), np.sqrt(v.var(0) + 1e-5)
+        slope = ((v - mean) * (y - y.mean(0))).sum(0) / ((v - mean) ** 2).sum(0)
+        used_mean = mean - y.mean(0) / slope
+        ulp = lambda a: np.spacing(np.abs(a).astype(np.float32)).astype(np.float64)  # noqa: E731
+        assert (np.abs(used_mean - mean) <= 0.5 * ulp(mean) + 2.0 ** -24 * sigma).all(), (np.abs(used_mean - mean) / sigma).max()
+        assert (np.abs(slope - 1.0 / sigma) <= 1.25 * ulp(1.0 / sigma)).all(), (np.abs(slope - 1.0 / sigma) / ulp(1.0 / sigma)).max()
