@@ -1276,10 +1276,10 @@ int hpf_estimate_op_costs(const hpf_op* ops, int32_t n_ops, const int32_t in_sha
     hpf_model* tmp = nullptr;
     int rc = hpf_model_create(ops, n_ops, in_shape, nullptr, 0, 1, &tmp);
     if (rc) return rc;
-    // Calibration (B200, micro-batch 16, one stream): a bottleneck block costs 113 / 115 / 149 us at 32x32 / 16x16 / 8x8,
-    // which a fixed cost per kernel, 0.39 us per tensor-core K step (8 channels of one tap, forward plus data
-    // gradient) and 1.4 TB/s of effective bandwidth reproduce.
-    const double us_per_k8 = 0.39, bytes_per_us = 1.4e6;
+    // Calibration (B200, one stream, one block a partition, both ways): 119 blocks of post-activation, bottleneck and ImageNet networks at
+    // micro-batches of 4..64, 50..430 us.  A fixed cost per op, 0.11 us per tensor-core K step (8 channels of one tap, forward plus
+    // data gradient) and 2.4 TB/s of effective bandwidth reproduce them to 13 % (standard deviation; 35 % at most).
+    const double us_per_k8 = 0.11, bytes_per_us = 2.4e6;
     for (int i = 0; i < n_ops; ++i) {
         const OpInfo& o = tmp->ops[i];
         const double in_el = (double)in_shape[0] * o.iH * o.iW * o.iC, out_el = (double)in_shape[0] * o.H * o.W * o.C;
@@ -1288,12 +1288,12 @@ int hpf_estimate_op_costs(const hpf_op* ops, int32_t n_ops, const int32_t in_sha
         case HPF_OP_CONV: {
             const int taps = o.op.ksize * o.op.ksize;
             const double k8 = taps * (o.op.c_in / 8.0) + (o.op.src0 >= 0 ? taps * (o.op.c_out / 8.0) : 0.0);
-            c = 8.0 + us_per_k8 * k8 + 4.0 * 2.0 * (in_el + out_el) / bytes_per_us;
+            c = 18.0 + us_per_k8 * k8 + 4.0 * 2.0 * (in_el + out_el) / bytes_per_us;
             break;
         }
-        case HPF_OP_BNRELU: c = 9.0 + 20.0 * out_el / bytes_per_us; break;
-        case HPF_OP_BN: c = 18.0 + 20.0 * out_el / bytes_per_us; break;        // its own reduce + apply kernels, both ways
-        case HPF_OP_RELU: c = 6.0 + 20.0 * out_el / bytes_per_us; break;
+        case HPF_OP_BNRELU: c = 2.0 + 20.0 * out_el / bytes_per_us; break;      // rides in the convolutions around it, but for its data gradient's second half
+        case HPF_OP_BN: c = 7.0 + 20.0 * out_el / bytes_per_us; break;          // one kernel each way; the forward one also does the sum and the ReLU behind it
+        case HPF_OP_RELU: c = 5.0 + 20.0 * out_el / bytes_per_us; break;
         case HPF_OP_ADD: c = 0.0; break;                       // fused into the producing convolution
         case HPF_OP_MAXPOOL: c = 6.0 + 4.0 * 2.0 * (in_el + out_el) / bytes_per_us; break;
         default: c = 20.0; break;                               // head: a handful of tiny kernels

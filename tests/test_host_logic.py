@@ -180,6 +180,20 @@ def test_load_balancer_cuts():
     assert m.num_partitions() == 8
 
 
+def test_modelled_costs_of_blocks_follow_the_measured_ones():
+    """Blocks with and without a stage's change of size, post-activation ones (whose end is one launch forward) and bottlenecks, at
+    micro-batches of 16: microseconds both ways on one stream.  Cuts depend on the ratios alone."""
+    v1 = wl.resnet_v1_cifar(3)
+    v2 = wl.resnet_v2_cifar(3)
+    measured = {(0, 1): 74.5, (0, 3): 108.5, (0, 4): 61.0, (0, 6): 124.7, (0, 7): 80.3, (1, 1): 95.5, (1, 3): 106.6, (1, 4): 78.0, (1, 6): 126.5, (1, 7): 94.5}
+    ratios = []
+    for net, ops in enumerate((v1, v2)):
+        ends = [i + (2 if net == 0 else 1) for i, o in enumerate(ops) if o.kind == wl.ADD]
+        cost = hpf.estimate_op_costs(ops, (16, 32, 32, 3))
+        ratios += [sum(cost[a:b]) / measured[net, k + 1] for k, (a, b) in enumerate(zip(ends, ends[1:])) if (net, k + 1) in measured]
+    assert len(ratios) == len(measured) and max(ratios) / min(ratios) < 1.5, ratios
+
+
 def test_microbatch_tuner_search_order():
     """Section 5.3: pipeline stages range from 1 to the batch size; the search starts at the batch size and halves."""
     from paper_1911_05146_b200.tuner import halving_candidates
