@@ -114,14 +114,14 @@ int hpf_model_destroy(hpf_model *model);
  *   HPF_OPT_BN_CLUSTER     1 (default): the backward of a BN whose micro-batch tensor is small enough to sit in the
  *                          registers of a few thread-block clusters is one launch (the CTAs of a cluster exchange their
  *                          per-channel sums through distributed shared memory); 0: always the reduce + apply pair.
- *   HPF_OPT_PDL_LATE_FROM  N (default 8): with programmatic dependent launch, the forward convolutions of a cell that runs while at
- *                          least N cells of the one-graph schedule are under way let their successor be scheduled only when
- *                          their accumulator is complete, not at their first instruction: a successor scheduled early sits in
- *                          its SM slots for the whole life of its predecessor, which shortens a lone stage's chain of kernels
- *                          but costs throughput once every stage is busy.  0: always late; a large N: always early.
- *                          Only launches of one micro-batch run many cells at once: with the default grouped launches two
- *                          cells at most are under way and N matters from 2 down.  0 against the default there: ResNet-11
- *                          0.328 / 0.334 ms, ResNet-110 6.28 / 6.24, ResNet-152 35.4 / 35.5, ResNet-1001 60.1 / 59.7 (before the write-out was rewritten).
+ *   HPF_OPT_PDL_LATE_FROM  N (default 0): with programmatic dependent launch, the forward convolutions of a cell that runs while at
+ *                          least N cells of the one-graph schedule are under way let their successor be scheduled only when they
+ *                          have issued their last MMAs, not at their first instruction: a successor scheduled early sits in
+ *                          its SM slots for the whole life of its predecessor.  0: always late; a large N: always early.
+ *                          Always early against always late, ms: with the default grouped launches ResNet-11 0.278 / 0.271,
+ *                          ResNet-110 5.45 / 5.39, ResNet-152 33.8 / 33.7, ResNet-1001 51.0 / 50.4, scoring ResNet-182 5.95 / 5.81;
+ *                          cells one by one ResNet-11 0.335 / 0.315, ResNet-110 5.60 / 5.47; one launch a micro-batch
+ *                          ResNet-110 8.34 / 8.17, ResNet-1001 93.1 / 91.5, but ResNet-11 0.379 / 0.387.
  *   HPF_OPT_STAGE_LANES    L (default 1): a stage keeps up to L of its micro-batches under way at once, micro-batch m on lane
  *                          m mod L, every lane with its own streams and scratch memory.  L = 1 is the schedule of Section 5.3
  *                          as the paper's one-process-per-partition runs it: a stage works through its micro-batches one
@@ -149,8 +149,8 @@ int hpf_model_destroy(hpf_model *model);
  *                          them (Section 5.3's stage as one resident grid instead of a chain of launches).  The cells of
  *                          all partitions must fit the GPU together (hpf_bind: HPF_ERR_UNSUPPORTED otherwise).  Results
  *                          are bit-identical to N = 0.  0: one launch per convolution, and the faster one: a step with the
- *                          most CTAs that fit against the default, ResNet-11 0.50 / 0.33 ms, ResNet-110 9.4 (one partition) and
- *                          15.0 (four) / 6.2, ResNet-152 45.7 and 87.5 / 35.5, ResNet-1001 87 and 249 / 59.7 (both from before the write-out was rewritten). */
+ *                          most CTAs that fit against the default, ResNet-11 0.38 / 0.28 ms, ResNet-110 7.4 (one partition) and
+ *                          11.4 (four) / 5.4, ResNet-152 38.2 and 65.8 / 33.8, ResNet-1001 63.9 and 161 (eight) / 50.9. */
 typedef enum { HPF_OPT_GRAPH = 1, HPF_OPT_CONV_PATH = 2, HPF_OPT_SINGLE_STREAM = 3, HPF_OPT_KEEP_MESSAGES = 4,
                HPF_OPT_FUSE_ADD = 5, HPF_OPT_PDL = 6, HPF_OPT_WGRAD_PASSES = 7, HPF_OPT_FUSE_BN = 8, HPF_OPT_CELL_TIMES = 9,
                HPF_OPT_BN_CLUSTER = 10, HPF_OPT_CELL_CTAS = 11, HPF_OPT_PDL_LATE_FROM = 12,

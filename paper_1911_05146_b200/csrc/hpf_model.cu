@@ -148,7 +148,7 @@ struct hpf_model {
     int lanes() const { return opt_lanes < M ? opt_lanes : M; }
     int n_slots() const { return P * lanes(); }
     int slot_of(int p, int m) const { return p * lanes() + m % lanes(); }
-    int opt_pdl_late_from = 8;   // forward cells that run while at least this many cells are under way trigger their successors late
+    int opt_pdl_late_from = 0;   // forward cells that run while at least this many cells are under way trigger their successors late
     // Groups: on one GPU the stages share the same SMs, and a micro-batch's launches are too small to fill them, so one launch
     // covers all micro-batches of a stage wherever nothing asks for cells of their own (then one micro-batch).  Every micro-batch keeps
     // its own statistics, losses and gradient slot, formed in the same order whatever the size of the group.

@@ -146,3 +146,16 @@ def test_statistics_of_a_plain_batch_norm_behind_a_convolution(C, ks, size, batc
         ulp = lambda a: np.spacing(np.abs(a).astype(np.float32)).astype(np.float64)  # noqa: E731
         assert (np.abs(used_mean - mean) <= 0.5 * ulp(mean) + 2.0 ** -24 * sigma).all(), (np.abs(used_mean - mean) / sigma).max()
         assert (np.abs(slope - 1.0 / sigma) <= 1.25 * ulp(1.0 / sigma)).all(), (np.abs(slope - 1.0 / sigma) / ulp(1.0 / sigma)).max()
+
+
+def test_when_launches_trigger_their_successors_changes_no_bit():
+    """Every forward convolution late (the default), those of cells that run beside another one, and none."""
+    ops = wl.resnet_v2_cifar(1)
+    x, labels, theta = seeded(ops, (32, 32, 3), 8, 32)
+    out = []
+    for options in ({}, {hpf.OPT_PDL_LATE_FROM: 2}, {hpf.OPT_PDL_LATE_FROM: 1000}, {hpf.OPT_PDL: 0}):
+        bd = Bound(ops, (32, 32, 3), 8, 2, [9], theta, options, backward_streams=True)
+        bd.upload(x, labels)
+        out.append((bd.step(one_graph=True), bd.slots.cpu().numpy()))
+    for loss, slots in out[1:]:
+        assert loss == out[0][0] and np.array_equal(slots, out[0][1])
