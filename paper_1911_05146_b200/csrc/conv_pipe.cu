@@ -26,7 +26,7 @@
 // Measured alone, batch 128, three passes (graph of ten launches), before and since the write-out reads rows (write_out), the MMAs are
 // issued in straight lines (mma_role) and the operand of a 1x1 window is copied by lanes: 3x3 16->16 @32 19.8 -> 15.5 us,
 // 64->64 @8 15.1 -> 11.6; 1x1 64->16 @32 21.8 -> 13.7, 16->64 @32 17.8 -> 14.3; batch 64: 3x3 64->64 @56 90 -> 74, 256->256 @14 82 -> 73;
-// 1x1 64->256 @56 70 -> 73, 256->64 @56 86 -> 69, 512->128 @28 54 -> 43, 1024->256 @14 56 -> 41.
+// 1x1 64->256 @56 70 -> 71, 256->64 @56 86 -> 69, 512->128 @28 54 -> 43, 1024->256 @14 56 -> 41.
 #include "conv_pipe.h"
 #include "tc_ptx.cuh"
 
@@ -40,7 +40,7 @@ namespace hpf {
 namespace {
 
 constexpr int kSplitWarps = 4, kEpiWarps = 8;
-constexpr int kFirstSplit = 4;                        // warps 0..2: operand copies, weight copies, MMAs; 3 idle
+constexpr int kFirstSplit = 4;                        // warps 0..2: operand copies, weight copies, MMAs; 3: barriers, half of a 1x1 operand's copies
 constexpr int kSplitThreads = 32 * kSplitWarps, kRowStep = 8 * kSplitWarps;
 constexpr int kPipeThreads = 32 * (kFirstSplit + kSplitWarps + kEpiWarps);
 constexpr int kMaxBlockRows = 768, kRowBatch = 2;     // operand rows of a block at most; rows a splitter thread has in flight (code counts: 1 / 2 / 4 / 8: ResNet-110 5.47 / 5.44 / 5.46 / 5.59 ms)
@@ -423,9 +423,10 @@ __device__ __forceinline__ void mma_role(const PipeScalars& p, const MmaEnv& e, 
         *e.b_used = b_it; *e.a_used = a_it;
     }
     // The late trigger.  Here, where a CTA has one last unit whatever its patches and sets of write-out warps are: tied to the write-out's
-    // walk it missed every launch with several patches a unit.  Ten launches in a row, late from the write-out where it could / now:
-    // 3x3 128 -> 128 @16, batch 128, 44.2 / 43.4 us, 1x1 128 -> 512 @28, batch 64, 47.1 / 45.0, 256 -> 64 @8, batch 128, dgrad 8.0 / 7.4, 64 -> 256 @56,
-    // batch 64, 72.8 / 70.7; the one slower one is 3x3 16 -> 16 @32 in one pass, 11.8 / 12.1.
+    // walk it missed every launch with several patches a unit.  Launches in a row, without it / with it, three passes, batch 128:
+    // 3x3 128 -> 128 @16 45.2 / 42.6 us, 32 -> 128 @16 19.0 / 17.6, 64 -> 64 @32 53.3 / 51.4, 1x1 256 -> 64 @8 data gradient 8.0 / 7.4; batch 64: 64 -> 256 @56
+    // 72.8 / 70.7; slower 3x3 256 -> 256 @8 73.2 / 76.1 and 16 -> 16 @32 14.9 / 15.3.  Behind the last
+    // accumulator of a set instead the same or up to 2 % slower.
     if (!CELL && p.pdl_late) pdl_launch_dependents();
     if (CELL) {                  // wait until every barrier has seen its last arrival: they are used again
 #pragma unroll 1
@@ -1072,82 +1073,78 @@ __device__ __forceinline__ void pipe_cta(const PipeParams& gp, const PipeScalars
             }
 #pragma unroll 1
             for (int c = kb + ahead; c < ke; c += groups) {
-                {
-                    ok = mbar_wait(a_raw + 8 * s, par, &abort_flag) && ok;
-                    // (after a wait that gave up the warps run through the rest without waiting: they still have to meet at
-                    // the named barriers)
-                    if (!ok && lane == 0) report(p.status, 26);
-                    uint8_t* hi = smem + (uint32_t)s * p.a_stage_bytes + at_hi;
-                    uint8_t* lo = smem + (uint32_t)s * p.a_stage_bytes + at_lo;
-                    if (BN_IN) {
-                        const int ch = 16 * c + 4 * cph;
-                        const float4 mu = *reinterpret_cast<const float4*>(tab + ch), rs = *reinterpret_cast<const float4*>(tab + C + ch);
-                        const float4 g = *reinterpret_cast<const float4*>(tab + 2 * C + ch), b = *reinterpret_cast<const float4*>(tab + 3 * C + ch);
-                        float* ydst = p.bn_y + (long long)cu.m * p.in_ms + 16 * c + 4 * cph;
-                        int yo = (sp.pos0 + row0) * C;                   // FLAT: offset of this thread's first row
-                        int pn = 0, py = 0, px = 0;                      // otherwise its map, row and column
-                        if (!FLAT) {
-                            int pos = sp.pos0 + row0;
-                            if (pos < 0) { pos += p.img_pos; pn = -1; }
-                            const int q = div_magic(pos, p.img_pos, p.magic_img);
-                            pn += q; pos -= q * p.img_pos;
-                            py = div_magic(pos, p.Wp, p.magic_w); px = pos - py * p.Wp;
-                        }
-                        // two rows in flight; the block is allocated in whole batches, so the last one needs no bounds
+                ok = mbar_wait(a_raw + 8 * s, par, &abort_flag) && ok;
+                // (after a wait that gave up the warps run through the rest without waiting: they still have to meet at
+                // the named barriers)
+                if (!ok && lane == 0) report(p.status, 26);
+                uint8_t* hi = smem + (uint32_t)s * p.a_stage_bytes + at_hi;
+                uint8_t* lo = smem + (uint32_t)s * p.a_stage_bytes + at_lo;
+                if (BN_IN) {
+                    const int ch = 16 * c + 4 * cph;
+                    const float4 mu = *reinterpret_cast<const float4*>(tab + ch), rs = *reinterpret_cast<const float4*>(tab + C + ch);
+                    const float4 g = *reinterpret_cast<const float4*>(tab + 2 * C + ch), b = *reinterpret_cast<const float4*>(tab + 3 * C + ch);
+                    float* ydst = p.bn_y + (long long)cu.m * p.in_ms + 16 * c + 4 * cph;
+                    int yo = (sp.pos0 + row0) * C;                   // FLAT: offset of this thread's first row
+                    int pn = 0, py = 0, px = 0;                      // otherwise its map, row and column
+                    if (!FLAT) {
+                        int pos = sp.pos0 + row0;
+                        if (pos < 0) { pos += p.img_pos; pn = -1; }
+                        const int q = div_magic(pos, p.img_pos, p.magic_img);
+                        pn += q; pos -= q * p.img_pos;
+                        py = div_magic(pos, p.Wp, p.magic_w); px = pos - py * p.Wp;
+                    }
+                    // two rows in flight; the block is allocated in whole batches, so the last one needs no bounds
 #pragma unroll 1
-                        for (int row = row0; row < sp.rows; row += kRowBatch * row_step, hi += kRowBatch * byte_step, lo += kRowBatch * byte_step) {
-                            float4 v[kRowBatch];
+                    for (int row = row0; row < sp.rows; row += kRowBatch * row_step, hi += kRowBatch * byte_step, lo += kRowBatch * byte_step) {
+                        float4 v[kRowBatch];
 #pragma unroll
-                            for (int j = 0; j < kRowBatch; ++j) v[j] = *reinterpret_cast<const float4*>(hi + byte_step * j);
-                            int off[kRowBatch];
-                            bool inside[kRowBatch], own[kRowBatch];
+                        for (int j = 0; j < kRowBatch; ++j) v[j] = *reinterpret_cast<const float4*>(hi + byte_step * j);
+                        int off[kRowBatch];
+                        bool inside[kRowBatch], own[kRowBatch];
 #pragma unroll
-                            for (int j = 0; j < kRowBatch; ++j) {
-                                const int r = row + row_step * j;
-                                if (FLAT) {
-                                    inside[j] = own[j] = r < valid;
-                                    off[j] = yo; yo += row_step * C;
-                                } else {
-                                    inside[j] = px < p.W && py < p.Hv && pn >= 0 && r < valid;
-                                    own[j] = inside[j] && r >= own_lo && r < own_hi;
-                                    off[j] = pn * p.in_sn + py * p.in_sh + px * p.in_sw;
-                                    px += dx; py += dy; pn += dn;
-                                    if (px >= p.Wp) { px -= p.Wp; ++py; }
-                                    if (py >= Hp) { py -= Hp; ++pn; }
-                                }
+                        for (int j = 0; j < kRowBatch; ++j) {
+                            const int r = row + row_step * j;
+                            if (FLAT) {
+                                inside[j] = own[j] = r < valid;
+                                off[j] = yo; yo += row_step * C;
+                            } else {
+                                inside[j] = px < p.W && py < p.Hv && pn >= 0 && r < valid;
+                                own[j] = inside[j] && r >= own_lo && r < own_hi;
+                                off[j] = pn * p.in_sn + py * p.in_sh + px * p.in_sw;
+                                px += dx; py += dy; pn += dn;
+                                if (px >= p.Wp) { px -= p.Wp; ++py; }
+                                if (py >= Hp) { py -= Hp; ++pn; }
                             }
-#pragma unroll
-                            for (int j = 0; j < kRowBatch; ++j) {
-                                const float4 z = fma4(g, mul4(sub4(v[j], mu), rs), b);
-                                v[j] = make_float4(fmaxf(z.x, 0.f), fmaxf(z.y, 0.f), fmaxf(z.z, 0.f), fmaxf(z.w, 0.f));
-                                if (!inside[j]) v[j] = make_float4(0.f, 0.f, 0.f, 0.f);      // the padding is zero AFTER the activation
-                                *reinterpret_cast<float4*>(hi + byte_step * j) = v[j];
-                            }
-                            if (three)
-#pragma unroll
-                                for (int j = 0; j < kRowBatch; ++j)
-                                    *reinterpret_cast<float4*>(lo + byte_step * j) =
-                                        lo_part(v[j]);
-                            if (store_y)
-#pragma unroll
-                                for (int j = 0; j < kRowBatch; ++j) if (own[j]) *reinterpret_cast<float4*>(ydst + off[j]) = v[j];
                         }
-                    } else if (three) {
-#pragma unroll 1
-                        for (int row = row0; row < sp.rows; row += kRowBatch * row_step, hi += kRowBatch * byte_step, lo += kRowBatch * byte_step) {
-                            float4 v[kRowBatch];
 #pragma unroll
-                            for (int j = 0; j < kRowBatch; ++j) v[j] = *reinterpret_cast<const float4*>(hi + byte_step * j);
+                        for (int j = 0; j < kRowBatch; ++j) {
+                            const float4 z = fma4(g, mul4(sub4(v[j], mu), rs), b);
+                            v[j] = make_float4(fmaxf(z.x, 0.f), fmaxf(z.y, 0.f), fmaxf(z.z, 0.f), fmaxf(z.w, 0.f));
+                            if (!inside[j]) v[j] = make_float4(0.f, 0.f, 0.f, 0.f);      // the padding is zero AFTER the activation
+                            *reinterpret_cast<float4*>(hi + byte_step * j) = v[j];
+                        }
+                        if (three)
 #pragma unroll
                             for (int j = 0; j < kRowBatch; ++j)
-                                *reinterpret_cast<float4*>(lo + byte_step * j) =
-                                    lo_part(v[j]);
-                        }
+                                *reinterpret_cast<float4*>(lo + byte_step * j) = lo_part(v[j]);
+                        if (store_y)
+#pragma unroll
+                            for (int j = 0; j < kRowBatch; ++j) if (own[j]) *reinterpret_cast<float4*>(ydst + off[j]) = v[j];
                     }
-                    fence_async_smem();               // generic-proxy writes -> tensor-core reads
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(a_full + 8 * s);
+                } else if (three) {
+#pragma unroll 1
+                    for (int row = row0; row < sp.rows; row += kRowBatch * row_step, hi += kRowBatch * byte_step, lo += kRowBatch * byte_step) {
+                        float4 v[kRowBatch];
+#pragma unroll
+                        for (int j = 0; j < kRowBatch; ++j) v[j] = *reinterpret_cast<const float4*>(hi + byte_step * j);
+#pragma unroll
+                        for (int j = 0; j < kRowBatch; ++j)
+                            *reinterpret_cast<float4*>(lo + byte_step * j) = lo_part(v[j]);
+                    }
                 }
+                fence_async_smem();               // generic-proxy writes -> tensor-core reads
+                __syncwarp();
+                if (lane == 0) mbar_arrive(a_full + 8 * s);
                 s += groups;
                 if (s >= S) { s -= S; par ^= 1u; }
                 ahead += groups;
@@ -1668,8 +1665,10 @@ bool conv_pipe_geom(const ConvShape& s, int pass, int passes, int launched, Conv
 
 bool conv_pipe_can_fuse_bn_output(const ConvPipeGeom& g) { return g.n_chunk <= 128; }      // a warp keeps the moments of two groups of 32 channels
 // (No column strips.)  Every channel slice of a launch repeats the work on its operand, about 1200 clocks for 128 rows of 16 channels
-// instead of 400: with four and more slices of a 1x1 window that is what the launch takes, and BN+ReLU in kernels of their own
+// instead of 400: with four and more slices of 128 channels of a 1x1 window that is what the launch takes, and BN+ReLU in kernels of their own
 // cost less (256->1024 @14 and the like: ResNet-152 35.0 -> 34.1 ms).  Two slices pay: 64->256 @56 would take 16 us to read and write.
+// So do four slices of 64 channels, which launches have that leave SMs idle otherwise: ResNet-11 285.8 us, 287.0 with BN kernels there
+// instead, ResNet-29 858 and 865.
 bool conv_pipe_can_fuse_bn_input(const ConvShape& s) { return s.stride == 1 && s.C % 16 == 0 && s.C <= 512 && s.W <= 254 && (s.R > 1 || s.K <= 256); }
 
 size_t conv_pipe_splitk_bytes(const ConvPipeGeom& g)

@@ -962,7 +962,7 @@ __global__ void __launch_bounds__(192) conv_tc_wgrad_direct_kernel(const __grid_
             float* obase = p.out + (long long)micro * p.out_ms + (long long)split * p.split_stride + (m0 + row0) * row_stride + cn0 + 2 * q;
             const bool pairs = (reinterpret_cast<uintptr_t>(obase) & 7u) == 0;      // (every other term is a whole number of 16-byte pieces)
             if (quad * 32 < p.m_chunk)                       // a whole warp of lanes beyond the chunk has nothing to read
-{
+            {
                 // W / 2 groups of eight columns a round: 32 columns where the slot is a multiple of them
                 auto write_out = [&](auto width) {
                     constexpr int W = decltype(width)::value;
@@ -1444,9 +1444,12 @@ int unfused_n_chunk(int c_out, int tiles)
 // Measured on 136 drawn 1x1 shapes both ways (16..512 channels, maps of 4..56, batch 4..128, one and three passes, calls back to
 // back): inside the line 0.61 of the pipelined launch's time (geometric mean of 189, one of them above 1.05: 9.6 us against 8.8;
 // 512 -> 32 channels on 10 maps of 17 x 17 12 us against 29, 64 -> 16 on 16 maps of 32 x 32 5.0 against 9.1), outside 1.15
-// (83).  3x3 windows: 1.25 of its time (248).  For a 1x1 window both add the products in the same order.  Since the pipelined kernel's
-// write-out and MMA issue were rewritten the line still holds but closely: 28 calls of 14 shapes inside it, 0.96 (512 -> 16 on 60
-// maps of 10 x 10 9.5 against 13.2 us, 16 -> 64 on 128 of 16 x 16 both 7.0, 256 -> 512 on 16 of 7 x 7 10.7 against 9.0).
+// (83).  3x3 windows: 1.25 of its time (248).  For a 1x1 window both add the products in the same order (the same bits).
+// Since the pipelined kernel's write-out and MMA issue were rewritten the line holds closely: 267 calls of 150 shapes inside it, three
+// runs, 0.96 of the pipelined launch's time in graphs of 20 calls, 103 of them above 1.05; 0.98 one by one; 0.95 in a Python loop, which
+// the host's work bounds.  The channels would sort them better than the sizes do: four times as many in as out and more 0.71 (67;
+// 512 -> 16 on 60 maps of 10 x 10 9.5 against 13.2 us), twice 0.87 (52), about as many 1.02 (60), twice as many out 1.12 (42), four times 1.32 (46;
+// 256 -> 512 on 16 of 7 x 7 10.7 against 9.0).
 bool conv_tc_faster_alone(const ConvShape& s, int pass, int passes)
 {
     const long long tiles = ((long long)s.N * s.P * s.Q + kTileM - 1) / kTileM;
