@@ -159,3 +159,15 @@ def test_when_launches_trigger_their_successors_changes_no_bit():
         out.append((bd.step(one_graph=True), bd.slots.cpu().numpy()))
     for loss, slots in out[1:]:
         assert loss == out[0][0] and np.array_equal(slots, out[0][1])
+
+
+def test_persistent_cells_form_a_plain_batch_norms_moments_like_single_launches():
+    """(In a cell the fp64 sums are a branch of the write-out, alone a kernel of their own.)"""
+    c = wl.config("r8v1")
+    x, labels, theta = seeded(c["ops"], c["in_hwc"], c["B"], 33, 0.2)
+    out = []
+    for ctas in (0, 16):
+        bd = Bound(c["ops"], c["in_hwc"], c["B"], c["M"], c["cuts"], theta, {hpf.OPT_CELL_CTAS: ctas, hpf.OPT_GROUP_LAUNCHES: 0})
+        bd.upload(x, labels)
+        out.append((bd.step(), bd.slots.cpu().numpy(), bd.model.launch_count()))
+    assert out[1][2] < out[0][2] and out[0][0] == out[1][0] and np.array_equal(out[0][1], out[1][1])
